@@ -77,7 +77,7 @@ int quantize_for_products(dbp_ctx *ctx, const void *delta, int dtype, long long 
         sp = *q_out;
     }
     const int k = ctx->code_set;
-    if ((rc = ws_reserve(ctx, ctx->dense_codes[k], static_cast<size_t>(numel) + 16))) return rc;
+    if ((want8 || q_out) && (rc = ws_reserve(ctx, ctx->dense_codes[k], static_cast<size_t>(numel) + 16))) return rc;
     int8_t *dense = static_cast<int8_t *>(ctx->dense_codes[k].ptr);
     // The set's previous readers (an earlier call's dW kernels on the second stream) must be done before its step
     // size and its codes are written again. The wait stands in front of the statistics kernel, where the stream
@@ -146,6 +146,53 @@ int quantize_for_products(dbp_ctx *ctx, const void *delta, int dtype, long long 
     return DBP_OK;
 }
 
+// A linear layer's products on the tensor cores (linear_tc.cu). The statistics kernel re-writes on the side the operands
+// the copy engine cannot address as they are (fp32 ones: two bf16 pieces; rows whose pitch is no multiple of 16 bytes)
+// and clears dW where its reduction is split. Both products leave in one launch on the context's stream.
+int linear_tc_backward(dbp_ctx *ctx, const void *delta, const void *X, const void *W, int io, long long B, long long N,
+                       long long K, unsigned long long seed, float scale, const float *delta_in, dbp_sparse *q_out, float *dW,
+                       void *dX, float *db, unsigned flags) {
+    const int pieces = io == DBP_F32 ? 2 : 1;
+    const LinearPlan pl = linear_plan(ctx, B, N, K, pieces, dW != nullptr, dX != nullptr);
+    // a *_host call: X is still on its way up on another stream
+    if (dW && ctx->hook_before_dw && cudaStreamWaitEvent(ctx->stream, ctx->hook_before_dw, 0) != cudaSuccess) return DBP_ECUDA;
+    SideJobs jobs;
+    int rc;
+    long long x_pitch = K, w_pitch = K;
+    auto rewrite = [&](const void *&src, Workspace &ws, long long rows, long long &pitch) {
+        pitch = linear_pitch(K);
+        if (int r = ws_reserve(ctx, ws, static_cast<size_t>(rows) * pitch * 2 * pieces)) return r;
+        jobs.rows[jobs.nrows++] = RowsJob{src, ws.ptr, io == DBP_F32, rows, K, pitch};
+        src = ws.ptr;
+        return static_cast<int>(DBP_OK);
+    };
+    if (io == DBP_F32 || K % 8 != 0) {
+        if (dW && (rc = rewrite(X, ctx->lin_x, B, x_pitch))) return rc;
+        if (dX && (rc = rewrite(W, ctx->lin_w, N, w_pitch))) return rc;
+    }
+    if (dW && pl.dw_split > 1) { jobs.zero = dW; jobs.zero_bytes = sizeof(float) * static_cast<size_t>(N) * K; }
+    const float *delta_p = nullptr;
+    const int8_t *codes = nullptr;
+    const void *codes16 = nullptr;
+    rc = quantize_for_products(ctx, delta, io, B * N, seed, scale, delta_in, q_out, &delta_p, &codes, false, N, linear_pitch(N),
+                               &codes16, nullptr, nullptr, jobs);
+    if (rc) return rc;
+    if (dW || dX) {
+        KernelTimer t(ctx, DBP_K_DX_DENSE);
+        const bool dx_bf16 = io == DBP_BF16 && !(flags & DBP_DX_F32);
+        rc = launch_linear_products(ctx, pl, codes16, X, W, pieces, x_pitch, w_pitch, delta_p, B, N, K, dW, dX, dx_bf16,
+                                    &ctx->state->tc_timeout);
+        if (rc) return rc;
+    }
+    if (db) {
+        KernelTimer t(ctx, DBP_K_DB);
+        rc = launch_column_sums(ctx, codes16, B, N, delta_p, db, (dW || dX) && !ctx->profiling);
+        if (rc) return rc;
+    }
+    if (ctx->hook_after_dx && cudaEventRecord(ctx->hook_after_dx, ctx->stream) != cudaSuccess) return DBP_ECUDA;
+    return DBP_OK;
+}
+
 int conv_backward_impl(dbp_ctx *ctx, const void *delta, const void *X, const void *W, int io,
                        const ConvShape &s, unsigned long long seed, float scale,
                        const float *delta_in, dbp_sparse *q_out, float *dW, void *dX, float *db,
@@ -166,6 +213,8 @@ int conv_backward_impl(dbp_ctx *ctx, const void *delta, const void *X, const voi
     const bool t3_dw_only = !t3_full && dW && !dX && tc3_tma_dw_supported(s, io);
     const bool can_dense = tc_supported(s, io) || t3_full || t3_dw_only;
     if ((flags & DBP_FORCE_DENSE) && !can_dense) return DBP_EUNSUPPORTED;
+    // linear layers of either type and any size: both products in one tensor-core launch
+    const bool linear = s.k == 1 && s.H == 1 && s.W == 1 && linear_tc_supported(s.B, s.Cout, s.Cin, io == DBP_F32 ? 2 : 1);
     DeviceGuard guard(ctx->device);
     if (!guard.ok) return DBP_ECUDA;
     const long long numel = s.B * s.Cout * s.H * s.W;
@@ -232,15 +281,17 @@ int conv_backward_impl(dbp_ctx *ctx, const void *delta, const void *X, const voi
     float density_estimate = 1.0f;
     for (const auto &e : ctx->densities)
         if (e.key == shape_key) density_estimate = e.density;
-    const bool dense = can_dense && !(flags & DBP_FORCE_SPARSE) &&
+    const bool dense = (can_dense || linear) && !(flags & DBP_FORCE_SPARSE) &&
                        ((flags & DBP_FORCE_DENSE) || ctx->crossover <= 0.f || density_estimate > ctx->crossover);
+    const bool lin = dense && linear;
     // which dense kernels run: the TMA-fed ones read bf16 code planes, the others int8 codes
-    const bool dx_tma = dense && dX && tma_dx_supported(s, io);
-    const bool dw_tma = dense && dW && tma_dw_supported(s, io);
+    const bool dx_tma = dense && !lin && dX && tma_dx_supported(s, io);
+    const bool dw_tma = dense && !lin && dW && tma_dw_supported(s, io);
     const bool any_tma = dx_tma || dw_tma;
     // a call that does not itself fork its dW first orders the earlier calls' outstanding dW work into the
     // stream: it may use the workspaces that work is still using
-    if (ctx->aux_pending && !(dense && dX && dW)) {
+    // (a linear layer stays on the stream and shares no workspace with that work: its set of code buffers is waited for)
+    if (ctx->aux_pending && !lin && !(dense && dX && dW)) {
         const int jr = dbp_join(ctx);
         if (jr) return jr;
     }
@@ -257,6 +308,21 @@ int conv_backward_impl(dbp_ctx *ctx, const void *delta, const void *X, const voi
         const int gr = launch_relu_backward(ctx, static_cast<const float *>(delta), mask, static_cast<float *>(ctx->dz_tmp.ptr), numel);
         if (gr) return gr;
         delta = ctx->dz_tmp.ptr;
+    }
+    // the density decides nothing while the threshold is 0: no read-back then, one stream operation less
+    auto read_density = [&] {
+        if (capturing || !(ctx->crossover > 0.f) || ctx->nnz_pending || !ctx->nnz_host || !ctx->nnz_event) return;
+        ctx->nnz_host_numel = numel;
+        ctx->nnz_host_key = shape_key;
+        if (cudaMemcpyAsync(ctx->nnz_host, &ctx->state->nnz, sizeof(unsigned long long), cudaMemcpyDeviceToHost,
+                            ctx->stream) == cudaSuccess &&
+            cudaEventRecord(ctx->nnz_event, ctx->stream) == cudaSuccess)
+            ctx->nnz_pending = true;
+    };
+    if (lin) {
+        const int lr = linear_tc_backward(ctx, delta, X, W, io, s.B, s.Cout, s.Cin, seed, scale, delta_in, q_out, dW, dX, db, flags);
+        if (!lr) read_density();
+        return lr;
     }
     const bool need8 = !dense || db || (!t3 && ((dX && !dx_tma) || (dW && !dw_tma)));
     const void *codes16 = nullptr, *codes_n = nullptr;
@@ -291,15 +357,7 @@ int conv_backward_impl(dbp_ctx *ctx, const void *delta, const void *X, const voi
                                    s.H * s.W, any_tma ? tma_code_pitch(s) : 0, any_tma ? &codes16 : nullptr,
                                    t3 ? &s : nullptr, t3 ? &codes_n : nullptr, jobs, stack_g, &codes_st, t3 ? mask_q : nullptr);
     if (rc) return rc;
-    // (the density decides nothing while the threshold is 0: no read-back then, one stream operation less)
-    if (!capturing && ctx->crossover > 0.f && !ctx->nnz_pending && ctx->nnz_host && ctx->nnz_event) {
-        ctx->nnz_host_numel = numel;
-        ctx->nnz_host_key = shape_key;
-        if (cudaMemcpyAsync(ctx->nnz_host, &ctx->state->nnz, sizeof(unsigned long long), cudaMemcpyDeviceToHost,
-                            ctx->stream) == cudaSuccess &&
-            cudaEventRecord(ctx->nnz_event, ctx->stream) == cudaSuccess)
-            ctx->nnz_pending = true;
-    }
+    read_density();
     if (dense) {
         // dX and dW read the same codes and nothing of each other: with both asked for, dW goes to the
         // context's second stream, so that its CTAs start as SMs come free instead of after the last dX CTA
@@ -549,7 +607,7 @@ int dbp_destroy(dbp_ctx *ctx) {
     cudaStreamSynchronize(ctx->stream);
     if (ctx->aux) cudaStreamSynchronize(ctx->aux);
     Workspace *all[] = {&ctx->dense_codes[0], &ctx->dense_codes[1], &ctx->codes16[0], &ctx->codes16[1],
-                        &ctx->codes_nhwc[0], &ctx->codes_nhwc[1], &ctx->codes_stack[0], &ctx->codes_stack[1], &ctx->dz_tmp, &ctx->s2_x, &ctx->s2_w, &ctx->s2_dx, &ctx->s2_dw, &ctx->dw_acc, &ctx->x_padded, &ctx->w_taps, &ctx->sp_bitmap, &ctx->sp_offsets, &ctx->sp_values,
+                        &ctx->codes_nhwc[0], &ctx->codes_nhwc[1], &ctx->codes_stack[0], &ctx->codes_stack[1], &ctx->dz_tmp, &ctx->s2_x, &ctx->s2_w, &ctx->s2_dx, &ctx->s2_dw, &ctx->dw_acc, &ctx->x_padded, &ctx->lin_x, &ctx->lin_w, &ctx->db_sums, &ctx->w_taps, &ctx->sp_bitmap, &ctx->sp_offsets, &ctx->sp_values,
                         &ctx->tc_partials};
     for (Workspace *w : all) if (w->ptr) cudaFree(w->ptr);
     for (Workspace &w : ctx->io) if (w.ptr) cudaFree(w.ptr);

@@ -48,6 +48,8 @@ struct dbp_ctx {
     // one call may still read their set while the next call's quantization writes the other one.
     dbp::Workspace dense_codes[2];      // int8 per element of delta
     dbp::Workspace x_padded;            // activations copied to 16-byte aligned planes
+    dbp::Workspace db_sums;             // bias gradient: counters that are zero between calls, then partial sums
+    dbp::Workspace lin_x, lin_w;        // a linear layer's operands as bf16 rows the copy engine can address
     dbp::Workspace codes16[2];          // bf16 code planes for the TMA-fed kernels
     dbp::Workspace w_taps;              // fp32 weights as [Cout][k*k][Cin]
     dbp::Workspace sp_bitmap, sp_offsets, sp_values;  // internal dbp_sparse
@@ -108,9 +110,19 @@ int ws_reserve(dbp_ctx *ctx, Workspace &w, size_t bytes);
 // and this saves launches): clearing a buffer (16-byte aligned, a multiple of 16 bytes), and re-laying 3x3
 // weights [Cout][Cin][9] as [Cout][taps][Cin] bf16 (taps = 9 for bf16 weights; 18 for fp32 weights, split into
 // two bf16 pieces: taps 0-8 the rounded values, 9-17 what the rounding left over).
+// Rows of a matrix as bf16 rows of `pitch` values (a multiple of 8, extra columns zero), which the copy engine can
+// address: fp32 rows become two pieces, rows * pitch apart (the rounded values, and the remainders rounded).
+struct RowsJob {
+    const void *src = nullptr;
+    void *dst = nullptr;
+    int f32 = 0;
+    long long rows = 0, cols = 0, pitch = 0;
+};
 struct SideJobs {
+    RowsJob rows[2];
+    int nrows = 0;
     void *zero = nullptr;
-    size_t zero_bytes = 0;
+    size_t zero_bytes = 0;             // a multiple of 4
     const void *w_src = nullptr;       // null: no weights to re-lay
     void *w_dst = nullptr;
     int w_f32 = 0;
@@ -143,6 +155,21 @@ bool small_linear_fits(const dbp_ctx *ctx, long long B, long long N, long long K
 int launch_small_linear(dbp_ctx *ctx, const float *delta, const float *X, const float *W, long long B, long long N,
                         long long K, unsigned long long seed, float scale, const float *delta_in, float *dW, float *dX,
                         float *db, float *delta_set, const uint8_t *mask = nullptr);
+
+// ---- linear_tc.cu: both products of a linear layer in one launch; codes as bf16 [B][linear_pitch(N)]
+struct LinearPlan {
+    int TN = 0;                       // columns per tile
+    long long dw_split = 1, dw_per_split = 0;   // > 1: dW is added up from parts and must have been cleared
+};
+bool linear_tc_supported(long long B, long long N, long long K, int pieces);
+long long linear_pitch(long long cols);
+LinearPlan linear_plan(const dbp_ctx *ctx, long long B, long long N, long long K, int pieces, bool want_dw, bool want_dx);
+// X, W: bf16 [pieces][rows][pitch]; pieces = 2 for fp32 operands split by a RowsJob
+int launch_linear_products(dbp_ctx *ctx, const LinearPlan &pl, const void *codes, const void *X, const void *W, int pieces,
+                           long long x_pitch, long long w_pitch, const float *delta_p, long long B, long long N, long long K,
+                           float *dW, void *dX, bool dx_bf16, int *err_flag);
+int launch_column_sums(dbp_ctx *ctx, const void *codes, long long rows, long long cols, const float *delta_p, float *db,
+                       bool after_products);
 
 // ---- product_kernels.cu
 struct ConvShape {

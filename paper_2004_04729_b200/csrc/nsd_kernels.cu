@@ -83,28 +83,93 @@ __device__ __forceinline__ void mask4(const unsigned char *mask, long long e, fl
 template <bool MASKED>
 __device__ __forceinline__ void mask4(const unsigned char *, long long, float (&)[8]) {}   // bf16 tensors take no mask
 
+// Rows of a matrix re-written as bf16 rows of `pitch` values (a multiple of 8, the extra columns zero): bf16 rows
+// copied, fp32 rows as two pieces, [rows][pitch] the rounded values and, rows * pitch further on, what the rounding
+// left over, rounded again. A thread takes eight columns of one row.
+__device__ __forceinline__ void rows_job(const RowsJob &j, long long first, long long stride) {
+    const unsigned gpr = static_cast<unsigned>(j.pitch / 8);
+    const long long n = j.rows * gpr, piece = j.rows * j.pitch;
+    for (long long i = first; i < n; i += stride) {
+        long long row;
+        unsigned g;
+        if ((n >> 31) == 0) {                      // 32-bit divisions cost a fraction of 64-bit ones
+            row = static_cast<unsigned>(i) / gpr;
+            g = static_cast<unsigned>(i) - static_cast<unsigned>(row) * gpr;
+        } else {
+            row = i / gpr;
+            g = static_cast<unsigned>(i - row * gpr);
+        }
+        const long long c0 = g * 8ll, left = j.cols - c0;          // left > 0
+        unsigned short *dst = static_cast<unsigned short *>(j.dst) + row * j.pitch + c0;
+        if (j.f32) {
+            const float *src = static_cast<const float *>(j.src) + row * j.cols + c0;
+            float x[8];
+            if (left >= 8 && (j.cols & 3) == 0) {
+                const float4 a = __ldg(reinterpret_cast<const float4 *>(src)), b = __ldg(reinterpret_cast<const float4 *>(src + 4));
+                x[0] = a.x; x[1] = a.y; x[2] = a.z; x[3] = a.w; x[4] = b.x; x[5] = b.y; x[6] = b.z; x[7] = b.w;
+            } else {
+#pragma unroll
+                for (int e = 0; e < 8; ++e) x[e] = e < left ? __ldg(src + e) : 0.f;
+            }
+            unsigned h[4], l[4];
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+                const __nv_bfloat162 hh = __floats2bfloat162_rn(x[2 * e], x[2 * e + 1]);
+                const float2 hf = __bfloat1622float2(hh);
+                const __nv_bfloat162 ll = __floats2bfloat162_rn(x[2 * e] - hf.x, x[2 * e + 1] - hf.y);
+                h[e] = *reinterpret_cast<const unsigned *>(&hh);
+                l[e] = *reinterpret_cast<const unsigned *>(&ll);
+            }
+            *reinterpret_cast<uint4 *>(dst) = make_uint4(h[0], h[1], h[2], h[3]);
+            *reinterpret_cast<uint4 *>(dst + piece) = make_uint4(l[0], l[1], l[2], l[3]);
+        } else {
+            const unsigned short *src = static_cast<const unsigned short *>(j.src) + row * j.cols + c0;
+            unsigned w[4];
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+                const unsigned a = 2 * e < left ? __ldg(src + 2 * e) : 0u, b = 2 * e + 1 < left ? __ldg(src + 2 * e + 1) : 0u;
+                w[e] = a | (b << 16);
+            }
+            *reinterpret_cast<uint4 *>(dst) = make_uint4(w[0], w[1], w[2], w[3]);
+        }
+    }
+}
+
+__global__ void __launch_bounds__(kThreads) rows_job_kernel(const RowsJob j) {
+    chain_wait();
+    chain_release();
+    rows_job(j, static_cast<long long>(blockIdx.x) * kThreads + threadIdx.x, static_cast<long long>(gridDim.x) * kThreads);
+}
+
 template <typename T, bool MASKED = false>
 __global__ void __launch_bounds__(kThreads)
 statistics_kernel(const T *__restrict__ x, long long n, double *__restrict__ partials,
                   DeviceState *__restrict__ st, float scale, float *__restrict__ delta_out,
-                  unsigned long long *__restrict__ nnz_out, uint4 *__restrict__ zero_ptr, long long zero_n16,
-                  const void *__restrict__ w_src, unsigned short *__restrict__ w_dst, int w_f32, long long w_cout, int w_cin,
-                  const unsigned char *__restrict__ mask, int w_phase_cin) {
+                  unsigned long long *__restrict__ nnz_out, const unsigned char *__restrict__ mask, const SideJobs jobs) {
     constexpr int EPT = Elem<T>::EPT;
     const long long nvec = n / EPT;
     chain_wait();
     chain_release();
     // side job for the layer's weight-gradient kernel, which adds its partial sums into dW: clear it
-    for (long long i = static_cast<long long>(blockIdx.x) * kThreads + threadIdx.x; i < zero_n16;
-         i += static_cast<long long>(gridDim.x) * kThreads)
-        zero_ptr[i] = make_uint4(0u, 0u, 0u, 0u);
+    {
+        const long long first = static_cast<long long>(blockIdx.x) * kThreads + threadIdx.x, step = static_cast<long long>(gridDim.x) * kThreads;
+        const long long zero_n16 = static_cast<long long>(jobs.zero_bytes / 16);
+        for (long long i = first; i < zero_n16; i += step) static_cast<uint4 *>(jobs.zero)[i] = make_uint4(0u, 0u, 0u, 0u);
+        if (first < static_cast<long long>(jobs.zero_bytes / 4) - 4 * zero_n16) static_cast<unsigned *>(jobs.zero)[4 * zero_n16 + first] = 0u;
+        // side jobs for the layer's product kernels: operands re-written as bf16 rows the copy engine can address
+        for (int j = 0; j < jobs.nrows; ++j) rows_job(jobs.rows[j], first, step);
+    }
     // side job for the layer's 3x3 input-gradient kernel: weights [co][ci][9] -> [co][tap][ci] bf16 (for fp32
     // weights two pieces: taps 0-8 the values rounded to bf16, taps 9-17 the remainders rounded to bf16).
     // w_phase_cin > 0: the layer is a stride-2 layer run on the four phase images of its input; w_src holds that
     // layer's own weights [co][w_phase_cin][9] and channel ph * w_phase_cin + c of the re-laid weights is phase
     // ph = 2 py + px of channel c, whose tap (ty, tx) is the strided layer's tap ky = 0 for (py, ty) = (1, 0),
     // 1 for (0, 1), 2 for (1, 1), kx likewise, and zero for every other pair.
-    if (w_src != nullptr) {
+    if (jobs.w_src != nullptr) {
+        const void *w_src = jobs.w_src;
+        unsigned short *w_dst = static_cast<unsigned short *>(jobs.w_dst);
+        const int w_f32 = jobs.w_f32, w_cin = static_cast<int>(jobs.Cin), w_phase_cin = jobs.phase_cin;
+        const long long w_cout = jobs.Cout;
         const int per_co = 9 * w_cin, taps = w_f32 ? 18 : 9;
         for (long long co = blockIdx.x; co < w_cout; co += gridDim.x) {
             unsigned short *dst = w_dst + co * taps * w_cin;
@@ -460,12 +525,13 @@ int launch_statistics(dbp_ctx *ctx, const void *delta, int dtype, long long nume
                       const float *delta_in, float *delta_out, unsigned long long *nnz_out, const SideJobs &jobs,
                       const uint8_t *mask) {
     if (mask != nullptr && dtype != DBP_F32) return DBP_EUNSUPPORTED;
-    uint4 *zp = static_cast<uint4 *>(jobs.zero);
-    const long long zn = jobs.zero ? static_cast<long long>(jobs.zero_bytes / 16) : 0;
-    unsigned short *wd = static_cast<unsigned short *>(jobs.w_dst);
-    const int wci = static_cast<int>(jobs.Cin);
     if (!(scale > 0.f)) {      // the step size is given: no statistics kernel, so no side jobs either (the caller sees to the weights)
         if (jobs.zero && cudaMemsetAsync(jobs.zero, 0, jobs.zero_bytes, ctx->stream) != cudaSuccess) return fail_cuda("clearing dW");
+        for (int j = 0; j < jobs.nrows; ++j) {
+            long long b = (jobs.rows[j].rows * (jobs.rows[j].pitch / 8) + kThreads - 1) / kThreads;
+            if (b > static_cast<long long>(ctx->sm_count) * 8) b = static_cast<long long>(ctx->sm_count) * 8;
+            if (int rc = cuda_ok(launch_chained(rows_job_kernel, dim3(static_cast<unsigned>(b)), dim3(kThreads), 0, ctx->stream, jobs.rows[j]))) return rc;
+        }
         note_launch();
         set_step_kernel<<<1, 1, 0, ctx->stream>>>(delta_in, ctx->state, delta_out, nnz_out);
         return cuda_ok(cudaGetLastError());
@@ -476,24 +542,25 @@ int launch_statistics(dbp_ctx *ctx, const void *delta, int dtype, long long nume
     // the side jobs want blocks of their own when the tensor is small (a block beyond the tensor's tiles adds zeros)
     if (jobs.w_src != nullptr && blocks < jobs.Cout) blocks = jobs.Cout;
     if (jobs.zero != nullptr && blocks < static_cast<long long>(jobs.zero_bytes / (16 * kThreads * 4))) blocks = static_cast<long long>(jobs.zero_bytes / (16 * kThreads * 4));
+    for (int j = 0; j < jobs.nrows; ++j) {         // two eight-column groups per thread
+        const long long b = jobs.rows[j].rows * (jobs.rows[j].pitch / 8) / (2 * kThreads);
+        if (blocks < b) blocks = b;
+    }
     if (blocks > ctx->partial_blocks) blocks = ctx->partial_blocks;
     // two resident blocks per SM, each walking several tiles, finish sooner than one block per tile: fewer partial
     // sums for the last block to add and fewer tickets (measured on the ResNet-50 layer set: 0.70 against 0.73 ms
     // per step for 48 layers; one block per SM: 0.76). The weight re-laying side job wants one block per output channel.
     if (jobs.w_src == nullptr && blocks > static_cast<long long>(ctx->sm_count) * kStatBlocksPerSM)
         blocks = static_cast<long long>(ctx->sm_count) * kStatBlocksPerSM;
-    cudaError_t e;
-    const unsigned char *nomask = nullptr;
-    if (dtype == DBP_F32 && mask != nullptr)
-        e = launch_chained(statistics_kernel<float, true>, dim3(static_cast<unsigned>(blocks)), dim3(kThreads), 0, ctx->stream,
-                           static_cast<const float *>(delta), numel, ctx->partials, ctx->state, scale, delta_out, nnz_out, zp, zn, jobs.w_src, wd, jobs.w_f32, jobs.Cout, wci,
-                           static_cast<const unsigned char *>(mask), jobs.phase_cin);
-    else if (dtype == DBP_F32)
-        e = launch_chained(statistics_kernel<float, false>, dim3(static_cast<unsigned>(blocks)), dim3(kThreads), 0, ctx->stream,
-                           static_cast<const float *>(delta), numel, ctx->partials, ctx->state, scale, delta_out, nnz_out, zp, zn, jobs.w_src, wd, jobs.w_f32, jobs.Cout, wci, nomask, jobs.phase_cin);
-    else
-        e = launch_chained(statistics_kernel<__nv_bfloat16, false>, dim3(static_cast<unsigned>(blocks)), dim3(kThreads), 0, ctx->stream,
-                           static_cast<const __nv_bfloat16 *>(delta), numel, ctx->partials, ctx->state, scale, delta_out, nnz_out, zp, zn, jobs.w_src, wd, jobs.w_f32, jobs.Cout, wci, nomask, jobs.phase_cin);
+    auto go = [&](auto kern, auto x, const unsigned char *m) {
+        return launch_chained(kern, dim3(static_cast<unsigned>(blocks)), dim3(kThreads), 0, ctx->stream, x, numel, ctx->partials,
+                              ctx->state, scale, delta_out, nnz_out, m, jobs);
+    };
+    const unsigned char *m = static_cast<const unsigned char *>(mask);
+    const float *xf = static_cast<const float *>(delta);
+    const cudaError_t e = dtype != DBP_F32 ? go(statistics_kernel<__nv_bfloat16, false>, static_cast<const __nv_bfloat16 *>(delta), m)
+                          : mask != nullptr ? go(statistics_kernel<float, true>, xf, m)
+                                            : go(statistics_kernel<float, false>, xf, m);
     return cuda_ok(e);
 }
 
