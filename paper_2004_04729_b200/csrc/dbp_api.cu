@@ -57,6 +57,18 @@ struct DeviceGuard {
     ~DeviceGuard() { if (prev >= 0) cudaSetDevice(prev); }
 };
 
+// The current set's previous readers (an earlier call's dW kernels on the second stream) must be done before its step
+// size and its codes are written again. The wait stands in front of a call's first kernel, where the stream
+// already holds the previous call's fork event: stream operations between two kernels stop their programmatic
+// overlap, so they are kept at one boundary per call.
+int wait_code_set(dbp_ctx *ctx) {
+    const int k = ctx->code_set;
+    if (!ctx->set_busy[k]) return DBP_OK;
+    if (cudaStreamWaitEvent(ctx->stream, ctx->ev_set_free[k], 0) != cudaSuccess) return fail_cuda("waiting for the code buffers");
+    ctx->set_busy[k] = false;
+    return DBP_OK;
+}
+
 // Quantize delta into `sp` (caller's arrays, or the context's internal ones) and into the
 // context's dense code buffer, which the product kernels read.
 int quantize_for_products(dbp_ctx *ctx, const void *delta, int dtype, long long numel,
@@ -79,14 +91,7 @@ int quantize_for_products(dbp_ctx *ctx, const void *delta, int dtype, long long 
     const int k = ctx->code_set;
     if ((want8 || q_out) && (rc = ws_reserve(ctx, ctx->dense_codes[k], static_cast<size_t>(numel) + 16))) return rc;
     int8_t *dense = static_cast<int8_t *>(ctx->dense_codes[k].ptr);
-    // The set's previous readers (an earlier call's dW kernels on the second stream) must be done before its step
-    // size and its codes are written again. The wait stands in front of the statistics kernel, where the stream
-    // already holds the previous call's fork event: stream operations between two kernels stop their programmatic
-    // overlap, so they are kept at one boundary per call.
-    if (ctx->set_busy[k]) {
-        if (cudaStreamWaitEvent(ctx->stream, ctx->ev_set_free[k], 0) != cudaSuccess) return fail_cuda("waiting for the code buffers");
-        ctx->set_busy[k] = false;
-    }
+    if ((rc = wait_code_set(ctx))) return rc;
     {
         KernelTimer t(ctx, DBP_K_STATISTICS);
         // without a caller's dbp_sparse the step size also goes to the set's own scalar: the product kernels
@@ -167,8 +172,8 @@ int linear_tc_backward(dbp_ctx *ctx, const void *delta, const void *X, const voi
         return static_cast<int>(DBP_OK);
     };
     if (io == DBP_F32 || K % 8 != 0) {
-        if (dW && (rc = rewrite(X, ctx->lin_x, B, x_pitch))) return rc;
-        if (dX && (rc = rewrite(W, ctx->lin_w, N, w_pitch))) return rc;
+        if (dW && (rc = rewrite(X, ctx->rows_x, B, x_pitch))) return rc;
+        if (dX && (rc = rewrite(W, ctx->rows_w, N, w_pitch))) return rc;
     }
     if (dW && pl.dw_split > 1) { jobs.zero = dW; jobs.zero_bytes = sizeof(float) * static_cast<size_t>(N) * K; }
     const float *delta_p = nullptr;
@@ -186,10 +191,60 @@ int linear_tc_backward(dbp_ctx *ctx, const void *delta, const void *X, const voi
     }
     if (db) {
         KernelTimer t(ctx, DBP_K_DB);
-        rc = launch_column_sums(ctx, codes16, B, N, delta_p, db, (dW || dX) && !ctx->profiling);
+        rc = launch_column_sums(ctx, codes16, B, N, delta_p, db, dW || dX);
         if (rc) return rc;
     }
     if (ctx->hook_after_dx && cudaEventRecord(ctx->hook_after_dx, ctx->stream) != cudaSuccess) return DBP_ECUDA;
+    return DBP_OK;
+}
+
+// The sparse gather kernels: int8 codes, fp32 FMAs on the non-zero ones.
+template <typename ReadDensity>
+int gather_backward(dbp_ctx *ctx, const void *delta, const void *X, const void *W, int io, const ConvShape &s,
+                    unsigned long long seed, float scale, const float *delta_in, dbp_sparse *q_out, float *dW, void *dX,
+                    float *db, unsigned flags, const ReadDensity &read_density) {
+    const float *delta_p = nullptr;
+    const int8_t *codes = nullptr;
+    if (ctx->phase_w_src != nullptr && dX) {      // a stride-2 layer on phase images: W is a workspace not yet written
+        KernelTimer t(ctx, DBP_K_GLUE);
+        const int pr = launch_phase_weights(ctx, ctx->phase_w_src, const_cast<void *>(W), io, s.Cout, s.Cin / 4);
+        if (pr) return pr;
+    }
+    int rc = quantize_for_products(ctx, delta, io, s.B * s.Cout * s.H * s.W, seed, scale, delta_in, q_out, &delta_p, &codes);
+    if (rc) return rc;
+    read_density();
+    if (dX) {
+        const size_t wb = sizeof(float) * static_cast<size_t>(s.Cout) * s.Cin * s.k * s.k;
+        if ((rc = ws_reserve(ctx, ctx->w_taps, wb))) return rc;
+        void *wt = ctx->w_taps.ptr;
+        const bool dx_bf16 = (io == DBP_BF16) && !(flags & DBP_DX_F32);
+        // streamed kernel: weight rows must be 16-byte multiples; otherwise the generic one
+        const bool streamed = s.k != 5 && (s.Cin * static_cast<long long>(elem_size(io))) % 16 == 0;
+        {
+            KernelTimer t(ctx, DBP_K_WEIGHT_TAPS);
+            rc = launch_weight_taps(ctx, W, io, s, wt, !streamed);
+        }
+        if (rc) return rc;
+        {
+            KernelTimer t(ctx, DBP_K_DX);
+            rc = streamed ? launch_conv_dx_streamed(ctx, codes, wt, io, delta_p, s, dX, dx_bf16)
+                          : launch_conv_dx(ctx, codes, static_cast<const float *>(wt), delta_p, s, dX, dx_bf16);
+        }
+        if (rc) return rc;
+    }
+    if (ctx->hook_after_dx && cudaEventRecord(ctx->hook_after_dx, ctx->stream) != cudaSuccess) return DBP_ECUDA;
+    if (dW && ctx->hook_before_dw && cudaStreamWaitEvent(ctx->stream, ctx->hook_before_dw, 0) != cudaSuccess) return DBP_ECUDA;
+    if (dW) {
+        KernelTimer t(ctx, DBP_K_DW);
+        rc = s.k == 5 ? DBP_EUNSUPPORTED : launch_conv_dw_streamed(ctx, codes, X, io, delta_p, s, dW);
+        if (rc == DBP_EUNSUPPORTED) rc = launch_conv_dw(ctx, codes, X, io, delta_p, s, dW);
+        if (rc) return rc;
+    }
+    if (db) {
+        KernelTimer t(ctx, DBP_K_DB);
+        rc = launch_bias_grad(ctx, codes, delta_p, s, db);
+        if (rc) return rc;
+    }
     return DBP_OK;
 }
 
@@ -208,13 +263,15 @@ int conv_backward_impl(dbp_ctx *ctx, const void *delta, const void *X, const voi
     if ((dW && !X) || (dX && !W)) return DBP_EINVAL;
     if (!aligned16(delta) || !aligned16(X) || !aligned16(W) || !aligned16(dW) || !aligned16(dX)) return DBP_EINVAL;
     if ((flags & DBP_FORCE_SPARSE) && (flags & DBP_FORCE_DENSE)) return DBP_EINVAL;
-    // 3x3 on the tensor cores: both products, or (fp32, any Cin: a network's first layer) the weight gradient alone
-    const bool t3_full = tc3_tma_supported(s, io);
-    const bool t3_dw_only = !t3_full && dW && !dX && tc3_tma_dw_supported(s, io);
-    const bool can_dense = tc_supported(s, io) || t3_full || t3_dw_only;
-    if ((flags & DBP_FORCE_DENSE) && !can_dense) return DBP_EUNSUPPORTED;
-    // linear layers of either type and any size: both products in one tensor-core launch
+    // What the tensor-core kernels take: linear layers, 1x1 and 3x3 layers of either type and any channel counts
     const bool linear = s.k == 1 && s.H == 1 && s.W == 1 && linear_tc_supported(s.B, s.Cout, s.Cin, io == DBP_F32 ? 2 : 1);
+    const bool conv1 = tma_dx_supported(s, io), conv3 = tc3_tma_supported(s, io);
+    const bool can_dense = linear || conv1 || conv3;
+    // DBP_FORCE_DENSE keeps its documented range: channel counts that are multiples of 8 (of an fp32 3x3 layer's weight
+    // gradient alone, only the output channels), and no fp32 linear or 1x1 layers
+    const bool force_ok = s.k == 1 ? io == DBP_BF16 && s.Cin % 8 == 0
+                                   : s.Cout % 8 == 0 && (s.Cin % 8 == 0 || (io == DBP_F32 && dW && !dX));
+    if ((flags & DBP_FORCE_DENSE) && !(can_dense && force_ok)) return DBP_EUNSUPPORTED;
     DeviceGuard guard(ctx->device);
     if (!guard.ok) return DBP_ECUDA;
     const long long numel = s.B * s.Cout * s.H * s.W;
@@ -238,13 +295,9 @@ int conv_backward_impl(dbp_ctx *ctx, const void *delta, const void *X, const voi
         delta = ctx->dz_tmp.ptr;
         mask = nullptr;
     }
-    const bool mask_vec = true;
-    if (io == DBP_F32 && s.k == 1 && s.H == 1 && s.W == 1 && !q_out && (dW || dX) && (!db || dW) && mask_vec &&
+    if (io == DBP_F32 && s.k == 1 && s.H == 1 && s.W == 1 && !q_out && (dW || dX) && (!db || dW) &&
         !(flags & (DBP_FORCE_SPARSE | DBP_FORCE_DENSE)) && small_linear_fits(ctx, s.B, s.Cout, s.Cin, dW != nullptr, dX != nullptr)) {
-        if (ctx->aux_pending) {
-            const int jr = dbp_join(ctx);
-            if (jr) return jr;
-        }
+        if (int wr = wait_code_set(ctx)) return wr;
         // a *_host call: X is still on its way up on another stream, and dX is read back after an event
         if (dW && ctx->hook_before_dw && cudaStreamWaitEvent(ctx->stream, ctx->hook_before_dw, 0) != cudaSuccess) return DBP_ECUDA;
         int rc;
@@ -281,13 +334,9 @@ int conv_backward_impl(dbp_ctx *ctx, const void *delta, const void *X, const voi
     float density_estimate = 1.0f;
     for (const auto &e : ctx->densities)
         if (e.key == shape_key) density_estimate = e.density;
-    const bool dense = (can_dense || linear) && !(flags & DBP_FORCE_SPARSE) &&
+    const bool dense = can_dense && !(flags & DBP_FORCE_SPARSE) &&
                        ((flags & DBP_FORCE_DENSE) || ctx->crossover <= 0.f || density_estimate > ctx->crossover);
     const bool lin = dense && linear;
-    // which dense kernels run: the TMA-fed ones read bf16 code planes, the others int8 codes
-    const bool dx_tma = dense && !lin && dX && tma_dx_supported(s, io);
-    const bool dw_tma = dense && !lin && dW && tma_dw_supported(s, io);
-    const bool any_tma = dx_tma || dw_tma;
     // a call that does not itself fork its dW first orders the earlier calls' outstanding dW work into the
     // stream: it may use the workspaces that work is still using
     // (a linear layer stays on the stream and shares no workspace with that work: its set of code buffers is waited for)
@@ -295,11 +344,11 @@ int conv_backward_impl(dbp_ctx *ctx, const void *delta, const void *X, const voi
         const int jr = dbp_join(ctx);
         if (jr) return jr;
     }
-    // 3x3 layers: the TMA-fed kernels read the codes position-major
-    const bool t3 = dense && (dX || dW) && (t3_full || t3_dw_only);
+    // 3x3 layers read the codes position-major, 1x1 layers as planes
+    const bool t3 = dense && (dX || dW) && conv3, t1 = dense && (dX || dW) && conv1;
     // fp32 3x3 layers on the tensor-core kernels apply the mask while they read delta_a (statistics and the
     // position-major quantizer); with a caller's sparse structure, or on any other path, delta_z is made first
-    const bool fold3 = mask && mask_vec && io == DBP_F32 && !q_out && t3;
+    const bool fold3 = mask && io == DBP_F32 && !q_out && t3;
     const uint8_t *mask_q = fold3 ? mask : nullptr;
     if (mask && !fold3) {      // every other path reads delta_z from memory: make it
         const int wr = ws_reserve(ctx, ctx->dz_tmp, static_cast<size_t>(numel) * sizeof(float));
@@ -324,16 +373,24 @@ int conv_backward_impl(dbp_ctx *ctx, const void *delta, const void *X, const voi
         if (!lr) read_density();
         return lr;
     }
-    const bool need8 = !dense || db || (!t3 && ((dX && !dx_tma) || (dW && !dw_tma)));
-    const void *codes16 = nullptr, *codes_n = nullptr;
-    // what the statistics kernel does on the side: the TMA-fed 1x1 dW kernel adds its partial sums into dW, so dW
-    // is cleared; the 3x3 dX kernel reads the weights tap by tap, so they are re-laid
+    if (!t3 && !t1) return gather_backward(ctx, delta, X, W, io, s, seed, scale, delta_in, q_out, dW, dX, db, flags, read_density);
+    const int pieces = io == DBP_F32 ? 2 : 1, k = ctx->code_set;
+    const bool dx_bf16 = io == DBP_BF16 && !(flags & DBP_DX_F32);
+    // what the statistics kernel does on the side: the 1x1 dW kernel adds its partial sums into dW, so dW is cleared;
+    // weights the copy engine cannot address as they are are re-written as bf16 rows, 3x3 weights tap by tap
     SideJobs jobs;
-    if (dw_tma) { jobs.zero = dW; jobs.zero_bytes = sizeof(float) * static_cast<size_t>(s.Cout) * s.Cin; }
+    if (t1 && dW) { jobs.zero = dW; jobs.zero_bytes = sizeof(float) * static_cast<size_t>(s.Cout) * s.Cin; }
+    long long w_pitch = s.Cin;
+    if (t1 && dX && (io == DBP_F32 || s.Cin % 8 != 0)) {
+        w_pitch = linear_pitch(s.Cin);
+        const int wr = ws_reserve(ctx, ctx->rows_w, static_cast<size_t>(s.Cout) * w_pitch * 2 * pieces);
+        if (wr) return wr;
+        jobs.rows[jobs.nrows++] = RowsJob{W, ctx->rows_w.ptr, io == DBP_F32, s.Cout, s.Cin, w_pitch};
+        W = ctx->rows_w.ptr;
+    }
     const bool w_side = t3 && dX && scale > 0.f;
     if (w_side) {
-        const int taps = io == DBP_F32 ? 18 : 9;
-        const int wr = ws_reserve(ctx, ctx->w_taps, sizeof(__nv_bfloat16) * static_cast<size_t>(s.Cout) * s.Cin * taps);
+        const int wr = ws_reserve(ctx, ctx->w_taps, sizeof(__nv_bfloat16) * static_cast<size_t>(s.Cout) * linear_pitch(s.Cin) * 9 * pieces);
         if (wr) return wr;
         jobs.w_src = W; jobs.w_dst = ctx->w_taps.ptr; jobs.w_f32 = io == DBP_F32; jobs.Cout = s.Cout; jobs.Cin = s.Cin;
     }
@@ -352,96 +409,83 @@ int conv_backward_impl(dbp_ctx *ctx, const void *delta, const void *X, const voi
     }
     // tiny planes: the weight-gradient kernel reads the images stacked into tall ones
     const int stack_g = (t3 && dW) ? tc3_stack_images(s, io) : 0;
-    const void *codes_st = nullptr;
-    int rc = quantize_for_products(ctx, delta, io, numel, seed, scale, delta_in, q_out, &delta_p, &codes, need8,
-                                   s.H * s.W, any_tma ? tma_code_pitch(s) : 0, any_tma ? &codes16 : nullptr,
+    const void *codes_st = nullptr, *codes16 = nullptr, *codes_n = nullptr;
+    int rc = quantize_for_products(ctx, delta, io, numel, seed, scale, delta_in, q_out, &delta_p, &codes, false,
+                                   s.H * s.W, t1 ? tma_code_pitch(s) : 0, t1 ? &codes16 : nullptr,
                                    t3 ? &s : nullptr, t3 ? &codes_n : nullptr, jobs, stack_g, &codes_st, t3 ? mask_q : nullptr);
     if (rc) return rc;
-    read_density();
-    if (dense) {
-        // dX and dW read the same codes and nothing of each other: with both asked for, dW goes to the
-        // context's second stream, so that its CTAs start as SMs come free instead of after the last dX CTA
-        const bool forked = dX && dW && ctx->aux != nullptr;
-        // (forking after the dX kernel instead, which would keep the quantizer -> dX boundary free of stream
-        // operations, measured slower: dW then starts a kernel later and meets the next layer's dX)
-        if (forked && (cudaEventRecord(ctx->ev_fork, ctx->stream) != cudaSuccess ||
-                       cudaStreamWaitEvent(ctx->aux, ctx->ev_fork, 0) != cudaSuccess))
-            return fail_cuda("forking the dW stream");
-        if (dX) {
-            KernelTimer t(ctx, DBP_K_DX_DENSE);
-            const bool dx_bf16 = (io == DBP_BF16) && !(flags & DBP_DX_F32);
-            rc = dx_tma ? launch_tma_dx(ctx, codes16, W, delta_p, s, dX, dx_bf16, &ctx->state->tc_timeout)
-                 : t3   ? launch_tc3_tma_dx(ctx, codes_n, W, io, delta_p, s, dX, dx_bf16, &ctx->state->tc_timeout, w_side)
-                        : launch_tc_dx(ctx, codes, W, delta_p, s, dX, dx_bf16, &ctx->state->tc_timeout);
-            if (rc) return rc;
-        }
-        if (ctx->hook_after_dx && cudaEventRecord(ctx->hook_after_dx, ctx->stream) != cudaSuccess) return DBP_ECUDA;
-        cudaStream_t caller = ctx->stream;
-        if (forked) ctx->stream = ctx->aux;          // the dW launchers enqueue on the context's stream
-        if (dW && ctx->hook_before_dw && cudaStreamWaitEvent(ctx->stream, ctx->hook_before_dw, 0) != cudaSuccess) rc = DBP_ECUDA;
-        if (dW && !rc) {
-            KernelTimer t(ctx, DBP_K_DW_DENSE);
-            rc = dw_tma ? launch_tma_dw(ctx, codes16, X, delta_p, s, dW, &ctx->state->tc_timeout)
-                 : (t3 && stack_g > 0)
-                     ? launch_tc3_tma_dw(ctx, codes_st, X, io, delta_p,
-                                         ConvShape{s.B / stack_g, s.Cin, s.Cout, static_cast<long long>(stack_g) * (s.H + 1), s.W, 3}, dW,
-                                         &ctx->state->tc_timeout, stack_g, static_cast<int>(s.H))
-                 : t3   ? launch_tc3_tma_dw(ctx, codes_n, X, io, delta_p, s, dW, &ctx->state->tc_timeout)
-                        : launch_tc_dw(ctx, codes, X, delta_p, s, dW, &ctx->state->tc_timeout);
-        }
-        ctx->stream = caller;
-        if (forked) {
-            // the set's buffers are free once the dW kernels are done; with DBP_DW_ASYNC the caller's stream is
-            // ordered after them only by the next user of the set, by dbp_join or by a synchronising call
-            const int k = ctx->code_set;
-            if (cudaEventRecord(ctx->ev_set_free[k], ctx->aux) != cudaSuccess) return fail_cuda("recording the end of dW");
-            if ((flags & DBP_DW_ASYNC) && !rc) {
-                ctx->set_busy[k] = true;
-                ctx->aux_pending = true;
-                ctx->code_set = k ^ 1;
-            } else if (cudaStreamWaitEvent(caller, ctx->ev_set_free[k], 0) != cudaSuccess) {
-                return fail_cuda("joining the dW stream");
-            }
-        }
-        if (rc) return rc;
-        if (db) {
-            KernelTimer t(ctx, DBP_K_DB);
-            rc = launch_bias_grad(ctx, codes, delta_p, s, db);
-            if (rc) return rc;
-        }
-        return DBP_OK;
+    // Activations the copy engine cannot address as they are (fp32: two bf16 pieces; planes that are no multiple of 16
+    // bytes; stacked tiny planes) are re-written into the set's own buffer: beside the quantizer where the call ends with
+    // its dW, on the stream of the dW kernels where that stream runs behind the caller's anyway (DBP_DW_ASYNC: 4 % on the
+    // VGG-16 layer set) or where a *_host call's activations are still on their way up.
+    const void *Xp = X;
+    long long x_pitch = s.H * s.W;
+    const bool rewrite_x = dW && (io == DBP_F32 || x_pitch % 8 != 0);
+    const bool forked = dX && dW && ctx->aux != nullptr;
+    const bool late_x = ctx->hook_before_dw != nullptr || (forked && (flags & DBP_DW_ASYNC));
+    auto write_x = [&](bool beside) -> int {
+        KernelTimer t(ctx, DBP_K_DW_DENSE);
+        return stack_g > 0 ? launch_x_stacked(ctx, static_cast<const float *>(X), ctx->x_padded[k].ptr, s, stack_g, beside)
+                           : launch_rows_job(ctx, RowsJob{X, ctx->x_padded[k].ptr, io == DBP_F32, s.B * s.Cin, s.H * s.W, x_pitch}, beside);
+    };
+    if (rewrite_x) {
+        const long long rows = stack_g > 0 ? s.B / stack_g * s.Cin : s.B * s.Cin;
+        x_pitch = linear_pitch(stack_g > 0 ? stack_g * (s.H + 1) * s.W : s.H * s.W);
+        if ((rc = ws_reserve(ctx, ctx->x_padded[k], static_cast<size_t>(rows) * x_pitch * 2 * pieces))) return rc;
+        Xp = ctx->x_padded[k].ptr;
+        // (with a caller's structure the last kernel is not the position-major or plane quantizer's chained launch alone)
+        if (!late_x && (rc = write_x(!q_out))) return rc;
     }
+    read_density();
+    // dX and dW read the same codes and nothing of each other: with both asked for, dW goes to the
+    // context's second stream, so that its CTAs start as SMs come free instead of after the last dX CTA
+    // (forking after the dX kernel instead, which would keep the quantizer -> dX boundary free of stream
+    // operations, measured slower: dW then starts a kernel later and meets the next layer's dX)
+    if (forked && (cudaEventRecord(ctx->ev_fork, ctx->stream) != cudaSuccess ||
+                   cudaStreamWaitEvent(ctx->aux, ctx->ev_fork, 0) != cudaSuccess))
+        return fail_cuda("forking the dW stream");
     if (dX) {
-        const size_t wb = sizeof(float) * static_cast<size_t>(s.Cout) * s.Cin * s.k * s.k;
-        if ((rc = ws_reserve(ctx, ctx->w_taps, wb))) return rc;
-        void *wt = ctx->w_taps.ptr;
-        const bool dx_bf16 = (io == DBP_BF16) && !(flags & DBP_DX_F32);
-        // streamed kernel: weight rows must be 16-byte multiples; otherwise the generic one
-        const bool streamed = s.k != 5 && (s.Cin * static_cast<long long>(elem_size(io))) % 16 == 0;
-        {
-            KernelTimer t(ctx, DBP_K_WEIGHT_TAPS);
-            rc = launch_weight_taps(ctx, W, io, s, wt, !streamed);
-        }
-        if (rc) return rc;
-        {
-            KernelTimer t(ctx, DBP_K_DX);
-            rc = streamed ? launch_conv_dx_streamed(ctx, codes, wt, io, delta_p, s, dX, dx_bf16)
-                          : launch_conv_dx(ctx, codes, static_cast<const float *>(wt), delta_p, s, dX, dx_bf16);
-        }
+        KernelTimer t(ctx, DBP_K_DX_DENSE);
+        rc = t1 ? launch_tma_dx(ctx, codes16, W, pieces, w_pitch, delta_p, s, dX, dx_bf16, &ctx->state->tc_timeout)
+                : launch_tc3_tma_dx(ctx, codes_n, W, io, delta_p, s, dX, dx_bf16, &ctx->state->tc_timeout, w_side);
         if (rc) return rc;
     }
     if (ctx->hook_after_dx && cudaEventRecord(ctx->hook_after_dx, ctx->stream) != cudaSuccess) return DBP_ECUDA;
-    if (dW && ctx->hook_before_dw && cudaStreamWaitEvent(ctx->stream, ctx->hook_before_dw, 0) != cudaSuccess) return DBP_ECUDA;
-    if (dW) {
-        KernelTimer t(ctx, DBP_K_DW);
-        rc = s.k == 5 ? DBP_EUNSUPPORTED : launch_conv_dw_streamed(ctx, codes, X, io, delta_p, s, dW);
-        if (rc == DBP_EUNSUPPORTED) rc = launch_conv_dw(ctx, codes, X, io, delta_p, s, dW);
+    if (db && dX) {
+        KernelTimer t(ctx, DBP_K_DB);
+        rc = t1 ? launch_plane_sums(ctx, codes16, s.B, s.Cout, s.H * s.W, tma_code_pitch(s), delta_p, db, !ctx->hook_after_dx)
+                : launch_column_sums(ctx, codes_n, s.B * s.H * s.W, s.Cout, delta_p, db, !ctx->hook_after_dx);
         if (rc) return rc;
     }
-    if (db) {
+    cudaStream_t caller = ctx->stream;
+    if (forked) ctx->stream = ctx->aux;          // the dW launchers enqueue on the context's stream
+    if (dW && ctx->hook_before_dw && cudaStreamWaitEvent(ctx->stream, ctx->hook_before_dw, 0) != cudaSuccess) rc = DBP_ECUDA;
+    if (!rc && rewrite_x && late_x) rc = write_x(false);
+    if (dW && !rc) {
+        KernelTimer t(ctx, DBP_K_DW_DENSE);
+        ConvShape sw = s;
+        if (stack_g > 0) sw = ConvShape{s.B / stack_g, s.Cin, s.Cout, static_cast<long long>(stack_g) * (s.H + 1), s.W, 3};
+        rc = t1 ? launch_tma_dw(ctx, codes16, Xp, pieces, x_pitch, delta_p, s, dW, &ctx->state->tc_timeout)
+                : launch_tc3_tma_dw(ctx, stack_g > 0 ? codes_st : codes_n, Xp, pieces, x_pitch, delta_p, sw, dW, &ctx->state->tc_timeout);
+    }
+    ctx->stream = caller;
+    if (forked) {
+        // the set's buffers are free once the dW kernels are done; with DBP_DW_ASYNC the caller's stream is
+        // ordered after them only by the next user of the set, by dbp_join or by a synchronising call
+        if (cudaEventRecord(ctx->ev_set_free[k], ctx->aux) != cudaSuccess) return fail_cuda("recording the end of dW");
+        if ((flags & DBP_DW_ASYNC) && !rc) {
+            ctx->set_busy[k] = true;
+            ctx->aux_pending = true;
+            ctx->code_set = k ^ 1;
+        } else if (cudaStreamWaitEvent(caller, ctx->ev_set_free[k], 0) != cudaSuccess) {
+            return fail_cuda("joining the dW stream");
+        }
+    }
+    if (rc) return rc;
+    if (db && !dX) {
         KernelTimer t(ctx, DBP_K_DB);
-        rc = launch_bias_grad(ctx, codes, delta_p, s, db);
-        if (rc) return rc;
+        return t1 ? launch_plane_sums(ctx, codes16, s.B, s.Cout, s.H * s.W, tma_code_pitch(s), delta_p, db, dW != nullptr)
+                  : launch_column_sums(ctx, codes_n, s.B * s.H * s.W, s.Cout, delta_p, db, dW != nullptr);
     }
     return DBP_OK;
 }
@@ -607,8 +651,7 @@ int dbp_destroy(dbp_ctx *ctx) {
     cudaStreamSynchronize(ctx->stream);
     if (ctx->aux) cudaStreamSynchronize(ctx->aux);
     Workspace *all[] = {&ctx->dense_codes[0], &ctx->dense_codes[1], &ctx->codes16[0], &ctx->codes16[1],
-                        &ctx->codes_nhwc[0], &ctx->codes_nhwc[1], &ctx->codes_stack[0], &ctx->codes_stack[1], &ctx->dz_tmp, &ctx->s2_x, &ctx->s2_w, &ctx->s2_dx, &ctx->s2_dw, &ctx->dw_acc, &ctx->x_padded, &ctx->lin_x, &ctx->lin_w, &ctx->db_sums, &ctx->w_taps, &ctx->sp_bitmap, &ctx->sp_offsets, &ctx->sp_values,
-                        &ctx->tc_partials};
+                        &ctx->codes_nhwc[0], &ctx->codes_nhwc[1], &ctx->codes_stack[0], &ctx->codes_stack[1], &ctx->dz_tmp, &ctx->s2_x, &ctx->s2_w, &ctx->s2_dx, &ctx->s2_dw, &ctx->dw_acc, &ctx->x_padded[0], &ctx->x_padded[1], &ctx->rows_x, &ctx->rows_w, &ctx->db_sums, &ctx->w_taps, &ctx->sp_bitmap, &ctx->sp_offsets, &ctx->sp_values};
     for (Workspace *w : all) if (w->ptr) cudaFree(w->ptr);
     for (Workspace &w : ctx->io) if (w.ptr) cudaFree(w.ptr);
     for (ProfSlot &p : ctx->prof) { cudaEventDestroy(p.begin); cudaEventDestroy(p.end); }

@@ -47,13 +47,12 @@ struct dbp_ctx {
     // The codes of a layer exist in two sets of buffers used in turn: with DBP_DW_ASYNC the dW kernels of
     // one call may still read their set while the next call's quantization writes the other one.
     dbp::Workspace dense_codes[2];      // int8 per element of delta
-    dbp::Workspace x_padded;            // activations copied to 16-byte aligned planes
+    dbp::Workspace x_padded[2];         // activations re-written as 16-byte aligned bf16 planes, one per set of codes
     dbp::Workspace db_sums;             // bias gradient: counters that are zero between calls, then partial sums
-    dbp::Workspace lin_x, lin_w;        // a linear layer's operands as bf16 rows the copy engine can address
+    dbp::Workspace rows_x, rows_w;      // operands re-written as bf16 rows the copy engine can address: a linear layer's X, W
     dbp::Workspace codes16[2];          // bf16 code planes for the TMA-fed kernels
     dbp::Workspace w_taps;              // fp32 weights as [Cout][k*k][Cin]
     dbp::Workspace sp_bitmap, sp_offsets, sp_values;  // internal dbp_sparse
-    dbp::Workspace tc_partials;         // split-K partial blocks of the dense dW kernel
     dbp::Workspace codes_nhwc[2];       // bf16 codes [B][position][Cout] for the TMA-fed 3x3 kernels
     const uint8_t *next_mask = nullptr; // ReLU mask for the next backward call (dbp_set_relu_mask)
     dbp::Workspace dz_tmp;              // delta_z = delta_a (.) mask when that call cannot fold the mask into its loads
@@ -132,6 +131,8 @@ struct SideJobs {
 int launch_statistics(dbp_ctx *ctx, const void *delta, int dtype, long long numel, float scale,
                       const float *delta_in, float *delta_out, unsigned long long *nnz_out,
                       const SideJobs &jobs = SideJobs(), const uint8_t *mask = nullptr);
+// beside: the kernel before it on the stream is the quantizer; the job runs beside it
+int launch_rows_job(dbp_ctx *ctx, const RowsJob &job, bool beside);
 int launch_quantize(dbp_ctx *ctx, const void *delta, int dtype, long long numel,
                     unsigned long long seed, const float *delta_p, uint32_t *bitmap,
                     uint16_t *offsets, int8_t *values, int8_t *dense,
@@ -168,8 +169,13 @@ LinearPlan linear_plan(const dbp_ctx *ctx, long long B, long long N, long long K
 int launch_linear_products(dbp_ctx *ctx, const LinearPlan &pl, const void *codes, const void *X, const void *W, int pieces,
                            long long x_pitch, long long w_pitch, const float *delta_p, long long B, long long N, long long K,
                            float *dW, void *dX, bool dx_bf16, int *err_flag);
+
+// ---- bias_grad.cu: db from bf16 codes, rows [rows][cols rounded up to 8] or planes [B][channels][pitch]
+// beside: the call may run beside the kernel before it on the stream (a product, which writes nothing it reads)
 int launch_column_sums(dbp_ctx *ctx, const void *codes, long long rows, long long cols, const float *delta_p, float *db,
-                       bool after_products);
+                       bool beside);
+int launch_plane_sums(dbp_ctx *ctx, const void *codes, long long B, long long channels, long long hw, long long pitch,
+                      const float *delta_p, float *db, bool beside);
 
 // ---- product_kernels.cu
 struct ConvShape {
@@ -187,34 +193,26 @@ int launch_conv_dw(dbp_ctx *ctx, const int8_t *codes, const void *X, int dtype,
                    const float *delta_p, const ConvShape &s, float *dW);
 int launch_conv_dw_streamed(dbp_ctx *ctx, const int8_t *codes, const void *X, int dtype,
                             const float *delta_p, const ConvShape &s, float *dW);
-// ---- tc_dense.cu
-bool tc_supported(const ConvShape &s, int io);
-int launch_tc_dw(dbp_ctx *ctx, const int8_t *codes, const void *X, const float *delta_p,
-                 const ConvShape &s, float *dW, int *err_flag);
-int launch_tc_dx(dbp_ctx *ctx, const int8_t *codes, const void *W, const float *delta_p,
-                 const ConvShape &s, void *dX, bool dx_bf16, int *err_flag);
 // ---- tma_dx.cu: 1x1 dX with TMA-fed operands; codes as bf16 planes [B*Cout][tma_code_pitch]
 bool tma_dx_supported(const ConvShape &s, int io);
 long long tma_code_pitch(const ConvShape &s);
-int launch_tma_dx(dbp_ctx *ctx, const void *codes_bf16, const void *W, const float *delta_p,
+// W: bf16 [pieces][Cout][w_pitch]; X: bf16 [pieces of B images][Cin][x_pitch] (pitches multiples of 8)
+int launch_tma_dx(dbp_ctx *ctx, const void *codes_bf16, const void *W, int pieces, long long w_pitch, const float *delta_p,
                   const ConvShape &s, void *dX, bool dx_bf16, int *err_flag);
 // ---- tma_dw.cu: 1x1 dW with TMA-fed operands (same code planes)
-bool tma_dw_supported(const ConvShape &s, int io);
-int launch_tma_dw(dbp_ctx *ctx, const void *codes_bf16, const void *X, const float *delta_p,
+int launch_tma_dw(dbp_ctx *ctx, const void *codes_bf16, const void *X, int pieces, long long x_pitch, const float *delta_p,
                   const ConvShape &s, float *dW, int *err_flag);
-// planes of H x W bf16 values -> rows of Wp values (multiple of 8), extra columns zero
-int launch_pad_planes(dbp_ctx *ctx, const void *in, void *out, long long planes, int H, int W, int Wp);
-// dW = Delta * sum of nsplit partial blocks of nw floats (nw % 4 == 0), fixed order
-int launch_dw_sum(dbp_ctx *ctx, const float *partials, int nsplit, long long nw, const float *delta_p, float *dW);
-// ---- tc3_tma_dx.cu / tc3_tma_dw.cu: 3x3 products with TMA-fed operands; codes as bf16 [B][H*W][Cout]
+// ---- tc3_tma_dx.cu / tc3_tma_dw.cu: 3x3 products with TMA-fed operands; codes as bf16 [B][H*W][Cout rounded up to 8]
 bool tc3_tma_supported(const ConvShape &s, int io);
-bool tc3_tma_dw_supported(const ConvShape &s, int io);     // dW alone: also fp32 layers with any Cin
 // io: the operands' type; fp32 weights / activations are split into two bf16 pieces on the way in
 // weights_ready: ctx->w_taps already holds the re-laid weights (the statistics kernel did it on the side)
 int launch_tc3_tma_dx(dbp_ctx *ctx, const void *codes_nhwc, const void *W, int io, const float *delta_p,
                       const ConvShape &s, void *dX, bool dx_bf16, int *err_flag, bool weights_ready = false);
-int launch_tc3_tma_dw(dbp_ctx *ctx, const void *codes_nhwc, const void *X, int io, const float *delta_p,
-                      const ConvShape &s, float *dW, int *err_flag, int stack_g = 0, int real_h = 0);
+// X: bf16 planes of x_pitch values, pieces of every image one after the other
+int launch_tc3_tma_dw(dbp_ctx *ctx, const void *codes_nhwc, const void *X, int pieces, long long x_pitch, const float *delta_p,
+                      const ConvShape &s, float *dW, int *err_flag);
+// fp32 activations split and stacked for it (out: [2][B / G][Cin][pitch]); beside: as for launch_rows_job
+int launch_x_stacked(dbp_ctx *ctx, const float *X, void *out, const ConvShape &s, int stack_g, bool beside);
 // Planes of fewer than 64 positions: how many images of a batch to stack into one tall image (one zero row after
 // every image) for the weight-gradient kernel, whose work comes in segments of one image; 0: do not stack.
 int tc3_stack_images(const ConvShape &s, int io);

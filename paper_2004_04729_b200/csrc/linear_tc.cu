@@ -273,83 +273,6 @@ linear_products_kernel(const __grid_constant__ LinMaps maps, const __grid_consta
     }
 }
 
-// db[j] = Delta * sum_b q[b][j] from the bf16 codes [B][pitch]. A block owns 64 columns and a range of rows, a thread
-// eight of the columns and every 32nd row, four 16-byte loads in flight. A thread's own sum is exact in fp32 (integers
-// below 2^24 up to four million rows of full-scale codes); the threads' and the blocks' sums are added as integers, the
-// last block of a column group adding up the ranges and putting its counter back to zero.
-// The kernel reads only what the kernel before the products wrote, and the products kernel lets it start when all of
-// its CTAs have seen that one complete: so it works first and waits for the products (whose tensor-bound main loop it
-// runs beside) only before it ends.
-__global__ void __launch_bounds__(256)
-column_sums_kernel(const unsigned short *__restrict__ codes, long long rows, int cols, long long pitch, long long per_split,
-                   int *__restrict__ partials, unsigned *__restrict__ tickets, const float *__restrict__ delta_p,
-                   float *__restrict__ db, int wait_first) {
-    __shared__ int sum_s[64];
-    __shared__ bool is_last;
-    if (threadIdx.x < 64) sum_s[threadIdx.x] = 0;
-    __syncthreads();
-    if (wait_first) chain_wait();
-    chain_release();
-    const int c0 = blockIdx.x * 64 + (threadIdx.x & 7) * 8;
-    const long long r1 = (blockIdx.y + 1) * per_split < rows ? (blockIdx.y + 1) * per_split : rows;
-    float facc[8] = {};
-    if (c0 < cols) {
-        auto add = [&](const uint4 &v) {
-            const unsigned w[4] = {v.x, v.y, v.z, v.w};
-#pragma unroll
-            for (int i = 0; i < 4; ++i) {
-                facc[2 * i] += __uint_as_float(w[i] << 16);
-                facc[2 * i + 1] += __uint_as_float(w[i] & 0xffff0000u);
-            }
-        };
-        long long r = blockIdx.y * per_split + (threadIdx.x >> 3);
-        const unsigned short *src = codes + r * pitch + c0;
-        for (; r + 96 < r1; r += 128, src += 128 * pitch) {
-            uint4 v[4];
-#pragma unroll
-            for (int u = 0; u < 4; ++u) v[u] = __ldcg(reinterpret_cast<const uint4 *>(src + 32 * u * pitch));
-#pragma unroll
-            for (int u = 0; u < 4; ++u) add(v[u]);
-        }
-        for (; r < r1; r += 32, src += 32 * pitch) add(__ldcg(reinterpret_cast<const uint4 *>(src)));
-    }
-    // the four row groups of a warp, then the warps (padding columns may hold anything; they are not stored)
-    int acc[8];
-#pragma unroll
-    for (int i = 0; i < 8; ++i) {
-        acc[i] = static_cast<int>(facc[i]);
-        acc[i] += __shfl_xor_sync(0xffffffffu, acc[i], 8);
-        acc[i] += __shfl_xor_sync(0xffffffffu, acc[i], 16);
-    }
-    if ((threadIdx.x & 31) < 8)
-#pragma unroll
-        for (int i = 0; i < 8; ++i) atomicAdd(&sum_s[(threadIdx.x & 7) * 8 + i], acc[i]);
-    __syncthreads();
-    const int c = blockIdx.x * 64 + threadIdx.x;
-    int total = threadIdx.x < 64 ? sum_s[threadIdx.x] : 0;
-    if (gridDim.y > 1) {
-        if (threadIdx.x < 64) __stcg(partials + (blockIdx.y * static_cast<long long>(gridDim.x) + blockIdx.x) * 64 + threadIdx.x, total);
-        __threadfence();
-        __syncthreads();
-        if (threadIdx.x == 0) {
-            is_last = atomicAdd(tickets + blockIdx.x, 1u) == gridDim.y - 1;
-            if (is_last) tickets[blockIdx.x] = 0u;
-        }
-        __syncthreads();
-        if (is_last && threadIdx.x < 64) {
-            __threadfence();
-            total = 0;
-#pragma unroll 4
-            for (unsigned s = 0; s < gridDim.y; ++s)
-                total += __ldcg(partials + (s * static_cast<long long>(gridDim.x) + blockIdx.x) * 64 + threadIdx.x);
-        }
-        if (is_last && threadIdx.x < 64 && c < cols) db[c] = static_cast<float>(total) * (*delta_p);
-    } else if (threadIdx.x < 64 && c < cols) {
-        db[c] = static_cast<float>(total) * (*delta_p);
-    }
-    if (!wait_first) chain_wait();
-}
-
 bool fits_int(long long v) { return v > 0 && v < (1ll << 30); }
 
 }  // namespace
@@ -461,37 +384,6 @@ int launch_linear_products(dbp_ctx *ctx, const LinearPlan &pl, const void *codes
         return fail_cuda("shared memory size");
     const int grid = p.tiles < ctx->sm_count ? p.tiles : ctx->sm_count;
     return cuda_ok(launch_chained(linear_products_kernel, dim3(static_cast<unsigned>(grid)), dim3(kThreadsL), smem, ctx->stream, maps, p));
-}
-
-// after_products: the kernel enqueued before this one on the stream is linear_products_kernel
-int launch_column_sums(dbp_ctx *ctx, const void *codes, long long rows, long long cols, const float *delta_p, float *db,
-                       bool after_products) {
-    const long long groups = (cols + 63) / 64;
-    // ranges of at least 128 rows (four loads per thread), about two blocks per SM
-    long long split = 2ll * ctx->sm_count / groups;
-    if (split > (rows + 127) / 128) split = (rows + 127) / 128;
-    constexpr long long kMaxGroups = 16384;
-    if (split < 1 || groups > kMaxGroups) split = 1;
-    const long long per = (rows + split - 1) / split;
-    split = (rows + per - 1) / per;
-    int *partials = nullptr;
-    unsigned *tickets = nullptr;
-    if (split > 1) {
-        // the counters lie at the start of the workspace and are zero between calls
-        const size_t had = ctx->db_sums.bytes, counter_bytes = kMaxGroups * sizeof(unsigned);
-        int rc = ws_reserve(ctx, ctx->db_sums, counter_bytes + static_cast<size_t>(split) * groups * 256);
-        if (rc) return rc;
-        if (ctx->db_sums.bytes != had) {
-            if (cudaMemsetAsync(ctx->db_sums.ptr, 0, counter_bytes, ctx->stream) != cudaSuccess)
-                return fail_cuda("clearing the counters of the bias gradient");
-            after_products = false;                                  // the memset lies between the two kernels
-        }
-        tickets = static_cast<unsigned *>(ctx->db_sums.ptr);
-        partials = reinterpret_cast<int *>(static_cast<unsigned char *>(ctx->db_sums.ptr) + counter_bytes);
-    }
-    return cuda_ok(launch_chained(column_sums_kernel, dim3(static_cast<unsigned>(groups), static_cast<unsigned>(split)), dim3(256), 0,
-                                  ctx->stream, static_cast<const unsigned short *>(codes), rows, static_cast<int>(cols),
-                                  linear_pitch(cols), per, partials, tickets, delta_p, db, after_products ? 0 : 1));
 }
 
 }  // namespace dbp

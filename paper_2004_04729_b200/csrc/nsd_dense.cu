@@ -340,6 +340,8 @@ __device__ __forceinline__ void apply_mask(const unsigned char *mask, long long 
 }
 __device__ __forceinline__ void apply_mask(const unsigned char *, long long, float (&)[8]) {}
 
+// Channel counts that are no multiple of 8: rows of the output are padded to one (the padding is not written: the copy
+// engine never reads it), and small planes take the paths of large ones.
 template <typename T, int V, bool STACK, bool MASKED>
 __global__ void __launch_bounds__(kThreads)
 quantize_nhwc_kernel(const T *__restrict__ x, int B, int C, int HW, unsigned long long seed,
@@ -358,7 +360,8 @@ quantize_nhwc_kernel(const T *__restrict__ x, int B, int C, int HW, unsigned lon
     const float inv = live ? __fdiv_rn(1.0f, delta) : 0.f;
     const int ct = (C + kTC - 1) / kTC, pt = (HW + kTP - 1) / kTP;
     const long long ntiles = static_cast<long long>(B) * ct * pt;
-    const bool flat = HW < kTP;
+    const bool flat = HW < kTP && (C & 7) == 0;
+    const int pitch = (C + 7) & ~7;
     unsigned nnz = 0, sat = 0;
     float nz = 0.f;
     int buf = 0;
@@ -396,20 +399,22 @@ quantize_nhwc_kernel(const T *__restrict__ x, int B, int C, int HW, unsigned lon
                 const int v = threadIdx.x + kThreads * i;
                 const int c = 2 * (v / VPR), pv = (v % VPR) * VV;
                 float f0[VV] = {}, f1[VV] = {};
-                const bool in = c0 + c < C && p0 + pv < HW;       // C is even, HW % V == 0: whole vectors, both channels
+                const bool in = c0 + c < C && p0 + pv < HW, in1 = in && c0 + c + 1 < C;       // HW % V == 0: whole vectors
                 const long long e0 = (static_cast<long long>(b) * C + c0 + c) * HW + p0 + pv, e1 = e0 + HW;
                 if (in && live) {
                     float a0[VV], a1[VV];
                     TileLoad<T, VV>::ld(x + e0, a0);
-                    TileLoad<T, VV>::ld(x + e1, a1);
+                    if (in1) TileLoad<T, VV>::ld(x + e1, a1);
                     apply_mask(mask, e0, a0);
-                    apply_mask(mask, e1, a1);
                     codes_of<VV>(a0, e0, seed, inv, f0, nz, sat);
-                    codes_of<VV>(a1, e1, seed, inv, f1, nz, sat);
+                    if (in1) {
+                        apply_mask(mask, e1, a1);
+                        codes_of<VV>(a1, e1, seed, inv, f1, nz, sat);
+                    }
                 }
                 if (in && dense8 != nullptr) {
                     store_bytes<VV>(dense8, e0, f0);
-                    store_bytes<VV>(dense8, e1, f1);
+                    if (in1) store_bytes<VV>(dense8, e1, f1);
                 }
 #pragma unroll
                 for (int j = 0; j < VV; ++j)
@@ -437,7 +442,7 @@ quantize_nhwc_kernel(const T *__restrict__ x, int B, int C, int HW, unsigned lon
             const int v = threadIdx.x + kThreads * i;
             const int pp = v >> 3, ch = v & 7;
             if (p0 + pp < HW && c0 + ch * 8 < C)
-                *reinterpret_cast<uint4 *>(out + (static_cast<long long>(b) * HW + p0 + pp) * C + c0 + ch * 8) =
+                *reinterpret_cast<uint4 *>(out + (static_cast<long long>(b) * HW + p0 + pp) * pitch + c0 + ch * 8) =
                     *reinterpret_cast<const uint4 *>(tl + tile_off(pp, ch * 8));
             // Second copy for the weight-gradient kernel of tiny planes: the images one below the other as tall
             // images, a row of zeros after every image (what a tap that leaves an image must read).
@@ -576,16 +581,16 @@ int launch_quantize_dense(dbp_ctx *ctx, const void *delta, int dtype, long long 
     return cuda_ok(e);
 }
 
-// delta_z [B][C][HW] -> bf16 codes [B][HW][C] (C % 8 == 0) and, when dense8 is not null, int8 codes
+// delta_z [B][C][HW] -> bf16 codes [B][HW][C rounded up to a multiple of 8] and, when dense8 is not null, int8 codes
 // in delta_z's order
 int launch_quantize_nhwc(dbp_ctx *ctx, const void *delta, int dtype, long long B, long long C, long long HW,
                          unsigned long long seed, const float *delta_p, void *codes_nhwc, int8_t *dense8, bool count,
                          void *codes_stack, int plane_w, int stack_g, const uint8_t *mask) {
-    if (C % 8 != 0 || B * C * HW >= (1ll << 40) || HW >= (1ll << 30)) return DBP_EUNSUPPORTED;
+    if (B * C * HW >= (1ll << 40) || HW >= (1ll << 30)) return DBP_EUNSUPPORTED;
     if (mask != nullptr && dtype != DBP_F32) return DBP_EUNSUPPORTED;
     // the stacked copy is written by the path for planes smaller than a tile; the rows of image b start at
     // b (HW + W) however many images make up a tall image: the stacking only adds the zero rows
-    if (codes_stack != nullptr && (HW >= kTP || plane_w <= 0 || stack_g <= 0 || HW + plane_w > kTP)) return DBP_EINVAL;
+    if (codes_stack != nullptr && (HW >= kTP || C % 8 != 0 || plane_w <= 0 || stack_g <= 0 || HW + plane_w > kTP)) return DBP_EINVAL;
     const int b = static_cast<int>(B), c = static_cast<int>(C), hw = static_cast<int>(HW);
     cudaError_t e;
     if (dtype == DBP_F32)

@@ -123,22 +123,36 @@ __device__ __forceinline__ void rows_job(const RowsJob &j, long long first, long
             *reinterpret_cast<uint4 *>(dst) = make_uint4(h[0], h[1], h[2], h[3]);
             *reinterpret_cast<uint4 *>(dst + piece) = make_uint4(l[0], l[1], l[2], l[3]);
         } else {
-            const unsigned short *src = static_cast<const unsigned short *>(j.src) + row * j.cols + c0;
-            unsigned w[4];
+            // 32-bit loads whatever the row's start: a row that starts on an odd element is shifted by half a word
+            const long long off = row * j.cols + c0, total = j.rows * j.cols;
+            const unsigned short *src = static_cast<const unsigned short *>(j.src);
+            const int odd = static_cast<int>(off & 1), nv = left < 8 ? static_cast<int>(left) : 8;
+            unsigned v[5], w[4];
+#pragma unroll
+            for (int e = 0; e < 5; ++e) {
+                const long long i0 = (off & ~1ll) + 2 * e;
+                v[e] = 0u;
+                if (2 * e < odd + nv) v[e] = i0 + 1 < total ? __ldg(reinterpret_cast<const unsigned *>(src + i0)) : __ldg(src + i0);
+            }
 #pragma unroll
             for (int e = 0; e < 4; ++e) {
-                const unsigned a = 2 * e < left ? __ldg(src + 2 * e) : 0u, b = 2 * e + 1 < left ? __ldg(src + 2 * e + 1) : 0u;
-                w[e] = a | (b << 16);
+                w[e] = odd ? __byte_perm(v[e], v[e + 1], 0x5432) : v[e];
+                if (2 * e >= nv) w[e] = 0u;
+                else if (2 * e + 1 >= nv) w[e] &= 0xffffu;
             }
             *reinterpret_cast<uint4 *>(dst) = make_uint4(w[0], w[1], w[2], w[3]);
         }
     }
 }
 
-__global__ void __launch_bounds__(kThreads) rows_job_kernel(const RowsJob j) {
-    chain_wait();
+// beside: the kernel before this one on the stream writes nothing this one reads (the quantizer, whose CTAs let this
+// kernel start once they have seen everything before them complete): it works beside that kernel, whose issue slots are
+// what is busy, and waits for it only before it ends, so that the kernels behind this one still come after both.
+__global__ void __launch_bounds__(kThreads) rows_job_kernel(const RowsJob j, int beside) {
+    if (!beside) chain_wait();
     chain_release();
     rows_job(j, static_cast<long long>(blockIdx.x) * kThreads + threadIdx.x, static_cast<long long>(gridDim.x) * kThreads);
+    if (beside) chain_wait();
 }
 
 template <typename T, bool MASKED = false>
@@ -169,10 +183,11 @@ statistics_kernel(const T *__restrict__ x, long long n, double *__restrict__ par
         const void *w_src = jobs.w_src;
         unsigned short *w_dst = static_cast<unsigned short *>(jobs.w_dst);
         const int w_f32 = jobs.w_f32, w_cin = static_cast<int>(jobs.Cin), w_phase_cin = jobs.phase_cin;
+        const int w_pitch = (w_cin + 7) & ~7;      // rows of a multiple of 16 bytes, for the copy engine
         const long long w_cout = jobs.Cout;
-        const int per_co = 9 * w_cin, taps = w_f32 ? 18 : 9;
+        const int per_co = 9 * w_pitch, taps = w_f32 ? 18 : 9;
         for (long long co = blockIdx.x; co < w_cout; co += gridDim.x) {
-            unsigned short *dst = w_dst + co * taps * w_cin;
+            unsigned short *dst = w_dst + co * taps * w_pitch;
             // a thread takes one channel and all nine taps: nine independent loads, then stores that run along ci
             for (int ci = threadIdx.x; ci < w_cin; ci += kThreads) {
                 int ph = 0;
@@ -200,8 +215,8 @@ statistics_kernel(const T *__restrict__ x, long long n, double *__restrict__ par
                     for (int t = 0; t < 9; ++t) {
                         const __nv_bfloat16 hi = __float2bfloat16_rn(w[t]);
                         const __nv_bfloat16 lo = __float2bfloat16_rn(w[t] - __bfloat162float(hi));
-                        dst[t * w_cin + ci] = *reinterpret_cast<const unsigned short *>(&hi);
-                        dst[per_co + t * w_cin + ci] = *reinterpret_cast<const unsigned short *>(&lo);
+                        dst[t * w_pitch + ci] = *reinterpret_cast<const unsigned short *>(&hi);
+                        dst[per_co + t * w_pitch + ci] = *reinterpret_cast<const unsigned short *>(&lo);
                     }
                 } else {
                     unsigned short w[9];
@@ -209,7 +224,7 @@ statistics_kernel(const T *__restrict__ x, long long n, double *__restrict__ par
                     for (int t = 0; t < 9; ++t)
                         w[t] = k[t] >= 0 ? __ldg(static_cast<const unsigned short *>(w_src) + base + k[t]) : static_cast<unsigned short>(0);
 #pragma unroll
-                    for (int t = 0; t < 9; ++t) dst[t * w_cin + ci] = w[t];
+                    for (int t = 0; t < 9; ++t) dst[t * w_pitch + ci] = w[t];
                 }
             }
         }
@@ -521,17 +536,20 @@ decode_kernel(const uint32_t *__restrict__ bitmap, const uint16_t *__restrict__ 
 
 constexpr int kStatBlocksPerSM = 2;
 
+int launch_rows_job(dbp_ctx *ctx, const RowsJob &job, bool beside) {
+    long long b = (job.rows * (job.pitch / 8) + kThreads - 1) / kThreads;
+    if (b > static_cast<long long>(ctx->sm_count) * 8) b = static_cast<long long>(ctx->sm_count) * 8;
+    return cuda_ok(launch_chained(rows_job_kernel, dim3(static_cast<unsigned>(b)), dim3(kThreads), 0, ctx->stream, job, beside ? 1 : 0));
+}
+
 int launch_statistics(dbp_ctx *ctx, const void *delta, int dtype, long long numel, float scale,
                       const float *delta_in, float *delta_out, unsigned long long *nnz_out, const SideJobs &jobs,
                       const uint8_t *mask) {
     if (mask != nullptr && dtype != DBP_F32) return DBP_EUNSUPPORTED;
     if (!(scale > 0.f)) {      // the step size is given: no statistics kernel, so no side jobs either (the caller sees to the weights)
         if (jobs.zero && cudaMemsetAsync(jobs.zero, 0, jobs.zero_bytes, ctx->stream) != cudaSuccess) return fail_cuda("clearing dW");
-        for (int j = 0; j < jobs.nrows; ++j) {
-            long long b = (jobs.rows[j].rows * (jobs.rows[j].pitch / 8) + kThreads - 1) / kThreads;
-            if (b > static_cast<long long>(ctx->sm_count) * 8) b = static_cast<long long>(ctx->sm_count) * 8;
-            if (int rc = cuda_ok(launch_chained(rows_job_kernel, dim3(static_cast<unsigned>(b)), dim3(kThreads), 0, ctx->stream, jobs.rows[j]))) return rc;
-        }
+        for (int j = 0; j < jobs.nrows; ++j)
+            if (int rc = launch_rows_job(ctx, jobs.rows[j], false)) return rc;
         note_launch();
         set_step_kernel<<<1, 1, 0, ctx->stream>>>(delta_in, ctx->state, delta_out, nnz_out);
         return cuda_ok(cudaGetLastError());

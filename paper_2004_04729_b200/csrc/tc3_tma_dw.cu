@@ -423,82 +423,26 @@ tc3_dw_finish_phases_kernel(float *__restrict__ acc, const float *__restrict__ d
     }
 }
 
-// fp32 activations [B][Cin][HW] -> two bf16 tensors [B][cin_pad][pitch], one after the other: the values rounded
-// to bf16 and what that rounding left over, rounded again (the two pieces add up to the fp32 value to within
-// 2^-18 of it). Rows are padded to `pitch` (a multiple of 8) and channels to cin_pad (a multiple of 8) with zeros.
-// A thread takes eight consecutive positions of one plane: two 16-byte loads where the plane allows it, one 16-byte
-// store per piece.
-__global__ void __launch_bounds__(256)
-x_split_kernel(const float *__restrict__ X, __nv_bfloat16 *__restrict__ out, long long B, int Cin, int cin_pad, int HW, int pitch) {
-    chain_wait();
-    chain_release();
-    const int gpp = pitch / 8;                                   // groups of eight positions per plane
-    const long long planes = B * cin_pad, ngroups = planes * gpp;
-    const long long n = planes * pitch;
-    const bool vec = (HW % 4 == 0);
-    for (long long gi = blockIdx.x * 256ll + threadIdx.x; gi < ngroups; gi += gridDim.x * 256ll) {
-        long long pl;
-        int gq;
-        if ((ngroups >> 31) == 0) {                              // 32-bit divisions cost a fraction of 64-bit ones
-            const unsigned u = static_cast<unsigned>(gi);
-            pl = u / static_cast<unsigned>(gpp);
-            gq = static_cast<int>(u - static_cast<unsigned>(pl) * static_cast<unsigned>(gpp));
-        } else {
-            pl = gi / gpp;
-            gq = static_cast<int>(gi - pl * gpp);
-        }
-        const long long b = pl / cin_pad;
-        const int ci = static_cast<int>(pl - b * cin_pad);
-        const int pp0 = gq * 8;
-        float x[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-        if (ci < Cin && pp0 < HW) {
-            const float *src = X + (b * Cin + ci) * HW + pp0;
-            if (vec) {
-                const float4 v0 = __ldg(reinterpret_cast<const float4 *>(src));
-                x[0] = v0.x; x[1] = v0.y; x[2] = v0.z; x[3] = v0.w;
-                if (pp0 + 4 < HW) {
-                    const float4 v1 = __ldg(reinterpret_cast<const float4 *>(src + 4));
-                    x[4] = v1.x; x[5] = v1.y; x[6] = v1.z; x[7] = v1.w;
-                }
-            } else {
-#pragma unroll
-                for (int i = 0; i < 8; ++i)
-                    if (pp0 + i < HW) x[i] = __ldg(src + i);
-            }
-        }
-        unsigned h[4], l[4];
-#pragma unroll
-        for (int i = 0; i < 4; ++i) {
-            const __nv_bfloat162 hh = __floats2bfloat162_rn(x[2 * i], x[2 * i + 1]);
-            const float2 hf = __bfloat1622float2(hh);
-            const __nv_bfloat162 ll = __floats2bfloat162_rn(x[2 * i] - hf.x, x[2 * i + 1] - hf.y);
-            h[i] = *reinterpret_cast<const unsigned *>(&hh);
-            l[i] = *reinterpret_cast<const unsigned *>(&ll);
-        }
-        const long long o = pl * pitch + pp0;
-        *reinterpret_cast<uint4 *>(out + o) = make_uint4(h[0], h[1], h[2], h[3]);
-        *reinterpret_cast<uint4 *>(out + n + o) = make_uint4(l[0], l[1], l[2], l[3]);
-    }
-}
-
-// The same for tiny planes stacked into tall images (one row of zeros after every image): out is
-// [2][B / G][cin_pad][pitch] with G (H + 1) W positions per tall image; position q of tall image t is position
+// fp32 activations of tiny planes stacked into tall images (one row of zeros after every image), as two bf16 tensors, one
+// after the other: the values rounded to bf16 and what that rounding left over, rounded again. out is
+// [2][B / G][Cin][pitch] with G (H + 1) W positions per tall image; position q of tall image t is position
 // q % ((H + 1) W) of image t G + q / ((H + 1) W), or zero in the extra row and in the padding.
+// beside: see rows_job_kernel (nsd_kernels.cu).
 __global__ void __launch_bounds__(256)
-x_split_stacked_kernel(const float *__restrict__ X, __nv_bfloat16 *__restrict__ out, long long Bt, int G, int Cin, int cin_pad,
-                       int HW, int W, int pitch) {
-    chain_wait();
+x_split_stacked_kernel(const float *__restrict__ X, __nv_bfloat16 *__restrict__ out, long long Bt, int G, int Cin,
+                       int HW, int W, int pitch, int beside) {
+    if (!beside) chain_wait();
     chain_release();
-    const long long n = Bt * cin_pad * pitch;
+    const long long n = Bt * Cin * pitch;
     const int per_img = HW + W;
     for (long long i = blockIdx.x * 256ll + threadIdx.x; i < n; i += gridDim.x * 256ll) {
         const long long pl = i / pitch;
         const int q = static_cast<int>(i - pl * pitch);
-        const long long t = pl / cin_pad;
-        const int ci = static_cast<int>(pl - t * cin_pad);
+        const long long t = pl / Cin;
+        const int ci = static_cast<int>(pl - t * Cin);
         const int g = q / per_img, r = q - g * per_img;
         __nv_bfloat16 hi = __float2bfloat16_rn(0.f), lo = hi;
-        if (g < G && r < HW && ci < Cin) {
+        if (g < G && r < HW) {
             const float x = __ldg(X + ((t * G + g) * Cin + ci) * HW + r);
             hi = __float2bfloat16_rn(x);
             lo = __float2bfloat16_rn(x - __bfloat162float(hi));
@@ -506,6 +450,7 @@ x_split_stacked_kernel(const float *__restrict__ X, __nv_bfloat16 *__restrict__ 
         out[i] = hi;
         out[n + i] = lo;
     }
+    if (beside) chain_wait();
 }
 
 int round_up(int v, int m) { return (v + m - 1) / m * m; }
@@ -515,23 +460,28 @@ int round_up(int v, int m) { return (v + m - 1) / m * m; }
 // DBP_EUNSUPPORTED: the shape does not fit (the caller uses another kernel)
 int tc3_stack_images(const ConvShape &s, int io) {
     const long long HW = s.H * s.W, per_img = HW + s.W;
-    if (io != DBP_F32 || s.k != 3 || HW >= 64 || per_img > 64 || s.B < 2) return 0;
+    if (io != DBP_F32 || s.k != 3 || HW >= 64 || per_img > 64 || s.B < 2 || s.Cout % 8 != 0) return 0;
     // the largest divisor of the batch whose tall image stays within one segment of the kernel
     for (long long g = s.B; g >= 2; --g)
         if (s.B % g == 0 && g * per_img <= 320) return static_cast<int>(g);
     return 0;
 }
 
-// stack_g > 0: `s` describes the tall images (B / G of them, G (H + 1) rows) and the codes are the stacked copy;
-// real_h is the height of one image
-int launch_tc3_tma_dw(dbp_ctx *ctx, const void *codes_nhwc, const void *X, int io, const float *delta_p,
-                      const ConvShape &s, float *dW, int *err_flag, int stack_g, int real_h) {
-    if (!tc3_tma_dw_supported(s, io)) return DBP_EUNSUPPORTED;
-    if (stack_g > 0 && io != DBP_F32) return DBP_EINVAL;
-    const int pieces = io == DBP_F32 ? 2 : 1;
-    // fp32 activations are re-written anyway (split into two bf16 pieces): their channels are padded to a
-    // multiple of 8 on the way, so any Cin works there
-    const long long cin_pad = io == DBP_F32 ? (s.Cin + 7) / 8 * 8 : s.Cin;
+int launch_x_stacked(dbp_ctx *ctx, const float *X, void *out, const ConvShape &s, int stack_g, bool beside) {
+    const long long tall = s.B / stack_g, pitch = (stack_g * (s.H + 1) * s.W + 7) / 8 * 8;
+    long long blocks = (tall * s.Cin * pitch + 255) / 256;
+    if (blocks > ctx->sm_count * 8) blocks = ctx->sm_count * 8;
+    return cuda_ok(launch_chained(x_split_stacked_kernel, dim3(static_cast<unsigned>(blocks)), dim3(256), 0, ctx->stream, X,
+                                  static_cast<__nv_bfloat16 *>(out), tall, stack_g, static_cast<int>(s.Cin), static_cast<int>(s.H * s.W),
+                                  static_cast<int>(s.W), static_cast<int>(pitch), beside ? 1 : 0));
+}
+
+// X: bf16 planes of x_pitch values (a multiple of 8); fp32 activations as two pieces (as if the batch were twice as long).
+// Tiny planes stacked into tall images: `s` describes the tall images and codes and X are their stacked copies.
+int launch_tc3_tma_dw(dbp_ctx *ctx, const void *codes_nhwc, const void *X, int pieces, long long x_pitch, const float *delta_p,
+                      const ConvShape &s, float *dW, int *err_flag) {
+    // the scratch's rows are padded to a multiple of 16 bytes
+    const long long cin_pad = (s.Cin + 7) / 8 * 8, q_pitch = (s.Cout + 7) / 8 * 8;
     const long long HW = s.H * s.W;
     Dw3T p{};
     p.Cin = static_cast<int>(cin_pad); p.Cout = static_cast<int>(s.Cout); p.W = static_cast<int>(s.W); p.HW = static_cast<int>(HW);
@@ -562,7 +512,7 @@ int launch_tc3_tma_dw(dbp_ctx *ctx, const void *codes_nhwc, const void *X, int i
     p.nseg = s.B * pieces * p.segs_per_img;
     // a stride-2 layer on phase images whose phases are whole channel tiles: 6 of the 12 (phase, kernel column)
     // pairs carry taps of the strided layer
-    p.phase_tiles = (ctx->phase_cin > 0 && ctx->phase_cin % 128 == 0 && cin_pad == 4ll * ctx->phase_cin && stack_g == 0)
+    p.phase_tiles = (ctx->phase_cin > 0 && ctx->phase_cin % 128 == 0 && cin_pad == 4ll * ctx->phase_cin)
                         ? ctx->phase_cin / 128 : 0;
     const long long tiles = p.phase_tiles > 0 ? static_cast<long long>(p.co_tiles) * 6 * p.phase_tiles
                                               : static_cast<long long>(p.ci_tiles) * p.co_tiles * 3;
@@ -580,37 +530,6 @@ int launch_tc3_tma_dw(dbp_ctx *ctx, const void *codes_nhwc, const void *X, int i
     }
     float *acc = static_cast<float *>(ctx->dw_acc.ptr);
     p.stage_chunks = static_cast<int>((smem - 1024) / 16384);
-    // fp32 activations are split into two bf16 pieces (as if the batch were twice as long); bf16 ones whose
-    // planes do not start on 16-byte boundaries are first copied to padded planes
-    const void *Xsrc = X;
-    long long xpitch = HW;
-    if (io == DBP_F32) {
-        xpitch = (HW + 7) / 8 * 8;
-        const long long planes = s.B * cin_pad;
-        if ((rc = ws_reserve(ctx, ctx->x_padded, static_cast<size_t>(planes) * xpitch * 2 * 2))) return rc;
-        long long blocks = (planes * (xpitch / 8) + 255) / 256;
-        if (blocks > ctx->sm_count * 16) blocks = ctx->sm_count * 16;
-        if (stack_g > 0) {
-            blocks = (planes * xpitch + 255) / 256;
-            if (blocks > ctx->sm_count * 16) blocks = ctx->sm_count * 16;
-            rc = cuda_ok(launch_chained(x_split_stacked_kernel, dim3(static_cast<unsigned>(blocks)), dim3(256), 0, ctx->stream,
-                                        static_cast<const float *>(X), static_cast<__nv_bfloat16 *>(ctx->x_padded.ptr), s.B, stack_g,
-                                        static_cast<int>(s.Cin), static_cast<int>(cin_pad), static_cast<int>(real_h * s.W),
-                                        static_cast<int>(s.W), static_cast<int>(xpitch)));
-        } else {
-            rc = cuda_ok(launch_chained(x_split_kernel, dim3(static_cast<unsigned>(blocks)), dim3(256), 0, ctx->stream,
-                                        static_cast<const float *>(X), static_cast<__nv_bfloat16 *>(ctx->x_padded.ptr), s.B,
-                                        static_cast<int>(s.Cin), static_cast<int>(cin_pad), static_cast<int>(HW), static_cast<int>(xpitch)));
-        }
-        if (rc) return rc;
-        Xsrc = ctx->x_padded.ptr;
-    } else if (HW % 8 != 0) {
-        xpitch = (HW + 7) / 8 * 8;
-        if ((rc = ws_reserve(ctx, ctx->x_padded, static_cast<size_t>(s.B) * s.Cin * xpitch * 2))) return rc;
-        if ((rc = launch_pad_planes(ctx, X, ctx->x_padded.ptr, s.B * s.Cin, 1, static_cast<int>(HW), static_cast<int>(xpitch))))
-            return rc;
-        Xsrc = ctx->x_padded.ptr;
-    }
     CUtensorMap map_q, map_x, map_acc;
     {
         const unsigned long long dims[2] = {static_cast<unsigned long long>(cin_pad), static_cast<unsigned long long>(s.Cout) * 9};
@@ -621,18 +540,18 @@ int launch_tc3_tma_dw(dbp_ctx *ctx, const void *codes_nhwc, const void *X, int i
     {
         const unsigned long long dims[3] = {static_cast<unsigned long long>(s.Cout), static_cast<unsigned long long>(HW),
                                             static_cast<unsigned long long>(s.B)};
-        const unsigned long long str[2] = {static_cast<unsigned long long>(s.Cout) * 2,
-                                           static_cast<unsigned long long>(s.Cout) * 2 * HW};
+        const unsigned long long str[2] = {static_cast<unsigned long long>(q_pitch) * 2,
+                                           static_cast<unsigned long long>(q_pitch) * 2 * HW};
         const unsigned box[3] = {64, static_cast<unsigned>(p.rows_box), 1};
         if (!encode_map_bf16(&map_q, codes_nhwc, 3, dims, str, box)) return fail_cuda("tensor map of the code panels");
     }
     {
-        const unsigned long long dims[3] = {static_cast<unsigned long long>(HW), static_cast<unsigned long long>(cin_pad),
+        const unsigned long long dims[3] = {static_cast<unsigned long long>(HW), static_cast<unsigned long long>(s.Cin),
                                             static_cast<unsigned long long>(s.B) * pieces};
-        const unsigned long long str[2] = {static_cast<unsigned long long>(xpitch) * 2,
-                                           static_cast<unsigned long long>(xpitch) * 2 * cin_pad};
+        const unsigned long long str[2] = {static_cast<unsigned long long>(x_pitch) * 2,
+                                           static_cast<unsigned long long>(x_pitch) * 2 * s.Cin};
         const unsigned box[3] = {64, 128, 1};
-        if (!encode_map_bf16(&map_x, Xsrc, 3, dims, str, box)) return fail_cuda("tensor map of the activations");
+        if (!encode_map_bf16(&map_x, X, 3, dims, str, box)) return fail_cuda("tensor map of the activations");
     }
     auto kern = NP == 2 ? tc3_tma_dw_kernel<2> : tc3_tma_dw_kernel<1>;
     if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem)) != cudaSuccess)

@@ -360,33 +360,24 @@ tc3_tma_dx_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
     }
 }
 
-// weights [Cout][Cin][3][3] -> [Cout][9][Cin] (the tap's [co][ci] matrix with ci contiguous)
+// weights [Cout][Cin][3][3] -> [Cout][9][pitch] bf16 (the tap's [co][ci] matrix with ci contiguous, the row pitch a
+// multiple of 8). fp32 weights -> [Cout][18][pitch]: taps 0-8 hold the values rounded to bf16, taps 9-17 what that
+// rounding left over, rounded to bf16 again. The sum of the two pieces differs from the fp32 value by at most 2^-18 of
+// it, and a code times a piece is exact in the fp32 accumulator. Used when the step size is given; otherwise the
+// statistics kernel does this on the side.
+template <typename T>
 __global__ void __launch_bounds__(256)
-w_taps_bf16_kernel(const unsigned short *__restrict__ W, unsigned short *__restrict__ out, long long Cout, long long Cin) {
+w_taps_rows_kernel(const T *__restrict__ W, __nv_bfloat16 *__restrict__ out, long long Cout, long long Cin, long long pitch) {
     chain_wait();
     chain_release();
+    constexpr int TAPS = sizeof(T) == 4 ? 18 : 9;
     const long long n = Cout * Cin * 9;
     for (long long i = blockIdx.x * 256ll + threadIdx.x; i < n; i += gridDim.x * 256ll) {
         const long long ci = i % Cin, t = (i / Cin) % 9, co = i / (Cin * 9);
-        out[i] = __ldg(W + (co * Cin + ci) * 9 + t);
-    }
-}
-
-// fp32 weights -> [Cout][18][Cin] bf16: taps 0-8 hold the values rounded to bf16, taps 9-17 what that
-// rounding left over, rounded to bf16 again. The sum of the two pieces differs from the fp32 value by
-// at most 2^-18 of it, and a code times a piece is exact in the fp32 accumulator.
-__global__ void __launch_bounds__(256)
-w_taps_split_kernel(const float *__restrict__ W, __nv_bfloat16 *__restrict__ out, long long Cout, long long Cin) {
-    chain_wait();
-    chain_release();
-    const long long n = Cout * Cin * 9;
-    for (long long i = blockIdx.x * 256ll + threadIdx.x; i < n; i += gridDim.x * 256ll) {
-        const long long ci = i % Cin, t = (i / Cin) % 9, co = i / (Cin * 9);
-        const float w = __ldg(W + (co * Cin + ci) * 9 + t);
+        const float w = static_cast<float>(W[(co * Cin + ci) * 9 + t]);
         const __nv_bfloat16 hi = __float2bfloat16_rn(w);
-        const __nv_bfloat16 lo = __float2bfloat16_rn(w - __bfloat162float(hi));
-        out[(co * 18 + t) * Cin + ci] = hi;
-        out[(co * 18 + 9 + t) * Cin + ci] = lo;
+        out[(co * TAPS + t) * pitch + ci] = hi;
+        if (TAPS == 18) out[(co * TAPS + 9 + t) * pitch + ci] = __float2bfloat16_rn(w - __bfloat162float(hi));
     }
 }
 
@@ -394,21 +385,10 @@ int round_up(int v, int m) { return (v + m - 1) / m * m; }
 
 }  // namespace
 
-// Shapes the TMA-fed 3x3 kernels take: channel counts that keep every row of the position-major
-// codes, of the re-laid weights and of the activations on 16-byte boundaries. fp32 operands are
-// split into two bf16 pieces each (the codes are exact in bf16), so they take the same kernels.
+// Shapes the TMA-fed 3x3 kernels take. fp32 operands are split into two bf16 pieces each (the codes are exact in bf16);
+// rows of the codes, of the re-laid weights and of the activations that are no multiple of 16 bytes are padded to one.
 bool tc3_tma_supported(const ConvShape &s, int io) {
-    return (io == DBP_BF16 || io == DBP_F32) && s.k == 3 && s.Cin % 8 == 0 && s.Cout % 8 == 0 && s.W >= 1 && s.W <= 62 &&
-           s.H <= 4096 && s.B * s.H * s.W < (1ll << 30);
-}
-
-// The weight-gradient kernel alone also takes fp32 layers whose input channel count is no multiple of 8 (a
-// network's first layer): its activations are re-written channel-padded anyway.
-bool tc3_tma_dw_supported(const ConvShape &s, int io) {
-    if (tc3_tma_supported(s, io)) return true;
-    ConvShape t = s;
-    t.Cin = (s.Cin + 7) / 8 * 8;
-    return io == DBP_F32 && tc3_tma_supported(t, io);
+    return (io == DBP_BF16 || io == DBP_F32) && s.k == 3 && s.W >= 1 && s.W <= 62 && s.H <= 4096 && s.B * s.H * s.W < (1ll << 30);
 }
 
 // DBP_EUNSUPPORTED: the shape does not fit (the caller uses another kernel)
@@ -493,36 +473,36 @@ int launch_tc3_tma_dx(dbp_ctx *ctx, const void *codes_nhwc, const void *W, int i
     const size_t smem = fixed + static_cast<size_t>(p.nw) * p.w_slot;
 
     // re-laid weights
-    const size_t wb = sizeof(__nv_bfloat16) * static_cast<size_t>(s.Cout) * s.Cin * p.ntaps;
+    const long long w_pitch = (s.Cin + 7) / 8 * 8, q_pitch = (s.Cout + 7) / 8 * 8;
+    const size_t wb = sizeof(__nv_bfloat16) * static_cast<size_t>(s.Cout) * w_pitch * p.ntaps;
     int rc = ws_reserve(ctx, ctx->w_taps, wb);
     if (rc) return rc;
     if (!weights_ready) {
         long long blocks = (static_cast<long long>(s.Cout) * s.Cin * 9 + 255) / 256;
         if (blocks > sms * 8) blocks = sms * 8;
+        __nv_bfloat16 *taps = static_cast<__nv_bfloat16 *>(ctx->w_taps.ptr);
         if (io == DBP_F32)
-            rc = cuda_ok(launch_chained(w_taps_split_kernel, dim3(static_cast<unsigned>(blocks)), dim3(256), 0, ctx->stream,
-                                        static_cast<const float *>(W), static_cast<__nv_bfloat16 *>(ctx->w_taps.ptr), s.Cout, s.Cin));
+            rc = cuda_ok(launch_chained(w_taps_rows_kernel<float>, dim3(static_cast<unsigned>(blocks)), dim3(256), 0, ctx->stream,
+                                        static_cast<const float *>(W), taps, s.Cout, s.Cin, w_pitch));
         else
-            rc = cuda_ok(launch_chained(w_taps_bf16_kernel, dim3(static_cast<unsigned>(blocks)), dim3(256), 0, ctx->stream,
-                                        static_cast<const unsigned short *>(W), static_cast<unsigned short *>(ctx->w_taps.ptr),
-                                        s.Cout, s.Cin));
+            rc = cuda_ok(launch_chained(w_taps_rows_kernel<__nv_bfloat16>, dim3(static_cast<unsigned>(blocks)), dim3(256), 0, ctx->stream,
+                                        static_cast<const __nv_bfloat16 *>(W), taps, s.Cout, s.Cin, w_pitch));
         if (rc) return rc;
     }
     CUtensorMap map_q, map_w;
     {
         const unsigned long long dims[4] = {static_cast<unsigned long long>(s.Cout), static_cast<unsigned long long>(s.W),
                                             static_cast<unsigned long long>(s.H), static_cast<unsigned long long>(s.B)};
-        const unsigned long long str[3] = {static_cast<unsigned long long>(s.Cout) * 2,
-                                           static_cast<unsigned long long>(s.Cout) * 2 * s.W,
-                                           static_cast<unsigned long long>(s.Cout) * 2 * s.W * s.H};
+        const unsigned long long row = static_cast<unsigned long long>(q_pitch) * 2;
+        const unsigned long long str[3] = {row, row * s.W, row * s.W * s.H};
         const unsigned box[4] = {64, static_cast<unsigned>(p.Wp), static_cast<unsigned>(p.Ht + 2), static_cast<unsigned>(p.nb)};
         if (!encode_map_bf16(&map_q, codes_nhwc, 4, dims, str, box)) return fail_cuda("tensor map of the code patches");
     }
     {
         const unsigned long long dims[3] = {static_cast<unsigned long long>(s.Cin), static_cast<unsigned long long>(p.ntaps),
                                             static_cast<unsigned long long>(s.Cout)};
-        const unsigned long long str[2] = {static_cast<unsigned long long>(s.Cin) * 2,
-                                           static_cast<unsigned long long>(s.Cin) * 2 * p.ntaps};
+        const unsigned long long str[2] = {static_cast<unsigned long long>(w_pitch) * 2,
+                                           static_cast<unsigned long long>(w_pitch) * 2 * p.ntaps};
         const unsigned box[3] = {64, 1, 64};
         if (!encode_map_bf16(&map_w, ctx->w_taps.ptr, 3, dims, str, box)) return fail_cuda("tensor map of the weights");
     }

@@ -25,9 +25,12 @@ constexpr int kStageW = 32 * 128;                // one warp's staged 32 x 32 fp
 
 struct DwT {
     const float *delta_p;
+    float *dW;
+    int tma_out;                  // rows of dW are multiples of 16 bytes: blocks are added by the copy engine, else by atomics
+    int code_batch;               // images of the code tensor (fp32 activations are two pieces of every image, one after the other)
     int Cin, Cout, HW;
     int cpi;                      // 64-position chunks per image
-    long long nchunks;            // B * cpi
+    long long nchunks;            // images of the activation tensor * cpi
     int ci_tiles, nsplit;
     long long per_split;          // chunks per CTA
     int NT, NTp, MA, stages;      // ci tile, its accumulator stride (multiple of 32), accumulators
@@ -68,7 +71,7 @@ tma_dw_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant__
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         tma_prefetch_desc(&map_q);
         tma_prefetch_desc(&map_x);
-        tma_prefetch_desc(&map_dw);
+        if (p.tma_out) tma_prefetch_desc(&map_dw);
     }
     if (warp == 1) tmem_alloc(&pipe.tmem_base, p.tmem_cols);
     tc_fence_before();
@@ -90,8 +93,9 @@ tma_dw_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant__
                 if (!mbar_wait_timed(&pipe.empty[s], parity, p.err_flag, waited)) break;
                 unsigned char *st = smem + s * stage_bytes;
                 mbar_expect_tx(&pipe.full[s], bytes);
+                const int bq = static_cast<int>(b % p.code_batch);
                 for (int a = 0; a < p.MA; ++a)
-                    tma_load_3d(st + a * kATile, &map_q, c * 64, co0 + a * 128, static_cast<int>(b), &pipe.full[s]);
+                    tma_load_3d(st + a * kATile, &map_q, c * 64, co0 + a * 128, bq, &pipe.full[s]);
                 tma_load_3d(st + p.MA * kATile, &map_x, c * 64, ci0, static_cast<int>(b), &pipe.full[s]);
                 if (++c == p.cpi) { c = 0; ++b; }
                 if (++s == S) { s = 0; parity ^= 1u; }
@@ -163,6 +167,18 @@ tma_dw_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant__
                         *reinterpret_cast<float4 *>(stage + lane * 128 + ((j ^ (lane & 7)) << 4)) =
                             make_float4(__uint_as_float(v[4 * j]) * delta, __uint_as_float(v[4 * j + 1]) * delta,
                                         __uint_as_float(v[4 * j + 2]) * delta, __uint_as_float(v[4 * j + 3]) * delta);
+                    if (!p.tma_out) {
+                        __syncwarp();
+                        const int nr = p.Cout - co_w < 32 ? p.Cout - co_w : 32;
+                        const int ci = ci0 + c0 + lane;
+                        float *dst = p.dW + static_cast<long long>(co_w) * p.Cin + ci;
+                        if (ci < p.Cin)
+                            for (int r = 0; r < nr; ++r)
+                                atomicAdd(dst + static_cast<long long>(r) * p.Cin,
+                                          *reinterpret_cast<const float *>(stage + r * 128 + (((lane >> 2) ^ (r & 7)) << 4) + (lane & 3) * 4));
+                        __syncwarp();
+                        continue;
+                    }
                     fence_async_proxy();
                     __syncwarp();
                     // rows past Cout and columns past Cin are skipped by the engine
@@ -186,19 +202,15 @@ tma_dw_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant__
 
 }  // namespace
 
-bool tma_dw_supported(const ConvShape &s, int io) {
-    const long long HW = s.H * s.W;
-    return io == DBP_BF16 && s.k == 1 && s.Cin % 8 == 0 && HW >= 16 && HW < (1ll << 30) &&
-           s.B * ((HW + 63) / 64) >= 4;
-}
-
-int launch_tma_dw(dbp_ctx *ctx, const void *codes_bf16, const void *X, const float *delta_p,
+// X: bf16 planes of x_pitch values (a multiple of 8), pieces of every image one after the other
+int launch_tma_dw(dbp_ctx *ctx, const void *codes_bf16, const void *X, int pieces, long long x_pitch, const float *delta_p,
                   const ConvShape &s, float *dW, int *err_flag) {
     const long long HW = s.H * s.W, pitch = tma_code_pitch(s);
     DwT p{};
     p.Cin = static_cast<int>(s.Cin); p.Cout = static_cast<int>(s.Cout); p.HW = static_cast<int>(HW);
     p.cpi = static_cast<int>((HW + 63) / 64);
-    p.nchunks = s.B * p.cpi;
+    p.code_batch = static_cast<int>(s.B);
+    p.nchunks = s.B * pieces * p.cpi;
     p.NT = s.Cin >= 256 ? 256 : static_cast<int>((s.Cin + 15) / 16 * 16);
     p.NTp = (p.NT + 31) / 32 * 32;
     p.MA = s.Cout > 128 ? 2 : 1;
@@ -209,25 +221,22 @@ int launch_tma_dw(dbp_ctx *ctx, const void *codes_bf16, const void *X, const flo
     const long long co_tiles = (s.Cout + 128 * p.MA - 1) / (128 * p.MA);
     const long long tiles = co_tiles * p.ci_tiles;
     long long per = 0;
-    const long long nsplit = choose_split(tiles, p.nchunks, ctx->sm_count, &per);
+    long long nsplit = choose_split(tiles, p.nchunks, ctx->sm_count, &per);
+    // an accumulator is truncated, not rounded, when an MMA adds to it (about 1e-8 of its value per MMA): an fp32 layer's
+    // parts are kept to 128 chunks of four MMAs
+    if (pieces == 2 && per > 128) {
+        per = 128;
+        nsplit = (p.nchunks + per - 1) / per;
+    }
     p.nsplit = static_cast<int>(nsplit);
     p.per_split = per;
     p.err_flag = err_flag;
     p.stats = ctx->wait_stats;
     p.delta_p = delta_p;
-    int rc = DBP_OK;
-    // activations whose planes do not start on 16-byte boundaries are first copied to padded planes
-    const void *Xsrc = X;
-    long long xpitch = HW;
-    if (HW % 8 != 0) {
-        xpitch = pitch;
-        if ((rc = ws_reserve(ctx, ctx->x_padded, static_cast<size_t>(s.B) * s.Cin * xpitch * 2))) return rc;
-        if ((rc = launch_pad_planes(ctx, X, ctx->x_padded.ptr, s.B * s.Cin, 1, static_cast<int>(HW), static_cast<int>(xpitch))))
-            return rc;
-        Xsrc = ctx->x_padded.ptr;
-    }
-    CUtensorMap map_q, map_x, map_dw;
-    {
+    CUtensorMap map_q, map_x, map_dw{};
+    p.dW = dW;
+    p.tma_out = s.Cin % 4 == 0 ? 1 : 0;
+    if (p.tma_out) {
         const unsigned long long dims[2] = {static_cast<unsigned long long>(s.Cin), static_cast<unsigned long long>(s.Cout)};
         const unsigned long long str[1] = {static_cast<unsigned long long>(s.Cin) * 4};
         const unsigned box[2] = {32, 32};
@@ -243,11 +252,11 @@ int launch_tma_dw(dbp_ctx *ctx, const void *codes_bf16, const void *X, const flo
     }
     {
         const unsigned long long dims[3] = {static_cast<unsigned long long>(HW), static_cast<unsigned long long>(s.Cin),
-                                            static_cast<unsigned long long>(s.B)};
-        const unsigned long long str[2] = {static_cast<unsigned long long>(xpitch) * 2,
-                                           static_cast<unsigned long long>(xpitch) * 2 * s.Cin};
+                                            static_cast<unsigned long long>(s.B) * pieces};
+        const unsigned long long str[2] = {static_cast<unsigned long long>(x_pitch) * 2,
+                                           static_cast<unsigned long long>(x_pitch) * 2 * s.Cin};
         const unsigned box[3] = {64, static_cast<unsigned>(p.NT), 1};
-        if (!encode_map_bf16(&map_x, Xsrc, 3, dims, str, box)) return DBP_ECUDA;
+        if (!encode_map_bf16(&map_x, X, 3, dims, str, box)) return fail_cuda("tensor map of the activations");
     }
     const size_t smem = static_cast<size_t>(p.stages) * (p.MA * kATile + kBMax) + 1024;       // >= 4 warps x 4 staging blocks
     if (cudaFuncSetAttribute(tma_dw_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem)) != cudaSuccess)
@@ -255,58 +264,6 @@ int launch_tma_dw(dbp_ctx *ctx, const void *codes_bf16, const void *X, const flo
     // dW has been cleared by this layer's statistics kernel
     return cuda_ok(launch_chained(tma_dw_kernel, dim3(static_cast<unsigned>(tiles * nsplit)), dim3(kThreadsW), smem,
                                   ctx->stream, map_q, map_x, map_dw, p));
-}
-
-}  // namespace dbp
-
-namespace dbp {
-
-namespace {
-
-// Copies planes of H x W bf16 values into rows of Wp >= W values (Wp a multiple of 8), the extra
-// columns zero, so that every row of every plane starts on a 16-byte boundary: the copy engine
-// cannot address planes whose pitch is not a multiple of 16 bytes.
-__global__ void __launch_bounds__(256)
-pad_planes_kernel(const unsigned short *__restrict__ in, unsigned short *__restrict__ out, long long planes,
-                  int H, int W, int Wp) {
-    const int groups_per_row = Wp / 8;
-    const long long ngroups = planes * H * groups_per_row;
-    chain_wait();
-    chain_release();
-    for (long long g = blockIdx.x * 256ll + threadIdx.x; g < ngroups; g += gridDim.x * 256ll) {
-        const long long row = g / groups_per_row;           // (plane, y)
-        const int x0 = static_cast<int>(g - row * groups_per_row) * 8;
-        const unsigned short *src = in + row * W + x0;
-        unsigned short v[8];
-        if ((W & 3) == 0 && x0 + 8 <= W) {          // rows start on 8-byte boundaries: two 8-byte loads
-            const uint2 a = __ldg(reinterpret_cast<const uint2 *>(src)), b = __ldg(reinterpret_cast<const uint2 *>(src + 4));
-            v[0] = static_cast<unsigned short>(a.x); v[1] = static_cast<unsigned short>(a.x >> 16);
-            v[2] = static_cast<unsigned short>(a.y); v[3] = static_cast<unsigned short>(a.y >> 16);
-            v[4] = static_cast<unsigned short>(b.x); v[5] = static_cast<unsigned short>(b.x >> 16);
-            v[6] = static_cast<unsigned short>(b.y); v[7] = static_cast<unsigned short>(b.y >> 16);
-        } else {
-#pragma unroll
-            for (int j = 0; j < 8; ++j) v[j] = (x0 + j < W) ? __ldg(src + j) : static_cast<unsigned short>(0);
-        }
-        uint4 o;
-        o.x = v[0] | (static_cast<unsigned>(v[1]) << 16);
-        o.y = v[2] | (static_cast<unsigned>(v[3]) << 16);
-        o.z = v[4] | (static_cast<unsigned>(v[5]) << 16);
-        o.w = v[6] | (static_cast<unsigned>(v[7]) << 16);
-        *reinterpret_cast<uint4 *>(out + row * Wp + x0) = o;
-    }
-}
-
-}  // namespace
-
-int launch_pad_planes(dbp_ctx *ctx, const void *in, void *out, long long planes, int H, int W, int Wp) {
-    const long long ngroups = planes * H * (Wp / 8);
-    long long blocks = (ngroups + 255) / 256;
-    const long long cap = static_cast<long long>(ctx->sm_count) * 16;
-    if (blocks > cap) blocks = cap;
-    if (blocks < 1) blocks = 1;
-    return cuda_ok(launch_chained(pad_planes_kernel, dim3(static_cast<unsigned>(blocks)), dim3(256), 0, ctx->stream,
-                                  static_cast<const unsigned short *>(in), static_cast<unsigned short *>(out), planes, H, W, Wp));
 }
 
 }  // namespace dbp

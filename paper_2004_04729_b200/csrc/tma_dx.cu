@@ -86,11 +86,12 @@ struct DxT {
     const float *delta_p;
     void *dX;                     // [B][Cin][HW], bf16 or fp32
     int dx_f32;
-    int tma_out;                  // bf16 dX whose rows are multiples of 16 bytes: chunks leave through the copy engine
+    int tma_out;                  // rows of dX are multiples of 16 bytes: chunks leave through the copy engine
     int Cin, Cout, HW;
     int chunks_per_img;
     long long nchunks;            // B * chunks_per_img
-    int ci_tiles, ksteps;
+    int ci_tiles, ksteps;         // ksteps: 64-channel steps of the reduction, over all pieces of the weights
+    int ks_piece, pieces;         // fp32 weights come as two bf16 pieces: the codes are then gone through twice
     int nct;                      // 64-position chunks per tile (4, or fewer when that gives too few tiles)
     int MA;                       // accumulators per tile: 1 (128 channels, two tiles in flight) or 2 (256 channels)
     long long ntiles;             // tiles are taken from the last one down: the quantizer has just written the codes front to
@@ -161,13 +162,15 @@ tma_dx_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constant__
                     if (!ok) break;
                     if (elect_one()) {
                         unsigned char *st = smem + s * stage_bytes;
+                        // the low pieces first: the accumulator is still small when they are added
+                        const int kp = ks / p.ks_piece, co0 = (ks - kp * p.ks_piece) * 64;
                         mbar_expect_tx(&pipe.full[s], tx);
                         for (int h = 0; h < 2 * MA; ++h)
-                            tma_load_2d(st + h * kPanel, &map_w, ci0 + 64 * h, ks * 64, &pipe.full[s]);
+                            tma_load_3d(st + h * kPanel, &map_w, ci0 + 64 * h, co0, p.pieces - 1 - kp, &pipe.full[s]);
                         st += a_bytes;
                         int b = b0, c = c0;
                         for (int i = 0; i < nch; ++i, st += kPanel) {
-                            tma_load_3d(st, &map_q, c * 64, ks * 64, b, &pipe.full[s]);
+                            tma_load_3d(st, &map_q, c * 64, co0, b, &pipe.full[s]);
                             if (++c == p.chunks_per_img) { c = 0; ++b; }
                         }
                     }
@@ -238,7 +241,6 @@ tma_dx_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constant__
             const int a = slot0 + am;
             const long long tr = p.ntiles - 1 - t;
             const int ci_w = (static_cast<int>(tr % p.ci_tiles) * MA + am) * 128 + q * 32;
-            const int ci = ci_w + lane;
             const long long g0 = (tr / p.ci_tiles) * p.nct;
             const int nch = static_cast<int>(p.nchunks - g0 < p.nct ? p.nchunks - g0 : p.nct);
             ok = mbar_wait_timed(&pipe.acc_full[a], uses & 1u, p.err_flag, we);
@@ -247,7 +249,7 @@ tma_dx_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constant__
             for (int c = part; c < nch; c += kEpiWarps / 4) {
                 const long long b = (g0 + c) / p.chunks_per_img;
                 const int p0 = static_cast<int>((g0 + c) % p.chunks_per_img) * 64;
-                if (p.tma_out) {
+                if (p.tma_out && !p.dx_f32) {
                     // the chunk's 32 channels x 64 positions: both halves out of TMEM, scaled and rounded, into the
                     // staging block as swizzled 128-byte rows, then one tiled store (which skips what lies
                     // outside the tensor). The block is free again once the previous store has read it.
@@ -295,22 +297,30 @@ tma_dx_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constant__
                     if (pp >= p.HW) break;                         // warp-uniform
                     unsigned v[32];
                     tmem_ld32(tmem_base + (static_cast<unsigned>(q * 32) << 16) + a * kAccCols + c * 64 + half * 32, v);
-                    if (ci >= p.Cin && p.dx_f32) continue;
-                    const long long o = (b * p.Cin + ci) * p.HW + pp;
                     const int nval = p.HW - pp < 32 ? p.HW - pp : 32;
                     if (p.dx_f32) {
-                        float *dst = static_cast<float *>(p.dX) + o;
-                        if (vw >= 4) {
+                        // 32 channels x 32 positions as swizzled 128-byte rows: one tiled store, or lanes along the positions
+                        if (p.tma_out && lane == 0) bulk_wait_read_all();
+                        __syncwarp();
 #pragma unroll
-                            for (int j = 0; j < 32; j += 4)
-                                if (j < nval)
-                                    *reinterpret_cast<float4 *>(dst + j) =
-                                        make_float4(__uint_as_float(v[j]) * delta, __uint_as_float(v[j + 1]) * delta,
-                                                    __uint_as_float(v[j + 2]) * delta, __uint_as_float(v[j + 3]) * delta);
+                        for (int j = 0; j < 8; ++j)
+                            *reinterpret_cast<float4 *>(stage + lane * 128 + ((j ^ (lane & 7)) << 4)) =
+                                make_float4(__uint_as_float(v[4 * j]) * delta, __uint_as_float(v[4 * j + 1]) * delta,
+                                            __uint_as_float(v[4 * j + 2]) * delta, __uint_as_float(v[4 * j + 3]) * delta);
+                        if (p.tma_out) fence_async_proxy();
+                        __syncwarp();
+                        if (p.tma_out) {
+                            if (lane == 0 && ci_w < p.Cin) {
+                                tma_store_3d(&map_dx, pp, ci_w, static_cast<int>(b), stage);
+                                bulk_commit();
+                            }
                         } else {
-#pragma unroll
-                            for (int j = 0; j < 32; ++j)
-                                if (j < nval) dst[j] = __uint_as_float(v[j]) * delta;
+                            const int nr = p.Cin - ci_w < 32 ? p.Cin - ci_w : 32;
+                            float *dst = static_cast<float *>(p.dX) + (b * p.Cin + ci_w) * p.HW + pp + lane;
+                            for (int r = 0; r < nr; ++r)
+                                if (lane < nval)
+                                    dst[static_cast<long long>(r) * p.HW] =
+                                        *reinterpret_cast<const float *>(stage + r * 128 + (((lane >> 2) ^ (r & 7)) << 4) + (lane & 3) * 4);
                         }
                     } else {
                         // bf16: my 32 values go to the warp's staging block, which holds the chunk
@@ -359,7 +369,7 @@ tma_dx_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constant__
                                     *reinterpret_cast<uint2 *>(base + static_cast<long long>(r) * p.HW + pc * 4) =
                                         *reinterpret_cast<const uint2 *>(stage + r * 128 + (((pc >> 1) ^ (r & 7)) << 4) + (pc & 1) * 8);
                             }
-                        } else if (p.chunks_per_img == 1) {
+                        } else if (p.chunks_per_img == 1 && (p.Cin & 7) == 0) {
                             const int n16 = nrows * nv / 8;          // nrows is a multiple of 8: whole 16-byte pieces
                             for (int i = lane; i < n16; i += 32)
                                 reinterpret_cast<uint4 *>(base)[i] = reinterpret_cast<const uint4 *>(stage)[i];
@@ -399,21 +409,25 @@ tma_dx_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constant__
 
 }  // namespace
 
+// An accumulator is truncated, not rounded, when an MMA adds to it (about 1e-8 of its value per MMA): the reduction of
+// an fp32 layer is kept to 8192 channels here.
 bool tma_dx_supported(const ConvShape &s, int io) {
-    return io == DBP_BF16 && s.k == 1 && s.Cin % 8 == 0 && s.H * s.W >= 16 && s.H * s.W < (1ll << 30);
+    return s.k == 1 && s.H * s.W > 1 && s.H * s.W < (1ll << 30) && (io == DBP_BF16 || s.Cout <= 8192);
 }
 
 long long tma_code_pitch(const ConvShape &s) { return (s.H * s.W + 7) / 8 * 8; }
 
-int launch_tma_dx(dbp_ctx *ctx, const void *codes_bf16, const void *W, const float *delta_p,
+int launch_tma_dx(dbp_ctx *ctx, const void *codes_bf16, const void *W, int pieces, long long w_pitch, const float *delta_p,
                   const ConvShape &s, void *dX, bool dx_bf16, int *err_flag) {
     const long long HW = s.H * s.W, pitch = tma_code_pitch(s);
     CUtensorMap map_w, map_q;
     {
-        const unsigned long long dims[2] = {static_cast<unsigned long long>(s.Cin), static_cast<unsigned long long>(s.Cout)};
-        const unsigned long long str[1] = {static_cast<unsigned long long>(s.Cin) * 2};
-        const unsigned box[2] = {64, 64};
-        if (!encode_map_bf16(&map_w, W, 2, dims, str, box)) return DBP_ECUDA;
+        const unsigned long long dims[3] = {static_cast<unsigned long long>(s.Cin), static_cast<unsigned long long>(s.Cout),
+                                            static_cast<unsigned long long>(pieces)};
+        const unsigned long long str[2] = {static_cast<unsigned long long>(w_pitch) * 2,
+                                           static_cast<unsigned long long>(w_pitch) * 2 * s.Cout};
+        const unsigned box[3] = {64, 64, 1};
+        if (!encode_map_bf16(&map_w, W, 3, dims, str, box)) return fail_cuda("tensor map of the weights");
     }
     {
         const unsigned long long dims[3] = {static_cast<unsigned long long>(HW), static_cast<unsigned long long>(s.Cout),
@@ -426,18 +440,22 @@ int launch_tma_dx(dbp_ctx *ctx, const void *codes_bf16, const void *W, const flo
     DxT p{};
     p.delta_p = delta_p; p.dX = dX; p.dx_f32 = dx_bf16 ? 0 : 1;
     CUtensorMap map_dx = map_w;                  // a valid map when the store path is not used
-    p.tma_out = (dx_bf16 && HW % 8 == 0) ? 1 : 0;
+    p.tma_out = HW % (dx_bf16 ? 8 : 4) == 0 ? 1 : 0;
     if (p.tma_out) {
+        const unsigned long long es = dx_bf16 ? 2 : 4;
         const unsigned long long dims[3] = {static_cast<unsigned long long>(HW), static_cast<unsigned long long>(s.Cin),
                                             static_cast<unsigned long long>(s.B)};
-        const unsigned long long str[2] = {static_cast<unsigned long long>(HW) * 2, static_cast<unsigned long long>(HW) * 2 * s.Cin};
-        const unsigned box[3] = {64, 32, 1};
-        if (!encode_map_bf16(&map_dx, dX, 3, dims, str, box)) return DBP_ECUDA;
+        const unsigned long long str[2] = {static_cast<unsigned long long>(HW) * es, static_cast<unsigned long long>(HW) * es * s.Cin};
+        const unsigned box[3] = {dx_bf16 ? 64u : 32u, 32, 1};
+        if (!(dx_bf16 ? encode_map_bf16(&map_dx, dX, 3, dims, str, box) : encode_map_f32_sw128(&map_dx, dX, 3, dims, str, box)))
+            return fail_cuda("tensor map of dX");
     }
     p.Cin = static_cast<int>(s.Cin); p.Cout = static_cast<int>(s.Cout); p.HW = static_cast<int>(HW);
     p.chunks_per_img = static_cast<int>((HW + 63) / 64);
     p.nchunks = s.B * p.chunks_per_img;
-    p.ksteps = static_cast<int>((s.Cout + 63) / 64);
+    p.ks_piece = static_cast<int>((s.Cout + 63) / 64);
+    p.pieces = pieces;
+    p.ksteps = p.ks_piece * pieces;
     // Two accumulators halve the code traffic per MMA but leave half as many tiles and no second
     // tile in flight: worth it for long reductions that still fill the GPU. Few tiles: narrower ones.
     const long long ntile4 = (p.nchunks + kNChunks - 1) / kNChunks;

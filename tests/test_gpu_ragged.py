@@ -1,0 +1,59 @@
+"""1x1 and 3x3 layers of either type with channel counts and planes that no tile or 16-byte row fits, as the calls run by
+default (no sparse structure, no forced path): parity with the oracle. Delta and nnz come back through dbp_last_step and
+the oracle's codes, given that Delta, stand behind every gradient entry."""
+import numpy as np
+import pytest
+import torch
+
+import oracle
+import workloads as wl
+
+pytestmark = pytest.mark.gpu
+TOL = 1e-5
+
+
+@pytest.fixture(scope="module")
+def ctx():
+    import paper_2004_04729_b200 as dbp
+    c = dbp.Context(0)
+    yield c
+    c.close()
+
+
+@pytest.mark.parametrize("B,Ci,Co,H,W,k", [
+    (2, 72, 136, 27, 19, 1),      # odd planes
+    (3, 130, 33, 8, 8, 1),        # channel counts on neither side a multiple of 8
+    (5, 3, 5, 4, 6, 1),           # dW rows no multiple of 16 bytes
+    (2, 300, 70, 5, 5, 1),        # three tiles of input channels, two accumulators' worth
+    (9, 20, 24, 1, 2, 1),         # the smallest plane
+    (4, 64, 40, 3, 3, 1), (1, 257, 129, 16, 12, 1),
+    (2, 3, 8, 6, 6, 3), (2, 12, 20, 9, 9, 3), (3, 130, 65, 7, 5, 3), (2, 65, 67, 8, 8, 3), (4, 10, 6, 2, 3, 3),
+    (1, 33, 129, 20, 17, 3)])
+@pytest.mark.parametrize("dtype", ["f32", "bf16"])
+def test_layers_of_awkward_sizes(ctx, dtype, B, Ci, Co, H, W, k):
+    import paper_2004_04729_b200 as dbp
+    L = wl.conv_layer(B, Ci, Co, H, W, k, data_seed=B + Ci + 3 * Co + H, scale=2.0, seed=5, dtype=dtype)
+    tdt = torch.bfloat16 if dtype == "bf16" else torch.float32
+    d, X, Wt = (torch.from_numpy(np.ascontiguousarray(a)).to(tdt).cuda() for a in (L.delta, L.X, L.W))
+    out = dbp.dithered_conv_backward(ctx, d, X, Wt, L.seed, L.scale, need_db=True, flags=dbp.DBP_DX_F32)
+    D, nnz = ctx.last_step()
+    assert ctx.last_device_status() == (0, 0)
+    D = np.float32(D)
+    codes, onnz, _ = oracle.nsd_codes(L.delta, L.seed, D)
+    assert nnz == onnz
+    ref = oracle.conv_backward(codes, D, L.X, L.W, with_abs=True)
+    for key in ("dW", "dX", "db"):
+        g = out[key].double().cpu().numpy()
+        assert np.linalg.norm(g - ref[key]) <= TOL * np.linalg.norm(ref[key]) + 1e-30, key
+        assert np.all(np.abs(g - ref[key]) <= TOL * ref["S_" + key] + 1e-30), key
+    # a given step size (no statistics kernel), each product by itself, dW overlapped: the same numbers
+    step = torch.tensor([float(D)], device="cuda")
+    only_x = dbp.dithered_conv_backward(ctx, d, X, Wt, L.seed, 0.0, delta_in=step, need_dW=False, need_db=True, flags=dbp.DBP_DX_F32)
+    only_w = dbp.dithered_conv_backward(ctx, d, X, Wt, L.seed, 0.0, delta_in=step, need_dX=False, need_db=True)
+    both = dbp.dithered_conv_backward(ctx, d, X, Wt, L.seed, L.scale, flags=dbp.DBP_DW_ASYNC)
+    ctx.join()
+    assert torch.equal(only_x["dX"], out["dX"]) and torch.equal(only_x["db"], out["db"]) and torch.equal(only_w["db"], out["db"])
+    top = out["dW"].abs().max().item()
+    for r in (only_w, both):
+        assert (r["dW"] - out["dW"]).abs().max().item() <= 1e-5 * top
+    assert torch.equal(both["dX"], out["dX"].to(both["dX"].dtype))
