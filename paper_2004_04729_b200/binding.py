@@ -42,6 +42,7 @@ class _Sparse(ctypes.Structure):
 
 
 _lib = None
+_native = None          # the hot calls' host side (native/binding.cpp), bound when the library is loaded
 
 
 def lib_path() -> str:
@@ -101,6 +102,8 @@ def load_library():
     lib.dbp_last_error.argtypes = []
     lib.dbp_last_error.restype = ctypes.c_char_p
     _lib = lib
+    global _native
+    from . import _native       # linked against the library: an ImportError here means it has not been built
     return lib
 
 
@@ -161,6 +164,10 @@ class Context:
     def set_relu_mask(self, mask: Optional[torch.Tensor]):
         """The next backward call on this context quantizes delta (.) mask (uint8, one byte per element, non-zero
         where the forward pre-activation was positive); fp32 only. Consumed by that call."""
+        if mask is not None:
+            rc = _native.set_relu_mask(self._h.value, mask)
+            if rc is not None:
+                return _check(rc, "dbp_set_relu_mask")
         if mask is not None and not (mask.is_cuda and mask.is_contiguous() and mask.dtype == torch.uint8):
             raise ValueError("mask must be a contiguous CUDA uint8 tensor")
         _check(load_library().dbp_set_relu_mask(self._h, _ptr(mask)), "dbp_set_relu_mask")
@@ -243,6 +250,7 @@ class SparseGradient:
         self.nnz = torch.zeros(1, dtype=torch.int64, device=dev)
         self._c = _Sparse(self.bitmap.data_ptr(), self.offsets.data_ptr(), self.values.data_ptr(),
                           self.delta.data_ptr(), self.nnz.data_ptr(), self.numel)
+        self._addr = ctypes.addressof(self._c)
 
     def c(self):
         return ctypes.byref(self._c)
@@ -252,6 +260,11 @@ def nsd_quantize(ctx: Context, delta: torch.Tensor, seed: int, scale: float,
                  delta_in: Optional[torch.Tensor] = None,
                  out: Optional[SparseGradient] = None) -> SparseGradient:
     """Algorithm 1: (codes, Delta, nnz) of `delta` as a SparseGradient."""
+    if out is not None:
+        rc = _native.quantize(ctx._h.value, delta, seed, scale, delta_in, out._addr)
+        if rc is not None:
+            _check(rc, "nsd_quantize")
+            return out
     _dev(delta, "delta")
     out = out or SparseGradient(delta.numel(), ctx.device)
     _check(load_library().nsd_quantize(ctx._h, _ptr(delta), _dtype_code(delta), delta.numel(),
@@ -261,8 +274,12 @@ def nsd_quantize(ctx: Context, delta: torch.Tensor, seed: int, scale: float,
 
 
 def nsd_decode_dense(ctx: Context, q: SparseGradient, shape=None) -> torch.Tensor:
-    codes = torch.empty(q.numel, dtype=torch.int8, device=q.values.device)
-    _check(load_library().nsd_decode_dense(ctx._h, q.c(), _ptr(codes)), "nsd_decode_dense")
+    codes = _native.decode(ctx._h.value, q._addr, q.numel, q.values)
+    if codes is None:
+        codes = torch.empty(q.numel, dtype=torch.int8, device=q.values.device)
+        _check(load_library().nsd_decode_dense(ctx._h, q.c(), _ptr(codes)), "nsd_decode_dense")
+    elif type(codes) is int:
+        raise DbpError(codes, "nsd_decode_dense")
     return codes if shape is None else codes.view(shape)
 
 
@@ -274,6 +291,12 @@ def dithered_linear_backward(ctx: Context, delta, X, W, seed: int, scale: float,
                              delta_in=None, q_out: Optional[SparseGradient] = None,
                              need_dW=True, need_dX=True, need_db=False, flags: int = 0):
     """delta [B,N], X [B,K], W [N,K] -> dict(dW [N,K] fp32, dX [B,K], db [N] fp32)."""
+    r = _native.linear_backward(ctx._h.value, delta, X, W, seed, scale, delta_in, q_out and q_out._addr, need_dW, need_dX, need_db,
+                                flags)
+    if type(r) is dict:
+        return r
+    if r is not None:
+        raise DbpError(r, "dithered_linear_backward")
     _dev(delta, "delta"), _dev(X, "X"), _dev(W, "W")
     B, N = delta.shape
     K = X.shape[1]
@@ -296,6 +319,12 @@ def dithered_conv_backward(ctx: Context, delta, X, W, seed: int, scale: float, *
                            need_dW=True, need_dX=True, need_db=False, flags: int = 0,
                            stride: int = 1, pad: Optional[int] = None):
     """delta [B,Cout,H/stride,W/stride], X [B,Cin,H,W], W [Cout,Cin,k,k] (NCHW) -> dict(dW, dX, db)."""
+    r = _native.conv_backward(ctx._h.value, delta, X, W, seed, scale, delta_in, q_out and q_out._addr, need_dW, need_dX, need_db,
+                              flags, stride, (W.shape[2] - 1) // 2 if pad is None else pad)
+    if type(r) is dict:
+        return r
+    if r is not None:
+        raise DbpError(r, "dithered_conv_backward")
     _dev(delta, "delta"), _dev(X, "X"), _dev(W, "W")
     B, Co = delta.shape[:2]
     Ci, k = X.shape[1], W.shape[2]
@@ -364,6 +393,11 @@ def relu_backward(ctx: Context, delta_a: torch.Tensor, mask_u8: torch.Tensor) ->
 
 
 def maxpool2x2_backward(ctx: Context, g: torch.Tensor, argmax_i8: torch.Tensor) -> torch.Tensor:
+    r = _native.maxpool2x2(ctx._h.value, g, argmax_i8)
+    if type(r) is int:
+        raise DbpError(r, "dbp_maxpool2x2_backward")
+    if r is not None:
+        return r
     B, C, h, w = g.shape
     out = torch.empty((B, C, 2 * h, 2 * w), dtype=g.dtype, device=g.device)
     _check(load_library().dbp_maxpool2x2_backward(ctx._h, _ptr(g), _ptr(argmax_i8), _ptr(out),
@@ -409,6 +443,13 @@ def network_backward(ctx: Context, kinds, Xs, Ws, relu_masks, pool_argmax, delta
     Returns one dict per layer with dW, dX (None for layer 0 unless asked), Delta, nnz, and
     optionally the delta_z that was quantized and its SparseGradient. with_sparse=False asks for
     no sparse structure (Delta and nnz are then None; the library runs its leaner quantizer)."""
+    if not with_sparse and not keep_delta_z:
+        r = _native.network_backward(ctx._h.value, list(kinds), list(Xs), list(Ws), list(relu_masks), list(pool_argmax), delta_out,
+                                     scale, seed, first_layer_dX, flags)
+        if type(r) is list:
+            return r
+        if r is not None:
+            raise DbpError(r, "network_backward")
     L = len(kinds)
     res = [None] * L
     delta_a = delta_out

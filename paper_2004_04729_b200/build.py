@@ -1,4 +1,4 @@
-"""Builds the CUDA library (`libdbp.so`) in-tree with nvcc for sm_100a.
+"""Builds the CUDA library (`libdbp.so`, nvcc for sm_100a) and the binding's native part (`_native`, g++) in-tree.
 
 `python -m paper_2004_04729_b200.build [--force] [--verbose]`
 """
@@ -6,6 +6,7 @@ import glob
 import os
 import subprocess
 import sys
+import sysconfig
 
 HERE = os.path.dirname(os.path.abspath(__file__))
 ROOT = os.path.dirname(HERE)
@@ -40,6 +41,7 @@ def build(force: bool = False, verbose: bool = False) -> str:
     """One object per source file (compiled in parallel, rebuilt only when the source, a header
     or this script changed), linked into the shared library."""
     if not force and not _stale():
+        build_native()
         return LIB
     from concurrent.futures import ThreadPoolExecutor
     objdir = os.path.join(HERE, "_build")
@@ -56,7 +58,33 @@ def build(force: bool = False, verbose: bool = False) -> str:
         list(pool.map(_compile, jobs))
     nvcc = os.environ.get("NVCC", "nvcc")
     subprocess.check_call([nvcc, "-shared", "-gencode", "arch=compute_100a,code=sm_100a", "-o", LIB] + objs)
+    build_native(force)
     return LIB
+
+
+def native_path() -> str:
+    return os.path.join(HERE, "_native" + sysconfig.get_config_var("EXT_SUFFIX"))
+
+
+def build_native(force: bool = False) -> str:
+    """The CPython extension of the binding (native/binding.cpp, g++), linked against the library beside it."""
+    src, out = os.path.join(HERE, "native", "binding.cpp"), native_path()
+    deps = [src, os.path.join(ROOT, "include", "dbp.h"), __file__]
+    if not force and os.path.exists(out) and all(os.path.getmtime(out) >= os.path.getmtime(p) for p in deps):
+        return out
+    import torch
+    from torch.utils import cpp_extension
+    tlib = os.path.join(os.path.dirname(torch.__file__), "lib")
+    cuda = os.environ.get("CUDA_HOME", "/usr/local/cuda")
+    cmd = [os.environ.get("CXX", "g++"), "-O2", "-std=c++17", "-fPIC", "-shared", "-fvisibility=hidden",
+           f"-D_GLIBCXX_USE_CXX11_ABI={int(torch._C._GLIBCXX_USE_CXX11_ABI)}", src, "-o", out,
+           "-I", os.path.join(ROOT, "include"), "-I", sysconfig.get_paths()["include"], "-I", os.path.join(cuda, "include")]
+    for p in cpp_extension.include_paths():
+        cmd += ["-isystem", p]
+    cmd += ["-L", HERE, "-l:libdbp.so", "-L", tlib, "-lc10", "-ltorch", "-ltorch_cpu", "-ltorch_cuda", "-ltorch_python",
+            "-Wl,-rpath,$ORIGIN", "-Wl,-rpath," + tlib]
+    subprocess.check_call(cmd)
+    return out
 
 
 if __name__ == "__main__":

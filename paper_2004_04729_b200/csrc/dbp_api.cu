@@ -48,13 +48,13 @@ bool aligned16(const void *p) { return (reinterpret_cast<uintptr_t>(p) & 15u) ==
 size_t elem_size(int dtype) { return dtype == DBP_F32 ? 4 : 2; }
 
 struct DeviceGuard {
-    int prev = -1;
+    int prev = -1, now = -1;
     bool ok = true;
-    explicit DeviceGuard(int dev) {
+    explicit DeviceGuard(int dev) : now(dev) {
         if (cudaGetDevice(&prev) != cudaSuccess) { ok = false; return; }
         if (prev != dev && cudaSetDevice(dev) != cudaSuccess) ok = false;
     }
-    ~DeviceGuard() { if (prev >= 0) cudaSetDevice(prev); }
+    ~DeviceGuard() { if (prev >= 0 && prev != now) cudaSetDevice(prev); }
 };
 
 // The current set's previous readers (an earlier call's dW kernels on the second stream) must be done before its step
@@ -89,15 +89,17 @@ int quantize_for_products(dbp_ctx *ctx, const void *delta, int dtype, long long 
         sp = *q_out;
     }
     const int k = ctx->code_set;
-    if ((want8 || q_out) && (rc = ws_reserve(ctx, ctx->dense_codes[k], static_cast<size_t>(numel) + 16))) return rc;
+    if (want8 && (rc = ws_reserve(ctx, ctx->dense_codes[k], static_cast<size_t>(numel) + 16))) return rc;
     int8_t *dense = static_cast<int8_t *>(ctx->dense_codes[k].ptr);
     if ((rc = wait_code_set(ctx))) return rc;
+    StepSource step;
     {
         KernelTimer t(ctx, DBP_K_STATISTICS);
-        // without a caller's dbp_sparse the step size also goes to the set's own scalar: the product kernels
-        // read it there (the context's scalar is overwritten by the next call's statistics)
-        rc = launch_statistics(ctx, delta, dtype, numel, scale, delta_in, q_out ? sp.delta : ctx->delta_sets + k,
-                               reinterpret_cast<unsigned long long *>(sp.nnz), jobs, mask);
+        // the step size also goes to the set's own scalar: the product kernels read it there (the context's scalar is
+        // overwritten by the next call's quantizer)
+        float *const publish[2] = {ctx->delta_sets + k, sp.delta};
+        rc = launch_statistics(ctx, delta, dtype, numel, scale, delta_in, publish, reinterpret_cast<unsigned long long *>(sp.nnz), &step,
+                               jobs, mask);
     }
     if (rc) return rc;
     {
@@ -126,27 +128,24 @@ int quantize_for_products(dbp_ctx *ctx, const void *delta, int dtype, long long 
             *codes_stack = ps;
         }
         if (q_out) {
-            rc = launch_quantize(ctx, delta, dtype, numel, seed, &ctx->state->delta, sp.bitmap, sp.offsets,
-                                 sp.values, dense, reinterpret_cast<unsigned long long *>(sp.nnz));
+            rc = launch_quantize(ctx, delta, dtype, numel, seed, step, sp.bitmap, sp.offsets,
+                                 sp.values, want8 ? dense : nullptr, reinterpret_cast<unsigned long long *>(sp.nnz));
             if (!rc && p16)
-                rc = launch_quantize_dense(ctx, delta, dtype, numel, seed, &ctx->state->delta, nullptr, p16,
+                rc = launch_quantize_dense(ctx, delta, dtype, numel, seed, step, nullptr, p16,
                                            planes_hw, planes_pitch, false);
             if (!rc && pn)
                 rc = launch_quantize_nhwc(ctx, delta, dtype, nhwc->B, nhwc->Cout, nhwc->H * nhwc->W, seed,
-                                          &ctx->state->delta, pn, nullptr, false, ps, static_cast<int>(nhwc->W), stack_g);
+                                          step, pn, nullptr, false, ps, static_cast<int>(nhwc->W));
         } else if (pn) {
             rc = launch_quantize_nhwc(ctx, delta, dtype, nhwc->B, nhwc->Cout, nhwc->H * nhwc->W, seed,
-                                      &ctx->state->delta, pn, want8 ? dense : nullptr, true, ps, static_cast<int>(nhwc->W), stack_g, mask);
+                                      step, pn, want8 ? dense : nullptr, true, ps, static_cast<int>(nhwc->W), mask);
         } else {
-            rc = launch_quantize_dense(ctx, delta, dtype, numel, seed, &ctx->state->delta, want8 ? dense : nullptr,
+            rc = launch_quantize_dense(ctx, delta, dtype, numel, seed, step, want8 ? dense : nullptr,
                                        p16, planes_hw, planes_pitch, true);
         }
     }
     if (rc) return rc;
-    *delta_p = q_out ? &ctx->state->delta : ctx->delta_sets + k;
-    if (q_out && cudaMemcpyAsync(ctx->delta_sets + k, &ctx->state->delta, sizeof(float), cudaMemcpyDeviceToDevice, ctx->stream) != cudaSuccess)
-        return fail_cuda("copying the step size");
-    if (q_out) *delta_p = ctx->delta_sets + k;
+    *delta_p = ctx->delta_sets + k;
     *codes = dense;
     return DBP_OK;
 }
@@ -791,14 +790,15 @@ int nsd_quantize(dbp_ctx *ctx, const void *delta, int dtype, long long numel, un
     if (!guard.ok) return DBP_ECUDA;
     out->numel = numel;
     int rc;
+    StepSource step;
     {
         KernelTimer t(ctx, DBP_K_STATISTICS);
-        rc = launch_statistics(ctx, delta, dtype, numel, scale, delta_in, out->delta,
-                               reinterpret_cast<unsigned long long *>(out->nnz));
+        float *const publish[2] = {out->delta, nullptr};
+        rc = launch_statistics(ctx, delta, dtype, numel, scale, delta_in, publish, reinterpret_cast<unsigned long long *>(out->nnz), &step);
     }
     if (rc) return rc;
     KernelTimer t(ctx, DBP_K_QUANTIZE);
-    return launch_quantize(ctx, delta, dtype, numel, seed, &ctx->state->delta, out->bitmap, out->offsets,
+    return launch_quantize(ctx, delta, dtype, numel, seed, step, out->bitmap, out->offsets,
                            out->values, nullptr, reinterpret_cast<unsigned long long *>(out->nnz));
 }
 

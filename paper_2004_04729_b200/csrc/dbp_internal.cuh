@@ -18,7 +18,6 @@ constexpr int kWordsPerSegment = kSegment / 32;
 struct DeviceState {
     float delta;                        // step size of the internal quantization
     int nonfinite;                      // set when delta_z held NaN/Inf
-    unsigned int ticket;                // last-block election of the statistics kernel
     int tc_timeout;                     // a bounded wait of a tensor-core kernel expired
     unsigned long long nnz;             // non-zero codes of the internal quantization
     unsigned long long saturated;       // clipped codes since the last report
@@ -104,6 +103,16 @@ namespace dbp {
 
 int ws_reserve(dbp_ctx *ctx, Workspace &w, size_t bytes);
 
+// Where a quantizer takes the step size from: the statistics kernel's partial sums, or a device scalar.
+struct StepSource {
+    const float *given = nullptr;
+    const double *partials = nullptr;   // (sum, sum of squares) of each statistics block, about the pivot
+    int nparts = 0;
+    double numel = 0;
+    float scale = 0.f;
+    float *publish[3] = {nullptr, nullptr, nullptr};   // where the quantizer writes it for the kernels behind it
+};
+
 // ---- nsd_kernels.cu
 // Work the statistics kernel does on the side for the layer's product kernels (its blocks have time to spare
 // and this saves launches): clearing a buffer (16-byte aligned, a multiple of 16 bytes), and re-laying 3x3
@@ -128,26 +137,28 @@ struct SideJobs {
     long long Cout = 0, Cin = 0;
     int phase_cin = 0;                 // > 0: w_src holds a stride-2 layer's own weights [Cout][phase_cin][9], Cin = 4 phase_cin
 };
+// publish: where the quantizer is to write the step size beside the context's state (entries may be null); *step tells
+// the quantizer where to take it from
 int launch_statistics(dbp_ctx *ctx, const void *delta, int dtype, long long numel, float scale,
-                      const float *delta_in, float *delta_out, unsigned long long *nnz_out,
+                      const float *delta_in, float *const (&publish)[2], unsigned long long *nnz_out, StepSource *step,
                       const SideJobs &jobs = SideJobs(), const uint8_t *mask = nullptr);
 // beside: the kernel before it on the stream is the quantizer; the job runs beside it
 int launch_rows_job(dbp_ctx *ctx, const RowsJob &job, bool beside);
 int launch_quantize(dbp_ctx *ctx, const void *delta, int dtype, long long numel,
-                    unsigned long long seed, const float *delta_p, uint32_t *bitmap,
+                    unsigned long long seed, const StepSource &step, uint32_t *bitmap,
                     uint16_t *offsets, int8_t *values, int8_t *dense,
                     unsigned long long *nnz_out);
 // ---- nsd_dense.cu: the same codes, dense array only (no sparse structure)
 // dense: int8 codes in delta's order (or null); planes_bf16: bf16 codes as [numel / hw][pitch]
 // (or null), pitch a multiple of 8
 int launch_quantize_dense(dbp_ctx *ctx, const void *delta, int dtype, long long numel,
-                          unsigned long long seed, const float *delta_p, int8_t *dense,
+                          unsigned long long seed, const StepSource &step, int8_t *dense,
                           void *planes_bf16, long long hw, long long pitch, bool count);
 // position-major bf16 codes [B][HW][C] for the TMA-fed 3x3 kernels (and int8 codes in delta's order
 // when dense8 is not null)
 int launch_quantize_nhwc(dbp_ctx *ctx, const void *delta, int dtype, long long B, long long C, long long HW,
-                         unsigned long long seed, const float *delta_p, void *codes_nhwc, int8_t *dense8, bool count,
-                         void *codes_stack = nullptr, int plane_w = 0, int stack_g = 0, const uint8_t *mask = nullptr);
+                         unsigned long long seed, const StepSource &step, void *codes_nhwc, int8_t *dense8, bool count,
+                         void *codes_stack = nullptr, int plane_w = 0, const uint8_t *mask = nullptr);
 int launch_decode(dbp_ctx *ctx, const uint32_t *bitmap, const uint16_t *offsets,
                   const int8_t *values, long long numel, int8_t *dense);
 

@@ -1,95 +1,22 @@
-// NSD quantization for the product kernels (Section 3.1, Eq. (nsd)): the same codes as
-// quantize_kernel, written only as the dense array the dX / dW kernels read, without the
-// bitmap / offsets / packed-values structure. Used when the caller did not ask for the sparse
-// structure, so the pass costs one read of delta_z and one write of the codes.
+// NSD quantization for the product kernels (Section 3.1, Eq. (nsd)): the same codes as quantize_kernel, written only as
+// the dense arrays the dX / dW kernels read, without the bitmap / offsets / packed-values structure. Used when the caller
+// did not ask for the sparse structure, so the pass costs one read of delta_z and one write of the codes.
 //
-// The common case (every |x / Delta + u| <= 127, no NaN) runs without clamping or conversions:
-// the code is the round-down sum with 1.5 * 2^23, less that constant (a float holding a small
-// integer, whose upper half is its bf16). A vector that holds a NaN or a value outside that range
-// is redone element by element with the clipped, counted decision.
-#include "dbp_internal.cuh"
+// The kernels are bound by instruction issue (the SplitMix64 draw of a pair of elements is about 19 instructions), so
+// the arithmetic around it works on pairs (nsd_common.cuh). A thread's first vectors of delta_z and their dithers need
+// nothing of the statistics kernel that runs before: they are loaded and drawn before the wait for it. That is safe
+// because the statistics kernel lets this one start only once all of its own blocks have seen the kernels before it
+// complete. In the loop the next vectors are loaded before the current ones are stored.
+#include "nsd_common.cuh"
 
 namespace dbp {
 
 namespace {
 
-constexpr int kThreads = 256;
-#ifndef DBP_Q_BLOCKS_PER_SM
-#define DBP_Q_BLOCKS_PER_SM 4
-#endif
-constexpr int kBlocksPerSM = DBP_Q_BLOCKS_PER_SM;   // resident blocks the dense quantizer is compiled for
-constexpr unsigned kFull = 0xffffffffu;
-constexpr unsigned long long kGamma = 0x9E3779B97F4A7C15ull;
+using namespace nsd;
 
-__device__ __forceinline__ unsigned long long mix64(unsigned long long z) {
-    z = (z ^ (z >> 30)) * 0xBF58476D1CE4E5B9ull;
-    z = (z ^ (z >> 27)) * 0x94D049BB133111EBull;
-    return z ^ (z >> 31);
-}
-// u = (2k+1) 2^-24, k = top 23 bits of h: the funnel shift builds 1 + k 2^-23 in one step
-__device__ __forceinline__ float dither(unsigned h) {
-    return __uint_as_float(__funnelshift_r(h, 0x7fu, 9)) - 0.99999994f;
-}
-constexpr float kMagic = 12582912.0f;             // 1.5 * 2^23: a float in [2^23, 2^24) has unit spacing
-// careful decision: clipped to [-127, 127], clipped codes counted, NaN gives 0. Returns the bits of
-// kMagic + code (the low byte is the code's two's-complement byte).
-__device__ __forceinline__ unsigned careful_bits(float x, float inv, float u, unsigned &sat) {
-    const float t = __fmaf_rn(x, inv, u);
-    const float tc = fminf(fmaxf(t, -127.f), 127.99999f);
-    const bool num = (t == t);
-    sat += (num && tc != t) ? 1u : 0u;
-    return num ? __float_as_uint(__fadd_rd(tc, kMagic)) : __float_as_uint(kMagic);
-}
-__device__ __forceinline__ unsigned careful_byte(float x, float inv, float u, unsigned &sat) {
-    return careful_bits(x, inv, u, sat) & 0xffu;
-}
-// Codes of the V elements x[0..V) whose first element has the (even) linear index e0, as floats
-// (exact small integers). V is 4 or 8. The common case (every |t| <= 127, no NaN) is recognised by
-// the sum of the squares of t = x / Delta + u and needs no clamp: floor(t) is the round-down sum
-// with kMagic, less kMagic. The number of non-zero codes is added to nz (a float: exact below 2^24).
-template <int V>
-__device__ __forceinline__ void codes_of(const float (&x)[V], long long e0, unsigned long long seed,
-                                         float inv, float (&f)[V], float &nz, unsigned &sat) {
-    unsigned long long z = seed + (static_cast<unsigned long long>(e0 >> 1) + 1ull) * kGamma;
-    float u[V];
-#pragma unroll
-    for (int j = 0; j < V; j += 2) {
-        const unsigned long long r = mix64(z);
-        z += kGamma;
-        u[j] = dither(static_cast<unsigned>(r));
-        u[j + 1] = dither(static_cast<unsigned>(r >> 32));
-    }
-    float s2 = 0.f;
-#pragma unroll
-    for (int j = 0; j < V; ++j) {
-        const float t = __fmaf_rn(x[j], inv, u[j]);
-        s2 = __fmaf_rn(t, t, s2);                   // NaN or inf if some t is; > 127^2 if some |t| > 127
-        f[j] = __fadd_rd(t, kMagic) - kMagic;
-    }
-    if (!(s2 <= 16128.f)) {                         // rare: clip, count, NaN
-#pragma unroll
-        for (int j = 0; j < V; ++j) f[j] = __uint_as_float(careful_bits(x[j], inv, u[j], sat)) - kMagic;
-    }
-#pragma unroll
-    for (int j = 0; j < V; ++j) nz += __saturatef(f[j] * f[j]);
-}
-// the codes' bytes, four to a word in element order
-template <int V>
-__device__ __forceinline__ void pack_bytes(const float (&f)[V], unsigned (&pk)[V / 4]) {
-    unsigned b[V];
-#pragma unroll
-    for (int j = 0; j < V; ++j) b[j] = __float_as_uint(f[j] + kMagic);     // low byte: the code
-#pragma unroll
-    for (int w = 0; w < V / 4; ++w)
-        pk[w] = __byte_perm(__byte_perm(b[4 * w], b[4 * w + 1], 0x0040), __byte_perm(b[4 * w + 2], b[4 * w + 3], 0x0040), 0x5410);
-}
-// the codes as bf16, two to a word: an integer of at most 8 bits is exact in bf16, which is the
-// float's upper half
-template <int V>
-__device__ __forceinline__ void pack_bf16(const float (&f)[V], unsigned (&h)[V / 2]) {
-#pragma unroll
-    for (int j = 0; j < V / 2; ++j) h[j] = __byte_perm(__float_as_uint(f[2 * j]), __float_as_uint(f[2 * j + 1]), 0x7632);
-}
+constexpr int kThreads = 256;
+constexpr int kBlocksPerSM = 3;                   // resident blocks the dense quantizer is compiled for
 
 // Where the codes go. dense8: one byte per element, same order as delta_z (may be null).
 // planes16: bf16 codes as [plane][pitch] with plane = e / hw (may be null); the pitch is a
@@ -114,8 +41,9 @@ __device__ __forceinline__ void split_index(long long e, long long hw, long long
     }
 }
 
+// f: the codes as floats, h: as packed bf16
 template <int V>
-__device__ __forceinline__ void store_codes(const CodeSinks &o, long long e0, const float (&f)[V]) {
+__device__ __forceinline__ void store_codes(const CodeSinks &o, long long e0, const float (&f)[V], const unsigned (&h)[V / 2]) {
     if (o.dense8 != nullptr) {
         unsigned pk[V / 4];
         pack_bytes<V>(f, pk);
@@ -123,8 +51,6 @@ __device__ __forceinline__ void store_codes(const CodeSinks &o, long long e0, co
         else *reinterpret_cast<uint2 *>(o.dense8 + e0) = make_uint2(pk[0], pk[V / 4 - 1]);
     }
     if (o.planes16 != nullptr) {
-        unsigned h[V / 2];
-        pack_bf16<V>(f, h);
         if (o.pitch == o.hw) {                      // planes are back to back: same order as delta_z
             if (V == 4) *reinterpret_cast<uint2 *>(o.planes16 + e0) = make_uint2(h[0], h[1]);
             else *reinterpret_cast<uint4 *>(o.planes16 + e0) = make_uint4(h[0], h[1], h[V / 2 - 2], h[V / 2 - 1]);
@@ -174,100 +100,64 @@ __device__ __forceinline__ void store_code(const CodeSinks &o, long long e, unsi
 }
 
 template <typename T>
-struct Vec;
-template <>
-struct Vec<float> {
-    static constexpr int V = 4;
-    __device__ static void load(const float *p, float (&v)[4]) {
-        const float4 q = __ldg(reinterpret_cast<const float4 *>(p));
-        v[0] = q.x; v[1] = q.y; v[2] = q.z; v[3] = q.w;
-    }
-    __device__ static float one(const float *p) { return __ldg(p); }
-};
-template <>
-struct Vec<__nv_bfloat16> {
-    static constexpr int V = 8;
-    __device__ static void load(const __nv_bfloat16 *p, float (&v)[8]) {
-        const uint4 q = __ldg(reinterpret_cast<const uint4 *>(p));
-        const unsigned w[4] = {q.x, q.y, q.z, q.w};
-#pragma unroll
-        for (int i = 0; i < 4; ++i) {
-            v[2 * i] = __uint_as_float(w[i] << 16);
-            v[2 * i + 1] = __uint_as_float(w[i] & 0xffff0000u);
-        }
-    }
-    __device__ static float one(const __nv_bfloat16 *p) {
-        return __uint_as_float(static_cast<unsigned>(__ldg(reinterpret_cast<const unsigned short *>(p))) << 16);
-    }
-};
-
-template <typename T>
 __global__ void __launch_bounds__(kThreads, kBlocksPerSM)
-quantize_dense_kernel(const T *__restrict__ x, long long n, unsigned long long seed,
-                      const float *__restrict__ delta_p, const CodeSinks out,
-                      DeviceState *__restrict__ st) {
+quantize_dense_kernel(const T *__restrict__ x, long long n, unsigned long long seed, const StepSource step,
+                      const CodeSinks out, DeviceState *__restrict__ st) {
     constexpr int V = Vec<T>::V;
     const long long nvec = n / V;
     const long long stride = static_cast<long long>(gridDim.x) * kThreads;
     long long i = static_cast<long long>(blockIdx.x) * kThreads + threadIdx.x;
+    // two vectors per thread and round: i and i + stride
+    uint4 r0, r1;
+    unsigned long long u0[V / 2], u1[V / 2];
+    auto load = [&](long long k) {
+        r0 = k < nvec ? Vec<T>::raw(x + k * V) : make_uint4(0u, 0u, 0u, 0u);
+        r1 = k + stride < nvec ? Vec<T>::raw(x + (k + stride) * V) : make_uint4(0u, 0u, 0u, 0u);
+    };
+    auto draw = [&](long long k) {
+        dithers_of<V>(k * V, seed, u0);
+        dithers_of<V>((k + stride) * V, seed, u1);
+    };
+    load(i);
+    draw(i);
     chain_wait();
     chain_release();
-    const float delta = *delta_p;
-    const bool live = (delta > 0.f) && (delta < __int_as_float(0x7f800000));
-    if (!live) {                                    // sigma = 0 or non-finite input: every code is 0
-        for (; i < nvec; i += stride) {
-            const float zero[V] = {};
-            store_codes<V>(out, i * V, zero);
+    const float delta = step_of<kThreads>(step, st);
+    const float inv = delta > 0.f ? __fdiv_rn(1.0f, delta) : 0.f;      // Delta = 0: x * 0 + u < 1, every code 0 (NaN too)
+    unsigned sat = 0, nz2 = 0, nnz = 0;
+    for (; i < nvec; ) {
+        float v[V], f0[V], f1[V];
+        Vec<T>::values(r0, v);
+        decide<V>(v, u0, inv, f0, sat);
+        Vec<T>::values(r1, v);
+        const bool two = i + stride < nvec;
+        decide<V>(v, u1, inv, f1, sat);
+        const long long k = i;
+        i += 2 * stride;
+        load(i);
+        unsigned h0[V / 2], h1[V / 2];
+        pack_bf16<V>(f0, h0);
+        pack_bf16<V>(f1, h1);
+        count_pairs<V>(h0, nz2);
+        store_codes<V>(out, k * V, f0, h0);
+        if (two) {
+            count_pairs<V>(h1, nz2);
+            store_codes<V>(out, (k + stride) * V, f1, h1);
         }
-        if (blockIdx.x == 0 && threadIdx.x == 0)
-            for (long long e = nvec * V; e < n; ++e) store_code(out, e, 0u);
-        return;
+        if (nz2 & 0x80008000u) { nnz += pairs_total(nz2); nz2 = 0; }
+        if (i < nvec) draw(i);
     }
-    const float inv = __fdiv_rn(1.0f, delta);
-    unsigned nnz = 0, sat = 0;
-    float nz = 0.f;
-    // two vectors in flight per thread
-    for (; i + stride < nvec; i += 2 * stride) {
-        float a[V], b[V];
-        Vec<T>::load(x + i * V, a);
-        Vec<T>::load(x + (i + stride) * V, b);
-        float fa[V], fb[V];
-        codes_of<V>(a, i * V, seed, inv, fa, nz, sat);
-        codes_of<V>(b, (i + stride) * V, seed, inv, fb, nz, sat);
-        store_codes<V>(out, i * V, fa);
-        store_codes<V>(out, (i + stride) * V, fb);
-    }
-    if (i < nvec) {
-        float a[V];
-        Vec<T>::load(x + i * V, a);
-        float fa[V];
-        codes_of<V>(a, i * V, seed, inv, fa, nz, sat);
-        store_codes<V>(out, i * V, fa);
-    }
-    nnz = static_cast<unsigned>(nz);                // a thread's share is far below 2^24 elements
+    nnz += pairs_total(nz2);
     if (blockIdx.x == 0 && threadIdx.x == 0) {      // the n % V last elements, one by one
         for (long long e = nvec * V; e < n; ++e) {
-            const unsigned long long r = mix64(seed + (static_cast<unsigned long long>(e >> 1) + 1ull) * kGamma);
-            const float u = dither((e & 1) ? static_cast<unsigned>(r >> 32) : static_cast<unsigned>(r));
-            const unsigned q = careful_byte(Vec<T>::one(x + e), inv, u, sat);
+            float ua, ub;
+            unpack2(dither2(counter_of(e & ~1ll, seed)), ua, ub);
+            const unsigned q = careful_bits(Vec<T>::one(x + e), inv, (e & 1) ? ub : ua, sat) & 0xffu;
             store_code(out, e, q);
             nnz += q != 0u;
         }
     }
-    nnz = __reduce_add_sync(kFull, nnz);
-    sat = __reduce_add_sync(kFull, sat);
-    __shared__ unsigned s_nnz, s_sat;
-    if (threadIdx.x == 0) { s_nnz = 0; s_sat = 0; }
-    __syncthreads();
-    if ((threadIdx.x & 31) == 0) {
-        if (nnz) atomicAdd(&s_nnz, nnz);
-        if (sat) atomicAdd(&s_sat, sat);
-    }
-    __syncthreads();
-    if (threadIdx.x == 0 && out.count) {
-        if (s_nnz) atomicAdd(&st->nnz, static_cast<unsigned long long>(s_nnz));
-        if (s_sat) atomicAdd(&st->saturated, static_cast<unsigned long long>(s_sat));
-    }
+    if (out.count) publish_counts<kThreads>(nnz, delta > 0.f ? sat : 0u, st, nullptr);
 }
 
 
@@ -289,34 +179,28 @@ __device__ __forceinline__ unsigned tile_off(int p, int c) {
            ((static_cast<unsigned>(c) & 7u) << 1);
 }
 
-// one element by itself (planes whose size is odd: the pair that shares a draw may straddle two
-// vectors); same decision as codes_of. Returns the code as a float.
-__device__ __forceinline__ float code_single(float x, long long e, unsigned long long seed, float inv, unsigned &sat) {
-    const unsigned long long r = mix64(seed + (static_cast<unsigned long long>(e >> 1) + 1ull) * kGamma);
-    const float u = dither((e & 1) ? static_cast<unsigned>(r >> 32) : static_cast<unsigned>(r));
-    const float t = __fmaf_rn(x, inv, u);
-    if (fabsf(t) <= 127.f) return __fadd_rd(t, kMagic) - kMagic;
-    return __uint_as_float(careful_bits(x, inv, u, sat)) - kMagic;
+// mask (fp32 tensors only): x is delta_a and the gradient is delta_a where mask != 0, else 0. The four mask bytes of a
+// vector as one word.
+__device__ __forceinline__ unsigned mask_word(const unsigned char *mask, long long e) { return __ldg(reinterpret_cast<const unsigned *>(mask + e)); }
+__device__ __forceinline__ void apply_mask(unsigned m, float (&v)[4]) {
+#pragma unroll
+    for (int j = 0; j < 4; ++j) v[j] = (m >> (8 * j)) & 0xffu ? v[j] : 0.f;
 }
+__device__ __forceinline__ void apply_mask(unsigned, float (&)[8]) {}                 // bf16 tensors take no mask
 
+// V of the elements of a 128-bit vector (8-byte loads for bf16 planes that are only a multiple of 4)
 template <typename T, int V>
-struct TileLoad;
-template <>
-struct TileLoad<__nv_bfloat16, 8> {
-    __device__ static void ld(const __nv_bfloat16 *p, float (&v)[8]) { Vec<__nv_bfloat16>::load(p, v); }
-};
-template <>
-struct TileLoad<__nv_bfloat16, 4> {
-    __device__ static void ld(const __nv_bfloat16 *p, float (&v)[4]) {
-        const uint2 q = __ldg(reinterpret_cast<const uint2 *>(p));
-        v[0] = __uint_as_float(q.x << 16); v[1] = __uint_as_float(q.x & 0xffff0000u);
-        v[2] = __uint_as_float(q.y << 16); v[3] = __uint_as_float(q.y & 0xffff0000u);
-    }
-};
-template <>
-struct TileLoad<float, 4> {
-    __device__ static void ld(const float *p, float (&v)[4]) { Vec<float>::load(p, v); }
-};
+__device__ __forceinline__ uint4 load_raw(const T *p) {
+    if (sizeof(T) * V == 16) return __ldg(reinterpret_cast<const uint4 *>(p));
+    const uint2 q = __ldg(reinterpret_cast<const uint2 *>(p));
+    return make_uint4(q.x, q.y, 0u, 0u);
+}
+__device__ __forceinline__ void values_of(const float *, const uint4 &q, float (&v)[4]) { Vec<float>::values(q, v); }
+__device__ __forceinline__ void values_of(const __nv_bfloat16 *, const uint4 &q, float (&v)[8]) { Vec<__nv_bfloat16>::values(q, v); }
+__device__ __forceinline__ void values_of(const __nv_bfloat16 *, const uint4 &q, float (&v)[4]) {
+    v[0] = __uint_as_float(q.x << 16); v[1] = __uint_as_float(q.x & 0xffff0000u);
+    v[2] = __uint_as_float(q.y << 16); v[3] = __uint_as_float(q.y & 0xffff0000u);
+}
 
 template <int V>
 __device__ __forceinline__ void store_bytes(int8_t *dense8, long long e0, const float (&f)[V]) {
@@ -326,113 +210,157 @@ __device__ __forceinline__ void store_bytes(int8_t *dense8, long long e0, const 
     else *reinterpret_cast<uint2 *>(dense8 + e0) = make_uint2(pk[0], pk[V / 4 - 1]);
 }
 
-// V: elements per load (plane size % V == 0), or 1 for element-wise loads (any plane size).
-// Three ways to fill a tile. Planes smaller than a tile's 64 positions: the tile's 64 channels of one
-// image are one contiguous run of delta_z, read as whole vectors whatever the plane size. Otherwise,
-// plane size % V == 0: a thread takes the same V positions of two neighbouring channels and writes
-// the two codes of a position as one word. Otherwise element by element.
-// mask (fp32 tensors only, may be null): x is delta_a and the gradient is delta_a where mask != 0, else 0
-__device__ __forceinline__ void apply_mask(const unsigned char *mask, long long e, float (&v)[4]) {
-    if (mask != nullptr) {
-        const uchar4 m = __ldg(reinterpret_cast<const uchar4 *>(mask + e));
-        v[0] = m.x ? v[0] : 0.f; v[1] = m.y ? v[1] : 0.f; v[2] = m.z ? v[2] : 0.f; v[3] = m.w ? v[3] : 0.f;
-    }
-}
-__device__ __forceinline__ void apply_mask(const unsigned char *, long long, float (&)[8]) {}
+// Three ways to fill a tile:
+//   kFlat: planes smaller than a tile's 64 positions (C % 8 == 0): the tile's 64 channels of one image are one contiguous
+//          run of delta_z, read as whole vectors whatever the plane size;
+//   kPair: plane size % V == 0: a thread takes the same V positions of two neighbouring channels and writes the two codes
+//          of a position as one word;
+//   kOdd:  any other plane: a channel's row of the tile is covered by the aligned vectors that touch it (one more than a
+//          row holds), and what lies outside the row is dropped.
+// The output's rows are padded to a multiple of eight channels (the padding is not written: the copy engine never reads
+// it). The first tile's loads and dithers, and every next tile's loads, are under way before they are needed (see above).
+enum { kFlat, kPair, kOdd };
 
-// Channel counts that are no multiple of 8: rows of the output are padded to one (the padding is not written: the copy
-// engine never reads it), and small planes take the paths of large ones.
-template <typename T, int V, bool STACK, bool MASKED>
-__global__ void __launch_bounds__(kThreads)
-quantize_nhwc_kernel(const T *__restrict__ x, int B, int C, int HW, unsigned long long seed,
-                     const float *__restrict__ delta_p, unsigned short *__restrict__ out,
-                     int8_t *__restrict__ dense8, DeviceState *__restrict__ st, int count,
-                     unsigned short *__restrict__ out_stack, int plane_w, int stack_g,
-                     const unsigned char *__restrict__ mask_in) {
-    const unsigned char *mask = MASKED ? mask_in : nullptr;
+template <typename T, int V, int PATH, bool STACK, bool MASKED>
+__global__ void __launch_bounds__(kThreads, kBlocksPerSM)
+quantize_nhwc_kernel(const T *__restrict__ x, int B, int C, int HW, unsigned long long seed, const StepSource step,
+                     unsigned short *__restrict__ out, int8_t *__restrict__ dense8, DeviceState *__restrict__ st, int count,
+                     unsigned short *__restrict__ out_stack, int plane_w, const unsigned char *__restrict__ mask) {
     __shared__ __align__(16) unsigned char tile[2][kTileBytes];
-    constexpr int VV = (V > 1) ? V : 4;               // vector length of the paired path
-    constexpr int VF = Vec<T>::V;                     // vector length of the contiguous path
+    constexpr int VPR = kTP / V;                                   // kPair: vectors per channel row of the tile
+    constexpr int NI = kTC * kTP / V / kThreads;                   // vectors per thread and tile (kFlat: at most)
+    const unsigned ct = (C + kTC - 1) / kTC, pt = (HW + kTP - 1) / kTP, per_img = ct * pt, ntiles = B * per_img;
+    const int pitch = (C + 7) & ~7;
+
+    uint4 raw[NI];
+    unsigned msk[MASKED ? NI : 1];
+    unsigned long long u[NI][V / 2];
+    struct Tile { int b, c0, p0; };
+    auto tile_of = [&](unsigned t) {
+        Tile r;
+        r.b = t / per_img;
+        const unsigned rem = t - r.b * per_img;
+        r.c0 = (rem / pt) * kTC;
+        r.p0 = (rem - rem / pt * pt) * kTP;
+        return r;
+    };
+    // vector i of this thread: its first element, and whether it exists
+    auto vec_of = [&](const Tile &tl, int i, long long &e0) {
+        if (PATH == kFlat) {
+            const int v = threadIdx.x + kThreads * i, nch = C - tl.c0 < kTC ? C - tl.c0 : kTC;
+            e0 = (static_cast<long long>(tl.b) * C + tl.c0) * HW + v * V;
+            return v * V < nch * HW;
+        }
+        const int it = threadIdx.x + kThreads * (i >> 1), c = 2 * (it / VPR) + (i & 1), pv = (it % VPR) * V;
+        e0 = (static_cast<long long>(tl.b) * C + tl.c0 + c) * HW + tl.p0 + pv;
+        return tl.c0 + c < C && tl.p0 + pv < HW;
+    };
+    auto load = [&](const Tile &tl) {
+#pragma unroll
+        for (int i = 0; i < NI; ++i) {
+            long long e0;
+            const bool in = vec_of(tl, i, e0);
+            raw[i] = in ? load_raw<T, V>(x + e0) : make_uint4(0u, 0u, 0u, 0u);
+            if (MASKED) msk[i] = in ? mask_word(mask, e0) : 0u;
+        }
+    };
+    auto draw = [&](const Tile &tl) {
+#pragma unroll
+        for (int i = 0; i < NI; ++i) {
+            long long e0;
+            vec_of(tl, i, e0);
+            dithers_of<V>(e0, seed, u[i]);
+        }
+    };
+    unsigned t = blockIdx.x;
+    Tile cur = tile_of(t);
+    if (PATH != kOdd) {
+        load(cur);
+        draw(cur);
+    }
     chain_wait();
     chain_release();
-    const float delta = *delta_p;
-    const bool live = (delta > 0.f) && (delta < __int_as_float(0x7f800000));
-    const float inv = live ? __fdiv_rn(1.0f, delta) : 0.f;
-    const int ct = (C + kTC - 1) / kTC, pt = (HW + kTP - 1) / kTP;
-    const long long ntiles = static_cast<long long>(B) * ct * pt;
-    const bool flat = HW < kTP && (C & 7) == 0;
-    const int pitch = (C + 7) & ~7;
-    unsigned nnz = 0, sat = 0;
-    float nz = 0.f;
+    const float delta = step_of<kThreads>(step, st);
+    const float inv = delta > 0.f ? __fdiv_rn(1.0f, delta) : 0.f;      // Delta = 0: every code 0
+    unsigned nnz = 0, sat = 0, nz2 = 0;
     int buf = 0;
-    for (long long t = blockIdx.x; t < ntiles; t += gridDim.x, buf ^= 1) {
-        const int b = static_cast<int>(t / (ct * pt));
-        const int rem = static_cast<int>(t - static_cast<long long>(b) * ct * pt);
-        const int c0 = (rem / pt) * kTC, p0 = (rem % pt) * kTP;
+    for (; t < ntiles; buf ^= 1) {
         unsigned char *tl = tile[buf];
-        if (flat) {
-            // (b, c0 .. c0+63, every position): C % 8 == 0, so the run starts on a 16-byte boundary and on
-            // an even element, and holds a whole number of vectors
-            const int nch = C - c0 < kTC ? C - c0 : kTC;
-            const long long base = (static_cast<long long>(b) * C + c0) * HW;
-            const int nvec = nch * HW / VF;
-            for (int v = threadIdx.x; v < nvec; v += kThreads) {
-                float f[VF] = {};
-                if (live) {
-                    float a[VF];
-                    Vec<T>::load(x + base + v * VF, a);
-                    apply_mask(mask, base + v * VF, a);
-                    codes_of<VF>(a, base + v * VF, seed, inv, f, nz, sat);
-                }
-                if (dense8 != nullptr) store_bytes<VF>(dense8, base + v * VF, f);
-                int c = (v * VF) / HW, pp = v * VF - c * HW;
+        const int b = cur.b, c0 = cur.c0, p0 = cur.p0;
+        const unsigned next = t + gridDim.x;
+        const Tile nxt = tile_of(next < ntiles ? next : t);
+        if (PATH != kOdd) {
+            float f[NI][V];
 #pragma unroll
-                for (int j = 0; j < VF; ++j) {
-                    *reinterpret_cast<unsigned short *>(tl + tile_off(pp, c)) = static_cast<unsigned short>(__float_as_uint(f[j]) >> 16);
-                    if (++pp == HW) { pp = 0; ++c; }
-                }
+            for (int i = 0; i < NI; ++i) {
+                float v[V];
+                values_of(x, raw[i], v);
+                if (MASKED) apply_mask(msk[i], v);
+                decide<V>(v, u[i], inv, f[i], sat);
             }
-        } else if (V > 1) {
-            constexpr int VPR = kTP / VV;            // vectors per channel row of the tile
+            load(nxt);
 #pragma unroll
-            for (int i = 0; i < (kTC / 2 * VPR) / kThreads; ++i) {
-                const int v = threadIdx.x + kThreads * i;
-                const int c = 2 * (v / VPR), pv = (v % VPR) * VV;
-                float f0[VV] = {}, f1[VV] = {};
-                const bool in = c0 + c < C && p0 + pv < HW, in1 = in && c0 + c + 1 < C;       // HW % V == 0: whole vectors
-                const long long e0 = (static_cast<long long>(b) * C + c0 + c) * HW + p0 + pv, e1 = e0 + HW;
-                if (in && live) {
-                    float a0[VV], a1[VV];
-                    TileLoad<T, VV>::ld(x + e0, a0);
-                    if (in1) TileLoad<T, VV>::ld(x + e1, a1);
-                    apply_mask(mask, e0, a0);
-                    codes_of<VV>(a0, e0, seed, inv, f0, nz, sat);
-                    if (in1) {
-                        apply_mask(mask, e1, a1);
-                        codes_of<VV>(a1, e1, seed, inv, f1, nz, sat);
+            for (int i = 0; i < NI; ++i) {
+                long long e0;
+                if (vec_of(cur, i, e0)) {
+                    unsigned h[V / 2];
+                    pack_bf16<V>(f[i], h);
+                    count_pairs<V>(h, nz2);
+                    if (dense8 != nullptr) store_bytes<V>(dense8, e0, f[i]);
+                    if (PATH == kFlat) {
+                        const int v = threadIdx.x + kThreads * i;
+                        int c = (v * V) / HW, pp = v * V - c * HW;
+#pragma unroll
+                        for (int j = 0; j < V; ++j) {
+                            *reinterpret_cast<unsigned short *>(tl + tile_off(pp, c)) = static_cast<unsigned short>(h[j >> 1] >> (16 * (j & 1)));
+                            if (++pp == HW) { pp = 0; ++c; }
+                        }
                     }
                 }
-                if (in && dense8 != nullptr) {
-                    store_bytes<VV>(dense8, e0, f0);
-                    if (in1) store_bytes<VV>(dense8, e1, f1);
-                }
-#pragma unroll
-                for (int j = 0; j < VV; ++j)
-                    *reinterpret_cast<unsigned *>(tl + tile_off(pv + j, c)) =
-                        __byte_perm(__float_as_uint(f0[j]), __float_as_uint(f1[j]), 0x7632);
             }
+            if (PATH == kPair) {
+                // (a vector that does not exist was decided as zeros: code 0, never stored beyond the tile)
+#pragma unroll
+                for (int i = 0; i < NI / 2; ++i) {
+                    const int it = threadIdx.x + kThreads * i, c = 2 * (it / VPR), pv = (it % VPR) * V;
+#pragma unroll
+                    for (int j = 0; j < V; ++j)
+                        *reinterpret_cast<unsigned *>(tl + tile_off(pv + j, c)) =
+                            __byte_perm(__float_as_uint(f[2 * i][j]), __float_as_uint(f[2 * i + 1][j]), 0x7632);
+                }
+            }
+            if (next < ntiles) draw(nxt);
         } else {
-#pragma unroll 4
-            for (int i = 0; i < (kTC * kTP) / kThreads; ++i) {
-                const int id = threadIdx.x + kThreads * i;
-                const int c = id / kTP, pp = id % kTP;
-                float f = 0.f;
-                const bool in = c0 + c < C && p0 + pp < HW;
-                const long long e = (static_cast<long long>(b) * C + c0 + c) * HW + p0 + pp;
-                if (in && live) f = code_single((mask == nullptr || __ldg(mask + e)) ? Vec<T>::one(x + e) : 0.f, e, seed, inv, sat);
-                if (in && dense8 != nullptr) dense8[e] = static_cast<int8_t>(static_cast<int>(f));
-                nnz += f != 0.f;
-                *reinterpret_cast<unsigned short *>(tl + tile_off(pp, c)) = static_cast<unsigned short>(__float_as_uint(f) >> 16);
+            constexpr int VO = kTP / V + 1;                        // aligned vectors that may touch a row of the tile
+            const int len = HW - p0 < kTP ? HW - p0 : kTP, nch = C - c0 < kTC ? C - c0 : kTC;
+            const long long total = static_cast<long long>(B) * C * HW;
+            for (int it = threadIdx.x; it < nch * VO; it += kThreads) {
+                const int c = it / VO;
+                const long long row0 = (static_cast<long long>(b) * C + c0 + c) * HW + p0;
+                const long long e0 = (row0 & ~static_cast<long long>(V - 1)) + (it - c * VO) * V;
+                const int pp = static_cast<int>(e0 - row0);        // position of the vector's first element in the row
+                if (pp >= len) continue;
+                float v[V], f[V];
+                if (e0 + V <= total) {
+                    values_of(x, load_raw<T, V>(x + e0), v);
+                    if (MASKED) apply_mask(mask_word(mask, e0), v);
+                } else {
+#pragma unroll
+                    for (int j = 0; j < V; ++j)
+                        v[j] = e0 + j < total && (!MASKED || __ldg(mask + e0 + j)) ? Vec<T>::one(x + e0 + j) : 0.f;
+                }
+                // what lies outside the row belongs to other rows: it is not counted here, clipped or not
+#pragma unroll
+                for (int j = 0; j < V; ++j) v[j] = pp + j >= 0 && pp + j < len ? v[j] : 0.f;
+                dithers_of<V>(e0, seed, u[0]);
+                decide<V>(v, u[0], inv, f, sat);
+#pragma unroll
+                for (int j = 0; j < V; ++j)
+                    if (pp + j >= 0 && pp + j < len) {
+                        nnz += f[j] != 0.f;
+                        *reinterpret_cast<unsigned short *>(tl + tile_off(pp + j, c)) = static_cast<unsigned short>(__float_as_uint(f[j]) >> 16);
+                        if (dense8 != nullptr) dense8[e0 + j] = static_cast<int8_t>(static_cast<int>(f[j]));
+                    }
             }
         }
         __syncthreads();
@@ -453,32 +381,33 @@ quantize_nhwc_kernel(const T *__restrict__ x, int B, int C, int HW, unsigned lon
             }
         }
         // the other buffer is written next; this one again only after the next barrier
+        if (nz2 & 0x80008000u) { nnz += pairs_total(nz2); nz2 = 0; }
+        t = next;
+        cur = nxt;
     }
-    nnz += static_cast<unsigned>(nz);
-    nnz = __reduce_add_sync(kFull, nnz);
-    sat = __reduce_add_sync(kFull, sat);
-    if ((threadIdx.x & 31) == 0 && count) {
-        if (nnz) atomicAdd(&st->nnz, static_cast<unsigned long long>(nnz));
-        if (sat) atomicAdd(&st->saturated, static_cast<unsigned long long>(sat));
-    }
+    nnz += pairs_total(nz2);
+    if (count) publish_counts<kThreads>(nnz, delta > 0.f ? sat : 0u, st, nullptr);
 }
 
-template <typename T, int V>
-cudaError_t run_nhwc(dbp_ctx *ctx, const void *delta, int B, int C, int HW, unsigned long long seed, const float *delta_p,
-                     void *out, int8_t *dense8, bool count, void *out_stack, int plane_w, int stack_g, const uint8_t *mask) {
+template <typename T, int V, int PATH>
+cudaError_t run_nhwc(dbp_ctx *ctx, const void *delta, int B, int C, int HW, unsigned long long seed, const StepSource &step,
+                     void *out, int8_t *dense8, bool count, void *out_stack, int plane_w, const uint8_t *mask) {
     const long long ntiles = static_cast<long long>(B) * ((C + kTC - 1) / kTC) * ((HW + kTP - 1) / kTP);
-    long long blocks = ntiles < static_cast<long long>(ctx->sm_count) * 6 ? ntiles : static_cast<long long>(ctx->sm_count) * 6;
-    if (blocks < 1) blocks = 1;
-    const unsigned char *m = static_cast<const unsigned char *>(mask);
-    auto go = [&](auto kern, unsigned short *stack) {
+    const long long cap = static_cast<long long>(ctx->sm_count) * kBlocksPerSM, blocks = ntiles < cap ? ntiles : cap;
+    auto go = [&](auto kern) {
         return launch_chained(kern, dim3(static_cast<unsigned>(blocks)), dim3(kThreads), 0, ctx->stream,
-                              static_cast<const T *>(delta), B, C, HW, seed, delta_p, static_cast<unsigned short *>(out), dense8,
-                              ctx->state, count ? 1 : 0, stack, stack ? plane_w : 0, stack ? stack_g : 0, m);
+                              static_cast<const T *>(delta), B, C, HW, seed, step, static_cast<unsigned short *>(out), dense8,
+                              ctx->state, count ? 1 : 0, static_cast<unsigned short *>(out_stack), plane_w,
+                              static_cast<const unsigned char *>(mask));
     };
-    unsigned short *st = static_cast<unsigned short *>(out_stack);
-    if (mask != nullptr)      // fp32 only (checked by the caller)
-        return st ? go(quantize_nhwc_kernel<T, V, true, true>, st) : go(quantize_nhwc_kernel<T, V, false, true>, st);
-    return st ? go(quantize_nhwc_kernel<T, V, true, false>, st) : go(quantize_nhwc_kernel<T, V, false, false>, st);
+    if constexpr (sizeof(T) == 4) {
+        if (mask != nullptr) {
+            if constexpr (PATH == kFlat) { if (out_stack) return go(quantize_nhwc_kernel<T, V, PATH, true, true>); }
+            return go(quantize_nhwc_kernel<T, V, PATH, false, true>);
+        }
+    }
+    if constexpr (PATH == kFlat) { if (out_stack) return go(quantize_nhwc_kernel<T, V, PATH, true, false>); }
+    return go(quantize_nhwc_kernel<T, V, PATH, false, false>);
 }
 
 // ---------------------------------------------------------------- bf16 planes of odd sizes
@@ -492,58 +421,77 @@ constexpr int kOddMaxSmem = 12 * 1024;            // bytes of the staged run (pl
 template <typename T>
 __global__ void __launch_bounds__(kThreads)
 quantize_planes_odd_kernel(const T *__restrict__ x, long long nplanes, int hw, int pitch, int planes_per_run,
-                           unsigned long long seed, const float *__restrict__ delta_p, unsigned short *__restrict__ out,
+                           unsigned long long seed, const StepSource step, unsigned short *__restrict__ out,
                            int8_t *__restrict__ dense8, DeviceState *__restrict__ st, int count) {
     constexpr int V = Vec<T>::V;
+    constexpr int NP = 2;                                           // vectors of the first run loaded and drawn ahead
     __shared__ __align__(16) unsigned short run_s[kOddMaxSmem / 2];
+    const long long nruns = (nplanes + planes_per_run - 1) / planes_per_run;
+    uint4 raw[NP];
+    unsigned long long u[NP][V / 2];
+    {
+        const long long e_base = blockIdx.x * static_cast<long long>(planes_per_run) * hw, n = nplanes * hw;
+#pragma unroll
+        for (int i = 0; i < NP; ++i) {
+            const long long e0 = e_base + (threadIdx.x + kThreads * i) * V;
+            raw[i] = e0 < n ? Vec<T>::raw(x + e0) : make_uint4(0u, 0u, 0u, 0u);
+        }
+#pragma unroll
+        for (int i = 0; i < NP; ++i) dithers_of<V>(e_base + (threadIdx.x + kThreads * i) * V, seed, u[i]);
+    }
     chain_wait();
     chain_release();
-    const float delta = *delta_p;
-    const bool live = (delta > 0.f) && (delta < __int_as_float(0x7f800000));
-    const float inv = live ? __fdiv_rn(1.0f, delta) : 0.f;
-    const long long nruns = (nplanes + planes_per_run - 1) / planes_per_run;
-    unsigned sat = 0;
-    float nz = 0.f;
+    const float delta = step_of<kThreads>(step, st);
+    const float inv = delta > 0.f ? __fdiv_rn(1.0f, delta) : 0.f;      // Delta = 0: every code 0
+    unsigned sat = 0, nz2 = 0, nnz = 0;
     for (long long r = blockIdx.x; r < nruns; r += gridDim.x) {
         const long long pl0 = r * planes_per_run;
         const int np = static_cast<int>(nplanes - pl0 < planes_per_run ? nplanes - pl0 : planes_per_run);   // a multiple of 8
         const long long e_base = pl0 * hw;
         const int nvec = np * hw / V;
-        for (int v = threadIdx.x; v < nvec; v += kThreads) {
-            float f[V] = {};
-            const long long e0 = e_base + static_cast<long long>(v) * V;
-            if (live) {
-                float a[V];
-                Vec<T>::load(x + e0, a);
-                codes_of<V>(a, e0, seed, inv, f, nz, sat);
-            }
-            if (dense8 != nullptr) store_bytes<V>(dense8, e0, f);
+        auto place = [&](int v, const uint4 &q, const unsigned long long (&d)[V / 2]) {
+            float a[V], f[V];
+            unsigned h[V / 2];
+            Vec<T>::values(q, a);
+            decide<V>(a, d, inv, f, sat);
+            pack_bf16<V>(f, h);
+            count_pairs<V>(h, nz2);
+            if (dense8 != nullptr) store_bytes<V>(dense8, e_base + static_cast<long long>(v) * V, f);
             int pl = (v * V) / hw, pp = v * V - pl * hw;
 #pragma unroll
             for (int j = 0; j < V; ++j) {
-                run_s[pl * pitch + pp] = static_cast<unsigned short>(__float_as_uint(f[j]) >> 16);
+                run_s[pl * pitch + pp] = static_cast<unsigned short>(h[j >> 1] >> (16 * (j & 1)));
                 if (++pp == hw) { pp = 0; ++pl; }
             }
+        };
+        int v = threadIdx.x;
+        if (r == blockIdx.x) {
+#pragma unroll
+            for (int i = 0; i < NP; ++i, v += kThreads)
+                if (v < nvec) place(v, raw[i], u[i]);
+        }
+        for (; v < nvec; v += kThreads) {
+            const long long e0 = e_base + static_cast<long long>(v) * V;
+            const uint4 q = Vec<T>::raw(x + e0);
+            unsigned long long d[V / 2];
+            dithers_of<V>(e0, seed, d);
+            place(v, q, d);
         }
         __syncthreads();
         const int n16 = np * pitch / 8;
         uint4 *dst = reinterpret_cast<uint4 *>(out + pl0 * pitch);
         for (int i = threadIdx.x; i < n16; i += kThreads) dst[i] = reinterpret_cast<const uint4 *>(run_s)[i];
         __syncthreads();
+        if (nz2 & 0x80008000u) { nnz += pairs_total(nz2); nz2 = 0; }
     }
-    unsigned nnz = static_cast<unsigned>(nz);
-    nnz = __reduce_add_sync(kFull, nnz);
-    sat = __reduce_add_sync(kFull, sat);
-    if ((threadIdx.x & 31) == 0 && count) {
-        if (nnz) atomicAdd(&st->nnz, static_cast<unsigned long long>(nnz));
-        if (sat) atomicAdd(&st->saturated, static_cast<unsigned long long>(sat));
-    }
+    nnz += pairs_total(nz2);
+    if (count) publish_counts<kThreads>(nnz, delta > 0.f ? sat : 0u, st, nullptr);
 }
 
 }  // namespace
 
 int launch_quantize_dense(dbp_ctx *ctx, const void *delta, int dtype, long long numel,
-                          unsigned long long seed, const float *delta_p, int8_t *dense,
+                          unsigned long long seed, const StepSource &step, int8_t *dense,
                           void *planes_bf16, long long hw, long long pitch, bool count) {
     const int v = dtype == DBP_F32 ? 4 : 8;
     // odd plane sizes at a padded pitch: whole runs of planes through shared memory
@@ -559,11 +507,11 @@ int launch_quantize_dense(dbp_ctx *ctx, const void *delta, int dtype, long long 
         if (dtype == DBP_F32)
             e = launch_chained(quantize_planes_odd_kernel<float>, dim3(static_cast<unsigned>(blocks)), dim3(kThreads), 0, ctx->stream,
                                static_cast<const float *>(delta), nplanes, static_cast<int>(hw), static_cast<int>(pitch), per_run, seed,
-                               delta_p, static_cast<unsigned short *>(planes_bf16), dense, ctx->state, count ? 1 : 0);
+                               step, static_cast<unsigned short *>(planes_bf16), dense, ctx->state, count ? 1 : 0);
         else
             e = launch_chained(quantize_planes_odd_kernel<__nv_bfloat16>, dim3(static_cast<unsigned>(blocks)), dim3(kThreads), 0, ctx->stream,
                                static_cast<const __nv_bfloat16 *>(delta), nplanes, static_cast<int>(hw), static_cast<int>(pitch), per_run,
-                               seed, delta_p, static_cast<unsigned short *>(planes_bf16), dense, ctx->state, count ? 1 : 0);
+                               seed, step, static_cast<unsigned short *>(planes_bf16), dense, ctx->state, count ? 1 : 0);
         return cuda_ok(e);
     }
     long long blocks = (numel / v + 2 * kThreads - 1) / (2 * kThreads);
@@ -574,33 +522,35 @@ int launch_quantize_dense(dbp_ctx *ctx, const void *delta, int dtype, long long 
     cudaError_t e;
     if (dtype == DBP_F32)
         e = launch_chained(quantize_dense_kernel<float>, dim3(static_cast<unsigned>(blocks)), dim3(kThreads), 0, ctx->stream,
-                           static_cast<const float *>(delta), numel, seed, delta_p, out, ctx->state);
+                           static_cast<const float *>(delta), numel, seed, step, out, ctx->state);
     else
         e = launch_chained(quantize_dense_kernel<__nv_bfloat16>, dim3(static_cast<unsigned>(blocks)), dim3(kThreads), 0,
-                           ctx->stream, static_cast<const __nv_bfloat16 *>(delta), numel, seed, delta_p, out, ctx->state);
+                           ctx->stream, static_cast<const __nv_bfloat16 *>(delta), numel, seed, step, out, ctx->state);
     return cuda_ok(e);
 }
 
 // delta_z [B][C][HW] -> bf16 codes [B][HW][C rounded up to a multiple of 8] and, when dense8 is not null, int8 codes
 // in delta_z's order
 int launch_quantize_nhwc(dbp_ctx *ctx, const void *delta, int dtype, long long B, long long C, long long HW,
-                         unsigned long long seed, const float *delta_p, void *codes_nhwc, int8_t *dense8, bool count,
-                         void *codes_stack, int plane_w, int stack_g, const uint8_t *mask) {
+                         unsigned long long seed, const StepSource &step, void *codes_nhwc, int8_t *dense8, bool count,
+                         void *codes_stack, int plane_w, const uint8_t *mask) {
     if (B * C * HW >= (1ll << 40) || HW >= (1ll << 30)) return DBP_EUNSUPPORTED;
+    if (B * ((C + kTC - 1) / kTC) * ((HW + kTP - 1) / kTP) >= (1ll << 31)) return DBP_EUNSUPPORTED;
     if (mask != nullptr && dtype != DBP_F32) return DBP_EUNSUPPORTED;
     // the stacked copy is written by the path for planes smaller than a tile; the rows of image b start at
     // b (HW + W) however many images make up a tall image: the stacking only adds the zero rows
-    if (codes_stack != nullptr && (HW >= kTP || C % 8 != 0 || plane_w <= 0 || stack_g <= 0 || HW + plane_w > kTP)) return DBP_EINVAL;
+    if (codes_stack != nullptr && (HW >= kTP || C % 8 != 0 || plane_w <= 0 || HW + plane_w > kTP)) return DBP_EINVAL;
     const int b = static_cast<int>(B), c = static_cast<int>(C), hw = static_cast<int>(HW);
-    cudaError_t e;
+    const bool flat = HW < kTP && C % 8 == 0;
+    auto run = [&](auto kern) { return kern(ctx, delta, b, c, hw, seed, step, codes_nhwc, dense8, count, codes_stack, plane_w, mask); };
     if (dtype == DBP_F32)
-        e = hw % 4 == 0 ? run_nhwc<float, 4>(ctx, delta, b, c, hw, seed, delta_p, codes_nhwc, dense8, count, codes_stack, plane_w, stack_g, mask)
-                        : run_nhwc<float, 1>(ctx, delta, b, c, hw, seed, delta_p, codes_nhwc, dense8, count, codes_stack, plane_w, stack_g, mask);
-    else
-        e = hw % 8 == 0   ? run_nhwc<__nv_bfloat16, 8>(ctx, delta, b, c, hw, seed, delta_p, codes_nhwc, dense8, count, codes_stack, plane_w, stack_g, mask)
-            : hw % 4 == 0 ? run_nhwc<__nv_bfloat16, 4>(ctx, delta, b, c, hw, seed, delta_p, codes_nhwc, dense8, count, codes_stack, plane_w, stack_g, mask)
-                          : run_nhwc<__nv_bfloat16, 1>(ctx, delta, b, c, hw, seed, delta_p, codes_nhwc, dense8, count, codes_stack, plane_w, stack_g, mask);
-    return cuda_ok(e);
+        return cuda_ok(flat          ? run(run_nhwc<float, 4, kFlat>)
+                       : hw % 4 == 0 ? run(run_nhwc<float, 4, kPair>)
+                                     : run(run_nhwc<float, 4, kOdd>));
+    return cuda_ok(flat          ? run(run_nhwc<__nv_bfloat16, 8, kFlat>)
+                   : hw % 8 == 0 ? run(run_nhwc<__nv_bfloat16, 8, kPair>)
+                   : hw % 4 == 0 ? run(run_nhwc<__nv_bfloat16, 4, kPair>)
+                                 : run(run_nhwc<__nv_bfloat16, 8, kOdd>));
 }
 
 }  // namespace dbp

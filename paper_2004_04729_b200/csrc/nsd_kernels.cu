@@ -3,74 +3,29 @@
 //
 // Both streaming kernels are bound by HBM bandwidth: 128-bit loads of delta_z, 128-bit stores
 // of the packed codes, bitmap words and offsets assembled with warp shuffles.
-#include "dbp_internal.cuh"
+#include "nsd_common.cuh"
 
 namespace dbp {
 
 namespace {
 
+using namespace nsd;
+
 constexpr int kThreads = 256;
-constexpr unsigned kFull = 0xffffffffu;
 
-template <typename T>
-struct Elem;
-
-template <>
-struct Elem<float> {
-    static constexpr int EPT = 4;  // elements per 128-bit load
-    __device__ static void load(const float *p, float (&v)[4]) {
-        float4 q = __ldg(reinterpret_cast<const float4 *>(p));
-        v[0] = q.x; v[1] = q.y; v[2] = q.z; v[3] = q.w;
-    }
-    __device__ static float one(const float *p) { return __ldg(p); }
-    // read-once data: do not keep the line in L1
-    __device__ static void load_stream(const float *p, float (&v)[4]) {
-        unsigned a, b, c, d;
-        asm volatile("ld.global.nc.L1::no_allocate.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(a), "=r"(b), "=r"(c), "=r"(d) : "l"(p));
-        v[0] = __uint_as_float(a); v[1] = __uint_as_float(b); v[2] = __uint_as_float(c); v[3] = __uint_as_float(d);
-    }
-};
-
-template <>
-struct Elem<__nv_bfloat16> {
-    static constexpr int EPT = 8;
-    __device__ static void load(const __nv_bfloat16 *p, float (&v)[8]) {
-        uint4 q = __ldg(reinterpret_cast<const uint4 *>(p));
-        const unsigned w[4] = {q.x, q.y, q.z, q.w};
-#pragma unroll
-        for (int i = 0; i < 4; ++i) {
-            v[2 * i] = __uint_as_float(w[i] << 16);           // bf16 -> fp32 is exact
-            v[2 * i + 1] = __uint_as_float(w[i] & 0xffff0000u);
-        }
-    }
-    __device__ static float one(const __nv_bfloat16 *p) {
-        return __uint_as_float(static_cast<unsigned>(__ldg(reinterpret_cast<const unsigned short *>(p))) << 16);
-    }
-    __device__ static void load_stream(const __nv_bfloat16 *p, float (&v)[8]) {
-        unsigned w[4];
-        asm volatile("ld.global.nc.L1::no_allocate.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(w[0]), "=r"(w[1]), "=r"(w[2]), "=r"(w[3]) : "l"(p));
-#pragma unroll
-        for (int i = 0; i < 4; ++i) {
-            v[2 * i] = __uint_as_float(w[i] << 16);
-            v[2 * i + 1] = __uint_as_float(w[i] & 0xffff0000u);
-        }
-    }
-};
-
-__device__ __forceinline__ double warp_sum(double v) {
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(kFull, v, o);
-    return v;
+// read-once data: do not keep the line in L1
+__device__ __forceinline__ uint4 load_stream(const void *p) {
+    uint4 q;
+    asm volatile("ld.global.nc.L1::no_allocate.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(q.x), "=r"(q.y), "=r"(q.z), "=r"(q.w) : "l"(p));
+    return q;
 }
 
 // ---------------------------------------------------------------- statistics (sigma, Delta)
 // Sum and sum of squares of every element's distance from a pivot (the tensor's first element):
-// fp32 inside one 128-bit chunk, fp64 across chunks, per-block partials combined in a fixed order
-// by the last block to finish, so the step size does not depend on scheduling. The variance is
-// shift-invariant, and with the pivot inside the data's range the moments stay of the order of
-// sigma: a constant tensor gives exactly 0 and a mean far from 0 costs no accuracy (raw moments
-// would cancel). sigma is the population standard deviation about the mean; Delta = scale * sigma
-// rounded once to fp32.
+// fp32 inside one 128-bit chunk, fp64 across chunks, one pair of partial sums per block; the quantizer that follows adds
+// the blocks' sums up in a fixed order (step_of, nsd_common.cuh), so the step size does not depend on scheduling. The
+// variance is shift-invariant, and with the pivot inside the data's range the moments stay of the order of sigma: a
+// constant tensor gives exactly 0 and a mean far from 0 costs no accuracy (raw moments would cancel).
 // MASKED (fp32 only): the tensor is delta_a and the statistics are those of delta_a where mask != 0, else 0 (the
 // ReLU derivative folded into the read; one byte per element).
 template <bool MASKED>
@@ -123,6 +78,12 @@ __device__ __forceinline__ void rows_job(const RowsJob &j, long long first, long
             *reinterpret_cast<uint4 *>(dst) = make_uint4(h[0], h[1], h[2], h[3]);
             *reinterpret_cast<uint4 *>(dst + piece) = make_uint4(l[0], l[1], l[2], l[3]);
         } else {
+            if (left >= 8 && (j.cols & 3) == 0) {                     // rows start on 8-byte boundaries
+                const unsigned short *src8 = static_cast<const unsigned short *>(j.src) + row * j.cols + c0;
+                const uint2 a = __ldg(reinterpret_cast<const uint2 *>(src8)), b = __ldg(reinterpret_cast<const uint2 *>(src8 + 4));
+                *reinterpret_cast<uint4 *>(dst) = make_uint4(a.x, a.y, b.x, b.y);
+                continue;
+            }
             // 32-bit loads whatever the row's start: a row that starts on an odd element is shifted by half a word
             const long long off = row * j.cols + c0, total = j.rows * j.cols;
             const unsigned short *src = static_cast<const unsigned short *>(j.src);
@@ -158,9 +119,9 @@ __global__ void __launch_bounds__(kThreads) rows_job_kernel(const RowsJob j, int
 template <typename T, bool MASKED = false>
 __global__ void __launch_bounds__(kThreads)
 statistics_kernel(const T *__restrict__ x, long long n, double *__restrict__ partials,
-                  DeviceState *__restrict__ st, float scale, float *__restrict__ delta_out,
-                  unsigned long long *__restrict__ nnz_out, const unsigned char *__restrict__ mask, const SideJobs jobs) {
-    constexpr int EPT = Elem<T>::EPT;
+                  DeviceState *__restrict__ st, unsigned long long *__restrict__ nnz_out,
+                  const unsigned char *__restrict__ mask, const SideJobs jobs) {
+    constexpr int EPT = Vec<T>::V;
     const long long nvec = n / EPT;
     chain_wait();
     chain_release();
@@ -230,7 +191,11 @@ statistics_kernel(const T *__restrict__ x, long long n, double *__restrict__ par
         }
     }
     double d1 = 0.0, d2 = 0.0;
-    const float pivot = (!MASKED || __ldg(mask)) ? Elem<T>::one(x) : 0.f;
+    if (blockIdx.x == 0 && threadIdx.x == 0) {      // the quantizer counts into these
+        st->nnz = 0ull;
+        if (nnz_out) *nnz_out = 0ull;
+    }
+    const float pivot = (!MASKED || __ldg(mask)) ? Vec<T>::one(x) : 0.f;
     const long long stride = static_cast<long long>(gridDim.x) * kThreads;
     // whole tiles of kUnroll x kThreads 128-bit vectors, a block at a time: kUnroll loads in flight
     // per thread, consecutive threads on consecutive vectors
@@ -240,7 +205,7 @@ statistics_kernel(const T *__restrict__ x, long long n, double *__restrict__ par
         const T *p = x + (t * tile + threadIdx.x) * EPT;
         float v[kUnroll][EPT];
 #pragma unroll
-        for (int u = 0; u < kUnroll; ++u) Elem<T>::load_stream(p + static_cast<long long>(u) * kThreads * EPT, v[u]);
+        for (int u = 0; u < kUnroll; ++u) Vec<T>::values(load_stream(p + static_cast<long long>(u) * kThreads * EPT), v[u]);
 #pragma unroll
         for (int u = 0; u < kUnroll; ++u) mask4<MASKED>(mask, (t * tile + threadIdx.x + static_cast<long long>(u) * kThreads) * EPT, v[u]);
 #pragma unroll
@@ -260,7 +225,7 @@ statistics_kernel(const T *__restrict__ x, long long n, double *__restrict__ par
     long long i = ntile * tile + static_cast<long long>(blockIdx.x) * kThreads + threadIdx.x;
     for (; i < nvec; i += stride) {
         float v[EPT];
-        Elem<T>::load(x + i * EPT, v);
+        Vec<T>::values(Vec<T>::raw(x + i * EPT), v);
         mask4<MASKED>(mask, i * EPT, v);
         float s1 = 0.f, s2 = 0.f;
 #pragma unroll
@@ -274,14 +239,13 @@ statistics_kernel(const T *__restrict__ x, long long n, double *__restrict__ par
     }
     if (blockIdx.x == 0 && threadIdx.x == 0) {
         for (long long i = nvec * EPT; i < n; ++i) {
-            const float xi = (!MASKED || __ldg(mask + i)) ? Elem<T>::one(x + i) : 0.f;
+            const float xi = (!MASKED || __ldg(mask + i)) ? Vec<T>::one(x + i) : 0.f;
             const double c = static_cast<double>(xi) - static_cast<double>(pivot);
             d1 += c;
             d2 += c * c;
         }
     }
     __shared__ double sh1[kThreads / 32], sh2[kThreads / 32];
-    __shared__ bool is_last;
     d1 = warp_sum(d1);
     d2 = warp_sum(d2);
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -290,236 +254,149 @@ statistics_kernel(const T *__restrict__ x, long long n, double *__restrict__ par
     if (threadIdx.x == 0) {
         double a = 0.0, b = 0.0;
         for (int w = 0; w < kThreads / 32; ++w) { a += sh1[w]; b += sh2[w]; }
-        partials[2 * blockIdx.x] = a;
-        partials[2 * blockIdx.x + 1] = b;
-        __threadfence();
-        const unsigned t = atomicAdd(&st->ticket, 1u);
-        is_last = (t == gridDim.x - 1);
-    }
-    __syncthreads();
-    if (!is_last) return;
-    // the last block adds the partials: every thread a strided share (loads independent of one
-    // another), then warps and the block in a fixed order
-    __threadfence();
-    double a = 0.0, b = 0.0;
-#pragma unroll 4
-    for (int blk = threadIdx.x; blk < static_cast<int>(gridDim.x); blk += kThreads) {
-        a += __ldcg(partials + 2 * blk);
-        b += __ldcg(partials + 2 * blk + 1);
-    }
-    a = warp_sum(a);
-    b = warp_sum(b);
-    __syncthreads();                 // sh1/sh2 were read by thread 0 above
-    if (lane == 0) { sh1[warp] = a; sh2[warp] = b; }
-    __syncthreads();
-    if (warp != 0) return;
-    a = 0.0; b = 0.0;
-    for (int w = 0; w < kThreads / 32; ++w) { a += sh1[w]; b += sh2[w]; }
-    if (lane == 0) {
-        float delta = 0.f;
-        if (!isfinite(a) || !isfinite(b)) {
-            st->nonfinite = 1;                      // every code becomes 0
-        } else {
-            const double mean = a / static_cast<double>(n);
-            double var = b / static_cast<double>(n) - mean * mean;
-            if (var < 0.0) var = 0.0;
-            delta = static_cast<float>(static_cast<double>(scale) * sqrt(var));
-        }
-        st->delta = delta;
-        st->nnz = 0ull;
-        st->ticket = 0u;
-        if (delta_out) *delta_out = delta;
-        if (nnz_out) *nnz_out = 0ull;
+        reinterpret_cast<double2 *>(partials)[blockIdx.x] = make_double2(a, b);
     }
 }
 
-__global__ void set_step_kernel(const float *__restrict__ delta_in, DeviceState *st,
-                                float *delta_out, unsigned long long *nnz_out) {
-    const float d = *delta_in;
-    st->delta = d;
+// A given step size: no statistics; the counters the quantizer adds to are cleared.
+__global__ void clear_counts_kernel(DeviceState *st, unsigned long long *nnz_out) {
+    chain_wait();
+    chain_release();
     st->nnz = 0ull;
-    if (delta_out) *delta_out = d;
     if (nnz_out) *nnz_out = 0ull;
 }
 
 // ---------------------------------------------------------------- dither + quantize + compact
-// SplitMix64 output number c of the sequence started at `seed` (counter-based: no state).
-__device__ __forceinline__ unsigned long long splitmix64_mix(unsigned long long z) {
-    z = (z ^ (z >> 30)) * 0xBF58476D1CE4E5B9ull;
-    z = (z ^ (z >> 27)) * 0x94D049BB133111EBull;
-    return z ^ (z >> 31);
-}
+// One warp owns one 1024-element segment at a time, one lane 32 consecutive elements of it: one bitmap word, so a word
+// and its popcount need no exchange between lanes, and one scan per segment gives every word's offset. The codes of a
+// lane are dumped to shared memory as bytes and the non-zero ones are picked out by walking the word's bits (a few per
+// lane at the sparsities this is used at); the segment leaves as coalesced stores of the 32 words, the 32 offsets and
+// the packed codes.
+constexpr int kLanePitch = 36;                    // bytes between two lanes' codes: an odd number of words
 
-// u = (2k+1) 2^-24 from the top 23 bits k of h: (1 + k 2^-23) - (1 - 2^-24), exact.
-__device__ __forceinline__ float dither_from_bits(unsigned h) {
-    return __uint_as_float(0x3f800000u | (h >> 9)) - 0.99999994f;
-}
-
-// q = floor(x / Delta + u) with one rounding, clipped to [-127, 127]; NaN gives 0.
-// floor and the conversion to int are one round-down addition of 1.5 * 2^23 (exact for the
-// clamped range) and an integer subtraction.
-__device__ __forceinline__ int quantize_one(float x, float inv, float u, unsigned &sat) {
-    const float t = __fmaf_rn(x, inv, u);
-    const float tc = fminf(fmaxf(t, -127.f), 127.99999f);
-    const bool num = (t == t);
-    sat += (num && tc != t) ? 1u : 0u;
-    const int q = __float_as_int(__fadd_rd(tc, 12582912.0f)) - 0x4B400000;
-    return num ? q : 0;
-}
-
-// One warp owns one 1024-element segment at a time: ITER 128-bit loads per lane, codes
-// packed through a per-warp shared staging line, one coalesced store each of the 32 bitmap
-// words, the 32 offsets and the packed codes.
 template <typename T>
 __global__ void __launch_bounds__(kThreads)
-quantize_kernel(const T *__restrict__ x, long long n, unsigned long long seed,
-                const float *__restrict__ delta_p, uint32_t *__restrict__ bitmap,
-                uint16_t *__restrict__ offsets, int8_t *__restrict__ values,
-                int8_t *__restrict__ dense, DeviceState *__restrict__ st,
-                unsigned long long *__restrict__ nnz_out) {
-    constexpr int EPT = Elem<T>::EPT;
-    constexpr int ITER = kSegment / (32 * EPT);  // 8 (fp32) or 4 (bf16)
-    constexpr int LPW = 32 / EPT;                // lanes that share one bitmap word
-    constexpr int NW = EPT / 4;                  // packed code words per lane and iteration
-    __shared__ __align__(16) int8_t stage[kThreads / 32][kSegment];
-
+quantize_kernel(const T *__restrict__ x, long long n, unsigned long long seed, const StepSource step,
+                uint32_t *__restrict__ bitmap, uint16_t *__restrict__ offsets, int8_t *__restrict__ values,
+                int8_t *__restrict__ dense, DeviceState *__restrict__ st, unsigned long long *__restrict__ nnz_out) {
+    constexpr int V = Vec<T>::V;
+    constexpr int NV = 32 / V;                                       // vectors per lane and segment
+    __shared__ __align__(16) unsigned char stage[kThreads / 32][kSegment];
+    __shared__ __align__(16) unsigned char byte_s[kThreads / 32][32 * kLanePitch];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const long long nseg = (n + kSegment - 1) / kSegment;
     const long long nwarps = static_cast<long long>(gridDim.x) * (kThreads / 32);
-    const long long first = static_cast<long long>(blockIdx.x) * (kThreads / 32) + warp;
-    const float delta = *delta_p;
-    const bool live = (delta > 0.f) && (delta < __int_as_float(0x7f800000));
-    if (!live) {   // sigma = 0 or non-finite input: every code is 0
-        for (long long seg = first; seg < nseg; seg += nwarps) {
-            bitmap[seg * kWordsPerSegment + lane] = 0u;
-            offsets[seg * kWordsPerSegment + lane] = 0;
-            if (dense != nullptr) {
-                const long long e0 = seg * kSegment + lane * 32;
-                if (e0 + 32 <= n) {
-                    reinterpret_cast<uint4 *>(dense + e0)[0] = make_uint4(0u, 0u, 0u, 0u);
-                    reinterpret_cast<uint4 *>(dense + e0)[1] = make_uint4(0u, 0u, 0u, 0u);
-                } else {
-                    for (int j = 0; j < 32; ++j)
-                        if (e0 + j < n) dense[e0 + j] = 0;
-                }
+    long long seg = static_cast<long long>(blockIdx.x) * (kThreads / 32) + warp;
+    uint4 raw[NV];
+    auto load = [&](long long sg) {
+        const long long e0 = sg * kSegment + lane * 32;
+#pragma unroll
+        for (int i = 0; i < NV; ++i) raw[i] = e0 + (i + 1) * V <= n ? Vec<T>::raw(x + e0 + i * V) : make_uint4(0u, 0u, 0u, 0u);
+    };
+    load(seg < nseg ? seg : 0);
+    chain_wait();
+    chain_release();
+    const float delta = step_of<kThreads>(step, st);
+    const float inv = delta > 0.f ? __fdiv_rn(1.0f, delta) : 0.f;      // Delta = 0: every code 0
+    unsigned nnz = 0, sat = 0;
+    for (; seg < nseg; seg += nwarps) {
+        const long long e0 = seg * kSegment + lane * 32;
+        unsigned word = 0, pk[8];
+#pragma unroll
+        for (int i = 0; i < NV; ++i) {
+            float v[V], f[V];
+            Vec<T>::values(raw[i], v);
+            const long long e = e0 + i * V;
+            if (e < n && e + V > n)                                  // the tensor's last, partial vector
+#pragma unroll
+                for (int j = 0; j < V; ++j) v[j] = e + j < n ? Vec<T>::one(x + e + j) : 0.f;
+            unsigned long long u[V / 2];
+            dithers_of<V>(e, seed, u);
+            decide<V>(v, u, inv, f, sat);                            // elements past the end were read as 0: code 0
+            unsigned b[V / 4];
+            pack_bytes<V>(f, b);
+#pragma unroll
+            for (int w = 0; w < V / 4; ++w) {
+                pk[i * (V / 4) + w] = b[w];
+                // one bit per non-zero byte: bit 7 of each byte, gathered by a multiplication
+                const unsigned y = (((b[w] & 0x7f7f7f7fu) + 0x7f7f7f7fu) | b[w]) & 0x80808080u;
+                word |= ((y >> 7) * 0x01020408u >> 24) << (i * V + 4 * w);
             }
         }
-        return;
-    }
-    const float inv = __fdiv_rn(1.0f, delta);
-    const int sub = lane % LPW;                  // my position inside the word
-    unsigned long long nnz_local = 0ull;
-    unsigned sat = 0;
-
-    for (long long seg = first; seg < nseg; seg += nwarps) {
-        const bool full = (seg + 1) * kSegment <= n;
-        unsigned running = 0, my_word = 0, my_off = 0;
+        if (seg + nwarps < nseg) load(seg + nwarps);
+        const unsigned pc = __popc(word);
+        unsigned incl = pc;
 #pragma unroll
-        for (int it = 0; it < ITER; ++it) {
-            const long long e0 = seg * kSegment + it * (32 * EPT) + lane * EPT;
-            float v[EPT];
-            if (full || e0 + EPT <= n) {
-                Elem<T>::load(x + e0, v);
+        for (int o = 1; o < 32; o <<= 1) {
+            const unsigned up = __shfl_up_sync(kFull, incl, o);
+            if (lane >= o) incl += up;
+        }
+        const unsigned total = __shfl_sync(kFull, incl, 31);
+        bitmap[seg * kWordsPerSegment + lane] = word;
+        offsets[seg * kWordsPerSegment + lane] = static_cast<uint16_t>(incl - pc);
+        unsigned *mine = reinterpret_cast<unsigned *>(byte_s[warp] + lane * kLanePitch);
+#pragma unroll
+        for (int w = 0; w < 8; ++w) mine[w] = pk[w];
+        if (dense != nullptr) {
+            if (e0 + 32 <= n) {
+                reinterpret_cast<uint4 *>(dense + e0)[0] = make_uint4(pk[0], pk[1], pk[2], pk[3]);
+                reinterpret_cast<uint4 *>(dense + e0)[1] = make_uint4(pk[4], pk[5], pk[6], pk[7]);
             } else {
-#pragma unroll
-                for (int j = 0; j < EPT; ++j) v[j] = (e0 + j < n) ? Elem<T>::one(x + e0 + j) : 0.f;
+                for (int j = 0; j < 32; ++j)
+                    if (e0 + j < n) dense[e0 + j] = static_cast<int8_t>(reinterpret_cast<const unsigned char *>(mine)[j]);
             }
-            unsigned pk[NW];
-#pragma unroll
-            for (int w = 0; w < NW; ++w) pk[w] = 0u;
-            unsigned bits = 0;
-            unsigned long long z = seed + (static_cast<unsigned long long>(e0 >> 1) + 1ull) * 0x9E3779B97F4A7C15ull;
-#pragma unroll
-            for (int j = 0; j < EPT; j += 2) {
-                const unsigned long long r = splitmix64_mix(z);
-                z += 0x9E3779B97F4A7C15ull;
-                const int q0 = quantize_one(v[j], inv, dither_from_bits(static_cast<unsigned>(r)), sat);
-                const int q1 = quantize_one(v[j + 1], inv, dither_from_bits(static_cast<unsigned>(r >> 32)), sat);
-                pk[j >> 2] |= (static_cast<unsigned>(q0) & 0xffu) << (8 * (j & 3));
-                pk[j >> 2] |= (static_cast<unsigned>(q1) & 0xffu) << (8 * ((j + 1) & 3));
-                bits |= (q0 != 0 ? 1u : 0u) << j;
-                bits |= (q1 != 0 ? 1u : 0u) << (j + 1);
-            }
-            if (!full) {   // elements past the end carry no code (their x was read as 0 already)
-#pragma unroll
-                for (int j = 0; j < EPT; ++j)
-                    if (e0 + j >= n) { bits &= ~(1u << j); pk[j >> 2] &= ~(0xffu << (8 * (j & 3))); }
-            }
-            // bitmap word shared by LPW consecutive lanes
-            unsigned word = bits << (EPT * sub);
-#pragma unroll
-            for (int o = 1; o < LPW; o <<= 1) word |= __shfl_xor_sync(kFull, word, o);
-            // exclusive rank of my first code inside the segment: warp scan of the lane counts
-            const unsigned pc = __popc(bits);
-            unsigned incl = pc;
-#pragma unroll
-            for (int o = 1; o < 32; o <<= 1) {
-                const unsigned up = __shfl_up_sync(kFull, incl, o);
-                if (lane >= o) incl += up;
-            }
-            const unsigned total = __shfl_sync(kFull, incl, 31);
-            unsigned rank = running + incl - pc;
-            const unsigned word_off = rank;      // for a word's first lane: codes before the word
-            // non-zero codes to the staging line, in element order
-            unsigned b = bits;
-            while (b) {
-                const int j = __ffs(b) - 1;
-                b &= b - 1;
-                const unsigned wsel = (NW == 1 || j < 4) ? pk[0] : pk[NW - 1];
-                stage[warp][rank++] = static_cast<int8_t>((wsel >> (8 * (j & 3))) & 0xffu);
-            }
-            if (dense != nullptr) {
-                if (full || e0 + EPT <= n) {
-                    if (EPT == 4) *reinterpret_cast<unsigned *>(dense + e0) = pk[0];
-                    else *reinterpret_cast<uint2 *>(dense + e0) = make_uint2(pk[0], pk[NW - 1]);
-                } else {
-#pragma unroll
-                    for (int j = 0; j < EPT; ++j)
-                        if (e0 + j < n) dense[e0 + j] = static_cast<int8_t>((pk[j >> 2] >> (8 * (j & 3))) & 0xffu);
-                }
-            }
-            // lane (it*EPT + w) keeps word w of this iteration and its offset
-            const unsigned wv = __shfl_sync(kFull, word, (lane % EPT) * LPW);
-            const unsigned ov = __shfl_sync(kFull, word_off, (lane % EPT) * LPW);
-            if (lane / EPT == it) { my_word = wv; my_off = ov; }
-            running += total;
         }
+        unsigned char *dst = stage[warp] + (incl - pc);
+        const unsigned char *src = reinterpret_cast<const unsigned char *>(mine);
+        for (unsigned m = word; m; m &= m - 1) *dst++ = src[__ffs(m) - 1];
         __syncwarp();
-        bitmap[seg * kWordsPerSegment + lane] = my_word;
-        offsets[seg * kWordsPerSegment + lane] = static_cast<uint16_t>(my_off);
-        for (unsigned i = lane * 16; i < running; i += 512)
-            *reinterpret_cast<uint4 *>(values + seg * kSegment + i) =
-                *reinterpret_cast<const uint4 *>(&stage[warp][i]);
+        for (unsigned i = lane * 16; i < total; i += 512)
+            *reinterpret_cast<uint4 *>(values + seg * kSegment + i) = *reinterpret_cast<const uint4 *>(&stage[warp][i]);
         __syncwarp();
-        nnz_local += running;
+        nnz += lane == 0 ? total : 0u;
     }
-    sat = __reduce_add_sync(kFull, sat);
-    if (lane == 0) {
-        if (nnz_local) {
-            atomicAdd(&st->nnz, nnz_local);
-            if (nnz_out) atomicAdd(nnz_out, nnz_local);
-        }
-        if (sat) atomicAdd(&st->saturated, static_cast<unsigned long long>(sat));
-    }
+    publish_counts<kThreads>(nnz, delta > 0.f ? sat : 0u, st, nnz_out);
 }
 
-// One warp per segment, one lane per bitmap word: 32 codes written as two 128-bit stores.
+// One warp per segment, one lane per bitmap word. The segment's packed codes come in as whole lines; a lane takes its
+// word four bits at a time: the next codes (a 32-bit window at the running rank, from two words of shared memory) are
+// spread to the bytes whose bits are set by one byte permutation, whose selector for the sixteen patterns is a table.
 __global__ void __launch_bounds__(kThreads)
 decode_kernel(const uint32_t *__restrict__ bitmap, const uint16_t *__restrict__ offsets,
               const int8_t *__restrict__ values, long long n, int8_t *__restrict__ dense) {
-    const int lane = threadIdx.x & 31;
+    __shared__ __align__(16) unsigned char stage[kThreads / 32][kSegment + 16];
+    __shared__ unsigned sel_s[16];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    if (threadIdx.x < 16) {
+        unsigned sel = 0, r = 0;
+        for (int b = 0; b < 4; ++b) sel |= ((threadIdx.x >> b) & 1 ? r++ : 4u) << (4 * b);      // selector 4: a zero byte
+        sel_s[threadIdx.x] = sel;
+    }
+    __syncthreads();
+    chain_wait();
+    chain_release();
     const long long nseg = (n + kSegment - 1) / kSegment;
     const long long nwarps = static_cast<long long>(gridDim.x) * (kThreads / 32);
-    for (long long seg = static_cast<long long>(blockIdx.x) * (kThreads / 32) + (threadIdx.x >> 5); seg < nseg; seg += nwarps) {
+    for (long long seg = static_cast<long long>(blockIdx.x) * (kThreads / 32) + warp; seg < nseg; seg += nwarps) {
         const long long w = seg * kWordsPerSegment + lane;
-        unsigned word = bitmap[w];
-        const int8_t *src = values + seg * kSegment + offsets[w];
-        unsigned pk[8] = {0, 0, 0, 0, 0, 0, 0, 0};
-        while (word) {
-            const int b = __ffs(word) - 1;
-            word &= word - 1;
-            pk[b >> 2] |= (static_cast<unsigned>(*src++) & 0xffu) << (8 * (b & 3));
+        const unsigned word = __ldcg(bitmap + w), off = __ldcg(offsets + w);
+        // a first line is on its way with the words: at the usual sparsities the segment has few more
+        uint4 *line = reinterpret_cast<uint4 *>(stage[warp]);
+        const uint4 *src = reinterpret_cast<const uint4 *>(values + seg * kSegment);
+        if (lane < 8) line[lane] = __ldcg(src + lane);
+        const unsigned total = __shfl_sync(kFull, off + __popc(word), 31);
+        for (unsigned i = lane + 8; i * 16 < total; i += 32) line[i] = __ldcg(src + i);
+        __syncwarp();
+        const unsigned *codes = reinterpret_cast<const unsigned *>(stage[warp]);
+        unsigned pk[8], r = off;
+#pragma unroll
+        for (int g = 0; g < 8; ++g) {
+            const unsigned m = (word >> (4 * g)) & 15u;
+            const unsigned win = __funnelshift_r(codes[r >> 2], codes[(r >> 2) + 1], 8 * (r & 3));
+            pk[g] = __byte_perm(win, 0u, sel_s[m]);
+            r += __popc(m);
         }
+        __syncwarp();
         const long long e0 = w * 32;
         if (e0 + 32 <= n) {
             uint4 *dst = reinterpret_cast<uint4 *>(dense + e0);
@@ -543,16 +420,18 @@ int launch_rows_job(dbp_ctx *ctx, const RowsJob &job, bool beside) {
 }
 
 int launch_statistics(dbp_ctx *ctx, const void *delta, int dtype, long long numel, float scale,
-                      const float *delta_in, float *delta_out, unsigned long long *nnz_out, const SideJobs &jobs,
-                      const uint8_t *mask) {
+                      const float *delta_in, float *const (&publish)[2], unsigned long long *nnz_out, StepSource *step,
+                      const SideJobs &jobs, const uint8_t *mask) {
     if (mask != nullptr && dtype != DBP_F32) return DBP_EUNSUPPORTED;
+    step->publish[0] = &ctx->state->delta;
+    step->publish[1] = publish[0];
+    step->publish[2] = publish[1];
     if (!(scale > 0.f)) {      // the step size is given: no statistics kernel, so no side jobs either (the caller sees to the weights)
         if (jobs.zero && cudaMemsetAsync(jobs.zero, 0, jobs.zero_bytes, ctx->stream) != cudaSuccess) return fail_cuda("clearing dW");
         for (int j = 0; j < jobs.nrows; ++j)
             if (int rc = launch_rows_job(ctx, jobs.rows[j], false)) return rc;
-        note_launch();
-        set_step_kernel<<<1, 1, 0, ctx->stream>>>(delta_in, ctx->state, delta_out, nnz_out);
-        return cuda_ok(cudaGetLastError());
+        step->given = delta_in;
+        return cuda_ok(launch_chained(clear_counts_kernel, dim3(1), dim3(1), 0, ctx->stream, ctx->state, nnz_out));
     }
     const int ept = dtype == DBP_F32 ? 4 : 8;
     long long blocks = numel / ept / (kThreads * 8);          // one block per tile of eight vectors per thread
@@ -572,8 +451,12 @@ int launch_statistics(dbp_ctx *ctx, const void *delta, int dtype, long long nume
         blocks = static_cast<long long>(ctx->sm_count) * kStatBlocksPerSM;
     auto go = [&](auto kern, auto x, const unsigned char *m) {
         return launch_chained(kern, dim3(static_cast<unsigned>(blocks)), dim3(kThreads), 0, ctx->stream, x, numel, ctx->partials,
-                              ctx->state, scale, delta_out, nnz_out, m, jobs);
+                              ctx->state, nnz_out, m, jobs);
     };
+    step->partials = ctx->partials;
+    step->nparts = static_cast<int>(blocks);
+    step->numel = static_cast<double>(numel);
+    step->scale = scale;
     const unsigned char *m = static_cast<const unsigned char *>(mask);
     const float *xf = static_cast<const float *>(delta);
     const cudaError_t e = dtype != DBP_F32 ? go(statistics_kernel<__nv_bfloat16, false>, static_cast<const __nv_bfloat16 *>(delta), m)
@@ -583,22 +466,19 @@ int launch_statistics(dbp_ctx *ctx, const void *delta, int dtype, long long nume
 }
 
 int launch_quantize(dbp_ctx *ctx, const void *delta, int dtype, long long numel,
-                    unsigned long long seed, const float *delta_p, uint32_t *bitmap,
+                    unsigned long long seed, const StepSource &step, uint32_t *bitmap,
                     uint16_t *offsets, int8_t *values, int8_t *dense,
                     unsigned long long *nnz_out) {
     const long long nseg = (numel + kSegment - 1) / kSegment;
     long long blocks = (nseg + kThreads / 32 - 1) / (kThreads / 32);
-    const long long cap = static_cast<long long>(ctx->sm_count) * 8;
+    const long long cap = static_cast<long long>(ctx->sm_count) * 4;
     if (blocks > cap) blocks = cap;
-    if (dtype == DBP_F32)
-        { note_launch(); quantize_kernel<float><<<static_cast<unsigned>(blocks), kThreads, 0, ctx->stream>>>(
-            static_cast<const float *>(delta), numel, seed, delta_p, bitmap, offsets, values, dense,
-            ctx->state, nnz_out); }
-    else
-        { note_launch(); quantize_kernel<__nv_bfloat16><<<static_cast<unsigned>(blocks), kThreads, 0, ctx->stream>>>(
-            static_cast<const __nv_bfloat16 *>(delta), numel, seed, delta_p, bitmap, offsets, values,
-            dense, ctx->state, nnz_out); }
-    return cuda_ok(cudaGetLastError());
+    auto go = [&](auto kern, auto x) {
+        return cuda_ok(launch_chained(kern, dim3(static_cast<unsigned>(blocks)), dim3(kThreads), 0, ctx->stream, x, numel, seed, step,
+                                      bitmap, offsets, values, dense, ctx->state, nnz_out));
+    };
+    return dtype == DBP_F32 ? go(quantize_kernel<float>, static_cast<const float *>(delta))
+                            : go(quantize_kernel<__nv_bfloat16>, static_cast<const __nv_bfloat16 *>(delta));
 }
 
 int launch_decode(dbp_ctx *ctx, const uint32_t *bitmap, const uint16_t *offsets,
@@ -607,10 +487,8 @@ int launch_decode(dbp_ctx *ctx, const uint32_t *bitmap, const uint16_t *offsets,
     long long blocks = (nseg + kThreads / 32 - 1) / (kThreads / 32);
     const long long cap = static_cast<long long>(ctx->sm_count) * 8;
     if (blocks > cap) blocks = cap;
-    note_launch();
-    decode_kernel<<<static_cast<unsigned>(blocks), kThreads, 0, ctx->stream>>>(bitmap, offsets, values,
-                                                                            numel, dense);
-    return cuda_ok(cudaGetLastError());
+    return cuda_ok(launch_chained(decode_kernel, dim3(static_cast<unsigned>(blocks)), dim3(kThreads), 0, ctx->stream, bitmap,
+                                  offsets, values, numel, dense));
 }
 
 }  // namespace dbp
