@@ -108,7 +108,7 @@ struct StepSource {
     const float *given = nullptr;
     const double *partials = nullptr;   // (sum, sum of squares) of each statistics block, about the pivot
     int nparts = 0;
-    double numel = 0;
+    double inv_numel = 0;
     float scale = 0.f;
     float *publish[3] = {nullptr, nullptr, nullptr};   // where the quantizer writes it for the kernels behind it
 };
@@ -319,6 +319,24 @@ inline cudaError_t launch_chained(void (*kern)(KArgs...), dim3 grid, dim3 block,
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
+    note_launch();
+    return cudaLaunchKernelEx(&cfg, kern, static_cast<KArgs>(args)...);
+}
+// The same for a grid that is one cluster of `ctas` blocks.
+template <typename... KArgs, typename... Args>
+inline cudaError_t launch_chained_cluster(void (*kern)(KArgs...), unsigned ctas, dim3 block, cudaStream_t stream, Args... args) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(ctas);
+    cfg.blockDim = block;
+    cfg.stream = stream;
+    cudaLaunchAttribute attr[2];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    attr[1].id = cudaLaunchAttributeClusterDimension;
+    attr[1].val.clusterDim.x = ctas;
+    attr[1].val.clusterDim.y = attr[1].val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 2;
     note_launch();
     return cudaLaunchKernelEx(&cfg, kern, static_cast<KArgs>(args)...);
 }

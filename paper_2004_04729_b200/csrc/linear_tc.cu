@@ -23,11 +23,11 @@ namespace {
 
 using namespace tc;
 
-constexpr int kStagesL = 4;
+constexpr int kStagesL = 8;                      // most stages of the ring (narrow tiles)
 constexpr int kPanelL = 64 * 128;                // 64 rows x 128 bytes
 constexpr int kABytesL = 2 * kPanelL;            // 128 x 64 bf16 either way round
 constexpr int kMaxNL = 256;
-constexpr int kStageBytesL = kABytesL + (kMaxNL / 64) * kPanelL;
+constexpr int kRingL = 4 * (kABytesL + (kMaxNL / 64) * kPanelL);     // bytes of the ring: four stages of the widest tile
 constexpr int kEpiWarpsL = 8;
 constexpr int kThreadsL = 64 + 32 * kEpiWarpsL;
 constexpr int kOutBlock = 32 * 128;              // one warp's staged block: 32 rows of 128 bytes
@@ -46,6 +46,7 @@ struct LinProduct {
 struct LinArgs {
     LinProduct pr[2];             // the product with the longer tiles first
     int nprod, tiles, TN;
+    int stages, stage_bytes;      // as many stages as the ring holds: a narrow tile's steps are bound by the copies' latency
     const float *delta_p;
     int *err_flag;
 };
@@ -70,9 +71,10 @@ linear_products_kernel(const __grid_constant__ LinMaps maps, const __grid_consta
     unsigned char *smem = reinterpret_cast<unsigned char *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
     __shared__ PipeL pipe;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int S = p.stages, stage_bytes = p.stage_bytes;
 
     if (threadIdx.x == 0) {
-        for (int s = 0; s < kStagesL; ++s) {
+        for (int s = 0; s < S; ++s) {
             mbar_init(&pipe.full[s], 1);
             mbar_init(&pipe.empty[s], 1);
         }
@@ -125,7 +127,7 @@ linear_products_kernel(const __grid_constant__ LinMaps maps, const __grid_consta
                 ok = __all_sync(0xffffffffu, mbar_wait(&pipe.empty[s], parity, p.err_flag));
                 if (!ok) break;
                 if (elect_one()) {
-                    unsigned char *st = smem + s * kStageBytesL;
+                    unsigned char *st = smem + s * stage_bytes;
                     // the low pieces first: the accumulator is still small when they are added
                     const int kp = k / q.ks, piece = q.pieces - 1 - kp, r0 = (k - kp * q.ks) * 64;
                     mbar_expect_tx(&pipe.full[s], tx);
@@ -139,7 +141,7 @@ linear_products_kernel(const __grid_constant__ LinMaps maps, const __grid_consta
                     for (int i = 0; i < nb; ++i)
                         tma_load_3d(st + i * kPanelL, &maps.b[tl.i], tl.n0 + 64 * i, r0, piece, &pipe.full[s]);
                 }
-                if (++s == kStagesL) { s = 0; parity ^= 1u; }
+                if (++s == S) { s = 0; parity ^= 1u; }
             }
         }
     } else if (warp == 1) {
@@ -160,7 +162,7 @@ linear_products_kernel(const __grid_constant__ LinMaps maps, const __grid_consta
                 ok = __all_sync(0xffffffffu, mbar_wait(&pipe.full[s], parity, p.err_flag));
                 if (!ok) break;
                 tc_fence_after();
-                const unsigned a_addr = smem_u32(smem + s * kStageBytesL);
+                const unsigned a_addr = smem_u32(smem + s * stage_bytes);
                 const unsigned long long bd = make_desc(a_addr + kABytesL, kPanelL, 1024);
                 if (elect_one()) {
                     if (kmaj) {
@@ -176,7 +178,7 @@ linear_products_kernel(const __grid_constant__ LinMaps maps, const __grid_consta
                     }
                     mma_commit(&pipe.empty[s]);
                 }
-                if (++s == kStagesL) { s = 0; parity ^= 1u; }
+                if (++s == S) { s = 0; parity ^= 1u; }
             }
             if (ok && elect_one()) mma_commit(&pipe.acc_full[slot]);
         }
@@ -184,7 +186,7 @@ linear_products_kernel(const __grid_constant__ LinMaps maps, const __grid_consta
         // epilogue: TMEM lane = output row, column = output column; two warps per lane quarter take turns at the
         // blocks of 32 fp32 or 64 bf16 columns (128 bytes of a row)
         const int q4 = warp & 3, part = (warp - 2) >> 2;
-        unsigned char *stage = smem + kStagesL * kStageBytesL + (warp - 2) * kOutBlock;
+        unsigned char *stage = smem + kRingL + (warp - 2) * kOutBlock;
         const float delta = *p.delta_p;
         bool ok = true;
         int it = 0;
@@ -292,11 +294,25 @@ long long linear_pitch(long long cols) { return (cols + 7) / 8 * 8; }
 // kernel runs (it clears dW on the side).
 LinearPlan linear_plan(const dbp_ctx *ctx, long long B, long long N, long long K, int pieces, bool want_dw, bool want_dx) {
     LinearPlan pl;
-    pl.TN = K > 128 ? 256 : (K > 64 ? 128 : 64);
+    const long long dw_steps = ((B + 63) / 64) * pieces, dx_steps = ((N + 63) / 64) * pieces;
+    // The shortest makespan of tiles of 256, 128 or 64 columns: a step of a 128 x 256 tile is 512 clocks of the tensor
+    // pipe, narrower ones are bound by their copies and hand-overs (about 420 and 400 clocks); a tile ends with a drain of
+    // about 4 clocks a column. Measured, us, for 64 / 128 / 256 columns: bf16 1024 -> 4096, B 4096: 213 / 144 / 96; fp32
+    // 1024 -> 100, B 1024: 25 / 15.2 / 16.2; bf16 512 -> 512, B 512: 11.9 / 12.3 / 14.0.
+    double best = 1e300;
+    for (int tn = 64; tn <= 256; tn *= 2) {
+        if (tn > 64 && tn / 2 >= K) break;
+        const double step = tn == 256 ? 520.0 : tn == 128 ? 420.0 : 400.0, drain = 4.0 * tn + 500.0;
+        const double nt = static_cast<double>((K + tn - 1) / tn);
+        const double dx = want_dx ? dx_steps * step + drain : 0.0, dw = want_dw ? dw_steps * step + drain : 0.0;
+        const double all = nt * ((B + 127) / 128) * dx + nt * ((N + 127) / 128) * dw;
+        double longest = dx;                                            // (long dW reductions are split)
+        if (longest < all / ctx->sm_count) longest = all / ctx->sm_count;
+        if (longest < best) { best = longest; pl.TN = tn; }
+    }
     const long long nt = (K + pl.TN - 1) / pl.TN;
     const long long dx_tiles = want_dx ? ((B + 127) / 128) * nt : 0;
     const long long dw_tiles = want_dw ? ((N + 127) / 128) * nt : 0;
-    const long long dw_steps = ((B + 63) / 64) * pieces;
     // Split the weight gradient's reduction when its tiles leave SMs idle (parts of at least four steps) and when it
     // is too long for one accumulator. dX is not split: its sums keep one order, so that the gradient handed to the
     // layer below is reproducible.
@@ -320,6 +336,8 @@ int launch_linear_products(dbp_ctx *ctx, const LinearPlan &pl, const void *codes
     LinMaps maps;
     const long long q_pitch = linear_pitch(N);
     p.TN = pl.TN;
+    p.stage_bytes = kABytesL + pl.TN / 64 * kPanelL;
+    p.stages = kRingL / p.stage_bytes < kStagesL ? kRingL / p.stage_bytes : kStagesL;
     p.delta_p = delta_p;
     p.err_flag = err_flag;
     const int nt = static_cast<int>((K + pl.TN - 1) / pl.TN);
@@ -379,7 +397,7 @@ int launch_linear_products(dbp_ctx *ctx, const LinearPlan &pl, const void *codes
     if (!rc && dW) rc = fill(false);
     if (!rc && dX && !dx_first) rc = fill(true);
     if (rc) return rc;
-    const size_t smem = static_cast<size_t>(kStagesL) * kStageBytesL + kEpiWarpsL * kOutBlock + 1024;
+    const size_t smem = static_cast<size_t>(kRingL) + kEpiWarpsL * kOutBlock + 1024;
     if (cudaFuncSetAttribute(linear_products_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem)) != cudaSuccess)
         return fail_cuda("shared memory size");
     const int grid = p.tiles < ctx->sm_count ? p.tiles : ctx->sm_count;

@@ -194,8 +194,8 @@ __device__ __forceinline__ float step_of(const StepSource &s, DeviceState *st) {
         if (!isfinite(a) || !isfinite(b)) {
             if (blockIdx.x == 0) st->nonfinite = 1;
         } else {
-            const double mean = a / s.numel;
-            double var = b / s.numel - mean * mean;
+            const double mean = a * s.inv_numel;
+            double var = b * s.inv_numel - mean * mean;
             if (var < 0.0) var = 0.0;
             d = static_cast<float>(static_cast<double>(s.scale) * sqrt(var));
         }

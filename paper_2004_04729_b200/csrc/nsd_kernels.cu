@@ -455,7 +455,7 @@ int launch_statistics(dbp_ctx *ctx, const void *delta, int dtype, long long nume
     };
     step->partials = ctx->partials;
     step->nparts = static_cast<int>(blocks);
-    step->numel = static_cast<double>(numel);
+    step->inv_numel = 1.0 / static_cast<double>(numel);
     step->scale = scale;
     const unsigned char *m = static_cast<const unsigned char *>(mask);
     const float *xf = static_cast<const float *>(delta);

@@ -3,12 +3,13 @@
 //
 // For gradients of a few tens of thousands of elements every separate kernel (statistics, quantizer,
 // weight re-layout, dX, dW) is a handful of microseconds of work behind a launch and a dependent wait,
-// and the layer is bound by those.
-//   1. small_linear_quantize_kernel: every CTA computes sigma and Delta = s * sigma over the whole
-//      tensor by itself (the tensor sits in L2; every CTA adds in the same order, so all of them hold the
-//      same Delta and no grid-wide step separates statistics from quantization), then quantizes its own
-//      4096 elements into bf16 codes [B][N rounded up to 8] and counts the non-zero and clipped ones.
-//      The first CTA publishes Delta; the second kernel adds up the counts.
+// and the layer is bound by those round trips.
+//   1. small_linear_quantize_kernel: ONE cluster of up to eight CTAs holds the whole gradient in registers. The dithers
+//      are drawn before the kernel waits for what came before it; every CTA adds up its share, the eight pairs of sums
+//      are exchanged through distributed shared memory and added in rank order, so all CTAs hold the same Delta, and
+//      each quantizes its share into bf16 codes [B][N rounded up to 8] and counts the non-zero and clipped ones. The
+//      first CTA publishes Delta; the second kernel adds up the counts. (Before: every CTA of 4096 elements read the
+//      whole gradient for its sums.)
 //   2. small_linear_products_kernel: every CTA owns one 64 x 64 tile of dW or of dX and accumulates it
 //      on the tensor cores: the codes are exact in bf16, the fp32 operand (X or W) is split into two
 //      bf16 pieces (the value rounded to bf16 and what that left over, rounded again: the pair is within
@@ -16,32 +17,26 @@
 //      once at the end. Warp-level MMAs (not the CTA-wide ones with accumulators in tensor memory)
 //      because a whole tile is a few hundred of them and nothing here can hide a tensor-memory
 //      allocation, a commit and a read-back. The dW tiles of column 0 add up the bias gradient.
-// The second kernel is launched with programmatic stream serialization: it becomes resident while the first
-// runs, loads its first tiles of X and W, and reads the codes as soon as the first one has finished.
-#include "dbp_internal.cuh"
+//      X and W are inputs of the call: a tile's operand of up to 512 reduction indices is loaded, split and laid in shared
+//      memory while the first kernel runs; what is left after it is one round trip for the codes and the MMAs.
+// The second kernel is launched with programmatic stream serialization: it becomes resident while the first runs.
+#include "nsd_common.cuh"
+#include "tc_common.cuh"
 
 namespace dbp {
 
 namespace {
 
+using namespace nsd;
+
 constexpr int kThreads = 512;
-constexpr unsigned kFull = 0xffffffffu;
 constexpr int kRows = 64, kCols = 64, kRed = 64;      // output tile and reduction chunk
 constexpr int kPitch = 72;                            // halfwords per shared-memory row: a 16-byte multiple whose eight
                                                       // consecutive rows fall into different 16-byte bank groups
-constexpr int kQuantPerCta = kThreads * 8;            // elements a CTA of the first kernel quantizes
-constexpr unsigned long long kGamma = 0x9E3779B97F4A7C15ull;
-constexpr float kMagic = 12582912.0f;                 // 1.5 * 2^23: floats in [2^23, 2^24) have unit spacing
-
-__device__ __forceinline__ unsigned long long mix64(unsigned long long z) {
-    z = (z ^ (z >> 30)) * 0xBF58476D1CE4E5B9ull;
-    z = (z ^ (z >> 27)) * 0x94D049BB133111EBull;
-    return z ^ (z >> 31);
-}
-// u = (2k+1) 2^-24, k = top 23 bits of h
-__device__ __forceinline__ float dither(unsigned h) {
-    return __uint_as_float(__funnelshift_r(h, 0x7fu, 9)) - 0.99999994f;
-}
+constexpr int kChunkTile = 64 * kPitch;               // halfwords of one operand's chunk
+constexpr int kMaxChunks = 8;                         // chunks whose operands lie in shared memory at once (three tiles each)
+constexpr int kMaxCluster = 8;
+constexpr int kMaxVec = 8;                            // 16-byte vectors per thread of the first kernel
 
 __device__ __forceinline__ unsigned smem_addr(const void *p) { return static_cast<unsigned>(__cvta_generic_to_shared(p)); }
 // four 8x8 matrices of 16-bit elements from shared memory: lane l gives the address of row l % 8 of matrix l / 8;
@@ -62,12 +57,6 @@ __device__ __forceinline__ void mma_bf16_16816(float (&d)[4], const unsigned (&a
                  : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
 }
 
-__device__ __forceinline__ double warp_sum(double v) {
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(kFull, v, o);
-    return v;
-}
-
 struct SmallLinP {
     const float *delta, *X, *W;   // [B][N], [B][K], [N][K]
     const uint8_t *mask;          // not null: delta is delta_a and the gradient is delta_a where mask != 0, else 0
@@ -79,149 +68,181 @@ struct SmallLinP {
     DeviceState *st;
     float *delta_set;             // second place the step size goes to (may be null)
     unsigned short *codes;        // bf16 [B][Np]
-    unsigned *slots;              // one non-zero count per CTA of the first kernel
+    unsigned *slots;              // one non-zero count per warp of the first kernel
+    double inv_numel;
     int tiles_k, n_dw, n_dx, n_qctas;
     int vec4;                     // K % 4 == 0: 16-byte accesses along K
+    int chunks;                   // chunks of the reduction in shared memory at once
 };
 
 // ---------------------------------------------------------------- step size and codes
+// stores a double at the same place of another CTA's shared memory; its 8 bytes are counted on that CTA's barrier
+__device__ __forceinline__ void store_remote(double *p, unsigned long long *bar, unsigned rank, double v) {
+    unsigned addr, baddr;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(addr) : "r"(smem_addr(p)), "r"(rank));
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(baddr) : "r"(smem_addr(bar)), "r"(rank));
+    asm volatile("st.async.shared::cluster.mbarrier::complete_tx::bytes.b64 [%0], %1, [%2];"
+                 ::"r"(addr), "l"(__double_as_longlong(v)), "r"(baddr) : "memory");
+}
+
+// NV: vectors of four elements per thread (vector i of a thread: blockIdx.x * kThreads + tid + i * all threads)
+template <int NV>
 __global__ void __launch_bounds__(kThreads)
 small_linear_quantize_kernel(const SmallLinP p) {
-    __shared__ double red1[kThreads / 32], red2[kThreads / 32];
-    __shared__ unsigned cnt_s[2];
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    __shared__ double red_s[2][kThreads / 32];
+    __shared__ double all_s[kMaxCluster][2];
+    __shared__ unsigned long long bar_s;           // counts the bytes of the sums that arrive from the cluster's CTAs
+    __shared__ float delta_s;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nctas = gridDim.x;
+    const int n = static_cast<int>(p.B * p.N), nvec = (n + 3) / 4, step = nctas * kThreads;
+    const int v0 = blockIdx.x * kThreads + tid;
+    unsigned long long u[NV][2];
+#pragma unroll
+    for (int i = 0; i < NV; ++i) dithers_of<4>(4ll * (v0 + i * step), p.seed, u[i]);
+    if (tid == 0) {
+        tc::mbar_init(&bar_s, 1);
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+        tc::mbar_expect_tx(&bar_s, 16u * nctas);
+    }
+    // every CTA's barrier is there before anybody's sums leave (long before: this is in front of the wait)
+    asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
     chain_wait();
     chain_release();
-    const long long n = p.B * p.N;
-    if (tid < 2) cnt_s[tid] = 0u;
 
-    // step size: shifted moments about the first element, fp32 inside a 16-byte load, fp64 across
+    float x[NV][4];
+#pragma unroll
+    for (int i = 0; i < NV; ++i) {
+        const int e = 4 * (v0 + i * step);
+        if (e + 4 <= n) {
+            const float4 q = __ldcg(reinterpret_cast<const float4 *>(p.delta + e));
+            x[i][0] = q.x; x[i][1] = q.y; x[i][2] = q.z; x[i][3] = q.w;
+        } else {
+#pragma unroll
+            for (int j = 0; j < 4; ++j) x[i][j] = e + j < n ? __ldcg(p.delta + e + j) : 0.f;
+        }
+    }
+    if (p.mask != nullptr) {
+#pragma unroll
+        for (int i = 0; i < NV; ++i) {
+            const int e = 4 * (v0 + i * step);
+            if (e + 4 <= n) {
+                const uchar4 m = __ldg(reinterpret_cast<const uchar4 *>(p.mask + e));
+                x[i][0] = m.x ? x[i][0] : 0.f; x[i][1] = m.y ? x[i][1] : 0.f; x[i][2] = m.z ? x[i][2] : 0.f; x[i][3] = m.w ? x[i][3] : 0.f;
+            } else {
+#pragma unroll
+                for (int j = 0; j < 4; ++j)
+                    if (e + j < n && !__ldg(p.mask + e + j)) x[i][j] = 0.f;
+            }
+        }
+    }
+    // step size: shifted moments about the first element, fp32 inside a vector, fp64 across
     float delta;
     bool nonfinite = false;
     if (p.scale > 0.f) {
-        const bool masked = p.mask != nullptr;
-        const float pivot = (!masked || __ldg(p.mask)) ? __ldg(p.delta) : 0.f;
-        const uchar4 *m4 = reinterpret_cast<const uchar4 *>(p.mask);
+        const float pivot = (p.mask == nullptr || __ldg(p.mask)) ? __ldcg(p.delta) : 0.f;
         double d1 = 0.0, d2 = 0.0;
-        const long long nvec = n / 4;
-        const float4 *v4 = reinterpret_cast<const float4 *>(p.delta);
-        constexpr int kU = 20;                          // loads in flight per thread: one round trip for 10 K vectors
-        for (long long i0 = 0; i0 < nvec; i0 += kThreads * kU) {
-            float4 v[kU];
 #pragma unroll
-            for (int u = 0; u < kU; ++u) {
-                const long long i = i0 + u * kThreads + tid;
-                v[u] = i < nvec ? __ldg(v4 + i) : make_float4(pivot, pivot, pivot, pivot);
-                if (masked && i < nvec) {
-                    const uchar4 m = __ldg(m4 + i);
-                    v[u].x = m.x ? v[u].x : 0.f; v[u].y = m.y ? v[u].y : 0.f;
-                    v[u].z = m.z ? v[u].z : 0.f; v[u].w = m.w ? v[u].w : 0.f;
-                }
-            }
+        for (int i = 0; i < NV; ++i) {
+            const int e = 4 * (v0 + i * step);
+            float s1 = 0.f, s2 = 0.f;
 #pragma unroll
-            for (int u = 0; u < kU; ++u) {
-                const float c0 = v[u].x - pivot, c1 = v[u].y - pivot, c2 = v[u].z - pivot, c3 = v[u].w - pivot;
-                const float s1 = (c0 + c1) + (c2 + c3);
-                const float s2 = fmaf(c0, c0, fmaf(c1, c1, fmaf(c2, c2, c3 * c3)));
-                d1 += static_cast<double>(s1);
-                d2 += static_cast<double>(s2);
+            for (int j = 0; j < 4; ++j) {
+                const float c = e + j < n ? x[i][j] - pivot : 0.f;
+                s1 += c;
+                s2 = fmaf(c, c, s2);
             }
+            d1 += static_cast<double>(s1);
+            d2 += static_cast<double>(s2);
         }
-        if (tid == 0)
-            for (long long i = nvec * 4; i < n; ++i) {
-                const float xi = (!masked || __ldg(p.mask + i)) ? __ldg(p.delta + i) : 0.f;
-                const double c = static_cast<double>(xi) - static_cast<double>(pivot);
-                d1 += c;
-                d2 += c * c;
-            }
         d1 = warp_sum(d1);
         d2 = warp_sum(d2);
-        if (lane == 0) { red1[warp] = d1; red2[warp] = d2; }
+        if (lane == 0) { red_s[0][warp] = d1; red_s[1][warp] = d2; }
         __syncthreads();
-        double a = 0.0, b = 0.0;
+        if (warp == 0) {
+            // sixteen partial sums of each moment in the two halves of the warp
+            double v = red_s[lane >> 4][lane & 15];
 #pragma unroll
-        for (int w = 0; w < kThreads / 32; ++w) { a += red1[w]; b += red2[w]; }
-        if (!isfinite(a) || !isfinite(b)) {
-            nonfinite = true;
-            delta = 0.f;
-        } else {
-            const double mean = a / static_cast<double>(n);
-            double var = b / static_cast<double>(n) - mean * mean;
-            if (var < 0.0) var = 0.0;
-            delta = static_cast<float>(static_cast<double>(p.scale) * sqrt(var));
-        }
-    } else {
-        delta = __ldg(p.delta_in);
-    }
-    const bool live = (delta > 0.f) && (delta < __int_as_float(0x7f800000));
-    const float inv = live ? __fdiv_rn(1.0f, delta) : 0.f;
-
-    // codes of this thread's eight consecutive elements (the first index is even: a pair shares a draw)
-    const long long e0 = static_cast<long long>(blockIdx.x) * kQuantPerCta + static_cast<long long>(tid) * 8;
-    unsigned nnz = 0, sat = 0;
-    if (e0 < n) {
-        float f[8];
-        unsigned long long z = p.seed + (static_cast<unsigned long long>(e0 >> 1) + 1ull) * kGamma;
-#pragma unroll
-        for (int j = 0; j < 8; j += 2) {
-            const unsigned long long r = mix64(z);
-            z += kGamma;
-            const float u[2] = {dither(static_cast<unsigned>(r)), dither(static_cast<unsigned>(r >> 32))};
-#pragma unroll
-            for (int h = 0; h < 2; ++h) {
-                float q = 0.f;
-                if (live && e0 + j + h < n) {
-                    const float xe = (p.mask == nullptr || __ldg(p.mask + e0 + j + h)) ? __ldg(p.delta + e0 + j + h) : 0.f;
-                    const float t = __fmaf_rn(xe, inv, u[h]);
-                    const float tc = fminf(fmaxf(t, -127.f), 127.99999f);      // clipped codes are counted, NaN gives 0
-                    const bool num = (t == t);
-                    sat += (num && tc != t) ? 1u : 0u;
-                    q = num ? __fadd_rd(tc, kMagic) - kMagic : 0.f;
-                }
-                f[j + h] = q;
-                nnz += q != 0.f;
+            for (int o = 8; o > 0; o >>= 1) v += __shfl_xor_sync(kFull, v, o);
+            const double a = __shfl_sync(kFull, v, 0), b = __shfl_sync(kFull, v, 16);
+            if (lane < nctas) {                                        // the grid is one cluster: rank = blockIdx.x
+                store_remote(&all_s[blockIdx.x][0], &bar_s, lane, a);
+                store_remote(&all_s[blockIdx.x][1], &bar_s, lane, b);
             }
         }
-        // to [b][Np]: one division for the first element, then step and wrap; small integers are exact in
-        // bf16 (the float's upper half)
-        long long b = e0 / p.N;
-        long long j = e0 - b * p.N;
-        unsigned short *dst = p.codes + b * p.Np + j;
+        // (a CTA ends only after all sums have arrived here, so nothing is still on its way to it then)
+        const bool here = tc::mbar_wait(&bar_s, 0, &p.st->tc_timeout);
+        if (tid == 0) {
+            double a = 0.0, b = 0.0;
 #pragma unroll
-        for (int i = 0; i < 8; ++i) {
-            if (e0 + i < n) *dst = static_cast<unsigned short>(__float_as_uint(f[i]) >> 16);
-            ++dst;
-            if (++j == p.N) { j = 0; dst += p.Np - p.N; }
+            for (int r = 0; r < kMaxCluster; ++r)
+                if (r < nctas) { a += all_s[r][0]; b += all_s[r][1]; }
+            if (!here) a = b = 0.0;
+            delta = 0.f;
+            if (!isfinite(a) || !isfinite(b)) {
+                nonfinite = true;
+            } else {
+                const double mean = a * p.inv_numel;
+                double var = b * p.inv_numel - mean * mean;
+                if (var < 0.0) var = 0.0;
+                delta = static_cast<float>(static_cast<double>(p.scale) * sqrt(var));
+            }
+            delta_s = delta;
+        }
+        __syncthreads();
+        delta = delta_s;
+    } else {
+        delta = __ldcg(p.delta_in);
+    }
+    const bool live = (delta > 0.f) && (delta < __int_as_float(0x7f800000));
+    const float inv = live ? __fdiv_rn(1.0f, delta) : 0.f;             // Delta = 0: every code 0
+
+    unsigned nz2 = 0, sat = 0;
+    const unsigned N = static_cast<unsigned>(p.N);
+#pragma unroll
+    for (int i = 0; i < NV; ++i) {
+        const int e = 4 * (v0 + i * step);
+        if (v0 + i * step < nvec) {
+            float f[4];
+            unsigned h[2];
+            decide<4>(x[i], u[i], inv, f, sat);                        // elements past the end were read as 0: code 0
+            pack_bf16<4>(f, h);
+            count_pairs<4>(h, nz2);
+            const unsigned b = static_cast<unsigned>(e) / N, j = static_cast<unsigned>(e) - b * N;
+            unsigned short *dst = p.codes + b * p.Np + j;
+            if ((N & 3u) == 0) {                                       // four codes of one row
+                *reinterpret_cast<uint2 *>(dst) = make_uint2(h[0], h[1]);
+            } else {
+                unsigned jj = j;
+#pragma unroll
+                for (int k = 0; k < 4; ++k) {
+                    if (e + k < n) *dst = static_cast<unsigned short>(h[k >> 1] >> (16 * (k & 1)));
+                    ++dst;
+                    if (++jj == N) { jj = 0; dst += p.Np - N; }
+                }
+            }
         }
     }
-    nnz = __reduce_add_sync(kFull, nnz);
-    sat = __reduce_add_sync(kFull, sat);
-    __syncthreads();                                     // cnt_s is initialised (and red1 / red2 have been read)
+    const unsigned nnz = __reduce_add_sync(kFull, pairs_total(nz2));
+    sat = __reduce_add_sync(kFull, live ? sat : 0u);
+    // The counts of the warps are added up by the products kernel, which runs when all of them are done. Every CTA holds
+    // the same Delta, so the first one publishes it.
     if (lane == 0) {
-        if (nnz) atomicAdd(&cnt_s[0], nnz);
-        if (sat) atomicAdd(&cnt_s[1], sat);
+        p.slots[blockIdx.x * (kThreads / 32) + warp] = nnz;
+        if (sat) atomicAdd(&p.st->saturated, static_cast<unsigned long long>(sat));
     }
-    __syncthreads();
-    // Every CTA holds the same Delta, so the first one publishes it; the counts of the CTAs are added up by the
-    // products kernel, which runs when all of them are done (no election of a last CTA, no extra round trips here).
-    if (tid == 0) {
-        p.slots[blockIdx.x] = cnt_s[0];
-        if (cnt_s[1]) atomicAdd(&p.st->saturated, static_cast<unsigned long long>(cnt_s[1]));
-        if (blockIdx.x == 0) {
-            p.st->delta = delta;
-            if (nonfinite) p.st->nonfinite = 1;
-            if (p.delta_set) *p.delta_set = delta;
-        }
+    if (blockIdx.x == 0 && tid == 0) {
+        p.st->delta = delta;
+        if (nonfinite) p.st->nonfinite = 1;
+        if (p.delta_set) *p.delta_set = delta;
     }
 }
 
 // ---------------------------------------------------------------- both products
 __global__ void __launch_bounds__(kThreads)
 small_linear_products_kernel(const SmallLinP p) {
-    // codes: dX tiles [row][reduction index], dW tiles [reduction index][row] (the order they are stored in either way)
-    __shared__ __align__(16) unsigned short As[64 * kPitch];
-    // rows of X (dW) or W (dX), [reduction index][column], as two bf16 pieces
-    __shared__ __align__(16) unsigned short Bh[kRed * kPitch], Bl[kRed * kPitch];
+    // per chunk of 64 reduction indices: codes (dX tiles [row][reduction index], dW tiles [reduction index][row], the order
+    // they are stored in either way), then rows of X (dW) or W (dX), [reduction index][column], as two bf16 pieces
+    extern __shared__ __align__(16) unsigned short tiles_s[];
     __shared__ float db_s[kRows];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
 
@@ -266,103 +287,123 @@ small_linear_products_kernel(const SmallLinP p) {
             b_reg[h] = v;
         }
     };
-    // codes outside the tensor (and the padding of a row) read as zero
-    auto load_a = [&](long long r0, uint4 &a_reg) {
+    // Codes outside the tensor read as zero; the padding of a row is cleared when a vector is used (clear_pad), so that the
+    // loads of all chunks are in flight together.
+    auto load_a = [&](long long r0) {
         const long long bb = is_dw ? r0 + hi : row0 + hi;            // image (row of delta_z)
         const long long jj = is_dw ? row0 + lo : r0 + lo;            // first of eight output channels
-        uint4 v = make_uint4(0u, 0u, 0u, 0u);
-        if (bb < p.B && jj < p.N) {
-            v = __ldcg(reinterpret_cast<const uint4 *>(p.codes + bb * p.Np + jj));
-            const long long left = p.N - jj;                         // valid codes from jj on
-            if (left < 8) {
-                unsigned w[4] = {v.x, v.y, v.z, v.w};
+        return bb < p.B && jj < p.N ? __ldcg(reinterpret_cast<const uint4 *>(p.codes + bb * p.Np + jj)) : make_uint4(0u, 0u, 0u, 0u);
+    };
+    auto clear_pad = [&](long long r0, uint4 &v) {
+        const long long left = p.N - (is_dw ? row0 + lo : r0 + lo);  // valid codes from the vector's first on
+        if (left < 8) {
+            unsigned w[4] = {v.x, v.y, v.z, v.w};
 #pragma unroll
-                for (int i = 0; i < 4; ++i) {
-                    if (2 * i >= left) w[i] = 0u;
-                    else if (2 * i + 1 >= left) w[i] &= 0xffffu;
-                }
-                v = make_uint4(w[0], w[1], w[2], w[3]);
+            for (int i = 0; i < 4; ++i) {
+                if (2 * i >= left) w[i] = 0u;
+                else if (2 * i + 1 >= left) w[i] &= 0xffffu;
             }
+            v = make_uint4(w[0], w[1], w[2], w[3]);
         }
-        a_reg = v;
     };
     // the addresses this lane hands to the 8x8-matrix loads (lane l: row l % 8 of matrix l / 8)
     const int lm = lane >> 3, lr = lane & 7;
     // A, four matrices: (rows 0-7, k 0-7), (rows 8-15, k 0-7), (rows 0-7, k 8-15), (rows 8-15, k 8-15);
     // dW tiles hold them [k][row] and load them transposed
-    const unsigned a_base = smem_addr(As) + 2u * (is_dw ? static_cast<unsigned>(((lm >> 1) * 8 + lr) * kPitch + wr + (lm & 1) * 8)
-                                                        : static_cast<unsigned>((wr + (lm & 1) * 8 + lr) * kPitch + (lm >> 1) * 8));
+    const unsigned a_base = smem_addr(tiles_s) + 2u * (is_dw ? static_cast<unsigned>(((lm >> 1) * 8 + lr) * kPitch + wr + (lm & 1) * 8)
+                                                             : static_cast<unsigned>((wr + (lm & 1) * 8 + lr) * kPitch + (lm >> 1) * 8));
     const unsigned a_kstep = 2u * (is_dw ? 16u * kPitch : 16u);
     // B, four matrices: (k 0-7, n 0-7), (k 8-15, n 0-7), (k 0-7, n 8-15), (k 8-15, n 8-15), stored [k][n]: transposed loads
-    const unsigned b_off = 2u * static_cast<unsigned>(((lm & 1) * 8 + lr) * kPitch + wc + (lm >> 1) * 8);
-    const unsigned bh_base = smem_addr(Bh) + b_off, bl_base = smem_addr(Bl) + b_off;
+    const unsigned b_base = smem_addr(tiles_s) + 2u * static_cast<unsigned>(kChunkTile + ((lm & 1) * 8 + lr) * kPitch + wc + (lm >> 1) * 8);
 
-    // one chunk: registers -> shared memory, the loads of the chunk after next, then the MMAs
-    auto step = [&](long long r0, uint4 &a_reg, float4 (&b_reg)[2]) {
-        __syncthreads();                                 // the previous chunk has been used
-        {
-            *reinterpret_cast<uint4 *>(As + hi * kPitch + lo) = a_reg;
-            if (do_db) {
-                const unsigned w[4] = {a_reg.x, a_reg.y, a_reg.z, a_reg.w};
+    // fp32 operand of `count` chunks from r0 on -> its two pieces in shared memory, four chunks' loads in flight
+    auto fill_b = [&](long long r0, int count) {
+        for (int c0 = 0; c0 < count; c0 += 4) {
+            float4 b_reg[4][2];
 #pragma unroll
-                for (int i = 0; i < 4; ++i) {
-                    dbacc[2 * i] += __uint_as_float(w[i] << 16);
-                    dbacc[2 * i + 1] += __uint_as_float(w[i] & 0xffff0000u);
+            for (int c = 0; c < 4; ++c)
+                if (c0 + c < count) load_b(r0 + (c0 + c) * kRed, b_reg[c]);
+#pragma unroll
+            for (int c = 0; c < 4; ++c)
+                if (c0 + c < count) {
+                    const float v[8] = {b_reg[c][0].x, b_reg[c][0].y, b_reg[c][0].z, b_reg[c][0].w,
+                                        b_reg[c][1].x, b_reg[c][1].y, b_reg[c][1].z, b_reg[c][1].w};
+                    unsigned h2[4], l2[4];
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) {
+                        const __nv_bfloat162 hh = __floats2bfloat162_rn(v[2 * i], v[2 * i + 1]);
+                        const float2 hf = __bfloat1622float2(hh);
+                        const __nv_bfloat162 ll = __floats2bfloat162_rn(v[2 * i] - hf.x, v[2 * i + 1] - hf.y);
+                        h2[i] = *reinterpret_cast<const unsigned *>(&hh);
+                        l2[i] = *reinterpret_cast<const unsigned *>(&ll);
+                    }
+                    unsigned short *dst = tiles_s + (c0 + c) * 3 * kChunkTile + kChunkTile + hi * kPitch + lo;
+                    *reinterpret_cast<uint4 *>(dst) = make_uint4(h2[0], h2[1], h2[2], h2[3]);
+                    *reinterpret_cast<uint4 *>(dst + kChunkTile) = make_uint4(l2[0], l2[1], l2[2], l2[3]);
                 }
-            }
-            const float v[8] = {b_reg[0].x, b_reg[0].y, b_reg[0].z, b_reg[0].w, b_reg[1].x, b_reg[1].y, b_reg[1].z, b_reg[1].w};
-            unsigned h2[4], l2[4];
-#pragma unroll
-            for (int i = 0; i < 4; ++i) {
-                const __nv_bfloat162 hh = __floats2bfloat162_rn(v[2 * i], v[2 * i + 1]);
-                const float2 hf = __bfloat1622float2(hh);
-                const __nv_bfloat162 ll = __floats2bfloat162_rn(v[2 * i] - hf.x, v[2 * i + 1] - hf.y);
-                h2[i] = *reinterpret_cast<const unsigned *>(&hh);
-                l2[i] = *reinterpret_cast<const unsigned *>(&ll);
-            }
-            *reinterpret_cast<uint4 *>(Bh + hi * kPitch + lo) = make_uint4(h2[0], h2[1], h2[2], h2[3]);
-            *reinterpret_cast<uint4 *>(Bl + hi * kPitch + lo) = make_uint4(l2[0], l2[1], l2[2], l2[3]);
-        }
-        __syncthreads();
-        if (r0 + 2 * kRed < nred) {                      // in flight during this chunk's and the next one's MMAs
-            load_a(r0 + 2 * kRed, a_reg);
-            load_b(r0 + 2 * kRed, b_reg);
-        }
-#pragma unroll
-        for (int ks = 0; ks < kRed / 16; ++ks) {
-            unsigned a[4], bh[4], bl[4];
-            if (is_dw) ldmatrix_x4_trans(a, a_base + ks * a_kstep);
-            else ldmatrix_x4(a, a_base + ks * a_kstep);
-            ldmatrix_x4_trans(bh, bh_base + ks * 2u * 16u * kPitch);
-            ldmatrix_x4_trans(bl, bl_base + ks * 2u * 16u * kPitch);
-            mma_bf16_16816(acc[0], a, bh[0], bh[1]);
-            mma_bf16_16816(acc[0], a, bl[0], bl[1]);
-            mma_bf16_16816(acc[1], a, bh[2], bh[3]);
-            mma_bf16_16816(acc[1], a, bl[2], bl[3]);
         }
     };
-
-    uint4 a0, a1 = make_uint4(0u, 0u, 0u, 0u);
-    float4 b0[2], b1[2];
-    // X and W are inputs of the call: their first chunks are on their way before the first kernel is done
-    load_b(0, b0);
-    if (kRed < nred) load_b(kRed, b1);
+    // codes of `count` chunks: one round trip for all of them
+    auto fill_a = [&](long long r0, int count) {
+        {
+            uint4 a_reg[kMaxChunks];
+#pragma unroll
+            for (int c = 0; c < kMaxChunks; ++c)
+                a_reg[c] = c < count ? load_a(r0 + c * kRed) : make_uint4(0u, 0u, 0u, 0u);
+#pragma unroll
+            for (int c = 0; c < kMaxChunks; ++c)
+                if (c < count) {
+                    clear_pad(r0 + c * kRed, a_reg[c]);
+                    *reinterpret_cast<uint4 *>(tiles_s + c * 3 * kChunkTile + hi * kPitch + lo) = a_reg[c];
+                    if (do_db) {
+                        const unsigned w[4] = {a_reg[c].x, a_reg[c].y, a_reg[c].z, a_reg[c].w};
+#pragma unroll
+                        for (int i = 0; i < 4; ++i) {
+                            dbacc[2 * i] += __uint_as_float(w[i] << 16);
+                            dbacc[2 * i + 1] += __uint_as_float(w[i] & 0xffff0000u);
+                        }
+                    }
+                }
+        }
+    };
+    const int nchunks = static_cast<int>((nred + kRed - 1) / kRed);
+    // X and W are inputs of the call: the first chunks' operand is laid out before the first kernel is done
+    int count = nchunks < p.chunks ? nchunks : p.chunks;
+    fill_b(0, count);
     chain_wait();
     chain_release();
     const float delta = __ldcg(&p.st->delta);
     const float dscale = (delta > 0.f && delta < __int_as_float(0x7f800000)) ? delta : 0.f;
     if (blockIdx.x == 0 && warp == 0) {                  // nnz of the step: the first kernel's per-CTA counts
         unsigned long long total = 0;
-        for (int i = lane; i < p.n_qctas; i += 32) total += __ldcg(p.slots + i);
+        for (int i = lane; i < p.n_qctas * (kThreads / 32); i += 32) total += __ldcg(p.slots + i);
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) total += __shfl_xor_sync(kFull, total, o);
         if (lane == 0) p.st->nnz = total;
     }
-    load_a(0, a0);
-    if (kRed < nred) load_a(kRed, a1);
-    for (long long r0 = 0; r0 < nred; r0 += 2 * kRed) {
-        step(r0, a0, b0);
-        if (r0 + kRed < nred) step(r0 + kRed, a1, b1);
+    for (int c0 = 0; c0 < nchunks; c0 += p.chunks) {
+        count = nchunks - c0 < p.chunks ? nchunks - c0 : p.chunks;
+        if (c0 > 0) {
+            __syncthreads();                             // the previous chunks have been used
+            fill_b(static_cast<long long>(c0) * kRed, count);
+        }
+        fill_a(static_cast<long long>(c0) * kRed, count);
+        __syncthreads();
+        for (int c = 0; c < count; ++c) {
+            const unsigned off = 2u * static_cast<unsigned>(c * 3 * kChunkTile);
+#pragma unroll
+            for (int ks = 0; ks < kRed / 16; ++ks) {
+                unsigned a[4], bh[4], bl[4];
+                if (is_dw) ldmatrix_x4_trans(a, a_base + off + ks * a_kstep);
+                else ldmatrix_x4(a, a_base + off + ks * a_kstep);
+                ldmatrix_x4_trans(bh, b_base + off + ks * 2u * 16u * kPitch);
+                ldmatrix_x4_trans(bl, b_base + off + 2u * kChunkTile + ks * 2u * 16u * kPitch);
+                mma_bf16_16816(acc[0], a, bh[0], bh[1]);
+                mma_bf16_16816(acc[1], a, bh[2], bh[3]);
+                mma_bf16_16816(acc[0], a, bl[0], bl[1]);
+                mma_bf16_16816(acc[1], a, bl[2], bl[3]);
+            }
+        }
     }
 
     // the tile, scaled by Delta once: accumulator t holds rows g and g + 8, columns 2 tig, 2 tig + 1 of n-tile t
@@ -394,18 +435,19 @@ small_linear_products_kernel(const SmallLinP p) {
 
 }  // namespace
 
-// Shapes the two-launch path takes: small enough that every CTA of the first kernel can read the whole
-// gradient for its statistics (gradient size times CTA count is the L2 traffic of that: at most 32 x 2^17 elements).
+// Shapes the two-launch path takes: a gradient that one cluster holds in registers, and one tile per SM at most. The legacy
+// warp-level MMA runs at about 550 multiply-adds per clock and SM here (a 64 x 64 x 16 step with two pieces takes 240
+// clocks), so a second tile per SM costs more than the third launch of the CTA-wide kernels (linear_tc.cu). Measured, us,
+// this path against that one: 784 -> 300, B 128 (91 tiles): 9.5 against 14.9; 512 -> 1000, B 128 (144): 22.4 against
+// 22.8; 1024 -> 100, B 1024 (288): 24.2 against 15.0.
 bool small_linear_fits(const dbp_ctx *ctx, long long B, long long N, long long K, bool want_dw, bool want_dx) {
     const long long n = B * N;
-    if (n <= 0 || n > (1ll << 17) || K <= 0 || K > (1ll << 24)) return false;
+    if (n <= 0 || n > 4ll * kMaxCluster * kThreads * kMaxVec || K <= 0 || K > (1ll << 24)) return false;
     const long long tiles_k = (K + kCols - 1) / kCols;
     const long long n_dw = want_dw ? ((N + kRows - 1) / kRows) * tiles_k : 0;
     const long long n_dx = want_dx ? ((B + kRows - 1) / kRows) * tiles_k : 0;
     const long long ctas = n_dw + n_dx;
-    if (ctas <= 0 || ctas > 65535) return false;
-    const long long qctas = (n + kQuantPerCta - 1) / kQuantPerCta;
-    return qctas * static_cast<long long>(sizeof(unsigned)) <= static_cast<long long>(sizeof(double)) * 2 * ctx->partial_blocks;
+    return ctas > 0 && ctas <= ctx->sm_count;
 }
 
 int launch_small_linear(dbp_ctx *ctx, const float *delta, const float *X, const float *W, long long B, long long N,
@@ -424,11 +466,25 @@ int launch_small_linear(dbp_ctx *ctx, const float *delta, const float *X, const 
     p.n_dw = dW ? static_cast<int>((N + kRows - 1) / kRows) * p.tiles_k : 0;
     p.n_dx = dX ? static_cast<int>((B + kRows - 1) / kRows) * p.tiles_k : 0;
     p.vec4 = (K % 4 == 0) ? 1 : 0;
-    const long long n = B * N;
-    const unsigned qctas = static_cast<unsigned>((n + kQuantPerCta - 1) / kQuantPerCta);
-    p.n_qctas = static_cast<int>(qctas);
-    if (int rc = cuda_ok(launch_chained(small_linear_quantize_kernel, dim3(qctas), dim3(kThreads), 0, ctx->stream, p))) return rc;
-    return cuda_ok(launch_chained(small_linear_products_kernel, dim3(static_cast<unsigned>(p.n_dw + p.n_dx)), dim3(kThreads), 0,
+    // the cluster grows before the vectors per thread do
+    const long long n = B * N, nvec = (n + 3) / 4;
+    int ctas = 1;
+    while (ctas < kMaxCluster && ctas * kThreads < nvec) ctas *= 2;
+    const int per = static_cast<int>((nvec + ctas * kThreads - 1) / (ctas * kThreads));
+    p.n_qctas = ctas;
+    p.inv_numel = 1.0 / static_cast<double>(n);
+    auto kern = per <= 1 ? small_linear_quantize_kernel<1> : per <= 2 ? small_linear_quantize_kernel<2>
+              : per <= 5 ? small_linear_quantize_kernel<5> : small_linear_quantize_kernel<kMaxVec>;
+    if (int rc = cuda_ok(launch_chained_cluster(kern, static_cast<unsigned>(ctas), dim3(kThreads), ctx->stream, p))) return rc;
+    const long long red = (dW && (!dX || B > N)) ? B : N;               // the longest reduction of the tiles
+    const long long chunks = (red + kRed - 1) / kRed;
+    const int most = p.n_dw + p.n_dx > ctx->sm_count ? kMaxChunks / 2 : kMaxChunks;      // two CTAs per SM when there are more tiles
+    p.chunks = chunks < most ? static_cast<int>(chunks) : most;
+    const size_t smem = static_cast<size_t>(p.chunks) * 3 * kChunkTile * 2;
+    if (cudaFuncSetAttribute(small_linear_products_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             kMaxChunks * 3 * kChunkTile * 2) != cudaSuccess)
+        return fail_cuda("shared memory size");
+    return cuda_ok(launch_chained(small_linear_products_kernel, dim3(static_cast<unsigned>(p.n_dw + p.n_dx)), dim3(kThreads), smem,
                                   ctx->stream, p));
 }
 
