@@ -141,7 +141,7 @@ int quantize_for_products(dbp_ctx *ctx, const void *delta, int dtype, long long 
                                       step, pn, want8 ? dense : nullptr, true, ps, static_cast<int>(nhwc->W), mask);
         } else {
             rc = launch_quantize_dense(ctx, delta, dtype, numel, seed, step, want8 ? dense : nullptr,
-                                       p16, planes_hw, planes_pitch, true);
+                                       p16, planes_hw, planes_pitch, true, mask);
         }
     }
     if (rc) return rc;
@@ -155,7 +155,7 @@ int quantize_for_products(dbp_ctx *ctx, const void *delta, int dtype, long long 
 // and clears dW where its reduction is split. Both products leave in one launch on the context's stream.
 int linear_tc_backward(dbp_ctx *ctx, const void *delta, const void *X, const void *W, int io, long long B, long long N,
                        long long K, unsigned long long seed, float scale, const float *delta_in, dbp_sparse *q_out, float *dW,
-                       void *dX, float *db, unsigned flags) {
+                       void *dX, float *db, unsigned flags, const uint8_t *mask) {
     const int pieces = io == DBP_F32 ? 2 : 1;
     const LinearPlan pl = linear_plan(ctx, B, N, K, pieces, dW != nullptr, dX != nullptr);
     // a *_host call: X is still on its way up on another stream
@@ -179,7 +179,7 @@ int linear_tc_backward(dbp_ctx *ctx, const void *delta, const void *X, const voi
     const int8_t *codes = nullptr;
     const void *codes16 = nullptr;
     rc = quantize_for_products(ctx, delta, io, B * N, seed, scale, delta_in, q_out, &delta_p, &codes, false, N, linear_pitch(N),
-                               &codes16, nullptr, nullptr, jobs);
+                               &codes16, nullptr, nullptr, jobs, 0, nullptr, mask);
     if (rc) return rc;
     if (dW || dX) {
         KernelTimer t(ctx, DBP_K_DX_DENSE);
@@ -197,11 +197,12 @@ int linear_tc_backward(dbp_ctx *ctx, const void *delta, const void *X, const voi
     return DBP_OK;
 }
 
-// The sparse gather kernels: int8 codes, fp32 FMAs on the non-zero ones.
+// What the tensor-core kernels do not take: 5x5 layers of few channels by FMAs on the dense codes, everything else on the
+// sparse gather kernels (int8 codes, fp32 FMAs on the non-zero ones).
 template <typename ReadDensity>
 int gather_backward(dbp_ctx *ctx, const void *delta, const void *X, const void *W, int io, const ConvShape &s,
                     unsigned long long seed, float scale, const float *delta_in, dbp_sparse *q_out, float *dW, void *dX,
-                    float *db, unsigned flags, const ReadDensity &read_density) {
+                    float *db, unsigned flags, const uint8_t *mask, const ReadDensity &read_density) {
     const float *delta_p = nullptr;
     const int8_t *codes = nullptr;
     if (ctx->phase_w_src != nullptr && dX) {      // a stride-2 layer on phase images: W is a workspace not yet written
@@ -209,9 +210,27 @@ int gather_backward(dbp_ctx *ctx, const void *delta, const void *X, const void *
         const int pr = launch_phase_weights(ctx, ctx->phase_w_src, const_cast<void *>(W), io, s.Cout, s.Cin / 4);
         if (pr) return pr;
     }
-    int rc = quantize_for_products(ctx, delta, io, s.B * s.Cout * s.H * s.W, seed, scale, delta_in, q_out, &delta_p, &codes);
+    const bool direct = !(flags & DBP_FORCE_SPARSE) && direct5_supported(s, dW != nullptr, dX != nullptr);
+    SideJobs jobs;
+    if (direct && dW) { jobs.zero = dW; jobs.zero_bytes = sizeof(float) * static_cast<size_t>(s.Cout) * s.Cin * 25; }
+    // a *_host call: X is still on its way up on another stream
+    if (direct && dW && ctx->hook_before_dw && cudaStreamWaitEvent(ctx->stream, ctx->hook_before_dw, 0) != cudaSuccess) return DBP_ECUDA;
+    int rc = quantize_for_products(ctx, delta, io, s.B * s.Cout * s.H * s.W, seed, scale, delta_in, q_out, &delta_p, &codes, true, 0, 0,
+                                   nullptr, nullptr, nullptr, jobs, 0, nullptr, mask);
     if (rc) return rc;
     read_density();
+    if (direct) {
+        {
+            KernelTimer t(ctx, DBP_K_DX);
+            rc = launch_direct5(ctx, codes, X, W, io, delta_p, s, dW, dX, io == DBP_BF16 && !(flags & DBP_DX_F32));
+        }
+        if (!rc && ctx->hook_after_dx && cudaEventRecord(ctx->hook_after_dx, ctx->stream) != cudaSuccess) return DBP_ECUDA;
+        if (!rc && db) {
+            KernelTimer t(ctx, DBP_K_DB);
+            rc = launch_bias_grad(ctx, codes, delta_p, s, db);
+        }
+        return rc;
+    }
     if (dX) {
         const size_t wb = sizeof(float) * static_cast<size_t>(s.Cout) * s.Cin * s.k * s.k;
         if ((rc = ws_reserve(ctx, ctx->w_taps, wb))) return rc;
@@ -345,11 +364,11 @@ int conv_backward_impl(dbp_ctx *ctx, const void *delta, const void *X, const voi
     }
     // 3x3 layers read the codes position-major, 1x1 layers as planes
     const bool t3 = dense && (dX || dW) && conv3, t1 = dense && (dX || dW) && conv1;
-    // fp32 3x3 layers on the tensor-core kernels apply the mask while they read delta_a (statistics and the
-    // position-major quantizer); with a caller's sparse structure, or on any other path, delta_z is made first
-    const bool fold3 = mask && io == DBP_F32 && !q_out && t3;
-    const uint8_t *mask_q = fold3 ? mask : nullptr;
-    if (mask && !fold3) {      // every other path reads delta_z from memory: make it
+    // the statistics kernel and the quantizers apply the mask while they read delta_a; with a caller's sparse structure
+    // delta_z is made first
+    const bool fold = mask && !q_out;
+    const uint8_t *mask_q = fold ? mask : nullptr;
+    if (mask && !fold) {
         const int wr = ws_reserve(ctx, ctx->dz_tmp, static_cast<size_t>(numel) * sizeof(float));
         if (wr) return wr;
         KernelTimer t(ctx, DBP_K_GLUE);
@@ -368,11 +387,11 @@ int conv_backward_impl(dbp_ctx *ctx, const void *delta, const void *X, const voi
             ctx->nnz_pending = true;
     };
     if (lin) {
-        const int lr = linear_tc_backward(ctx, delta, X, W, io, s.B, s.Cout, s.Cin, seed, scale, delta_in, q_out, dW, dX, db, flags);
+        const int lr = linear_tc_backward(ctx, delta, X, W, io, s.B, s.Cout, s.Cin, seed, scale, delta_in, q_out, dW, dX, db, flags, mask_q);
         if (!lr) read_density();
         return lr;
     }
-    if (!t3 && !t1) return gather_backward(ctx, delta, X, W, io, s, seed, scale, delta_in, q_out, dW, dX, db, flags, read_density);
+    if (!t3 && !t1) return gather_backward(ctx, delta, X, W, io, s, seed, scale, delta_in, q_out, dW, dX, db, flags, mask_q, read_density);
     const int pieces = io == DBP_F32 ? 2 : 1, k = ctx->code_set;
     const bool dx_bf16 = io == DBP_BF16 && !(flags & DBP_DX_F32);
     // what the statistics kernel does on the side: the 1x1 dW kernel adds its partial sums into dW, so dW is cleared;
@@ -411,7 +430,7 @@ int conv_backward_impl(dbp_ctx *ctx, const void *delta, const void *X, const voi
     const void *codes_st = nullptr, *codes16 = nullptr, *codes_n = nullptr;
     int rc = quantize_for_products(ctx, delta, io, numel, seed, scale, delta_in, q_out, &delta_p, &codes, false,
                                    s.H * s.W, t1 ? tma_code_pitch(s) : 0, t1 ? &codes16 : nullptr,
-                                   t3 ? &s : nullptr, t3 ? &codes_n : nullptr, jobs, stack_g, &codes_st, t3 ? mask_q : nullptr);
+                                   t3 ? &s : nullptr, t3 ? &codes_n : nullptr, jobs, stack_g, &codes_st, mask_q);
     if (rc) return rc;
     // Activations the copy engine cannot address as they are (fp32: two bf16 pieces; planes that are no multiple of 16
     // bytes; stacked tiny planes) are re-written into the set's own buffer: beside the quantizer where the call ends with

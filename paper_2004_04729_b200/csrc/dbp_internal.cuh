@@ -153,7 +153,7 @@ int launch_quantize(dbp_ctx *ctx, const void *delta, int dtype, long long numel,
 // (or null), pitch a multiple of 8
 int launch_quantize_dense(dbp_ctx *ctx, const void *delta, int dtype, long long numel,
                           unsigned long long seed, const StepSource &step, int8_t *dense,
-                          void *planes_bf16, long long hw, long long pitch, bool count);
+                          void *planes_bf16, long long hw, long long pitch, bool count, const uint8_t *mask = nullptr);
 // position-major bf16 codes [B][HW][C] for the TMA-fed 3x3 kernels (and int8 codes in delta's order
 // when dense8 is not null)
 int launch_quantize_nhwc(dbp_ctx *ctx, const void *delta, int dtype, long long B, long long C, long long HW,
@@ -233,6 +233,11 @@ int launch_relu_backward(dbp_ctx *ctx, const float *da, const uint8_t *mask, flo
                          long long n);
 int launch_maxpool_backward(dbp_ctx *ctx, const float *g, const int8_t *argmax, float *out,
                             long long planes, long long h, long long w);
+
+// ---- direct5.cu: both products of a 5x5 layer of few channels by FMAs on the dense codes (dW cleared by the caller)
+bool direct5_supported(const ConvShape &s, bool want_dw, bool want_dx);
+int launch_direct5(dbp_ctx *ctx, const int8_t *codes, const void *X, const void *W, int io, const float *delta_p,
+                   const ConvShape &s, float *dW, void *dX, bool dx_bf16);
 
 // ---- strided_conv.cu: layout changes around a stride-2 layer run as a stride-1 layer on the input's phase images
 // (phases = 4: all four, channel (py*2+px)*Cin + ci; phases = 1: the even rows and columns only)

@@ -99,20 +99,34 @@ __device__ __forceinline__ void store_code(const CodeSinks &o, long long e, unsi
     }
 }
 
-template <typename T>
+// mask (fp32 tensors only): x is delta_a and the gradient is delta_a where mask != 0, else 0. The four mask bytes of a
+// vector as one word.
+__device__ __forceinline__ unsigned mask_word(const unsigned char *mask, long long e) { return __ldg(reinterpret_cast<const unsigned *>(mask + e)); }
+__device__ __forceinline__ void apply_mask(unsigned m, float (&v)[4]) {
+#pragma unroll
+    for (int j = 0; j < 4; ++j) v[j] = (m >> (8 * j)) & 0xffu ? v[j] : 0.f;
+}
+__device__ __forceinline__ void apply_mask(unsigned, float (&)[8]) {}                 // bf16 tensors take no mask
+
+template <typename T, bool MASKED>
 __global__ void __launch_bounds__(kThreads, kBlocksPerSM)
 quantize_dense_kernel(const T *__restrict__ x, long long n, unsigned long long seed, const StepSource step,
-                      const CodeSinks out, DeviceState *__restrict__ st) {
+                      const CodeSinks out, DeviceState *__restrict__ st, const unsigned char *__restrict__ mask) {
     constexpr int V = Vec<T>::V;
     const long long nvec = n / V;
     const long long stride = static_cast<long long>(gridDim.x) * kThreads;
     long long i = static_cast<long long>(blockIdx.x) * kThreads + threadIdx.x;
     // two vectors per thread and round: i and i + stride
     uint4 r0, r1;
+    unsigned m0 = 0, m1 = 0;
     unsigned long long u0[V / 2], u1[V / 2];
     auto load = [&](long long k) {
         r0 = k < nvec ? Vec<T>::raw(x + k * V) : make_uint4(0u, 0u, 0u, 0u);
         r1 = k + stride < nvec ? Vec<T>::raw(x + (k + stride) * V) : make_uint4(0u, 0u, 0u, 0u);
+        if (MASKED) {
+            m0 = k < nvec ? mask_word(mask, k * V) : 0u;
+            m1 = k + stride < nvec ? mask_word(mask, (k + stride) * V) : 0u;
+        }
     };
     auto draw = [&](long long k) {
         dithers_of<V>(k * V, seed, u0);
@@ -128,8 +142,10 @@ quantize_dense_kernel(const T *__restrict__ x, long long n, unsigned long long s
     for (; i < nvec; ) {
         float v[V], f0[V], f1[V];
         Vec<T>::values(r0, v);
+        if (MASKED) apply_mask(m0, v);
         decide<V>(v, u0, inv, f0, sat);
         Vec<T>::values(r1, v);
+        if (MASKED) apply_mask(m1, v);
         const bool two = i + stride < nvec;
         decide<V>(v, u1, inv, f1, sat);
         const long long k = i;
@@ -152,7 +168,7 @@ quantize_dense_kernel(const T *__restrict__ x, long long n, unsigned long long s
         for (long long e = nvec * V; e < n; ++e) {
             float ua, ub;
             unpack2(dither2(counter_of(e & ~1ll, seed)), ua, ub);
-            const unsigned q = careful_bits(Vec<T>::one(x + e), inv, (e & 1) ? ub : ua, sat) & 0xffu;
+            const unsigned q = careful_bits(!MASKED || __ldg(mask + e) ? Vec<T>::one(x + e) : 0.f, inv, (e & 1) ? ub : ua, sat) & 0xffu;
             store_code(out, e, q);
             nnz += q != 0u;
         }
@@ -178,15 +194,6 @@ __device__ __forceinline__ unsigned tile_off(int p, int c) {
     return static_cast<unsigned>(p) * 128u + (((static_cast<unsigned>(c) >> 3) ^ ((static_cast<unsigned>(p) >> 3) & 7u)) << 4) +
            ((static_cast<unsigned>(c) & 7u) << 1);
 }
-
-// mask (fp32 tensors only): x is delta_a and the gradient is delta_a where mask != 0, else 0. The four mask bytes of a
-// vector as one word.
-__device__ __forceinline__ unsigned mask_word(const unsigned char *mask, long long e) { return __ldg(reinterpret_cast<const unsigned *>(mask + e)); }
-__device__ __forceinline__ void apply_mask(unsigned m, float (&v)[4]) {
-#pragma unroll
-    for (int j = 0; j < 4; ++j) v[j] = (m >> (8 * j)) & 0xffu ? v[j] : 0.f;
-}
-__device__ __forceinline__ void apply_mask(unsigned, float (&)[8]) {}                 // bf16 tensors take no mask
 
 // V of the elements of a 128-bit vector (8-byte loads for bf16 planes that are only a multiple of 4)
 template <typename T, int V>
@@ -418,11 +425,12 @@ cudaError_t run_nhwc(dbp_ctx *ctx, const void *delta, int B, int C, int HW, unsi
 // and the run leaves as one contiguous copy (the padding of a plane is never read by anybody).
 constexpr int kOddMaxSmem = 12 * 1024;            // bytes of the staged run (planes x pitch bf16)
 
-template <typename T>
+template <typename T, bool MASKED>
 __global__ void __launch_bounds__(kThreads)
 quantize_planes_odd_kernel(const T *__restrict__ x, long long nplanes, int hw, int pitch, int planes_per_run,
                            unsigned long long seed, const StepSource step, unsigned short *__restrict__ out,
-                           int8_t *__restrict__ dense8, DeviceState *__restrict__ st, int count) {
+                           int8_t *__restrict__ dense8, DeviceState *__restrict__ st, int count,
+                           const unsigned char *__restrict__ mask) {
     constexpr int V = Vec<T>::V;
     constexpr int NP = 2;                                           // vectors of the first run loaded and drawn ahead
     __shared__ __align__(16) unsigned short run_s[kOddMaxSmem / 2];
@@ -453,6 +461,7 @@ quantize_planes_odd_kernel(const T *__restrict__ x, long long nplanes, int hw, i
             float a[V], f[V];
             unsigned h[V / 2];
             Vec<T>::values(q, a);
+            if (MASKED) apply_mask(mask_word(mask, e_base + static_cast<long long>(v) * V), a);
             decide<V>(a, d, inv, f, sat);
             pack_bf16<V>(f, h);
             count_pairs<V>(h, nz2);
@@ -492,41 +501,42 @@ quantize_planes_odd_kernel(const T *__restrict__ x, long long nplanes, int hw, i
 
 int launch_quantize_dense(dbp_ctx *ctx, const void *delta, int dtype, long long numel,
                           unsigned long long seed, const StepSource &step, int8_t *dense,
-                          void *planes_bf16, long long hw, long long pitch, bool count) {
+                          void *planes_bf16, long long hw, long long pitch, bool count, const uint8_t *mask) {
+    if (mask != nullptr && dtype != DBP_F32) return DBP_EUNSUPPORTED;
+    const unsigned char *m = static_cast<const unsigned char *>(mask);
+    unsigned short *planes = static_cast<unsigned short *>(planes_bf16);
     const int v = dtype == DBP_F32 ? 4 : 8;
+    const float *xf = static_cast<const float *>(delta);
+    const __nv_bfloat16 *xb = static_cast<const __nv_bfloat16 *>(delta);
     // odd plane sizes at a padded pitch: whole runs of planes through shared memory
-    if (planes_bf16 != nullptr && hw > 0 && pitch != hw && (hw & 3) != 0 && numel % hw == 0 && (numel / hw) % 8 == 0 &&
+    if (planes != nullptr && hw > 0 && pitch != hw && (hw & 3) != 0 && numel % hw == 0 && (numel / hw) % 8 == 0 &&
         8 * pitch * 2 <= kOddMaxSmem && hw < (1 << 20)) {
         const long long nplanes = numel / hw;
         int per_run = static_cast<int>(kOddMaxSmem / 2 / pitch / 8 * 8);          // planes per run: a multiple of 8
         const long long want = (4096 + 8 * hw - 1) / (8 * hw) * 8;               // about 4096 elements a run
         if (per_run > want) per_run = static_cast<int>(want);
-        long long nruns = (nplanes + per_run - 1) / per_run;
-        long long blocks = nruns < static_cast<long long>(ctx->sm_count) * 8 ? nruns : static_cast<long long>(ctx->sm_count) * 8;
-        cudaError_t e;
-        if (dtype == DBP_F32)
-            e = launch_chained(quantize_planes_odd_kernel<float>, dim3(static_cast<unsigned>(blocks)), dim3(kThreads), 0, ctx->stream,
-                               static_cast<const float *>(delta), nplanes, static_cast<int>(hw), static_cast<int>(pitch), per_run, seed,
-                               step, static_cast<unsigned short *>(planes_bf16), dense, ctx->state, count ? 1 : 0);
-        else
-            e = launch_chained(quantize_planes_odd_kernel<__nv_bfloat16>, dim3(static_cast<unsigned>(blocks)), dim3(kThreads), 0, ctx->stream,
-                               static_cast<const __nv_bfloat16 *>(delta), nplanes, static_cast<int>(hw), static_cast<int>(pitch), per_run,
-                               seed, step, static_cast<unsigned short *>(planes_bf16), dense, ctx->state, count ? 1 : 0);
-        return cuda_ok(e);
+        const long long nruns = (nplanes + per_run - 1) / per_run, cap = static_cast<long long>(ctx->sm_count) * 8;
+        auto go = [&](auto kern, auto x) {
+            return cuda_ok(launch_chained(kern, dim3(static_cast<unsigned>(nruns < cap ? nruns : cap)), dim3(kThreads), 0, ctx->stream, x,
+                                          nplanes, static_cast<int>(hw), static_cast<int>(pitch), per_run, seed, step, planes, dense,
+                                          ctx->state, count ? 1 : 0, m));
+        };
+        return dtype != DBP_F32 ? go(quantize_planes_odd_kernel<__nv_bfloat16, false>, xb)
+               : m              ? go(quantize_planes_odd_kernel<float, true>, xf)
+                                : go(quantize_planes_odd_kernel<float, false>, xf);
     }
     long long blocks = (numel / v + 2 * kThreads - 1) / (2 * kThreads);
     if (blocks < 1) blocks = 1;
     const long long cap = static_cast<long long>(ctx->sm_count) * kBlocksPerSM;
     if (blocks > cap) blocks = cap;
-    CodeSinks out{dense, static_cast<unsigned short *>(planes_bf16), hw > 0 ? hw : 1, pitch > 0 ? pitch : 1, count ? 1 : 0};
-    cudaError_t e;
-    if (dtype == DBP_F32)
-        e = launch_chained(quantize_dense_kernel<float>, dim3(static_cast<unsigned>(blocks)), dim3(kThreads), 0, ctx->stream,
-                           static_cast<const float *>(delta), numel, seed, step, out, ctx->state);
-    else
-        e = launch_chained(quantize_dense_kernel<__nv_bfloat16>, dim3(static_cast<unsigned>(blocks)), dim3(kThreads), 0,
-                           ctx->stream, static_cast<const __nv_bfloat16 *>(delta), numel, seed, step, out, ctx->state);
-    return cuda_ok(e);
+    const CodeSinks out{dense, planes, hw > 0 ? hw : 1, pitch > 0 ? pitch : 1, count ? 1 : 0};
+    auto go = [&](auto kern, auto x) {
+        return cuda_ok(launch_chained(kern, dim3(static_cast<unsigned>(blocks)), dim3(kThreads), 0, ctx->stream, x, numel, seed, step, out,
+                                      ctx->state, m));
+    };
+    return dtype != DBP_F32 ? go(quantize_dense_kernel<__nv_bfloat16, false>, xb)
+           : m              ? go(quantize_dense_kernel<float, true>, xf)
+                            : go(quantize_dense_kernel<float, false>, xf);
 }
 
 // delta_z [B][C][HW] -> bf16 codes [B][HW][C rounded up to a multiple of 8] and, when dense8 is not null, int8 codes

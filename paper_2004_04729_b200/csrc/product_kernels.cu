@@ -318,6 +318,8 @@ __global__ void __launch_bounds__(256) bias_grad_kernel(const int8_t *__restrict
 // the size and the pointers allow
 __global__ void __launch_bounds__(256) relu_backward_kernel(const float *__restrict__ da, const uint8_t *__restrict__ mask,
                                                             float *__restrict__ dz, long long n, int vec) {
+    chain_wait();
+    chain_release();
     const long long stride = static_cast<long long>(gridDim.x) * blockDim.x;
     long long i = blockIdx.x * static_cast<long long>(blockDim.x) + threadIdx.x;
     if (vec) {
@@ -336,6 +338,8 @@ __global__ void __launch_bounds__(256) relu_backward_kernel(const float *__restr
 // its four outputs (two pairs); argmax in {0,1,2,3} is the row-major position of the forward maximum
 __global__ void __launch_bounds__(256) maxpool_backward_kernel(const float *__restrict__ g, const int8_t *__restrict__ am,
                                                                float *__restrict__ out, long long planes, int h, int w) {
+    chain_wait();
+    chain_release();
     const long long n = planes * h * w;
     for (long long i = blockIdx.x * static_cast<long long>(blockDim.x) + threadIdx.x; i < n;
          i += static_cast<long long>(gridDim.x) * blockDim.x) {
@@ -493,19 +497,16 @@ int launch_bias_grad(dbp_ctx *ctx, const int8_t *codes, const float *delta_p, co
 }
 
 int launch_relu_backward(dbp_ctx *ctx, const float *da, const uint8_t *mask, float *dz, long long n) {
-    note_launch();
     const int vec = (n % 4 == 0) && ((reinterpret_cast<uintptr_t>(da) | reinterpret_cast<uintptr_t>(dz)) % 16 == 0) &&
                     (reinterpret_cast<uintptr_t>(mask) % 4 == 0);
-    relu_backward_kernel<<<blocks_for(vec ? n / 4 : n, 256, ctx->sm_count * 8), 256, 0, ctx->stream>>>(da, mask, dz, n, vec);
-    return cuda_ok(cudaGetLastError());
+    return cuda_ok(launch_chained(relu_backward_kernel, dim3(blocks_for(vec ? n / 4 : n, 256, ctx->sm_count * 8)), dim3(256), 0,
+                                  ctx->stream, da, mask, dz, n, vec));
 }
 
 int launch_maxpool_backward(dbp_ctx *ctx, const float *g, const int8_t *argmax, float *out,
                             long long planes, long long h, long long w) {
-    note_launch();
-    maxpool_backward_kernel<<<blocks_for(planes * h * w, 256, ctx->sm_count * 8), 256, 0, ctx->stream>>>(
-        g, argmax, out, planes, static_cast<int>(h), static_cast<int>(w));
-    return cuda_ok(cudaGetLastError());
+    return cuda_ok(launch_chained(maxpool_backward_kernel, dim3(blocks_for(planes * h * w, 256, ctx->sm_count * 8)), dim3(256), 0,
+                                  ctx->stream, g, argmax, out, planes, static_cast<int>(h), static_cast<int>(w)));
 }
 
 }  // namespace dbp

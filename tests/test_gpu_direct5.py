@@ -1,0 +1,50 @@
+"""5x5 layers of few channels (both products in one launch on the dense codes): parity with the oracle at the edges of the
+kernel's register tiles, with a folded ReLU mask, each product by itself and more images than CTAs."""
+import numpy as np
+import pytest
+import torch
+
+import oracle
+import workloads as wl
+
+pytestmark = pytest.mark.gpu
+TOL = 1e-5
+
+
+@pytest.fixture(scope="module")
+def ctx():
+    import paper_2004_04729_b200 as dbp
+    c = dbp.Context(0)
+    yield c
+    c.close()
+
+
+@pytest.mark.parametrize("B,Ci,Co,H,W,dtype", [
+    (3, 1, 6, 32, 32, "f32"), (5, 6, 16, 16, 16, "f32"),     # LeNet-5-like
+    (2, 3, 5, 7, 9, "f32"),                                  # odd everything: rows of 9, an odd input channel, dW size % 4 != 0
+    (2, 1, 1, 1, 1, "f32"), (1, 12, 32, 18, 18, "f32"), (2, 2, 3, 5, 2, "bf16"), (300, 2, 4, 6, 6, "f32"), (3, 7, 12, 9, 8, "bf16")])
+def test_layers_of_few_channels(ctx, B, Ci, Co, H, W, dtype):
+    import paper_2004_04729_b200 as dbp
+    L = wl.conv_layer(B, Ci, Co, H, W, 5, data_seed=B + Ci + Co + H, scale=2.0, seed=4, dtype=dtype)
+    mask = (np.random.default_rng(B + H).random(L.delta.shape) < 0.6) if dtype == "f32" else np.ones(L.delta.shape, bool)
+    dz = (L.delta * mask).astype(np.float32)
+    tdt = torch.bfloat16 if dtype == "bf16" else torch.float32
+    d, X, Wt = (torch.from_numpy(np.ascontiguousarray(a)).to(tdt).cuda() for a in (L.delta, L.X, L.W))
+    m = torch.from_numpy(mask.astype(np.uint8)).cuda()
+    def call(**kw):
+        if dtype == "f32":
+            ctx.set_relu_mask(m)
+        return dbp.dithered_conv_backward(ctx, d, X, Wt, L.seed, L.scale, flags=dbp.DBP_DX_F32, **kw)
+    out = call(need_db=True)
+    D, nnz = ctx.last_step()
+    assert ctx.last_device_status() == (0, 0)
+    D = np.float32(D)
+    codes, onnz, _ = oracle.nsd_codes(dz, L.seed, D)
+    assert nnz == onnz
+    ref = oracle.conv_backward(codes, D, L.X, L.W, with_abs=True)
+    for key in ("dW", "dX", "db"):
+        g = out[key].double().cpu().numpy()
+        assert np.linalg.norm(g - ref[key]) <= TOL * np.linalg.norm(ref[key]) + 1e-30, key
+        assert np.all(np.abs(g - ref[key]) <= TOL * ref["S_" + key] + 1e-30), key
+    assert torch.equal(call(need_dW=False)["dX"], out["dX"])
+    assert (call(need_dX=False)["dW"] - out["dW"]).abs().max().item() <= 1e-5 * out["dW"].abs().max().item() + 1e-30
