@@ -43,8 +43,9 @@ __device__ __forceinline__ void mbar_arrive_on_cp_async(unsigned long long *bar)
 }
 // Waits for the phase with the given parity. try_wait suspends the thread in hardware until the
 // phase completes or a short system time limit passes, so a waiter wakes as soon as the barrier
-// flips (a test_wait/nanosleep poll adds its sleep to every hand-over). Returns false, with the
-// error flag set, when the phase did not complete within about half a second.
+// flips (a test_wait/nanosleep poll adds its sleep to every hand-over; a bare test_wait loop of a CTA's
+// epilogue warps takes shared-memory bandwidth from the MMAs' operands: VGG-16 layer set 1074 against
+// 1048 us). Returns false, with the error flag set, when the phase did not complete within about half a second.
 __device__ __forceinline__ bool mbar_try(unsigned addr, unsigned parity) {
     unsigned done;
     asm volatile(
@@ -70,8 +71,8 @@ __device__ __forceinline__ bool mbar_wait(unsigned long long *bar, unsigned pari
     const long long t0 = clock64();
     do {
 #pragma unroll 1
-        for (int i = 0; i < 64; ++i)
-            if (mbar_test(addr, parity)) return true;
+        for (int i = 0; i < 16; ++i)
+            if (mbar_try(addr, parity)) return true;
     } while (clock64() - t0 <= budget);
     atomicExch(err_flag, 1);
     return false;
