@@ -419,6 +419,7 @@ int conv_backward_impl(dbp_ctx *ctx, const void *delta, const void *X, const voi
         if (w_side && ctx->phase_cin > 0 && s.Cin == 4ll * ctx->phase_cin) {
             jobs.w_src = ctx->phase_w_src;
             jobs.phase_cin = ctx->phase_cin;
+            jobs.skip_dead = ctx->phase_cin % 128 == 0;      // whole channel tiles of one phase: see tc3_tma_dx.cu
         } else {
             KernelTimer t(ctx, DBP_K_GLUE);
             const int pr = launch_phase_weights(ctx, ctx->phase_w_src, const_cast<void *>(W), io, s.Cout, s.Cin / 4);
@@ -426,7 +427,7 @@ int conv_backward_impl(dbp_ctx *ctx, const void *delta, const void *X, const voi
         }
     }
     // tiny planes: the weight-gradient kernel reads the images stacked into tall ones
-    const int stack_g = (t3 && dW) ? tc3_stack_images(s, io) : 0;
+    const int stack_g = (t3 && dW && !ctx->strided) ? tc3_stack_images(s, io) : 0;
     const void *codes_st = nullptr, *codes16 = nullptr, *codes_n = nullptr;
     int rc = quantize_for_products(ctx, delta, io, numel, seed, scale, delta_in, q_out, &delta_p, &codes, false,
                                    s.H * s.W, t1 ? tma_code_pitch(s) : 0, t1 ? &codes16 : nullptr,
@@ -438,11 +439,13 @@ int conv_backward_impl(dbp_ctx *ctx, const void *delta, const void *X, const voi
     // VGG-16 layer set) or where a *_host call's activations are still on their way up.
     const void *Xp = X;
     long long x_pitch = s.H * s.W;
-    const bool rewrite_x = dW && (io == DBP_F32 || x_pitch % 8 != 0);
+    const StridedLayer *st2 = ctx->strided;
+    const bool rewrite_x = dW && (st2 || io == DBP_F32 || x_pitch % 8 != 0);
     const bool forked = dX && dW && ctx->aux != nullptr;
     const bool late_x = ctx->hook_before_dw != nullptr || (forked && (flags & DBP_DW_ASYNC));
     auto write_x = [&](bool beside) -> int {
         KernelTimer t(ctx, DBP_K_DW_DENSE);
+        if (st2) return launch_phase_rows(ctx, st2->X, ctx->x_padded[k].ptr, io, s.B, st2->Cin, st2->H, st2->W, st2->phases, x_pitch, beside);
         return stack_g > 0 ? launch_x_stacked(ctx, static_cast<const float *>(X), ctx->x_padded[k].ptr, s, stack_g, beside)
                            : launch_rows_job(ctx, RowsJob{X, ctx->x_padded[k].ptr, io == DBP_F32, s.B * s.Cin, s.H * s.W, x_pitch}, beside);
     };
@@ -468,6 +471,11 @@ int conv_backward_impl(dbp_ctx *ctx, const void *delta, const void *X, const voi
                 : launch_tc3_tma_dx(ctx, codes_n, W, io, delta_p, s, dX, dx_bf16, &ctx->state->tc_timeout, w_side);
         if (rc) return rc;
     }
+    if (dX && st2) {                             // from the phase images to the layer's own dX, beside the dW kernels
+        KernelTimer t(ctx, DBP_K_GLUE);
+        rc = launch_from_phases(ctx, dX, st2->dX, st2->dx_f32, s.B, st2->Cin, st2->H, st2->W, st2->phases);
+        if (rc) return rc;
+    }
     if (ctx->hook_after_dx && cudaEventRecord(ctx->hook_after_dx, ctx->stream) != cudaSuccess) return DBP_ECUDA;
     if (db && dX) {
         KernelTimer t(ctx, DBP_K_DB);
@@ -485,6 +493,8 @@ int conv_backward_impl(dbp_ctx *ctx, const void *delta, const void *X, const voi
         if (stack_g > 0) sw = ConvShape{s.B / stack_g, s.Cin, s.Cout, static_cast<long long>(stack_g) * (s.H + 1), s.W, 3};
         rc = t1 ? launch_tma_dw(ctx, codes16, Xp, pieces, x_pitch, delta_p, s, dW, &ctx->state->tc_timeout)
                 : launch_tc3_tma_dw(ctx, stack_g > 0 ? codes_st : codes_n, Xp, pieces, x_pitch, delta_p, sw, dW, &ctx->state->tc_timeout);
+        if (!rc && st2 && s.k == 3 && !ctx->phase_dw_done)
+            rc = launch_strided_dw(ctx, dW, st2->dW, s.Cout, st2->Cin);
     }
     ctx->stream = caller;
     if (forked) {
@@ -509,9 +519,10 @@ int conv_backward_impl(dbp_ctx *ctx, const void *delta, const void *X, const voi
 }
 
 // A stride-2 layer (k = 1 or 3, pad (k-1)/2, even H and W) as the stride-1 layer on the phase images of X
-// (strided_conv.cu): delta is that layer's own gradient [B][Cout][H/2][W/2] and is quantized as it is; X, W, dX
-// and dW pass through layout kernels on the context's stream. The weight-gradient kernels of such a call are
-// always joined before it returns (the workspaces they read are reused by the next strided call).
+// (strided_conv.cu): delta is that layer's own gradient [B][Cout][H/2][W/2] and is quantized as it is. On the tensor-core
+// path X is re-laid beside the quantizer as the padded rows its dW kernels read, and dX leaves the phase layout right behind
+// its kernel, beside dW. On the gather kernels X, W, dX and dW pass through layout kernels on the context's stream. The
+// weight gradient is always joined before the call returns.
 int conv_backward_stride2(dbp_ctx *ctx, const void *delta, const void *X, const void *W, int io, const ConvShape &s,
                           unsigned long long seed, float scale, const float *delta_in, dbp_sparse *q_out, float *dW,
                           void *dX, float *db, unsigned flags) {
@@ -533,10 +544,34 @@ int conv_backward_stride2(dbp_ctx *ctx, const void *delta, const void *X, const 
     const bool dx_f32 = io == DBP_F32 || (flags & DBP_DX_F32);
     const size_t nxp = static_cast<size_t>(in.B) * in.Cin * Ho * Wo, nwp = static_cast<size_t>(in.Cout) * in.Cin * s.k * s.k;
     int rc;
-    if (dW && (rc = ws_reserve(ctx, ctx->s2_x, nxp * es))) return rc;
+    const bool tensor = (dW || dX) && !(flags & DBP_FORCE_SPARSE) && ((flags & DBP_FORCE_DENSE) || ctx->crossover <= 0.f) &&
+                        (s.k == 3 ? tc3_tma_supported(in, io) : tma_dx_supported(in, io));
     if (dX && (rc = ws_reserve(ctx, ctx->s2_dx, nxp * (dx_f32 ? 4 : 2)))) return rc;
     if (dX && s.k == 3 && (rc = ws_reserve(ctx, ctx->s2_w, nwp * es))) return rc;
     if (dW && s.k == 3 && (rc = ws_reserve(ctx, ctx->s2_dw, nwp * sizeof(float)))) return rc;
+    const void *Win = dX ? (s.k == 3 ? ctx->s2_w.ptr : W) : nullptr;
+    float *dWin = dW ? (s.k == 3 ? static_cast<float *>(ctx->s2_dw.ptr) : dW) : nullptr;
+    auto run = [&](const void *Xin, unsigned f) {
+        ctx->next_mask = mask;
+        ctx->phase_cin = s.k == 3 ? static_cast<int>(s.Cin) : 0;  // the 3x3 tensor-core kernels skip the taps that are zero by construction
+        ctx->phase_dw_out = (s.k == 3 && dW) ? dW : nullptr;
+        ctx->phase_w_src = (s.k == 3 && dX) ? W : nullptr;        // the phase weights are made inside, in the form the path wants
+        ctx->phase_dw_done = false;
+        const int r = conv_backward_impl(ctx, delta, dW ? Xin : nullptr, Win, io, in, seed, scale, delta_in, q_out, dWin,
+                                         dX ? ctx->s2_dx.ptr : nullptr, db, f);
+        ctx->phase_cin = 0;
+        ctx->phase_dw_out = nullptr;
+        ctx->phase_w_src = nullptr;
+        return r;
+    };
+    if (tensor) {
+        const StridedLayer st2{X, dX, dx_f32 ? 1 : 0, dW, s.Cin, static_cast<int>(s.H), static_cast<int>(s.W), phases};
+        ctx->strided = &st2;
+        rc = run(X, flags & ~DBP_DW_ASYNC);
+        ctx->strided = nullptr;
+        return rc;
+    }
+    if (dW && (rc = ws_reserve(ctx, ctx->s2_x, nxp * es))) return rc;
     // a *_host call: X is still on its way up on another stream, and dX is read back after an event
     cudaEvent_t after_dx = ctx->hook_after_dx;
     ctx->hook_after_dx = nullptr;
@@ -546,18 +581,7 @@ int conv_backward_stride2(dbp_ctx *ctx, const void *delta, const void *X, const 
         KernelTimer t(ctx, DBP_K_GLUE);
         if ((rc = launch_phases_of(ctx, X, ctx->s2_x.ptr, io, s.B, s.Cin, static_cast<int>(s.H), static_cast<int>(s.W), phases))) return rc;
     }
-    ctx->next_mask = mask;
-    ctx->phase_cin = s.k == 3 ? static_cast<int>(s.Cin) : 0;      // the 3x3 tensor-core kernels skip the taps that are zero by construction
-    ctx->phase_dw_out = (s.k == 3 && dW) ? dW : nullptr;
-    ctx->phase_w_src = (s.k == 3 && dX) ? W : nullptr;            // the phase weights are made inside, in the form the path wants
-    ctx->phase_dw_done = false;
-    rc = conv_backward_impl(ctx, delta, dW ? ctx->s2_x.ptr : nullptr, dX ? (s.k == 3 ? ctx->s2_w.ptr : W) : nullptr, io, in,
-                            seed, scale, delta_in, q_out,
-                            dW ? (s.k == 3 ? static_cast<float *>(ctx->s2_dw.ptr) : dW) : nullptr,
-                            dX ? ctx->s2_dx.ptr : nullptr, db, flags & ~DBP_DW_ASYNC);
-    ctx->phase_cin = 0;
-    ctx->phase_dw_out = nullptr;
-    ctx->phase_w_src = nullptr;
+    rc = run(ctx->s2_x.ptr, flags & ~DBP_DW_ASYNC);
     if (rc) return rc;
     if (dX) {
         KernelTimer t(ctx, DBP_K_GLUE);

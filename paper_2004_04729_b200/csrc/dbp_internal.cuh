@@ -33,6 +33,16 @@ struct Workspace {
     size_t bytes = 0;
 };
 
+// A stride-2 layer's own tensors, while the tensor-core path runs it as a stride-1 layer on phase images.
+struct StridedLayer {
+    const void *X;                      // [B][Cin][H][W]
+    void *dX;                           // the same shape, fp32 or the layer's type
+    int dx_f32;
+    float *dW;                          // [Cout][Cin][k][k]
+    long long Cin;
+    int H, W, phases;
+};
+
 }  // namespace dbp
 
 struct dbp_ctx {
@@ -60,6 +70,7 @@ struct dbp_ctx {
     float *phase_dw_out = nullptr;      // that layer's dW: the 3x3 weight-gradient kernels write it directly when they run in phase mode ...
     bool phase_dw_done = false;         // ... and say so here
     int phase_cin = 0;                  // > 0 while a stride-2 3x3 layer runs as a stride-1 layer on phase images: its own channel count
+    const dbp::StridedLayer *strided = nullptr;   // set while a stride-2 layer runs as a stride-1 layer on phase images made inside
     dbp::Workspace s2_x, s2_w, s2_dx, s2_dw;   // stride-2 layers: phase images of X, phase weights, and the two products in that layout
     float *delta_sets = nullptr;        // device float[2]: the step size that belongs to each set
     int code_set = 0;                   // the set the next call writes
@@ -116,7 +127,7 @@ struct StepSource {
 // ---- nsd_kernels.cu
 // Work the statistics kernel does on the side for the layer's product kernels (its blocks have time to spare
 // and this saves launches): clearing a buffer (16-byte aligned, a multiple of 16 bytes), and re-laying 3x3
-// weights [Cout][Cin][9] as [Cout][taps][Cin] bf16 (taps = 9 for bf16 weights; 18 for fp32 weights, split into
+// weights [Cout][Cin][9] as [taps][Cout][Cin rounded up to 8] bf16 (taps = 9 for bf16 weights; 18 for fp32 weights, split into
 // two bf16 pieces: taps 0-8 the rounded values, 9-17 what the rounding left over).
 // Rows of a matrix as bf16 rows of `pitch` values (a multiple of 8, extra columns zero), which the copy engine can
 // address: fp32 rows become two pieces, rows * pitch apart (the rounded values, and the remainders rounded).
@@ -136,6 +147,7 @@ struct SideJobs {
     int w_f32 = 0;
     long long Cout = 0, Cin = 0;
     int phase_cin = 0;                 // > 0: w_src holds a stride-2 layer's own weights [Cout][phase_cin][9], Cin = 4 phase_cin
+    int skip_dead = 0;                 // ... whose taps that are zero by construction nobody reads: they are not written
 };
 // publish: where the quantizer is to write the step size beside the context's state (entries may be null); *step tells
 // the quantizer where to take it from
@@ -242,6 +254,9 @@ int launch_direct5(dbp_ctx *ctx, const int8_t *codes, const void *X, const void 
 // ---- strided_conv.cu: layout changes around a stride-2 layer run as a stride-1 layer on the input's phase images
 // (phases = 4: all four, channel (py*2+px)*Cin + ci; phases = 1: the even rows and columns only)
 int launch_phases_of(dbp_ctx *ctx, const void *X, void *Xp, int io, long long B, long long Cin, int H, int W, int phases);
+// the same as bf16 rows for the copy engine (fp32: two pieces), [pieces][B][phases * Cin][pitch]; beside: as launch_rows_job
+int launch_phase_rows(dbp_ctx *ctx, const void *X, void *Xp, int io, long long B, long long Cin, int H, int W, int phases,
+                      long long pitch, bool beside);
 int launch_from_phases(dbp_ctx *ctx, const void *dXp, void *dX, int f32, long long B, long long Cin, int H, int W, int phases);
 int launch_phase_weights(dbp_ctx *ctx, const void *W, void *Wp, int io, long long Cout, long long Cin);
 int launch_strided_dw(dbp_ctx *ctx, const float *dWp, float *dW, long long Cout, long long Cin);

@@ -134,7 +134,7 @@ statistics_kernel(const T *__restrict__ x, long long n, double *__restrict__ par
         // side jobs for the layer's product kernels: operands re-written as bf16 rows the copy engine can address
         for (int j = 0; j < jobs.nrows; ++j) rows_job(jobs.rows[j], first, step);
     }
-    // side job for the layer's 3x3 input-gradient kernel: weights [co][ci][9] -> [co][tap][ci] bf16 (for fp32
+    // side job for the layer's 3x3 input-gradient kernel: weights [co][ci][9] -> [tap][co][ci] bf16 (for fp32
     // weights two pieces: taps 0-8 the values rounded to bf16, taps 9-17 the remainders rounded to bf16).
     // w_phase_cin > 0: the layer is a stride-2 layer run on the four phase images of its input; w_src holds that
     // layer's own weights [co][w_phase_cin][9] and channel ph * w_phase_cin + c of the re-laid weights is phase
@@ -146,9 +146,9 @@ statistics_kernel(const T *__restrict__ x, long long n, double *__restrict__ par
         const int w_f32 = jobs.w_f32, w_cin = static_cast<int>(jobs.Cin), w_phase_cin = jobs.phase_cin;
         const int w_pitch = (w_cin + 7) & ~7;      // rows of a multiple of 16 bytes, for the copy engine
         const long long w_cout = jobs.Cout;
-        const int per_co = 9 * w_pitch, taps = w_f32 ? 18 : 9;
+        const long long per_tap = w_cout * w_pitch;     // taps outermost: the copy engine takes several taps in one box
         for (long long co = blockIdx.x; co < w_cout; co += gridDim.x) {
-            unsigned short *dst = w_dst + co * taps * w_pitch;
+            unsigned short *dst = w_dst + co * w_pitch;
             // a thread takes one channel and all nine taps: nine independent loads, then stores that run along ci
             for (int ci = threadIdx.x; ci < w_cin; ci += kThreads) {
                 int ph = 0;
@@ -174,10 +174,11 @@ statistics_kernel(const T *__restrict__ x, long long n, double *__restrict__ par
                     for (int t = 0; t < 9; ++t) w[t] = k[t] >= 0 ? __ldg(static_cast<const float *>(w_src) + base + k[t]) : 0.f;
 #pragma unroll
                     for (int t = 0; t < 9; ++t) {
+                        if (k[t] < 0 && jobs.skip_dead) continue;
                         const __nv_bfloat16 hi = __float2bfloat16_rn(w[t]);
                         const __nv_bfloat16 lo = __float2bfloat16_rn(w[t] - __bfloat162float(hi));
-                        dst[t * w_pitch + ci] = *reinterpret_cast<const unsigned short *>(&hi);
-                        dst[per_co + t * w_pitch + ci] = *reinterpret_cast<const unsigned short *>(&lo);
+                        dst[t * per_tap + ci] = *reinterpret_cast<const unsigned short *>(&hi);
+                        dst[(9 + t) * per_tap + ci] = *reinterpret_cast<const unsigned short *>(&lo);
                     }
                 } else {
                     unsigned short w[9];
@@ -185,7 +186,8 @@ statistics_kernel(const T *__restrict__ x, long long n, double *__restrict__ par
                     for (int t = 0; t < 9; ++t)
                         w[t] = k[t] >= 0 ? __ldg(static_cast<const unsigned short *>(w_src) + base + k[t]) : static_cast<unsigned short>(0);
 #pragma unroll
-                    for (int t = 0; t < 9; ++t) dst[t * w_pitch + ci] = w[t];
+                    for (int t = 0; t < 9; ++t)
+                        if (k[t] >= 0 || !jobs.skip_dead) dst[t * per_tap + ci] = w[t];
                 }
             }
         }

@@ -32,6 +32,7 @@ template <> struct Cols<float, 1> { using vec = float2; using half = float; };
 template <> struct Cols<float, 2> { using vec = float4; using half = float2; };
 template <> struct Cols<__nv_bfloat16, 1> { using vec = unsigned; using half = unsigned short; };
 template <> struct Cols<__nv_bfloat16, 2> { using vec = uint2; using half = unsigned; };
+template <> struct Cols<__nv_bfloat16, 4> { using vec = uint4; using half = uint2; };
 
 // even-numbered and odd-numbered elements of a vector of 2 NP columns
 __device__ __forceinline__ void split_cols(const float2 v, float &e, float &o) { e = v.x; o = v.y; }
@@ -49,6 +50,9 @@ __device__ __forceinline__ unsigned join_cols(const unsigned short e, const unsi
 }
 __device__ __forceinline__ uint2 join_cols(const unsigned e, const unsigned o) {
     return make_uint2(__byte_perm(e, o, 0x5410), __byte_perm(e, o, 0x7632));
+}
+__device__ __forceinline__ uint4 join_cols(const uint2 e, const uint2 o) {
+    return make_uint4(__byte_perm(e.x, o.x, 0x5410), __byte_perm(e.x, o.x, 0x7632), __byte_perm(e.y, o.y, 0x5410), __byte_perm(e.y, o.y, 0x7632));
 }
 
 // X [planes][H][W] -> X' [b][phase][ci][H/2][W/2]. One thread per run of 2 NP neighbouring input columns (one aligned
@@ -80,30 +84,115 @@ __global__ void __launch_bounds__(256) phases_of_kernel(const T *__restrict__ X,
     }
 }
 
-// dX' [b][phase][ci][H/2][W/2] -> dX [b][ci][H][W], one thread per run of 2 NP neighbouring output columns;
-// phases = 1: only even rows and columns receive a value, the rest is zero.
+// X [planes][H][W] -> bf16 rows for the copy engine, [piece][b][phase * Cin + ci][pitch] (pitch >= H/2 * W/2, a multiple of
+// 8; what lies behind a plane is never read). A thread takes eight consecutive positions of one plane's rows of parity py
+// and writes both column parities' rows (phases = 4; phases = 1: the even rows and columns only). fp32 values leave as two
+// pieces (rounded, and the remainder rounded). VEC: W/2 is a multiple of four, so four positions are one or two vectors.
+// beside: see rows_job_kernel (nsd_kernels.cu).
+template <typename T, bool VEC>
+__global__ void __launch_bounds__(256) phase_rows_kernel(const T *__restrict__ X, unsigned short *__restrict__ out, unsigned planes,
+                                                         unsigned Cin, unsigned H, unsigned W, unsigned pitch, int phases, int beside) {
+    if (!beside) chain_wait();
+    chain_release();
+    const unsigned Ho = H / 2, Wo = W / 2, HW = Ho * Wo, gpp = pitch / 8, npy = phases == 1 ? 1 : 2;
+    const unsigned n = planes * npy * gpp;
+    const size_t phase_stride = static_cast<size_t>(Cin) * pitch;
+    const size_t piece = static_cast<size_t>(planes) * phases * pitch;
+    for (unsigned i = blockIdx.x * 256u + threadIdx.x; i < n; i += gridDim.x * 256u) {
+        const unsigned r = i / gpp, g = i - r * gpp, py = npy == 2 ? r & 1u : 0u, plane = npy == 2 ? r >> 1 : r;
+        const unsigned b = plane / Cin, ci = plane - b * Cin, p0 = g * 8;
+        const T *src = X + static_cast<size_t>(plane) * H * W + py * W;      // row py of the plane; row 2 y + py is 2 y W further
+        float e[8], o[8];
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            const unsigned p4 = p0 + 4 * h;
+            if (VEC) {
+                const unsigned y = p4 / Wo, x = p4 - y * Wo;
+                float v[8] = {};
+                if (p4 < HW) {
+                    const T *q = src + static_cast<size_t>(2 * y) * W + 2 * x;
+                    if (sizeof(T) == 4) {
+                        const float4 a = __ldg(reinterpret_cast<const float4 *>(q)), c = __ldg(reinterpret_cast<const float4 *>(q) + 1);
+                        v[0] = a.x; v[1] = a.y; v[2] = a.z; v[3] = a.w; v[4] = c.x; v[5] = c.y; v[6] = c.z; v[7] = c.w;
+                    } else {
+                        const uint4 a = __ldg(reinterpret_cast<const uint4 *>(q));
+                        const unsigned w[4] = {a.x, a.y, a.z, a.w};
+#pragma unroll
+                        for (int k = 0; k < 4; ++k) { v[2 * k] = __uint_as_float(w[k] << 16); v[2 * k + 1] = __uint_as_float(w[k] & 0xffff0000u); }
+                    }
+                }
+#pragma unroll
+                for (int k = 0; k < 4; ++k) { e[4 * h + k] = v[2 * k]; o[4 * h + k] = v[2 * k + 1]; }
+            } else {
+#pragma unroll
+                for (int k = 0; k < 4; ++k) {
+                    const unsigned pos = p4 + k, y = pos / Wo, x = pos - y * Wo;
+                    e[4 * h + k] = o[4 * h + k] = 0.f;
+                    if (pos < HW) {
+                        const T *q = src + static_cast<size_t>(2 * y) * W + 2 * x;
+                        if (sizeof(T) == 4) {
+                            const float2 a = __ldg(reinterpret_cast<const float2 *>(q));
+                            e[4 * h + k] = a.x; o[4 * h + k] = a.y;
+                        } else {
+                            const unsigned a = __ldg(reinterpret_cast<const unsigned *>(q));
+                            e[4 * h + k] = __uint_as_float(a << 16); o[4 * h + k] = __uint_as_float(a & 0xffff0000u);
+                        }
+                    }
+                }
+            }
+        }
+        unsigned short *dst = out + (static_cast<size_t>(b) * phases + (phases == 1 ? 0u : py * 2)) * phase_stride +
+                              static_cast<size_t>(ci) * pitch + p0;
+#pragma unroll
+        for (int px = 0; px < 2; ++px) {
+            if (px == 1 && phases == 1) break;
+            const float *v = px ? o : e;
+            unsigned hi[4], lo[4];
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                const __nv_bfloat162 hh = __floats2bfloat162_rn(v[2 * k], v[2 * k + 1]);
+                hi[k] = *reinterpret_cast<const unsigned *>(&hh);
+                if (sizeof(T) == 4) {
+                    const float2 hf = __bfloat1622float2(hh);
+                    const __nv_bfloat162 ll = __floats2bfloat162_rn(v[2 * k] - hf.x, v[2 * k + 1] - hf.y);
+                    lo[k] = *reinterpret_cast<const unsigned *>(&ll);
+                }
+            }
+            *reinterpret_cast<uint4 *>(dst + px * phase_stride) = make_uint4(hi[0], hi[1], hi[2], hi[3]);
+            if (sizeof(T) == 4) *reinterpret_cast<uint4 *>(dst + px * phase_stride + piece) = make_uint4(lo[0], lo[1], lo[2], lo[3]);
+        }
+    }
+    if (beside) chain_wait();
+}
+
+// dX' [b][phase][ci][H/2][W/2] -> dX [b][ci][H][W]: one thread per run of 2 NP neighbouring output columns of a pair of rows
+// (the rows of both parities); phases = 1: only even rows and columns receive a value, the rest is zero.
 template <typename T, int NP>
 __global__ void __launch_bounds__(256) from_phases_kernel(const T *__restrict__ dXp, T *__restrict__ dX, unsigned planes,
                                                           unsigned Cin, unsigned H, unsigned W, int phases) {
     using V = typename Cols<T, NP>::vec;
     using Hf = typename Cols<T, NP>::half;
+    chain_wait();
+    chain_release();
     const unsigned Ho = H / 2, Wo = W / 2, Wq = Wo / NP;
-    const unsigned n = planes * H * Wq;
+    const unsigned n = planes * Ho * Wq;
     const size_t phase_stride = static_cast<size_t>(Cin) * Ho * Wo;
     for (unsigned i = blockIdx.x * 256u + threadIdx.x; i < n; i += gridDim.x * 256u) {
         const unsigned r = i / Wq, xq = i - r * Wq;
-        const unsigned plane = r / H, y = r - plane * H;
+        const unsigned plane = r / Ho, yo = r - plane * Ho;
         const unsigned b = plane / Cin, ci = plane - b * Cin;
-        const unsigned py = y & 1, yo = y >> 1;
-        Hf e = Hf(), o = Hf();                                     // zero bits are zero values in both types
+        Hf v[4] = {};                                                  // [py][px]; zero bits are zero values in both types
+        const size_t in = static_cast<size_t>(yo) * Wo + NP * xq;
         if (phases != 1) {
-            const T *src = dXp + ((static_cast<size_t>(b) * 4 + py * 2) * Cin + ci) * Ho * Wo + static_cast<size_t>(yo) * Wo + NP * xq;
-            e = *reinterpret_cast<const Hf *>(src);
-            o = *reinterpret_cast<const Hf *>(src + phase_stride);
-        } else if (py == 0) {
-            e = *reinterpret_cast<const Hf *>(dXp + (static_cast<size_t>(plane) * Ho + yo) * Wo + NP * xq);
+            const T *src = dXp + (static_cast<size_t>(b) * 4 * Cin + ci) * Ho * Wo + in;
+#pragma unroll
+            for (int ph = 0; ph < 4; ++ph) v[ph] = *reinterpret_cast<const Hf *>(src + ph * phase_stride);
+        } else {
+            v[0] = *reinterpret_cast<const Hf *>(dXp + static_cast<size_t>(plane) * Ho * Wo + in);
         }
-        *reinterpret_cast<V *>(dX + (static_cast<size_t>(plane) * H + y) * W + 2 * NP * xq) = join_cols(e, o);
+        T *dst = dX + (static_cast<size_t>(plane) * H + 2 * yo) * W + 2 * NP * xq;
+        *reinterpret_cast<V *>(dst) = join_cols(v[0], v[1]);
+        *reinterpret_cast<V *>(dst + W) = join_cols(v[2], v[3]);
     }
 }
 
@@ -169,25 +258,40 @@ int launch_phases_of(dbp_ctx *ctx, const void *X, void *Xp, int io, long long B,
     return cuda_ok(cudaGetLastError());
 }
 
+int launch_phase_rows(dbp_ctx *ctx, const void *X, void *Xp, int io, long long B, long long Cin, int H, int W, int phases,
+                      long long pitch, bool beside) {
+    const long long n = B * Cin * (phases == 1 ? 1 : 2) * (pitch / 8);
+    if (!fits32(n) || !fits32(B * Cin)) return DBP_EUNSUPPORTED;
+    const int g = blocks_of(n, 256, ctx->sm_count * 8);
+    const bool vec = (W / 2) % 4 == 0;
+    auto go = [&](auto kern, auto x) {
+        return cuda_ok(launch_chained(kern, dim3(g), dim3(256), 0, ctx->stream, x, static_cast<unsigned short *>(Xp), static_cast<unsigned>(B * Cin),
+                                      static_cast<unsigned>(Cin), static_cast<unsigned>(H), static_cast<unsigned>(W),
+                                      static_cast<unsigned>(pitch), phases, beside ? 1 : 0));
+    };
+    const float *xf = static_cast<const float *>(X);
+    const __nv_bfloat16 *xb = static_cast<const __nv_bfloat16 *>(X);
+    if (io == DBP_F32) return vec ? go(phase_rows_kernel<float, true>, xf) : go(phase_rows_kernel<float, false>, xf);
+    return vec ? go(phase_rows_kernel<__nv_bfloat16, true>, xb) : go(phase_rows_kernel<__nv_bfloat16, false>, xb);
+}
+
 int launch_from_phases(dbp_ctx *ctx, const void *dXp, void *dX, int f32, long long B, long long Cin, int H, int W, int phases) {
-    const int np = W % 4 == 0 ? 2 : 1;
-    const long long n = B * Cin * H * (W / 2 / np);
     if (!fits32(B * Cin * H * (W / 2))) return DBP_EUNSUPPORTED;
-    const int g = blocks_of(n, 256, ctx->sm_count * 16);
-    const unsigned planes = static_cast<unsigned>(B * Cin), c = static_cast<unsigned>(Cin), h = H, w = W;
-    note_launch();
+    const int np = W % 8 == 0 && !f32 ? 4 : W % 4 == 0 ? 2 : 1;
+    const int g = blocks_of(B * Cin * (H / 2) * (W / 2 / np), 256, ctx->sm_count * 16);
+    auto go = [&](auto kern, auto in, auto out) {
+        return cuda_ok(launch_chained(kern, dim3(g), dim3(256), 0, ctx->stream, in, out, static_cast<unsigned>(B * Cin),
+                                      static_cast<unsigned>(Cin), static_cast<unsigned>(H), static_cast<unsigned>(W), phases));
+    };
     if (f32) {
         const float *in = static_cast<const float *>(dXp);
         float *out = static_cast<float *>(dX);
-        if (np == 2) from_phases_kernel<float, 2><<<g, 256, 0, ctx->stream>>>(in, out, planes, c, h, w, phases);
-        else from_phases_kernel<float, 1><<<g, 256, 0, ctx->stream>>>(in, out, planes, c, h, w, phases);
-    } else {
-        const __nv_bfloat16 *in = static_cast<const __nv_bfloat16 *>(dXp);
-        __nv_bfloat16 *out = static_cast<__nv_bfloat16 *>(dX);
-        if (np == 2) from_phases_kernel<__nv_bfloat16, 2><<<g, 256, 0, ctx->stream>>>(in, out, planes, c, h, w, phases);
-        else from_phases_kernel<__nv_bfloat16, 1><<<g, 256, 0, ctx->stream>>>(in, out, planes, c, h, w, phases);
+        return np == 2 ? go(from_phases_kernel<float, 2>, in, out) : go(from_phases_kernel<float, 1>, in, out);
     }
-    return cuda_ok(cudaGetLastError());
+    const __nv_bfloat16 *in = static_cast<const __nv_bfloat16 *>(dXp);
+    __nv_bfloat16 *out = static_cast<__nv_bfloat16 *>(dX);
+    return np == 4 ? go(from_phases_kernel<__nv_bfloat16, 4>, in, out) : np == 2 ? go(from_phases_kernel<__nv_bfloat16, 2>, in, out)
+                                                                                 : go(from_phases_kernel<__nv_bfloat16, 1>, in, out);
 }
 
 int launch_phase_weights(dbp_ctx *ctx, const void *W, void *Wp, int io, long long Cout, long long Cin) {

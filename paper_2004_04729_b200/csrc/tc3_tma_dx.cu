@@ -13,7 +13,7 @@
 // two columns per image row that belong to the halo (x = W, W+1) are computed and thrown away.
 // Small images (the whole image in one patch) are taken several at a time along the same row space.
 //
-//   A = weights of one tap [64 co][128 ci]  (M = input channels, MN-major; from W re-laid as [co][tap][ci])
+//   A = weights of one tap [64 co][128 ci]  (M = input channels, MN-major; from W re-laid as [tap][co][ci])
 //   B = code patch         [rows][64 co]    (N = up to 256 patch positions, K-major)
 //   K = (64-channel block of co) x (nine taps), four MMAs of 16 channels each
 //
@@ -56,7 +56,7 @@ struct Dx3T {
     int ntaps;                    // 9, or 18 for fp32 weights split into two bf16 pieces (taps 9-17: the low pieces)
     int es;                       // bytes per element of dX (2 or 4)
     int G;                        // taps per weight slot (one hand-over): 9, 3 or 1
-    int w_slot;                   // bytes of a weight slot: G * a_panels * 8 KB
+    int w_slot;                   // bytes of a weight slot, [panel][tap][64 co][64 ci]: a_panels * G * 8 KB
     int nq, nw;                   // ring sizes
     int resident;                 // the weights of all taps and co blocks stay in shared memory (one ci block)
     int run;                      // Ht * W: staged positions per image
@@ -167,7 +167,6 @@ tc3_tma_dx_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
             int s = 0;
             unsigned parity = 1;
             bool ok = true;
-            const unsigned w_tx = static_cast<unsigned>(p.w_slot);
             long long waited = 0;
             for (long long t = blockIdx.x; t < p.ntiles && ok; t += gridDim.x) {
                 int ci0, b0, y0;
@@ -178,12 +177,27 @@ tc3_tma_dx_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
                             ok = mbar_wait_timed(&pipe.w_empty[s], parity, p.err_flag, waited);
                             if (!ok) break;
                         }
-                        mbar_expect_tx(&pipe.w_full[s], w_tx);
-                        // one arrival for the whole slot: the taps' panels are separate copies under one barrier
+                        // One arrival for the whole slot, one copy per panel (all taps of the slot in one box). In phase mode
+                        // taps that carry no weights in this channel tile are neither copied nor multiplied: a quarter of
+                        // the layer's weights is what there is to copy then, tap by tap.
                         unsigned char *dst = w_s + s * p.w_slot;
-                        for (int gg = 0; gg < p.G; ++gg)
-                            for (int h = 0; h < p.a_panels; ++h, dst += kWPanel)
-                                tma_load_3d(dst, &map_w, ci0 + 64 * h, g * p.G + gg, c * 64, &pipe.w_full[s]);
+                        if (p.phase_cin == 0) {
+                            mbar_expect_tx(&pipe.w_full[s], static_cast<unsigned>(p.w_slot));
+                            for (int h = 0; h < p.a_panels; ++h)
+                                tma_load_3d(dst + h * p.G * kWPanel, &map_w, ci0 + 64 * h, c * 64, g * p.G, &pipe.w_full[s]);
+                        } else {
+                            const int ph = ci0 / p.phase_cin, ly = (ph & 2) ? 3 : 2, lx = (ph & 1) ? 3 : 2;
+                            unsigned live = 0;
+                            for (int gg = 0; gg < p.G; ++gg) {
+                                const int t9 = (g * p.G + gg) % 9;
+                                if (((ly >> (t9 / 3)) & 1) && ((lx >> (t9 % 3)) & 1)) live |= 1u << gg;
+                            }
+                            mbar_expect_tx(&pipe.w_full[s], static_cast<unsigned>(__popc(live) * p.a_panels * kWPanel));
+                            for (int gg = 0; gg < p.G; ++gg, dst += kWPanel)
+                                if ((live >> gg) & 1u)
+                                    for (int h = 0; h < p.a_panels; ++h)
+                                        tma_load_3d(dst + h * p.G * kWPanel, &map_w, ci0 + 64 * h, c * 64, g * p.G + gg, &pipe.w_full[s]);
+                        }
                         if (++s == p.nw) { s = 0; parity ^= 1u; }
                     }
                 if (p.resident) break;             // one ci block: every tile uses the same weights (all slots are loaded now)
@@ -196,7 +210,7 @@ tc3_tma_dx_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
             // start row of tap (ky, kx) inside the patch is (2 - ky) Wp + (2 - kx); as a descriptor offset
             // (16-byte units, 8 per row) it starts at tap_first and moves by -8, -8, +16 - 8 Wp, ...
             const int tap_first = (2 * p.Wp + 2) * 8, tap_wrap = (2 - p.Wp) * 8;
-            const unsigned a_tap = static_cast<unsigned>(p.a_panels * kWPanel) >> 4;     // one tap further inside a slot
+            const unsigned a_tap = static_cast<unsigned>(kWPanel) >> 4;                  // one tap further inside a slot
             int qs = 0, ws = 0;
             unsigned qpar = 0, wpar = 0;
             bool ok = true;
@@ -230,7 +244,7 @@ tc3_tma_dx_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
                         tc_fence_after();
                         // with one panel of ci (Cin <= 64) the upper 64 rows of the MMA re-read the same panel (their
                         // results are never stored) instead of whatever follows the slot
-                        unsigned long long ad = make_desc(smem_u32(w_s + ws * p.w_slot), p.a_panels == 2 ? kWPanel : 0, 1024);
+                        unsigned long long ad = make_desc(smem_u32(w_s + ws * p.w_slot), p.a_panels == 2 ? p.G * kWPanel : 0, 1024);
                         for (int gg = 0; gg < p.G; ++gg, ad += a_tap) {
                             const unsigned long long bd = bd0 + static_cast<unsigned>(toff);
                             const bool live = ((live_y >> ky) & 1) && ((live_x >> kx) & 1);
@@ -285,7 +299,7 @@ tc3_tma_dx_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
             ok = epilogue_all(mbar_wait_timed(&pipe.acc_full[slot], uses & 1u, p.err_flag, we));
             if (!ok) break;                                          // the same decision in every epilogue thread
             tc_fence_after();
-            const int ci_l = q * 32 + lane, ci = ci0 + ci_l;
+            const int ci_l = q * 32 + lane;
             const int rows_valid = p.H - y0 < p.Ht ? p.H - y0 : p.Ht;
             // ---- phase A: accumulator -> staging block (rows of bf16 or fp32 values per channel)
             if (ci0 + q * 32 < p.Cin) {                              // warp-uniform: some of my 32 channels exist
@@ -360,8 +374,8 @@ tc3_tma_dx_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
     }
 }
 
-// weights [Cout][Cin][3][3] -> [Cout][9][pitch] bf16 (the tap's [co][ci] matrix with ci contiguous, the row pitch a
-// multiple of 8). fp32 weights -> [Cout][18][pitch]: taps 0-8 hold the values rounded to bf16, taps 9-17 what that
+// weights [Cout][Cin][3][3] -> [9][Cout][pitch] bf16 (the tap's [co][ci] matrix with ci contiguous, the row pitch a
+// multiple of 8). fp32 weights -> [18][Cout][pitch]: taps 0-8 hold the values rounded to bf16, taps 9-17 what that
 // rounding left over, rounded to bf16 again. The sum of the two pieces differs from the fp32 value by at most 2^-18 of
 // it, and a code times a piece is exact in the fp32 accumulator. Used when the step size is given; otherwise the
 // statistics kernel does this on the side.
@@ -376,8 +390,8 @@ w_taps_rows_kernel(const T *__restrict__ W, __nv_bfloat16 *__restrict__ out, lon
         const long long ci = i % Cin, t = (i / Cin) % 9, co = i / (Cin * 9);
         const float w = static_cast<float>(W[(co * Cin + ci) * 9 + t]);
         const __nv_bfloat16 hi = __float2bfloat16_rn(w);
-        out[(co * TAPS + t) * pitch + ci] = hi;
-        if (TAPS == 18) out[(co * TAPS + 9 + t) * pitch + ci] = __float2bfloat16_rn(w - __bfloat162float(hi));
+        out[(t * Cout + co) * pitch + ci] = hi;
+        if (TAPS == 18) out[((9 + t) * Cout + co) * pitch + ci] = __float2bfloat16_rn(w - __bfloat162float(hi));
     }
 }
 
@@ -499,11 +513,11 @@ int launch_tc3_tma_dx(dbp_ctx *ctx, const void *codes_nhwc, const void *W, int i
         if (!encode_map_bf16(&map_q, codes_nhwc, 4, dims, str, box)) return fail_cuda("tensor map of the code patches");
     }
     {
-        const unsigned long long dims[3] = {static_cast<unsigned long long>(s.Cin), static_cast<unsigned long long>(p.ntaps),
-                                            static_cast<unsigned long long>(s.Cout)};
+        const unsigned long long dims[3] = {static_cast<unsigned long long>(s.Cin), static_cast<unsigned long long>(s.Cout),
+                                            static_cast<unsigned long long>(p.ntaps)};
         const unsigned long long str[2] = {static_cast<unsigned long long>(w_pitch) * 2,
-                                           static_cast<unsigned long long>(w_pitch) * 2 * p.ntaps};
-        const unsigned box[3] = {64, 1, 64};
+                                           static_cast<unsigned long long>(w_pitch) * 2 * s.Cout};
+        const unsigned box[3] = {64, 64, static_cast<unsigned>(p.phase_cin > 0 ? 1 : p.G)};
         if (!encode_map_bf16(&map_w, ctx->w_taps.ptr, 3, dims, str, box)) return fail_cuda("tensor map of the weights");
     }
     if (cudaFuncSetAttribute(tc3_tma_dx_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem)) != cudaSuccess)
