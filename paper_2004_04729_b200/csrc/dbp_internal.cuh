@@ -342,18 +342,20 @@ inline cudaError_t launch_chained(void (*kern)(KArgs...), dim3 grid, dim3 block,
     note_launch();
     return cudaLaunchKernelEx(&cfg, kern, static_cast<KArgs>(args)...);
 }
-// The same for a grid that is one cluster of `ctas` blocks.
+// The same for a grid of clusters of `cluster` consecutive blocks.
 template <typename... KArgs, typename... Args>
-inline cudaError_t launch_chained_cluster(void (*kern)(KArgs...), unsigned ctas, dim3 block, cudaStream_t stream, Args... args) {
+inline cudaError_t launch_chained_cluster(void (*kern)(KArgs...), unsigned ctas, unsigned cluster, dim3 block, size_t smem,
+                                          cudaStream_t stream, Args... args) {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(ctas);
     cfg.blockDim = block;
+    cfg.dynamicSmemBytes = smem;
     cfg.stream = stream;
     cudaLaunchAttribute attr[2];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     attr[1].id = cudaLaunchAttributeClusterDimension;
-    attr[1].val.clusterDim.x = ctas;
+    attr[1].val.clusterDim.x = cluster;
     attr[1].val.clusterDim.y = attr[1].val.clusterDim.z = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 2;

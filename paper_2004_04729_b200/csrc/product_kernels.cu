@@ -334,24 +334,45 @@ __global__ void __launch_bounds__(256) relu_backward_kernel(const float *__restr
     for (; i < n; i += stride) dz[i] = mask[i] ? da[i] : 0.f;
 }
 
-// Routing of a pooled gradient g [planes][h][w] to out [planes][2h][2w]: one thread per window, which writes
-// its four outputs (two pairs); argmax in {0,1,2,3} is the row-major position of the forward maximum
+// Routing of a pooled gradient g [planes][h][w] to out [planes][2h][2w]: a thread takes NW windows of one row (w % NW == 0)
+// and writes their two output rows; argmax in {0,1,2,3} is the row-major position of the forward maximum
+template <int NW>
 __global__ void __launch_bounds__(256) maxpool_backward_kernel(const float *__restrict__ g, const int8_t *__restrict__ am,
-                                                               float *__restrict__ out, long long planes, int h, int w) {
+                                                               float *__restrict__ out, long long n, int w) {
     chain_wait();
     chain_release();
-    const long long n = planes * h * w;
+    const int wq = w / NW;
     for (long long i = blockIdx.x * static_cast<long long>(blockDim.x) + threadIdx.x; i < n;
          i += static_cast<long long>(gridDim.x) * blockDim.x) {
-        const long long row = i / w;                    // (plane, y)
-        const int x = static_cast<int>(i - row * w);
-        const long long pl = row / h;
-        const int y = static_cast<int>(row - pl * h);
-        const float v = __ldg(g + i);
-        const int which = am[i];
-        float *o = out + ((pl * 2 * h + 2 * y) * 2ll * w + 2 * x);
-        *reinterpret_cast<float2 *>(o) = make_float2(which == 0 ? v : 0.f, which == 1 ? v : 0.f);
-        *reinterpret_cast<float2 *>(o + 2 * w) = make_float2(which == 2 ? v : 0.f, which == 3 ? v : 0.f);
+        // row (plane, y) starts at element row * w of g and row * 4 w of out
+        const long long row = (n >> 31) == 0 ? static_cast<unsigned>(i) / static_cast<unsigned>(wq) : i / wq;
+        const int x = static_cast<int>(i - row * wq) * NW;
+        float v[NW];
+        int8_t which[NW];
+        if (NW == 4) {
+            const float4 q = __ldcs(reinterpret_cast<const float4 *>(g + i * NW));
+            const char4 c = __ldg(reinterpret_cast<const char4 *>(am + i * NW));
+            const float qv[4] = {q.x, q.y, q.z, q.w};
+            const int8_t cv[4] = {c.x, c.y, c.z, c.w};
+#pragma unroll
+            for (int k = 0; k < NW; ++k) { v[k] = qv[k]; which[k] = cv[k]; }
+        } else {
+            v[0] = g[i];
+            which[0] = am[i];
+        }
+        float *o = out + row * 4ll * w + 2 * x;
+#pragma unroll
+        for (int half = 0; half < 2; ++half, o += 2 * w) {
+            if (NW == 4) {
+#pragma unroll
+                for (int k = 0; k + 1 < NW; k += 2)
+                    *reinterpret_cast<float4 *>(o + 2 * k) =
+                        make_float4(which[k] == 2 * half ? v[k] : 0.f, which[k] == 2 * half + 1 ? v[k] : 0.f,
+                                    which[k + 1] == 2 * half ? v[k + 1] : 0.f, which[k + 1] == 2 * half + 1 ? v[k + 1] : 0.f);
+            } else {
+                *reinterpret_cast<float2 *>(o) = make_float2(which[0] == 2 * half ? v[0] : 0.f, which[0] == 2 * half + 1 ? v[0] : 0.f);
+            }
+        }
     }
 }
 
@@ -505,8 +526,13 @@ int launch_relu_backward(dbp_ctx *ctx, const float *da, const uint8_t *mask, flo
 
 int launch_maxpool_backward(dbp_ctx *ctx, const float *g, const int8_t *argmax, float *out,
                             long long planes, long long h, long long w) {
-    return cuda_ok(launch_chained(maxpool_backward_kernel, dim3(blocks_for(planes * h * w, 256, ctx->sm_count * 8)), dim3(256), 0,
-                                  ctx->stream, g, argmax, out, planes, static_cast<int>(h), static_cast<int>(w)));
+    // four windows per thread where rows and pointers allow 16-byte accesses
+    const bool vec = w % 4 == 0 && ((reinterpret_cast<uintptr_t>(g) | reinterpret_cast<uintptr_t>(out)) & 15) == 0 &&
+                     (reinterpret_cast<uintptr_t>(argmax) & 3) == 0;
+    const long long n = planes * h * w / (vec ? 4 : 1);
+    return cuda_ok(launch_chained(vec ? maxpool_backward_kernel<4> : maxpool_backward_kernel<1>,
+                                  dim3(blocks_for(n, 256, ctx->sm_count * 4)), dim3(256), 0, ctx->stream, g, argmax, out, n,
+                                  static_cast<int>(w)));
 }
 
 }  // namespace dbp

@@ -475,7 +475,7 @@ int launch_small_linear(dbp_ctx *ctx, const float *delta, const float *X, const 
     p.inv_numel = 1.0 / static_cast<double>(n);
     auto kern = per <= 1 ? small_linear_quantize_kernel<1> : per <= 2 ? small_linear_quantize_kernel<2>
               : per <= 5 ? small_linear_quantize_kernel<5> : small_linear_quantize_kernel<kMaxVec>;
-    if (int rc = cuda_ok(launch_chained_cluster(kern, static_cast<unsigned>(ctas), dim3(kThreads), ctx->stream, p))) return rc;
+    if (int rc = cuda_ok(launch_chained_cluster(kern, static_cast<unsigned>(ctas), static_cast<unsigned>(ctas), dim3(kThreads), 0, ctx->stream, p))) return rc;
     const long long red = (dW && (!dX || B > N)) ? B : N;               // the longest reduction of the tiles
     const long long chunks = (red + kRed - 1) / kRed;
     const int most = p.n_dw + p.n_dx > ctx->sm_count ? kMaxChunks / 2 : kMaxChunks;      // two CTAs per SM when there are more tiles

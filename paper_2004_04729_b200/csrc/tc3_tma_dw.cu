@@ -121,7 +121,6 @@ tc3_tma_dw_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
     tc_fence_after();
     const unsigned tmem_base = pipe.tmem_base;
     chain_wait();        // from here on the kernel reads what earlier kernels wrote
-    chain_release();
 
     // segment g: image, first position, number of 64-position stages
     auto seg_of = [&](long long g, int &b, int &u0, int &ns) {
@@ -227,17 +226,24 @@ tc3_tma_dw_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
                     const int nk = left >= 64 ? 4 : (left + 15) >> 4;
                     const unsigned long long ad = make_desc(smem_u32(x_s + slot * kXSlot + j * kXTile), 16, 1024);
                     const unsigned radv = static_cast<unsigned>(64 * k * 8);
-                    if (elect_one())
-                    for (int kk = 0; kk < nk; ++kk) {
+                    auto slice = [&](int kk, unsigned on) {
                         const unsigned adv = radv + kk * 128;                 // 16 rows = 2048 bytes
                         if (NP == 2) {
-                            if (live_lo == 0) mma_bf16(tmem_base, ad + 2 * kk, bA + adv, idesc128, acc_on);
-                            mma_bf16(tmem_base + 128, ad + 2 * kk, bB + adv, idesc128, acc_on);
-                            if (live_hi == 3) mma_bf16(tmem_base + 256, ad + 2 * kk, bC + adv, idesc128, acc_on);
+                            if (live_lo == 0) mma_bf16(tmem_base, ad + 2 * kk, bA + adv, idesc128, on);
+                            mma_bf16(tmem_base + 128, ad + 2 * kk, bB + adv, idesc128, on);
+                            if (live_hi == 3) mma_bf16(tmem_base + 256, ad + 2 * kk, bC + adv, idesc128, on);
                         } else {
-                            mma_bf16(tmem_base, ad + 2 * kk, bA + adv, idesc192, acc_on);
+                            mma_bf16(tmem_base, ad + 2 * kk, bA + adv, idesc192, on);
                         }
-                        acc_on = 1u;
+                    };
+                    if (elect_one()) {
+                        slice(0, acc_on);
+                        if (nk == 4) {
+#pragma unroll
+                            for (int kk = 1; kk < 4; ++kk) slice(kk, 1u);
+                        } else {
+                            for (int kk = 1; kk < nk; ++kk) slice(kk, 1u);
+                        }
                     }
                     acc_on = 1u;
                     ++j;
@@ -303,6 +309,9 @@ tc3_tma_dw_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
             ok = r != 0;
         }
         if (ok) {
+            // the finish kernel may come now, not earlier: its blocks would hold thread slots that the kernels of the other
+            // stream want (VGG-16 layer set: 1033 against 989 us)
+            chain_release();
             tc_fence_after();
             const long long t_epi = clock64();
             const int nchunks = c_hi;                  // only the rows the layer wants are handed over
@@ -428,27 +437,38 @@ tc3_dw_finish_phases_kernel(float *__restrict__ acc, const float *__restrict__ d
 // [2][B / G][Cin][pitch] with G (H + 1) W positions per tall image; position q of tall image t is position
 // q % ((H + 1) W) of image t G + q / ((H + 1) W), or zero in the extra row and in the padding.
 // beside: see rows_job_kernel (nsd_kernels.cu).
+// A thread takes eight consecutive positions of one tall image's row: index arithmetic in 32 bits, one division per row and
+// then step and wrap, one 16-byte store per piece (the previous form, a position per thread with 64-bit divisions, took 25 to
+// 50 us beside a dX kernel at 512 channels of 4x4; the data are 4 MB).
 __global__ void __launch_bounds__(256)
-x_split_stacked_kernel(const float *__restrict__ X, __nv_bfloat16 *__restrict__ out, long long Bt, int G, int Cin,
-                       int HW, int W, int pitch, int beside) {
+x_split_stacked_kernel(const float *__restrict__ X, __nv_bfloat16 *__restrict__ out, unsigned Bt, unsigned G, unsigned Cin,
+                       unsigned HW, unsigned W, unsigned pitch, int beside) {
     if (!beside) chain_wait();
     chain_release();
-    const long long n = Bt * Cin * pitch;
-    const int per_img = HW + W;
-    for (long long i = blockIdx.x * 256ll + threadIdx.x; i < n; i += gridDim.x * 256ll) {
-        const long long pl = i / pitch;
-        const int q = static_cast<int>(i - pl * pitch);
-        const long long t = pl / Cin;
-        const int ci = static_cast<int>(pl - t * Cin);
-        const int g = q / per_img, r = q - g * per_img;
-        __nv_bfloat16 hi = __float2bfloat16_rn(0.f), lo = hi;
-        if (g < G && r < HW) {
-            const float x = __ldg(X + ((t * G + g) * Cin + ci) * HW + r);
-            hi = __float2bfloat16_rn(x);
-            lo = __float2bfloat16_rn(x - __bfloat162float(hi));
+    const unsigned gpp = pitch / 8, per_img = HW + W, n = Bt * Cin * gpp;
+    const size_t piece = static_cast<size_t>(Bt) * Cin * pitch, img_stride = static_cast<size_t>(Cin) * HW;
+    for (unsigned i = blockIdx.x * 256u + threadIdx.x; i < n; i += gridDim.x * 256u) {
+        const unsigned pl = i / gpp, q0 = (i - pl * gpp) * 8, t = pl / Cin, ci = pl - t * Cin;
+        unsigned g = q0 / per_img, r = q0 - g * per_img;
+        const float *src = X + (static_cast<size_t>(t) * G + g) * img_stride + static_cast<size_t>(ci) * HW;
+        float x[8];
+#pragma unroll
+        for (int e = 0; e < 8; ++e) {
+            x[e] = (g < G && r < HW) ? __ldg(src + r) : 0.f;
+            if (++r == per_img) { r = 0; ++g; src += img_stride; }
         }
-        out[i] = hi;
-        out[n + i] = lo;
+        unsigned h[4], l[4];
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            const __nv_bfloat162 hh = __floats2bfloat162_rn(x[2 * k], x[2 * k + 1]);
+            const float2 hf = __bfloat1622float2(hh);
+            const __nv_bfloat162 ll = __floats2bfloat162_rn(x[2 * k] - hf.x, x[2 * k + 1] - hf.y);
+            h[k] = *reinterpret_cast<const unsigned *>(&hh);
+            l[k] = *reinterpret_cast<const unsigned *>(&ll);
+        }
+        const size_t o = static_cast<size_t>(pl) * pitch + q0;
+        *reinterpret_cast<uint4 *>(out + o) = make_uint4(h[0], h[1], h[2], h[3]);
+        *reinterpret_cast<uint4 *>(out + piece + o) = make_uint4(l[0], l[1], l[2], l[3]);
     }
     if (beside) chain_wait();
 }
@@ -461,6 +481,7 @@ int round_up(int v, int m) { return (v + m - 1) / m * m; }
 int tc3_stack_images(const ConvShape &s, int io) {
     const long long HW = s.H * s.W, per_img = HW + s.W;
     if (io != DBP_F32 || s.k != 3 || HW >= 64 || per_img > 64 || s.B < 2 || s.Cout % 8 != 0) return 0;
+    if (s.B * s.Cin * per_img >= (1ll << 31)) return 0;          // the stacking kernel indexes in 32 bits
     // the largest divisor of the batch whose tall image stays within one segment of the kernel
     for (long long g = s.B; g >= 2; --g)
         if (s.B % g == 0 && g * per_img <= 320) return static_cast<int>(g);
@@ -469,11 +490,12 @@ int tc3_stack_images(const ConvShape &s, int io) {
 
 int launch_x_stacked(dbp_ctx *ctx, const float *X, void *out, const ConvShape &s, int stack_g, bool beside) {
     const long long tall = s.B / stack_g, pitch = (stack_g * (s.H + 1) * s.W + 7) / 8 * 8;
-    long long blocks = (tall * s.Cin * pitch + 255) / 256;
-    if (blocks > ctx->sm_count * 8) blocks = ctx->sm_count * 8;
+    long long blocks = (tall * s.Cin * (pitch / 8) + 255) / 256;
+    if (blocks > ctx->sm_count * 4) blocks = ctx->sm_count * 4;
     return cuda_ok(launch_chained(x_split_stacked_kernel, dim3(static_cast<unsigned>(blocks)), dim3(256), 0, ctx->stream, X,
-                                  static_cast<__nv_bfloat16 *>(out), tall, stack_g, static_cast<int>(s.Cin), static_cast<int>(s.H * s.W),
-                                  static_cast<int>(s.W), static_cast<int>(pitch), beside ? 1 : 0));
+                                  static_cast<__nv_bfloat16 *>(out), static_cast<unsigned>(tall), static_cast<unsigned>(stack_g),
+                                  static_cast<unsigned>(s.Cin), static_cast<unsigned>(s.H * s.W), static_cast<unsigned>(s.W),
+                                  static_cast<unsigned>(pitch), beside ? 1 : 0));
 }
 
 // X: bf16 planes of x_pitch values (a multiple of 8); fp32 activations as two pieces (as if the batch were twice as long).

@@ -3,23 +3,32 @@
 //   dX[b][ci][y][x] = Delta * sum_(co,ky,kx) q[b][co][y+1-ky][x+1-kx] * W[co][ci][ky][kx]
 //
 // The quantizer has written the codes position-major, [b][y][x][co] in bf16, so a patch of
-// (Ht+2) x (W+2) positions x 64 output channels is ONE 4-D tiled copy whose out-of-image rows and
+// (Ht+2) x Wp positions x 64 output channels is ONE 4-D tiled copy whose out-of-image rows and
 // columns the copy engine fills with zeros: the convolution's zero padding costs nothing. In
 // shared memory the patch is a K-major operand, one 128-byte row of 64 channels per position,
-// rows numbered r = yy * (W+2) + xx. The output position (y, x) of the patch is accumulator column
-// n = (y-y0) * (W+2) + x, and the code a tap (ky, kx) needs for it sits in row
-// n + (2-ky) * (W+2) + (2-kx): a tap is only a different start row of the same operand (the 128-byte
+// rows numbered r = yy * Wp + xx, xx = 0 being column -1. The output position (y, x) of the patch is
+// accumulator column n = (y-y0) * Wp + x, and the code a tap (ky, kx) needs for it sits in row
+// n + (2-ky) * Wp + (2-kx): a tap is only a different start row of the same operand (the 128-byte
 // swizzle is a function of the shared-memory address, so a descriptor may start at any row). The
-// two columns per image row that belong to the halo (x = W, W+1) are computed and thrown away.
-// Small images (the whole image in one patch) are taken several at a time along the same row space.
+// columns that belong to the halo are computed and thrown away, so halos are shared: Wp = W + 1 (the zero
+// right of a row is the zero left of the next one; bf16 rows of even W keep W + 2, which keeps pairs of
+// outputs on even columns), and small images, taken several at a time along the same row space, have
+// one row of zeros between them. What a tap reads behind the last row is zeroed once.
 //
 //   A = weights of one tap [64 co][128 ci]  (M = input channels, MN-major; from W re-laid as [tap][co][ci])
 //   B = code patch         [rows][64 co]    (N = up to 256 patch positions, K-major)
 //   K = (64-channel block of co) x (nine taps), four MMAs of 16 channels each
 //
+// An MMA of N columns takes max(N/2, 32 + N/4) clocks (measured; the second term is its operands' way out of shared
+// memory: 4 KB of A, 32 bytes per column of B), and streamed weights take shared-memory and L2 bandwidth on top. So N is
+// made large, and where that leaves fewer tiles than SMs the reduction over co is split over a cluster of KS CTAs, whose
+// partial sums are read through distributed shared memory and added in rank order (fixed: dX does not depend on timing).
+// fp32 layers of at most 64 input channels put the two pieces of their weights on the two halves of the accumulator's
+// lanes (9 taps instead of 18 with half-empty MMAs); the halves are added on the way out.
+//
 // A CTA is persistent over (patch, 128-channel block of ci) tiles. Warp 0 copies code patches,
-// warp 1 copies weight tiles, warp 2 issues the MMAs into one of two accumulators in tensor memory,
-// warps 4-19 drain the other one: scale by Delta, convert, compact the valid columns into a
+// warp 1 copies weight tiles, warps 2 and 3 issue the MMAs of alternate tiles into two accumulators in tensor
+// memory, warps 4-19 drain them: scale by Delta, convert, compact the valid columns into a
 // shared staging block [ci][positions] and write whole runs of consecutive positions per channel.
 // Every wait is bounded.
 #include "tc_common.cuh"
@@ -30,7 +39,7 @@ namespace {
 
 using namespace tc;
 
-constexpr int kThreadsX = 20 * 32;               // copy, copy, MMA, spare, sixteen epilogue warps
+constexpr int kThreadsX = 20 * 32;               // copy, copy, MMA, MMA, sixteen epilogue warps
 constexpr int kWPanel = 8192;                    // [64 co][64 ci] bf16
 constexpr int kMaxQ = 2;                         // code patches in flight
 constexpr int kMaxW = 18;                        // weight slots (ring, or all of them when they stay resident)
@@ -42,10 +51,12 @@ struct Dx3T {
     void *dX;
     int dx_f32;
     int B, Cin, Cout, H, W, Wp;
+    int KS;                       // CTAs (a cluster) that share a tile's reduction; > 1: one tile per cluster
+    int split;                    // the low piece of the weights is the upper panel (fp32, Cin <= 64)
     int Ht;                       // image rows per patch
     int nb;                       // images per patch (> 1 only when Ht == H)
     int tiles_y;                  // patches per image (nb == 1)
-    int img_rows;                 // (Ht + 2) * Wp: patch rows per image
+    int img_rows;                 // patch rows per image: (Ht + 2) * Wp, or (H + 1) * Wp with several images
     int N;                        // accumulator columns in use (multiple of 16)
     int q_bytes;                  // bytes of one patch buffer (multiple of 1024)
     int q_tx;                     // bytes one patch copy delivers
@@ -55,7 +66,7 @@ struct Dx3T {
     int a_panels;                 // 64-channel panels of ci per weight tile (1 or 2)
     int ntaps;                    // 9, or 18 for fp32 weights split into two bf16 pieces (taps 9-17: the low pieces)
     int es;                       // bytes per element of dX (2 or 4)
-    int G;                        // taps per weight slot (one hand-over): 9, 3 or 1
+    int G;                        // taps per weight slot (one hand-over): 9, 3 or 1; phase mode: 2
     int w_slot;                   // bytes of a weight slot, [panel][tap][64 co][64 ci]: a_panels * G * 8 KB
     int nq, nw;                   // ring sizes
     int resident;                 // the weights of all taps and co blocks stay in shared memory (one ci block)
@@ -70,7 +81,7 @@ struct Dx3T {
 };
 
 struct PipeX {
-    unsigned long long q_full[kMaxQ], q_empty[kMaxQ], w_full[kMaxW], w_empty[kMaxW], acc_full[2], acc_empty[2];
+    unsigned long long q_full[kMaxQ], q_empty[kMaxQ], w_full[kMaxW], w_empty[kMaxW], acc_full[2], acc_empty[2], turn[2];
     unsigned tmem_base;
 };
 
@@ -79,6 +90,26 @@ __device__ __forceinline__ void tma_load_4d(void *dst, const CUtensorMap *map, i
     asm volatile(
         "cp.async.bulk.tensor.4d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4, %5, %6}], [%2];"
         ::"r"(smem_u32(dst)), "l"(map), "r"(smem_u32(bar)), "r"(c0), "r"(c1), "r"(c2), "r"(c3) : "memory");
+}
+
+// dst[0 .. n) = value(0 .. n), lanes along the run, four values per lane in flight
+template <typename T, typename F>
+__device__ __forceinline__ void copy_run(T *dst, int n, int lane, const F &value) {
+    for (int i0 = lane; i0 < n; i0 += 128) {
+        T v[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u)
+            if (i0 + 32 * u < n) v[u] = value(i0 + 32 * u);
+#pragma unroll
+        for (int u = 0; u < 4; ++u)
+            if (i0 + 32 * u < n) dst[i0 + 32 * u] = v[u];
+    }
+}
+
+// All threads of the cluster; writes to distributed shared memory before it are visible behind it.
+__device__ __forceinline__ void cluster_barrier() {
+    __syncwarp();
+    asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
 
 // Barrier over the epilogue threads that also tells every one of them whether all of them are
@@ -104,11 +135,14 @@ tc3_tma_dx_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
     unsigned char *stage = reinterpret_cast<unsigned char *>(s_off) + 512;   // [128 ci][pitch]
     __shared__ PipeX pipe;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int rank = p.KS > 1 ? static_cast<int>(blockIdx.x) % p.KS : 0;      // consecutive CTAs are a cluster
+    const long long t_first = blockIdx.x / p.KS, t_step = gridDim.x / p.KS;
+    const int c_lo = rank * p.ncb / p.KS, c_hi = (rank + 1) * p.ncb / p.KS;   // my 64-channel blocks of co
 
     if (threadIdx.x == 0) {
         for (int s = 0; s < kMaxQ; ++s) { mbar_init(&pipe.q_full[s], 1); mbar_init(&pipe.q_empty[s], 1); }
         for (int s = 0; s < kMaxW; ++s) { mbar_init(&pipe.w_full[s], 1); mbar_init(&pipe.w_empty[s], 1); }
-        for (int a = 0; a < 2; ++a) { mbar_init(&pipe.acc_full[a], 1); mbar_init(&pipe.acc_empty[a], kEpiThreads / 32); }
+        for (int a = 0; a < 2; ++a) { mbar_init(&pipe.turn[a], 1); mbar_init(&pipe.acc_full[a], 1); mbar_init(&pipe.acc_empty[a], kEpiThreads / 32); }
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         tma_prefetch_desc(&map_q);
         tma_prefetch_desc(&map_w);
@@ -121,13 +155,18 @@ tc3_tma_dx_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
         const int yy = rem / p.Wp, xx = rem - yy * p.Wp;
         s_off[n] = (n < p.N && img < p.nb && yy < p.Ht && xx < p.W) ? static_cast<short>(img * p.run + yy * p.W + xx) : static_cast<short>(-1);
     }
+    // the rows behind a patch: the last row's right-hand zero and the zeros below the last image; copies never reach them
+    for (int q = 0; q < p.nq; ++q)
+        for (int i = p.img_rows * p.nb * 8 + threadIdx.x; i < p.q_bytes / 16; i += kThreadsX)
+            reinterpret_cast<uint4 *>(q_s + q * p.q_bytes)[i] = make_uint4(0u, 0u, 0u, 0u);
+    fence_async_proxy();
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
     const unsigned tmem_base = pipe.tmem_base;
+    if (p.KS > 1) cluster_barrier();       // every CTA of the cluster is there before anybody writes into its staging block
     // everything above touched only this CTA's shared and tensor memory
     chain_wait();
-    chain_release();
 
     // tile t -> (patch, ci block); patch -> first image and first image row
     auto tile_of = [&](long long t, int &ci0, int &b0, int &y0) {
@@ -141,7 +180,10 @@ tc3_tma_dx_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
             y0 = 0;
         }
     };
-    const int slots_per_cb = p.ntaps / p.G;
+    // Weight slots per 64-channel block of co. In phase mode a slot is one kernel row's taps kx = 0, 1, and only rows that
+    // carry weights in the tile's phase have one: ky = 1 (py = 0), or ky = 0 and 1 (py = 1).
+    auto phase_of = [&](long long t) { return static_cast<int>(t % p.ci_tiles) * 128 / p.phase_cin; };
+    auto slots_of = [&](long long t) { return p.phase_cin == 0 ? p.ntaps / p.G : ((phase_of(t) & 2) ? 2 : 1) * (p.ntaps / 9); };
 
     if (warp == 0) {
         if (lane == 0) {
@@ -149,10 +191,10 @@ tc3_tma_dx_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
             unsigned parity = 1;                   // a fresh barrier passes a wait on the previous phase
             bool ok = true;
             long long waited = 0;
-            for (long long t = blockIdx.x; t < p.ntiles && ok; t += gridDim.x) {
+            for (long long t = t_first; t < p.ntiles && ok; t += t_step) {
                 int ci0, b0, y0;
                 tile_of(t, ci0, b0, y0);
-                for (int c = 0; c < p.ncb && ok; ++c) {
+                for (int c = c_lo; c < c_hi && ok; ++c) {
                     ok = mbar_wait_timed(&pipe.q_empty[s], parity, p.err_flag, waited);
                     if (!ok) break;
                     mbar_expect_tx(&pipe.q_full[s], static_cast<unsigned>(p.q_tx));
@@ -160,6 +202,8 @@ tc3_tma_dx_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
                     if (++s == p.nq) { s = 0; parity ^= 1u; }
                 }
             }
+            chain_release();       // every copy is issued: the next kernel may take the slots that come free (earlier it would
+                                   // hold thread slots that the dW stream's kernels want: stride-2 set 796 against 745 us)
             report_wait(p.stats, 3, waited);
         }
     } else if (warp == 1) {
@@ -168,35 +212,31 @@ tc3_tma_dx_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
             unsigned parity = 1;
             bool ok = true;
             long long waited = 0;
-            for (long long t = blockIdx.x; t < p.ntiles && ok; t += gridDim.x) {
+            for (long long t = t_first; t < p.ntiles && ok; t += t_step) {
                 int ci0, b0, y0;
                 tile_of(t, ci0, b0, y0);
-                for (int c = 0; c < p.ncb && ok; ++c)
-                    for (int g = 0; g < slots_per_cb; ++g) {
+                const int slots = slots_of(t);
+                for (int c = c_lo; c < c_hi && ok; ++c)
+                    for (int g = 0; g < slots; ++g) {
                         if (!p.resident) {
                             ok = mbar_wait_timed(&pipe.w_empty[s], parity, p.err_flag, waited);
                             if (!ok) break;
                         }
-                        // One arrival for the whole slot, one copy per panel (all taps of the slot in one box). In phase mode
-                        // taps that carry no weights in this channel tile are neither copied nor multiplied: a quarter of
-                        // the layer's weights is what there is to copy then, tap by tap.
+                        // One arrival for the whole slot, one copy per panel (all taps of the slot in one box; in phase mode
+                        // the live taps one by one: a quarter of the layer's weights is what there is to copy then).
                         unsigned char *dst = w_s + s * p.w_slot;
                         if (p.phase_cin == 0) {
                             mbar_expect_tx(&pipe.w_full[s], static_cast<unsigned>(p.w_slot));
                             for (int h = 0; h < p.a_panels; ++h)
-                                tma_load_3d(dst + h * p.G * kWPanel, &map_w, ci0 + 64 * h, c * 64, g * p.G, &pipe.w_full[s]);
+                                tma_load_3d(dst + h * p.G * kWPanel, &map_w, p.split ? 0 : ci0 + 64 * h, c * 64,
+                                            g * p.G + (p.split ? 9 * h : 0), &pipe.w_full[s]);
                         } else {
-                            const int ph = ci0 / p.phase_cin, ly = (ph & 2) ? 3 : 2, lx = (ph & 1) ? 3 : 2;
-                            unsigned live = 0;
-                            for (int gg = 0; gg < p.G; ++gg) {
-                                const int t9 = (g * p.G + gg) % 9;
-                                if (((ly >> (t9 / 3)) & 1) && ((lx >> (t9 % 3)) & 1)) live |= 1u << gg;
-                            }
-                            mbar_expect_tx(&pipe.w_full[s], static_cast<unsigned>(__popc(live) * p.a_panels * kWPanel));
-                            for (int gg = 0; gg < p.G; ++gg, dst += kWPanel)
-                                if ((live >> gg) & 1u)
-                                    for (int h = 0; h < p.a_panels; ++h)
-                                        tma_load_3d(dst + h * p.G * kWPanel, &map_w, ci0 + 64 * h, c * 64, g * p.G + gg, &pipe.w_full[s]);
+                            const int ph = phase_of(t), ky = (ph & 2) ? g & 1 : 1, kx0 = (ph & 1) ? 0 : 1;
+                            const int piece = (ph & 2) ? g >> 1 : g;
+                            mbar_expect_tx(&pipe.w_full[s], static_cast<unsigned>((2 - kx0) * 2 * kWPanel));
+                            for (int kx = kx0; kx < 2; ++kx)
+                                for (int h = 0; h < 2; ++h)
+                                    tma_load_3d(dst + (2 * h + kx) * kWPanel, &map_w, ci0 + 64 * h, c * 64, 9 * piece + ky * 3 + kx, &pipe.w_full[s]);
                         }
                         if (++s == p.nw) { s = 0; parity ^= 1u; }
                     }
@@ -204,81 +244,103 @@ tc3_tma_dx_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
             }
             report_wait(p.stats, 4, waited);
         }
-    } else if (warp == 2) {
-        {   // the whole warp runs the loop (uniform control flow and operands); one elected lane issues
-            const unsigned idesc = make_idesc(128, p.N, true, false);
-            // start row of tap (ky, kx) inside the patch is (2 - ky) Wp + (2 - kx); as a descriptor offset
-            // (16-byte units, 8 per row) it starts at tap_first and moves by -8, -8, +16 - 8 Wp, ...
-            const int tap_first = (2 * p.Wp + 2) * 8, tap_wrap = (2 - p.Wp) * 8;
-            const unsigned a_tap = static_cast<unsigned>(kWPanel) >> 4;                  // one tap further inside a slot
-            int qs = 0, ws = 0;
-            unsigned qpar = 0, wpar = 0;
-            bool ok = true;
-            long long it = 0;
-            long long wq = 0, ww = 0, wa = 0;
-            const long long born = clock64();
-            for (long long t = blockIdx.x; t < p.ntiles && ok; t += gridDim.x, ++it) {
-                const int slot = static_cast<int>(it & 1);
-                const unsigned uses = static_cast<unsigned>(it >> 1);
-                ok = __all_sync(0xffffffffu, mbar_wait_timed(&pipe.acc_empty[slot], (uses & 1u) ^ 1u, p.err_flag, wa));
+    } else if (warp < 4) {
+        // Two warps issue MMAs, each for every other tile (its own accumulator): what one does between tiles (waits,
+        // descriptors: more than a thousand clocks) then lies beside the other's MMAs. The whole warp runs the loop (uniform
+        // control flow and operands); one elected lane issues.
+        const unsigned idesc = make_idesc(128, p.N, true, false);
+        // Start row of tap (ky, kx) inside the patch is (2 - ky) Wp + (2 - kx), in descriptor units (16 bytes) eight times
+        // that; one tap further inside a slot is kWPanel. The three taps of a kernel row are issued by one elected lane
+        // from straight-line code (a loop with address stepping and an election per tap left the tensor pipe idle for long).
+        constexpr unsigned a_tap = static_cast<unsigned>(kWPanel) >> 4;
+        const unsigned row_step = static_cast<unsigned>(p.Wp * 8);
+        const unsigned long long q_desc = make_desc(smem_u32(q_s), 16, 1024);
+        // with one panel of ci (Cin <= 64) the upper 64 rows of the MMA re-read the same panel (their results are never
+        // stored) instead of whatever follows the slot
+        const unsigned long long w_desc = make_desc(smem_u32(w_s), p.a_panels == 2 ? p.G * kWPanel : 0, 1024);
+        const unsigned q_step = static_cast<unsigned>(p.q_bytes) >> 4, w_step = static_cast<unsigned>(p.w_slot) >> 4;
+        const int slot = warp - 2, ncbl = c_hi - c_lo;
+        const unsigned tmem_d = tmem_base + slot * kAccCols;
+        bool ok = true;
+        long long wq = 0, ww = 0, wa = 0;
+        const long long born = clock64();
+        int it = slot;
+        unsigned n_w = slot ? ncbl * slots_of(t_first) : 0;
+        for (long long t = t_first + slot * t_step; t < p.ntiles && ok; t += 2 * t_step, it += 2) {
+            // ring positions of this tile's first patch and weight slot (and, behind them, of this warp's next tile)
+            const unsigned n_q = static_cast<unsigned>(it) * ncbl;
+            const int slots = slots_of(t);
+            int qs = n_q % p.nq, ws = n_w % p.nw;
+            unsigned qpar = (n_q / p.nq) & 1u, wpar = (n_w / p.nw) & 1u;
+            if (p.resident) { ws = 0; wpar = 0; }          // completed barriers stay passable on parity 0
+            n_w += ncbl * (slots + slots_of(t + t_step));
+            unsigned acc_on = 0u;
+            const int ph = p.phase_cin > 0 ? phase_of(t) : 0;
+            ok = __all_sync(0xffffffffu, mbar_wait_timed(&pipe.acc_empty[slot], ((static_cast<unsigned>(it) >> 1) & 1u) ^ 1u, p.err_flag, wa));
+            // The rings' barriers may be waited for one phase ahead, not more: the other warp must have seen every stage of the
+            // tile before this one arrive. It says so in front of its last slot's MMAs, which is early enough.
+            if (ok && it > 0)
+                ok = __all_sync(0xffffffffu, mbar_wait(&pipe.turn[slot], ((static_cast<unsigned>(it - 1) >> 1)) & 1u, p.err_flag));
+            if (!ok) break;
+            for (int c = c_lo; c < c_hi && ok; ++c) {
+                ok = __all_sync(0xffffffffu, mbar_wait_timed(&pipe.q_full[qs], qpar, p.err_flag, wq));
                 if (!ok) break;
-                tc_fence_after();
-                const unsigned tmem_d = tmem_base + slot * kAccCols;
-                unsigned acc_on = 0u;
-                int live_y = 7, live_x = 7;                // bit t: taps with coordinate t carry non-zero weights
-                if (p.phase_cin > 0) {
-                    const int ph = static_cast<int>(t % p.ci_tiles) * 128 / p.phase_cin;
-                    live_y = (ph & 2) ? 3 : 2;
-                    live_x = (ph & 1) ? 3 : 2;
-                }
-                if (p.resident) { ws = 0; wpar = 0; }      // completed barriers stay passable on parity 0
-                for (int c = 0; c < p.ncb && ok; ++c) {
-                    ok = __all_sync(0xffffffffu, mbar_wait_timed(&pipe.q_full[qs], qpar, p.err_flag, wq));
+                const unsigned long long bd0 = q_desc + static_cast<unsigned>(qs) * q_step;
+                int ky = 0, kx1 = 0;                       // kernel row of the next slot (G >= 3), its tap (G == 1)
+                for (int g = 0; g < slots && ok; ++g) {
+                    ok = __all_sync(0xffffffffu, mbar_wait_timed(&pipe.w_full[ws], wpar, p.err_flag, ww));
                     if (!ok) break;
+                    if (c == c_hi - 1 && g == slots - 1 && elect_one()) mbar_arrive(&pipe.turn[slot ^ 1]);
                     tc_fence_after();
-                    const unsigned long long bd0 = make_desc(smem_u32(q_s + qs * p.q_bytes), 16, 1024);
-                    int toff = tap_first, kx = 0, ky = 0;
-                    for (int g = 0; g < slots_per_cb && ok; ++g) {
-                        ok = __all_sync(0xffffffffu, mbar_wait_timed(&pipe.w_full[ws], wpar, p.err_flag, ww));
-                        if (!ok) break;
-                        tc_fence_after();
-                        // with one panel of ci (Cin <= 64) the upper 64 rows of the MMA re-read the same panel (their
-                        // results are never stored) instead of whatever follows the slot
-                        unsigned long long ad = make_desc(smem_u32(w_s + ws * p.w_slot), p.a_panels == 2 ? p.G * kWPanel : 0, 1024);
-                        for (int gg = 0; gg < p.G; ++gg, ad += a_tap) {
-                            const unsigned long long bd = bd0 + static_cast<unsigned>(toff);
-                            const bool live = ((live_y >> ky) & 1) && ((live_x >> kx) & 1);
-                            if (kx == 2) {
-                                kx = 0;
-                                toff += tap_wrap;
-                                if (++ky == 3) { ky = 0; toff = tap_first; }      // the second piece's taps start over
-                            } else {
-                                ++kx;
-                                toff -= 8;
+                    unsigned long long ad = w_desc + static_cast<unsigned>(ws) * w_step;
+                    if (p.phase_cin > 0) {
+                        const unsigned long long bd = bd0 + (2 - ((ph & 2) ? g & 1 : 1)) * row_step;
+                        if (elect_one()) {
+                            if (ph & 1) {
+#pragma unroll
+                                for (int k = 0; k < 4; ++k) mma_bf16(tmem_d, ad + 128 * k, bd + 16 + 2 * k, idesc, k ? 1u : acc_on);
                             }
-                            if (!live) continue;
+#pragma unroll
+                            for (int k = 0; k < 4; ++k)
+                                mma_bf16(tmem_d, ad + a_tap + 128 * k, bd + 8 + 2 * k, idesc, (k || (ph & 1)) ? 1u : acc_on);
+                        }
+                        acc_on = 1u;
+                    } else if (p.G == 1) {
+                        const unsigned long long bd = bd0 + (2 - ky) * row_step + (2 - kx1) * 8;
+                        if (elect_one()) {
+#pragma unroll
+                            for (int k = 0; k < 4; ++k) mma_bf16(tmem_d, ad + 128 * k, bd + 2 * k, idesc, k ? 1u : acc_on);
+                        }
+                        acc_on = 1u;
+                        if (++kx1 == 3) { kx1 = 0; if (++ky == 3) ky = 0; }       // the second piece's taps start over
+                    } else {
+                        for (int r = 0; r < p.G; r += 3, ad += 3 * a_tap) {
+                            const unsigned long long bd = bd0 + (2 - ky) * row_step;
+                            if (++ky == 3) ky = 0;
                             if (elect_one()) {
 #pragma unroll
-                                for (int k = 0; k < 4; ++k)   // 16 co: 16 rows of A (2048 bytes), 32 bytes along a row of B
-                                    mma_bf16(tmem_d, ad + 128 * k, bd + 2 * k, idesc, k ? 1u : acc_on);
+                                for (int kx = 0; kx < 3; ++kx)
+#pragma unroll
+                                    for (int k = 0; k < 4; ++k)   // 16 co: 16 rows of A (2048 bytes), 32 bytes along a row of B
+                                        mma_bf16(tmem_d, ad + kx * a_tap + 128 * k, bd + (2 - kx) * 8 + 2 * k, idesc, kx + k ? 1u : acc_on);
                             }
                             acc_on = 1u;
                         }
-                        if (!p.resident && elect_one()) mma_commit(&pipe.w_empty[ws]);
-                        if (++ws == p.nw) { ws = 0; wpar ^= 1u; }
                     }
-                    if (ok && elect_one()) mma_commit(&pipe.q_empty[qs]);
-                    if (++qs == p.nq) { qs = 0; qpar ^= 1u; }
+                    if (!p.resident && elect_one()) mma_commit(&pipe.w_empty[ws]);
+                    if (++ws == p.nw) { ws = 0; wpar ^= 1u; }
                 }
-                if (ok && elect_one()) mma_commit(&pipe.acc_full[slot]);
+                if (ok && elect_one()) mma_commit(&pipe.q_empty[qs]);
+                if (++qs == p.nq) { qs = 0; qpar ^= 1u; }
             }
-            if (lane == 0) {
-                report_wait(p.stats, 0, wq);
-                report_wait(p.stats, 1, ww);
-                report_wait(p.stats, 2, wa);
-                report_wait(p.stats, 6, clock64() - born);
-                report_wait(p.stats, 7, 1);
-            }
+            if (ok && elect_one()) mma_commit(&pipe.acc_full[slot]);
+        }
+        if (lane == 0 && it > slot) {
+            report_wait(p.stats, 0, wq);
+            report_wait(p.stats, 1, ww);
+            report_wait(p.stats, 2, wa);
+            report_wait(p.stats, 6, clock64() - born);
+            report_wait(p.stats, 7, 1);
         }
     } else if (warp >= 4) {
         // epilogue: TMEM lane = input channel, column = patch position. Warp (q, part): lane quarter q,
@@ -291,7 +353,7 @@ tc3_tma_dx_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
         bool ok = true;
         long long it = 0;
         long long we = 0;
-        for (long long t = blockIdx.x; t < p.ntiles; t += gridDim.x, ++it) {
+        for (long long t = t_first; t < p.ntiles; t += t_step, ++it) {
             const int slot = static_cast<int>(it & 1);
             const unsigned uses = static_cast<unsigned>(it >> 1);
             int ci0, b0, y0;
@@ -302,7 +364,7 @@ tc3_tma_dx_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
             const int ci_l = q * 32 + lane;
             const int rows_valid = p.H - y0 < p.Ht ? p.H - y0 : p.Ht;
             // ---- phase A: accumulator -> staging block (rows of bf16 or fp32 values per channel)
-            if (ci0 + q * 32 < p.Cin) {                              // warp-uniform: some of my 32 channels exist
+            if (ci0 + (p.split ? (q & 1) * 32 : q * 32) < p.Cin) {   // warp-uniform: some of my 32 channels exist
                 unsigned char *row = stage + ci_l * p.pitch;
                 for (int chn = ch_lo; chn < ch_hi; ++chn) {
                     unsigned v[32];
@@ -313,11 +375,12 @@ tc3_tma_dx_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
                     const uint4 t0 = tp[0], t1 = tp[1], t2 = tp[2], t3 = tp[3];
                     const unsigned tw[16] = {t0.x, t0.y, t0.z, t0.w, t1.x, t1.y, t1.z, t1.w,
                                              t2.x, t2.y, t2.z, t2.w, t3.x, t3.y, t3.z, t3.w};
-                    if (p.es == 4) {
+                    if (p.es == 4 || p.KS > 1) {
+                        const float f = p.KS > 1 ? 1.f : delta;      // partial sums are scaled when they have met
 #pragma unroll
                         for (int j = 0; j < 32; ++j) {
                             const int o = static_cast<int>(static_cast<short>((tw[j >> 1] >> (16 * (j & 1))) & 0xffffu));
-                            if (o >= 0) *reinterpret_cast<float *>(row + 4 * o) = __uint_as_float(v[j]) * delta;
+                            if (o >= 0) *reinterpret_cast<float *>(row + 4 * o) = __uint_as_float(v[j]) * f;
                         }
                     } else if (p.pairs) {
                         // entry 2i tells where columns 2i, 2i+1 go
@@ -336,6 +399,7 @@ tc3_tma_dx_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
                     }
                 }
             }
+            if (p.KS > 1) continue;                                  // one tile per cluster: the sums meet below
             // the accumulator is free once every epilogue warp has read its part
             tc_fence_before();
             warp_arrive(&pipe.acc_empty[slot]);
@@ -351,12 +415,16 @@ tc3_tma_dx_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
                     for (int r = et >> 5; r < ncv; r += kEpiThreads / 32) {
                         const unsigned char *src = stage + r * p.pitch + p.es * img * p.run;
                         unsigned char *dst = dst0 + ((static_cast<long long>(b0 + img) * p.Cin + ci0 + r) * HW + y0 * p.W) * p.es;
-                        if (words) {
-                            for (int i = lane; i < nwords; i += 32)
-                                reinterpret_cast<unsigned *>(dst)[i] = reinterpret_cast<const unsigned *>(src)[i];
+                        // four independent loads per lane and round: one by one the round trips through shared memory
+                        // were what an epilogue took its time for
+                        if (p.split) {                           // the low pieces' sums, 64 rows further, and the high pieces'
+                            const float *hi = reinterpret_cast<const float *>(src), *lo = reinterpret_cast<const float *>(src + 64 * p.pitch);
+                            copy_run(reinterpret_cast<float *>(dst), len, lane, [&](int i) { return hi[i] + lo[i]; });
+                        } else if (words) {
+                            copy_run(reinterpret_cast<unsigned *>(dst), nwords, lane, [&](int i) { return reinterpret_cast<const unsigned *>(src)[i]; });
                         } else {
-                            for (int i = lane; i < len; i += 32)
-                                reinterpret_cast<unsigned short *>(dst)[i] = reinterpret_cast<const unsigned short *>(src)[i];
+                            copy_run(reinterpret_cast<unsigned short *>(dst), len, lane,
+                                     [&](int i) { return reinterpret_cast<const unsigned short *>(src)[i]; });
                         }
                     }
                 }
@@ -365,6 +433,46 @@ tc3_tma_dx_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
             asm volatile("bar.sync 1, %0;" ::"n"(kEpiThreads) : "memory");
         }
         if (et == 0) report_wait(p.stats, 5, we);
+    }
+    if (p.KS > 1) {
+        cluster_barrier();                 // every CTA's partial sums are staged
+        // this CTA finishes 128 / KS channels: rows read from all staging blocks, lanes along the positions
+        int ci0, b0, y0;
+        tile_of(t_first, ci0, b0, y0);
+        const int per = 128 / p.KS, rows_valid = p.H - y0 < p.Ht ? p.H - y0 : p.Ht, len = rows_valid * p.W, HW = p.H * p.W;
+        const int nimg = p.B - b0 < p.nb ? p.B - b0 : p.nb, row_len = (nimg - 1) * p.run + len;
+        const float delta = *p.delta_p;
+        unsigned base[8];
+#pragma unroll
+        for (int k = 0; k < 8; ++k)
+            if (k < p.KS) asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(base[k]) : "r"(smem_u32(stage)), "r"(k));
+        for (int r = warp; r < per; r += kThreadsX / 32) {
+            const int cl = rank * per + r, ci = ci0 + cl;
+            if (ci >= p.Cin) break;
+            for (int i0 = lane; i0 < row_len; i0 += 128) {           // whole images are back to back in the staged row
+                float v[4][8];
+#pragma unroll
+                for (int u = 0; u < 4; ++u)
+#pragma unroll
+                    for (int k = 0; k < 8; ++k)
+                        if (k < p.KS && i0 + 32 * u < row_len)
+                            asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(v[u][k]) : "r"(base[k] + cl * p.pitch + 4 * (i0 + 32 * u)));
+#pragma unroll
+                for (int u = 0; u < 4; ++u) {
+                    const int i = i0 + 32 * u;
+                    if (i >= row_len) break;
+                    float sum = 0.f;
+#pragma unroll
+                    for (int k = 0; k < 8; ++k)
+                        if (k < p.KS) sum += v[u][k];
+                    const int img = i / p.run, pos = i - img * p.run;
+                    const long long o = (static_cast<long long>(b0 + img) * p.Cin + ci) * HW + y0 * p.W + pos;
+                    if (p.es == 4) static_cast<float *>(p.dX)[o] = sum * delta;
+                    else static_cast<__nv_bfloat16 *>(p.dX)[o] = __float2bfloat16_rn(sum * delta);
+                }
+            }
+        }
+        cluster_barrier();                 // nobody leaves while its staging block is still being read
     }
     tc_fence_before();
     __syncthreads();
@@ -414,81 +522,94 @@ int launch_tc3_tma_dx(dbp_ctx *ctx, const void *codes_nhwc, const void *W, int i
     p.es = dx_bf16 ? 2 : 4;
     p.ntaps = io == DBP_F32 ? 18 : 9;
     p.B = static_cast<int>(s.B); p.Cin = static_cast<int>(s.Cin); p.Cout = static_cast<int>(s.Cout);
-    p.H = static_cast<int>(s.H); p.W = static_cast<int>(s.W); p.Wp = p.W + 2;
+    p.H = static_cast<int>(s.H); p.W = static_cast<int>(s.W);
     p.err_flag = err_flag;
     p.stats = ctx->wait_stats;
     p.phase_cin = (ctx->phase_cin > 0 && ctx->phase_cin % 128 == 0 && s.Cin == 4ll * ctx->phase_cin) ? ctx->phase_cin : 0;
     p.ncb = (p.Cout + 63) / 64;
     p.ci_tiles = (p.Cin + 127) / 128;
-    p.a_panels = p.Cin <= 64 ? 1 : 2;
-    const size_t tap_bytes = static_cast<size_t>(p.a_panels) * kWPanel;
-    const size_t budget = 227 * 1024 - 2048;
-    // patch geometry: the cheapest of the candidates by (waves of one CTA per SM) x (columns per tile;
-    // a narrow MMA takes as long to issue as one of about 200 columns takes to run). A candidate must
-    // leave room for its two patch buffers, its staging block and at least three weight taps.
-    const int sms = ctx->sm_count;
-    int best_ht = 0, best_nb = 1;
-    double best_cost = 1e300;
-    auto patch_bytes = [&](int ht, int nb, int n) {
-        const int img_rows = (ht + 2) * p.Wp, rows_read = n + 2 * p.Wp + 2;
-        return round_up((rows_read > img_rows * nb ? rows_read : img_rows * nb) * 128, 1024);
-    };
-    auto stage_pitch = [&](int ht, int nb) {
-        int pitch = round_up(nb * ht * p.W * p.es, 4);
-        if ((pitch / 4) % 2 == 0) pitch += 4;      // an odd number of words: see below
-        return pitch;
-    };
-    auto consider = [&](int ht, int nb) {
-        const int img_rows = (ht + 2) * p.Wp;
-        const int last = (nb - 1) * img_rows + (ht - 1) * p.Wp + p.W - 1;     // last column that holds an output
-        const int n = round_up(last + 1, 16);
-        if (n > 256 || img_rows * nb > 1024) return;
-        if (2 * static_cast<size_t>(patch_bytes(ht, nb, n)) + 128 * static_cast<size_t>(stage_pitch(ht, nb)) + 1536 + 3 * tap_bytes > budget) return;
-        const long long tiles = nb == 1 ? static_cast<long long>(p.B) * ((p.H + ht - 1) / ht) : (p.B + nb - 1) / nb;
-        const long long waves = (tiles * p.ci_tiles + sms - 1) / sms;
-        const double cost = static_cast<double>(waves) * ((n < 208 ? 208 : n) + 64);      // an MMA takes >= ~100 clocks to issue
-        if (cost < best_cost) { best_cost = cost; best_ht = ht; best_nb = nb; }
-    };
-    for (int ht = 1; ht <= p.H; ++ht) consider(ht, 1);
-    for (int nb = 2; nb <= 16 && nb <= p.B; ++nb) consider(p.H, nb);
-    if (best_ht == 0) return DBP_EUNSUPPORTED;
-    p.Ht = best_ht; p.nb = best_nb;
-    p.tiles_y = (p.H + p.Ht - 1) / p.Ht;
-    p.img_rows = (p.Ht + 2) * p.Wp;
-    p.N = round_up((p.nb - 1) * p.img_rows + (p.Ht - 1) * p.Wp + p.W, 16);
-    p.pos_tiles = p.nb == 1 ? static_cast<long long>(p.B) * p.tiles_y : (p.B + p.nb - 1) / p.nb;
-    p.ntiles = p.pos_tiles * p.ci_tiles;
-    p.q_tx = p.img_rows * p.nb * 128;
-    // the last tap of the last column reads row N - 1 + 2 Wp + 2; rows past the copied patch hold
-    // stale data, which only reaches columns that are never stored
-    p.q_bytes = patch_bytes(p.Ht, p.nb, p.N);
-    p.run = p.Ht * p.W;
-    // an odd number of 32-bit words per row: the 32 channels of a warp hit 32 different banks when
-    // they stage the same position
-    p.pitch = stage_pitch(p.Ht, p.nb);
-    p.pairs = p.W % 2 == 0 ? 1 : 0;
-    const size_t stage_bytes = static_cast<size_t>(128) * p.pitch;
-    // Weights: a slot holds G taps and is handed over with one barrier (the hand-over, not the copy
-    // instruction, is what costs time). With one ci block and room for all taps of all co blocks they
-    // are loaded once and stay; otherwise they stream through a ring of slots.
+    p.split = io == DBP_F32 && p.Cin <= 64 ? 1 : 0;
+    p.a_panels = p.Cin <= 64 && !p.split ? 1 : 2;
+    const int map_taps = p.ntaps;
+    if (p.split) p.ntaps = 9;
     p.nq = kMaxQ;
-    const size_t fixed = static_cast<size_t>(p.nq) * p.q_bytes + stage_bytes + 512 + 1024;
-    const size_t room = budget - fixed;
-    const int slots_all = p.ncb * (p.ntaps / 9);
-    if (p.ci_tiles == 1 && slots_all <= kMaxW && static_cast<size_t>(slots_all) * 9 * tap_bytes <= room) {
-        p.resident = 1; p.G = 9; p.nw = slots_all;
-    } else if (room >= 2 * 3 * tap_bytes) {
-        p.resident = 0; p.G = 3; p.nw = static_cast<int>(room / (3 * tap_bytes));
-    } else {
-        p.resident = 0; p.G = 1; p.nw = static_cast<int>(room / tap_bytes);
+    const int sms = ctx->sm_count;
+    size_t smem = 0;
+    double best = 1e300;
+    Dx3T chosen{};
+    // The cheapest of the candidate patches (rows of one image, or several whole images) and reduction splits by a count of
+    // clocks (see the head of this file; 6 KB per clock is about what the L2 delivers to all SMs together). Returns whether the
+    // patch still fits the accumulator.
+    auto consider = [&](int ht, int nb, int ks) -> bool {
+        Dx3T q = p;
+        q.Ht = ht; q.nb = nb; q.KS = ks;
+        q.Wp = (p.W % 2 == 0 && p.es == 2 && ks == 1) ? p.W + 2 : p.W + 1;
+        q.img_rows = (nb == 1 ? ht + 2 : ht + 1) * q.Wp;
+        q.N = round_up((nb - 1) * q.img_rows + (ht - 1) * q.Wp + p.W, 16);    // up to the last column that holds an output
+        if (q.N > 256) return false;
+        const int rows_read = q.N + 2 * q.Wp + 2;
+        q.q_bytes = round_up((rows_read > q.img_rows * nb ? rows_read : q.img_rows * nb) * 128, 1024);
+        q.q_tx = q.img_rows * nb * 128;
+        q.tiles_y = (p.H + ht - 1) / ht;
+        q.pos_tiles = nb == 1 ? static_cast<long long>(p.B) * q.tiles_y : (p.B + nb - 1) / nb;
+        q.ntiles = q.pos_tiles * p.ci_tiles;
+        // one round of clusters; a GPC's SMs are no multiple of 4 or 8, so not all of them can be covered (36 clusters of 4
+        // took 39 us where 32 took 24)
+        if (ks > 1 && q.ntiles * ks > (ks == 2 ? sms : ks == 4 ? sms * 7 / 8 : sms * 3 / 4)) return true;
+        q.run = ht * p.W;
+        // an odd number of 32-bit words per row: the 32 channels of a warp hit 32 different banks when they stage the same
+        // position
+        const int es = ks > 1 ? 4 : p.es;
+        q.pitch = round_up(nb * q.run * es, 4);
+        if ((q.pitch / 4) % 2 == 0) q.pitch += 4;
+        q.pairs = p.W % 2 == 0 ? 1 : 0;
+        // Weights: a slot holds G taps and is handed over with one barrier (the hand-over, not the copy instruction, is what
+        // costs time). With one ci block and room for all taps of all co blocks they are loaded once and stay; otherwise they
+        // stream through a ring of slots.
+        const size_t tap_bytes = static_cast<size_t>(p.a_panels) * kWPanel, budget = 227 * 1024 - 2048;
+        const size_t fixed = static_cast<size_t>(q.nq) * q.q_bytes + static_cast<size_t>(128) * q.pitch + 512 + 1024;
+        if (fixed + 3 * tap_bytes > budget) return true;
+        const size_t room = budget - fixed;
+        const int slots_all = p.ncb * (p.ntaps / 9);
+        if (p.phase_cin > 0) {
+            q.resident = 0; q.G = 2; q.nw = static_cast<int>(room / (2 * tap_bytes));
+            if (q.nw < 2) return true;
+        } else if (ks == 1 && p.ci_tiles == 1 && slots_all <= kMaxW && static_cast<size_t>(slots_all) * 9 * tap_bytes <= room) {
+            q.resident = 1; q.G = 9; q.nw = slots_all;
+        } else if (room >= 2 * 3 * tap_bytes) {
+            q.resident = 0; q.G = 3; q.nw = static_cast<int>(room / (3 * tap_bytes));
+        } else {
+            q.resident = 0; q.G = 1; q.nw = static_cast<int>(room / tap_bytes);
+        }
+        if (q.nw > kMaxW) q.nw = kMaxW;
+        q.w_slot = static_cast<int>(q.G * tap_bytes);
+        const double live = p.phase_cin > 0 ? 0.25 : 1.0;
+        const long long ctas = q.ntiles * ks, waves = (ctas + sms - 1) / sms, active = ctas < sms ? ctas : sms;
+        double mma = 32.0 + 0.25 * q.N + (q.resident ? 0.0 : 16.0 * p.a_panels);
+        if (mma < 0.5 * q.N) mma = 0.5 * q.N;
+        const double l2 = q.resident ? 0.0 : 2048.0 * p.a_panels * static_cast<double>(active) / 6000.0;
+        if (mma < l2) mma = l2;
+        const int cbs = (p.ncb + ks - 1) / ks;
+        const double body = cbs * (p.ntaps * live * 4.0 * mma + (q.resident ? 0.0 : 250.0 * (p.phase_cin > 0 ? p.ntaps / 6.0 : static_cast<double>(p.ntaps) / q.G)) + q.q_tx / 128.0 + 300.0);
+        const double staged = (p.Cin <= 64 && !p.split ? 64.0 : 128.0) * nb * q.run * es;
+        const double epi = 2000.0 + staged / 20.0 + (ks > 1 ? 2000.0 + staged / 8.0 : 0.0);
+        const double cost = static_cast<double>(waves) * (500.0 + (body > epi ? body : epi)) + (waves > 1 ? (body < epi ? body : epi) : epi);
+        if (cost < best) { best = cost; chosen = q; smem = fixed + static_cast<size_t>(q.nw) * q.w_slot; }
+        return true;
+    };
+    for (int ht = 1; ht <= p.H; ++ht)
+        if (!consider(ht, 1, 1)) break;
+    for (int ks = 1; ks <= 8; ks *= 2) {
+        if (ks > p.ncb || (ks > 1 && p.split)) break;
+        for (int nb = ks > 1 ? 1 : 2; nb <= 64 && nb <= p.B; ++nb)
+            if (!consider(p.H, nb, ks)) break;
     }
-    if (p.nw > kMaxW) p.nw = kMaxW;
-    p.w_slot = static_cast<int>(p.G * tap_bytes);
-    const size_t smem = fixed + static_cast<size_t>(p.nw) * p.w_slot;
+    if (smem == 0) return DBP_EUNSUPPORTED;
+    p = chosen;
 
     // re-laid weights
     const long long w_pitch = (s.Cin + 7) / 8 * 8, q_pitch = (s.Cout + 7) / 8 * 8;
-    const size_t wb = sizeof(__nv_bfloat16) * static_cast<size_t>(s.Cout) * w_pitch * p.ntaps;
+    const size_t wb = sizeof(__nv_bfloat16) * static_cast<size_t>(s.Cout) * w_pitch * map_taps;
     int rc = ws_reserve(ctx, ctx->w_taps, wb);
     if (rc) return rc;
     if (!weights_ready) {
@@ -509,12 +630,12 @@ int launch_tc3_tma_dx(dbp_ctx *ctx, const void *codes_nhwc, const void *W, int i
                                             static_cast<unsigned long long>(s.H), static_cast<unsigned long long>(s.B)};
         const unsigned long long row = static_cast<unsigned long long>(q_pitch) * 2;
         const unsigned long long str[3] = {row, row * s.W, row * s.W * s.H};
-        const unsigned box[4] = {64, static_cast<unsigned>(p.Wp), static_cast<unsigned>(p.Ht + 2), static_cast<unsigned>(p.nb)};
+        const unsigned box[4] = {64, static_cast<unsigned>(p.Wp), static_cast<unsigned>(p.img_rows / p.Wp), static_cast<unsigned>(p.nb)};
         if (!encode_map_bf16(&map_q, codes_nhwc, 4, dims, str, box)) return fail_cuda("tensor map of the code patches");
     }
     {
         const unsigned long long dims[3] = {static_cast<unsigned long long>(s.Cin), static_cast<unsigned long long>(s.Cout),
-                                            static_cast<unsigned long long>(p.ntaps)};
+                                            static_cast<unsigned long long>(map_taps)};
         const unsigned long long str[2] = {static_cast<unsigned long long>(w_pitch) * 2,
                                            static_cast<unsigned long long>(w_pitch) * 2 * s.Cout};
         const unsigned box[3] = {64, 64, static_cast<unsigned>(p.phase_cin > 0 ? 1 : p.G)};
@@ -522,6 +643,9 @@ int launch_tc3_tma_dx(dbp_ctx *ctx, const void *codes_nhwc, const void *W, int i
     }
     if (cudaFuncSetAttribute(tc3_tma_dx_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem)) != cudaSuccess)
         return fail_cuda("shared memory size");
+    if (p.KS > 1)
+        return cuda_ok(launch_chained_cluster(tc3_tma_dx_kernel, static_cast<unsigned>(p.ntiles) * p.KS, static_cast<unsigned>(p.KS),
+                                              dim3(kThreadsX), smem, ctx->stream, map_q, map_w, p));
     const long long grid = p.ntiles < sms ? p.ntiles : sms;
     return cuda_ok(launch_chained(tc3_tma_dx_kernel, dim3(static_cast<unsigned>(grid)), dim3(kThreadsX), smem, ctx->stream,
                                   map_q, map_w, p));

@@ -140,7 +140,6 @@ tma_dx_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constant__
     // everything above touched only this CTA's shared and tensor memory; what follows reads what
     // earlier kernels wrote
     chain_wait();
-    chain_release();
 
     if (warp == 0) {
         {   // the whole warp runs the loop (uniform control flow and operands); one elected lane issues
@@ -177,6 +176,8 @@ tma_dx_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constant__
                     if (++s == S) { s = 0; parity ^= 1u; }
                 }
             }
+            chain_release();       // every copy is issued: the next kernel may take the slots that come free (earlier it would
+                                   // hold thread slots that the dW stream's kernels want: stride-2 set 796 against 745 us)
             if (lane == 0) report_wait(p.stats, 3, waited);
         }
     } else if (warp == 1) {

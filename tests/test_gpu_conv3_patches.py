@@ -1,0 +1,44 @@
+"""3x3 input gradients whose patches share halos, whose reduction over output channels is split over a cluster of CTAs, or
+whose weight pieces share the accumulator: parity with the oracle and bit-identical repeats."""
+import numpy as np
+import pytest
+import torch
+
+import oracle
+import workloads as wl
+
+pytestmark = pytest.mark.gpu
+TOL = 1e-5
+
+
+@pytest.fixture(scope="module")
+def ctx():
+    import paper_2004_04729_b200 as dbp
+    c = dbp.Context(0)
+    yield c
+    c.close()
+
+
+@pytest.mark.parametrize("B,Ci,Co,H,W,dtype", [
+    (1, 512, 512, 7, 7, "bf16"), (9, 256, 512, 7, 7, "bf16"), (5, 200, 320, 4, 6, "bf16"),    # clusters, partial last patches
+    (3, 128, 576, 2, 2, "bf16"),                                                              # nine blocks of channels over a cluster
+    (30, 512, 136, 2, 2, "f32"), (7, 136, 512, 4, 4, "f32"), (2, 264, 128, 14, 14, "f32"),
+    (1, 128, 128, 1, 1, "f32"),
+    (3, 64, 64, 13, 32, "f32"), (2, 40, 72, 9, 11, "f32"), (1, 3, 200, 33, 62, "f32")])      # both weight pieces in one MMA
+def test_input_gradient(ctx, B, Ci, Co, H, W, dtype):
+    import paper_2004_04729_b200 as dbp
+    L = wl.conv_layer(B, Ci, Co, H, W, 3, data_seed=B + Ci + 5 * Co + H, scale=2.0, seed=9, dtype=dtype)
+    tdt = torch.bfloat16 if dtype == "bf16" else torch.float32
+    d, X, Wt = (torch.from_numpy(np.ascontiguousarray(a)).to(tdt).cuda() for a in (L.delta, L.X, L.W))
+    out = dbp.dithered_conv_backward(ctx, d, X, Wt, L.seed, L.scale, flags=dbp.DBP_DX_F32)
+    D, _ = ctx.last_step()
+    assert ctx.last_device_status() == (0, 0)
+    codes, _, _ = oracle.nsd_codes(L.delta, L.seed, np.float32(D))
+    ref = oracle.conv_backward(codes, np.float32(D), L.X, L.W, with_abs=True)
+    for key in ("dX", "dW"):
+        g = out[key].double().cpu().numpy()
+        assert np.linalg.norm(g - ref[key]) <= TOL * np.linalg.norm(ref[key]) + 1e-30, key
+        assert np.all(np.abs(g - ref[key]) <= TOL * ref["S_" + key] + 1e-30), key
+    for _ in range(3):
+        again = dbp.dithered_conv_backward(ctx, d, X, Wt, L.seed, L.scale, need_dW=False)["dX"]
+        assert torch.equal(again, out["dX"].to(again.dtype))
