@@ -434,15 +434,14 @@ int conv_backward_impl(dbp_ctx *ctx, const void *delta, const void *X, const voi
                                    t3 ? &s : nullptr, t3 ? &codes_n : nullptr, jobs, stack_g, &codes_st, mask_q);
     if (rc) return rc;
     // Activations the copy engine cannot address as they are (fp32: two bf16 pieces; planes that are no multiple of 16
-    // bytes; stacked tiny planes) are re-written into the set's own buffer: beside the quantizer where the call ends with
-    // its dW, on the stream of the dW kernels where that stream runs behind the caller's anyway (DBP_DW_ASYNC: 4 % on the
-    // VGG-16 layer set) or where a *_host call's activations are still on their way up.
+    // bytes; stacked tiny planes) are re-written into the set's own buffer, beside the quantizer. A *_host call's
+    // activations are still on their way up: there it is done on the stream that waits for them.
     const void *Xp = X;
     long long x_pitch = s.H * s.W;
     const StridedLayer *st2 = ctx->strided;
     const bool rewrite_x = dW && (st2 || io == DBP_F32 || x_pitch % 8 != 0);
     const bool forked = dX && dW && ctx->aux != nullptr;
-    const bool late_x = ctx->hook_before_dw != nullptr || (forked && (flags & DBP_DW_ASYNC));
+    const bool late_x = ctx->hook_before_dw != nullptr;
     auto write_x = [&](bool beside) -> int {
         KernelTimer t(ctx, DBP_K_DW_DENSE);
         if (st2) return launch_phase_rows(ctx, st2->X, ctx->x_padded[k].ptr, io, s.B, st2->Cin, st2->H, st2->W, st2->phases, x_pitch, beside);
