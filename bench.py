@@ -688,6 +688,19 @@ def main():
 
     # every kind by itself: one product per call, so nothing runs beside anything else (the quantization kinds
     # are taken from the dX-only pass)
+    # layers whose quantization and products are one kernel
+    ctx.profile_enable(True)
+    ctx.profile_select(["fused"])
+    ctx.profile_read()
+    fused_layers = set()
+    for i, item in enumerate(layers):
+        run_layer(*item)
+        torch.cuda.synchronize()
+        if ctx.profile_read()["fused"][1]:
+            fused_layers.add(i)
+    ctx.join()
+    ctx.profile_enable(False)
+    ctx.profile_select(None)
     alone = {}
     for want_dw, want_dx in ((False, True), (True, False)):
         step(want_dw, want_dx)
@@ -764,10 +777,12 @@ def main():
     dense_on = prof["dx_dense"][1] > 0
     is_dense = lambda L: (dense_on and L.dtype == "bf16" and L.X.shape[1] % 8 == 0 and L.delta.shape[1] % 8 == 0)
     work = {k: 0.0 for k in ("statistics", "quantize", "dx", "dw", "dx_dense", "dw_dense", "fused")}
-    for (L, d, X, W, dW, dX) in layers:
+    for i, (L, d, X, W, dW, dX) in enumerate(layers):
         nd, nx, nw = d.numel(), X.numel(), W.numel()
-        if prof["fused"][1] > 0:                                       # two chained launches per layer: dense MMAs on the codes
+        if i in fused_layers:                                          # dense MMAs on the codes
             work["fused"] += L.dense_flops
+            if L.kind != "linear":
+                work["statistics"] += nd * e
             continue
         cb = 2 if is_dense(L) else 1                                   # bytes per code the product kernels read
         work["statistics"] += nd * e                                   # bytes
@@ -785,11 +800,15 @@ def main():
         kern[top]["ms_per_step_timed_region"] = t_s * 1e3
     if top == "fused":
         ach = work[top] / t_s / 1e12
-        roof = {"kernel": "small linear backward (small_linear_quantize_kernel + small_linear_products_kernel)", "bound": "tensor",
+        conv = any(layers[i][0].kind != "linear" for i in fused_layers)
+        roof = {"kernel": "thin 1x1 backward (fused1x1_kernel)" if conv else
+                          "small linear backward (small_linear_quantize_kernel + small_linear_products_kernel)", "bound": "tensor",
                 "achieved": ach, "peak": tensor_peak()[0], "unit": "TFLOP/s", "frac": ach / tensor_peak()[0], "traffic": None,
                 "peak_source": tensor_peak()[1],
-                "note": "dense-equivalent flops of both products (2 * 2 * B * N * K) / time of the two launches; at these sizes they "
-                        "are bound by launch and load latency, not by the tensor pipe (warp-level MMAs, two bf16 pieces per fp32 operand)"}
+                "note": "dense-equivalent flops of both products / time of the launches" + (
+                        "; bound by the quantization's instruction issue, not by the tensor pipe" if conv else
+                        " (2 * 2 * B * N * K per layer); at these sizes they are bound by launch and load latency, not by the "
+                        "tensor pipe (warp-level MMAs, two bf16 pieces per fp32 operand)")}
     elif top in ("dx", "dw"):
         ach = work[top] / t_s / 1e12
         roof = {"kernel": f"sparse {top} (conv_{top}2_kernel)", "bound": "alu", "achieved": ach,

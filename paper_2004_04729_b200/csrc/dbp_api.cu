@@ -426,6 +426,23 @@ int conv_backward_impl(dbp_ctx *ctx, const void *delta, const void *X, const voi
             if (pr) return pr;
         }
     }
+    // thin 1x1 layers: nothing but the statistics runs in front of one kernel that quantizes and multiplies
+    if (t1 && dW && dX && !db && !q_out && dx_bf16 && !ctx->strided && !ctx->hook_before_dw && fused1x1_supported(ctx, s, io)) {
+        if (int wr = wait_code_set(ctx)) return wr;
+        StepSource step;
+        float *const publish[2] = {ctx->delta_sets + k, nullptr};
+        {
+            KernelTimer t(ctx, DBP_K_STATISTICS);
+            if (int sr = launch_statistics(ctx, delta, io, numel, scale, delta_in, publish, nullptr, &step, jobs)) return sr;
+        }
+        {
+            KernelTimer t(ctx, DBP_K_FUSED);
+            if (int fr = launch_fused1x1(ctx, delta, X, W, s, seed, step, dW, dX, &ctx->state->tc_timeout)) return fr;
+        }
+        if (ctx->hook_after_dx && cudaEventRecord(ctx->hook_after_dx, ctx->stream) != cudaSuccess) return DBP_ECUDA;
+        read_density();
+        return ctx->aux_pending && !(flags & DBP_DW_ASYNC) ? dbp_join(ctx) : DBP_OK;
+    }
     // tiny planes: the weight-gradient kernel reads the images stacked into tall ones
     const int stack_g = (t3 && dW && !ctx->strided) ? tc3_stack_images(s, io) : 0;
     const void *codes_st = nullptr, *codes16 = nullptr, *codes_n = nullptr;

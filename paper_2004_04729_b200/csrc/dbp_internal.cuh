@@ -246,6 +246,11 @@ int launch_relu_backward(dbp_ctx *ctx, const float *da, const uint8_t *mask, flo
 int launch_maxpool_backward(dbp_ctx *ctx, const float *g, const int8_t *argmax, float *out,
                             long long planes, long long h, long long w);
 
+// ---- fused1x1.cu: quantization and both products of a thin bf16 1x1 layer in one kernel (dW cleared by the caller, bf16 dX)
+bool fused1x1_supported(const dbp_ctx *ctx, const ConvShape &s, int io);
+int launch_fused1x1(dbp_ctx *ctx, const void *delta, const void *X, const void *W, const ConvShape &s, unsigned long long seed,
+                    const StepSource &step, float *dW, void *dX, int *err_flag);
+
 // ---- direct5.cu: both products of a 5x5 layer of few channels by FMAs on the dense codes (dW cleared by the caller)
 bool direct5_supported(const ConvShape &s, bool want_dw, bool want_dx);
 int launch_direct5(dbp_ctx *ctx, const int8_t *codes, const void *X, const void *W, int io, const float *delta_p,
