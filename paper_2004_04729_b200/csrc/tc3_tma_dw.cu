@@ -18,6 +18,9 @@
 // on either side), an output tile of 128 input channels x 64 or 128 output channels, the three
 // taps ky of its kx as three accumulators in tensor memory. With 64 output channels the taps ky = 1
 // and ky = 0 share one MMA of N = 128: its second 64-column group starts W rows further on.
+// fp32 activations are two bf16 pieces, one after the other along the batch. Layers of at most 64 input channels put both
+// pieces of a position on the two halves of one tile (half as many MMAs, the codes are read once; 64 -> 64 at 32x32, batch
+// 128: 100 -> 91 us for the whole call).
 // Warp 0 copies code panels, warp 1 activation tiles, warp 2 issues the MMAs, warp 3 zeroes the
 // masked rows, warps 4-7 stage the accumulators in shared memory and the copy engine adds them into a
 // zero-initialised fp32 scratch [tap][co][ci] (the reduction over CTAs; the order of the additions,
@@ -40,6 +43,7 @@ constexpr int kMaxNX = 6;
 struct Dw3T {
     int Cin, Cout, W, HW;
     int code_batch;               // images of the code tensor (the activations may hold two pieces of every image, one after the other)
+    int split;                    // both pieces of (at most 64) channels share a tile: rows 0-63 the high ones, 64-127 the low ones
     int SEG;                      // positions per segment (multiple of 64)
     int segs_per_img;
     long long nseg, per_split;
@@ -173,8 +177,11 @@ tc3_tma_dw_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
                         mbar_expect_tx(&pipe.x_full[s], kXSlot);
                         // positions past the image's end read as zero (a block past its end is all zero)
 #pragma unroll
-                        for (int i = 0; i < kXS; ++i)
+                        for (int i = 0; i < kXS; ++i) {
                             tma_load_3d(dst + i * kXTile, &map_x, (blk + i) * 64, ci0, b, &pipe.x_full[s]);
+                            if (p.split)
+                                tma_load_3d(dst + i * kXTile + kXTile / 2, &map_x, (blk + i) * 64, 0, b + p.code_batch, &pipe.x_full[s]);
+                        }
                         if (++s == p.nx) { s = 0; parity ^= 1u; }
                         j = 0;
                     }
@@ -321,9 +328,10 @@ tc3_tma_dw_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
                 for (int i = 0; i < nb; ++i) {
                     unsigned v[32];
                     tmem_ld32(tmem_base + (static_cast<unsigned>(q * 32) << 16) + (c0 + i) * 32, v);
-                    float *dst = stg + i * 4096 + q * 32 + lane;
+                    float *dst = stg + i * 4096 + (p.split ? (q >> 1) * 2048 + (q & 1) * 32 : q * 32) + lane;
+                    const int pitch = p.split ? 64 : 128;
 #pragma unroll
-                    for (int j = 0; j < 32; ++j) dst[j * 128] = __uint_as_float(v[j]);
+                    for (int j = 0; j < 32; ++j) dst[j * pitch] = __uint_as_float(v[j]);
                 }
                 fence_async_proxy();
                 asm volatile("bar.sync 1, 128;" ::: "memory");
@@ -335,6 +343,7 @@ tc3_tma_dw_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
                         else { ky = 2 - (c >> 1); col0 = (c & 1) * 32; }       // columns 0-63: ky = 2, 64-127: ky = 1, 128-191: ky = 0
                         // columns past Cout hold exact zeros (their codes were zero fill): adding them is harmless
                         tma_reduce_add_2d(&map_acc, ci0, (ky * 3 + kx) * p.Cout + co0 + col0, stg + i * 4096);
+                        if (p.split) tma_reduce_add_2d(&map_acc, 0, (ky * 3 + kx) * p.Cout + co0 + col0, stg + i * 4096 + 2048);
                     }
                     bulk_commit();
                     bulk_wait_read_all();
@@ -531,7 +540,8 @@ int launch_tc3_tma_dw(dbp_ctx *ctx, const void *codes_nhwc, const void *X, int p
     if (smem == 0) return DBP_EUNSUPPORTED;
     p.segs_per_img = (p.HW + p.SEG - 1) / p.SEG;
     p.code_batch = static_cast<int>(s.B);
-    p.nseg = s.B * pieces * p.segs_per_img;
+    p.split = pieces == 2 && s.Cin <= 64 ? 1 : 0;
+    p.nseg = s.B * (p.split ? 1 : pieces) * p.segs_per_img;
     // a stride-2 layer on phase images whose phases are whole channel tiles: 6 of the 12 (phase, kernel column)
     // pairs carry taps of the strided layer
     p.phase_tiles = (ctx->phase_cin > 0 && ctx->phase_cin % 128 == 0 && cin_pad == 4ll * ctx->phase_cin)
@@ -556,7 +566,7 @@ int launch_tc3_tma_dw(dbp_ctx *ctx, const void *codes_nhwc, const void *X, int p
     {
         const unsigned long long dims[2] = {static_cast<unsigned long long>(cin_pad), static_cast<unsigned long long>(s.Cout) * 9};
         const unsigned long long str[1] = {static_cast<unsigned long long>(cin_pad) * 4};
-        const unsigned box[2] = {128, 32};
+        const unsigned box[2] = {p.split ? 64u : 128u, 32};
         if (!encode_map_f32_rows(&map_acc, acc, 2, dims, str, box)) return fail_cuda("tensor map of the dW scratch");
     }
     {
@@ -572,7 +582,7 @@ int launch_tc3_tma_dw(dbp_ctx *ctx, const void *codes_nhwc, const void *X, int p
                                             static_cast<unsigned long long>(s.B) * pieces};
         const unsigned long long str[2] = {static_cast<unsigned long long>(x_pitch) * 2,
                                            static_cast<unsigned long long>(x_pitch) * 2 * s.Cin};
-        const unsigned box[3] = {64, 128, 1};
+        const unsigned box[3] = {64, p.split ? 64u : 128u, 1};
         if (!encode_map_bf16(&map_x, X, 3, dims, str, box)) return fail_cuda("tensor map of the activations");
     }
     auto kern = NP == 2 ? tc3_tma_dw_kernel<2> : tc3_tma_dw_kernel<1>;
