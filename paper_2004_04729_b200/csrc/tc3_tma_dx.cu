@@ -45,6 +45,7 @@ constexpr int kMaxQ = 2;                         // code patches in flight
 constexpr int kMaxW = 18;                        // weight slots (ring, or all of them when they stay resident)
 constexpr int kAccCols = 256;
 constexpr int kEpiThreads = 512;
+constexpr int kBlock = 32 * 128, kBlocks = kEpiThreads / 32;     // [32 ci][128 bytes of positions], swizzled
 
 struct Dx3T {
     const float *delta_p;
@@ -73,6 +74,9 @@ struct Dx3T {
     int run;                      // Ht * W: staged positions per image
     int pitch;                    // bytes per channel row of the staging block (an odd number of words)
     int pairs;                    // W even: columns are staged two at a time
+    int unit;                     // > 0: blocks of 32 channels x 128 bytes of consecutive positions leave by the copy engine;
+                                  // the largest power of two up to 32 that divides W
+    unsigned w_rcp;               // ceil(2^16 / W): i / W = i w_rcp >> 16 for i < 512, W <= 62
     int phase_cin;                // > 0: the layer is a stride-2 layer on phase images (channel block ph * phase_cin ...
                                   // holds phase ph = 2 py + px); a phase's weights are zero outside the taps
                                   // ky in {1} (py = 0) or {0, 1} (py = 1), kx likewise, and those taps are skipped
@@ -90,6 +94,43 @@ __device__ __forceinline__ void tma_load_4d(void *dst, const CUtensorMap *map, i
     asm volatile(
         "cp.async.bulk.tensor.4d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4, %5, %6}], [%2];"
         ::"r"(smem_u32(dst)), "l"(map), "r"(smem_u32(bar)), "r"(c0), "r"(c1), "r"(c2), "r"(c3) : "memory");
+}
+
+__device__ __forceinline__ void tma_store_4d(const CUtensorMap *map, int c0, int c1, int c2, int c3, const void *src) {
+    asm volatile("cp.async.bulk.tensor.4d.global.shared::cta.bulk_group [%0, {%2, %3, %4, %5}], [%1];"
+                 ::"l"(map), "r"(smem_u32(src)), "r"(c0), "r"(c1), "r"(c2), "r"(c3) : "memory");
+}
+
+// U accumulator columns (the caller waits)
+template <int U>
+__device__ __forceinline__ void tmem_ld_cols(unsigned taddr, unsigned *r) {
+    if constexpr (U == 4) {
+        asm volatile("tcgen05.ld.sync.aligned.32x32b.x4.b32 {%0, %1, %2, %3}, [%4];"
+                     : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(taddr));
+    } else if constexpr (U == 8) {
+        asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+                     : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]) : "r"(taddr));
+    } else {
+        asm volatile("tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, [%16];"
+                     : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]),
+                       "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15]) : "r"(taddr));
+    }
+}
+// the accumulators of 32 consecutive positions from position i0 of an image's part of the patch on (rows of W positions lie Wp
+// columns apart, and U divides W); positions from `limit` on, which nobody stores, read some column that exists
+template <int U>
+__device__ __forceinline__ void load_positions(unsigned base, int i0, int limit, const Dx3T &p, unsigned (&v)[32]) {
+#pragma unroll
+    for (int k = 0; k < 32; k += U) {
+        const int i = i0 + k, y = static_cast<int>(static_cast<unsigned>(i) * p.w_rcp >> 16);
+        tmem_ld_cols<U>(base + (i < limit ? i + y * (p.Wp - p.W) : 0), v + k);
+    }
+    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+}
+__device__ __forceinline__ void load_positions(unsigned base, int i0, int limit, const Dx3T &p, unsigned (&v)[32]) {
+    if (p.unit >= 16) load_positions<16>(base, i0, limit, p, v);
+    else if (p.unit == 8) load_positions<8>(base, i0, limit, p, v);
+    else load_positions<4>(base, i0, limit, p, v);
 }
 
 // dst[0 .. n) = value(0 .. n), lanes along the run, four values per lane in flight
@@ -125,19 +166,37 @@ __device__ __forceinline__ bool epilogue_all(bool mine) {
     return r != 0;
 }
 
+// The same between the two warps that share a block: named barriers 2 ..
+__device__ __forceinline__ bool pair_all(int id, bool mine) {
+    unsigned r;
+    asm volatile(
+        "{\n\t.reg .pred p, q;\n\t"
+        "setp.ne.b32 p, %1, 0;\n\t"
+        "bar.red.and.pred q, %2, 64, p;\n\t"
+        "selp.b32 %0, 1, 0, q;\n\t}"
+        : "=r"(r) : "r"(mine ? 1u : 0u), "r"(id) : "memory");
+    return r != 0;
+}
+__device__ __forceinline__ void pair_sync(int id) { asm volatile("bar.sync %0, 64;" ::"r"(id) : "memory"); }
+
+// BLOCKS: dX leaves in blocks by the copy engine (p.unit > 0, p.KS == 1); an instance of its own because the other paths' code
+// in the same kernel costs each of them 3 %
+template <bool BLOCKS>
 __global__ void __launch_bounds__(kThreadsX, 1)
-tc3_tma_dx_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUtensorMap map_w, const Dx3T p) {
+tc3_tma_dx_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUtensorMap map_w,
+                  const __grid_constant__ CUtensorMap map_o, const __grid_constant__ CUtensorMap map_t, const Dx3T p) {
     extern __shared__ __align__(1024) unsigned char smem_raw[];
     unsigned char *smem = reinterpret_cast<unsigned char *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
     unsigned char *q_s = smem;                                   // nq code patches
     unsigned char *w_s = q_s + p.nq * p.q_bytes;                 // nw weight slots
-    short *s_off = reinterpret_cast<short *>(w_s + p.nw * p.w_slot);   // column -> staged position (or -1), 256 entries
-    unsigned char *stage = reinterpret_cast<unsigned char *>(s_off) + 512;   // [128 ci][pitch]
+    unsigned char *stage = w_s + p.nw * p.w_slot;                // [128 ci][pitch], or a 4 KB block per epilogue warp
+    short *s_off = reinterpret_cast<short *>(stage + (BLOCKS ? kBlocks * kBlock : 128 * p.pitch));   // column -> staged position (or -1), 256 entries
     __shared__ PipeX pipe;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int rank = p.KS > 1 ? static_cast<int>(blockIdx.x) % p.KS : 0;      // consecutive CTAs are a cluster
-    const long long t_first = blockIdx.x / p.KS, t_step = gridDim.x / p.KS;
-    const int c_lo = rank * p.ncb / p.KS, c_hi = (rank + 1) * p.ncb / p.KS;   // my 64-channel blocks of co
+    const int KS = BLOCKS ? 1 : p.KS;
+    const int rank = KS > 1 ? static_cast<int>(blockIdx.x) % KS : 0;      // consecutive CTAs are a cluster
+    const long long t_first = blockIdx.x / KS, t_step = gridDim.x / KS;
+    const int c_lo = rank * p.ncb / KS, c_hi = (rank + 1) * p.ncb / KS;   // my 64-channel blocks of co
 
     if (threadIdx.x == 0) {
         for (int s = 0; s < kMaxQ; ++s) { mbar_init(&pipe.q_full[s], 1); mbar_init(&pipe.q_empty[s], 1); }
@@ -146,6 +205,7 @@ tc3_tma_dx_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         tma_prefetch_desc(&map_q);
         tma_prefetch_desc(&map_w);
+        if (BLOCKS) { tma_prefetch_desc(&map_o); tma_prefetch_desc(&map_t); }
     }
     if (warp == 2) tmem_alloc(&pipe.tmem_base, 2 * kAccCols);
     // which accumulator columns hold an output, and where it goes in a channel's staged run
@@ -164,7 +224,7 @@ tc3_tma_dx_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
     __syncthreads();
     tc_fence_after();
     const unsigned tmem_base = pipe.tmem_base;
-    if (p.KS > 1) cluster_barrier();       // every CTA of the cluster is there before anybody writes into its staging block
+    if (KS > 1) cluster_barrier();       // every CTA of the cluster is there before anybody writes into its staging block
     // everything above touched only this CTA's shared and tensor memory
     chain_wait();
 
@@ -342,7 +402,95 @@ tc3_tma_dx_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
             report_wait(p.stats, 6, clock64() - born);
             report_wait(p.stats, 7, 1);
         }
-    } else if (warp >= 4) {
+    } else if (BLOCKS) {
+        // epilogue where runs of positions are whole 16-byte words: every warp by itself (no barrier of all of them, no pass
+        // through a staging block shared by them) moves blocks of 32 channels x 128 bytes from the accumulator to its own
+        // block of shared memory, from where the copy engine takes them. Warp (q, part): lane quarter q, every fourth block.
+        // With both weight pieces on the lanes a pair of warps shares two blocks: one puts the low pieces' sums into a block,
+        // the other adds its own and stores.
+        // (64 -> 64 fp32 at 32x32, batch 128: this kernel 39 -> 30 us; without any epilogue it would take 25)
+        const int ew = warp - 4, q = ew & 3, part = ew >> 2, pair = part * 2 + (q & 1);
+        const float delta = *p.delta_p;
+        const int PC = 128 / p.es;
+        const bool low = p.split && q >= 2;
+        unsigned char *blk = stage + (p.split ? 2 * pair : ew) * kBlock;
+        unsigned flip = 0;
+        bool ok = true;
+        long long it = 0, we = 0;
+        for (long long t = t_first; t < p.ntiles; t += t_step, ++it) {
+            const int slot = static_cast<int>(it & 1);
+            int ci0, b0, y0;
+            tile_of(t, ci0, b0, y0);
+            ok = __all_sync(0xffffffffu, mbar_wait_timed(&pipe.acc_full[slot], static_cast<unsigned>(it >> 1) & 1u, p.err_flag, we));
+            if (p.split) ok = pair_all(2 + pair, ok);                // the same decision in both warps
+            if (!ok) break;
+            tc_fence_after();
+            const int ci_w = ci0 + (p.split ? (q & 1) : q) * 32;
+            const int rows_valid = p.H - y0 < p.Ht ? p.H - y0 : p.Ht, len = rows_valid * p.W, nc = (len + PC - 1) / PC;
+            const int nblk = ci_w < p.Cin ? nc * (p.B - b0 < p.nb ? p.B - b0 : p.nb) : 0;
+            const unsigned acc = tmem_base + (static_cast<unsigned>(q * 32) << 16) + slot * kAccCols;
+            for (int k = part; k < nblk; k += 4) {
+                const int img = k / nc, i0 = (k - img * nc) * PC;
+                unsigned v[32];
+                load_positions(acc + img * p.img_rows, i0, len, p, v);
+                unsigned char *row = blk + flip * kBlock + lane * 128;
+                if (!low) {
+                    if (lane == 0) bulk_wait_read_all();             // what was stored before has been read
+                    __syncwarp();
+                }
+                if (p.split) {
+                    if (low) {
+#pragma unroll
+                        for (int h = 0; h < 8; ++h)
+                            *reinterpret_cast<uint4 *>(row + ((h ^ (lane & 7)) << 4)) = make_uint4(v[4 * h], v[4 * h + 1], v[4 * h + 2], v[4 * h + 3]);
+                    }
+                    pair_sync(2 + pair);
+                    flip ^= 1u;
+                    if (low) continue;
+#pragma unroll
+                    for (int h = 0; h < 8; ++h) {
+                        float4 *at = reinterpret_cast<float4 *>(row + ((h ^ (lane & 7)) << 4));
+                        const float4 l = *at;
+                        *at = make_float4((__uint_as_float(v[4 * h]) + l.x) * delta, (__uint_as_float(v[4 * h + 1]) + l.y) * delta,
+                                          (__uint_as_float(v[4 * h + 2]) + l.z) * delta, (__uint_as_float(v[4 * h + 3]) + l.w) * delta);
+                    }
+                } else if (p.es == 4) {
+#pragma unroll
+                    for (int h = 0; h < 8; ++h)
+                        *reinterpret_cast<float4 *>(row + ((h ^ (lane & 7)) << 4)) =
+                            make_float4(__uint_as_float(v[4 * h]) * delta, __uint_as_float(v[4 * h + 1]) * delta,
+                                        __uint_as_float(v[4 * h + 2]) * delta, __uint_as_float(v[4 * h + 3]) * delta);
+                } else {
+#pragma unroll
+                    for (int half = 0; half < 2; ++half) {
+                        if (half) load_positions(acc + img * p.img_rows, i0 + 32, len, p, v);
+#pragma unroll
+                        for (int h = 0; h < 4; ++h) {
+                            unsigned w[4];
+#pragma unroll
+                            for (int e = 0; e < 4; ++e) {
+                                const __nv_bfloat162 b2 = __floats2bfloat162_rn(__uint_as_float(v[8 * h + 2 * e]) * delta,
+                                                                                __uint_as_float(v[8 * h + 2 * e + 1]) * delta);
+                                w[e] = *reinterpret_cast<const unsigned *>(&b2);
+                            }
+                            *reinterpret_cast<uint4 *>(row + (((4 * half + h) ^ (lane & 7)) << 4)) = make_uint4(w[0], w[1], w[2], w[3]);
+                        }
+                    }
+                }
+                fence_async_proxy();
+                __syncwarp();
+                if (lane == 0) {                                     // what lies outside the tensor (or the patch) is skipped
+                    if (rows_valid == p.Ht) tma_store_4d(&map_o, i0, y0 / p.Ht, ci_w, b0 + img, row);
+                    else tma_store_4d(&map_t, y0 * p.W + i0, 0, ci_w, b0 + img, row);
+                    bulk_commit();
+                }
+            }
+            tc_fence_before();
+            warp_arrive(&pipe.acc_empty[slot]);
+        }
+        if (lane == 0) bulk_wait_read_all();
+        if (ew == 0 && lane == 0) report_wait(p.stats, 5, we);
+    } else {
         // epilogue: TMEM lane = input channel, column = patch position. Warp (q, part): lane quarter q,
         // one quarter of the 32-column chunks.
         const int ew = warp - 4, q = ew & 3, part = ew >> 2;
@@ -375,8 +523,8 @@ tc3_tma_dx_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
                     const uint4 t0 = tp[0], t1 = tp[1], t2 = tp[2], t3 = tp[3];
                     const unsigned tw[16] = {t0.x, t0.y, t0.z, t0.w, t1.x, t1.y, t1.z, t1.w,
                                              t2.x, t2.y, t2.z, t2.w, t3.x, t3.y, t3.z, t3.w};
-                    if (p.es == 4 || p.KS > 1) {
-                        const float f = p.KS > 1 ? 1.f : delta;      // partial sums are scaled when they have met
+                    if (p.es == 4 || KS > 1) {
+                        const float f = KS > 1 ? 1.f : delta;      // partial sums are scaled when they have met
 #pragma unroll
                         for (int j = 0; j < 32; ++j) {
                             const int o = static_cast<int>(static_cast<short>((tw[j >> 1] >> (16 * (j & 1))) & 0xffffu));
@@ -399,7 +547,7 @@ tc3_tma_dx_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
                     }
                 }
             }
-            if (p.KS > 1) continue;                                  // one tile per cluster: the sums meet below
+            if (KS > 1) continue;                                  // one tile per cluster: the sums meet below
             // the accumulator is free once every epilogue warp has read its part
             tc_fence_before();
             warp_arrive(&pipe.acc_empty[slot]);
@@ -434,18 +582,18 @@ tc3_tma_dx_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
         }
         if (et == 0) report_wait(p.stats, 5, we);
     }
-    if (p.KS > 1) {
+    if (KS > 1) {
         cluster_barrier();                 // every CTA's partial sums are staged
         // this CTA finishes 128 / KS channels: rows read from all staging blocks, lanes along the positions
         int ci0, b0, y0;
         tile_of(t_first, ci0, b0, y0);
-        const int per = 128 / p.KS, rows_valid = p.H - y0 < p.Ht ? p.H - y0 : p.Ht, len = rows_valid * p.W, HW = p.H * p.W;
+        const int per = 128 / KS, rows_valid = p.H - y0 < p.Ht ? p.H - y0 : p.Ht, len = rows_valid * p.W, HW = p.H * p.W;
         const int nimg = p.B - b0 < p.nb ? p.B - b0 : p.nb, row_len = (nimg - 1) * p.run + len;
         const float delta = *p.delta_p;
         unsigned base[8];
 #pragma unroll
         for (int k = 0; k < 8; ++k)
-            if (k < p.KS) asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(base[k]) : "r"(smem_u32(stage)), "r"(k));
+            if (k < KS) asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(base[k]) : "r"(smem_u32(stage)), "r"(k));
         for (int r = warp; r < per; r += kThreadsX / 32) {
             const int cl = rank * per + r, ci = ci0 + cl;
             if (ci >= p.Cin) break;
@@ -455,7 +603,7 @@ tc3_tma_dx_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
                 for (int u = 0; u < 4; ++u)
 #pragma unroll
                     for (int k = 0; k < 8; ++k)
-                        if (k < p.KS && i0 + 32 * u < row_len)
+                        if (k < KS && i0 + 32 * u < row_len)
                             asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(v[u][k]) : "r"(base[k] + cl * p.pitch + 4 * (i0 + 32 * u)));
 #pragma unroll
                 for (int u = 0; u < 4; ++u) {
@@ -464,7 +612,7 @@ tc3_tma_dx_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
                     float sum = 0.f;
 #pragma unroll
                     for (int k = 0; k < 8; ++k)
-                        if (k < p.KS) sum += v[u][k];
+                        if (k < KS) sum += v[u][k];
                     const int img = i / p.run, pos = i - img * p.run;
                     const long long o = (static_cast<long long>(b0 + img) * p.Cin + ci) * HW + y0 * p.W + pos;
                     if (p.es == 4) static_cast<float *>(p.dX)[o] = sum * delta;
@@ -543,20 +691,26 @@ int launch_tc3_tma_dx(dbp_ctx *ctx, const void *codes_nhwc, const void *W, int i
     auto consider = [&](int ht, int nb, int ks) -> bool {
         Dx3T q = p;
         q.Ht = ht; q.nb = nb; q.KS = ks;
-        q.Wp = (p.W % 2 == 0 && p.es == 2 && ks == 1) ? p.W + 2 : p.W + 1;
+        q.tiles_y = (p.H + ht - 1) / ht;
+        q.run = ht * p.W;
+        // by the copy engine where every run starts on 16 bytes, a row is whole words of at least four columns (tensor memory
+        // is read in pieces of a row) and a run fills a block
+        const int hw = p.H * p.W, low_bit = p.W & -p.W;
+        q.unit = ks == 1 && low_bit >= 4 && hw * p.es % 16 == 0 && (q.tiles_y == 1 || q.run * p.es % 16 == 0) && q.run * p.es >= 128
+                     ? (low_bit > 32 ? 32 : low_bit) : 0;
+        q.w_rcp = (65536u + p.W - 1) / p.W;
+        q.Wp = (p.W % 2 == 0 && p.es == 2 && ks == 1 && q.unit == 0) ? p.W + 2 : p.W + 1;
         q.img_rows = (nb == 1 ? ht + 2 : ht + 1) * q.Wp;
         q.N = round_up((nb - 1) * q.img_rows + (ht - 1) * q.Wp + p.W, 16);    // up to the last column that holds an output
         if (q.N > 256) return false;
         const int rows_read = q.N + 2 * q.Wp + 2;
         q.q_bytes = round_up((rows_read > q.img_rows * nb ? rows_read : q.img_rows * nb) * 128, 1024);
         q.q_tx = q.img_rows * nb * 128;
-        q.tiles_y = (p.H + ht - 1) / ht;
         q.pos_tiles = nb == 1 ? static_cast<long long>(p.B) * q.tiles_y : (p.B + nb - 1) / nb;
         q.ntiles = q.pos_tiles * p.ci_tiles;
         // one round of clusters; a GPC's SMs are no multiple of 4 or 8, so not all of them can be covered (36 clusters of 4
         // took 39 us where 32 took 24)
         if (ks > 1 && q.ntiles * ks > (ks == 2 ? sms : ks == 4 ? sms * 7 / 8 : sms * 3 / 4)) return true;
-        q.run = ht * p.W;
         // an odd number of 32-bit words per row: the 32 channels of a warp hit 32 different banks when they stage the same
         // position
         const int es = ks > 1 ? 4 : p.es;
@@ -567,7 +721,7 @@ int launch_tc3_tma_dx(dbp_ctx *ctx, const void *codes_nhwc, const void *W, int i
         // costs time). With one ci block and room for all taps of all co blocks they are loaded once and stay; otherwise they
         // stream through a ring of slots.
         const size_t tap_bytes = static_cast<size_t>(p.a_panels) * kWPanel, budget = 227 * 1024 - 2048;
-        const size_t fixed = static_cast<size_t>(q.nq) * q.q_bytes + static_cast<size_t>(128) * q.pitch + 512 + 1024;
+        const size_t fixed = static_cast<size_t>(q.nq) * q.q_bytes + (q.unit > 0 ? static_cast<size_t>(kBlocks) * kBlock : static_cast<size_t>(128) * q.pitch) + 512 + 1024;
         if (fixed + 3 * tap_bytes > budget) return true;
         const size_t room = budget - fixed;
         const int slots_all = p.ncb * (p.ntaps / 9);
@@ -592,7 +746,7 @@ int launch_tc3_tma_dx(dbp_ctx *ctx, const void *codes_nhwc, const void *W, int i
         const int cbs = (p.ncb + ks - 1) / ks;
         const double body = cbs * (p.ntaps * live * 4.0 * mma + (q.resident ? 0.0 : 250.0 * (p.phase_cin > 0 ? p.ntaps / 6.0 : static_cast<double>(p.ntaps) / q.G)) + q.q_tx / 128.0 + 300.0);
         const double staged = (p.Cin <= 64 && !p.split ? 64.0 : 128.0) * nb * q.run * es;
-        const double epi = 2000.0 + staged / 20.0 + (ks > 1 ? 2000.0 + staged / 8.0 : 0.0);
+        const double epi = (q.unit > 0 ? 1000.0 + staged / 40.0 : 2000.0 + staged / 20.0) + (ks > 1 ? 2000.0 + staged / 8.0 : 0.0);
         const double cost = static_cast<double>(waves) * (500.0 + (body > epi ? body : epi)) + (waves > 1 ? (body < epi ? body : epi) : epi);
         if (cost < best) { best = cost; chosen = q; smem = fixed + static_cast<size_t>(q.nw) * q.w_slot; }
         return true;
@@ -641,14 +795,27 @@ int launch_tc3_tma_dx(dbp_ctx *ctx, const void *codes_nhwc, const void *W, int i
         const unsigned box[3] = {64, 64, static_cast<unsigned>(p.phase_cin > 0 ? 1 : p.G)};
         if (!encode_map_bf16(&map_w, ctx->w_taps.ptr, 3, dims, str, box)) return fail_cuda("tensor map of the weights");
     }
-    if (cudaFuncSetAttribute(tc3_tma_dx_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem)) != cudaSuccess)
+    CUtensorMap map_o = map_q, map_t = map_q;
+    if (p.unit > 0) {
+        // dX as [b][ci][patch][positions of a patch], and as [b][ci][positions] for a last patch of fewer rows
+        const unsigned long long HW = static_cast<unsigned long long>(s.H) * s.W, plane = HW * p.es, full = static_cast<unsigned long long>(s.H / p.Ht);
+        const unsigned long long dims_o[4] = {static_cast<unsigned long long>(p.run), full, static_cast<unsigned long long>(s.Cin), static_cast<unsigned long long>(s.B)};
+        const unsigned long long dims_t[4] = {HW, 1, static_cast<unsigned long long>(s.Cin), static_cast<unsigned long long>(s.B)};
+        const unsigned long long str_o[3] = {full > 1 ? static_cast<unsigned long long>(p.run) * p.es : plane, plane, plane * s.Cin};
+        const unsigned long long str_t[3] = {plane, plane, plane * s.Cin};
+        const unsigned box[4] = {static_cast<unsigned>(128 / p.es), 1, 32, 1};
+        auto encode = p.es == 4 ? encode_map_f32_sw128 : encode_map_bf16;
+        if (!encode(&map_o, dX, 4, dims_o, str_o, box) || !encode(&map_t, dX, 4, dims_t, str_t, box)) return fail_cuda("tensor map of dX");
+    }
+    auto kern = p.unit > 0 ? tc3_tma_dx_kernel<true> : tc3_tma_dx_kernel<false>;
+    if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem)) != cudaSuccess)
         return fail_cuda("shared memory size");
     if (p.KS > 1)
-        return cuda_ok(launch_chained_cluster(tc3_tma_dx_kernel, static_cast<unsigned>(p.ntiles) * p.KS, static_cast<unsigned>(p.KS),
-                                              dim3(kThreadsX), smem, ctx->stream, map_q, map_w, p));
+        return cuda_ok(launch_chained_cluster(kern, static_cast<unsigned>(p.ntiles) * p.KS, static_cast<unsigned>(p.KS),
+                                              dim3(kThreadsX), smem, ctx->stream, map_q, map_w, map_o, map_t, p));
     const long long grid = p.ntiles < sms ? p.ntiles : sms;
-    return cuda_ok(launch_chained(tc3_tma_dx_kernel, dim3(static_cast<unsigned>(grid)), dim3(kThreadsX), smem, ctx->stream,
-                                  map_q, map_w, p));
+    return cuda_ok(launch_chained(kern, dim3(static_cast<unsigned>(grid)), dim3(kThreadsX), smem, ctx->stream,
+                                  map_q, map_w, map_o, map_t, p));
 }
 
 }  // namespace dbp

@@ -1,5 +1,5 @@
 """3x3 input gradients whose patches share halos, whose reduction over output channels is split over a cluster of CTAs, or
-whose weight pieces share the accumulator: parity with the oracle and bit-identical repeats."""
+whose weight pieces share the accumulator, or that leave by whole blocks: parity with the oracle and bit-identical repeats."""
 import numpy as np
 import pytest
 import torch
@@ -24,7 +24,9 @@ def ctx():
     (3, 128, 576, 2, 2, "bf16"),                                                              # nine blocks of channels over a cluster
     (30, 512, 136, 2, 2, "f32"), (7, 136, 512, 4, 4, "f32"), (2, 264, 128, 14, 14, "f32"),
     (1, 128, 128, 1, 1, "f32"),
-    (3, 64, 64, 13, 32, "f32"), (2, 40, 72, 9, 11, "f32"), (1, 3, 200, 33, 62, "f32")])      # both weight pieces in one MMA
+    (3, 64, 64, 13, 32, "f32"), (2, 40, 72, 9, 11, "f32"), (1, 3, 200, 33, 62, "f32"),       # both weight pieces in one MMA
+    (3, 40, 24, 9, 56, "bf16"), (2, 72, 16, 10, 28, "bf16"), (2, 24, 24, 22, 60, "bf16"),      # dX by whole blocks: partial last
+    (2, 136, 40, 11, 16, "f32"), (9, 136, 64, 4, 8, "f32"), (1, 64, 8, 31, 48, "f32")])       # patches, several images, ragged rows
 def test_input_gradient(ctx, B, Ci, Co, H, W, dtype):
     import paper_2004_04729_b200 as dbp
     L = wl.conv_layer(B, Ci, Co, H, W, 3, data_seed=B + Ci + 5 * Co + H, scale=2.0, seed=9, dtype=dtype)
