@@ -229,11 +229,15 @@ int launch_tma_dw(dbp_ctx *ctx, const void *codes_bf16, const void *X, int piece
 bool tc3_tma_supported(const ConvShape &s, int io);
 // io: the operands' type; fp32 weights / activations are split into two bf16 pieces on the way in
 // weights_ready: ctx->w_taps already holds the re-laid weights (the statistics kernel did it on the side)
+// lean (may be null): the kernel may confine itself to half of every SM, so that the dW kernel (half) runs beside it; set to
+// whether it did. dX is the same either way.
 int launch_tc3_tma_dx(dbp_ctx *ctx, const void *codes_nhwc, const void *W, int io, const float *delta_p,
-                      const ConvShape &s, void *dX, bool dx_bf16, int *err_flag, bool weights_ready = false);
+                      const ConvShape &s, void *dX, bool dx_bf16, int *err_flag, bool weights_ready = false, bool *lean = nullptr);
+// Dynamic shared memory of a kernel two of whose CTAs share an SM (228 KB, of which a CTA takes 1 KB and the 1 KB of its own variables)
+constexpr size_t kHalfSm = 112 * 1024;
 // X: bf16 planes of x_pitch values, pieces of every image one after the other
 int launch_tc3_tma_dw(dbp_ctx *ctx, const void *codes_nhwc, const void *X, int pieces, long long x_pitch, const float *delta_p,
-                      const ConvShape &s, float *dW, int *err_flag);
+                      const ConvShape &s, float *dW, int *err_flag, bool half = false);
 // fp32 activations split and stacked for it (out: [2][B / G][Cin][pitch]); beside: as for launch_rows_job
 int launch_x_stacked(dbp_ctx *ctx, const float *X, void *out, const ConvShape &s, int stack_g, bool beside);
 // Planes of fewer than 64 positions: how many images of a batch to stack into one tall image (one zero row after

@@ -510,7 +510,7 @@ int launch_x_stacked(dbp_ctx *ctx, const float *X, void *out, const ConvShape &s
 // X: bf16 planes of x_pitch values (a multiple of 8); fp32 activations as two pieces (as if the batch were twice as long).
 // Tiny planes stacked into tall images: `s` describes the tall images and codes and X are their stacked copies.
 int launch_tc3_tma_dw(dbp_ctx *ctx, const void *codes_nhwc, const void *X, int pieces, long long x_pitch, const float *delta_p,
-                      const ConvShape &s, float *dW, int *err_flag) {
+                      const ConvShape &s, float *dW, int *err_flag, bool half) {
     // the scratch's rows are padded to a multiple of 16 bytes
     const long long cin_pad = (s.Cin + 7) / 8 * 8, q_pitch = (s.Cout + 7) / 8 * 8;
     const long long HW = s.H * s.W;
@@ -518,11 +518,14 @@ int launch_tc3_tma_dw(dbp_ctx *ctx, const void *codes_nhwc, const void *X, int p
     p.Cin = static_cast<int>(cin_pad); p.Cout = static_cast<int>(s.Cout); p.W = static_cast<int>(s.W); p.HW = static_cast<int>(HW);
     p.err_flag = err_flag;
     p.stats = ctx->wait_stats;
-    const int NP = s.Cout > 64 ? 2 : 1;
+    // half an SM has room for the 192 accumulator columns of 64 output channels (an MMA of N = 192 does as much per clock as
+    // three of 128); splits are still chosen for one CTA per SM, because every split adds its accumulators into the scratch
+    // (for two: 2 % slower on average over 60 drawn layers)
+    const int NP = s.Cout > 64 && !half ? 2 : 1;
     p.ci_tiles = static_cast<int>((cin_pad + 127) / 128);
     p.co_tiles = static_cast<int>((s.Cout + 64 * NP - 1) / (64 * NP));
     // the longest segment whose two code buffers fit beside at least three activation slots
-    const size_t budget = 227 * 1024 - 2048;
+    const size_t budget = half ? kHalfSm : 227 * 1024 - 2048;
     const int seg_cap = static_cast<int>(HW < 512 ? (HW + 63) / 64 * 64 : 512);
     size_t smem = 0;
     for (int seg = seg_cap; seg >= 64; seg -= 64) {
@@ -530,13 +533,14 @@ int launch_tc3_tma_dw(dbp_ctx *ctx, const void *codes_nhwc, const void *X, int p
         const int nload = (rows + 255) / 256, rows_box = (rows + nload - 1) / nload;
         const int panel = round_up(nload * rows_box * 128, 1024);
         const size_t fixed = 2 * static_cast<size_t>(NP) * panel + 1024;
-        if (fixed + 3 * kXSlot > budget) continue;
+        if (fixed + (half ? 2 : 3) * kXSlot > budget) continue;
         p.SEG = seg; p.nload = nload; p.rows_box = rows_box; p.panel_bytes = panel;
         p.nx = static_cast<int>((budget - fixed) / kXSlot);
         if (p.nx > kMaxNX) p.nx = kMaxNX;
         smem = fixed + static_cast<size_t>(p.nx) * kXSlot;
         break;
     }
+    if (smem == 0 && half) return launch_tc3_tma_dw(ctx, codes_nhwc, X, pieces, x_pitch, delta_p, s, dW, err_flag, false);
     if (smem == 0) return DBP_EUNSUPPORTED;
     p.segs_per_img = (p.HW + p.SEG - 1) / p.SEG;
     p.code_batch = static_cast<int>(s.B);
@@ -585,6 +589,7 @@ int launch_tc3_tma_dw(dbp_ctx *ctx, const void *codes_nhwc, const void *X, int p
         const unsigned box[3] = {64, p.split ? 64u : 128u, 1};
         if (!encode_map_bf16(&map_x, X, 3, dims, str, box)) return fail_cuda("tensor map of the activations");
     }
+    if (half) cudaFuncSetAttribute(tc3_tma_dw_kernel<1>, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
     auto kern = NP == 2 ? tc3_tma_dw_kernel<2> : tc3_tma_dw_kernel<1>;
     if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem)) != cudaSuccess)
         return fail_cuda("shared memory size");

@@ -39,13 +39,15 @@ namespace {
 
 using namespace tc;
 
-constexpr int kThreadsX = 20 * 32;               // copy, copy, MMA, MMA, sixteen epilogue warps
+template <bool LEAN>
+constexpr int kEpiWarps = LEAN ? 8 : 16;
+template <bool LEAN>
+constexpr int kThreads3 = (4 + kEpiWarps<LEAN>) * 32;            // copy, copy, MMA, MMA, epilogue warps
 constexpr int kWPanel = 8192;                    // [64 co][64 ci] bf16
 constexpr int kMaxQ = 2;                         // code patches in flight
 constexpr int kMaxW = 18;                        // weight slots (ring, or all of them when they stay resident)
 constexpr int kAccCols = 256;
-constexpr int kEpiThreads = 512;
-constexpr int kBlock = 32 * 128, kBlocks = kEpiThreads / 32;     // [32 ci][128 bytes of positions], swizzled
+constexpr int kBlock = 32 * 128;                 // one epilogue warp's [32 ci][128 bytes of positions], swizzled
 
 struct Dx3T {
     const float *delta_p;
@@ -72,6 +74,7 @@ struct Dx3T {
     int nq, nw;                   // ring sizes
     int resident;                 // the weights of all taps and co blocks stay in shared memory (one ci block)
     int run;                      // Ht * W: staged positions per image
+    int off_at;                   // where the column table lies
     int pitch;                    // bytes per channel row of the staging block (an odd number of words)
     int pairs;                    // W even: columns are staged two at a time
     int unit;                     // > 0: blocks of 32 channels x 128 bytes of consecutive positions leave by the copy engine;
@@ -155,6 +158,7 @@ __device__ __forceinline__ void cluster_barrier() {
 
 // Barrier over the epilogue threads that also tells every one of them whether all of them are
 // still fine: a thread whose bounded wait ran out arrives like the others, so nobody is left waiting.
+template <int THREADS>
 __device__ __forceinline__ bool epilogue_all(bool mine) {
     unsigned r;
     asm volatile(
@@ -162,7 +166,7 @@ __device__ __forceinline__ bool epilogue_all(bool mine) {
         "setp.ne.b32 p, %1, 0;\n\t"
         "bar.red.and.pred q, 1, %2, p;\n\t"
         "selp.b32 %0, 1, 0, q;\n\t}"
-        : "=r"(r) : "r"(mine ? 1u : 0u), "n"(kEpiThreads) : "memory");
+        : "=r"(r) : "r"(mine ? 1u : 0u), "n"(THREADS) : "memory");
     return r != 0;
 }
 
@@ -181,16 +185,20 @@ __device__ __forceinline__ void pair_sync(int id) { asm volatile("bar.sync %0, 6
 
 // BLOCKS: dX leaves in blocks by the copy engine (p.unit > 0, p.KS == 1); an instance of its own because the other paths' code
 // in the same kernel costs each of them 3 %
-template <bool BLOCKS>
-__global__ void __launch_bounds__(kThreadsX, 1)
+// LEAN: half an SM (shared memory, tensor memory, registers): one tile per CTA, a dW CTA beside it
+template <bool BLOCKS, bool LEAN>
+__global__ void __launch_bounds__(kThreads3<LEAN>, LEAN ? 2 : 1)
 tc3_tma_dx_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUtensorMap map_w,
                   const __grid_constant__ CUtensorMap map_o, const __grid_constant__ CUtensorMap map_t, const Dx3T p) {
+    constexpr int kThreadsX = kThreads3<LEAN>, EW = kEpiWarps<LEAN>, kEpiThreads = EW * 32, PARTS = EW / 4;
+    constexpr unsigned kTmem = LEAN ? kAccCols : 2 * kAccCols;
     extern __shared__ __align__(1024) unsigned char smem_raw[];
     unsigned char *smem = reinterpret_cast<unsigned char *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
     unsigned char *q_s = smem;                                   // nq code patches
     unsigned char *w_s = q_s + p.nq * p.q_bytes;                 // nw weight slots
-    unsigned char *stage = w_s + p.nw * p.w_slot;                // [128 ci][pitch], or a 4 KB block per epilogue warp
-    short *s_off = reinterpret_cast<short *>(stage + (BLOCKS ? kBlocks * kBlock : 128 * p.pitch));   // column -> staged position (or -1), 256 entries
+    // one tile per CTA: the staging block lies over the operands, which nobody reads any more by then
+    unsigned char *stage = LEAN ? smem : w_s + p.nw * p.w_slot;  // [128 ci][pitch], or a 4 KB block per epilogue warp
+    short *s_off = reinterpret_cast<short *>(LEAN ? smem + p.off_at : stage + (BLOCKS ? EW * kBlock : 128 * p.pitch));   // column -> staged position (or -1), 256 entries
     __shared__ PipeX pipe;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int KS = BLOCKS ? 1 : p.KS;
@@ -207,7 +215,7 @@ tc3_tma_dx_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
         tma_prefetch_desc(&map_w);
         if (BLOCKS) { tma_prefetch_desc(&map_o); tma_prefetch_desc(&map_t); }
     }
-    if (warp == 2) tmem_alloc(&pipe.tmem_base, 2 * kAccCols);
+    if (warp == 2) tmem_alloc(&pipe.tmem_base, kTmem);
     // which accumulator columns hold an output, and where it goes in a channel's staged run
     if (threadIdx.x >= 128 && threadIdx.x < 384) {
         const int n = threadIdx.x - 128;
@@ -429,7 +437,7 @@ tc3_tma_dx_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
             const int rows_valid = p.H - y0 < p.Ht ? p.H - y0 : p.Ht, len = rows_valid * p.W, nc = (len + PC - 1) / PC;
             const int nblk = ci_w < p.Cin ? nc * (p.B - b0 < p.nb ? p.B - b0 : p.nb) : 0;
             const unsigned acc = tmem_base + (static_cast<unsigned>(q * 32) << 16) + slot * kAccCols;
-            for (int k = part; k < nblk; k += 4) {
+            for (int k = part; k < nblk; k += PARTS) {
                 const int img = k / nc, i0 = (k - img * nc) * PC;
                 unsigned v[32];
                 load_positions(acc + img * p.img_rows, i0, len, p, v);
@@ -492,11 +500,11 @@ tc3_tma_dx_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
         if (ew == 0 && lane == 0) report_wait(p.stats, 5, we);
     } else {
         // epilogue: TMEM lane = input channel, column = patch position. Warp (q, part): lane quarter q,
-        // one quarter of the 32-column chunks.
+        // its share of the 32-column chunks.
         const int ew = warp - 4, q = ew & 3, part = ew >> 2;
         const int et = threadIdx.x - 128;                           // 0 .. 511
         const float delta = *p.delta_p;
-        const int nchunk = (p.N + 31) >> 5, ch_lo = (nchunk * part + 3) >> 2, ch_hi = (nchunk * (part + 1) + 3) >> 2;
+        const int nchunk = (p.N + 31) >> 5, ch_lo = (nchunk * part + PARTS - 1) >> (LEAN ? 1 : 2), ch_hi = (nchunk * (part + 1) + PARTS - 1) >> (LEAN ? 1 : 2);
         const int HW = p.H * p.W;
         bool ok = true;
         long long it = 0;
@@ -506,7 +514,7 @@ tc3_tma_dx_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
             const unsigned uses = static_cast<unsigned>(it >> 1);
             int ci0, b0, y0;
             tile_of(t, ci0, b0, y0);
-            ok = epilogue_all(mbar_wait_timed(&pipe.acc_full[slot], uses & 1u, p.err_flag, we));
+            ok = epilogue_all<kEpiThreads>(mbar_wait_timed(&pipe.acc_full[slot], uses & 1u, p.err_flag, we));
             if (!ok) break;                                          // the same decision in every epilogue thread
             tc_fence_after();
             const int ci_l = q * 32 + lane;
@@ -626,7 +634,7 @@ tc3_tma_dx_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
     __syncthreads();
     if (warp == 2) {
         __syncwarp();
-        tmem_dealloc(tmem_base, 2 * kAccCols);
+        tmem_dealloc(tmem_base, kTmem);
     }
 }
 
@@ -663,7 +671,7 @@ bool tc3_tma_supported(const ConvShape &s, int io) {
 
 // DBP_EUNSUPPORTED: the shape does not fit (the caller uses another kernel)
 int launch_tc3_tma_dx(dbp_ctx *ctx, const void *codes_nhwc, const void *W, int io, const float *delta_p,
-                      const ConvShape &s, void *dX, bool dx_bf16, int *err_flag, bool weights_ready) {
+                      const ConvShape &s, void *dX, bool dx_bf16, int *err_flag, bool weights_ready, bool *lean) {
     if (!tc3_tma_supported(s, io)) return DBP_EUNSUPPORTED;
     Dx3T p{};
     p.delta_p = delta_p; p.dX = dX; p.dx_f32 = dx_bf16 ? 0 : 1;
@@ -685,6 +693,8 @@ int launch_tc3_tma_dx(dbp_ctx *ctx, const void *codes_nhwc, const void *W, int i
     size_t smem = 0;
     double best = 1e300;
     Dx3T chosen{};
+    bool small = false;
+    int wide_ks = 1;
     // The cheapest of the candidate patches (rows of one image, or several whole images) and reduction splits by a count of
     // clocks (see the head of this file; 6 KB per clock is about what the L2 delivers to all SMs together). Returns whether the
     // patch still fits the accumulator.
@@ -711,6 +721,7 @@ int launch_tc3_tma_dx(dbp_ctx *ctx, const void *codes_nhwc, const void *W, int i
         // one round of clusters; a GPC's SMs are no multiple of 4 or 8, so not all of them can be covered (36 clusters of 4
         // took 39 us where 32 took 24)
         if (ks > 1 && q.ntiles * ks > (ks == 2 ? sms : ks == 4 ? sms * 7 / 8 : sms * 3 / 4)) return true;
+        if (small && (q.ntiles * ks > sms || ks != wide_ks)) return true;      // (the order of a sum does not depend on what else is asked for)
         // an odd number of 32-bit words per row: the 32 channels of a warp hit 32 different banks when they stage the same
         // position
         const int es = ks > 1 ? 4 : p.es;
@@ -720,8 +731,11 @@ int launch_tc3_tma_dx(dbp_ctx *ctx, const void *codes_nhwc, const void *W, int i
         // Weights: a slot holds G taps and is handed over with one barrier (the hand-over, not the copy instruction, is what
         // costs time). With one ci block and room for all taps of all co blocks they are loaded once and stay; otherwise they
         // stream through a ring of slots.
-        const size_t tap_bytes = static_cast<size_t>(p.a_panels) * kWPanel, budget = 227 * 1024 - 2048;
-        const size_t fixed = static_cast<size_t>(q.nq) * q.q_bytes + (q.unit > 0 ? static_cast<size_t>(kBlocks) * kBlock : static_cast<size_t>(128) * q.pitch) + 512 + 1024;
+        const size_t tap_bytes = static_cast<size_t>(p.a_panels) * kWPanel, budget = small ? kHalfSm : 227 * 1024 - 2048;
+        const size_t rings = static_cast<size_t>(q.nq) * q.q_bytes;
+        const size_t staging = (q.unit > 0 ? static_cast<size_t>(small ? kEpiWarps<true> : kEpiWarps<false>) * kBlock : static_cast<size_t>(128) * q.pitch);
+        const size_t fixed = rings + (small ? 0 : staging) + 512 + 1024;
+        if (small && staging + 512 + 1024 > budget) return true;
         if (fixed + 3 * tap_bytes > budget) return true;
         const size_t room = budget - fixed;
         const int slots_all = p.ncb * (p.ntaps / 9);
@@ -748,17 +762,42 @@ int launch_tc3_tma_dx(dbp_ctx *ctx, const void *codes_nhwc, const void *W, int i
         const double staged = (p.Cin <= 64 && !p.split ? 64.0 : 128.0) * nb * q.run * es;
         const double epi = (q.unit > 0 ? 1000.0 + staged / 40.0 : 2000.0 + staged / 20.0) + (ks > 1 ? 2000.0 + staged / 8.0 : 0.0);
         const double cost = static_cast<double>(waves) * (500.0 + (body > epi ? body : epi)) + (waves > 1 ? (body < epi ? body : epi) : epi);
-        if (cost < best) { best = cost; chosen = q; smem = fixed + static_cast<size_t>(q.nw) * q.w_slot; }
+        if (cost < best) {
+            best = cost;
+            const size_t operands = rings + static_cast<size_t>(q.nw) * q.w_slot, over = operands > staging ? operands : staging;
+            q.off_at = static_cast<int>(small ? over : operands + staging);
+            chosen = q;
+            smem = q.off_at + 512 + 1024;
+        }
         return true;
     };
-    for (int ht = 1; ht <= p.H; ++ht)
-        if (!consider(ht, 1, 1)) break;
-    for (int ks = 1; ks <= 8; ks *= 2) {
-        if (ks > p.ncb || (ks > 1 && p.split)) break;
-        for (int nb = ks > 1 ? 1 : 2; nb <= 64 && nb <= p.B; ++nb)
-            if (!consider(p.H, nb, ks)) break;
-    }
+    auto search = [&] {
+        for (int ht = 1; ht <= p.H; ++ht)
+            if (!consider(ht, 1, 1)) break;
+        for (int ks = 1; ks <= 8; ks *= 2) {
+            if (ks > p.ncb || (ks > 1 && p.split)) break;
+            for (int nb = ks > 1 ? 1 : 2; nb <= 64 && nb <= p.B; ++nb)
+                if (!consider(p.H, nb, ks)) break;
+        }
+    };
+    search();
     if (smem == 0) return DBP_EUNSUPPORTED;
+    // Half an SM's worth of it, when the caller can use the other half: only with one round of CTAs (then the staging block can
+    // lie over the operands), and not for phase images, whose slots of two taps do not fit
+    const bool one_wave = chosen.ntiles * chosen.KS <= sms;
+    if (lean != nullptr) {
+        const Dx3T wide = chosen;
+        const size_t wide_smem = smem;
+        if (one_wave && p.phase_cin == 0) {
+            small = true;
+            wide_ks = wide.KS;
+            best = 1e300;
+            smem = 0;
+            search();
+        }
+        *lean = small = small && smem != 0;
+        if (!small) { chosen = wide; smem = wide_smem; }
+    }
     p = chosen;
 
     // re-laid weights
@@ -807,14 +846,17 @@ int launch_tc3_tma_dx(dbp_ctx *ctx, const void *codes_nhwc, const void *W, int i
         auto encode = p.es == 4 ? encode_map_f32_sw128 : encode_map_bf16;
         if (!encode(&map_o, dX, 4, dims_o, str_o, box) || !encode(&map_t, dX, 4, dims_t, str_t, box)) return fail_cuda("tensor map of dX");
     }
-    auto kern = p.unit > 0 ? tc3_tma_dx_kernel<true> : tc3_tma_dx_kernel<false>;
+    auto kern = small ? (p.unit > 0 ? tc3_tma_dx_kernel<true, true> : tc3_tma_dx_kernel<false, true>)
+                      : (p.unit > 0 ? tc3_tma_dx_kernel<true, false> : tc3_tma_dx_kernel<false, false>);
+    const int threads = small ? kThreads3<true> : kThreads3<false>;
+    if (small) cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
     if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem)) != cudaSuccess)
         return fail_cuda("shared memory size");
     if (p.KS > 1)
         return cuda_ok(launch_chained_cluster(kern, static_cast<unsigned>(p.ntiles) * p.KS, static_cast<unsigned>(p.KS),
-                                              dim3(kThreadsX), smem, ctx->stream, map_q, map_w, map_o, map_t, p));
+                                              dim3(threads), smem, ctx->stream, map_q, map_w, map_o, map_t, p));
     const long long grid = p.ntiles < sms ? p.ntiles : sms;
-    return cuda_ok(launch_chained(kern, dim3(static_cast<unsigned>(grid)), dim3(kThreadsX), smem, ctx->stream,
+    return cuda_ok(launch_chained(kern, dim3(static_cast<unsigned>(grid)), dim3(threads), smem, ctx->stream,
                                   map_q, map_w, map_o, map_t, p));
 }
 

@@ -25,6 +25,7 @@ def ctx():
     (30, 512, 136, 2, 2, "f32"), (7, 136, 512, 4, 4, "f32"), (2, 264, 128, 14, 14, "f32"),
     (1, 128, 128, 1, 1, "f32"),
     (3, 64, 64, 13, 32, "f32"), (2, 40, 72, 9, 11, "f32"), (1, 3, 200, 33, 62, "f32"),       # both weight pieces in one MMA
+    (9, 40, 72, 6, 24, "bf16"), (5, 200, 72, 6, 25, "f32"), (40, 130, 136, 5, 5, "f32"),       # dX and dW share every SM, or not
     (3, 40, 24, 9, 56, "bf16"), (2, 72, 16, 10, 28, "bf16"), (2, 24, 24, 22, 60, "bf16"),      # dX by whole blocks: partial last
     (2, 136, 40, 11, 16, "f32"), (9, 136, 64, 4, 8, "f32"), (1, 64, 8, 31, 48, "f32")])       # patches, several images, ragged rows
 def test_input_gradient(ctx, B, Ci, Co, H, W, dtype):
