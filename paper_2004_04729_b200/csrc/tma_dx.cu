@@ -232,7 +232,6 @@ tma_dx_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constant__
         long long it = 0;
         long long we = 0;
         const float delta = *p.delta_p;
-        const int vw = (p.HW % 8 == 0) ? 8 : ((p.HW % 4 == 0) ? 4 : 1);
         unsigned char *stage = smem + kRing + (warp - 2) * kStageOut;
         const int part = (warp - 2) >> 2;          // which chunks of a tile this warp drains
         for (long long t = blockIdx.x; t < p.ntiles && ok; t += gridDim.x, ++it) {
@@ -291,7 +290,8 @@ tma_dx_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constant__
                     continue;
                 }
                 const int nv = p.HW - p0 < 64 ? p.HW - p0 : 64;           // valid positions of the chunk
-                const bool rows128 = nv == 64 && vw >= 4;                 // staged as swizzled 128-byte rows
+                // planes of less than a chunk, one after the other without a gap: packed; else staged as swizzled 128-byte rows
+                const bool packed = p.chunks_per_img == 1 && nv < 64 && (p.Cin & 7) == 0;
 #pragma unroll 1
                 for (int half = 0; half < 2; ++half) {
                     const int pp = p0 + half * 32;
@@ -325,8 +325,8 @@ tma_dx_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constant__
                         }
                     } else {
                         // bf16: my 32 values go to the warp's staging block, which holds the chunk
-                        // as [32 channels][nv positions] (16-byte pieces XOR-swizzled by the row
-                        // when a row is 128 bytes, packed rows otherwise)
+                        // as [32 channels][nv positions] (packed, or 128-byte rows with their 16-byte pieces
+                        // XOR-swizzled by the row)
                         unsigned w[16];
 #pragma unroll
                         for (int j = 0; j < 16; ++j) {
@@ -334,7 +334,7 @@ tma_dx_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constant__
                                                                            __uint_as_float(v[2 * j + 1]) * delta);
                             w[j] = *reinterpret_cast<const unsigned *>(&h);
                         }
-                        if (rows128) {
+                        if (!packed) {
 #pragma unroll
                             for (int j = 0; j < 4; ++j)
                                 *reinterpret_cast<uint4 *>(stage + lane * 128 + (((half * 4 + j) ^ (lane & 7)) << 4)) =
@@ -348,21 +348,19 @@ tma_dx_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constant__
                     }
                 }
                 if (!p.dx_f32) {
-                    // staging block -> dX with lanes along the positions: full 128-byte rows, or, when
-                    // the chunk is the whole plane, one contiguous run of 32 channels x HW positions
+                    // staging block -> dX with lanes along the positions: 8-byte pieces where every row starts on 8 bytes,
+                    // else words, shifted by one position in the rows that start between words (55 x 24 -> 56 channels at
+                    // 39x41: this kernel 80 -> 32 us; element by element before, all lanes on the same banks). When the
+                    // chunk is the whole plane: one contiguous run of 32 channels x HW positions
                     __syncwarp();
                     const int nrows = p.Cin - ci_w < 32 ? p.Cin - ci_w : 32;
                     __nv_bfloat16 *base = static_cast<__nv_bfloat16 *>(p.dX) + (b * p.Cin + ci_w) * p.HW + p0;
                     if (nrows > 0) {
-                        if (rows128 && vw == 8) {
-#pragma unroll
-                            for (int r0 = 0; r0 < 32; r0 += 4) {
-                                const int r = r0 + (lane >> 3), ch = lane & 7;
-                                if (r < nrows)
-                                    *reinterpret_cast<uint4 *>(base + static_cast<long long>(r) * p.HW + ch * 8) =
-                                        *reinterpret_cast<const uint4 *>(stage + r * 128 + ((ch ^ (r & 7)) << 4));
-                            }
-                        } else if (rows128) {
+                        if (packed) {
+                            const int n16 = nrows * nv / 8;          // nrows is a multiple of 8: whole 16-byte pieces
+                            for (int i = lane; i < n16; i += 32)
+                                reinterpret_cast<uint4 *>(base)[i] = reinterpret_cast<const uint4 *>(stage)[i];
+                        } else if (p.HW % 4 == 0 && nv == 64) {
 #pragma unroll
                             for (int r0 = 0; r0 < 32; r0 += 2) {
                                 const int r = r0 + (lane >> 4), pc = lane & 15;
@@ -370,23 +368,31 @@ tma_dx_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constant__
                                     *reinterpret_cast<uint2 *>(base + static_cast<long long>(r) * p.HW + pc * 4) =
                                         *reinterpret_cast<const uint2 *>(stage + r * 128 + (((pc >> 1) ^ (r & 7)) << 4) + (pc & 1) * 8);
                             }
-                        } else if (p.chunks_per_img == 1 && (p.Cin & 7) == 0) {
-                            const int n16 = nrows * nv / 8;          // nrows is a multiple of 8: whole 16-byte pieces
-                            for (int i = lane; i < n16; i += 32)
-                                reinterpret_cast<uint4 *>(base)[i] = reinterpret_cast<const uint4 *>(stage)[i];
-                        } else if (vw >= 4) {
+                        } else if (p.HW % 4 == 0) {
                             const int per_row = nv / 4, n8 = nrows * per_row;
                             for (int i = lane; i < n8; i += 32) {
                                 const int r = i / per_row, c4 = i - r * per_row;
                                 *reinterpret_cast<uint2 *>(base + static_cast<long long>(r) * p.HW + c4 * 4) =
-                                    reinterpret_cast<const uint2 *>(stage)[i];
+                                    *reinterpret_cast<const uint2 *>(stage + r * 128 + (((c4 >> 1) ^ (r & 7)) << 4) + (c4 & 1) * 8);
                             }
                         } else {
-                            const int n2 = nrows * nv;
-                            for (int i = lane; i < n2; i += 32) {
-                                const int r = i / nv, c1 = i - r * nv;
-                                reinterpret_cast<unsigned short *>(base + static_cast<long long>(r) * p.HW)[c1] =
-                                    reinterpret_cast<const unsigned short *>(stage)[i];
+                            for (int r0 = 0; r0 < nrows; r0 += 8) {
+                                unsigned x[8];
+#pragma unroll
+                                for (int i = 0; i < 8; ++i)
+                                    x[i] = *reinterpret_cast<const unsigned *>(stage + (r0 + i) * 128 + (((lane >> 2) ^ i) << 4) + (lane & 3) * 4);
+#pragma unroll
+                                for (int i = 0; i < 8; ++i) {
+                                    __nv_bfloat16 *row = base + static_cast<long long>(r0 + i) * p.HW;
+                                    const int odd = static_cast<int>(reinterpret_cast<uintptr_t>(row) >> 1) & 1, at = 2 * lane + odd;
+                                    const unsigned up = __shfl_down_sync(0xffffffffu, x[i], 1);
+                                    const unsigned w = odd ? __funnelshift_r(x[i], up, 16) : x[i];
+                                    if (r0 + i < nrows) {
+                                        if (at + 1 < nv) *reinterpret_cast<unsigned *>(row + at) = w;
+                                        else if (at < nv) *reinterpret_cast<unsigned short *>(row + at) = static_cast<unsigned short>(w);
+                                        if (odd && lane == 0) *reinterpret_cast<unsigned short *>(row) = static_cast<unsigned short>(x[i]);
+                                    }
+                                }
                             }
                         }
                     }
