@@ -159,7 +159,7 @@ typedef enum {
     DBP_K_DW = 4,         /* sparse weight-gradient product */
     DBP_K_DB = 5,         /* bias gradient */
     DBP_K_DECODE = 6,     /* sparse -> dense codes */
-    DBP_K_GLUE = 7,       /* ReLU derivative / max-pool routing */
+    DBP_K_GLUE = 7,       /* ReLU derivative, max-pool routing, re-laid activations, stride-2 layouts */
     DBP_K_DX_DENSE = 8,   /* tensor-core input-gradient product */
     DBP_K_DW_DENSE = 9,   /* tensor-core weight-gradient product (with its split-K reduction) */
     DBP_K_FUSED = 10,     /* whole backward pass of a small fp32 linear layer (two chained launches); quantization and
@@ -233,9 +233,9 @@ int nsd_decode_dense(dbp_ctx *ctx, const dbp_sparse *q, int8_t *codes);
  * is of dtype `io` (fp32 with DBP_DX_F32). Any of dW, dX, db may be NULL (skipped).
  * q_out may be NULL; otherwise it receives the sparse structure (arrays sized for B*N).
  * Outputs are overwritten, not accumulated.
- * fp32 layers with B*N <= 2^17, no q_out and no FORCE flag run as two chained kernels (statistics, dither
- * and quantization; then the products; profiling kind DBP_K_FUSED): same results to the same tolerances,
- * Delta and nnz through dbp_last_step.
+ * Small fp32 layers (at most 2^17 gradient elements, products of no more tiles than the GPU has SMs), no q_out and no
+ * FORCE flag, run as two chained kernels (statistics, dither and quantization; then the products; profiling kind
+ * DBP_K_FUSED): same results to the same tolerances, Delta and nnz through dbp_last_step.
  */
 int dithered_linear_backward(dbp_ctx *ctx, const void *delta, const void *X, const void *W,
                              int io, long long B, long long N, long long K,
@@ -246,7 +246,7 @@ int dithered_linear_backward(dbp_ctx *ctx, const void *delta, const void *X, con
 /*
  * The same for a convolution layer ("analogous for convolutional layers", Section 3):
  * cross-correlation, NCHW, square kernel k in {1, 3}, stride 1 or 2, zero padding (k-1)/2; also k = 5 with
- * stride 1 and padding 2 (the 5x5 layers of LeNet-5-like networks; these run on the gather kernels only).
+ * stride 1 and padding 2 (the 5x5 layers of LeNet-5-like networks; FMAs on the dense codes, no tensor cores).
  * H and Wd are the height and width of X. Stride 1: delta [B,Cout,H,W], X [B,Cin,H,W], W [Cout,Cin,k,k]:
  *     dX[b,ci,y,x]     = Delta sum_{co,ky,kx} q[b,co,y-ky+p,x-kx+p] W[co,ci,ky,kx]
  *     dW[co,ci,ky,kx]  = Delta sum_{b,y,x}    q[b,co,y,x] X[b,ci,y+ky-p,x+kx-p]
@@ -255,8 +255,8 @@ int dithered_linear_backward(dbp_ctx *ctx, const void *delta, const void *X, con
  * delta [B,Cout,H/2,W/2] is the gradient at the layer's own output positions, X and dX stay [B,Cin,H,W]:
  *     dW[co,ci,ky,kx]  = Delta sum_{b,y,x} q[b,co,y,x] X[b,ci,2y+ky-p,2x+kx-p]
  *     dX[b,ci,y',x']   = Delta sum of q[b,co,y,x] W[co,ci,ky,kx] over the (co,ky,kx,y,x) with 2y+ky-p = y', 2x+kx-p = x'
- * computed as the stride-1 layer on the four phase images of X (layout kernels on the context's stream around
- * the same quantizer and product kernels; workspaces of the size of X, dX and 4x the weights). Such a call always
+ * computed as the stride-1 layer on the four phase images of X (re-laid beside the quantizer, as the rows the dW kernels
+ * read; dX leaves the phase layout beside dW; workspaces of the size of X, dX and 4x the weights). Such a call always
  * joins its weight-gradient kernels before it returns (DBP_DW_ASYNC is ignored). q_out describes delta as given.
  * Other k, stride or pad return DBP_EUNSUPPORTED.
  */
@@ -289,9 +289,9 @@ int dithered_conv_backward_host(dbp_ctx *ctx, const void *delta, const void *X, 
  * (DEVICE, one byte per element of delta, non-zero where z > 0; must stay valid until that call's kernels have
  * run) makes the next dithered_linear_backward / dithered_conv_backward on this context treat its `delta`
  * argument as delta_a and quantize delta_a (.) mask. fp32 only (DBP_EUNSUPPORTED otherwise, at that call).
- * Small linear layers and fp32 3x3 layers on the tensor-core kernels apply the mask while they read delta_a
- * (no extra pass, no delta_z in memory; the mask must then start on a 4-byte boundary, else the next form is
- * taken); other layers run the ReLU-derivative kernel into a workspace first. The setting is consumed by that one call.
+ * Every layer's kernels apply the mask while they read delta_a (no extra pass, no delta_z in memory). A mask that does
+ * not start on a 4-byte boundary, and a call with q_out, run the ReLU-derivative kernel into a workspace first. The
+ * setting is consumed by that one call.
  * mask = NULL clears it.
  */
 int dbp_set_relu_mask(dbp_ctx *ctx, const uint8_t *mask);

@@ -460,7 +460,7 @@ int conv_backward_impl(dbp_ctx *ctx, const void *delta, const void *X, const voi
     const bool forked = dX && dW && ctx->aux != nullptr;
     const bool late_x = ctx->hook_before_dw != nullptr;
     auto write_x = [&](bool beside) -> int {
-        KernelTimer t(ctx, DBP_K_DW_DENSE);
+        KernelTimer t(ctx, DBP_K_GLUE);          // not with the dW kind: bracketing that must not put events between the caller's kernels
         if (st2) return launch_phase_rows(ctx, st2->X, ctx->x_padded[k].ptr, io, s.B, st2->Cin, st2->H, st2->W, st2->phases, x_pitch, beside);
         return stack_g > 0 ? launch_x_stacked(ctx, static_cast<const float *>(X), ctx->x_padded[k].ptr, s, stack_g, beside)
                            : launch_rows_job(ctx, RowsJob{X, ctx->x_padded[k].ptr, io == DBP_F32, s.B * s.Cin, s.H * s.W, x_pitch}, beside);
