@@ -115,7 +115,9 @@ int quantize_for_products(dbp_ctx *ctx, const void *delta, int dtype, long long 
         }
         void *pn = nullptr;
         if (nhwc) {
-            if ((rc = ws_reserve(ctx, ctx->codes_nhwc[k], static_cast<size_t>(numel) * 2 + 1024))) return rc;
+            // rows of the output channels rounded up to 16 bytes: the pitch the quantizer writes and every reader steps by
+            const size_t rows = static_cast<size_t>(nhwc->B) * nhwc->H * nhwc->W;
+            if ((rc = ws_reserve(ctx, ctx->codes_nhwc[k], rows * linear_pitch(nhwc->Cout) * 2 + 1024))) return rc;
             pn = ctx->codes_nhwc[k].ptr;
             *codes_nhwc = pn;
         }

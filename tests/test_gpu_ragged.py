@@ -57,3 +57,32 @@ def test_layers_of_awkward_sizes(ctx, dtype, B, Ci, Co, H, W, k):
     for r in (only_w, both):
         assert (r["dW"] - out["dW"]).abs().max().item() <= 1e-5 * top
     assert torch.equal(both["dX"], out["dX"].to(both["dX"].dtype))
+
+
+@pytest.mark.parametrize("B,Ci,Co,H,W,stride", [
+    (64, 8, 10, 28, 28, 1),       # 1.6 MB of codes in rows of 16 channels, 1.0 MB in rows of 10
+    (128, 16, 9, 32, 32, 1),      # 4.2 MB in rows of 16 channels, 2.4 MB in rows of 9
+    (64, 8, 10, 56, 56, 2)])
+@pytest.mark.parametrize("dtype", ["f32", "bf16"])
+def test_codes_whose_padded_rows_are_much_larger(dtype, B, Ci, Co, H, W, stride):
+    """3x3 layers whose codes lie in rows padded to 16 bytes, at sizes where the padding is more than any rounding of the
+    workspace's size: on a context of their own, so that no earlier, larger call has made room for them."""
+    import paper_2004_04729_b200 as dbp
+    L = wl.conv_layer(B, Ci, Co, H, W, 3, data_seed=B + Co + H, scale=2.0, seed=11, dtype=dtype, stride=stride)
+    tdt = torch.bfloat16 if dtype == "bf16" else torch.float32
+    d, X, Wt = (torch.from_numpy(np.ascontiguousarray(a)).to(tdt).cuda() for a in (L.delta, L.X, L.W))
+    own = dbp.Context(0)
+    try:
+        out = dbp.dithered_conv_backward(own, d, X, Wt, L.seed, L.scale, need_db=True, flags=dbp.DBP_DX_F32, stride=stride)
+        D, nnz = own.last_step()
+        assert own.last_device_status() == (0, 0)
+    finally:
+        own.close()
+    D = np.float32(D)
+    codes, onnz, _ = oracle.nsd_codes(L.delta, L.seed, D)
+    assert nnz == onnz
+    ref = oracle.conv_backward(codes, D, L.X, L.W, with_abs=True) if stride == 1 else \
+        oracle.conv_backward_strided(codes, D, L.X, L.W, stride, with_abs=True)
+    for key in ("dW", "dX", "db"):
+        g = out[key].double().cpu().numpy()
+        assert np.all(np.abs(g - ref[key]) <= TOL * ref["S_" + key] + 1e-30), key
