@@ -283,6 +283,11 @@ def nsd_decode_dense(ctx: Context, q: SparseGradient, shape=None) -> torch.Tenso
     return codes if shape is None else codes.view(shape)
 
 
+def _drop_mask(ctx):
+    """A call that is refused here still uses up the ReLU mask that was set for it."""
+    load_library().dbp_set_relu_mask(ctx._h, None)
+
+
 def _outputs(need, shape, dtype, device):
     return torch.empty(shape, dtype=dtype, device=device) if need else None
 
@@ -291,27 +296,31 @@ def dithered_linear_backward(ctx: Context, delta, X, W, seed: int, scale: float,
                              delta_in=None, q_out: Optional[SparseGradient] = None,
                              need_dW=True, need_dX=True, need_db=False, flags: int = 0):
     """delta [B,N], X [B,K], W [N,K] -> dict(dW [N,K] fp32, dX [B,K], db [N] fp32)."""
-    r = _native.linear_backward(ctx._h.value, delta, X, W, seed, scale, delta_in, q_out and q_out._addr, need_dW, need_dX, need_db,
-                                flags)
-    if type(r) is dict:
-        return r
-    if r is not None:
-        raise DbpError(r, "dithered_linear_backward")
-    _dev(delta, "delta"), _dev(X, "X"), _dev(W, "W")
-    B, N = delta.shape
-    K = X.shape[1]
-    assert X.shape == (B, K) and W.shape == (N, K) and X.dtype == delta.dtype == W.dtype
-    dev = delta.device
-    dx_dtype = torch.float32 if (flags & DBP_DX_F32) else delta.dtype
-    dW = _outputs(need_dW, (N, K), torch.float32, dev)
-    dX = _outputs(need_dX, (B, K), dx_dtype, dev)
-    db = _outputs(need_db, (N,), torch.float32, dev)
-    _check(load_library().dithered_linear_backward(
-        ctx._h, _ptr(delta), _ptr(X), _ptr(W), _dtype_code(delta), B, N, K,
-        int(seed) & (2 ** 64 - 1), float(scale), _ptr(delta_in),
-        q_out.c() if q_out is not None else None, _ptr(dW), _ptr(dX), _ptr(db), int(flags)),
-        "dithered_linear_backward")
-    return {"dW": dW, "dX": dX, "db": db}
+    try:
+        r = _native.linear_backward(ctx._h.value, delta, X, W, seed, scale, delta_in, q_out and q_out._addr, need_dW, need_dX, need_db,
+                                    flags)
+        if type(r) is dict:
+            return r
+        if r is not None:
+            raise DbpError(r, "dithered_linear_backward")
+        _dev(delta, "delta"), _dev(X, "X"), _dev(W, "W")
+        B, N = delta.shape
+        K = X.shape[1]
+        assert X.shape == (B, K) and W.shape == (N, K) and X.dtype == delta.dtype == W.dtype
+        dev = delta.device
+        dx_dtype = torch.float32 if (flags & DBP_DX_F32) else delta.dtype
+        dW = _outputs(need_dW, (N, K), torch.float32, dev)
+        dX = _outputs(need_dX, (B, K), dx_dtype, dev)
+        db = _outputs(need_db, (N,), torch.float32, dev)
+        _check(load_library().dithered_linear_backward(
+            ctx._h, _ptr(delta), _ptr(X), _ptr(W), _dtype_code(delta), B, N, K,
+            int(seed) & (2 ** 64 - 1), float(scale), _ptr(delta_in),
+            q_out.c() if q_out is not None else None, _ptr(dW), _ptr(dX), _ptr(db), int(flags)),
+            "dithered_linear_backward")
+        return {"dW": dW, "dX": dX, "db": db}
+    except Exception:
+        _drop_mask(ctx)
+        raise
 
 
 def dithered_conv_backward(ctx: Context, delta, X, W, seed: int, scale: float, *,
@@ -319,32 +328,36 @@ def dithered_conv_backward(ctx: Context, delta, X, W, seed: int, scale: float, *
                            need_dW=True, need_dX=True, need_db=False, flags: int = 0,
                            stride: int = 1, pad: Optional[int] = None):
     """delta [B,Cout,H/stride,W/stride], X [B,Cin,H,W], W [Cout,Cin,k,k] (NCHW) -> dict(dW, dX, db)."""
-    r = _native.conv_backward(ctx._h.value, delta, X, W, seed, scale, delta_in, q_out and q_out._addr, need_dW, need_dX, need_db,
-                              flags, stride, (W.shape[2] - 1) // 2 if pad is None else pad)
-    if type(r) is dict:
-        return r
-    if r is not None:
-        raise DbpError(r, "dithered_conv_backward")
-    _dev(delta, "delta"), _dev(X, "X"), _dev(W, "W")
-    B, Co = delta.shape[:2]
-    Ci, k = X.shape[1], W.shape[2]
-    H, Wd = X.shape[2], X.shape[3]
-    if stride not in (1, 2) or X.shape[0] != B or W.shape != (Co, Ci, k, k) or \
-            (H % stride, Wd % stride) != (0, 0) or tuple(delta.shape[2:]) != (H // stride, Wd // stride):
-        raise ValueError("shapes of delta, X and W do not belong to one layer")
-    assert X.dtype == delta.dtype == W.dtype
-    pad = (k - 1) // 2 if pad is None else pad
-    dev = delta.device
-    dx_dtype = torch.float32 if (flags & DBP_DX_F32) else delta.dtype
-    dW = _outputs(need_dW, (Co, Ci, k, k), torch.float32, dev)
-    dX = _outputs(need_dX, (B, Ci, H, Wd), dx_dtype, dev)
-    db = _outputs(need_db, (Co,), torch.float32, dev)
-    _check(load_library().dithered_conv_backward(
-        ctx._h, _ptr(delta), _ptr(X), _ptr(W), _dtype_code(delta), B, Ci, Co, H, Wd, k, stride, pad,
-        int(seed) & (2 ** 64 - 1), float(scale), _ptr(delta_in),
-        q_out.c() if q_out is not None else None, _ptr(dW), _ptr(dX), _ptr(db), int(flags)),
-        "dithered_conv_backward")
-    return {"dW": dW, "dX": dX, "db": db}
+    try:
+        r = _native.conv_backward(ctx._h.value, delta, X, W, seed, scale, delta_in, q_out and q_out._addr, need_dW, need_dX, need_db,
+                                  flags, stride, (W.shape[2] - 1) // 2 if pad is None else pad)
+        if type(r) is dict:
+            return r
+        if r is not None:
+            raise DbpError(r, "dithered_conv_backward")
+        _dev(delta, "delta"), _dev(X, "X"), _dev(W, "W")
+        B, Co = delta.shape[:2]
+        Ci, k = X.shape[1], W.shape[2]
+        H, Wd = X.shape[2], X.shape[3]
+        if stride not in (1, 2) or X.shape[0] != B or W.shape != (Co, Ci, k, k) or \
+                (H % stride, Wd % stride) != (0, 0) or tuple(delta.shape[2:]) != (H // stride, Wd // stride):
+            raise ValueError("shapes of delta, X and W do not belong to one layer")
+        assert X.dtype == delta.dtype == W.dtype
+        pad = (k - 1) // 2 if pad is None else pad
+        dev = delta.device
+        dx_dtype = torch.float32 if (flags & DBP_DX_F32) else delta.dtype
+        dW = _outputs(need_dW, (Co, Ci, k, k), torch.float32, dev)
+        dX = _outputs(need_dX, (B, Ci, H, Wd), dx_dtype, dev)
+        db = _outputs(need_db, (Co,), torch.float32, dev)
+        _check(load_library().dithered_conv_backward(
+            ctx._h, _ptr(delta), _ptr(X), _ptr(W), _dtype_code(delta), B, Ci, Co, H, Wd, k, stride, pad,
+            int(seed) & (2 ** 64 - 1), float(scale), _ptr(delta_in),
+            q_out.c() if q_out is not None else None, _ptr(dW), _ptr(dX), _ptr(db), int(flags)),
+            "dithered_conv_backward")
+        return {"dW": dW, "dX": dX, "db": db}
+    except Exception:
+        _drop_mask(ctx)
+        raise
 
 
 def _host(t: Optional[torch.Tensor], name):
@@ -356,33 +369,41 @@ def _host(t: Optional[torch.Tensor], name):
 def dithered_linear_backward_host(ctx: Context, delta, X, W, seed, scale, dW, dX, db=None,
                                   flags: int = 0):
     """Host tensors in and out (pinned memory recommended); returns (Delta, nnz)."""
-    for n, t in (("delta", delta), ("X", X), ("W", W), ("dW", dW), ("dX", dX), ("db", db)):
-        _host(t, n)
-    B, N = delta.shape
-    K = X.shape[1]
-    d, nnz = ctypes.c_float(), ctypes.c_longlong()
-    _check(load_library().dithered_linear_backward_host(
-        ctx._h, _ptr(delta), _ptr(X), _ptr(W), _dtype_code(delta), B, N, K,
-        int(seed) & (2 ** 64 - 1), float(scale), _ptr(dW), _ptr(dX), _ptr(db), int(flags),
-        ctypes.byref(d), ctypes.byref(nnz)), "dithered_linear_backward_host")
-    return d.value, nnz.value
+    try:
+        for n, t in (("delta", delta), ("X", X), ("W", W), ("dW", dW), ("dX", dX), ("db", db)):
+            _host(t, n)
+        B, N = delta.shape
+        K = X.shape[1]
+        d, nnz = ctypes.c_float(), ctypes.c_longlong()
+        _check(load_library().dithered_linear_backward_host(
+            ctx._h, _ptr(delta), _ptr(X), _ptr(W), _dtype_code(delta), B, N, K,
+            int(seed) & (2 ** 64 - 1), float(scale), _ptr(dW), _ptr(dX), _ptr(db), int(flags),
+            ctypes.byref(d), ctypes.byref(nnz)), "dithered_linear_backward_host")
+        return d.value, nnz.value
+    except Exception:
+        _drop_mask(ctx)
+        raise
 
 
 def dithered_conv_backward_host(ctx: Context, delta, X, W, seed, scale, dW, dX, db=None,
                                 flags: int = 0, stride: int = 1):
-    for n, t in (("delta", delta), ("X", X), ("W", W), ("dW", dW), ("dX", dX), ("db", db)):
-        _host(t, n)
-    B, Co = delta.shape[:2]
-    Ci, k = X.shape[1], W.shape[2]
-    H, Wd = X.shape[2], X.shape[3]
-    if tuple(delta.shape[2:]) != (H // stride, Wd // stride):
-        raise ValueError("shapes of delta and X do not belong to one layer")
-    d, nnz = ctypes.c_float(), ctypes.c_longlong()
-    _check(load_library().dithered_conv_backward_host(
-        ctx._h, _ptr(delta), _ptr(X), _ptr(W), _dtype_code(delta), B, Ci, Co, H, Wd, k, int(stride),
-        (k - 1) // 2, int(seed) & (2 ** 64 - 1), float(scale), _ptr(dW), _ptr(dX), _ptr(db),
-        int(flags), ctypes.byref(d), ctypes.byref(nnz)), "dithered_conv_backward_host")
-    return d.value, nnz.value
+    try:
+        for n, t in (("delta", delta), ("X", X), ("W", W), ("dW", dW), ("dX", dX), ("db", db)):
+            _host(t, n)
+        B, Co = delta.shape[:2]
+        Ci, k = X.shape[1], W.shape[2]
+        H, Wd = X.shape[2], X.shape[3]
+        if tuple(delta.shape[2:]) != (H // stride, Wd // stride):
+            raise ValueError("shapes of delta and X do not belong to one layer")
+        d, nnz = ctypes.c_float(), ctypes.c_longlong()
+        _check(load_library().dithered_conv_backward_host(
+            ctx._h, _ptr(delta), _ptr(X), _ptr(W), _dtype_code(delta), B, Ci, Co, H, Wd, k, int(stride),
+            (k - 1) // 2, int(seed) & (2 ** 64 - 1), float(scale), _ptr(dW), _ptr(dX), _ptr(db),
+            int(flags), ctypes.byref(d), ctypes.byref(nnz)), "dithered_conv_backward_host")
+        return d.value, nnz.value
+    except Exception:
+        _drop_mask(ctx)
+        raise
 
 
 def relu_backward(ctx: Context, delta_a: torch.Tensor, mask_u8: torch.Tensor) -> torch.Tensor:

@@ -57,6 +57,13 @@ struct DeviceGuard {
     ~DeviceGuard() { if (prev >= 0 && prev != now) cudaSetDevice(prev); }
 };
 
+// A ReLU mask set for the next backward call is gone when that call returns, whichever way it returns: the context must not
+// be left with the address of a tensor that its owner may free.
+struct MaskUse {
+    dbp_ctx *ctx;
+    ~MaskUse() { if (ctx) ctx->next_mask = nullptr; }
+};
+
 // The current set's previous readers (an earlier call's dW kernels on the second stream) must be done before its step
 // size and its codes are written again. The wait stands in front of a call's first kernel, where the stream
 // already holds the previous call's fork event: stream operations between two kernels stop their programmatic
@@ -904,6 +911,7 @@ int dithered_linear_backward(dbp_ctx *ctx, const void *delta, const void *X, con
                              long long B, long long N, long long K, unsigned long long seed, float scale,
                              const float *delta_in, dbp_sparse *q_out, float *dW, void *dX, float *db,
                              unsigned flags) {
+    const MaskUse mask_use{ctx};
     // [B,N] x [N,K]: the 1x1 convolution with one position per image has the same layout
     ConvShape s{B, K, N, 1, 1, 1};
     return conv_backward_impl(ctx, delta, X, W, io, s, seed, scale, delta_in, q_out, dW, dX, db, flags);
@@ -914,6 +922,7 @@ int dithered_conv_backward(dbp_ctx *ctx, const void *delta, const void *X, const
                            int stride, int pad, unsigned long long seed, float scale,
                            const float *delta_in, dbp_sparse *q_out, float *dW, void *dX, float *db,
                            unsigned flags) {
+    const MaskUse mask_use{ctx};
     if (!conv_form_supported(k, stride, pad)) return DBP_EUNSUPPORTED;
     ConvShape s{B, Cin, Cout, H, Wd, k};
     return conv_backward_any(ctx, delta, X, W, io, s, stride, seed, scale, delta_in, q_out, dW, dX, db, flags);
@@ -988,6 +997,7 @@ int dithered_linear_backward_host(dbp_ctx *ctx, const void *delta, const void *X
                                   long long B, long long N, long long K, unsigned long long seed,
                                   float scale, float *dW, void *dX, float *db, unsigned flags,
                                   float *delta_out, long long *nnz_out) {
+    const MaskUse mask_use{ctx};
     if (!(scale > 0.f)) return DBP_EINVAL;
     ConvShape s{B, K, N, 1, 1, 1};
     return host_backward(ctx, delta, X, W, io, s, seed, scale, dW, dX, db, flags, delta_out, nnz_out);
@@ -998,6 +1008,7 @@ int dithered_conv_backward_host(dbp_ctx *ctx, const void *delta, const void *X, 
                                 int k, int stride, int pad, unsigned long long seed, float scale,
                                 float *dW, void *dX, float *db, unsigned flags, float *delta_out,
                                 long long *nnz_out) {
+    const MaskUse mask_use{ctx};
     if (!conv_form_supported(k, stride, pad)) return DBP_EUNSUPPORTED;
     if (stride == 2 && ((H & 1) || (Wd & 1))) return DBP_EUNSUPPORTED;
     if (!(scale > 0.f)) return DBP_EINVAL;

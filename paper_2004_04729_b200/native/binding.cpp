@@ -43,6 +43,24 @@ PyObject *result(const at::Tensor &dW, const at::Tensor &dX, const at::Tensor &d
     return nullptr;
 }
 PyObject *none() { return Py_NewRef(Py_None); }
+// A mask that was set for a call is not left behind on the context when the call does not happen (an output that could not be
+// allocated, shapes that do not belong together).
+struct MaskUse {
+    dbp_ctx *ctx;
+    ~MaskUse() { dbp_set_relu_mask(ctx, nullptr); }
+};
+// Owns a reference until it is released.
+struct Owned {
+    PyObject *o;
+    explicit Owned(PyObject *object) : o(object) {}
+    Owned(const Owned &) = delete;
+    ~Owned() { Py_XDECREF(o); }
+    PyObject *release() {
+        PyObject *r = o;
+        o = nullptr;
+        return r;
+    }
+};
 // Other Python threads run while a call allocates and enqueues (either may block: a full launch queue, a growing pool).
 struct NoGil {
     PyThreadState *state = PyEval_SaveThread();
@@ -116,6 +134,7 @@ PyObject *layer_backward(PyObject *const *a, Py_ssize_t n, bool is_conv) {
     if (PyErr_Occurred()) { PyErr_Clear(); return none(); }
     int io;
     if (!same_kind(*d, *X, *W, io) || !(is_conv ? conv_shapes(*d, *X, *W, stride) : linear_shapes(*d, *X, *W))) return none();
+    const MaskUse mask_use{c.ctx};
     at::Tensor dW, dX, db;
     const int rc = is_conv ? conv(c, *d, *X, *W, io, static_cast<int>(stride), static_cast<int>(pad), dW, dX, db)
                            : linear(c, *d, *X, *W, io, dW, dX, db);
@@ -238,18 +257,18 @@ PyObject *network(PyObject *const *a, Py_ssize_t n) {
         if (l + 1 < L && (!y.mask || (y.conv && y.mask->dim() != 4))) return none();
     }
     if (!on_device(*d0) || d0->scalar_type() != at::kFloat) return none();
-    PyObject *res = PyList_New(L);
-    if (!res) return nullptr;
+    Owned res(PyList_New(L));
+    if (!res.o) return nullptr;
     at::Tensor delta = *d0;
     for (Py_ssize_t l = L - 1; l >= 0; --l) {
         const Layer &y = layers[l];
         int rc = 0;
         if (!(y.conv ? conv_shapes(delta, *y.X, *y.W, 1) : linear_shapes(delta, *y.X, *y.W)) ||
             (y.mask && y.mask->numel() != delta.numel())) {
-            Py_DECREF(res);
             if (l < L - 1) { PyErr_SetString(PyExc_ValueError, "shapes of the layers do not belong to one network"); return nullptr; }
             return none();
         }
+        const MaskUse mask_use{c.ctx};
         if (y.mask) rc = dbp_set_relu_mask(c.ctx, static_cast<const uint8_t *>(y.mask->data_ptr()));
         c.seed = dbp_layer_seed(seed, static_cast<int>(l));
         c.need_dX = l > 0 || first_dX;
@@ -257,17 +276,10 @@ PyObject *network(PyObject *const *a, Py_ssize_t n) {
         if (!rc)
             rc = y.conv ? conv(c, delta, *y.X, *y.W, DBP_F32, 1, static_cast<int>((y.W->size(2) - 1) / 2), dW, dX, db)
                         : linear(c, delta, *y.X, *y.W, DBP_F32, dW, dX, db);
-        if (rc) {
-            Py_DECREF(res);
-            return PyLong_FromLong(rc);
-        }
-        PyObject *d = result(dW, dX, db);
-        if (!d || PyDict_SetItem(d, key_Delta, Py_None) || PyDict_SetItem(d, key_nnz, Py_None)) {
-            Py_XDECREF(d);
-            Py_DECREF(res);
-            return nullptr;
-        }
-        PyList_SET_ITEM(res, l, d);
+        if (rc) return PyLong_FromLong(rc);
+        Owned d(result(dW, dX, db));
+        if (!d.o || PyDict_SetItem(d.o, key_Delta, Py_None) || PyDict_SetItem(d.o, key_nnz, Py_None)) return nullptr;
+        PyList_SET_ITEM(res.o, l, d.release());
         if (l == 0) break;
         const Layer &below = layers[l - 1];
         delta = dX;
@@ -278,19 +290,15 @@ PyObject *network(PyObject *const *a, Py_ssize_t n) {
         if (below.pool) {
             at::Tensor routed;
             if (delta.dim() != 4 || below.pool->numel() != delta.numel()) {
-                Py_DECREF(res);
                 PyErr_SetString(PyExc_ValueError, "shapes of a pool and its gradient differ");
                 return nullptr;
             }
             rc = maxpool(c.ctx, delta, *below.pool, routed);
-            if (rc) {
-                Py_DECREF(res);
-                return PyLong_FromLong(rc);
-            }
+            if (rc) return PyLong_FromLong(rc);
             delta = routed;
         }
     }
-    return res;
+    return res.release();
 }
 PyObject *network_backward(PyObject *, PyObject *const *a, Py_ssize_t n) {
     try { return network(a, n); } catch (const std::exception &e) { PyErr_SetString(PyExc_RuntimeError, e.what()); return nullptr; }

@@ -217,3 +217,46 @@ def test_relu_mask_corner_cases(ctx):
     out = dbp.dithered_linear_backward(ctx, db16, X16, W16, L.seed, L.scale)     # the mask is gone
     torch.cuda.synchronize()
     assert out["dW"].isfinite().all()
+
+
+def test_a_call_that_is_refused_uses_up_its_mask(ctx):
+    """A mask belongs to one call, also to one that never runs: a form the library does not have, shapes that do not
+    belong together (refused by the binding), a network whose layers do not fit. The next call reads no mask."""
+    import paper_2004_04729_b200 as dbp
+    rng = np.random.default_rng(6)
+    L = wl.linear_layer(40, 24, 56, data_seed=951, scale=2.0, seed=1)
+    d, X, W = _cu(L.delta), _cu(L.X), _cu(L.W)
+    mask = torch.from_numpy((rng.random(L.delta.shape) < 0.5).astype(np.uint8)).cuda()
+    want = dbp.dithered_linear_backward(ctx, d, X, W, L.seed, L.scale)
+    want_step = ctx.last_step()
+
+    def conv7():                                          # a 7x7 kernel: DBP_EUNSUPPORTED
+        z = torch.zeros(1, 8, 8, 8, device="cuda")
+        dbp.dithered_conv_backward(ctx, z, z, torch.zeros(8, 8, 7, 7, device="cuda"), 0, 2.0)
+
+    def no_matrix():
+        dbp.dithered_conv_backward(ctx, d, X, W, 0, 2.0)
+
+    def host_shapes():
+        z = torch.zeros(1, 8, 8, 8)
+        dbp.dithered_conv_backward_host(ctx, z, torch.zeros(1, 8, 9, 8), torch.zeros(8, 8, 3, 3), 0, 2.0, None, None)
+
+    def null_delta():
+        dbp.binding._check(dbp.load_library().dithered_conv_backward(ctx._h, None, None, None, 0, 1, 8, 8, 8, 8, 3, 2, 1, 0, 2.0, None,
+                                                                     None, None, None, None, 0), "dithered_conv_backward")
+
+    def shapes():
+        dbp.dithered_linear_backward(ctx, d, X, W[:, :-1].contiguous(), 0, 2.0)
+
+    def network():                                        # the masked layer's own call is refused: 7x7 kernels
+        z = torch.zeros(5, 8, 3, 3, device="cuda")
+        dbp.network_backward(ctx, ["conv"], [z], [torch.zeros(8, 8, 7, 7, device="cuda")], [mask.view(-1)[:360].view(5, 8, 3, 3)], [None],
+                             z, 2.0, 0, with_sparse=False)
+
+    for refused in (conv7, no_matrix, host_shapes, null_delta, shapes, network):
+        ctx.set_relu_mask(mask)
+        with pytest.raises(Exception):
+            refused()
+        got = dbp.dithered_linear_backward(ctx, d, X, W, L.seed, L.scale)
+        assert ctx.last_step() == want_step, refused.__name__
+        assert torch.equal(got["dX"], want["dX"]) and torch.equal(got["dW"], want["dW"]), refused.__name__
