@@ -341,9 +341,12 @@ tc3_tma_dw_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
                         int ky, col0;                           // tap and first output channel of these 32 columns
                         if (NP == 2) { ky = c >> 2; col0 = (c & 3) * 32; }     // columns 0-127: ky = 0, 128-255: ky = 1, ...
                         else { ky = 2 - (c >> 1); col0 = (c & 1) * 32; }       // columns 0-63: ky = 2, 64-127: ky = 1, 128-191: ky = 0
-                        // columns past Cout hold exact zeros (their codes were zero fill): adding them is harmless
-                        tma_reduce_add_2d(&map_acc, ci0, (ky * 3 + kx) * p.Cout + co0 + col0, stg + i * 4096);
-                        if (p.split) tma_reduce_add_2d(&map_acc, 0, (ky * 3 + kx) * p.Cout + co0 + col0, stg + i * 4096 + 2048);
+                        // The rows of output channels past Cout are outside the tap's matrix: the engine skips them. (They are
+                        // zeros only while the activations are finite: NaN added to the next tap's first rows would stay in
+                        // the scratch where nobody reads that tap.)
+                        if (co0 + col0 >= p.Cout) continue;
+                        tma_reduce_add_3d(&map_acc, ci0, co0 + col0, ky * 3 + kx, stg + i * 4096);
+                        if (p.split) tma_reduce_add_3d(&map_acc, 0, co0 + col0, ky * 3 + kx, stg + i * 4096 + 2048);
                     }
                     bulk_commit();
                     bulk_wait_read_all();
@@ -568,10 +571,10 @@ int launch_tc3_tma_dw(dbp_ctx *ctx, const void *codes_nhwc, const void *X, int p
     p.stage_chunks = static_cast<int>((smem - 1024) / 16384);
     CUtensorMap map_q, map_x, map_acc;
     {
-        const unsigned long long dims[2] = {static_cast<unsigned long long>(cin_pad), static_cast<unsigned long long>(s.Cout) * 9};
-        const unsigned long long str[1] = {static_cast<unsigned long long>(cin_pad) * 4};
-        const unsigned box[2] = {p.split ? 64u : 128u, 32};
-        if (!encode_map_f32_rows(&map_acc, acc, 2, dims, str, box)) return fail_cuda("tensor map of the dW scratch");
+        const unsigned long long dims[3] = {static_cast<unsigned long long>(cin_pad), static_cast<unsigned long long>(s.Cout), 9};
+        const unsigned long long str[2] = {static_cast<unsigned long long>(cin_pad) * 4, static_cast<unsigned long long>(pairs) * 4};
+        const unsigned box[3] = {p.split ? 64u : 128u, 32, 1};
+        if (!encode_map_f32_rows(&map_acc, acc, 3, dims, str, box)) return fail_cuda("tensor map of the dW scratch");
     }
     {
         const unsigned long long dims[3] = {static_cast<unsigned long long>(s.Cout), static_cast<unsigned long long>(HW),

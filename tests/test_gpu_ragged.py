@@ -28,7 +28,7 @@ def ctx():
     (9, 20, 24, 1, 2, 1),         # the smallest plane
     (4, 64, 40, 3, 3, 1), (1, 257, 129, 16, 12, 1),
     (2, 3, 8, 6, 6, 3), (2, 12, 20, 9, 9, 3), (3, 130, 65, 7, 5, 3), (2, 65, 67, 8, 8, 3), (4, 10, 6, 2, 3, 3),
-    (1, 33, 129, 20, 17, 3)])
+    (1, 33, 129, 20, 17, 3), (3, 9, 1, 6, 7, 3)])
 @pytest.mark.parametrize("dtype", ["f32", "bf16"])
 def test_layers_of_awkward_sizes(ctx, dtype, B, Ci, Co, H, W, k):
     import paper_2004_04729_b200 as dbp

@@ -180,6 +180,25 @@ def test_stride2_leaves_the_weight_gradient_scratch_clean(ctx):
             assert fro(a, strided_alone) <= 1e-5 and fro(b, plain_alone) <= 1e-5
 
 
+def test_a_non_finite_activation_does_not_outlive_its_call(ctx):
+    """72 output channels leave part of the last tile of 128 without a channel. With an infinity in X the accumulators of
+    that part hold NaN (0 * inf); nothing of them may stay in the scratch that the next layer's weight gradient is added
+    up in, least of all in the taps that a stride-2 layer never reads."""
+    import paper_2004_04729_b200 as dbp
+    bad = wl.conv_layer(2, 128, 72, 16, 16, 3, data_seed=77, scale=5.0, dtype="bf16", stride=2)
+    good = wl.conv_layer(2, 512, 72, 8, 8, 3, data_seed=78, scale=5.0, dtype="bf16")     # the same scratch, every tap read
+    bad.X[1, 5, 3, 4] = np.inf
+    d, X, W = (_dev(a, "bf16") for a in (good.delta, good.X, good.W))
+    want = dbp.dithered_conv_backward(ctx, d, X, W, good.seed, good.scale)
+    for _ in range(2):
+        out = dbp.dithered_conv_backward(ctx, *(_dev(a, "bf16") for a in (bad.delta, bad.X, bad.W)), bad.seed, bad.scale, stride=2)
+        other = torch.arange(128, device="cuda") != 5
+        assert torch.isfinite(out["dW"][:, other]).all() and not torch.isfinite(out["dW"][:, 5]).all()
+        got = dbp.dithered_conv_backward(ctx, d, X, W, good.seed, good.scale)
+        assert torch.equal(got["dX"], want["dX"])
+        assert (got["dW"] - want["dW"]).abs().max() <= 1e-5 * want["dW"].abs().max()
+
+
 @pytest.mark.parametrize("dtype", ["bf16", "f32"])
 def test_stride2_with_a_given_step_size(ctx, dtype):
     """scale <= 0 and a device step size: no statistics kernel runs, so the weights take the other route."""
