@@ -297,16 +297,25 @@ struct KernelTimer {
     }
 };
 
+// An accumulator of the tensor cores is truncated, not rounded, when an MMA adds to it: a sum of terms of one sign comes out
+// low by up to 1.7e-8 of itself per MMA (measured: bf16 1x1 dW, 680 and 1360 MMAs: 0.9e-5 and 2.3e-5; fp32 3x3 dW, 2100
+// MMAs: 4.8e-5). Longer reductions are cut into parts of at most this many, which are added with rounding; fp32 operands
+// enter as two bf16 pieces, which costs at most 2^-18 more, and together that stays below 1e-5 of the sum of the terms' sizes.
+constexpr int kMaxMmas = 512;
+
 // Split of a K loop of `kunits` steps over CTAs when `tiles` output tiles exist and one CTA fits
 // per SM: the CTAs run in ceil(tiles * split / sms) waves of ceil(kunits / split) steps each, so
 // a split that spills a few CTAs into another wave doubles the time. Picks the split with the
 // fewest wave-steps (a CTA's fixed cost counted as two steps, a small charge per split for the
-// partial sums); *per_split receives the steps per CTA. The returned split has no empty part.
-inline long long choose_split(long long tiles, long long kunits, int sms, long long *per_split) {
-    long long best = 1, best_per = kunits;
+// partial sums) among those of at most max_per steps per CTA; *per_split receives the steps per CTA.
+// The returned split has no empty part.
+inline long long choose_split(long long tiles, long long kunits, int sms, long long max_per, long long *per_split) {
+    const long long least = (kunits + max_per - 1) / max_per;
+    long long best = least, best_per = max_per;
     double best_cost = 1e300;
-    const long long smax = kunits < 4ll * sms ? kunits : 4ll * sms;
-    for (long long want = 1; want <= smax; ++want) {
+    long long smax = kunits < 4ll * sms ? kunits : 4ll * sms;
+    if (smax < least) smax = least;
+    for (long long want = least; want <= smax; ++want) {
         const long long per = (kunits + want - 1) / want, split = (kunits + per - 1) / per;
         const long long waves = (tiles * split + sms - 1) / sms;
         const double cost = static_cast<double>(waves) * static_cast<double>(per + 2) + 0.05 * static_cast<double>(split);

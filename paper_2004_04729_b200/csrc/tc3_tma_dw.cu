@@ -555,7 +555,8 @@ int launch_tc3_tma_dw(dbp_ctx *ctx, const void *codes_nhwc, const void *X, int p
                         ? ctx->phase_cin / 128 : 0;
     const long long tiles = p.phase_tiles > 0 ? static_cast<long long>(p.co_tiles) * 6 * p.phase_tiles
                                               : static_cast<long long>(p.ci_tiles) * p.co_tiles * 3;
-    const long long nsplit = choose_split(tiles, p.nseg, ctx->sm_count, &p.per_split);
+    // (an MMA takes 16 positions)
+    const long long nsplit = choose_split(tiles, p.nseg, ctx->sm_count, kMaxMmas * 16 / p.SEG, &p.per_split);
     p.nsplit = static_cast<int>(nsplit);
     if (tiles * nsplit >= (1ll << 31)) return DBP_EUNSUPPORTED;
     // fp32 scratch [9][Cout][Cin]: zero whenever no call is in flight

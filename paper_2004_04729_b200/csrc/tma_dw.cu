@@ -221,13 +221,8 @@ int launch_tma_dw(dbp_ctx *ctx, const void *codes_bf16, const void *X, int piece
     const long long co_tiles = (s.Cout + 128 * p.MA - 1) / (128 * p.MA);
     const long long tiles = co_tiles * p.ci_tiles;
     long long per = 0;
-    long long nsplit = choose_split(tiles, p.nchunks, ctx->sm_count, &per);
-    // an accumulator is truncated, not rounded, when an MMA adds to it (about 1e-8 of its value per MMA): an fp32 layer's
-    // parts are kept to 128 chunks of four MMAs
-    if (pieces == 2 && per > 128) {
-        per = 128;
-        nsplit = (p.nchunks + per - 1) / per;
-    }
+    // (an MMA takes 16 of a chunk's 64 positions)
+    const long long nsplit = choose_split(tiles, p.nchunks, ctx->sm_count, pieces == 2 ? kMaxMmas / 4 : p.nchunks, &per);
     p.nsplit = static_cast<int>(nsplit);
     p.per_split = per;
     p.err_flag = err_flag;

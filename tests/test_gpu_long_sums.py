@@ -1,0 +1,67 @@
+"""Sums of one sign over long reductions. The tensor cores' accumulators are truncated when an MMA adds to them, so such a sum
+comes out low by an amount that grows with its length; the kernels cut long reductions into parts. Every entry is compared
+with 64-bit sums of the library's own codes: within 1e-5 of it (all terms have one sign, so the sum is the sum of their sizes),
+the bound of every other layer."""
+import pytest
+import torch
+
+pytestmark = pytest.mark.gpu
+TOL = 1e-5
+
+
+@pytest.fixture(scope="module")
+def ctx():
+    import paper_2004_04729_b200 as dbp
+    c = dbp.Context(0)
+    yield c
+    c.close()
+
+
+def _positive(gen, dtype, *shape, scale=1.0):
+    return (torch.randn(*shape, generator=gen, device="cuda").abs() * scale).to(torch.bfloat16 if dtype == "bf16" else torch.float32)
+
+
+def _layer(ctx, dtype, B, Ci, Co, H, W, k):
+    """delta, X, W all positive, the codes and the step size of a call with seed 3 and scale 1."""
+    import paper_2004_04729_b200 as dbp
+    gen = torch.Generator(device="cuda")
+    gen.manual_seed(B + Ci + Co)
+    d = _positive(gen, dtype, B, Co, H, W, scale=1e-3)
+    X, Wt = _positive(gen, dtype, B, Ci, H, W), _positive(gen, dtype, Co, Ci, k, k)
+    q = dbp.nsd_quantize(ctx, d, 3, 1.0)
+    return d, X, Wt, dbp.nsd_decode_dense(ctx, q, d.shape), q.delta.double().item()
+
+
+def _some(n):
+    """A few channels, the first and the last among them."""
+    return torch.unique(torch.linspace(0, n - 1, min(n, 7), device="cuda").long())
+
+
+def _shifted(t, dy, dx):
+    """t[..., y + dy, x + dx], zero outside."""
+    return torch.nn.functional.pad(t, (1, 1, 1, 1))[..., 1 + dy:t.shape[-2] + 1 + dy, 1 + dx:t.shape[-1] + 1 + dx]
+
+
+def _check_dW(dW, codes, delta, X, k):
+    co, ci = _some(dW.shape[0]), _some(dW.shape[1])
+    q, x = codes[:, co].double(), X[:, ci].double()
+    for ky in range(k):
+        for kx in range(k):
+            ref = delta * torch.einsum("bcyx,bdyx->cd", q, x if k == 1 else _shifted(x, ky - 1, kx - 1))
+            rel = ((dW[co][:, ci][:, :, ky, kx].double() - ref) / ref).abs().max().item()
+            assert rel <= TOL, (ky, kx, rel)
+
+
+@pytest.mark.parametrize("dtype,B,Ci,Co,H,W", [
+    ("f32", 64, 512, 512, 28, 28),      # 50176 positions in two pieces on 48 tiles
+    ("f32", 256, 64, 64, 56, 56),       # both pieces in one tile
+    ("f32", 130, 128, 72, 56, 56),      # a ragged tile of output channels
+    ("bf16", 64, 512, 512, 28, 28),
+    ("bf16", 256, 128, 128, 56, 56)])
+def test_3x3_weight_gradients(ctx, dtype, B, Ci, Co, H, W):
+    import paper_2004_04729_b200 as dbp
+    d, X, Wt, codes, delta = _layer(ctx, dtype, B, Ci, Co, H, W, 3)
+    for need_dX in (False, True):       # the dW kernel by itself, and sharing the SMs with dX where it does
+        out = dbp.dithered_conv_backward(ctx, d, X, Wt, 3, 1.0, need_dX=need_dX)
+        _check_dW(out["dW"], codes, delta, X, 3)
+    assert ctx.last_device_status() == (0, 0)
