@@ -411,7 +411,9 @@ int launch_fused1x1(dbp_ctx *ctx, const void *delta, const void *X, const void *
     auto go = [&](auto kern) -> int {
         if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem)) != cudaSuccess)
             return fail_cuda("shared memory size");
-        const int grid = p.ntiles < ctx->sm_count ? p.ntiles : ctx->sm_count;
+        // One CTA per SM, or as many whole rounds of them as keep a CTA's dW accumulators to kMaxMmas (a chunk is four MMAs)
+        const long long most = kMaxMmas / (4 * nch), rounds = (p.ntiles + most * ctx->sm_count - 1) / (most * ctx->sm_count);
+        const long long grid = p.ntiles < ctx->sm_count * rounds ? p.ntiles : ctx->sm_count * rounds;
         return cuda_ok(launch_chained(kern, dim3(static_cast<unsigned>(grid)), dim3(kThreadsF), smem, ctx->stream, map_w, map_x, map_dx,
                                       map_dw, step, p));
     };

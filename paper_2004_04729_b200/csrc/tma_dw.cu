@@ -220,11 +220,9 @@ int launch_tma_dw(dbp_ctx *ctx, const void *codes_bf16, const void *X, int piece
     p.ci_tiles = static_cast<int>((s.Cin + p.NT - 1) / p.NT);
     const long long co_tiles = (s.Cout + 128 * p.MA - 1) / (128 * p.MA);
     const long long tiles = co_tiles * p.ci_tiles;
-    long long per = 0;
-    // (an MMA takes 16 of a chunk's 64 positions)
-    const long long nsplit = choose_split(tiles, p.nchunks, ctx->sm_count, pieces == 2 ? kMaxMmas / 4 : p.nchunks, &per);
+    // (a chunk of 64 positions is four MMAs)
+    const long long nsplit = choose_split(tiles, p.nchunks, ctx->sm_count, kMaxMmas / 4, &p.per_split);
     p.nsplit = static_cast<int>(nsplit);
-    p.per_split = per;
     p.err_flag = err_flag;
     p.stats = ctx->wait_stats;
     p.delta_p = delta_p;

@@ -65,3 +65,16 @@ def test_3x3_weight_gradients(ctx, dtype, B, Ci, Co, H, W):
         out = dbp.dithered_conv_backward(ctx, d, X, Wt, 3, 1.0, need_dX=need_dX)
         _check_dW(out["dW"], codes, delta, X, 3)
     assert ctx.last_device_status() == (0, 0)
+
+
+@pytest.mark.parametrize("dtype,B,Ci,Co,H,W", [
+    ("bf16", 1024, 64, 64, 56, 56),     # quantization and products in one kernel, whose dW accumulators live as long as it does
+    ("bf16", 400, 72, 200, 56, 56),     # the same with two panels of output channels
+    ("bf16", 1500, 512, 512, 14, 14),   # few tiles, long reductions
+    ("f32", 700, 512, 512, 14, 14)])
+def test_1x1_weight_gradients(ctx, dtype, B, Ci, Co, H, W):
+    import paper_2004_04729_b200 as dbp
+    d, X, Wt, codes, delta = _layer(ctx, dtype, B, Ci, Co, H, W, 1)
+    _check_dW(dbp.dithered_conv_backward(ctx, d, X, Wt, 3, 1.0)["dW"], codes, delta, X, 1)
+    assert ctx.last_step()[1] == int((codes != 0).sum())
+    assert ctx.last_device_status() == (0, 0)
