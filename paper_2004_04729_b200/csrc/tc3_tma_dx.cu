@@ -56,6 +56,8 @@ struct Dx3T {
     int B, Cin, Cout, H, W, Wp;
     int KS;                       // CTAs (a cluster) that share a tile's reduction; > 1: one tile per cluster
     int split;                    // the low piece of the weights is the upper panel (fp32, Cin <= 64)
+    int slots;                    // weight slots per block of co and pass (in phase mode of the tiles with one live kernel row)
+    int passes;                   // 2: the low pieces of the weights first, over all blocks of co, then the high ones
     int Ht;                       // image rows per patch
     int nb;                       // images per patch (> 1 only when Ht == H)
     int tiles_y;                  // patches per image (nb == 1)
@@ -251,7 +253,10 @@ tc3_tma_dx_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
     // Weight slots per 64-channel block of co. In phase mode a slot is one kernel row's taps kx = 0, 1, and only rows that
     // carry weights in the tile's phase have one: ky = 1 (py = 0), or ky = 0 and 1 (py = 1).
     auto phase_of = [&](long long t) { return static_cast<int>(t % p.ci_tiles) * 128 / p.phase_cin; };
-    auto slots_of = [&](long long t) { return p.phase_cin == 0 ? p.ntaps / p.G : ((phase_of(t) & 2) ? 2 : 1) * (p.ntaps / 9); };
+    auto slots_of = [&](long long t) { return p.phase_cin > 0 && (phase_of(t) & 2) ? 2 * p.slots : p.slots; };
+    // what a tile goes through: blocks of co, in two passes once with the low and once with the high pieces of the weights
+    const int ncbl = c_hi - c_lo, nblk = p.passes * ncbl;
+    auto block_of = [&](int i) { return c_lo + (i < ncbl ? i : i - ncbl); };
 
     if (warp == 0) {
         if (lane == 0) {
@@ -262,11 +267,11 @@ tc3_tma_dx_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
             for (long long t = t_first; t < p.ntiles && ok; t += t_step) {
                 int ci0, b0, y0;
                 tile_of(t, ci0, b0, y0);
-                for (int c = c_lo; c < c_hi && ok; ++c) {
+                for (int i = 0; i < nblk; ++i) {
                     ok = mbar_wait_timed(&pipe.q_empty[s], parity, p.err_flag, waited);
                     if (!ok) break;
                     mbar_expect_tx(&pipe.q_full[s], static_cast<unsigned>(p.q_tx));
-                    tma_load_4d(q_s + s * p.q_bytes, &map_q, c * 64, -1, y0 - 1, b0, &pipe.q_full[s]);
+                    tma_load_4d(q_s + s * p.q_bytes, &map_q, block_of(i) * 64, -1, y0 - 1, b0, &pipe.q_full[s]);
                     if (++s == p.nq) { s = 0; parity ^= 1u; }
                 }
             }
@@ -284,7 +289,8 @@ tc3_tma_dx_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
                 int ci0, b0, y0;
                 tile_of(t, ci0, b0, y0);
                 const int slots = slots_of(t);
-                for (int c = c_lo; c < c_hi && ok; ++c)
+                for (int i = 0; i < nblk && ok; ++i) {
+                    const int c = block_of(i), low = p.passes == 2 && i < ncbl ? 1 : 0;       // low: the piece of a two-pass tile
                     for (int g = 0; g < slots; ++g) {
                         if (!p.resident) {
                             ok = mbar_wait_timed(&pipe.w_empty[s], parity, p.err_flag, waited);
@@ -297,10 +303,10 @@ tc3_tma_dx_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
                             mbar_expect_tx(&pipe.w_full[s], static_cast<unsigned>(p.w_slot));
                             for (int h = 0; h < p.a_panels; ++h)
                                 tma_load_3d(dst + h * p.G * kWPanel, &map_w, p.split ? 0 : ci0 + 64 * h, c * 64,
-                                            g * p.G + (p.split ? 9 * h : 0), &pipe.w_full[s]);
+                                            g * p.G + 9 * (p.split ? h : low), &pipe.w_full[s]);
                         } else {
                             const int ph = phase_of(t), ky = (ph & 2) ? g & 1 : 1, kx0 = (ph & 1) ? 0 : 1;
-                            const int piece = (ph & 2) ? g >> 1 : g;
+                            const int piece = p.passes == 2 ? low : (ph & 2) ? g >> 1 : g;
                             mbar_expect_tx(&pipe.w_full[s], static_cast<unsigned>((2 - kx0) * 2 * kWPanel));
                             for (int kx = kx0; kx < 2; ++kx)
                                 for (int h = 0; h < 2; ++h)
@@ -308,6 +314,7 @@ tc3_tma_dx_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
                         }
                         if (++s == p.nw) { s = 0; parity ^= 1u; }
                     }
+                }
                 if (p.resident) break;             // one ci block: every tile uses the same weights (all slots are loaded now)
             }
             report_wait(p.stats, 4, waited);
@@ -327,21 +334,21 @@ tc3_tma_dx_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
         // stored) instead of whatever follows the slot
         const unsigned long long w_desc = make_desc(smem_u32(w_s), p.a_panels == 2 ? p.G * kWPanel : 0, 1024);
         const unsigned q_step = static_cast<unsigned>(p.q_bytes) >> 4, w_step = static_cast<unsigned>(p.w_slot) >> 4;
-        const int slot = warp - 2, ncbl = c_hi - c_lo;
+        const int slot = warp - 2;
         const unsigned tmem_d = tmem_base + slot * kAccCols;
         bool ok = true;
         long long wq = 0, ww = 0, wa = 0;
         const long long born = clock64();
         int it = slot;
-        unsigned n_w = slot ? ncbl * slots_of(t_first) : 0;
+        unsigned n_w = slot ? nblk * slots_of(t_first) : 0;
         for (long long t = t_first + slot * t_step; t < p.ntiles && ok; t += 2 * t_step, it += 2) {
             // ring positions of this tile's first patch and weight slot (and, behind them, of this warp's next tile)
-            const unsigned n_q = static_cast<unsigned>(it) * ncbl;
+            const unsigned n_q = static_cast<unsigned>(it) * nblk;
             const int slots = slots_of(t);
             int qs = n_q % p.nq, ws = n_w % p.nw;
             unsigned qpar = (n_q / p.nq) & 1u, wpar = (n_w / p.nw) & 1u;
             if (p.resident) { ws = 0; wpar = 0; }          // completed barriers stay passable on parity 0
-            n_w += ncbl * (slots + slots_of(t + t_step));
+            n_w += nblk * (slots + slots_of(t + t_step));
             unsigned acc_on = 0u;
             const int ph = p.phase_cin > 0 ? phase_of(t) : 0;
             ok = __all_sync(0xffffffffu, mbar_wait_timed(&pipe.acc_empty[slot], ((static_cast<unsigned>(it) >> 1) & 1u) ^ 1u, p.err_flag, wa));
@@ -350,7 +357,7 @@ tc3_tma_dx_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
             if (ok && it > 0)
                 ok = __all_sync(0xffffffffu, mbar_wait(&pipe.turn[slot], ((static_cast<unsigned>(it - 1) >> 1)) & 1u, p.err_flag));
             if (!ok) break;
-            for (int c = c_lo; c < c_hi && ok; ++c) {
+            for (int i = 0; i < nblk && ok; ++i) {
                 ok = __all_sync(0xffffffffu, mbar_wait_timed(&pipe.q_full[qs], qpar, p.err_flag, wq));
                 if (!ok) break;
                 const unsigned long long bd0 = q_desc + static_cast<unsigned>(qs) * q_step;
@@ -358,7 +365,7 @@ tc3_tma_dx_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
                 for (int g = 0; g < slots && ok; ++g) {
                     ok = __all_sync(0xffffffffu, mbar_wait_timed(&pipe.w_full[ws], wpar, p.err_flag, ww));
                     if (!ok) break;
-                    if (c == c_hi - 1 && g == slots - 1 && elect_one()) mbar_arrive(&pipe.turn[slot ^ 1]);
+                    if (i == nblk - 1 && g == slots - 1 && elect_one()) mbar_arrive(&pipe.turn[slot ^ 1]);
                     tc_fence_after();
                     unsigned long long ad = w_desc + static_cast<unsigned>(ws) * w_step;
                     if (p.phase_cin > 0) {
@@ -665,14 +672,18 @@ int round_up(int v, int m) { return (v + m - 1) / m * m; }
 
 // Shapes the TMA-fed 3x3 kernels take. fp32 operands are split into two bf16 pieces each (the codes are exact in bf16);
 // rows of the codes, of the re-laid weights and of the activations that are no multiple of 16 bytes are padded to one.
-bool tc3_tma_supported(const ConvShape &s, int io) {
-    return (io == DBP_BF16 || io == DBP_F32) && s.k == 3 && s.W >= 1 && s.W <= 62 && s.H <= 4096 && s.B * s.H * s.W < (1ll << 30);
+// An fp32 dX keeps to kMaxMmas per accumulator, and its reduction is cut into eight parts at most.
+constexpr int kMaxKS = 8;
+constexpr int kMaxBlocks = kMaxMmas / 36;        // 64-channel blocks of co per accumulator: nine taps of four MMAs each
+bool tc3_tma_supported(const ConvShape &s, int io, bool dx_f32) {
+    return (io == DBP_BF16 || io == DBP_F32) && s.k == 3 && s.W >= 1 && s.W <= 62 && s.H <= 4096 && s.B * s.H * s.W < (1ll << 30) &&
+           (!dx_f32 || s.Cout <= 64ll * kMaxBlocks * kMaxKS);
 }
 
 // DBP_EUNSUPPORTED: the shape does not fit (the caller uses another kernel)
 int launch_tc3_tma_dx(dbp_ctx *ctx, const void *codes_nhwc, const void *W, int io, const float *delta_p,
                       const ConvShape &s, void *dX, bool dx_bf16, int *err_flag, bool weights_ready, bool *lean) {
-    if (!tc3_tma_supported(s, io)) return DBP_EUNSUPPORTED;
+    if (!tc3_tma_supported(s, io, !dx_bf16)) return DBP_EUNSUPPORTED;
     Dx3T p{};
     p.delta_p = delta_p; p.dX = dX; p.dx_f32 = dx_bf16 ? 0 : 1;
     p.es = dx_bf16 ? 2 : 4;
@@ -684,7 +695,12 @@ int launch_tc3_tma_dx(dbp_ctx *ctx, const void *codes_nhwc, const void *W, int i
     p.phase_cin = (ctx->phase_cin > 0 && ctx->phase_cin % 128 == 0 && s.Cin == 4ll * ctx->phase_cin) ? ctx->phase_cin : 0;
     p.ncb = (p.Cout + 63) / 64;
     p.ci_tiles = (p.Cin + 127) / 128;
-    p.split = io == DBP_F32 && p.Cin <= 64 ? 1 : 0;
+    // Parts of a long reduction (an fp32 result's: bf16 rounds far coarser than the accumulators do). The two pieces of fp32
+    // weights then take a pass each, low ones first, because an MMA costs an accumulator as much for a small term as for a
+    // large one: up to kMaxBlocks / 2 blocks the sum of both pieces keeps to kMaxMmas anyway, and a block's codes are read once.
+    int min_ks = 1;
+    while (p.es == 4 && min_ks * kMaxBlocks < p.ncb) min_ks *= 2;
+    p.split = io == DBP_F32 && p.Cin <= 64 && min_ks == 1 ? 1 : 0;
     p.a_panels = p.Cin <= 64 && !p.split ? 1 : 2;
     const int map_taps = p.ntaps;
     if (p.split) p.ntaps = 9;
@@ -701,6 +717,8 @@ int launch_tc3_tma_dx(dbp_ctx *ctx, const void *codes_nhwc, const void *W, int i
     auto consider = [&](int ht, int nb, int ks) -> bool {
         Dx3T q = p;
         q.Ht = ht; q.nb = nb; q.KS = ks;
+        const int cbs = (p.ncb + ks - 1) / ks;
+        q.passes = p.ntaps == 18 && 2 * cbs > kMaxBlocks ? 2 : 1;
         q.tiles_y = (p.H + ht - 1) / ht;
         q.run = ht * p.W;
         // by the copy engine where every run starts on 16 bytes, a row is whole words of at least four columns (tensor memory
@@ -720,7 +738,7 @@ int launch_tc3_tma_dx(dbp_ctx *ctx, const void *codes_nhwc, const void *W, int i
         q.ntiles = q.pos_tiles * p.ci_tiles;
         // one round of clusters; a GPC's SMs are no multiple of 4 or 8, so not all of them can be covered (36 clusters of 4
         // took 39 us where 32 took 24)
-        if (ks > 1 && q.ntiles * ks > (ks == 2 ? sms : ks == 4 ? sms * 7 / 8 : sms * 3 / 4)) return true;
+        if (ks > min_ks && q.ntiles * ks > (ks == 2 ? sms : ks == 4 ? sms * 7 / 8 : sms * 3 / 4)) return true;
         if (small && (q.ntiles * ks > sms || ks != wide_ks)) return true;      // (the order of a sum does not depend on what else is asked for)
         // an odd number of 32-bit words per row: the 32 channels of a warp hit 32 different banks when they stage the same
         // position
@@ -751,14 +769,14 @@ int launch_tc3_tma_dx(dbp_ctx *ctx, const void *codes_nhwc, const void *W, int i
         }
         if (q.nw > kMaxW) q.nw = kMaxW;
         q.w_slot = static_cast<int>(q.G * tap_bytes);
+        q.slots = (p.phase_cin > 0 ? p.ntaps / 9 : p.ntaps / q.G) / q.passes;
         const double live = p.phase_cin > 0 ? 0.25 : 1.0;
         const long long ctas = q.ntiles * ks, waves = (ctas + sms - 1) / sms, active = ctas < sms ? ctas : sms;
         double mma = 32.0 + 0.25 * q.N + (q.resident ? 0.0 : 16.0 * p.a_panels);
         if (mma < 0.5 * q.N) mma = 0.5 * q.N;
         const double l2 = q.resident ? 0.0 : 2048.0 * p.a_panels * static_cast<double>(active) / 6000.0;
         if (mma < l2) mma = l2;
-        const int cbs = (p.ncb + ks - 1) / ks;
-        const double body = cbs * (p.ntaps * live * 4.0 * mma + (q.resident ? 0.0 : 250.0 * (p.phase_cin > 0 ? p.ntaps / 6.0 : static_cast<double>(p.ntaps) / q.G)) + q.q_tx / 128.0 + 300.0);
+        const double body = cbs * (p.ntaps * live * 4.0 * mma + (q.resident ? 0.0 : 250.0 * (p.phase_cin > 0 ? p.ntaps / 6.0 : static_cast<double>(p.ntaps) / q.G)) + q.passes * (q.q_tx / 128.0 + 300.0));
         const double staged = (p.Cin <= 64 && !p.split ? 64.0 : 128.0) * nb * q.run * es;
         const double epi = (q.unit > 0 ? 1000.0 + staged / 40.0 : 2000.0 + staged / 20.0) + (ks > 1 ? 2000.0 + staged / 8.0 : 0.0);
         const double cost = static_cast<double>(waves) * (500.0 + (body > epi ? body : epi)) + (waves > 1 ? (body < epi ? body : epi) : epi);
@@ -773,8 +791,8 @@ int launch_tc3_tma_dx(dbp_ctx *ctx, const void *codes_nhwc, const void *W, int i
     };
     auto search = [&] {
         for (int ht = 1; ht <= p.H; ++ht)
-            if (!consider(ht, 1, 1)) break;
-        for (int ks = 1; ks <= 8; ks *= 2) {
+            if (!consider(ht, 1, min_ks)) break;
+        for (int ks = min_ks; ks <= kMaxKS; ks *= 2) {
             if (ks > p.ncb || (ks > 1 && p.split)) break;
             for (int nb = ks > 1 ? 1 : 2; nb <= 64 && nb <= p.B; ++nb)
                 if (!consider(p.H, nb, ks)) break;

@@ -78,3 +78,55 @@ def test_1x1_weight_gradients(ctx, dtype, B, Ci, Co, H, W):
     _check_dW(dbp.dithered_conv_backward(ctx, d, X, Wt, 3, 1.0)["dW"], codes, delta, X, 1)
     assert ctx.last_step()[1] == int((codes != 0).sum())
     assert ctx.last_device_status() == (0, 0)
+
+
+def _check_dX(dX, codes, delta, W, k):
+    """The first and the last image, a few channels, every position."""
+    ci, im = _some(dX.shape[1]), torch.tensor([0, dX.shape[0] - 1], device="cuda")
+    q, w = codes[im].double(), W[:, ci].double()
+    ref = sum(torch.einsum("bcyx,cd->bdyx", q if k == 1 else _shifted(q, 1 - ky, 1 - kx), w[:, :, ky, kx]) for ky in range(k) for kx in range(k))
+    rel = ((dX[im][:, ci].double() - delta * ref) / (delta * ref)).abs().max().item()
+    assert rel <= TOL, rel
+
+
+@pytest.mark.parametrize("dtype,B,Ci,Co,H,W", [
+    ("f32", 8, 128, 512, 28, 28),       # the low pieces of the weights in a pass of their own
+    ("f32", 3, 72, 520, 9, 31),         # the same, ragged
+    ("f32", 8, 128, 1000, 28, 28),      # the reduction in two parts
+    ("f32", 2, 200, 2100, 5, 62),       # in four; rows as long as the kernel takes
+    ("f32", 4, 64, 2048, 28, 28),       # few channels: no longer both pieces on one accumulator's lanes
+    ("f32", 40, 24, 5000, 4, 4),        # in eight; several images per patch
+    ("bf16", 4, 128, 2048, 28, 28), ("bf16", 2, 40, 1030, 17, 12)])
+def test_3x3_input_gradients(ctx, dtype, B, Ci, Co, H, W):
+    import paper_2004_04729_b200 as dbp
+    d, X, Wt, codes, delta = _layer(ctx, dtype, B, Ci, Co, H, W, 3)
+    out = dbp.dithered_conv_backward(ctx, d, X, Wt, 3, 1.0, flags=dbp.DBP_DX_F32 | dbp.DBP_FORCE_DENSE * (Co % 8 == 0))
+    _check_dX(out["dX"], codes, delta, Wt, 3)
+    alone = dbp.dithered_conv_backward(ctx, d, X, Wt, 3, 1.0, need_dW=False, flags=dbp.DBP_DX_F32)["dX"]
+    assert torch.equal(alone, out["dX"])         # one order of the sums, whatever else is asked for
+    assert ctx.last_device_status() == (0, 0)
+
+
+def test_3x3_input_gradient_of_more_channels_than_the_parts_hold(ctx):
+    """fp32 from 7169 output channels on: the gather kernels (and none of the tensor cores' when those are insisted on)."""
+    import paper_2004_04729_b200 as dbp
+    d, X, Wt, codes, delta = _layer(ctx, "f32", 1, 8, 7176, 5, 5, 3)
+    _check_dX(dbp.dithered_conv_backward(ctx, d, X, Wt, 3, 1.0)["dX"], codes, delta, Wt, 3)
+    with pytest.raises(dbp.DbpError):
+        dbp.dithered_conv_backward(ctx, d, X, Wt, 3, 1.0, flags=dbp.DBP_FORCE_DENSE)
+
+
+@pytest.mark.parametrize("Ci,Co", [(128, 512), (128, 1024), (256, 72)])
+def test_stride_2_input_gradients_in_parts(ctx, Ci, Co):
+    """The phase images of a stride-2 layer go through the same passes and parts; positions (y, x) of dX take the taps whose
+    parity fits."""
+    import paper_2004_04729_b200 as dbp
+    B, H, W = 2, 12, 20
+    d, _, Wt, codes, delta = _layer(ctx, "f32", B, Ci, Co, H // 2, W // 2, 3)
+    X = torch.ones(B, Ci, H, W, device="cuda")
+    dX = dbp.dithered_conv_backward(ctx, d, X, Wt, 3, 1.0, stride=2)["dX"]
+    ci = _some(Ci)
+    up = torch.zeros(B, Co, H, W, dtype=torch.float64, device="cuda")
+    up[:, :, ::2, ::2] = codes.double()
+    ref = delta * sum(torch.einsum("bcyx,cd->bdyx", _shifted(up, 1 - ky, 1 - kx), Wt[:, ci, ky, kx].double()) for ky in range(3) for kx in range(3))
+    assert ((dX[:, ci].double() - ref).abs() <= TOL * ref).all()
