@@ -264,7 +264,7 @@ small_linear_products_kernel(const SmallLinP p) {
     // warp tiling of the 64 x 64 tile: 16 rows x 16 columns per warp (two 16 x 8 accumulators)
     const int wr = (warp >> 2) * 16, wc = (warp & 3) * 16;
     const int g = lane >> 2, tig = lane & 3;
-    float acc[2][4] = {};
+    float acc[2][4] = {}, sum[2][4] = {};
     float dbacc[8] = {};
 
     auto load_b = [&](long long r0, float4 (&b_reg)[2]) {
@@ -384,6 +384,9 @@ small_linear_products_kernel(const SmallLinP p) {
     for (int c0 = 0; c0 < nchunks; c0 += p.chunks) {
         count = nchunks - c0 < p.chunks ? nchunks - c0 : p.chunks;
         if (c0 > 0) {
+            // an accumulator is truncated when an MMA adds to it: after the 64 MMAs of eight chunks it is added to a sum that rounds
+#pragma unroll
+            for (int i = 0; i < 8; ++i) { sum[i >> 2][i & 3] += acc[i >> 2][i & 3]; acc[i >> 2][i & 3] = 0.f; }
             __syncthreads();                             // the previous chunks have been used
             fill_b(static_cast<long long>(c0) * kRed, count);
         }
@@ -416,7 +419,7 @@ small_linear_products_kernel(const SmallLinP p) {
             const long long col = k0 + wc + 8 * tn + 2 * tig;
             if (row >= nrows || col >= p.K) continue;
             float *dst = out + row * p.K + col;
-            const float v0 = acc[tn][2 * h] * dscale, v1 = acc[tn][2 * h + 1] * dscale;
+            const float v0 = (sum[tn][2 * h] + acc[tn][2 * h]) * dscale, v1 = (sum[tn][2 * h + 1] + acc[tn][2 * h + 1]) * dscale;
             if ((p.K & 1) == 0) {
                 *reinterpret_cast<float2 *>(dst) = make_float2(v0, v1);
             } else {

@@ -130,3 +130,20 @@ def test_stride_2_input_gradients_in_parts(ctx, Ci, Co):
     up[:, :, ::2, ::2] = codes.double()
     ref = delta * sum(torch.einsum("bcyx,cd->bdyx", _shifted(up, 1 - ky, 1 - kx), Wt[:, ci, ky, kx].double()) for ky in range(3) for kx in range(3))
     assert ((dX[:, ci].double() - ref).abs() <= TOL * ref).all()
+
+
+@pytest.mark.parametrize("dtype,B,N,K,want", [
+    ("f32", 8192, 16, 64, "dW"), ("f32", 2, 60000, 72, "dX"),       # one tile's reduction on warp-level MMAs
+    ("f32", 16384, 300, 256, "dW"), ("f32", 300, 8192, 256, "dX"),  # the longest parts of the CTA-wide kernel
+    ("f32", 260, 8300, 128, "both"),                                # beyond them: the gather kernels
+    ("bf16", 32768, 320, 512, "dW"), ("bf16", 300, 8192, 512, "dX")])
+def test_linear_layers(ctx, dtype, B, N, K, want):
+    import paper_2004_04729_b200 as dbp
+    d, X, Wt, codes, delta = _layer(ctx, dtype, B, K, N, 1, 1, 1)
+    out = dbp.dithered_linear_backward(ctx, d.view(B, N), X.view(B, K), Wt.view(N, K), 3, 1.0, need_dW=want != "dX", need_dX=want != "dW",
+                                       flags=dbp.DBP_DX_F32)
+    if want != "dX":
+        _check_dW(out["dW"].view(N, K, 1, 1), codes, delta, X, 1)
+    if want != "dW":
+        _check_dX(out["dX"].view(B, K, 1, 1), codes, delta, Wt, 1)
+    assert ctx.last_device_status() == (0, 0)
