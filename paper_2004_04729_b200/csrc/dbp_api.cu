@@ -725,7 +725,7 @@ int dbp_destroy(dbp_ctx *ctx) {
     cudaStreamSynchronize(ctx->stream);
     if (ctx->aux) cudaStreamSynchronize(ctx->aux);
     Workspace *all[] = {&ctx->dense_codes[0], &ctx->dense_codes[1], &ctx->codes16[0], &ctx->codes16[1],
-                        &ctx->codes_nhwc[0], &ctx->codes_nhwc[1], &ctx->codes_stack[0], &ctx->codes_stack[1], &ctx->dz_tmp, &ctx->s2_x, &ctx->s2_w, &ctx->s2_dx, &ctx->s2_dw, &ctx->dw_acc, &ctx->x_padded[0], &ctx->x_padded[1], &ctx->rows_x, &ctx->rows_w, &ctx->db_sums, &ctx->w_taps, &ctx->sp_bitmap, &ctx->sp_offsets, &ctx->sp_values};
+                        &ctx->codes_nhwc[0], &ctx->codes_nhwc[1], &ctx->codes_stack[0], &ctx->codes_stack[1], &ctx->dz_tmp, &ctx->s2_x, &ctx->s2_w, &ctx->s2_dx, &ctx->s2_dw, &ctx->dw_acc, &ctx->x_padded[0], &ctx->x_padded[1], &ctx->rows_x, &ctx->rows_w, &ctx->db_sums, &ctx->w_taps};
     for (Workspace *w : all) if (w->ptr) cudaFree(w->ptr);
     for (Workspace &w : ctx->io) if (w.ptr) cudaFree(w.ptr);
     for (ProfSlot &p : ctx->prof) { cudaEventDestroy(p.begin); cudaEventDestroy(p.end); }

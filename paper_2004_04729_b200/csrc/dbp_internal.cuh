@@ -61,7 +61,6 @@ struct dbp_ctx {
     dbp::Workspace rows_x, rows_w;      // operands re-written as bf16 rows the copy engine can address: a linear layer's X, W
     dbp::Workspace codes16[2];          // bf16 code planes for the TMA-fed kernels
     dbp::Workspace w_taps;              // fp32 weights as [Cout][k*k][Cin]
-    dbp::Workspace sp_bitmap, sp_offsets, sp_values;  // internal dbp_sparse
     dbp::Workspace codes_nhwc[2];       // bf16 codes [B][position][Cout] for the TMA-fed 3x3 kernels
     const uint8_t *next_mask = nullptr; // ReLU mask for the next backward call (dbp_set_relu_mask)
     dbp::Workspace dz_tmp;              // delta_z = delta_a (.) mask when that call cannot fold the mask into its loads

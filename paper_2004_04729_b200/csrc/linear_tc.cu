@@ -39,8 +39,8 @@ struct LinProduct {
     int a_kmajor;                 // A is [M][reduction] (dX) instead of [reduction][M] (dW)
     int ks, pieces, steps;        // 64-deep steps per piece; steps of all pieces
     int per_split, nsplit;
-    int mt, nt;
-    int tiles;                    // mt * nt * nsplit
+    int mt;
+    int tiles;                    // mt * column tiles * nsplit
 };
 
 struct LinArgs {
@@ -279,10 +279,9 @@ bool fits_int(long long v) { return v > 0 && v < (1ll << 30); }
 
 }  // namespace
 
-// An accumulator is truncated, not rounded, when an MMA adds to it: about 1e-8 of its value per MMA (measured: a sum of
-// 2500 MMAs came out 3e-5 low). Reductions are kept to kMaxSteps steps of four MMAs per accumulator: longer ones of dW
-// are split; a longer one of an fp32 dX (more than 8192 outputs) is left to the gather kernels.
-constexpr long long kMaxSteps = 128;
+// Steps of four MMAs per accumulator (see kMaxMmas): longer reductions of dW are split; a longer one of an fp32 layer's dX
+// (more than 8192 outputs) is left to the gather kernels.
+constexpr long long kMaxSteps = kMaxMmas / 4;
 
 bool linear_tc_supported(long long B, long long N, long long K, int pieces) {
     return fits_int(B) && fits_int(N) && fits_int(K) && (pieces == 1 || (N + 63) / 64 <= kMaxSteps);
@@ -360,7 +359,6 @@ int launch_linear_products(dbp_ctx *ctx, const LinearPlan &pl, const void *codes
         q.per_split = is_dx ? q.steps : static_cast<int>(pl.dw_per_split);
         q.add = q.nsplit > 1;
         q.mt = (q.M + 127) / 128;
-        q.nt = nt;
         const long long tiles = static_cast<long long>(q.mt) * nt * q.nsplit;
         if (tiles + p.tiles >= (1ll << 30)) return DBP_EUNSUPPORTED;
         q.tiles = static_cast<int>(tiles);

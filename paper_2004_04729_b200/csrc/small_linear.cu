@@ -481,8 +481,7 @@ int launch_small_linear(dbp_ctx *ctx, const float *delta, const float *X, const 
     if (int rc = cuda_ok(launch_chained_cluster(kern, static_cast<unsigned>(ctas), static_cast<unsigned>(ctas), dim3(kThreads), 0, ctx->stream, p))) return rc;
     const long long red = (dW && (!dX || B > N)) ? B : N;               // the longest reduction of the tiles
     const long long chunks = (red + kRed - 1) / kRed;
-    const int most = p.n_dw + p.n_dx > ctx->sm_count ? kMaxChunks / 2 : kMaxChunks;      // two CTAs per SM when there are more tiles
-    p.chunks = chunks < most ? static_cast<int>(chunks) : most;
+    p.chunks = chunks < kMaxChunks ? static_cast<int>(chunks) : kMaxChunks;
     const size_t smem = static_cast<size_t>(p.chunks) * 3 * kChunkTile * 2;
     if (cudaFuncSetAttribute(small_linear_products_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              kMaxChunks * 3 * kChunkTile * 2) != cudaSuccess)

@@ -41,7 +41,7 @@ constexpr int kXSlot = kXS * kXTile;
 constexpr int kMaxNX = 6;
 
 struct Dw3T {
-    int Cin, Cout, W, HW;
+    int Cout, W, HW;
     int code_batch;               // images of the code tensor (the activations may hold two pieces of every image, one after the other)
     int split;                    // both pieces of (at most 64) channels share a tile: rows 0-63 the high ones, 64-127 the low ones
     int SEG;                      // positions per segment (multiple of 64)
@@ -518,7 +518,7 @@ int launch_tc3_tma_dw(dbp_ctx *ctx, const void *codes_nhwc, const void *X, int p
     const long long cin_pad = (s.Cin + 7) / 8 * 8, q_pitch = (s.Cout + 7) / 8 * 8;
     const long long HW = s.H * s.W;
     Dw3T p{};
-    p.Cin = static_cast<int>(cin_pad); p.Cout = static_cast<int>(s.Cout); p.W = static_cast<int>(s.W); p.HW = static_cast<int>(HW);
+    p.Cout = static_cast<int>(s.Cout); p.W = static_cast<int>(s.W); p.HW = static_cast<int>(HW);
     p.err_flag = err_flag;
     p.stats = ctx->wait_stats;
     // half an SM has room for the 192 accumulator columns of 64 output channels (an MMA of N = 192 does as much per clock as

@@ -52,7 +52,6 @@ constexpr int kBlock = 32 * 128;                 // one epilogue warp's [32 ci][
 struct Dx3T {
     const float *delta_p;
     void *dX;
-    int dx_f32;
     int B, Cin, Cout, H, W, Wp;
     int KS;                       // CTAs (a cluster) that share a tile's reduction; > 1: one tile per cluster
     int split;                    // the low piece of the weights is the upper panel (fp32, Cin <= 64)
@@ -685,7 +684,7 @@ int launch_tc3_tma_dx(dbp_ctx *ctx, const void *codes_nhwc, const void *W, int i
                       const ConvShape &s, void *dX, bool dx_bf16, int *err_flag, bool weights_ready, bool *lean) {
     if (!tc3_tma_supported(s, io, !dx_bf16)) return DBP_EUNSUPPORTED;
     Dx3T p{};
-    p.delta_p = delta_p; p.dX = dX; p.dx_f32 = dx_bf16 ? 0 : 1;
+    p.delta_p = delta_p; p.dX = dX;
     p.es = dx_bf16 ? 2 : 4;
     p.ntaps = io == DBP_F32 ? 18 : 9;
     p.B = static_cast<int>(s.B); p.Cin = static_cast<int>(s.Cin); p.Cout = static_cast<int>(s.Cout);

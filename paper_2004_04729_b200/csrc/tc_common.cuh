@@ -1,4 +1,4 @@
-// tcgen05 / mbarrier / cp.async wrappers shared by the tensor-core kernels (inline PTX for sm_100a).
+// tcgen05 / mbarrier / bulk-copy wrappers shared by the tensor-core kernels (inline PTX for sm_100a).
 #pragma once
 
 #include "dbp_internal.cuh"
@@ -23,23 +23,6 @@ __device__ __forceinline__ void mbar_arrive(unsigned long long *bar) {
 __device__ __forceinline__ void warp_arrive(unsigned long long *bar) {
     __syncwarp();
     if ((threadIdx.x & 31) == 0) mbar_arrive(bar);
-}
-// cp.async groups: a thread closes a group after the copies of one stage and later waits until
-// at most `pending` newer groups are still in flight
-__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
-__device__ __forceinline__ void cp_async_wait_pending(int pending) {
-    switch (pending) {
-        case 5: asm volatile("cp.async.wait_group 5;" ::: "memory"); break;
-        case 4: asm volatile("cp.async.wait_group 4;" ::: "memory"); break;
-        case 3: asm volatile("cp.async.wait_group 3;" ::: "memory"); break;
-        case 2: asm volatile("cp.async.wait_group 2;" ::: "memory"); break;
-        case 1: asm volatile("cp.async.wait_group 1;" ::: "memory"); break;
-        default: asm volatile("cp.async.wait_group 0;" ::: "memory"); break;   // fewer pending is always safe
-    }
-}
-// arrival that fires when this thread's earlier cp.async copies have landed
-__device__ __forceinline__ void mbar_arrive_on_cp_async(unsigned long long *bar) {
-    asm volatile("cp.async.mbarrier.arrive.noinc.shared::cta.b64 [%0];" ::"r"(smem_u32(bar)) : "memory");
 }
 // Waits for the phase with the given parity. try_wait suspends the thread in hardware until the
 // phase completes or a short system time limit passes, so a waiter wakes as soon as the barrier
@@ -135,18 +118,6 @@ __device__ __forceinline__ void tmem_ld32(unsigned taddr, unsigned (&r)[32]) {
         : "r"(taddr));
     asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 }
-__device__ __forceinline__ void cp_async16(void *smem_dst, const void *gsrc, bool valid) {
-    const int n = valid ? 16 : 0;   // src-size 0: the 16 bytes are zero-filled
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(smem_u32(smem_dst)), "l"(gsrc), "r"(n) : "memory");
-}
-
-// 4- or 8-byte asynchronous copy (zero-filled when !valid); both addresses aligned to the size
-template <int BYTES>
-__device__ __forceinline__ void cp_async_small(void *smem_dst, const void *gsrc, bool valid) {
-    static_assert(BYTES == 4 || BYTES == 8, "cp.async.ca copies 4, 8 or 16 bytes");
-    const int n = valid ? BYTES : 0;
-    asm volatile("cp.async.ca.shared.global [%0], [%1], %2, %3;" ::"r"(smem_u32(smem_dst)), "l"(gsrc), "n"(BYTES), "r"(n) : "memory");
-}
 
 // Shared-memory matrix descriptor, 128-byte swizzle, descriptor version 1; lbo/sbo in bytes.
 // K-major operand: rows of 64 K-elements, 8-row groups sbo apart (lbo unused).
@@ -166,33 +137,6 @@ __host__ __device__ constexpr unsigned make_idesc(int M, int N, bool a_mn_major,
     return (1u << 4) | (1u << 7) | (1u << 10) | (a_mn_major ? (1u << 15) : 0u) | (b_mn_major ? (1u << 16) : 0u) |
            (static_cast<unsigned>(N >> 3) << 17) | (static_cast<unsigned>(M >> 4) << 24);
 }
-
-// byte offset of 16-byte chunk `chunk` (0..7) of row `row` inside a 128-byte-swizzled panel
-__device__ __forceinline__ unsigned swz(unsigned row, unsigned chunk) { return row * 128u + ((chunk ^ (row & 7u)) << 4); }
-
-// four int8 codes packed in a word -> two words of packed bf16 (exact).
-// byte ^ 0x80 = code + 128 as an unsigned byte; 0x4B0000xx read as a float is 2^23 + xx, so
-// subtracting 2^23 + 128 leaves the code as a float whose top 16 bits are its bf16 pattern.
-__device__ __forceinline__ void codes4_to_bf16(unsigned w, unsigned &lo, unsigned &hi) {
-    const unsigned x = w ^ 0x80808080u;
-    const float f0 = __uint_as_float(__byte_perm(x, 0x4B000000u, 0x7650)) - 8388736.0f;
-    const float f1 = __uint_as_float(__byte_perm(x, 0x4B000000u, 0x7651)) - 8388736.0f;
-    const float f2 = __uint_as_float(__byte_perm(x, 0x4B000000u, 0x7652)) - 8388736.0f;
-    const float f3 = __uint_as_float(__byte_perm(x, 0x4B000000u, 0x7653)) - 8388736.0f;
-    lo = __byte_perm(__float_as_uint(f0), __float_as_uint(f1), 0x7632);
-    hi = __byte_perm(__float_as_uint(f2), __float_as_uint(f3), 0x7632);
-}
-// eight int8 codes (two words) -> eight bf16 (one 16-byte chunk)
-__device__ __forceinline__ uint4 expand8(uint2 c) {
-    uint4 o;
-    codes4_to_bf16(c.x, o.x, o.y);
-    codes4_to_bf16(c.y, o.z, o.w);
-    return o;
-}
-__device__ __forceinline__ unsigned short code_to_bf16(int c) {
-    return static_cast<unsigned short>(__float_as_uint(static_cast<float>(c)) >> 16);
-}
-
 
 }  // namespace tc
 }  // namespace dbp

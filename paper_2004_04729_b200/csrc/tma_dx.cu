@@ -416,10 +416,10 @@ tma_dx_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constant__
 
 }  // namespace
 
-// An accumulator is truncated, not rounded, when an MMA adds to it (about 1e-8 of its value per MMA): the reduction of
-// an fp32 layer is kept to 8192 channels here.
+// The reduction of an fp32 layer is kept to kMaxMmas per accumulator, an MMA taking 16 channels (the low pieces of the
+// weights are added first and do not count).
 bool tma_dx_supported(const ConvShape &s, int io) {
-    return s.k == 1 && s.H * s.W > 1 && s.H * s.W < (1ll << 30) && (io == DBP_BF16 || s.Cout <= 8192);
+    return s.k == 1 && s.H * s.W > 1 && s.H * s.W < (1ll << 30) && (io == DBP_BF16 || s.Cout <= 16 * kMaxMmas);
 }
 
 long long tma_code_pitch(const ConvShape &s) { return (s.H * s.W + 7) / 8 * 8; }
