@@ -491,12 +491,14 @@ int conv_backward_impl(dbp_ctx *ctx, const void *delta, const void *X, const voi
                    cudaStreamWaitEvent(ctx->aux, ctx->ev_fork, 0) != cudaSuccess))
         return fail_cuda("forking the dW stream");
     // A 3x3 call that ends with its dW: where dX is one round of CTAs, its kernel and the dW kernel take half of every SM each
-    // and run beside one another, so that one's start and end (loads, partial sums, stores) lie beside the other's MMAs (60
-    // drawn layers: 5.5 % on average, 20 % at best; 512 -> 512 fp32 at 4x4, batch 128: 93 -> 82 us). An overlapped call's dW
-    // runs beside the next layer's quantization instead, and so leaves dX alone (VGG-16 set 864 us with, 828 without). Not
-    // for wide planes of many output channels: the dW kernel's segments get short beside their halos then (30x28: 5 % slower).
+    // and run beside one another, so that one's start and end (loads, partial sums, stores) lie beside the other's MMAs. Of 154
+    // layers on both sides of one round (planes 7 to 56 wide, 32 to 256 channels in, 32 to 512 out, both types) 84 share;
+    // those take 0.89 of their time on average, 0.79 at best, 1.06 at worst (512 outputs of 32 or 64 inputs: their dW is most
+    // of the call and gets half the SM for all of it). Not where the dW kernel does not fit half an SM (bf16 32 -> 72 at 62x60:
+    // 1.06). An overlapped call's dW runs beside the next layer's quantization instead, and so leaves dX alone (VGG-16 set
+    // 864 us with, 828 without).
     bool half = false;
-    const bool share = forked && !(flags & DBP_DW_ASYNC) && (s.W <= 24 || s.Cout <= 64);
+    const bool share = forked && t3 && !(flags & DBP_DW_ASYNC) && tc3_dw_fits_half(s);
     if (dX) {
         KernelTimer t(ctx, DBP_K_DX_DENSE);
         rc = t1 ? launch_tma_dx(ctx, codes16, W, pieces, w_pitch, delta_p, s, dX, dx_bf16, &ctx->state->tc_timeout)

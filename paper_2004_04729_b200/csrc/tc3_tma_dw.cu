@@ -487,7 +487,19 @@ x_split_stacked_kernel(const float *__restrict__ X, __nv_bfloat16 *__restrict__ 
 
 int round_up(int v, int m) { return (v + m - 1) / m * m; }
 
+// The code panel of a segment: its positions and W + 1 more on either side, in boxes of at most 256 rows
+struct Panel { int nload, rows_box, bytes; };
+Panel panel_of(int seg, int W) {
+    const int rows = seg + 2 * (W + 1), nload = (rows + 255) / 256, rows_box = (rows + nload - 1) / nload;
+    return Panel{nload, rows_box, round_up(nload * rows_box * 128, 1024)};
+}
+
 }  // namespace
+
+// Whether the kernel fits half an SM: two code buffers of the shortest segment beside two activation slots (W up to 59)
+bool tc3_dw_fits_half(const ConvShape &s) {
+    return 2 * static_cast<size_t>(panel_of(64, static_cast<int>(s.W)).bytes) + 1024 + 2 * kXSlot <= kHalfSm;
+}
 
 // DBP_EUNSUPPORTED: the shape does not fit (the caller uses another kernel)
 int tc3_stack_images(const ConvShape &s, int io) {
@@ -532,18 +544,15 @@ int launch_tc3_tma_dw(dbp_ctx *ctx, const void *codes_nhwc, const void *X, int p
     const int seg_cap = static_cast<int>(HW < 512 ? (HW + 63) / 64 * 64 : 512);
     size_t smem = 0;
     for (int seg = seg_cap; seg >= 64; seg -= 64) {
-        const int rows = seg + 2 * (p.W + 1);
-        const int nload = (rows + 255) / 256, rows_box = (rows + nload - 1) / nload;
-        const int panel = round_up(nload * rows_box * 128, 1024);
-        const size_t fixed = 2 * static_cast<size_t>(NP) * panel + 1024;
+        const Panel pn = panel_of(seg, p.W);
+        const size_t fixed = 2 * static_cast<size_t>(NP) * pn.bytes + 1024;
         if (fixed + (half ? 2 : 3) * kXSlot > budget) continue;
-        p.SEG = seg; p.nload = nload; p.rows_box = rows_box; p.panel_bytes = panel;
+        p.SEG = seg; p.nload = pn.nload; p.rows_box = pn.rows_box; p.panel_bytes = pn.bytes;
         p.nx = static_cast<int>((budget - fixed) / kXSlot);
         if (p.nx > kMaxNX) p.nx = kMaxNX;
         smem = fixed + static_cast<size_t>(p.nx) * kXSlot;
         break;
     }
-    if (smem == 0 && half) return launch_tc3_tma_dw(ctx, codes_nhwc, X, pieces, x_pitch, delta_p, s, dW, err_flag, false);
     if (smem == 0) return DBP_EUNSUPPORTED;
     p.segs_per_img = (p.HW + p.SEG - 1) / p.SEG;
     p.code_batch = static_cast<int>(s.B);

@@ -26,6 +26,7 @@ def ctx():
     (1, 128, 128, 1, 1, "f32"),
     (3, 64, 64, 13, 32, "f32"), (2, 40, 72, 9, 11, "f32"), (1, 3, 200, 33, 62, "f32"),       # both weight pieces in one MMA
     (9, 40, 72, 6, 24, "bf16"), (5, 200, 72, 6, 25, "f32"), (40, 130, 136, 5, 5, "f32"),       # dX and dW share every SM, or not
+    (3, 64, 72, 26, 26, "f32"), (2, 72, 136, 7, 56, "bf16"), (1, 256, 128, 12, 59, "f32"), (1, 136, 72, 9, 60, "bf16"),   # half an SM: widest rows
     (3, 40, 24, 9, 56, "bf16"), (2, 72, 16, 10, 28, "bf16"), (2, 24, 24, 22, 60, "bf16"),      # dX by whole blocks: partial last
     (2, 136, 40, 11, 16, "f32"), (9, 136, 64, 4, 8, "f32"), (1, 64, 8, 31, 48, "f32")])       # patches, several images, ragged rows
 def test_input_gradient(ctx, B, Ci, Co, H, W, dtype):
