@@ -538,7 +538,7 @@ tc3_tma_dx_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
                     const unsigned tw[16] = {t0.x, t0.y, t0.z, t0.w, t1.x, t1.y, t1.z, t1.w,
                                              t2.x, t2.y, t2.z, t2.w, t3.x, t3.y, t3.z, t3.w};
                     if (p.es == 4 || KS > 1) {
-                        const float f = KS > 1 ? 1.f : delta;      // partial sums are scaled when they have met
+                        const float f = KS > 1 || p.split ? 1.f : delta;      // parts of a sum are scaled when they have met
 #pragma unroll
                         for (int j = 0; j < 32; ++j) {
                             const int o = static_cast<int>(static_cast<short>((tw[j >> 1] >> (16 * (j & 1))) & 0xffffu));
@@ -581,7 +581,7 @@ tc3_tma_dx_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
                         // were what an epilogue took its time for
                         if (p.split) {                           // the low pieces' sums, 64 rows further, and the high pieces'
                             const float *hi = reinterpret_cast<const float *>(src), *lo = reinterpret_cast<const float *>(src + 64 * p.pitch);
-                            copy_run(reinterpret_cast<float *>(dst), len, lane, [&](int i) { return hi[i] + lo[i]; });
+                            copy_run(reinterpret_cast<float *>(dst), len, lane, [&](int i) { return (hi[i] + lo[i]) * delta; });
                         } else if (words) {
                             copy_run(reinterpret_cast<unsigned *>(dst), nwords, lane, [&](int i) { return reinterpret_cast<const unsigned *>(src)[i]; });
                         } else {

@@ -24,7 +24,8 @@ def ctx():
     (3, 128, 576, 2, 2, "bf16"),                                                              # nine blocks of channels over a cluster
     (30, 512, 136, 2, 2, "f32"), (7, 136, 512, 4, 4, "f32"), (2, 264, 128, 14, 14, "f32"),
     (1, 128, 128, 1, 1, "f32"),
-    (3, 64, 64, 13, 32, "f32"), (2, 40, 72, 9, 11, "f32"), (1, 3, 200, 33, 62, "f32"),       # both weight pieces in one MMA
+    (3, 64, 64, 13, 32, "f32"), (2, 40, 72, 9, 11, "f32"), (1, 3, 200, 33, 62, "f32"),       # both weight pieces in one MMA:
+    (9, 56, 352, 16, 16, "f32"), (12, 16, 88, 30, 30, "f32"), (6, 38, 98, 12, 12, "f32"),    # ... in whole blocks or not, as dW asks
     (9, 40, 72, 6, 24, "bf16"), (5, 200, 72, 6, 25, "f32"), (40, 130, 136, 5, 5, "f32"),       # dX and dW share every SM, or not
     (3, 64, 72, 26, 26, "f32"), (2, 72, 136, 7, 56, "bf16"), (1, 256, 128, 12, 59, "f32"), (1, 136, 72, 9, 60, "bf16"),   # half an SM: widest rows
     (3, 40, 24, 9, 56, "bf16"), (2, 72, 16, 10, 28, "bf16"), (2, 24, 24, 22, 60, "bf16"),      # dX by whole blocks: partial last
@@ -43,6 +44,7 @@ def test_input_gradient(ctx, B, Ci, Co, H, W, dtype):
         g = out[key].double().cpu().numpy()
         assert np.linalg.norm(g - ref[key]) <= TOL * np.linalg.norm(ref[key]) + 1e-30, key
         assert np.all(np.abs(g - ref[key]) <= TOL * ref["S_" + key] + 1e-30), key
-    for _ in range(3):
-        again = dbp.dithered_conv_backward(ctx, d, X, Wt, L.seed, L.scale, need_dW=False)["dX"]
-        assert torch.equal(again, out["dX"].to(again.dtype))
+    for kw in ({"need_dW": False}, {"need_dW": False}, {"flags": dbp.DBP_DW_ASYNC}, {}):
+        again = dbp.dithered_conv_backward(ctx, d, X, Wt, L.seed, L.scale, **kw)["dX"]
+        ctx.join()
+        assert torch.equal(again, out["dX"].to(again.dtype)), kw
