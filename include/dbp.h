@@ -50,8 +50,8 @@ typedef enum {
 #define DBP_FORCE_SPARSE 1u /* always use the sparse gather kernels */
 #define DBP_FORCE_DENSE  2u /* always use the dense tensor-core path; DBP_EUNSUPPORTED where it
                                does not exist (it covers bf16 linear and 1x1 layers and bf16 or fp32 3x3
-                               layers, channel counts multiples of 8, 3x3 images up to 62 wide; fp32
-                               operands enter the tensor cores as two bf16 pieces each) */
+                               layers, channel counts multiples of 8, 3x3 images up to 62 wide and, with an fp32 dX, up to
+                               7168 output channels; fp32 operands enter the tensor cores as two bf16 pieces each) */
 #define DBP_DX_F32       4u /* with io = DBP_BF16: write dX as fp32 instead of bf16 */
 #define DBP_DW_ASYNC     8u /* dense path with both dW and dX asked for: the call returns with dX (and db)
                                ordered on the context's stream as usual, while dW is still being computed on
@@ -233,6 +233,9 @@ int nsd_decode_dense(dbp_ctx *ctx, const dbp_sparse *q, int8_t *codes);
  * is of dtype `io` (fp32 with DBP_DX_F32). Any of dW, dX, db may be NULL (skipped).
  * q_out may be NULL; otherwise it receives the sparse structure (arrays sized for B*N).
  * Outputs are overwritten, not accumulated.
+ * dX and dW are within 1e-5 of the sum of their terms' sizes. Where operands are bf16, N is above 8192 and dX is asked for in
+ * fp32, a dX whose terms have one sign may be low by 1.7e-8 of itself for every 16 outputs (the tensor cores' accumulators
+ * truncate); fp32 operands of one and the same mantissa may cost up to 2^-17 on top.
  * Small fp32 layers (at most 2^17 gradient elements, products of no more tiles than the GPU has SMs), no q_out and no
  * FORCE flag, run as two chained kernels (statistics, dither and quantization; then the products; profiling kind
  * DBP_K_FUSED): same results to the same tolerances, Delta and nnz through dbp_last_step.
@@ -258,7 +261,7 @@ int dithered_linear_backward(dbp_ctx *ctx, const void *delta, const void *X, con
  * computed as the stride-1 layer on the four phase images of X (re-laid beside the quantizer, as the rows the dW kernels
  * read; dX leaves the phase layout beside dW; workspaces of the size of X, dX and 4x the weights). Such a call always
  * joins its weight-gradient kernels before it returns (DBP_DW_ASYNC is ignored). q_out describes delta as given.
- * Other k, stride or pad return DBP_EUNSUPPORTED.
+ * Other k, stride or pad return DBP_EUNSUPPORTED. Accuracy as for linear layers (bf16 1x1 layers: Cout in place of N).
  */
 int dithered_conv_backward(dbp_ctx *ctx, const void *delta, const void *X, const void *W,
                            int io, long long B, long long Cin, long long Cout, long long H,
@@ -291,7 +294,7 @@ int dithered_conv_backward_host(dbp_ctx *ctx, const void *delta, const void *X, 
  * argument as delta_a and quantize delta_a (.) mask. fp32 only (DBP_EUNSUPPORTED otherwise, at that call).
  * Every layer's kernels apply the mask while they read delta_a (no extra pass, no delta_z in memory). A mask that does
  * not start on a 4-byte boundary, and a call with q_out, run the ReLU-derivative kernel into a workspace first. The
- * setting is consumed by that one call.
+ * setting is consumed by that one call, whatever the call returns.
  * mask = NULL clears it.
  */
 int dbp_set_relu_mask(dbp_ctx *ctx, const uint8_t *mask);

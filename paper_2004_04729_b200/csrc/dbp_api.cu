@@ -305,7 +305,6 @@ int conv_backward_impl(dbp_ctx *ctx, const void *delta, const void *X, const voi
     const float *delta_p = nullptr;
     const int8_t *codes = nullptr;
     if (mask && io != DBP_F32) return DBP_EUNSUPPORTED;
-    // small fp32 layers with one position per image (linear layers): two chained launches
     // Masks are read four bytes at a time where they are folded into a kernel's loads. One that does not start on
     // a 4-byte boundary is applied by the ReLU-derivative kernel here and now, and the call goes on without it.
     if (mask != nullptr && (reinterpret_cast<uintptr_t>(mask) & 3) != 0) {
@@ -322,6 +321,7 @@ int conv_backward_impl(dbp_ctx *ctx, const void *delta, const void *X, const voi
         delta = ctx->dz_tmp.ptr;
         mask = nullptr;
     }
+    // small fp32 linear layers: two chained launches
     if (io == DBP_F32 && s.k == 1 && s.H == 1 && s.W == 1 && !q_out && (dW || dX) && (!db || dW) &&
         !(flags & (DBP_FORCE_SPARSE | DBP_FORCE_DENSE)) && small_linear_fits(ctx, s.B, s.Cout, s.Cin, dW != nullptr, dX != nullptr)) {
         if (int wr = wait_code_set(ctx)) return wr;

@@ -173,7 +173,7 @@ int launch_quantize_nhwc(dbp_ctx *ctx, const void *delta, int dtype, long long B
 int launch_decode(dbp_ctx *ctx, const uint32_t *bitmap, const uint16_t *offsets,
                   const int8_t *values, long long numel, int8_t *dense);
 
-// ---- small_linear.cu: one launch for the whole backward pass of a small fp32 linear layer
+// ---- small_linear.cu: the whole backward pass of a small fp32 linear layer in two chained launches
 bool small_linear_fits(const dbp_ctx *ctx, long long B, long long N, long long K, bool want_dw, bool want_dx);
 int launch_small_linear(dbp_ctx *ctx, const float *delta, const float *X, const float *W, long long B, long long N,
                         long long K, unsigned long long seed, float scale, const float *delta_in, float *dW, float *dX,
@@ -300,8 +300,9 @@ struct KernelTimer {
 
 // An accumulator of the tensor cores is truncated, not rounded, when an MMA adds to it: a sum of terms of one sign comes out
 // low by up to 1.7e-8 of itself per MMA (measured: bf16 1x1 dW, 680 and 1360 MMAs: 0.9e-5 and 2.3e-5; fp32 3x3 dW, 2100
-// MMAs: 4.8e-5). Longer reductions are cut into parts of at most this many, which are added with rounding; fp32 operands
-// enter as two bf16 pieces, which costs at most 2^-18 more, and together that stays below 1e-5 of the sum of the terms' sizes.
+// MMAs: 4.8e-5). Longer reductions are cut into parts of at most this many, which are added with rounding: at most 0.9e-5.
+// (fp32 operands enter as two bf16 pieces, whose sum is within 2^-17 of the value: errors of either sign, which average out
+// over the terms unless all operands have the same mantissa.)
 constexpr int kMaxMmas = 512;
 
 // Split of a K loop of `kunits` steps over CTAs when `tiles` output tiles exist and one CTA fits

@@ -15,7 +15,9 @@
 // Sixteen quantizer warps, and four that drain, rather than eight of each: the call above takes 84 against 139 us, because two
 // warps per scheduler do not hide the latencies of the dither's multiplications. The step size is added up from the statistics
 // kernel's partial sums by every CTA (step_of).
-// Bound by the quantizer's instruction issue (about 30 issue slots per vector element and warp, 19 of them the dither).
+// Bound by the quantizer's instructions, but not at their limit: 27 per element, 13 of them the dither, at 65 % of the issue
+// slots (ALU pipe 60 %); the warps wait for loads of delta, for the ALU pipe and for fixed latencies. With the draw left out
+// the kernel still takes 60 of its 71 us (by itself, cold).
 #include "nsd_common.cuh"
 #include "tc_common.cuh"
 

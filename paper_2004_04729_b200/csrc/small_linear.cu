@@ -13,7 +13,7 @@
 //   2. small_linear_products_kernel: every CTA owns one 64 x 64 tile of dW or of dX and accumulates it
 //      on the tensor cores: the codes are exact in bf16, the fp32 operand (X or W) is split into two
 //      bf16 pieces (the value rounded to bf16 and what that left over, rounded again: the pair is within
-//      2^-18 of the value), so a k-step is two warp-level MMAs with fp32 accumulation; Delta is applied
+//      2^-17 of the value), so a k-step is two warp-level MMAs with fp32 accumulation; Delta is applied
 //      once at the end. Warp-level MMAs (not the CTA-wide ones with accumulators in tensor memory)
 //      because a whole tile is a few hundred of them and nothing here can hide a tensor-memory
 //      allocation, a commit and a read-back. The dW tiles of column 0 add up the bias gradient.

@@ -17,7 +17,8 @@
 //
 //   A = weights of one tap [64 co][128 ci]  (M = input channels, MN-major; from W re-laid as [tap][co][ci])
 //   B = code patch         [rows][64 co]    (N = up to 256 patch positions, K-major)
-//   K = (64-channel block of co) x (nine taps), four MMAs of 16 channels each
+//   K = (64-channel block of co) x (nine taps), four MMAs of 16 channels each; for fp32 weights (two bf16 pieces)
+//       both pieces of a block, or, in long reductions, the low pieces of all blocks before the high ones
 //
 // An MMA of N columns takes max(N/2, 32 + N/4) clocks (measured; the second term is its operands' way out of shared
 // memory: 4 KB of A, 32 bytes per column of B), and streamed weights take shared-memory and L2 bandwidth on top. So N is
@@ -646,8 +647,8 @@ tc3_tma_dx_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
 
 // weights [Cout][Cin][3][3] -> [9][Cout][pitch] bf16 (the tap's [co][ci] matrix with ci contiguous, the row pitch a
 // multiple of 8). fp32 weights -> [18][Cout][pitch]: taps 0-8 hold the values rounded to bf16, taps 9-17 what that
-// rounding left over, rounded to bf16 again. The sum of the two pieces differs from the fp32 value by at most 2^-18 of
-// it, and a code times a piece is exact in the fp32 accumulator. Used when the step size is given; otherwise the
+// rounding left over, rounded to bf16 again. The sum of the two pieces differs from the fp32 value by at most 2^-17 of
+// it (2.4e-6 rms), and a code times a piece is exact in the fp32 accumulator. Used when the step size is given; otherwise the
 // statistics kernel does this on the side.
 template <typename T>
 __global__ void __launch_bounds__(256)

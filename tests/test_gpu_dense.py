@@ -112,7 +112,7 @@ def test_dense_path_conv3x3(ctx, B, Ci, Co, H, W):
 ])
 def test_dense_path_conv3x3_fp32_operands(ctx, B, Ci, Co, H, W):
     """fp32 layers on the tensor cores: weights and activations enter as two bf16 pieces each (the sum of the
-    pieces is within 2^-18 of the fp32 value, a code times a piece is exact), same bars as everywhere."""
+    pieces is within 2^-17 of the fp32 value, 2.4e-6 rms, a code times a piece is exact), same bars as everywhere."""
     import paper_2004_04729_b200 as dbp
     L = wl.conv_layer(B, Ci, Co, H, W, 3, data_seed=B + Ci + Co + H, scale=2.0, dtype="f32")
     _run(ctx, L, dbp.DBP_FORCE_DENSE)
