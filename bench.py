@@ -493,7 +493,7 @@ def crossover_sweep(torch, dbp, ctx):
 
 # DRAM bytes (read + written) of one config-5 bench step's launches of each kernel kind, from the ncu capture summarised
 # in profiles/bench_step_config5_launch_list.md; None = the kernels of that kind changed after the capture
-NCU_DRAM_BYTES_PER_STEP = {"statistics": 1156103424, "quantize": 1331695616, "dx_dense": 1309135360, "dw_dense": 2629219840}
+NCU_DRAM_BYTES_PER_STEP = {"statistics": 1152359936, "quantize": 740692480, "dx_dense": 745508864, "dw_dense": 1503840768}
 
 
 def main():
@@ -817,7 +817,7 @@ def main():
                 "note": "non-zero-code FMAs only (2*nnz*K_eff flops per product), summed over the layers that use it"}
     else:
         ach = work[top] / t_s / 1e9
-        # per launch, like the algorithmic bytes: a launch of a kind is one layer's use of it (48 per step)
+        # per launch, like the algorithmic bytes: a launch of a kind is one layer's use of it (41 or 48 per step)
         per_step = NCU_DRAM_BYTES_PER_STEP.get(top) if (args.config == 5 and not (args.only or args.single or args.batch)) else None
         n_launch = max(prof[top][1], 1)
         traffic = None if per_step is None else per_step / n_launch
@@ -831,7 +831,8 @@ def main():
                         "(CUDA events on the stream they run on; the dW kinds run beside the other kernels, which share the "
                         "SMs and the bandwidth with them: kernels[kind].frac_of_measured_hbm_alone is the same ratio with nothing "
                         "else running); traffic: DRAM read+write bytes per launch from the committed ncu launch list "
-                        "(profiles/bench_step_config5_launch_list.md; write-back L2: a kernel's own write counters see little of its output)"}
+                        "(profiles/bench_step_config5_launch_list.md; write-back L2: a kernel's own write counters see little of its output). "
+                        "Re-writing activations as rows the dW kernels can read is work of the glue kind, not of dw_dense"}
     for k in work:
         if k in kern:
             kern[k]["work_per_step"] = work[k]

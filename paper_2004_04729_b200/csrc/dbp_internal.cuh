@@ -90,7 +90,7 @@ struct dbp_ctx {
     cudaEvent_t ev_x_up = nullptr, ev_dx_done = nullptr;
     cudaEvent_t hook_after_dx = nullptr, hook_before_dw = nullptr;   // set only during a *_host call
     // density above which the dense path is preferred. Measured (sparse against dense time for a 1x1, a 3x3 and a
-    // linear layer, densities 22 % ... 0.6 %): the tensor-core path is 2.3x to 11x faster at every density, the gather
+    // linear layer, densities 22 % ... 0.6 %): the tensor-core path is 6.6x to 14x faster at every density, the gather
     // kernels' time being mostly the scan of the dense codes; so wherever the dense path exists it is the default.
     float crossover = 0.0f;
     // densities measured so far, by layer shape (the path choice of a call uses its own shape's entry)
