@@ -233,9 +233,8 @@ int nsd_decode_dense(dbp_ctx *ctx, const dbp_sparse *q, int8_t *codes);
  * is of dtype `io` (fp32 with DBP_DX_F32). Any of dW, dX, db may be NULL (skipped).
  * q_out may be NULL; otherwise it receives the sparse structure (arrays sized for B*N).
  * Outputs are overwritten, not accumulated.
- * dX and dW are within 1e-5 of the sum of their terms' sizes. Where operands are bf16, N is above 8192 and dX is asked for in
- * fp32, a dX whose terms have one sign may be low by 1.7e-8 of itself for every 16 outputs (the tensor cores' accumulators
- * truncate); fp32 operands of one and the same mantissa may cost up to 2^-17 on top.
+ * dX (in fp32) and dW are within 1e-5 of the sum of their terms' sizes; fp32 operands that all have one and the same mantissa
+ * may cost up to 2^-17 on top (they enter the tensor cores as two bf16 pieces).
  * Small fp32 layers (at most 2^17 gradient elements, products of no more tiles than the GPU has SMs), no q_out and no
  * FORCE flag, run as two chained kernels (statistics, dither and quantization; then the products; profiling kind
  * DBP_K_FUSED): same results to the same tolerances, Delta and nnz through dbp_last_step.
@@ -261,7 +260,7 @@ int dithered_linear_backward(dbp_ctx *ctx, const void *delta, const void *X, con
  * computed as the stride-1 layer on the four phase images of X (re-laid beside the quantizer, as the rows the dW kernels
  * read; dX leaves the phase layout beside dW; workspaces of the size of X, dX and 4x the weights). Such a call always
  * joins its weight-gradient kernels before it returns (DBP_DW_ASYNC is ignored). q_out describes delta as given.
- * Other k, stride or pad return DBP_EUNSUPPORTED. Accuracy as for linear layers (bf16 1x1 layers: Cout in place of N).
+ * Other k, stride or pad return DBP_EUNSUPPORTED. Accuracy as for linear layers.
  */
 int dithered_conv_backward(dbp_ctx *ctx, const void *delta, const void *X, const void *W,
                            int io, long long B, long long Cin, long long Cout, long long H,

@@ -291,7 +291,7 @@ int conv_backward_impl(dbp_ctx *ctx, const void *delta, const void *X, const voi
     if (!aligned16(delta) || !aligned16(X) || !aligned16(W) || !aligned16(dW) || !aligned16(dX)) return DBP_EINVAL;
     if ((flags & DBP_FORCE_SPARSE) && (flags & DBP_FORCE_DENSE)) return DBP_EINVAL;
     // What the tensor-core kernels take: linear layers, 1x1 and 3x3 layers of either type and any channel counts
-    const bool linear = s.k == 1 && s.H == 1 && s.W == 1 && linear_tc_supported(s.B, s.Cout, s.Cin, io == DBP_F32 ? 2 : 1);
+    const bool linear = s.k == 1 && s.H == 1 && s.W == 1 && linear_tc_supported(s.B, s.Cout, s.Cin);
     const bool conv1 = tma_dx_supported(s, io), conv3 = tc3_tma_supported(s, io, dX && (io == DBP_F32 || (flags & DBP_DX_F32)));
     const bool can_dense = linear || conv1 || conv3;
     // DBP_FORCE_DENSE keeps its documented range: channel counts that are multiples of 8 (of an fp32 3x3 layer's weight

@@ -184,7 +184,7 @@ struct LinearPlan {
     int TN = 0;                       // columns per tile
     long long dw_split = 1, dw_per_split = 0;   // > 1: dW is added up from parts and must have been cleared
 };
-bool linear_tc_supported(long long B, long long N, long long K, int pieces);
+bool linear_tc_supported(long long B, long long N, long long K);
 long long linear_pitch(long long cols);
 LinearPlan linear_plan(const dbp_ctx *ctx, long long B, long long N, long long K, int pieces, bool want_dw, bool want_dx);
 // X, W: bf16 [pieces][rows][pitch]; pieces = 2 for fp32 operands split by a RowsJob

@@ -34,7 +34,7 @@ constexpr int kOutBlock = 32 * 128;              // one warp's staged block: 32 
 
 struct LinProduct {
     void *out;                    // [M][cols], fp32 or bf16
-    int out_f32, tma_out, add;    // add: the parts of a split reduction are added up in a cleared fp32 output
+    int out_f32, tma_out, add;    // add: into an fp32 output that was cleared, or that holds the part of the reduction before this one
     int M, cols;
     int a_kmajor;                 // A is [M][reduction] (dX) instead of [reduction][M] (dW)
     int ks, pieces, steps;        // 64-deep steps per piece; steps of all pieces
@@ -279,13 +279,12 @@ bool fits_int(long long v) { return v > 0 && v < (1ll << 30); }
 
 }  // namespace
 
-// Steps of four MMAs per accumulator (see kMaxMmas): longer reductions of dW are split; a longer one of an fp32 layer's dX
-// (more than 8192 outputs) is left to the gather kernels.
+// Steps of four MMAs per accumulator (see kMaxMmas): longer reductions of dW are split, longer ones of an fp32 dX (more than
+// 8192 outputs) are cut into parts that follow one another, each added to the one before, so that the order of the sum is fixed.
+// (A bf16 dX rounds far coarser than an accumulator does and is one part.)
 constexpr long long kMaxSteps = kMaxMmas / 4;
 
-bool linear_tc_supported(long long B, long long N, long long K, int pieces) {
-    return fits_int(B) && fits_int(N) && fits_int(K) && (pieces == 1 || (N + 63) / 64 <= kMaxSteps);
-}
+bool linear_tc_supported(long long B, long long N, long long K) { return fits_int(B) && fits_int(N) && fits_int(K); }
 
 long long linear_pitch(long long cols) { return (cols + 7) / 8 * 8; }
 
@@ -328,9 +327,11 @@ LinearPlan linear_plan(const dbp_ctx *ctx, long long B, long long N, long long K
     return pl;
 }
 
-int launch_linear_products(dbp_ctx *ctx, const LinearPlan &pl, const void *codes, const void *X, const void *W, int pieces,
-                           long long x_pitch, long long w_pitch, const float *delta_p, long long B, long long N, long long K,
-                           float *dW, void *dX, bool dx_bf16, int *err_flag) {
+namespace {
+// dX from outputs [n0, n0 + len) of the reduction only
+int launch_products(dbp_ctx *ctx, const LinearPlan &pl, const void *codes, const void *X, const void *W, int pieces,
+                    long long x_pitch, long long w_pitch, const float *delta_p, long long B, long long N, long long K,
+                    long long n0, long long len, float *dW, void *dX, bool dx_bf16, int *err_flag) {
     LinArgs p{};
     LinMaps maps;
     const long long q_pitch = linear_pitch(N);
@@ -341,7 +342,7 @@ int launch_linear_products(dbp_ctx *ctx, const LinearPlan &pl, const void *codes
     p.err_flag = err_flag;
     const int nt = static_cast<int>((K + pl.TN - 1) / pl.TN);
     // the product whose tiles take more reduction steps goes first
-    const long long dx_steps = ((N + 63) / 64) * pieces;
+    const long long dx_steps = ((len + 63) / 64) * pieces;
     const bool dx_first = dX && (!dW || dx_steps >= pl.dw_per_split);
     auto fill = [&](bool is_dx) -> int {
         const int i = p.nprod++;
@@ -351,32 +352,33 @@ int launch_linear_products(dbp_ctx *ctx, const LinearPlan &pl, const void *codes
         q.M = static_cast<int>(is_dx ? B : N);
         q.cols = static_cast<int>(K);
         q.a_kmajor = is_dx ? 1 : 0;
-        const long long red = is_dx ? N : B;
+        const long long red = is_dx ? len : B;
         q.ks = static_cast<int>((red + 63) / 64);
         q.pieces = pieces;
         q.steps = q.ks * pieces;
         q.nsplit = is_dx ? 1 : static_cast<int>(pl.dw_split);
         q.per_split = is_dx ? q.steps : static_cast<int>(pl.dw_per_split);
-        q.add = q.nsplit > 1;
+        q.add = is_dx ? n0 > 0 : q.nsplit > 1;
         q.mt = (q.M + 127) / 128;
         const long long tiles = static_cast<long long>(q.mt) * nt * q.nsplit;
         if (tiles + p.tiles >= (1ll << 30)) return DBP_EUNSUPPORTED;
         q.tiles = static_cast<int>(tiles);
         p.tiles += q.tiles;
         {
-            const unsigned long long dims[2] = {static_cast<unsigned long long>(N), static_cast<unsigned long long>(B)};
+            const unsigned long long dims[2] = {static_cast<unsigned long long>(is_dx ? len : N), static_cast<unsigned long long>(B)};
             const unsigned long long str[1] = {static_cast<unsigned long long>(q_pitch) * 2};
             const unsigned box[2] = {64, is_dx ? 128u : 64u};
-            if (!encode_map_bf16(&maps.a[i], codes, 2, dims, str, box)) return fail_cuda("tensor map of the codes");
+            if (!encode_map_bf16(&maps.a[i], static_cast<const unsigned short *>(codes) + (is_dx ? n0 : 0), 2, dims, str, box)) return fail_cuda("tensor map of the codes");
         }
         {
             const long long pitch = is_dx ? w_pitch : x_pitch;
             const unsigned long long dims[3] = {static_cast<unsigned long long>(K), static_cast<unsigned long long>(red),
                                                 static_cast<unsigned long long>(pieces)};
             const unsigned long long str[2] = {static_cast<unsigned long long>(pitch) * 2,
-                                               static_cast<unsigned long long>(pitch) * 2 * red};
+                                               static_cast<unsigned long long>(pitch) * 2 * (is_dx ? N : B)};
             const unsigned box[3] = {64, 64, 1};
-            if (!encode_map_bf16(&maps.b[i], is_dx ? W : X, 3, dims, str, box)) return fail_cuda("tensor map of an operand");
+            const void *rows = is_dx ? static_cast<const unsigned short *>(W) + n0 * w_pitch : X;
+            if (!encode_map_bf16(&maps.b[i], rows, 3, dims, str, box)) return fail_cuda("tensor map of an operand");
         }
         const int es = q.out_f32 ? 4 : 2;
         q.tma_out = (K * es) % 16 == 0 ? 1 : 0;
@@ -400,6 +402,20 @@ int launch_linear_products(dbp_ctx *ctx, const LinearPlan &pl, const void *codes
         return fail_cuda("shared memory size");
     const int grid = p.tiles < ctx->sm_count ? p.tiles : ctx->sm_count;
     return cuda_ok(launch_chained(linear_products_kernel, dim3(static_cast<unsigned>(grid)), dim3(kThreadsL), smem, ctx->stream, maps, p));
+}
+}  // namespace
+
+int launch_linear_products(dbp_ctx *ctx, const LinearPlan &pl, const void *codes, const void *X, const void *W, int pieces,
+                           long long x_pitch, long long w_pitch, const float *delta_p, long long B, long long N, long long K,
+                           float *dW, void *dX, bool dx_bf16, int *err_flag) {
+    const long long most = dX && !dx_bf16 ? 64 * kMaxSteps : N;
+    for (long long n0 = 0; n0 < N; n0 += most) {          // dW leaves with the first part of dX
+        const long long len = N - n0 < most ? N - n0 : most;
+        if (int rc = launch_products(ctx, pl, codes, X, W, pieces, x_pitch, w_pitch, delta_p, B, N, K, n0, len, n0 ? nullptr : dW, dX,
+                                     dx_bf16, err_flag))
+            return rc;
+    }
+    return DBP_OK;
 }
 
 }  // namespace dbp

@@ -87,6 +87,7 @@ struct DxT {
     void *dX;                     // [B][Cin][HW], bf16 or fp32
     int dx_f32;
     int tma_out;                  // rows of dX are multiples of 16 bytes: chunks leave through the copy engine
+    int add;                      // fp32 dX: the results are added to what an earlier part of the reduction left there
     int Cin, Cout, HW;
     int chunks_per_img;
     long long nchunks;            // B * chunks_per_img
@@ -312,16 +313,19 @@ tma_dx_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constant__
                         __syncwarp();
                         if (p.tma_out) {
                             if (lane == 0 && ci_w < p.Cin) {
-                                tma_store_3d(&map_dx, pp, ci_w, static_cast<int>(b), stage);
+                                if (p.add) tma_reduce_add_3d(&map_dx, pp, ci_w, static_cast<int>(b), stage);
+                                else tma_store_3d(&map_dx, pp, ci_w, static_cast<int>(b), stage);
                                 bulk_commit();
                             }
                         } else {
                             const int nr = p.Cin - ci_w < 32 ? p.Cin - ci_w : 32;
                             float *dst = static_cast<float *>(p.dX) + (b * p.Cin + ci_w) * p.HW + pp + lane;
                             for (int r = 0; r < nr; ++r)
-                                if (lane < nval)
-                                    dst[static_cast<long long>(r) * p.HW] =
-                                        *reinterpret_cast<const float *>(stage + r * 128 + (((lane >> 2) ^ (r & 7)) << 4) + (lane & 3) * 4);
+                                if (lane < nval) {
+                                    float *o = dst + static_cast<long long>(r) * p.HW;
+                                    const float f = *reinterpret_cast<const float *>(stage + r * 128 + (((lane >> 2) ^ (r & 7)) << 4) + (lane & 3) * 4);
+                                    *o = p.add ? *o + f : f;
+                                }
                         }
                     } else {
                         // bf16: my 32 values go to the warp's staging block, which holds the chunk
@@ -416,20 +420,22 @@ tma_dx_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constant__
 
 }  // namespace
 
-// The reduction of an fp32 layer is kept to kMaxMmas per accumulator, an MMA taking 16 channels (the low pieces of the
-// weights are added first and do not count).
 bool tma_dx_supported(const ConvShape &s, int io) {
-    return s.k == 1 && s.H * s.W > 1 && s.H * s.W < (1ll << 30) && (io == DBP_BF16 || s.Cout <= 16 * kMaxMmas);
+    return (io == DBP_BF16 || io == DBP_F32) && s.k == 1 && s.H * s.W > 1 && s.H * s.W < (1ll << 30);
 }
 
 long long tma_code_pitch(const ConvShape &s) { return (s.H * s.W + 7) / 8 * 8; }
 
-int launch_tma_dx(dbp_ctx *ctx, const void *codes_bf16, const void *W, int pieces, long long w_pitch, const float *delta_p,
-                  const ConvShape &s, void *dX, bool dx_bf16, int *err_flag) {
+namespace {
+// output channels [co0, co0 + cout) of the reduction
+int launch_tma_dx_part(dbp_ctx *ctx, const void *codes_bf16, const void *W, int pieces, long long w_pitch, const float *delta_p,
+                       const ConvShape &s, long long co0, long long cout, void *dX, bool dx_bf16, int *err_flag) {
     const long long HW = s.H * s.W, pitch = tma_code_pitch(s);
+    codes_bf16 = static_cast<const unsigned short *>(codes_bf16) + co0 * pitch;
+    W = static_cast<const unsigned short *>(W) + co0 * w_pitch;
     CUtensorMap map_w, map_q;
     {
-        const unsigned long long dims[3] = {static_cast<unsigned long long>(s.Cin), static_cast<unsigned long long>(s.Cout),
+        const unsigned long long dims[3] = {static_cast<unsigned long long>(s.Cin), static_cast<unsigned long long>(cout),
                                             static_cast<unsigned long long>(pieces)};
         const unsigned long long str[2] = {static_cast<unsigned long long>(w_pitch) * 2,
                                            static_cast<unsigned long long>(w_pitch) * 2 * s.Cout};
@@ -437,7 +443,7 @@ int launch_tma_dx(dbp_ctx *ctx, const void *codes_bf16, const void *W, int piece
         if (!encode_map_bf16(&map_w, W, 3, dims, str, box)) return fail_cuda("tensor map of the weights");
     }
     {
-        const unsigned long long dims[3] = {static_cast<unsigned long long>(HW), static_cast<unsigned long long>(s.Cout),
+        const unsigned long long dims[3] = {static_cast<unsigned long long>(HW), static_cast<unsigned long long>(cout),
                                             static_cast<unsigned long long>(s.B)};
         const unsigned long long str[2] = {static_cast<unsigned long long>(pitch) * 2,
                                            static_cast<unsigned long long>(pitch) * 2 * s.Cout};
@@ -446,6 +452,7 @@ int launch_tma_dx(dbp_ctx *ctx, const void *codes_bf16, const void *W, int piece
     }
     DxT p{};
     p.delta_p = delta_p; p.dX = dX; p.dx_f32 = dx_bf16 ? 0 : 1;
+    p.add = co0 > 0 ? 1 : 0;
     CUtensorMap map_dx = map_w;                  // a valid map when the store path is not used
     p.tma_out = HW % (dx_bf16 ? 8 : 4) == 0 ? 1 : 0;
     if (p.tma_out) {
@@ -457,10 +464,10 @@ int launch_tma_dx(dbp_ctx *ctx, const void *codes_bf16, const void *W, int piece
         if (!(dx_bf16 ? encode_map_bf16(&map_dx, dX, 3, dims, str, box) : encode_map_f32_sw128(&map_dx, dX, 3, dims, str, box)))
             return fail_cuda("tensor map of dX");
     }
-    p.Cin = static_cast<int>(s.Cin); p.Cout = static_cast<int>(s.Cout); p.HW = static_cast<int>(HW);
+    p.Cin = static_cast<int>(s.Cin); p.Cout = static_cast<int>(cout); p.HW = static_cast<int>(HW);
     p.chunks_per_img = static_cast<int>((HW + 63) / 64);
     p.nchunks = s.B * p.chunks_per_img;
-    p.ks_piece = static_cast<int>((s.Cout + 63) / 64);
+    p.ks_piece = static_cast<int>((cout + 63) / 64);
     p.pieces = pieces;
     p.ksteps = p.ks_piece * pieces;
     // Two accumulators halve the code traffic per MMA but leave half as many tiles and no second
@@ -479,6 +486,20 @@ int launch_tma_dx(dbp_ctx *ctx, const void *codes_bf16, const void *W, int piece
     const long long grid = p.ntiles < ctx->sm_count ? p.ntiles : ctx->sm_count;
     return cuda_ok(launch_chained(tma_dx_kernel, dim3(static_cast<unsigned>(grid)), dim3(kThreadsT), smem, ctx->stream,
                                   map_w, map_q, map_dx, p));
+}
+}  // namespace
+
+// An fp32 dX keeps to kMaxMmas per accumulator, an MMA taking 16 channels (the low pieces of fp32 weights are added first and
+// do not count): longer reductions are parts that follow one another, each added to the one before, so the order of the sum is
+// fixed. A bf16 dX rounds far coarser than an accumulator does and is one part.
+int launch_tma_dx(dbp_ctx *ctx, const void *codes_bf16, const void *W, int pieces, long long w_pitch, const float *delta_p,
+                  const ConvShape &s, void *dX, bool dx_bf16, int *err_flag) {
+    const long long most = dx_bf16 ? s.Cout : 16 * kMaxMmas;
+    for (long long co0 = 0; co0 < s.Cout; co0 += most) {
+        const long long cout = s.Cout - co0 < most ? s.Cout - co0 : most;
+        if (int rc = launch_tma_dx_part(ctx, codes_bf16, W, pieces, w_pitch, delta_p, s, co0, cout, dX, dx_bf16, err_flag)) return rc;
+    }
+    return DBP_OK;
 }
 
 }  // namespace dbp

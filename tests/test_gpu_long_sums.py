@@ -135,7 +135,8 @@ def test_stride_2_input_gradients_in_parts(ctx, Ci, Co):
 @pytest.mark.parametrize("dtype,B,N,K,want", [
     ("f32", 8192, 16, 64, "dW"), ("f32", 2, 60000, 72, "dX"),       # one tile's reduction on warp-level MMAs
     ("f32", 16384, 300, 256, "dW"), ("f32", 300, 8192, 256, "dX"),  # the longest parts of the CTA-wide kernel
-    ("f32", 260, 8300, 128, "both"),                                # beyond them: the gather kernels
+    ("f32", 260, 8300, 128, "both"), ("f32", 70, 16500, 130, "both"), ("bf16", 300, 20000, 256, "dX"),     # dX in parts
+    ("bf16", 96, 24577, 131, "both"),
     ("bf16", 32768, 320, 512, "dW"), ("bf16", 300, 8192, 512, "dX")])
 def test_linear_layers(ctx, dtype, B, N, K, want):
     import paper_2004_04729_b200 as dbp
@@ -146,4 +147,21 @@ def test_linear_layers(ctx, dtype, B, N, K, want):
         _check_dW(out["dW"].view(N, K, 1, 1), codes, delta, X, 1)
     if want != "dW":
         _check_dX(out["dX"].view(B, K, 1, 1), codes, delta, Wt, 1)
+        for _ in range(3):                       # the parts are added in one order
+            again = dbp.dithered_linear_backward(ctx, d.view(B, N), X.view(B, K), Wt.view(N, K), 3, 1.0, need_dW=want != "dX", flags=dbp.DBP_DX_F32)
+            assert torch.equal(again["dX"], out["dX"])
+    assert ctx.last_device_status() == (0, 0)
+
+
+@pytest.mark.parametrize("dtype,B,Ci,Co,H,W", [
+    ("f32", 2, 72, 8192, 8, 8), ("f32", 2, 264, 8200, 9, 12), ("f32", 3, 40, 16500, 5, 5),    # whole words or not, two and three parts
+    ("bf16", 2, 136, 20000, 8, 8), ("bf16", 5, 24, 8257, 5, 7)])
+def test_1x1_input_gradients(ctx, dtype, B, Ci, Co, H, W):
+    import paper_2004_04729_b200 as dbp
+    d, X, Wt, codes, delta = _layer(ctx, dtype, B, Ci, Co, H, W, 1)
+    out = dbp.dithered_conv_backward(ctx, d, X, Wt, 3, 1.0, flags=dbp.DBP_DX_F32)
+    _check_dX(out["dX"], codes, delta, Wt, 1)
+    _check_dW(out["dW"], codes, delta, X, 1)
+    for _ in range(3):
+        assert torch.equal(dbp.dithered_conv_backward(ctx, d, X, Wt, 3, 1.0, flags=dbp.DBP_DX_F32)["dX"], out["dX"])
     assert ctx.last_device_status() == (0, 0)
