@@ -50,8 +50,10 @@ typedef enum {
 #define DBP_FORCE_SPARSE 1u /* always use the sparse gather kernels */
 #define DBP_FORCE_DENSE  2u /* always use the dense tensor-core path; DBP_EUNSUPPORTED where it
                                does not exist (it covers bf16 linear and 1x1 layers and bf16 or fp32 3x3
-                               layers, channel counts multiples of 8, 3x3 images up to 62 wide and, with an fp32 dX, up to
-                               7168 output channels; fp32 operands enter the tensor cores as two bf16 pieces each) */
+                               layers, channel counts multiples of 8, 3x3 images up to 62 wide; fp32 operands enter the
+                               tensor cores as two bf16 pieces each). An fp32 dX of 3x3 layers of more than 7168 output
+                               channels, which otherwise runs on the gather kernels, may then be low by 1.7e-8 of itself
+                               for every 14 channels more than that. */
 #define DBP_DX_F32       4u /* with io = DBP_BF16: write dX as fp32 instead of bf16 */
 #define DBP_DW_ASYNC     8u /* dense path with both dW and dX asked for: the call returns with dX (and db)
                                ordered on the context's stream as usual, while dW is still being computed on
@@ -201,6 +203,8 @@ int dbp_sparse_bytes(long long numel, size_t *bitmap_bytes, size_t *offsets_byte
  *   out      : arrays sized by dbp_sparse_bytes; out->numel is set by the call;
  *              *out->delta and *out->nnz are written on the device.
  * sigma = 0 is not an error (Delta = 0, every code 0).
+ * Delta is within 1e-6 of that for a spread of delta between 1e-18 and 1e18 (squares are formed in fp32, added up in
+ * fp64); below, it loses accuracy and ends at 0, above, the call reports DBP_ENONFINITE.
  */
 int nsd_quantize(dbp_ctx *ctx, const void *delta, int dtype, long long numel,
                  unsigned long long seed, float scale, const float *delta_in, dbp_sparse *out);

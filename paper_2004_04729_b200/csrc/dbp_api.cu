@@ -292,7 +292,7 @@ int conv_backward_impl(dbp_ctx *ctx, const void *delta, const void *X, const voi
     if ((flags & DBP_FORCE_SPARSE) && (flags & DBP_FORCE_DENSE)) return DBP_EINVAL;
     // What the tensor-core kernels take: linear layers, 1x1 and 3x3 layers of either type and any channel counts
     const bool linear = s.k == 1 && s.H == 1 && s.W == 1 && linear_tc_supported(s.B, s.Cout, s.Cin);
-    const bool conv1 = tma_dx_supported(s, io), conv3 = tc3_tma_supported(s, io, dX && (io == DBP_F32 || (flags & DBP_DX_F32)));
+    const bool conv1 = tma_dx_supported(s, io), conv3 = tc3_tma_supported(s, io, dX && !(flags & DBP_FORCE_DENSE) && (io == DBP_F32 || (flags & DBP_DX_F32)));
     const bool can_dense = linear || conv1 || conv3;
     // DBP_FORCE_DENSE keeps its documented range: channel counts that are multiples of 8 (of an fp32 3x3 layer's weight
     // gradient alone, only the output channels), and no fp32 linear or 1x1 layers
@@ -579,7 +579,7 @@ int conv_backward_stride2(dbp_ctx *ctx, const void *delta, const void *X, const 
     const size_t nxp = static_cast<size_t>(in.B) * in.Cin * Ho * Wo, nwp = static_cast<size_t>(in.Cout) * in.Cin * s.k * s.k;
     int rc;
     const bool tensor = (dW || dX) && !(flags & DBP_FORCE_SPARSE) && ((flags & DBP_FORCE_DENSE) || ctx->crossover <= 0.f) &&
-                        (s.k == 3 ? tc3_tma_supported(in, io, dX && dx_f32) : tma_dx_supported(in, io));
+                        (s.k == 3 ? tc3_tma_supported(in, io, dX && dx_f32 && !(flags & DBP_FORCE_DENSE)) : tma_dx_supported(in, io));
     if (dX && (rc = ws_reserve(ctx, ctx->s2_dx, nxp * (dx_f32 ? 4 : 2)))) return rc;
     if (dX && s.k == 3 && (rc = ws_reserve(ctx, ctx->s2_w, nwp * es))) return rc;
     if (dW && s.k == 3 && (rc = ws_reserve(ctx, ctx->s2_dw, nwp * sizeof(float)))) return rc;

@@ -225,7 +225,7 @@ int launch_tma_dx(dbp_ctx *ctx, const void *codes_bf16, const void *W, int piece
 int launch_tma_dw(dbp_ctx *ctx, const void *codes_bf16, const void *X, int pieces, long long x_pitch, const float *delta_p,
                   const ConvShape &s, float *dW, int *err_flag);
 // ---- tc3_tma_dx.cu / tc3_tma_dw.cu: 3x3 products with TMA-fed operands; codes as bf16 [B][H*W][Cout rounded up to 8]
-// dx_f32: an fp32 dX is wanted
+// dx_f32: an fp32 dX is wanted, to the accuracy of every other
 bool tc3_tma_supported(const ConvShape &s, int io, bool dx_f32);
 // io: the operands' type; fp32 weights / activations are split into two bf16 pieces on the way in
 // weights_ready: ctx->w_taps already holds the re-laid weights (the statistics kernel did it on the side)

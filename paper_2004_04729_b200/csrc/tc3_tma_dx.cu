@@ -672,7 +672,8 @@ int round_up(int v, int m) { return (v + m - 1) / m * m; }
 
 // Shapes the TMA-fed 3x3 kernels take. fp32 operands are split into two bf16 pieces each (the codes are exact in bf16);
 // rows of the codes, of the re-laid weights and of the activations that are no multiple of 16 bytes are padded to one.
-// An fp32 dX keeps to kMaxMmas per accumulator, and its reduction is cut into eight parts at most.
+// An fp32 dX keeps to kMaxMmas per accumulator, and its reduction is cut into eight parts at most: longer ones go to the gather
+// kernels unless the caller insists on these (a part then has more MMAs than that).
 constexpr int kMaxKS = 8;
 constexpr int kMaxBlocks = kMaxMmas / 36;        // 64-channel blocks of co per accumulator: nine taps of four MMAs each
 bool tc3_tma_supported(const ConvShape &s, int io, bool dx_f32) {
@@ -683,7 +684,7 @@ bool tc3_tma_supported(const ConvShape &s, int io, bool dx_f32) {
 // DBP_EUNSUPPORTED: the shape does not fit (the caller uses another kernel)
 int launch_tc3_tma_dx(dbp_ctx *ctx, const void *codes_nhwc, const void *W, int io, const float *delta_p,
                       const ConvShape &s, void *dX, bool dx_bf16, int *err_flag, bool weights_ready, bool *lean) {
-    if (!tc3_tma_supported(s, io, !dx_bf16)) return DBP_EUNSUPPORTED;
+    if (!tc3_tma_supported(s, io, false)) return DBP_EUNSUPPORTED;
     Dx3T p{};
     p.delta_p = delta_p; p.dX = dX;
     p.es = dx_bf16 ? 2 : 4;
@@ -699,7 +700,7 @@ int launch_tc3_tma_dx(dbp_ctx *ctx, const void *codes_nhwc, const void *W, int i
     // weights then take a pass each, low ones first, because an MMA costs an accumulator as much for a small term as for a
     // large one: up to kMaxBlocks / 2 blocks the sum of both pieces keeps to kMaxMmas anyway, and a block's codes are read once.
     int min_ks = 1;
-    while (p.es == 4 && min_ks * kMaxBlocks < p.ncb) min_ks *= 2;
+    while (p.es == 4 && min_ks < kMaxKS && min_ks * kMaxBlocks < p.ncb) min_ks *= 2;
     p.split = io == DBP_F32 && p.Cin <= 64 && min_ks == 1 ? 1 : 0;
     p.a_panels = p.Cin <= 64 && !p.split ? 1 : 2;
     const int map_taps = p.ntaps;

@@ -108,12 +108,11 @@ def test_3x3_input_gradients(ctx, dtype, B, Ci, Co, H, W):
 
 
 def test_3x3_input_gradient_of_more_channels_than_the_parts_hold(ctx):
-    """fp32 from 7169 output channels on: the gather kernels (and none of the tensor cores' when those are insisted on)."""
+    """fp32 from 7169 output channels on: the gather kernels; the tensor cores' when those are insisted on (540 MMAs a part)."""
     import paper_2004_04729_b200 as dbp
     d, X, Wt, codes, delta = _layer(ctx, "f32", 1, 8, 7176, 5, 5, 3)
     _check_dX(dbp.dithered_conv_backward(ctx, d, X, Wt, 3, 1.0)["dX"], codes, delta, Wt, 3)
-    with pytest.raises(dbp.DbpError):
-        dbp.dithered_conv_backward(ctx, d, X, Wt, 3, 1.0, flags=dbp.DBP_FORCE_DENSE)
+    _check_dX(dbp.dithered_conv_backward(ctx, d, X, Wt, 3, 1.0, flags=dbp.DBP_FORCE_DENSE)["dX"], codes, delta, Wt, 3)
 
 
 @pytest.mark.parametrize("Ci,Co", [(128, 512), (128, 1024), (256, 72)])
