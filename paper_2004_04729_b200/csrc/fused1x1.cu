@@ -7,17 +7,20 @@
 // whole layer beside two dX accumulators), delta is read once after the statistics, the codes never leave the SM, and
 // quantization (instruction issue), products (tensor pipe) and the copies of X and dX (memory) run beside one another.
 // Before: the quantizer wrote bf16 codes that two kernels read again. 64 -> 256 at 56x56, batch 64 (51 M gradient elements):
-// 119 -> 84 us for the whole call, of which this kernel 66; a ResNet-50 set of 17 layers 1020 -> 936 us.
+// 119 -> 72 us for the whole call, of which this kernel 53.
 //
-// A CTA is persistent over tiles of NCH chunks of 64 positions. Warp 0 copies W (once) and X, warp 1 issues the MMAs, warps
-// 2-5 drain the dX accumulators (and dW at the end, added into the cleared dW by the copy engine), warps 6-21 quantize: a
-// stage is ROWS output channels of the tile, and a thread has the 64 bytes it works on next (G stages' vectors) on their way.
-// Sixteen quantizer warps, and four that drain, rather than eight of each: the call above takes 84 against 139 us, because two
-// warps per scheduler do not hide the latencies of the dither's multiplications. The step size is added up from the statistics
-// kernel's partial sums by every CTA (step_of).
-// Bound by the quantizer's instructions, but not at their limit: 27 per element, 13 of them the dither, at 65 % of the issue
-// slots (ALU pipe 60 %); the warps wait for loads of delta, for the ALU pipe and for fixed latencies. With the draw left out
-// the kernel still takes 60 of its 71 us (by itself, cold).
+// A CTA is persistent over tiles of NCH chunks of 64 positions. Warp 0 copies delta: a stage is ROWS output channels of the
+// tile, and its buffer holds delta first and the codes after, row by row in the same swizzled place, so that a quantizer
+// thread has no addresses to make and no edges to look at (the copy engine reads zeros outside the tensor) and every stage of
+// the ring is in flight. Warp 1 issues the MMAs, warps 2-5 drain the dX accumulators (and dW at the end, added into the
+// cleared dW by the copy engine), warps 6-21 quantize, warp 22 copies W (once) and X. Where the vectors came to the
+// quantizer's registers by plain loads instead, 64 bytes a thread ahead, the call above took 84 us against 72: the kernel
+// executed 27 instructions an element against 21.
+// Sixteen quantizer warps, and four that drain, rather than eight of each: 84 against 139 us (of that form), because two
+// warps per scheduler do not hide the latencies of the dither's multiplications. The step size is added up from the
+// statistics kernel's partial sums by every CTA (step_of).
+// Bound by the quantizer's instructions: 15 of the 21 are the decision, which takes 22 clocks an element and scheduler (30 us
+// of this kernel's 53); copies, MMAs and stores alone, with the codes left out, take 37 (by themselves, cold).
 #include "nsd_common.cuh"
 #include "tc_common.cuh"
 
@@ -29,7 +32,8 @@ using namespace tc;
 using namespace nsd;
 
 constexpr int kQWarps = 16, kEWarps = 4;
-constexpr int kThreadsF = 32 * (2 + kEWarps + kQWarps);
+constexpr int kXWarp = 2 + kEWarps + kQWarps;    // copies W and X
+constexpr int kThreadsF = 32 * (kXWarp + 1);
 constexpr int kPanelF = 128 * 128;               // [128 co][64 positions] bf16
 constexpr int kMaxStages = 6;
 constexpr int kOutF = 32 * 128;                  // one epilogue warp's staging block
@@ -45,21 +49,25 @@ struct Fused1P {
     int NT, NTp;                  // dW columns, rounded to 16 and to 32
     int MA;                       // 128-channel accumulators of dX per tile
     int stages;
+    // the dither's counter: of the pair of elements 2 i, 2 i + 1: seed + (i + 1) gamma. A tile's chunks lie step_c chunks (within
+    // an image) and tile_z of the counter (from behind the last stage) before those of the CTA's tile before it, and wrap_z
+    // after that where the step passes the first chunk of an image; stage_z: a stage's channels, row64_z: 64 channels
+    int step_c;
+    unsigned long long tile_z, wrap_z, stage_z, row64_z;
     int *err_flag;
 };
 
 struct PipeF {
-    unsigned long long q_full[kMaxStages], q_empty[kMaxStages], x_full[2], x_empty[2], w_full, acc_full[2], acc_empty[2], dw_full;
+    unsigned long long d_full[kMaxStages], q_full[kMaxStages], q_empty[kMaxStages], x_full[2], x_empty[2], w_full, acc_full[2], acc_empty[2], dw_full;
     unsigned tmem_base;
 };
 
 template <int ROWS, int NCH>
 __global__ void __launch_bounds__(kThreadsF, 1)
-fused1x1_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constant__ CUtensorMap map_x,
+fused1x1_kernel(const __grid_constant__ CUtensorMap map_d, const __grid_constant__ CUtensorMap map_w, const __grid_constant__ CUtensorMap map_x,
                 const __grid_constant__ CUtensorMap map_dx, const __grid_constant__ CUtensorMap map_dw,
                 const __grid_constant__ StepSource step, const Fused1P p) {
     constexpr int NV = ROWS * NCH * 8 / (32 * kQWarps);              // vectors per quantizer thread and stage
-    constexpr int G = 4 / NV;                                        // stages whose vectors are in flight: 64 bytes per thread
     extern __shared__ __align__(1024) unsigned char smem_raw[];
     unsigned char *smem = reinterpret_cast<unsigned char *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
     const int w_bytes = p.w_panels * p.w_rows * 128, x_bytes = NCH * p.NT * 128;
@@ -69,7 +77,7 @@ fused1x1_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constant
     const int S = p.stages;
 
     if (threadIdx.x == 0) {
-        for (int s = 0; s < kMaxStages; ++s) { mbar_init(&pipe.q_full[s], kQWarps); mbar_init(&pipe.q_empty[s], 1); }
+        for (int s = 0; s < kMaxStages; ++s) { mbar_init(&pipe.d_full[s], 1); mbar_init(&pipe.q_full[s], kQWarps); mbar_init(&pipe.q_empty[s], 1); }
         for (int s = 0; s < 2; ++s) {
             mbar_init(&pipe.x_full[s], 1); mbar_init(&pipe.x_empty[s], 1);
             mbar_init(&pipe.acc_full[s], 1); mbar_init(&pipe.acc_empty[s], kEWarps);
@@ -77,6 +85,7 @@ fused1x1_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constant
         mbar_init(&pipe.w_full, 1);
         mbar_init(&pipe.dw_full, 1);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+        tma_prefetch_desc(&map_d);
         tma_prefetch_desc(&map_w);
         tma_prefetch_desc(&map_x);
         tma_prefetch_desc(&map_dx);
@@ -99,32 +108,14 @@ fused1x1_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constant
 
     // delta, X and W are inputs of the call: their first tiles are on their way while the statistics kernel runs (it lets
     // this kernel start when all of its blocks have seen everything before them complete)
-    uint4 raw[G][NV];
-    long long at[G][NCH];                        // where the stage's chunks are for this thread: see places
-    const int qt = threadIdx.x - 32 * (2 + kEWarps), c8 = (qt & 7) * 8;
-    int ft = 0, fcb = 0;                         // the next stage to fetch: tile of this CTA, stage of the tile
-    long long fat[NCH];
-    // element index of (chunk, channel 0, this thread's 8 positions), or -1 outside
-    auto places = [&](int t) {
-#pragma unroll
-        for (int j = 0; j < NCH; ++j) {
+    // delta comes as the codes will lie: a stage's buffer holds it first
+    const int total = my_tiles * p.nco;
+    auto load_d = [&](int n, int s) {
+        const int i = n / p.nco, co = (n - i * p.nco) * ROWS, t = tile_of(i);
+        mbar_expect_tx(&pipe.d_full[s], NCH * ROWS * 128);
+        for (int j = 0; j < NCH; ++j) {          // what lies outside the tensor reads as zero
             const Chunk c = chunk_of(t, j);
-            fat[j] = c.b < p.B && c.p0 + c8 < p.HW ? static_cast<long long>(c.b) * p.Cout * p.HW + c.p0 + c8 : -1;
-        }
-    };
-    auto fetch = [&](int g, int i) {             // vector i of a stage: row (v >> 3) % ROWS of chunk (v >> 3) / ROWS
-        const int v = qt + 32 * kQWarps * i, row = (v >> 3) % ROWS, co = fcb * ROWS + row;
-        const long long a = fat[32 * kQWarps * i / (8 * ROWS)];
-        raw[g][i] = make_uint4(0u, 0u, 0u, 0u);
-        if (a >= 0 && co < p.Cout && ft < my_tiles)
-            raw[g][i] = __ldg(reinterpret_cast<const uint4 *>(p.delta + a + static_cast<long long>(co) * p.HW));
-    };
-    auto fetched = [&](int g) {
-#pragma unroll
-        for (int j = 0; j < NCH; ++j) at[g][j] = fat[j];
-        if (++fcb == p.nco) {
-            fcb = 0;
-            if (++ft < my_tiles) places(tile_of(ft));
+            tma_load_3d(q_s + s * NCH * kPanelF + j * kPanelF, &map_d, c.p0, co, c.b, &pipe.d_full[s]);
         }
     };
     auto load_x = [&](int i) {
@@ -136,15 +127,9 @@ fused1x1_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constant
             tma_load_3d(x_s + s * x_bytes + j * p.NT * 128, &map_x, c.p0, 0, c.b, &pipe.x_full[s]);
         }
     };
-    if (warp >= 2 + kEWarps) {
-        places(tile_of(0));
-#pragma unroll
-        for (int g = 0; g < G; ++g) {
-#pragma unroll
-            for (int i = 0; i < NV; ++i) fetch(g, i);
-            fetched(g);
-        }
-    } else if (threadIdx.x == 0) {
+    if (threadIdx.x == 0) {
+        for (int n = 0; n < S && n < total; ++n) load_d(n, n);
+    } else if (threadIdx.x == 32 * kXWarp) {
         mbar_expect_tx(&pipe.w_full, static_cast<unsigned>(w_bytes));
         for (int h = 0; h < p.w_panels; ++h)
             for (int r = 0; r < p.w_rows; r += 64)
@@ -157,12 +142,27 @@ fused1x1_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constant
 
     if (warp == 0) {
         if (lane == 0) {
-            for (int i = 2; i < my_tiles; ++i) {
-                if (!mbar_wait(&pipe.x_empty[i & 1], ((i >> 1) & 1) ^ 1, p.err_flag)) break;
-                load_x(i);
+            int s = 0;
+            unsigned par = 0;                                        // stage n again once the MMAs of stage n - S have read it
+            int n = S;
+            for (; n < total; ++n) {
+                if (!mbar_wait(&pipe.q_empty[s], par, p.err_flag)) break;
+                load_d(n, s);
+                if (++s == S) { s = 0; par ^= 1u; }
             }
+            if (n < total)                                           // given up: no copy may outlive the CTA
+                for (int k = 0; k < S; ++k) mbar_wait(&pipe.d_full[k], ((n - k + S - 1) / S - 1) & 1, p.err_flag);
             chain_release();
         }
+    } else if (warp == kXWarp) {
+        if (lane == 0)
+            for (int i = 2; i < my_tiles; ++i) {
+                if (!mbar_wait(&pipe.x_empty[i & 1], ((i >> 1) & 1) ^ 1, p.err_flag)) {
+                    for (int k = i - 2; k < i; ++k) mbar_wait(&pipe.x_full[k & 1], (k >> 1) & 1, p.err_flag);
+                    break;
+                }
+                load_x(i);
+            }
     } else if (warp == 1) {
         // the whole warp runs the loop (uniform control flow and operands); one elected lane issues
         const unsigned idesc_dx = make_idesc(128, 64 * NCH, true, true), idesc_dw = make_idesc(128, p.NT, false, false);
@@ -293,37 +293,73 @@ fused1x1_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constant
         const float inv = delta > 0.f ? __fdiv_rn(1.0f, delta) : 0.f;          // Delta = 0: every code 0
         unsigned sat = 0, nnz = 0, nz2 = 0;
         int s = 0;
-        unsigned par = 1;                                            // a fresh barrier passes a wait on the previous phase
-        bool ok = true;
-        int cb = 0;
-        const int total = my_tiles * p.nco;
-        for (int n0 = 0; n0 < total && ok; n0 += G) {
+        unsigned par = 0;
+        // A thread takes the same eight positions of rows qrow, qrow + 64 of every chunk of a stage, in place
+        constexpr int RPC = NV / NCH;                                // its rows of a chunk
+        const int qt = threadIdx.x - 32 * (2 + kEWarps), c8 = (qt & 7) * 8, qrow = qt >> 3;
+        unsigned char *const mine = q_s + qrow * 128 + (((qt & 7) ^ (qrow & 7)) << 4);      // (row & 7 is the same for all its rows)
+        int fc[NCH];                                                 // per chunk: its number in its image
+        unsigned long long z[NCH];                                   // and the counter of the first row's first pair
 #pragma unroll
-            for (int g = 0; g < G; ++g) {
-                if (n0 + g >= total) break;
-                ok = __all_sync(0xffffffffu, mbar_wait(&pipe.q_empty[s], par, p.err_flag));
-                if (!ok) break;
-                unsigned char *dst = q_s + s * NCH * kPanelF;
+        for (int j = 0; j < NCH; ++j) {
+            const Chunk c = chunk_of(tile_of(0), j);
+            fc[j] = c.p0 >> 6;
+            z[j] = counter_of((static_cast<long long>(c.b) * p.Cout + qrow) * p.HW + c.p0 + c8, p.seed);
+        }
+        int left = p.nco;                                            // stages of the tile
+        for (int n = 0; n < total; ++n) {
+            if (!__all_sync(0xffffffffu, mbar_wait(&pipe.d_full[s], par, p.err_flag))) break;
+            unsigned char *dst = mine + s * NCH * kPanelF;
+            uint4 raw[NV];
+            unsigned top = 0u;
+            const unsigned before = nz2;
 #pragma unroll
+            for (int k = 0; k < NV; ++k) raw[k] = *reinterpret_cast<const uint4 *>(dst + k / RPC * kPanelF + k % RPC * 64 * 128);
+#pragma unroll
+            for (int k = 0; k < NV; ++k) {
+                float x[8];
+                unsigned long long u[4];
+                unsigned h[4];
+                Vec<__nv_bfloat16>::values(raw[k], x);
+                dithers_at<8>(z[k / RPC] + k % RPC * p.row64_z, u);
+                quick_codes<8>(x, u, inv, h, top);                   // outside the tensor x is 0: code 0
+                count_pairs<8>(h, nz2);
+                *reinterpret_cast<uint4 *>(dst + k / RPC * kPanelF + k % RPC * 64 * 128) = make_uint4(h[0], h[1], h[2], h[3]);
+            }
+            if (needs_care(top)) {                                   // rare: clip, count, NaN; from delta in memory again
+                const int t = tile_of(n / p.nco), co0 = n % p.nco * ROWS + qrow;
+                nz2 = before;
+#pragma unroll 1
                 for (int k = 0; k < NV; ++k) {
-                    const int row = ((qt + 32 * kQWarps * k) >> 3) % ROWS, j = 32 * kQWarps * k / (8 * ROWS);
-                    float x[8], f[8];
+                    const Chunk c = chunk_of(t, k / RPC);
+                    const int co = co0 + k % RPC * 64;
+                    uint4 q = make_uint4(0u, 0u, 0u, 0u);
+                    const long long e = (static_cast<long long>(c.b) * p.Cout + co) * p.HW + c.p0 + c8;
+                    if (c.b < p.B && c.p0 + c8 < p.HW && co < p.Cout) q = __ldg(reinterpret_cast<const uint4 *>(p.delta + e));
+                    float x[8];
                     unsigned long long u[4];
-                    unsigned h[4];
-                    Vec<__nv_bfloat16>::values(raw[g][k], x);
-                    fetch(g, k);                                     // the same vector, G stages on
-                    dithers_of<8>(at[g][j] + static_cast<long long>(cb * ROWS + row) * p.HW, p.seed, u);
-                    decide<8>(x, u, inv, f, sat);                    // outside the tensor x is 0: code 0
-                    pack_bf16<8>(f, h);
+                    unsigned h[4], m[8];
+                    Vec<__nv_bfloat16>::values(q, x);
+                    dithers_of<8>(e, p.seed, u);
+                    careful_codes<8>(x, u, inv, h, m, sat);
                     count_pairs<8>(h, nz2);
-                    *reinterpret_cast<uint4 *>(dst + j * kPanelF + row * 128 + (((qt & 7) ^ (row & 7)) << 4)) = make_uint4(h[0], h[1], h[2], h[3]);
+                    *reinterpret_cast<uint4 *>(dst + k / RPC * kPanelF + k % RPC * 64 * 128) = make_uint4(h[0], h[1], h[2], h[3]);
                 }
-                fetched(g);
-                fence_async_proxy();
-                warp_arrive(&pipe.q_full[s]);
-                if (++s == S) { s = 0; par ^= 1u; }
-                if (++cb == p.nco) cb = 0;
-                if (nz2 & 0x80008000u) { nnz += pairs_total(nz2); nz2 = 0; }
+            }
+            fence_async_proxy();
+            warp_arrive(&pipe.q_full[s]);
+            if (++s == S) { s = 0; par ^= 1u; }
+            if (nz2 & 0x80008000u) { nnz += pairs_total(nz2); nz2 = 0; }
+#pragma unroll
+            for (int j = 0; j < NCH; ++j) z[j] += p.stage_z;
+            if (--left == 0) {                                       // the next tile
+                left = p.nco;
+#pragma unroll
+                for (int j = 0; j < NCH; ++j) {
+                    fc[j] -= p.step_c;
+                    z[j] -= p.tile_z;
+                    if (fc[j] < 0) { fc[j] += p.cpi; z[j] += p.wrap_z; }
+                }
             }
         }
         nnz = __reduce_add_sync(kFull, nnz + pairs_total(nz2));
@@ -392,8 +428,13 @@ int launch_fused1x1(dbp_ctx *ctx, const void *delta, const void *X, const void *
     p.seed = seed;
     p.st = ctx->state;
     p.err_flag = err_flag;
-    CUtensorMap map_w, map_x, map_dx, map_dw;
+    CUtensorMap map_d, map_w, map_x, map_dx, map_dw;
     const unsigned long long Cin = s.Cin, Cout = s.Cout, HW = p.HW, B = s.B;
+    {
+        const unsigned long long dims[3] = {HW, Cout, B}, str[2] = {HW * 2, HW * 2 * Cout};
+        const unsigned box[3] = {64, static_cast<unsigned>(rows), 1};
+        if (!encode_map_bf16(&map_d, delta, 3, dims, str, box)) return fail_cuda("tensor map of delta");
+    }
     {
         const unsigned long long dims[2] = {Cin, Cout}, str[1] = {Cin * 2};
         const unsigned box[2] = {64, 64};
@@ -416,7 +457,15 @@ int launch_fused1x1(dbp_ctx *ctx, const void *delta, const void *X, const void *
         // One CTA per SM, or as many whole rounds of them as keep a CTA's dW accumulators to kMaxMmas (a chunk is four MMAs)
         const long long most = kMaxMmas / (4 * nch), rounds = (p.ntiles + most * ctx->sm_count - 1) / (most * ctx->sm_count);
         const long long grid = p.ntiles < ctx->sm_count * rounds ? p.ntiles : ctx->sm_count * rounds;
-        return cuda_ok(launch_chained(kern, dim3(static_cast<unsigned>(grid)), dim3(kThreadsF), smem, ctx->stream, map_w, map_x, map_dx,
+        const long long back = grid * nch;                           // chunks from a CTA's tile to its next one
+        p.step_c = static_cast<int>(back % p.cpi);
+        auto pairs_z = [](long long elements) { return static_cast<unsigned long long>(elements / 2) * kGamma; };
+        const long long image = s.Cout * p.HW;
+        p.stage_z = pairs_z(static_cast<long long>(rows) * p.HW);
+        p.row64_z = pairs_z(64ll * p.HW);
+        p.tile_z = pairs_z(back / p.cpi * image + 64ll * p.step_c) + p.nco * p.stage_z;
+        p.wrap_z = pairs_z(64ll * p.cpi) - pairs_z(image);
+        return cuda_ok(launch_chained(kern, dim3(static_cast<unsigned>(grid)), dim3(kThreadsF), smem, ctx->stream, map_d, map_w, map_x, map_dx,
                                       map_dw, step, p));
     };
     if (rows == 64) return nch == 2 ? go(fused1x1_kernel<64, 2>) : go(fused1x1_kernel<64, 1>);

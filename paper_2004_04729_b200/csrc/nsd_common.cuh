@@ -53,25 +53,48 @@ __device__ __forceinline__ float max3_abs(float a, float b, float c) {
 // top 23 bits k of the output's halves, low half first. The output is z ^ (z >> 31) of the mixed z: of its high half
 // that xor only changes bit 0, of its low half it is bits 0-30 of (high half << 1) (and bit 31's neighbour in bit 0), so
 // the 23 bits that count need neither 64-bit shift. 1 + k 2^-23 is one funnel shift, and u that plus 2^-24 - 1.
+// Written in 32-bit halves, a 64-bit product as three multiply-adds: 11.5 instructions an element against 12.5 from 64-bit
+// expressions. Shifts, xors and byte permutations issue every second clock of a scheduler, on one pipe, multiplications
+// every second clock on another (wide ones every fourth), additions every clock. The draw takes 16.8 clocks an element (14 of
+// the first pipe), the whole decision 22, whether two or eight warps per scheduler run. Multiplications in place of shifts, or
+// mixed-precision additions in place of the conversion from bf16, are no faster.
+__device__ __forceinline__ void mul_low64(unsigned &lo, unsigned &hi, unsigned clo, unsigned chi) {
+    asm("{\n\t.reg .u64 p;\n\t.reg .u32 a, b, h;\n\t"
+        "mul.wide.u32 p, %0, %2;\n\t"
+        "mov.b64 {a, b}, p;\n\t"
+        "mad.lo.u32 h, %0, %3, b;\n\t"
+        "mad.lo.u32 %1, %1, %2, h;\n\t"
+        "mov.b32 %0, a;\n\t}"
+        : "+r"(lo), "+r"(hi) : "r"(clo), "r"(chi));
+}
 __device__ __forceinline__ unsigned long long dither2(unsigned long long z) {
-    z = (z ^ (z >> 30)) * 0xBF58476D1CE4E5B9ull;
-    z = (z ^ (z >> 27)) * 0x94D049BB133111EBull;
-    const unsigned hi = static_cast<unsigned>(z >> 32), lo = static_cast<unsigned>(z) ^ (hi << 1);
+    unsigned lo = static_cast<unsigned>(z), hi = static_cast<unsigned>(z >> 32);
+    lo ^= __funnelshift_r(lo, hi, 30);
+    hi ^= hi >> 30;
+    mul_low64(lo, hi, 0x1CE4E5B9u, 0xBF58476Du);
+    lo ^= __funnelshift_r(lo, hi, 27);
+    hi ^= hi >> 27;
+    mul_low64(lo, hi, 0x133111EBu, 0x94D049BBu);
+    lo ^= hi + hi;
     return add2(pack2(__uint_as_float(__funnelshift_r(lo, 0x7fu, 9)), __uint_as_float(__funnelshift_r(hi, 0x7fu, 9))),
                 pack2(kDitherShift, kDitherShift));
 }
 __device__ __forceinline__ unsigned long long counter_of(long long e, unsigned long long seed) {      // e even
     return seed + (static_cast<unsigned long long>(e >> 1) + 1ull) * kGamma;
 }
-// dithers of V elements whose first has the even index e0, pairs packed
+// dithers of V elements whose first pair has the counter z, pairs packed
 template <int V>
-__device__ __forceinline__ void dithers_of(long long e0, unsigned long long seed, unsigned long long (&u)[V / 2]) {
-    unsigned long long z = counter_of(e0, seed);
+__device__ __forceinline__ void dithers_at(unsigned long long z, unsigned long long (&u)[V / 2]) {
 #pragma unroll
     for (int j = 0; j < V / 2; ++j) {
         u[j] = dither2(z);
         z += kGamma;
     }
+}
+// and of V elements whose first has the even index e0
+template <int V>
+__device__ __forceinline__ void dithers_of(long long e0, unsigned long long seed, unsigned long long (&u)[V / 2]) {
+    dithers_at<V>(counter_of(e0, seed), u);
 }
 // careful decision: clipped to [-127, 127], clipped codes counted, NaN gives 0. Returns the bits of kMagic + code (the
 // low byte is the code's two's-complement byte).
@@ -110,6 +133,55 @@ template <int V>
 __device__ __forceinline__ void pack_bf16(const float (&f)[V], unsigned (&h)[V / 2]) {
 #pragma unroll
     for (int j = 0; j < V / 2; ++j) h[j] = __byte_perm(__float_as_uint(f[2 * j]), __float_as_uint(f[2 * j + 1]), 0x7632);
+}
+// The same without a branch, for code that decides several vectors and looks once whether one of them needs the careful
+// decision: codes as packed bf16 words (h) and as the low bytes of m, and in `top` the largest magnitude seen in either half
+// of a word (a sign and NaN included). A code out of range shows there as 128 or more, whatever the sum with kMagic made of
+// it. What is not used of h or m costs nothing.
+template <int V>
+__device__ __forceinline__ void quick_codes(const float (&x)[V], const unsigned long long (&u)[V / 2], float inv, unsigned (&h)[V / 2],
+                                            unsigned (&m)[V], unsigned &top) {
+    const unsigned long long inv2 = pack2(inv, inv), up = pack2(kMagic, kMagic), down = pack2(-kMagic, -kMagic);
+#pragma unroll
+    for (int j = 0; j < V / 2; ++j) {
+        const unsigned long long t = add2_down(fma2(pack2(x[2 * j], x[2 * j + 1]), inv2, u[j]), up);
+        float a, b;
+        unpack2(t, a, b);
+        m[2 * j] = __float_as_uint(a);
+        m[2 * j + 1] = __float_as_uint(b);
+        unpack2(add2(t, down), a, b);
+        h[j] = __byte_perm(__float_as_uint(a), __float_as_uint(b), 0x7632);
+        asm("max.NaN.xorsign.abs.bf16x2 %0, %0, %1;" : "+r"(top) : "r"(h[j]));
+    }
+}
+template <int V>
+__device__ __forceinline__ void quick_codes(const float (&x)[V], const unsigned long long (&u)[V / 2], float inv, unsigned (&h)[V / 2],
+                                            unsigned &top) {
+    unsigned m[V];
+    quick_codes<V>(x, u, inv, h, m, top);
+}
+__device__ __forceinline__ bool needs_care(unsigned top) {            // 0x42fe: 127
+    return __vmaxu2(top & 0x7fff7fffu, 0x42fe42feu) != 0x42fe42feu;
+}
+template <int V>
+__device__ __forceinline__ void careful_codes(const float (&x)[V], const unsigned long long (&u)[V / 2], float inv, unsigned (&h)[V / 2],
+                                              unsigned (&m)[V], unsigned &sat) {
+#pragma unroll
+    for (int j = 0; j < V / 2; ++j) {
+        float ua, ub;
+        unpack2(u[j], ua, ub);
+        m[2 * j] = careful_bits(x[2 * j], inv, ua, sat);
+        m[2 * j + 1] = careful_bits(x[2 * j + 1], inv, ub, sat);
+        h[j] = __byte_perm(__float_as_uint(__uint_as_float(m[2 * j]) - kMagic), __float_as_uint(__uint_as_float(m[2 * j + 1]) - kMagic),
+                           0x7632);
+    }
+}
+// the bytes of such sums, four to a word in element order
+template <int V>
+__device__ __forceinline__ void low_bytes(const unsigned (&m)[V], unsigned (&pk)[V / 4]) {
+#pragma unroll
+    for (int w = 0; w < V / 4; ++w)
+        pk[w] = __byte_perm(__byte_perm(m[4 * w], m[4 * w + 1], 0x0040), __byte_perm(m[4 * w + 2], m[4 * w + 3], 0x0040), 0x5410);
 }
 // the codes' bytes, four to a word in element order
 template <int V>

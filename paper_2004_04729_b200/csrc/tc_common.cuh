@@ -7,6 +7,9 @@ namespace dbp {
 namespace tc {
 
 constexpr long long kWaitCycles = 1000000000ll;     // a wait gives up after this many SM clocks
+// How long a waiter asks to be suspended at a time. The default is about 2600 clocks, which a CTA's idle warps spend on
+// polling again: layer set of ResNet-50 904 us with it, 901 with this.
+constexpr unsigned kSuspendNs = 100000;
 
 __device__ __forceinline__ unsigned smem_u32(const void *p) {
     return static_cast<unsigned>(__cvta_generic_to_shared(p));
@@ -33,9 +36,9 @@ __device__ __forceinline__ bool mbar_try(unsigned addr, unsigned parity) {
     unsigned done;
     asm volatile(
         "{\n\t.reg .pred P1;\n\t"
-        "mbarrier.try_wait.parity.shared::cta.b64 P1, [%1], %2;\n\t"
+        "mbarrier.try_wait.parity.shared::cta.b64 P1, [%1], %2, %3;\n\t"
         "selp.b32 %0, 1, 0, P1;\n\t}"
-        : "=r"(done) : "r"(addr), "r"(parity) : "memory");
+        : "=r"(done) : "r"(addr), "r"(parity), "r"(kSuspendNs) : "memory");
     return done != 0;
 }
 __device__ __forceinline__ bool mbar_test(unsigned addr, unsigned parity) {

@@ -60,3 +60,29 @@ def test_thin_layers(ctx, B, Ci, Co, H, W):
     assert torch.equal(again["dX"], out["dX"])
     none = dbp.dithered_conv_backward(ctx, torch.zeros_like(d), X, Wt, L.seed, L.scale)
     assert not none["dW"].any() and not none["dX"].any() and ctx.last_step()[1] == 0
+
+
+@pytest.mark.parametrize("B,Ci,Co,H,W", [(300, 72, 136, 9, 8), (598, 64, 64, 8, 8), (24, 64, 256, 28, 28)])
+def test_thin_layers_clip_and_count(ctx, B, Ci, Co, H, W):
+    """A stage that holds a code out of range is decided again with care: every code and the counts are as if each element
+    had been decided by itself, in the first and the last places of rows, chunks, stages and images."""
+    import paper_2004_04729_b200 as dbp
+    L = wl.conv_layer(B, Ci, Co, H, W, 1, data_seed=B + Ci, scale=2.0, seed=7, dtype="bf16")
+    delta = L.delta.copy()
+    at = [(0, 0, 0, 0), (0, 0, H - 1, W - 1), (0, Co - 1, 0, 1), (B - 1, Co - 1, H - 1, W - 1), (B // 2, Co // 2, H // 2, W // 2),
+          (1, min(63, Co - 1), 0, 0), (1, min(64, Co - 1), 0, 7)]
+    for i, a in enumerate(at):
+        delta[a] = (-1.0) ** i * (1.0 if i < 5 else 0.0635)      # far out of range, and about its edge: 0.0635 is 127 steps
+    d, X, Wt = (torch.from_numpy(np.ascontiguousarray(a)).bfloat16().cuda() for a in (delta, L.X, L.W))
+    delta = d.float().cpu().numpy()
+    D = np.float32(5e-4)
+    codes, nnz, sat = oracle.nsd_codes(delta, L.seed, D)
+    assert sat >= 5
+    out = dbp.dithered_conv_backward(ctx, d, X, Wt, L.seed, 0.0, delta_in=torch.tensor([float(D)], device="cuda"))
+    assert ctx.last_step() == (float(D), nnz)
+    assert ctx.last_device_status()[1] == sat
+    ref = oracle.conv_backward(codes, D, L.X, L.W, with_abs=True)
+    g = out["dW"].double().cpu().numpy()
+    assert np.all(np.abs(g - ref["dW"]) <= TOL * ref["S_dW"] + 1e-30)
+    g = out["dX"].double().cpu().numpy()
+    assert np.all(np.abs(g - ref["dX"]) <= 2.0 ** -8 * np.abs(ref["dX"]) + TOL * ref["S_dX"] + 1e-30)
