@@ -144,10 +144,10 @@ int quantize_for_products(dbp_ctx *ctx, const void *delta, int dtype, long long 
                                            planes_hw, planes_pitch, false);
             if (!rc && pn)
                 rc = launch_quantize_nhwc(ctx, delta, dtype, nhwc->B, nhwc->Cout, nhwc->H * nhwc->W, seed,
-                                          step, pn, nullptr, false, ps, static_cast<int>(nhwc->W));
+                                          step, pn, false, ps, static_cast<int>(nhwc->W));
         } else if (pn) {
             rc = launch_quantize_nhwc(ctx, delta, dtype, nhwc->B, nhwc->Cout, nhwc->H * nhwc->W, seed,
-                                      step, pn, want8 ? dense : nullptr, true, ps, static_cast<int>(nhwc->W), mask);
+                                      step, pn, true, ps, static_cast<int>(nhwc->W), mask);
         } else {
             rc = launch_quantize_dense(ctx, delta, dtype, numel, seed, step, want8 ? dense : nullptr,
                                        p16, planes_hw, planes_pitch, true, mask);

@@ -160,15 +160,13 @@ int launch_quantize(dbp_ctx *ctx, const void *delta, int dtype, long long numel,
                     uint16_t *offsets, int8_t *values, int8_t *dense,
                     unsigned long long *nnz_out);
 // ---- nsd_dense.cu: the same codes, dense array only (no sparse structure)
-// dense: int8 codes in delta's order (or null); planes_bf16: bf16 codes as [numel / hw][pitch]
-// (or null), pitch a multiple of 8
+// either dense: int8 codes in delta's order, or planes_bf16: bf16 codes as [numel / hw][pitch], pitch a multiple of 8
 int launch_quantize_dense(dbp_ctx *ctx, const void *delta, int dtype, long long numel,
                           unsigned long long seed, const StepSource &step, int8_t *dense,
                           void *planes_bf16, long long hw, long long pitch, bool count, const uint8_t *mask = nullptr);
-// position-major bf16 codes [B][HW][C] for the TMA-fed 3x3 kernels (and int8 codes in delta's order
-// when dense8 is not null)
+// position-major bf16 codes [B][HW][C] for the TMA-fed 3x3 kernels
 int launch_quantize_nhwc(dbp_ctx *ctx, const void *delta, int dtype, long long B, long long C, long long HW,
-                         unsigned long long seed, const StepSource &step, void *codes_nhwc, int8_t *dense8, bool count,
+                         unsigned long long seed, const StepSource &step, void *codes_nhwc, bool count,
                          void *codes_stack = nullptr, int plane_w = 0, const uint8_t *mask = nullptr);
 int launch_decode(dbp_ctx *ctx, const uint32_t *bitmap, const uint16_t *offsets,
                   const int8_t *values, long long numel, int8_t *dense);

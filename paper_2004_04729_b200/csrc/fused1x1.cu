@@ -66,7 +66,7 @@ template <int ROWS, int NCH>
 __global__ void __launch_bounds__(kThreadsF, 1)
 fused1x1_kernel(const __grid_constant__ CUtensorMap map_d, const __grid_constant__ CUtensorMap map_w, const __grid_constant__ CUtensorMap map_x,
                 const __grid_constant__ CUtensorMap map_dx, const __grid_constant__ CUtensorMap map_dw,
-                const __grid_constant__ StepSource step, const Fused1P p) {
+                const StepSource step, const Fused1P p) {
     constexpr int NV = ROWS * NCH * 8 / (32 * kQWarps);              // vectors per quantizer thread and stage
     extern __shared__ __align__(1024) unsigned char smem_raw[];
     unsigned char *smem = reinterpret_cast<unsigned char *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
@@ -137,8 +137,9 @@ fused1x1_kernel(const __grid_constant__ CUtensorMap map_d, const __grid_constant
         load_x(0);
         if (my_tiles > 1) load_x(1);
     }
+    const StepSource from = step_ahead(step);
     chain_wait();
-    const float delta = step_of<kThreadsF>(step, p.st);
+    const float delta = step_of<kThreadsF>(from, p.st);
 
     if (warp == 0) {
         if (lane == 0) {

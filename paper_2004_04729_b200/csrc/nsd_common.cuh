@@ -96,6 +96,15 @@ template <int V>
 __device__ __forceinline__ void dithers_of(long long e0, unsigned long long seed, unsigned long long (&u)[V / 2]) {
     dithers_at<V>(counter_of(e0, seed), u);
 }
+// Dithers drawn ahead of a wait stay there: without this the compiler moves the arithmetic behind the wait (about 1 us of each
+// of the quantizers).
+template <int N, int P>
+__device__ __forceinline__ void keep_here(unsigned long long (&u)[N][P]) {
+#pragma unroll
+    for (int k = 0; k < N; ++k)
+#pragma unroll
+        for (int j = 0; j < P; ++j) asm volatile("" : "+l"(u[k][j]));
+}
 // careful decision: clipped to [-127, 127], clipped codes counted, NaN gives 0. Returns the bits of kMagic + code (the
 // low byte is the code's two's-complement byte).
 __device__ __forceinline__ unsigned careful_bits(float x, float inv, float u, unsigned &sat) {
@@ -159,6 +168,22 @@ __device__ __forceinline__ void quick_codes(const float (&x)[V], const unsigned 
                                             unsigned &top) {
     unsigned m[V];
     quick_codes<V>(x, u, inv, h, m, top);
+}
+// the same for the same elements of two rows: a word holds the codes of one place, row a's in its low half
+template <int V>
+__device__ __forceinline__ void quick_codes2(const float (&xa)[V], const float (&xb)[V], const unsigned long long (&ua)[V / 2],
+                                             const unsigned long long (&ub)[V / 2], float inv, unsigned (&w)[V], unsigned &top) {
+    const unsigned long long inv2 = pack2(inv, inv), up = pack2(kMagic, kMagic), down = pack2(-kMagic, -kMagic);
+#pragma unroll
+    for (int j = 0; j < V / 2; ++j) {
+        float a0, a1, b0, b1;
+        unpack2(add2(add2_down(fma2(pack2(xa[2 * j], xa[2 * j + 1]), inv2, ua[j]), up), down), a0, a1);
+        unpack2(add2(add2_down(fma2(pack2(xb[2 * j], xb[2 * j + 1]), inv2, ub[j]), up), down), b0, b1);
+        w[2 * j] = __byte_perm(__float_as_uint(a0), __float_as_uint(b0), 0x7632);
+        w[2 * j + 1] = __byte_perm(__float_as_uint(a1), __float_as_uint(b1), 0x7632);
+        asm("max.NaN.xorsign.abs.bf16x2 %0, %0, %1;" : "+r"(top) : "r"(w[2 * j]));
+        asm("max.NaN.xorsign.abs.bf16x2 %0, %0, %1;" : "+r"(top) : "r"(w[2 * j + 1]));
+    }
 }
 __device__ __forceinline__ bool needs_care(unsigned top) {            // 0x42fe: 127
     return __vmaxu2(top & 0x7fff7fffu, 0x42fe42feu) != 0x42fe42feu;
@@ -238,6 +263,12 @@ struct Vec<__nv_bfloat16> {
 // Delta = scale * sigma rounded once to fp32, sigma the population standard deviation about the mean; 0 (every code 0)
 // for constant and for non-finite tensors. The first CTA publishes it. All threads of the block call this.
 // Returns Delta, or 0 where no code can be non-zero.
+// The parameters it needs, in registers: read ahead of the wait for the statistics kernel.
+__device__ __forceinline__ StepSource step_ahead(StepSource s) {
+    asm volatile("" : "+l"(s.partials), "+r"(s.nparts), "+f"(s.scale), "+d"(s.inv_numel), "+l"(s.given), "+l"(s.publish[0]),
+                 "+l"(s.publish[1]), "+l"(s.publish[2]));
+    return s;
+}
 template <int THREADS>
 __device__ __forceinline__ float step_of(const StepSource &s, DeviceState *st) {
     __shared__ double sum_s[2][THREADS / 32];
@@ -245,7 +276,10 @@ __device__ __forceinline__ float step_of(const StepSource &s, DeviceState *st) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     if (s.given != nullptr) {
         const float d = __ldcg(s.given);
-        if (blockIdx.x == 0 && threadIdx.x < 3 && s.publish[threadIdx.x] != nullptr) *s.publish[threadIdx.x] = d;
+        if (blockIdx.x == 0 && threadIdx.x == 0)
+#pragma unroll
+            for (int i = 0; i < 3; ++i)
+                if (s.publish[i] != nullptr) *s.publish[i] = d;
         return d > 0.f && d < __int_as_float(0x7f800000) ? d : 0.f;
     }
     double a = 0.0, b = 0.0;

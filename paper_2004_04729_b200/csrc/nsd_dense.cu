@@ -11,6 +11,8 @@
 // complete. In the loop the next vectors are loaded before the current ones are stored.
 #include "nsd_common.cuh"
 
+#include <type_traits>
+
 namespace dbp {
 
 namespace {
@@ -20,13 +22,20 @@ using namespace nsd;
 constexpr int kThreads = 256;
 constexpr int kBlocksPerSM = 3;                   // resident blocks the dense quantizer is compiled for
 
-// Where the codes go. dense8: one byte per element, same order as delta_z (may be null).
-// planes16: bf16 codes as [plane][pitch] with plane = e / hw (may be null); the pitch is a
-// multiple of 8 so that every plane starts on a 16-byte boundary.
+// Where the codes of the flat quantizer go:
+//   kBytes: one byte per element, same order as delta_z;
+//   kSame:  bf16, same order;
+//   kPad4:  bf16 as [plane][hw + 4], planes of an odd multiple of four elements (so every plane starts on a 16-byte boundary);
+//   kAny:   bf16 as [plane][pitch], planes of any size.
+enum { kBytes, kSame, kPad4, kAny };
 struct CodeSinks {
     int8_t *dense8;
     unsigned short *planes16;
     long long hw, pitch;
+    // kPad4: from one of a thread's vectors to the next, and from its last one of a tile to the first of its next tile: whole
+    // planes and a rest, as the rest (elements) and the distance in the output without a plane's end between them
+    int rest1, rest2;
+    long long dist1, dist2;
     int count;                    // add nnz / clipped counts to the context's counters
 };
 
@@ -43,52 +52,26 @@ __device__ __forceinline__ void split_index(long long e, long long hw, long long
     }
 }
 
-// f: the codes as floats, h: as packed bf16
+// kAny: code by code, or two at a time where the pair starts on an even offset of its plane and does not run over the plane's end
 template <int V>
-__device__ __forceinline__ void store_codes(const CodeSinks &o, long long e0, const float (&f)[V], const unsigned (&h)[V / 2]) {
-    if (o.dense8 != nullptr) {
-        unsigned pk[V / 4];
-        pack_bytes<V>(f, pk);
-        if (V == 4) *reinterpret_cast<unsigned *>(o.dense8 + e0) = pk[0];
-        else *reinterpret_cast<uint2 *>(o.dense8 + e0) = make_uint2(pk[0], pk[V / 4 - 1]);
-    }
-    if (o.planes16 != nullptr) {
-        if (o.pitch == o.hw) {                      // planes are back to back: same order as delta_z
-            if (V == 4) *reinterpret_cast<uint2 *>(o.planes16 + e0) = make_uint2(h[0], h[1]);
-            else *reinterpret_cast<uint4 *>(o.planes16 + e0) = make_uint4(h[0], h[1], h[V / 2 - 2], h[V / 2 - 1]);
-        } else if ((o.hw & 3) == 0) {
-            // e0 and the plane size are multiples of 4: each group of four codes lies in one plane
-            // and starts on an 8-byte boundary there
-            long long plane, pp;
-            split_index(e0, o.hw, plane, pp);
+__device__ __forceinline__ void store_any(const CodeSinks &o, long long e0, const unsigned (&h)[V / 2]) {
+    long long plane, pp;
+    split_index(e0, o.hw, plane, pp);
+    unsigned short *dst = o.planes16 + plane * o.pitch + pp;
+    long long left = o.hw - pp;                           // codes until the plane ends
+    const long long gap = o.pitch - o.hw;
 #pragma unroll
-            for (int g = 0; g < V / 4; ++g) {
-                *reinterpret_cast<uint2 *>(o.planes16 + plane * o.pitch + pp) = make_uint2(h[2 * g], h[2 * g + 1]);
-                pp += 4;
-                if (pp == o.hw) { pp = 0; ++plane; }
-            }
+    for (int j = 0; j < V; j += 2) {
+        if (left >= 2 && (reinterpret_cast<uintptr_t>(dst) & 3) == 0) {
+            *reinterpret_cast<unsigned *>(dst) = h[j >> 1];
+            dst += 2;
+            left -= 2;
+            if (left == 0) { left = o.hw; dst += gap; }
         } else {
-            // odd plane sizes: code by code, or two at a time where the pair starts on an even offset
-            // of its plane and does not run over the plane's end
-            long long plane, pp;
-            split_index(e0, o.hw, plane, pp);
-            unsigned short *dst = o.planes16 + plane * o.pitch + pp;
-            long long left = o.hw - pp;                           // codes until the plane ends
-            const long long gap = o.pitch - o.hw;
-#pragma unroll
-            for (int j = 0; j < V; j += 2) {
-                if (left >= 2 && (reinterpret_cast<uintptr_t>(dst) & 3) == 0) {
-                    *reinterpret_cast<unsigned *>(dst) = h[j >> 1];
-                    dst += 2;
-                    left -= 2;
-                    if (left == 0) { left = o.hw; dst += gap; }
-                } else {
-                    *dst++ = static_cast<unsigned short>(h[j >> 1]);
-                    if (--left == 0) { left = o.hw; dst += gap; }
-                    *dst++ = static_cast<unsigned short>(h[j >> 1] >> 16);
-                    if (--left == 0) { left = o.hw; dst += gap; }
-                }
-            }
+            *dst++ = static_cast<unsigned short>(h[j >> 1]);
+            if (--left == 0) { left = o.hw; dst += gap; }
+            *dst++ = static_cast<unsigned short>(h[j >> 1] >> 16);
+            if (--left == 0) { left = o.hw; dst += gap; }
         }
     }
 }
@@ -100,6 +83,11 @@ __device__ __forceinline__ void store_code(const CodeSinks &o, long long e, unsi
         o.planes16[plane * o.pitch + (e - plane * o.hw)] = static_cast<unsigned short>(__float_as_uint(f) >> 16);
     }
 }
+template <int V>
+__device__ __forceinline__ void store_vec(unsigned short *dst, const unsigned (&h)[V / 2]) {
+    if (V == 4) *reinterpret_cast<uint2 *>(dst) = make_uint2(h[0], h[1]);
+    else *reinterpret_cast<uint4 *>(dst) = make_uint4(h[0], h[1], h[V / 2 - 2], h[V / 2 - 1]);
+}
 
 // mask (fp32 tensors only): x is delta_a and the gradient is delta_a where mask != 0, else 0. The four mask bytes of a
 // vector as one word.
@@ -110,60 +98,136 @@ __device__ __forceinline__ void apply_mask(unsigned m, float (&v)[4]) {
 }
 __device__ __forceinline__ void apply_mask(unsigned, float (&)[8]) {}                 // bf16 tensors take no mask
 
-template <typename T, bool MASKED>
+// A block takes tiles of 16 elements per thread: a thread's vectors lie 256 vectors apart, so that within a tile every address
+// and every counter of the dither is the first one's plus a constant, and from tile to tile all of them advance by constants.
+constexpr int kPerThread = 16;
+
+template <typename T, bool MASKED, int SINK>
 __global__ void __launch_bounds__(kThreads, kBlocksPerSM)
 quantize_dense_kernel(const T *__restrict__ x, long long n, unsigned long long seed, const StepSource step,
-                      const CodeSinks out, DeviceState *__restrict__ st, const unsigned char *__restrict__ mask) {
-    constexpr int V = Vec<T>::V;
-    const long long nvec = n / V;
-    const long long stride = static_cast<long long>(gridDim.x) * kThreads;
-    long long i = static_cast<long long>(blockIdx.x) * kThreads + threadIdx.x;
-    // two vectors per thread and round: i and i + stride
-    uint4 r0, r1;
-    unsigned m0 = 0, m1 = 0;
-    unsigned long long u0[V / 2], u1[V / 2];
-    auto load = [&](long long k) {
-        r0 = k < nvec ? Vec<T>::raw(x + k * V) : make_uint4(0u, 0u, 0u, 0u);
-        r1 = k + stride < nvec ? Vec<T>::raw(x + (k + stride) * V) : make_uint4(0u, 0u, 0u, 0u);
-        if (MASKED) {
-            m0 = k < nvec ? mask_word(mask, k * V) : 0u;
-            m1 = k + stride < nvec ? mask_word(mask, (k + stride) * V) : 0u;
+                      const __grid_constant__ CodeSinks out, DeviceState *__restrict__ st, const unsigned char *__restrict__ mask) {
+    constexpr int V = Vec<T>::V, NV = kPerThread / V, kTile = kThreads * kPerThread;
+    constexpr int kBetween = kThreads * V;                             // elements between two vectors of a thread
+    constexpr unsigned long long kBetweenZ = kBetween / 2 * kGamma;
+    const long long nvec = n / V, whole = nvec / (kTile / V);          // whole tiles; the next one holds what is left
+    const int ragged = static_cast<int>(nvec - whole * (kTile / V));   // vectors
+    const long long ntile = whole + (ragged > 0);
+    const long long stride_e = static_cast<long long>(gridDim.x) * kTile;
+    const unsigned long long stride_z = static_cast<unsigned long long>(stride_e / 2) * kGamma;
+    long long t = blockIdx.x;
+    long long e0 = t * kTile + threadIdx.x * V;                        // the thread's first element of the tile
+    unsigned long long z = counter_of(e0, seed);
+    uint4 raw[NV];
+    unsigned msk[MASKED ? NV : 1];
+    unsigned long long u[NV][V / 2];
+    auto there = [&](int k) { return static_cast<int>(threadIdx.x) + k * kThreads < ragged; };      // in the tile after the whole ones
+    auto load = [&](long long tile, long long e) {
+        if (tile < whole) {
+#pragma unroll
+            for (int k = 0; k < NV; ++k) {
+                raw[k] = Vec<T>::raw(x + e + k * kBetween);
+                if (MASKED) msk[k] = mask_word(mask, e + k * kBetween);
+            }
+        } else if (tile == whole) {
+#pragma unroll
+            for (int k = 0; k < NV; ++k) {
+                raw[k] = there(k) ? Vec<T>::raw(x + e + k * kBetween) : make_uint4(0u, 0u, 0u, 0u);
+                if (MASKED) msk[k] = there(k) ? mask_word(mask, e + k * kBetween) : 0u;
+            }
         }
     };
-    auto draw = [&](long long k) {
-        dithers_of<V>(k * V, seed, u0);
-        dithers_of<V>((k + stride) * V, seed, u1);
+    auto draw = [&](unsigned long long zz) {
+#pragma unroll
+        for (int k = 0; k < NV; ++k) dithers_at<V>(zz + k * kBetweenZ, u[k]);
     };
-    load(i);
-    draw(i);
+    load(t, e0);
+    draw(z);
+    keep_here(u);
+    const StepSource from = step_ahead(step);
     chain_wait();
     chain_release();
-    const float delta = step_of<kThreads>(step, st);
+    const float delta = step_of<kThreads>(from, st);
     const float inv = delta > 0.f ? __fdiv_rn(1.0f, delta) : 0.f;      // Delta = 0: x * 0 + u < 1, every code 0 (NaN too)
     unsigned sat = 0, nz2 = 0, nnz = 0;
-    for (; i < nvec; ) {
-        float v[V], f0[V], f1[V];
-        Vec<T>::values(r0, v);
-        if (MASKED) apply_mask(m0, v);
-        decide<V>(v, u0, inv, f0, sat);
-        Vec<T>::values(r1, v);
-        if (MASKED) apply_mask(m1, v);
-        const bool two = i + stride < nvec;
-        decide<V>(v, u1, inv, f1, sat);
-        const long long k = i;
-        i += 2 * stride;
-        load(i);
-        unsigned h0[V / 2], h1[V / 2];
-        pack_bf16<V>(f0, h0);
-        pack_bf16<V>(f1, h1);
-        count_pairs<V>(h0, nz2);
-        store_codes<V>(out, k * V, f0, h0);
-        if (two) {
-            count_pairs<V>(h1, nz2);
-            store_codes<V>(out, (k + stride) * V, f1, h1);
+    int pp = 0;                                                        // kPad4: place in the plane
+    unsigned short *po = out.planes16;                                 // and in the output
+    if (SINK == kPad4 && t < ntile) {
+        long long plane, r;
+        split_index(e0, out.hw, plane, r);
+        pp = static_cast<int>(r);
+        po += plane * (out.hw + 4) + r;
+    }
+    // vector k of the tile at e goes out; pp and po walk from one of the thread's vectors to its next
+    auto store = [&](long long e, int k, const unsigned (&h)[V / 2], const unsigned (&m)[V]) {
+        if (SINK == kBytes) {
+            unsigned pk[V / 4];
+            low_bytes<V>(m, pk);
+            int8_t *dst = out.dense8 + e + k * kBetween;
+            if (V == 4) *reinterpret_cast<unsigned *>(dst) = pk[0];
+            else *reinterpret_cast<uint2 *>(dst) = make_uint2(pk[0], pk[V / 4 - 1]);
+        } else if (SINK == kSame) {
+            store_vec<V>(out.planes16 + e + k * kBetween, h);
+        } else if (SINK == kPad4) {
+            // each group of four codes lies in one plane and starts on an 8-byte boundary there
+            *reinterpret_cast<uint2 *>(po) = make_uint2(h[0], h[1]);
+            if (V == 8) {
+                if (pp + 4 < static_cast<int>(out.hw)) *reinterpret_cast<uint2 *>(po + 4) = make_uint2(h[V / 2 - 2], h[V / 2 - 1]);
+                else *reinterpret_cast<uint2 *>(po + 8) = make_uint2(h[V / 2 - 2], h[V / 2 - 1]);
+            }
+        } else {
+            store_any<V>(out, e + k * kBetween, h);
+        }
+    };
+    auto walk = [&](int k) {
+        if (SINK != kPad4) return;
+        pp += k + 1 < NV ? out.rest1 : out.rest2;
+        po += k + 1 < NV ? out.dist1 : out.dist2;
+        if (pp >= static_cast<int>(out.hw)) { pp -= static_cast<int>(out.hw); po += 4; }
+    };
+    for (; t < ntile; t += gridDim.x) {
+        unsigned h[NV][V / 2], m[NV][V], top = 0u;
+        const unsigned before = nz2;
+#pragma unroll
+        for (int k = 0; k < NV; ++k) {
+            float v[V];
+            Vec<T>::values(raw[k], v);
+            if (MASKED) apply_mask(msk[k], v);
+            quick_codes<V>(v, u[k], inv, h[k], m[k], top);
+            count_pairs<V>(h[k], nz2);                                 // (a vector that does not exist is zeros: code 0)
+        }
+        const long long e = e0;
+        e0 += stride_e;
+        load(t + gridDim.x, e0);
+        if (needs_care(top)) {                                         // rare: clip, count, NaN
+            nz2 = before;
+#pragma unroll 1
+            for (int k = 0; k < NV; ++k) {
+                if (t < whole || there(k)) {
+                    float v[V];
+                    unsigned long long d[V / 2];
+                    unsigned hc[V / 2], mc[V];
+                    Vec<T>::values(Vec<T>::raw(x + e + k * kBetween), v);
+                    if (MASKED) apply_mask(mask_word(mask, e + k * kBetween), v);
+                    dithers_at<V>(z + k * kBetweenZ, d);
+                    careful_codes<V>(v, d, inv, hc, mc, sat);
+                    count_pairs<V>(hc, nz2);
+                    store(e, k, hc, mc);
+                }
+                walk(k);
+            }
+        } else if (t < whole) {
+#pragma unroll
+            for (int k = 0; k < NV; ++k) { store(e, k, h[k], m[k]); walk(k); }
+        } else {
+#pragma unroll
+            for (int k = 0; k < NV; ++k) {
+                if (there(k)) store(e, k, h[k], m[k]);
+                walk(k);
+            }
         }
         if (nz2 & 0x80008000u) { nnz += pairs_total(nz2); nz2 = 0; }
-        if (i < nvec) draw(i);
+        z += stride_z;
+        if (t + gridDim.x < ntile) draw(z);
     }
     nnz += pairs_total(nz2);
     if (blockIdx.x == 0 && threadIdx.x == 0) {      // the n % V last elements, one by one
@@ -184,16 +248,24 @@ quantize_dense_kernel(const T *__restrict__ x, long long n, unsigned long long s
 // kernels read this form: a row of 64 channels of one position is 128 contiguous bytes, so a
 // rectangular patch of positions with its halo is one tiled copy and a tap of the filter is a row
 // offset inside it). delta_z itself is [image][channel][position], so a block transposes tiles of
-// 64 channels x 64 positions through shared memory: rows of the input are read along the
+// 64 channels x up to 64 positions through shared memory: rows of the input are read along the
 // positions, rows of the output are written along the channels. The dither of an element is
-// still keyed on its index in delta_z's own order.
-constexpr int kTC = 64, kTP = 64;                 // channels x positions per tile
+// still keyed on its index in delta_z's own order. The output's rows are padded to a multiple of eight channels (the
+// padding is not written: the copy engine never reads it).
+//
+// Planes of a multiple of V elements. A tile is P positions of one image, or G whole images of small planes (P = HW); a thread
+// takes the same V positions of two neighbouring channels, NI times, and writes the two codes of a position as one word.
+// Where these lie in a tile, in the input, in shared memory and in the dither's sequence is the same for every tile and made
+// once; what changes from tile to tile is the same for all threads. The first tile's loads and dithers, and every next tile's
+// loads, are under way before they are needed (see above).
+constexpr int kTC = 64, kTP = 64;                 // channels, most positions of a tile
 constexpr int kTileBytes = kTP * kTC * 2;
 
-// shared-memory byte offset of (position p, channel c) inside a tile: 128-byte rows, the
-// 16-byte pieces of a row permuted by the row's group of eight
+// shared-memory byte offset of (position p, channel c) inside a tile: 128-byte rows, the 16-byte pieces of a row permuted by
+// the number of the row's group of V (the eight groups and four channel pairs of a warp's words lie in different banks)
+template <int V>
 __device__ __forceinline__ unsigned tile_off(int p, int c) {
-    return static_cast<unsigned>(p) * 128u + (((static_cast<unsigned>(c) >> 3) ^ ((static_cast<unsigned>(p) >> 3) & 7u)) << 4) +
+    return static_cast<unsigned>(p) * 128u + (((static_cast<unsigned>(c) >> 3) ^ ((static_cast<unsigned>(p) / V) & 7u)) << 4) +
            ((static_cast<unsigned>(c) & 7u) << 1);
 }
 
@@ -211,135 +283,242 @@ __device__ __forceinline__ void values_of(const __nv_bfloat16 *, const uint4 &q,
     v[2] = __uint_as_float(q.y << 16); v[3] = __uint_as_float(q.y & 0xffff0000u);
 }
 
-template <int V>
-__device__ __forceinline__ void store_bytes(int8_t *dense8, long long e0, const float (&f)[V]) {
-    unsigned pk[V / 4];
-    pack_bytes<V>(f, pk);
-    if (V == 4) *reinterpret_cast<unsigned *>(dense8 + e0) = pk[0];
-    else *reinterpret_cast<uint2 *>(dense8 + e0) = make_uint2(pk[0], pk[V / 4 - 1]);
-}
+struct NhwcP {
+    int B, C, HW;
+    int P, G;                     // positions of an image, images of a tile
+    int pt, ct, ntiles;           // tiles along the positions, along the channels, in all (positions first, images last)
+    int step_p, step_c, step_b;   // from one of a block's tiles to its next
+    int plane_w;                  // stacked copy: rows of zeros after every image
+    int count;
+};
 
-// Three ways to fill a tile:
-//   kFlat: planes smaller than a tile's 64 positions (C % 8 == 0): the tile's 64 channels of one image are one contiguous
-//          run of delta_z, read as whole vectors whatever the plane size;
-//   kPair: plane size % V == 0: a thread takes the same V positions of two neighbouring channels and writes the two codes
-//          of a position as one word;
-//   kOdd:  any other plane: a channel's row of the tile is covered by the aligned vectors that touch it (one more than a
-//          row holds), and what lies outside the row is dropped.
-// The output's rows are padded to a multiple of eight channels (the padding is not written: the copy engine never reads
-// it). The first tile's loads and dithers, and every next tile's loads, are under way before they are needed (see above).
-enum { kFlat, kPair, kOdd };
-
-template <typename T, int V, int PATH, bool STACK, bool MASKED>
+template <typename T, int V, bool STACK, bool MASKED>
 __global__ void __launch_bounds__(kThreads, kBlocksPerSM)
-quantize_nhwc_kernel(const T *__restrict__ x, int B, int C, int HW, unsigned long long seed, const StepSource step,
-                     unsigned short *__restrict__ out, int8_t *__restrict__ dense8, DeviceState *__restrict__ st, int count,
-                     unsigned short *__restrict__ out_stack, int plane_w, const unsigned char *__restrict__ mask) {
+quantize_nhwc_kernel(const T *__restrict__ x, const NhwcP p, unsigned long long seed, const StepSource step,
+                     unsigned short *__restrict__ out, unsigned short *__restrict__ out_stack, DeviceState *__restrict__ st,
+                     const unsigned char *__restrict__ mask) {
     __shared__ __align__(16) unsigned char tile[2][kTileBytes];
-    constexpr int VPR = kTP / V;                                   // kPair: vectors per channel row of the tile
-    constexpr int NI = kTC * kTP / V / kThreads;                   // vectors per thread and tile (kFlat: at most)
-    const unsigned ct = (C + kTC - 1) / kTC, pt = (HW + kTP - 1) / kTP, per_img = ct * pt, ntiles = B * per_img;
-    const int pitch = (C + 7) & ~7;
+    constexpr int NI = kTC * kTP / (2 * V) / kThreads;             // pairs of vectors per thread and tile (at most)
+    const int C = p.C, HW = p.HW, pitch = (C + 7) & ~7;
+    const unsigned long long row_z = static_cast<unsigned long long>(HW / 2) * kGamma;
 
-    uint4 raw[NI];
-    unsigned msk[MASKED ? NI : 1];
-    unsigned long long u[NI][V / 2];
-    struct Tile { int b, c0, p0; };
-    auto tile_of = [&](unsigned t) {
-        Tile r;
-        r.b = t / per_img;
-        const unsigned rem = t - r.b * per_img;
-        r.c0 = (rem / pt) * kTC;
-        r.p0 = (rem - rem / pt * pt) * kTP;
-        return r;
+    // this thread's pairs of vectors in any tile: four channel pairs run fastest, then the positions, eights of channels, images
+    int in_off[NI], row[NI], ch[NI];                               // first element; first row of the tile; first channel
+    unsigned long long off_z[NI];
+#pragma unroll
+    for (int i = 0; i < NI; ++i) {
+        const int s = threadIdx.x + kThreads * i, vpr = p.P / V, q = s >> 2, r = q / vpr, pv = (q - r * vpr) * V, g = r >> 3;
+        ch[i] = 8 * (r & 7) + 2 * (s & 3);
+        row[i] = g < p.G ? g * p.P + pv : kTP;                     // kTP: in no tile
+        in_off[i] = (g * C + ch[i]) * HW + pv;
+        off_z[i] = static_cast<unsigned long long>((static_cast<long long>(g) * C + ch[i]) * HW + pv) / 2 * kGamma;
+    }
+    struct Tile { int b, c, p; };                                  // group of images, 64 channels, positions
+    auto base_of = [&](const Tile &t) { return (static_cast<long long>(t.b) * p.G * C + t.c * kTC) * HW + t.p * p.P; };
+    auto rows_of = [&](const Tile &t) {                            // rows of the tile that exist
+        const int n = p.G == 1 ? HW - t.p * p.P : (p.B - t.b * p.G) * HW;
+        return n < p.G * p.P ? n : p.G * p.P;
     };
-    // vector i of this thread: its first element, and whether it exists
-    auto vec_of = [&](const Tile &tl, int i, long long &e0) {
-        if (PATH == kFlat) {
-            const int v = threadIdx.x + kThreads * i, nch = C - tl.c0 < kTC ? C - tl.c0 : kTC;
-            e0 = (static_cast<long long>(tl.b) * C + tl.c0) * HW + v * V;
-            return v * V < nch * HW;
+    uint4 raw[NI][2];
+    unsigned msk[MASKED ? NI : 1][2];
+    unsigned long long u[NI][2][V / 2];
+    auto load = [&](const Tile &t) {
+        const long long base = base_of(t);
+        const int rows = rows_of(t), cleft = C - t.c * kTC;
+        if (cleft >= kTC && rows == kTP) {                         // a whole tile
+#pragma unroll
+            for (int i = 0; i < NI; ++i)
+#pragma unroll
+                for (int h = 0; h < 2; ++h) {
+                    raw[i][h] = load_raw<T, V>(x + base + in_off[i] + h * HW);
+                    if (MASKED) msk[i][h] = mask_word(mask, base + in_off[i] + h * HW);
+                }
+        } else {
+#pragma unroll
+            for (int i = 0; i < NI; ++i)
+#pragma unroll
+                for (int h = 0; h < 2; ++h) {
+                    const bool in = row[i] < rows && ch[i] + h < cleft;
+                    raw[i][h] = in ? load_raw<T, V>(x + base + in_off[i] + h * HW) : make_uint4(0u, 0u, 0u, 0u);
+                    if (MASKED) msk[i][h] = in ? mask_word(mask, base + in_off[i] + h * HW) : 0u;
+                }
         }
-        const int it = threadIdx.x + kThreads * (i >> 1), c = 2 * (it / VPR) + (i & 1), pv = (it % VPR) * V;
-        e0 = (static_cast<long long>(tl.b) * C + tl.c0 + c) * HW + tl.p0 + pv;
-        return tl.c0 + c < C && tl.p0 + pv < HW;
     };
-    auto load = [&](const Tile &tl) {
+    auto draw = [&](const Tile &t) {
+        const unsigned long long z = counter_of(base_of(t), seed);
+        const int rows = rows_of(t);
 #pragma unroll
         for (int i = 0; i < NI; ++i) {
-            long long e0;
-            const bool in = vec_of(tl, i, e0);
-            raw[i] = in ? load_raw<T, V>(x + e0) : make_uint4(0u, 0u, 0u, 0u);
-            if (MASKED) msk[i] = in ? mask_word(mask, e0) : 0u;
-        }
-    };
-    auto draw = [&](const Tile &tl) {
-#pragma unroll
-        for (int i = 0; i < NI; ++i) {
-            long long e0;
-            vec_of(tl, i, e0);
-            dithers_of<V>(e0, seed, u[i]);
+            if (row[i] >= rows) continue;
+            dithers_at<V>(z + off_z[i], u[i][0]);
+            dithers_at<V>(z + off_z[i] + row_z, u[i][1]);
         }
     };
     unsigned t = blockIdx.x;
-    Tile cur = tile_of(t);
-    if (PATH != kOdd) {
-        load(cur);
-        draw(cur);
-    }
+    const unsigned ntiles = p.ntiles;
+    Tile cur;
+    cur.b = t / (p.pt * p.ct);
+    cur.c = (t - cur.b * p.pt * p.ct) / p.pt;
+    cur.p = t - (cur.b * p.ct + cur.c) * p.pt;
+    load(cur);
+    draw(cur);
+    const StepSource from = step_ahead(step);
     chain_wait();
     chain_release();
-    const float delta = step_of<kThreads>(step, st);
+    const float delta = step_of<kThreads>(from, st);
+    const float inv = delta > 0.f ? __fdiv_rn(1.0f, delta) : 0.f;      // Delta = 0: every code 0
+    unsigned nnz = 0, sat = 0, nz2 = 0;
+    // rows on the way out: eight lanes to a row of 64 channels, thread 8 r + k at row r and r + 32
+    const int orow = threadIdx.x >> 3, och = (threadIdx.x & 7) * 8;
+    for (int buf = 0; t < ntiles; buf ^= 1) {
+        unsigned char *tl = tile[buf];
+        const Tile now = cur;
+        const long long base = base_of(now);
+        const int rows = rows_of(now), cleft = C - now.c * kTC;
+        t += gridDim.x;
+        cur.p += p.step_p;
+        if (cur.p >= p.pt) { cur.p -= p.pt; ++cur.c; }
+        cur.c += p.step_c;
+        if (cur.c >= p.ct) { cur.c -= p.ct; ++cur.b; }
+        cur.b += p.step_b;
+        unsigned w[NI][V], top = 0u;
+        const unsigned before = nz2;
+#pragma unroll
+        for (int i = 0; i < NI; ++i) {
+            if (row[i] >= rows) continue;
+            float a[V], b[V];
+            values_of(x, raw[i][0], a);
+            values_of(x, raw[i][1], b);
+            if (MASKED) { apply_mask(msk[i][0], a); apply_mask(msk[i][1], b); }
+            quick_codes2<V>(a, b, u[i][0], u[i][1], inv, w[i], top);
+            count_pairs<2 * V>(w[i], nz2);
+        }
+        if (t < ntiles) load(cur);
+        if (needs_care(top)) {                                     // rare: clip, count, NaN
+            nz2 = before;
+#pragma unroll
+            for (int i = 0; i < NI; ++i) {
+                if (row[i] >= rows) continue;
+                unsigned m[2][V];
+#pragma unroll
+                for (int h = 0; h < 2; ++h) {
+                    float v[V];
+                    unsigned long long d[V / 2];
+                    unsigned hc[V / 2];
+                    const long long e = base + in_off[i] + h * HW;
+                    const bool in = ch[i] + h < cleft;
+                    values_of(x, in ? load_raw<T, V>(x + e) : make_uint4(0u, 0u, 0u, 0u), v);
+                    if (MASKED) apply_mask(in ? mask_word(mask, e) : 0u, v);
+                    dithers_of<V>(e, seed, d);
+                    careful_codes<V>(v, d, inv, hc, m[h], sat);
+                }
+#pragma unroll
+                for (int j = 0; j < V; ++j)
+                    w[i][j] = __byte_perm(__float_as_uint(__uint_as_float(m[0][j]) - kMagic),
+                                          __float_as_uint(__uint_as_float(m[1][j]) - kMagic), 0x7632);
+                count_pairs<2 * V>(w[i], nz2);
+            }
+        }
+#pragma unroll
+        for (int i = 0; i < NI; ++i) {
+            if (row[i] >= rows) continue;
+            unsigned char *dst = tl + tile_off<V>(row[i], ch[i]);
+#pragma unroll
+            for (int j = 0; j < V; ++j) *reinterpret_cast<unsigned *>(dst + j * 128) = w[i][j];
+        }
+        if (t < ntiles) draw(cur);
+        __syncthreads();
+        if (och < cleft) {
+            unsigned short *dst = out + (static_cast<long long>(now.b) * p.G * HW + now.p * p.P + orow) * pitch + now.c * kTC + och;
+#pragma unroll
+            for (int i = 0; i < kTP / 32; ++i)
+                if (orow + 32 * i < rows)
+                    *reinterpret_cast<uint4 *>(dst + static_cast<long long>(32 * i) * pitch) =
+                        *reinterpret_cast<const uint4 *>(tl + tile_off<V>(orow + 32 * i, och));
+            // Second copy for the weight-gradient kernel of tiny planes: the images one below the other as tall images, a row of
+            // zeros after every image (what a tap that leaves an image must read). Any number of images per tall image.
+            if (STACK) {
+                const int tall = HW + p.plane_w;
+                unsigned short *to = out_stack + static_cast<long long>(now.b) * p.G * tall * C + now.c * kTC + och;
+#pragma unroll
+                for (int i = 0; i < kTP / 32; ++i) {
+                    const int r = orow + 32 * i, g = r / HW;
+                    if (r < rows)
+                        *reinterpret_cast<uint4 *>(to + static_cast<long long>(r + g * p.plane_w) * C) =
+                            *reinterpret_cast<const uint4 *>(tl + tile_off<V>(r, och));
+                }
+                const int images = rows / HW;
+                for (int r = orow; r < images * p.plane_w; r += 32) {
+                    const int g = r / p.plane_w;
+                    *reinterpret_cast<uint4 *>(to + static_cast<long long>((g + 1) * HW + r) * C) = make_uint4(0u, 0u, 0u, 0u);
+                }
+            }
+        }
+        // the other buffer is written next; this one again only after the next barrier
+        if (nz2 & 0x80008000u) { nnz += pairs_total(nz2); nz2 = 0; }
+    }
+    nnz += pairs_total(nz2);
+    if (p.count) publish_counts<kThreads>(nnz, delta > 0.f ? sat : 0u, st, nullptr);
+}
+
+template <typename T, int V>
+cudaError_t run_nhwc(dbp_ctx *ctx, const void *delta, int B, int C, int HW, unsigned long long seed, const StepSource &step,
+                     void *out, bool count, void *out_stack, int plane_w, const uint8_t *mask) {
+    NhwcP p{};
+    p.B = B; p.C = C; p.HW = HW; p.plane_w = plane_w; p.count = count ? 1 : 0;
+    p.ct = (C + kTC - 1) / kTC;
+    p.G = 1;
+    if (HW >= kTP) {
+        // as few tiles as hold the plane, of nearly the same size: what a short last tile leaves empty is spread over whole warps
+        p.pt = (HW + kTP - 1) / kTP;
+        p.P = ((HW + p.pt - 1) / p.pt + V - 1) / V * V;
+    } else {
+        // whole images, as many as fit and as leave two tiles per SM
+        p.pt = 1;
+        p.P = HW;
+        const long long spread = static_cast<long long>(B) * p.ct / (2 * ctx->sm_count);
+        p.G = kTP / HW;
+        if (p.G > spread) p.G = spread > 1 ? static_cast<int>(spread) : 1;
+    }
+    const long long ntiles = static_cast<long long>((B + p.G - 1) / p.G) * p.ct * p.pt;
+    p.ntiles = static_cast<int>(ntiles);
+    const long long cap = static_cast<long long>(ctx->sm_count) * kBlocksPerSM, blocks = ntiles < cap ? ntiles : cap;
+    p.step_p = static_cast<int>(blocks % p.pt);
+    p.step_c = static_cast<int>(blocks / p.pt % p.ct);
+    p.step_b = static_cast<int>(blocks / p.pt / p.ct);
+    auto go = [&](auto kern) {
+        return launch_chained(kern, dim3(static_cast<unsigned>(blocks)), dim3(kThreads), 0, ctx->stream,
+                              static_cast<const T *>(delta), p, seed, step, static_cast<unsigned short *>(out),
+                              static_cast<unsigned short *>(out_stack), ctx->state, static_cast<const unsigned char *>(mask));
+    };
+    if constexpr (sizeof(T) == 4) {
+        if (mask != nullptr) return out_stack ? go(quantize_nhwc_kernel<T, V, true, true>) : go(quantize_nhwc_kernel<T, V, false, true>);
+    }
+    return out_stack ? go(quantize_nhwc_kernel<T, V, true, false>) : go(quantize_nhwc_kernel<T, V, false, false>);
+}
+
+// Planes of any size and channels of any number: a channel's row of the tile is covered by the aligned vectors that touch it
+// (one more than a row holds), and what lies outside the row is dropped.
+template <typename T, bool MASKED>
+__global__ void __launch_bounds__(kThreads, kBlocksPerSM)
+quantize_nhwc_any_kernel(const T *__restrict__ x, int B, int C, int HW, unsigned long long seed, const StepSource step,
+                         unsigned short *__restrict__ out, DeviceState *__restrict__ st, int count,
+                         unsigned short *__restrict__ out_stack, int plane_w, const unsigned char *__restrict__ mask) {
+    __shared__ __align__(16) unsigned char tile[2][kTileBytes];
+    constexpr int V = Vec<T>::V;
+    const unsigned ct = (C + kTC - 1) / kTC, pt = (HW + kTP - 1) / kTP, per_img = ct * pt, ntiles = B * per_img;
+    const int pitch = (C + 7) & ~7;
+    const StepSource from = step_ahead(step);
+    chain_wait();
+    chain_release();
+    const float delta = step_of<kThreads>(from, st);
     const float inv = delta > 0.f ? __fdiv_rn(1.0f, delta) : 0.f;      // Delta = 0: every code 0
     unsigned nnz = 0, sat = 0, nz2 = 0;
     int buf = 0;
-    for (; t < ntiles; buf ^= 1) {
+    for (unsigned t = blockIdx.x; t < ntiles; t += gridDim.x, buf ^= 1) {
         unsigned char *tl = tile[buf];
-        const int b = cur.b, c0 = cur.c0, p0 = cur.p0;
-        const unsigned next = t + gridDim.x;
-        const Tile nxt = tile_of(next < ntiles ? next : t);
-        if (PATH != kOdd) {
-            float f[NI][V];
-#pragma unroll
-            for (int i = 0; i < NI; ++i) {
-                float v[V];
-                values_of(x, raw[i], v);
-                if (MASKED) apply_mask(msk[i], v);
-                decide<V>(v, u[i], inv, f[i], sat);
-            }
-            load(nxt);
-#pragma unroll
-            for (int i = 0; i < NI; ++i) {
-                long long e0;
-                if (vec_of(cur, i, e0)) {
-                    unsigned h[V / 2];
-                    pack_bf16<V>(f[i], h);
-                    count_pairs<V>(h, nz2);
-                    if (dense8 != nullptr) store_bytes<V>(dense8, e0, f[i]);
-                    if (PATH == kFlat) {
-                        const int v = threadIdx.x + kThreads * i;
-                        int c = (v * V) / HW, pp = v * V - c * HW;
-#pragma unroll
-                        for (int j = 0; j < V; ++j) {
-                            *reinterpret_cast<unsigned short *>(tl + tile_off(pp, c)) = static_cast<unsigned short>(h[j >> 1] >> (16 * (j & 1)));
-                            if (++pp == HW) { pp = 0; ++c; }
-                        }
-                    }
-                }
-            }
-            if (PATH == kPair) {
-                // (a vector that does not exist was decided as zeros: code 0, never stored beyond the tile)
-#pragma unroll
-                for (int i = 0; i < NI / 2; ++i) {
-                    const int it = threadIdx.x + kThreads * i, c = 2 * (it / VPR), pv = (it % VPR) * V;
-#pragma unroll
-                    for (int j = 0; j < V; ++j)
-                        *reinterpret_cast<unsigned *>(tl + tile_off(pv + j, c)) =
-                            __byte_perm(__float_as_uint(f[2 * i][j]), __float_as_uint(f[2 * i + 1][j]), 0x7632);
-                }
-            }
-            if (next < ntiles) draw(nxt);
-        } else {
+        const int b = t / per_img, rem = t - b * per_img, c0 = (rem / pt) * kTC, p0 = (rem - rem / pt * pt) * kTP;
+        {
             constexpr int VO = kTP / V + 1;                        // aligned vectors that may touch a row of the tile
             const int len = HW - p0 < kTP ? HW - p0 : kTP, nch = C - c0 < kTC ? C - c0 : kTC;
             const long long total = static_cast<long long>(B) * C * HW;
@@ -350,6 +529,7 @@ quantize_nhwc_kernel(const T *__restrict__ x, int B, int C, int HW, unsigned lon
                 const int pp = static_cast<int>(e0 - row0);        // position of the vector's first element in the row
                 if (pp >= len) continue;
                 float v[V], f[V];
+                unsigned long long u[V / 2];
                 if (e0 + V <= total) {
                     values_of(x, load_raw<T, V>(x + e0), v);
                     if (MASKED) apply_mask(mask_word(mask, e0), v);
@@ -361,14 +541,13 @@ quantize_nhwc_kernel(const T *__restrict__ x, int B, int C, int HW, unsigned lon
                 // what lies outside the row belongs to other rows: it is not counted here, clipped or not
 #pragma unroll
                 for (int j = 0; j < V; ++j) v[j] = pp + j >= 0 && pp + j < len ? v[j] : 0.f;
-                dithers_of<V>(e0, seed, u[0]);
-                decide<V>(v, u[0], inv, f, sat);
+                dithers_of<V>(e0, seed, u);
+                decide<V>(v, u, inv, f, sat);
 #pragma unroll
                 for (int j = 0; j < V; ++j)
                     if (pp + j >= 0 && pp + j < len) {
                         nnz += f[j] != 0.f;
-                        *reinterpret_cast<unsigned short *>(tl + tile_off(pp + j, c)) = static_cast<unsigned short>(__float_as_uint(f[j]) >> 16);
-                        if (dense8 != nullptr) dense8[e0 + j] = static_cast<int8_t>(static_cast<int>(f[j]));
+                        *reinterpret_cast<unsigned short *>(tl + tile_off<8>(pp + j, c)) = static_cast<unsigned short>(__float_as_uint(f[j]) >> 16);
                     }
             }
         }
@@ -380,123 +559,221 @@ quantize_nhwc_kernel(const T *__restrict__ x, int B, int C, int HW, unsigned lon
             const int pp = v >> 3, ch = v & 7;
             if (p0 + pp < HW && c0 + ch * 8 < C)
                 *reinterpret_cast<uint4 *>(out + (static_cast<long long>(b) * HW + p0 + pp) * pitch + c0 + ch * 8) =
-                    *reinterpret_cast<const uint4 *>(tl + tile_off(pp, ch * 8));
-            // Second copy for the weight-gradient kernel of tiny planes: the images one below the other as tall
-            // images, a row of zeros after every image (what a tap that leaves an image must read).
-            if (STACK && pp < HW + plane_w && c0 + ch * 8 < C) {
-                const uint4 val = pp < HW ? *reinterpret_cast<const uint4 *>(tl + tile_off(pp, ch * 8)) : make_uint4(0u, 0u, 0u, 0u);
-                const long long row = static_cast<long long>(b) * (HW + plane_w) + pp;   // any number of images per tall image
+                    *reinterpret_cast<const uint4 *>(tl + tile_off<8>(pp, ch * 8));
+            if (out_stack != nullptr && pp < HW + plane_w && c0 + ch * 8 < C) {     // (planes of less than a tile: see above)
+                const uint4 val = pp < HW ? *reinterpret_cast<const uint4 *>(tl + tile_off<8>(pp, ch * 8)) : make_uint4(0u, 0u, 0u, 0u);
+                const long long row = static_cast<long long>(b) * (HW + plane_w) + pp;
                 *reinterpret_cast<uint4 *>(out_stack + row * C + c0 + ch * 8) = val;
             }
         }
         // the other buffer is written next; this one again only after the next barrier
         if (nz2 & 0x80008000u) { nnz += pairs_total(nz2); nz2 = 0; }
-        t = next;
-        cur = nxt;
     }
     nnz += pairs_total(nz2);
     if (count) publish_counts<kThreads>(nnz, delta > 0.f ? sat : 0u, st, nullptr);
-}
-
-template <typename T, int V, int PATH>
-cudaError_t run_nhwc(dbp_ctx *ctx, const void *delta, int B, int C, int HW, unsigned long long seed, const StepSource &step,
-                     void *out, int8_t *dense8, bool count, void *out_stack, int plane_w, const uint8_t *mask) {
-    const long long ntiles = static_cast<long long>(B) * ((C + kTC - 1) / kTC) * ((HW + kTP - 1) / kTP);
-    const long long cap = static_cast<long long>(ctx->sm_count) * kBlocksPerSM, blocks = ntiles < cap ? ntiles : cap;
-    auto go = [&](auto kern) {
-        return launch_chained(kern, dim3(static_cast<unsigned>(blocks)), dim3(kThreads), 0, ctx->stream,
-                              static_cast<const T *>(delta), B, C, HW, seed, step, static_cast<unsigned short *>(out), dense8,
-                              ctx->state, count ? 1 : 0, static_cast<unsigned short *>(out_stack), plane_w,
-                              static_cast<const unsigned char *>(mask));
-    };
-    if constexpr (sizeof(T) == 4) {
-        if (mask != nullptr) {
-            if constexpr (PATH == kFlat) { if (out_stack) return go(quantize_nhwc_kernel<T, V, PATH, true, true>); }
-            return go(quantize_nhwc_kernel<T, V, PATH, false, true>);
-        }
-    }
-    if constexpr (PATH == kFlat) { if (out_stack) return go(quantize_nhwc_kernel<T, V, PATH, true, false>); }
-    return go(quantize_nhwc_kernel<T, V, PATH, false, false>);
 }
 
 // ---------------------------------------------------------------- bf16 planes of odd sizes
 // Planes whose size is no multiple of 4 (7 x 7, 9 x 9, ...) written at a pitch that is a multiple of 8: the codes
 // of eight consecutive elements then belong to unaligned places of one or two planes. A block takes a run of
-// whole planes (a multiple of eight of them, so that the run starts on a 16-byte boundary and on an even
-// element), quantizes it with whole-vector loads as everywhere, places the codes in shared memory at their pitch,
-// and the run leaves as one contiguous copy (the padding of a plane is never read by anybody).
-constexpr int kOddMaxSmem = 12 * 1024;            // bytes of the staged run (planes x pitch bf16)
+// whole planes (as many as a vector has elements, or a multiple, so that the run starts on a 16-byte boundary and on an even
+// element), quantizes it with whole-vector loads as everywhere and keeps the codes as they come, in whole words of shared
+// memory; the output's 16-byte words are put together from them on the way out (five words each, shifted by half a word where
+// the piece starts on an odd element), and leave as one contiguous copy (the padding of a plane is never read by anybody).
+// Placing the codes one by one at their pitch instead took 52 instructions an element: 6.4 M elements of 7 x 7 planes 17.5 us,
+// 12 so.
+// NHWC: the run is a multiple of eight channels of one image, and leaves position-major: eight channels of a position are
+// eight 16-bit reads, a plane apart (in different banks for odd planes).
+constexpr int kOddElems = 6272;                   // most elements of a run
 
-template <typename T, bool MASKED>
-__global__ void __launch_bounds__(kThreads)
+struct NhwcOut {
+    int C;                        // channels: a multiple of 8, and of a run's
+    unsigned short *stack;        // the copy with rows of zeros after every image (may be null)
+    int plane_w;                  // how many
+};
+
+template <typename T, bool MASKED, bool NHWC>
+__global__ void __launch_bounds__(kThreads, kBlocksPerSM)
 quantize_planes_odd_kernel(const T *__restrict__ x, long long nplanes, int hw, int pitch, int planes_per_run,
                            unsigned long long seed, const StepSource step, unsigned short *__restrict__ out,
-                           int8_t *__restrict__ dense8, DeviceState *__restrict__ st, int count,
-                           const unsigned char *__restrict__ mask) {
+                           DeviceState *__restrict__ st, int count, const unsigned char *__restrict__ mask, const NhwcOut nhwc) {
     constexpr int V = Vec<T>::V;
-    constexpr int NP = 2;                                           // vectors of the first run loaded and drawn ahead
-    __shared__ __align__(16) unsigned short run_s[kOddMaxSmem / 2];
+    constexpr int NV = kPerThread / V;                              // vectors in hand per thread
+    constexpr int kBetween = kThreads * V;
+    constexpr unsigned long long kBetweenZ = kBetween / 2 * kGamma;
+    __shared__ __align__(16) unsigned run_s[kOddElems / 2 + 8];
     const long long nruns = (nplanes + planes_per_run - 1) / planes_per_run;
-    uint4 raw[NP];
-    unsigned long long u[NP][V / 2];
-    {
-        const long long e_base = blockIdx.x * static_cast<long long>(planes_per_run) * hw, n = nplanes * hw;
+    uint4 raw[NV];
+    unsigned msk[MASKED ? NV : 1];
+    unsigned long long u[NV][V / 2];
+    // the run's elements from e on that this thread holds: those of its vectors that lie before the run's end
+    auto load = [&](long long e, int left) {
 #pragma unroll
-        for (int i = 0; i < NP; ++i) {
-            const long long e0 = e_base + (threadIdx.x + kThreads * i) * V;
-            raw[i] = e0 < n ? Vec<T>::raw(x + e0) : make_uint4(0u, 0u, 0u, 0u);
+        for (int k = 0; k < NV; ++k) {
+            raw[k] = k * kBetween < left ? Vec<T>::raw(x + e + k * kBetween) : make_uint4(0u, 0u, 0u, 0u);
+            if (MASKED) msk[k] = k * kBetween < left ? mask_word(mask, e + k * kBetween) : 0u;
         }
+    };
+    auto draw = [&](unsigned long long zz) {
 #pragma unroll
-        for (int i = 0; i < NP; ++i) dithers_of<V>(e_base + (threadIdx.x + kThreads * i) * V, seed, u[i]);
-    }
+        for (int k = 0; k < NV; ++k) dithers_at<V>(zz + k * kBetweenZ, u[k]);
+    };
+    const long long run_e = static_cast<long long>(planes_per_run) * hw, total = nplanes * hw;
+    long long r = blockIdx.x, base = r * run_e;
+    auto run_len = [&](long long b) { return static_cast<int>(total - b < run_e ? total - b : run_e); };       // a multiple of 8
+    int len = run_len(base), done = threadIdx.x * V;                // elements of the run; the thread's place in it
+    const unsigned long long tid_z = counter_of(done, seed);
+    unsigned long long z = tid_z + static_cast<unsigned long long>(base / 2) * kGamma;
+    load(base + done, len - done);
+    draw(z);
+    keep_here(u);
+    const StepSource from = step_ahead(step);
     chain_wait();
     chain_release();
-    const float delta = step_of<kThreads>(step, st);
+    const float delta = step_of<kThreads>(from, st);
     const float inv = delta > 0.f ? __fdiv_rn(1.0f, delta) : 0.f;      // Delta = 0: every code 0
     unsigned sat = 0, nz2 = 0, nnz = 0;
-    for (long long r = blockIdx.x; r < nruns; r += gridDim.x) {
-        const long long pl0 = r * planes_per_run;
-        const int np = static_cast<int>(nplanes - pl0 < planes_per_run ? nplanes - pl0 : planes_per_run);   // a multiple of 8
-        const long long e_base = pl0 * hw;
-        const int nvec = np * hw / V;
-        auto place = [&](int v, const uint4 &q, const unsigned long long (&d)[V / 2]) {
-            float a[V], f[V];
-            unsigned h[V / 2];
-            Vec<T>::values(q, a);
-            if (MASKED) apply_mask(mask_word(mask, e_base + static_cast<long long>(v) * V), a);
-            decide<V>(a, d, inv, f, sat);
-            pack_bf16<V>(f, h);
-            count_pairs<V>(h, nz2);
-            if (dense8 != nullptr) store_bytes<V>(dense8, e_base + static_cast<long long>(v) * V, f);
-            int pl = (v * V) / hw, pp = v * V - pl * hw;
+    // 16-byte words of the output: of a plane, or of a position
+    const int words = NHWC ? planes_per_run / 8 : pitch / 8, q_plane = kThreads / words, r_plane = kThreads - q_plane * words;
+    const int first_plane = threadIdx.x / words, first_word = threadIdx.x - first_plane * words;
+    while (r < nruns) {
+        const long long here = base;
+        const int now = len;
+        // the run in rounds of 16 elements per thread; after its last one the next run's first is on its way
+        while (true) {
+            unsigned h[NV][V / 2], m[NV][V], top = 0u;
+            const unsigned before = nz2;
+            const int at = done, left = now - at;
+            const unsigned long long zz = z;
+            if (left > 0) {
 #pragma unroll
-            for (int j = 0; j < V; ++j) {
-                run_s[pl * pitch + pp] = static_cast<unsigned short>(h[j >> 1] >> (16 * (j & 1)));
-                if (++pp == hw) { pp = 0; ++pl; }
+                for (int k = 0; k < NV; ++k) {
+                    float v[V];
+                    Vec<T>::values(raw[k], v);
+                    if (MASKED) apply_mask(msk[k], v);
+                    quick_codes<V>(v, u[k], inv, h[k], m[k], top);
+                    count_pairs<V>(h[k], nz2);
+                }
             }
-        };
-        int v = threadIdx.x;
-        if (r == blockIdx.x) {
+            done += NV * kBetween;
+            z += NV * kBetweenZ;
+            const bool last = done - static_cast<int>(threadIdx.x) * V >= now;       // uniform
+            if (last) {
+                r += gridDim.x;
+                base += run_e * gridDim.x;
+                len = r < nruns ? run_len(base) : 0;
+                done = threadIdx.x * V;
+                z = tid_z + static_cast<unsigned long long>(base / 2) * kGamma;
+            }
+            load(base + done, len - done);
+            if (needs_care(top)) {                                  // rare: clip, count, NaN
+                nz2 = before;
+#pragma unroll 1
+                for (int k = 0; k < NV; ++k) {
+                    if (k * kBetween >= left) break;
+                    float v[V];
+                    unsigned long long d[V / 2];
+                    unsigned hc[V / 2], mc[V];
+                    Vec<T>::values(Vec<T>::raw(x + here + at + k * kBetween), v);
+                    if (MASKED) apply_mask(mask_word(mask, here + at + k * kBetween), v);
+                    dithers_at<V>(zz + k * kBetweenZ, d);
+                    careful_codes<V>(v, d, inv, hc, mc, sat);
+                    count_pairs<V>(hc, nz2);
+                    store_vec<V>(reinterpret_cast<unsigned short *>(run_s) + at + k * kBetween, hc);
+                }
+            } else {
 #pragma unroll
-            for (int i = 0; i < NP; ++i, v += kThreads)
-                if (v < nvec) place(v, raw[i], u[i]);
-        }
-        for (; v < nvec; v += kThreads) {
-            const long long e0 = e_base + static_cast<long long>(v) * V;
-            const uint4 q = Vec<T>::raw(x + e0);
-            unsigned long long d[V / 2];
-            dithers_of<V>(e0, seed, d);
-            place(v, q, d);
+                for (int k = 0; k < NV; ++k)
+                    if (k * kBetween < left) store_vec<V>(reinterpret_cast<unsigned short *>(run_s) + at + k * kBetween, h[k]);
+            }
+            if (last) break;
+            if (done < now) draw(z);
         }
         __syncthreads();
-        const int n16 = np * pitch / 8;
-        uint4 *dst = reinterpret_cast<uint4 *>(out + pl0 * pitch);
-        for (int i = threadIdx.x; i < n16; i += kThreads) dst[i] = reinterpret_cast<const uint4 *>(run_s)[i];
-        __syncthreads();
+        if (NHWC) {
+            const long long plane = here / hw, b = plane / nhwc.C;
+            const int c0 = static_cast<int>(plane - b * nhwc.C), tall = hw + (nhwc.stack ? nhwc.plane_w : 0);
+            unsigned short *dst = out + b * hw * nhwc.C + c0, *to = nhwc.stack + b * tall * nhwc.C + c0;
+            const unsigned short *src = reinterpret_cast<const unsigned short *>(run_s);
+            int pp = first_plane, w = first_word;
+            for (int i = threadIdx.x; i < tall * words; i += kThreads) {
+                uint4 v = make_uint4(0u, 0u, 0u, 0u);
+                if (pp < hw) {
+                    unsigned k[8];
+#pragma unroll
+                    for (int j = 0; j < 8; ++j) k[j] = src[(8 * w + j) * hw + pp];
+                    v = make_uint4(__byte_perm(k[0], k[1], 0x5410), __byte_perm(k[2], k[3], 0x5410), __byte_perm(k[4], k[5], 0x5410),
+                                   __byte_perm(k[6], k[7], 0x5410));
+                    *reinterpret_cast<uint4 *>(dst + static_cast<long long>(pp) * nhwc.C + 8 * w) = v;
+                }
+                if (nhwc.stack != nullptr) *reinterpret_cast<uint4 *>(to + static_cast<long long>(pp) * nhwc.C + 8 * w) = v;
+                pp += q_plane;
+                w += r_plane;
+                if (w >= words) { w -= words; ++pp; }
+            }
+        } else {
+            const int np = now / hw, n16 = np * words;
+            uint4 *dst = reinterpret_cast<uint4 *>(out + here / hw * pitch);
+            int pl = first_plane, w = first_word;
+            for (int i = threadIdx.x; i < n16; i += kThreads) {
+                const int s = pl * hw + 8 * w, sh = (s & 1) * 16;
+                const unsigned *src = run_s + (s >> 1);
+                const unsigned v0 = src[0], v1 = src[1], v2 = src[2], v3 = src[3], v4 = src[4];
+                dst[i] = make_uint4(__funnelshift_r(v0, v1, sh), __funnelshift_r(v1, v2, sh), __funnelshift_r(v2, v3, sh),
+                                    __funnelshift_r(v3, v4, sh));
+                pl += q_plane;
+                w += r_plane;
+                if (w >= words) { w -= words; ++pl; }
+            }
+        }
         if (nz2 & 0x80008000u) { nnz += pairs_total(nz2); nz2 = 0; }
+        if (r >= nruns) break;
+        draw(z);
+        __syncthreads();                                            // the buffer is written again
     }
     nnz += pairs_total(nz2);
     if (count) publish_counts<kThreads>(nnz, delta > 0.f ? sat : 0u, st, nullptr);
+}
+template <typename T, bool NHWC>
+int run_planes_odd(dbp_ctx *ctx, const void *delta, long long nplanes, int hw, int pitch, int per_run, unsigned long long seed,
+                   const StepSource &step, void *out, bool count, const uint8_t *mask, const NhwcOut &nhwc) {
+    const long long nruns = (nplanes + per_run - 1) / per_run, cap = static_cast<long long>(ctx->sm_count) * kBlocksPerSM;
+    auto go = [&](auto kern) {
+        return cuda_ok(launch_chained(kern, dim3(static_cast<unsigned>(nruns < cap ? nruns : cap)), dim3(kThreads), 0, ctx->stream,
+                                      static_cast<const T *>(delta), nplanes, hw, pitch, per_run, seed, step,
+                                      static_cast<unsigned short *>(out), ctx->state, count ? 1 : 0,
+                                      static_cast<const unsigned char *>(mask), nhwc));
+    };
+    if constexpr (sizeof(T) == 4) {
+        if (mask != nullptr) return go(quantize_planes_odd_kernel<T, true, NHWC>);
+    }
+    return go(quantize_planes_odd_kernel<T, false, NHWC>);
+}
+
+// Channels in a run of the position-major form: as many as fit of the numbers that divide C, at most 64 (a row of the output), but
+// fewer where the runs would not cover the SMs twice. 0: none does.
+int odd_channels_per_run(long long B, int C, int hw, int sms) {
+    int best = 0;
+    for (int n = 64; n >= 8; n -= 8) {
+        if (C % n != 0 || static_cast<long long>(n) * hw > kOddElems) continue;
+        best = n;
+        if (B * (C / n) >= 2ll * sms) break;
+    }
+    return best;
+}
+
+// Planes in a run: as many as fit, in units of a vector's elements, of those numbers the one that leaves the fewest of a round's places empty (a
+// round is 4096 elements), but not so many that the blocks would not cover the SMs twice.
+int odd_planes_per_run(long long nplanes, int hw, int unit, int sms) {
+    int best = 0;
+    double best_eff = 0.0;
+    for (int np = unit; static_cast<long long>(np) * hw <= kOddElems; np += unit) {
+        if (best && (nplanes + np - 1) / np < 2 * sms) break;
+        const int e = np * hw, rounds = (e + kThreads * kPerThread - 1) / (kThreads * kPerThread);
+        const double eff = static_cast<double>(e) / rounds;
+        if (eff >= best_eff) { best = np; best_eff = eff; }
+    }
+    return best;
 }
 
 }  // namespace
@@ -510,59 +787,83 @@ int launch_quantize_dense(dbp_ctx *ctx, const void *delta, int dtype, long long 
     const int v = dtype == DBP_F32 ? 4 : 8;
     const float *xf = static_cast<const float *>(delta);
     const __nv_bfloat16 *xb = static_cast<const __nv_bfloat16 *>(delta);
+    if ((dense != nullptr) == (planes != nullptr)) return DBP_EINVAL;          // one form a call
     // odd plane sizes at a padded pitch: whole runs of planes through shared memory
-    if (planes != nullptr && hw > 0 && pitch != hw && (hw & 3) != 0 && numel % hw == 0 && (numel / hw) % 8 == 0 &&
-        8 * pitch * 2 <= kOddMaxSmem && hw < (1 << 20)) {
+    if (planes != nullptr && hw > 0 && pitch != hw && (hw & 3) != 0 && numel % hw == 0 && (numel / hw) % v == 0 && v * hw <= kOddElems &&
+        pitch % 8 == 0 && pitch - hw < 8) {
         const long long nplanes = numel / hw;
-        int per_run = static_cast<int>(kOddMaxSmem / 2 / pitch / 8 * 8);          // planes per run: a multiple of 8
-        const long long want = (4096 + 8 * hw - 1) / (8 * hw) * 8;               // about 4096 elements a run
-        if (per_run > want) per_run = static_cast<int>(want);
-        const long long nruns = (nplanes + per_run - 1) / per_run, cap = static_cast<long long>(ctx->sm_count) * 8;
-        auto go = [&](auto kern, auto x) {
-            return cuda_ok(launch_chained(kern, dim3(static_cast<unsigned>(nruns < cap ? nruns : cap)), dim3(kThreads), 0, ctx->stream, x,
-                                          nplanes, static_cast<int>(hw), static_cast<int>(pitch), per_run, seed, step, planes, dense,
-                                          ctx->state, count ? 1 : 0, m));
-        };
-        return dtype != DBP_F32 ? go(quantize_planes_odd_kernel<__nv_bfloat16, false>, xb)
-               : m              ? go(quantize_planes_odd_kernel<float, true>, xf)
-                                : go(quantize_planes_odd_kernel<float, false>, xf);
+        const int per_run = odd_planes_per_run(nplanes, static_cast<int>(hw), v, ctx->sm_count);
+        const int h = static_cast<int>(hw), pt = static_cast<int>(pitch);
+        return dtype != DBP_F32 ? run_planes_odd<__nv_bfloat16, false>(ctx, delta, nplanes, h, pt, per_run, seed, step, planes, count, mask, {})
+                                : run_planes_odd<float, false>(ctx, delta, nplanes, h, pt, per_run, seed, step, planes, count, mask, {});
     }
-    long long blocks = (numel / v + 2 * kThreads - 1) / (2 * kThreads);
+    constexpr int kTile = kThreads * kPerThread;
+    long long blocks = (numel / v * v + kTile - 1) / kTile;
     if (blocks < 1) blocks = 1;
     const long long cap = static_cast<long long>(ctx->sm_count) * kBlocksPerSM;
     if (blocks > cap) blocks = cap;
-    const CodeSinks out{dense, planes, hw > 0 ? hw : 1, pitch > 0 ? pitch : 1, count ? 1 : 0};
+    CodeSinks out{};
+    out.dense8 = dense;
+    out.planes16 = planes;
+    out.hw = hw > 0 ? hw : 1;
+    out.pitch = pitch > 0 ? pitch : 1;
+    out.count = count ? 1 : 0;
+    const long long between = kThreads * v, next = blocks * kTile - (kTile - between);
+    out.rest1 = static_cast<int>(between % out.hw);
+    out.rest2 = static_cast<int>(next % out.hw);
+    out.dist1 = between / out.hw * out.pitch + out.rest1;
+    out.dist2 = next / out.hw * out.pitch + out.rest2;
+    const int sink = dense ? kBytes : out.pitch == out.hw ? kSame : (out.hw & 7) == 4 && out.pitch == out.hw + 4 && out.hw < (1 << 30) ? kPad4 : kAny;
     auto go = [&](auto kern, auto x) {
         return cuda_ok(launch_chained(kern, dim3(static_cast<unsigned>(blocks)), dim3(kThreads), 0, ctx->stream, x, numel, seed, step, out,
                                       ctx->state, m));
     };
-    return dtype != DBP_F32 ? go(quantize_dense_kernel<__nv_bfloat16, false>, xb)
-           : m              ? go(quantize_dense_kernel<float, true>, xf)
-                            : go(quantize_dense_kernel<float, false>, xf);
+    auto pick = [&](auto s) {
+        constexpr int S = decltype(s)::value;
+        return dtype != DBP_F32 ? go(quantize_dense_kernel<__nv_bfloat16, false, S>, xb)
+               : m              ? go(quantize_dense_kernel<float, true, S>, xf)
+                                : go(quantize_dense_kernel<float, false, S>, xf);
+    };
+    switch (sink) {
+        case kBytes: return pick(std::integral_constant<int, kBytes>());
+        case kSame: return pick(std::integral_constant<int, kSame>());
+        case kPad4: return pick(std::integral_constant<int, kPad4>());
+        default: return pick(std::integral_constant<int, kAny>());
+    }
 }
 
-// delta_z [B][C][HW] -> bf16 codes [B][HW][C rounded up to a multiple of 8] and, when dense8 is not null, int8 codes
-// in delta_z's order
+// delta_z [B][C][HW] -> bf16 codes [B][HW][C rounded up to a multiple of 8]
 int launch_quantize_nhwc(dbp_ctx *ctx, const void *delta, int dtype, long long B, long long C, long long HW,
-                         unsigned long long seed, const StepSource &step, void *codes_nhwc, int8_t *dense8, bool count,
+                         unsigned long long seed, const StepSource &step, void *codes_nhwc, bool count,
                          void *codes_stack, int plane_w, const uint8_t *mask) {
-    if (B * C * HW >= (1ll << 40) || HW >= (1ll << 30)) return DBP_EUNSUPPORTED;
+    if (B * C * HW >= (1ll << 40) || HW >= (1ll << 25)) return DBP_EUNSUPPORTED;
     if (B * ((C + kTC - 1) / kTC) * ((HW + kTP - 1) / kTP) >= (1ll << 31)) return DBP_EUNSUPPORTED;
     if (mask != nullptr && dtype != DBP_F32) return DBP_EUNSUPPORTED;
-    // the stacked copy is written by the path for planes smaller than a tile; the rows of image b start at
+    // the stacked copy is written by the paths for planes smaller than a tile; the rows of image b start at
     // b (HW + W) however many images make up a tall image: the stacking only adds the zero rows
     if (codes_stack != nullptr && (HW >= kTP || C % 8 != 0 || plane_w <= 0 || HW + plane_w > kTP)) return DBP_EINVAL;
     const int b = static_cast<int>(B), c = static_cast<int>(C), hw = static_cast<int>(HW);
-    const bool flat = HW < kTP && C % 8 == 0;
-    auto run = [&](auto kern) { return kern(ctx, delta, b, c, hw, seed, step, codes_nhwc, dense8, count, codes_stack, plane_w, mask); };
-    if (dtype == DBP_F32)
-        return cuda_ok(flat          ? run(run_nhwc<float, 4, kFlat>)
-                       : hw % 4 == 0 ? run(run_nhwc<float, 4, kPair>)
-                                     : run(run_nhwc<float, 4, kOdd>));
-    return cuda_ok(flat          ? run(run_nhwc<__nv_bfloat16, 8, kFlat>)
-                   : hw % 8 == 0 ? run(run_nhwc<__nv_bfloat16, 8, kPair>)
-                   : hw % 4 == 0 ? run(run_nhwc<__nv_bfloat16, 4, kPair>)
-                                 : run(run_nhwc<__nv_bfloat16, 8, kOdd>));
+    if (hw % 4 == 0) {
+        auto run = [&](auto kern) { return cuda_ok(kern(ctx, delta, b, c, hw, seed, step, codes_nhwc, count, codes_stack, plane_w, mask)); };
+        return dtype == DBP_F32 ? run(run_nhwc<float, 4>) : hw % 8 == 0 ? run(run_nhwc<__nv_bfloat16, 8>) : run(run_nhwc<__nv_bfloat16, 4>);
+    }
+    if (c % 8 == 0) {
+        if (const int n = odd_channels_per_run(B, c, hw, ctx->sm_count)) {
+            const NhwcOut nh{c, static_cast<unsigned short *>(codes_stack), plane_w};
+            return dtype != DBP_F32 ? run_planes_odd<__nv_bfloat16, true>(ctx, delta, B * C, hw, 8, n, seed, step, codes_nhwc, count, mask, nh)
+                                    : run_planes_odd<float, true>(ctx, delta, B * C, hw, 8, n, seed, step, codes_nhwc, count, mask, nh);
+        }
+    }
+    const long long ntiles = B * ((C + kTC - 1) / kTC) * ((HW + kTP - 1) / kTP), cap = static_cast<long long>(ctx->sm_count) * kBlocksPerSM;
+    auto go = [&](auto kern, auto x) {
+        return cuda_ok(launch_chained(kern, dim3(static_cast<unsigned>(ntiles < cap ? ntiles : cap)), dim3(kThreads), 0, ctx->stream, x, b, c,
+                                      hw, seed, step, static_cast<unsigned short *>(codes_nhwc), ctx->state, count ? 1 : 0,
+                                      static_cast<unsigned short *>(codes_stack), plane_w, static_cast<const unsigned char *>(mask)));
+    };
+    const float *xf = static_cast<const float *>(delta);
+    return dtype != DBP_F32 ? go(quantize_nhwc_any_kernel<__nv_bfloat16, false>, static_cast<const __nv_bfloat16 *>(delta))
+           : mask           ? go(quantize_nhwc_any_kernel<float, true>, xf)
+                            : go(quantize_nhwc_any_kernel<float, false>, xf);
 }
 
 }  // namespace dbp

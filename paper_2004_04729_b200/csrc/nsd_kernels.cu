@@ -297,9 +297,10 @@ quantize_kernel(const T *__restrict__ x, long long n, unsigned long long seed, c
         for (int i = 0; i < NV; ++i) raw[i] = e0 + (i + 1) * V <= n ? Vec<T>::raw(x + e0 + i * V) : make_uint4(0u, 0u, 0u, 0u);
     };
     load(seg < nseg ? seg : 0);
+    const StepSource from = step_ahead(step);
     chain_wait();
     chain_release();
-    const float delta = step_of<kThreads>(step, st);
+    const float delta = step_of<kThreads>(from, st);
     const float inv = delta > 0.f ? __fdiv_rn(1.0f, delta) : 0.f;      // Delta = 0: every code 0
     unsigned nnz = 0, sat = 0;
     for (; seg < nseg; seg += nwarps) {
