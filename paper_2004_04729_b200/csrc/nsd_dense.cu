@@ -287,7 +287,11 @@ struct NhwcP {
     int B, C, HW;
     int P, G;                     // positions of an image, images of a tile
     int pt, ct, ntiles;           // tiles along the positions, along the channels, in all (positions first, images last)
-    int step_p, step_c, step_b;   // from one of a block's tiles to its next
+    // From one of a block's tiles to its next: tiles along the positions, the channels and the images, and how much further
+    // everything is then that grows from tile to tile: the place in delta_z (elements), in the output, in the stacked copy, and
+    // the dither's counter. wrap_p: after that where the positions pass their end, wrap_c where the channels do.
+    int step_p, step_c, step_b;
+    struct Far { long long in, out, tall; unsigned long long z; } far, wrap_p, wrap_c;
     int plane_w;                  // stacked copy: rows of zeros after every image
     int count;
 };
@@ -304,62 +308,72 @@ quantize_nhwc_kernel(const T *__restrict__ x, const NhwcP p, unsigned long long 
 
     // this thread's pairs of vectors in any tile: four channel pairs run fastest, then the positions, eights of channels, images
     int in_off[NI], row[NI], ch[NI];                               // first element; first row of the tile; first channel
-    unsigned long long off_z[NI];
 #pragma unroll
     for (int i = 0; i < NI; ++i) {
         const int s = threadIdx.x + kThreads * i, vpr = p.P / V, q = s >> 2, r = q / vpr, pv = (q - r * vpr) * V, g = r >> 3;
         ch[i] = 8 * (r & 7) + 2 * (s & 3);
         row[i] = g < p.G ? g * p.P + pv : kTP;                     // kTP: in no tile
         in_off[i] = (g * C + ch[i]) * HW + pv;
-        off_z[i] = static_cast<unsigned long long>((static_cast<long long>(g) * C + ch[i]) * HW + pv) / 2 * kGamma;
     }
-    struct Tile { int b, c, p; };                                  // group of images, 64 channels, positions
-    auto base_of = [&](const Tile &t) { return (static_cast<long long>(t.b) * p.G * C + t.c * kTC) * HW + t.p * p.P; };
-    auto rows_of = [&](const Tile &t) {                            // rows of the tile that exist
+    auto off_z = [&](int i) { return static_cast<unsigned long long>(static_cast<unsigned>(in_off[i]) >> 1) * kGamma; };
+    // the tile: numbers along the positions, the channels and the images; places of its first element; rows and channels it has
+    struct Tile { int p, c, b; long long e; unsigned long long z; unsigned short *out, *tall; int rows, cleft; };
+    auto measure = [&](Tile &t) {
         const int n = p.G == 1 ? HW - t.p * p.P : (p.B - t.b * p.G) * HW;
-        return n < p.G * p.P ? n : p.G * p.P;
+        t.rows = n < p.G * p.P ? n : p.G * p.P;
+        t.cleft = C - t.c * kTC;
     };
+    auto go_in = [&](Tile &t, const NhwcP::Far &f) { t.e += f.in; t.z += f.z; };
+    auto go_out = [&](Tile &t, const NhwcP::Far &f) { t.out += f.out; if (STACK) t.tall += f.tall; };
     uint4 raw[NI][2];
     unsigned msk[MASKED ? NI : 1][2];
     unsigned long long u[NI][2][V / 2];
     auto load = [&](const Tile &t) {
-        const long long base = base_of(t);
-        const int rows = rows_of(t), cleft = C - t.c * kTC;
-        if (cleft >= kTC && rows == kTP) {                         // a whole tile
+        if (t.cleft >= kTC && t.rows == kTP) {                     // a whole tile
 #pragma unroll
             for (int i = 0; i < NI; ++i)
 #pragma unroll
                 for (int h = 0; h < 2; ++h) {
-                    raw[i][h] = load_raw<T, V>(x + base + in_off[i] + h * HW);
-                    if (MASKED) msk[i][h] = mask_word(mask, base + in_off[i] + h * HW);
+                    raw[i][h] = load_raw<T, V>(x + t.e + in_off[i] + h * HW);
+                    if (MASKED) msk[i][h] = mask_word(mask, t.e + in_off[i] + h * HW);
                 }
         } else {
 #pragma unroll
             for (int i = 0; i < NI; ++i)
 #pragma unroll
                 for (int h = 0; h < 2; ++h) {
-                    const bool in = row[i] < rows && ch[i] + h < cleft;
-                    raw[i][h] = in ? load_raw<T, V>(x + base + in_off[i] + h * HW) : make_uint4(0u, 0u, 0u, 0u);
-                    if (MASKED) msk[i][h] = in ? mask_word(mask, base + in_off[i] + h * HW) : 0u;
+                    const bool in = row[i] < t.rows && ch[i] + h < t.cleft;
+                    raw[i][h] = in ? load_raw<T, V>(x + t.e + in_off[i] + h * HW) : make_uint4(0u, 0u, 0u, 0u);
+                    if (MASKED) msk[i][h] = in ? mask_word(mask, t.e + in_off[i] + h * HW) : 0u;
                 }
         }
     };
     auto draw = [&](const Tile &t) {
-        const unsigned long long z = counter_of(base_of(t), seed);
-        const int rows = rows_of(t);
 #pragma unroll
         for (int i = 0; i < NI; ++i) {
-            if (row[i] >= rows) continue;
-            dithers_at<V>(z + off_z[i], u[i][0]);
-            dithers_at<V>(z + off_z[i] + row_z, u[i][1]);
+            if (row[i] >= t.rows) continue;
+            dithers_at<V>(t.z + off_z(i), u[i][0]);
+            dithers_at<V>(t.z + off_z(i) + row_z, u[i][1]);
         }
     };
     unsigned t = blockIdx.x;
     const unsigned ntiles = p.ntiles;
-    Tile cur;
-    cur.b = t / (p.pt * p.ct);
-    cur.c = (t - cur.b * p.pt * p.ct) / p.pt;
-    cur.p = t - (cur.b * p.ct + cur.c) * p.pt;
+    // rows on the way out: eight lanes to a row of 64 channels, thread 8 r + k at row r and r + 32
+    const int orow = threadIdx.x >> 3, och = (threadIdx.x & 7) * 8;
+    auto tile_at = [&](unsigned n) {
+        Tile r;
+        r.b = n / (p.pt * p.ct);
+        r.c = (n - r.b * p.pt * p.ct) / p.pt;
+        r.p = n - (r.b * p.ct + r.c) * p.pt;
+        const long long b0 = static_cast<long long>(r.b) * p.G;
+        r.e = (b0 * C + r.c * kTC) * HW + r.p * p.P;
+        r.z = counter_of(r.e, seed);
+        r.out = out + (b0 * HW + r.p * p.P + orow) * pitch + r.c * kTC + och;
+        r.tall = out_stack + b0 * (HW + p.plane_w) * C + r.c * kTC + och;
+        measure(r);
+        return r;
+    };
+    Tile cur = tile_at(t);
     load(cur);
     draw(cur);
     const StepSource from = step_ahead(step);
@@ -368,19 +382,19 @@ quantize_nhwc_kernel(const T *__restrict__ x, const NhwcP p, unsigned long long 
     const float delta = step_of<kThreads>(from, st);
     const float inv = delta > 0.f ? __fdiv_rn(1.0f, delta) : 0.f;      // Delta = 0: every code 0
     unsigned nnz = 0, sat = 0, nz2 = 0;
-    // rows on the way out: eight lanes to a row of 64 channels, thread 8 r + k at row r and r + 32
-    const int orow = threadIdx.x >> 3, och = (threadIdx.x & 7) * 8;
     for (int buf = 0; t < ntiles; buf ^= 1) {
         unsigned char *tl = tile[buf];
-        const Tile now = cur;
-        const long long base = base_of(now);
-        const int rows = rows_of(now), cleft = C - now.c * kTC;
+        const int rows = cur.rows, cleft = cur.cleft;
         t += gridDim.x;
         cur.p += p.step_p;
-        if (cur.p >= p.pt) { cur.p -= p.pt; ++cur.c; }
         cur.c += p.step_c;
-        if (cur.c >= p.ct) { cur.c -= p.ct; ++cur.b; }
         cur.b += p.step_b;
+        const bool past_p = cur.p >= p.pt;
+        go_in(cur, p.far);
+        if (past_p) { cur.p -= p.pt; ++cur.c; go_in(cur, p.wrap_p); }
+        const bool past_c = cur.c >= p.ct;
+        if (past_c) { cur.c -= p.ct; ++cur.b; go_in(cur, p.wrap_c); }
+        measure(cur);
         unsigned w[NI][V], top = 0u;
         const unsigned before = nz2;
 #pragma unroll
@@ -396,6 +410,7 @@ quantize_nhwc_kernel(const T *__restrict__ x, const NhwcP p, unsigned long long 
         if (t < ntiles) load(cur);
         if (needs_care(top)) {                                     // rare: clip, count, NaN
             nz2 = before;
+            const Tile now = tile_at(t - gridDim.x);
 #pragma unroll
             for (int i = 0; i < NI; ++i) {
                 if (row[i] >= rows) continue;
@@ -405,11 +420,10 @@ quantize_nhwc_kernel(const T *__restrict__ x, const NhwcP p, unsigned long long 
                     float v[V];
                     unsigned long long d[V / 2];
                     unsigned hc[V / 2];
-                    const long long e = base + in_off[i] + h * HW;
                     const bool in = ch[i] + h < cleft;
-                    values_of(x, in ? load_raw<T, V>(x + e) : make_uint4(0u, 0u, 0u, 0u), v);
-                    if (MASKED) apply_mask(in ? mask_word(mask, e) : 0u, v);
-                    dithers_of<V>(e, seed, d);
+                    values_of(x, in ? load_raw<T, V>(x + now.e + in_off[i] + h * HW) : make_uint4(0u, 0u, 0u, 0u), v);
+                    if (MASKED) apply_mask(in ? mask_word(mask, now.e + in_off[i] + h * HW) : 0u, v);
+                    dithers_at<V>(now.z + off_z(i) + h * row_z, d);
                     careful_codes<V>(v, d, inv, hc, m[h], sat);
                 }
 #pragma unroll
@@ -429,31 +443,31 @@ quantize_nhwc_kernel(const T *__restrict__ x, const NhwcP p, unsigned long long 
         if (t < ntiles) draw(cur);
         __syncthreads();
         if (och < cleft) {
-            unsigned short *dst = out + (static_cast<long long>(now.b) * p.G * HW + now.p * p.P + orow) * pitch + now.c * kTC + och;
 #pragma unroll
             for (int i = 0; i < kTP / 32; ++i)
                 if (orow + 32 * i < rows)
-                    *reinterpret_cast<uint4 *>(dst + static_cast<long long>(32 * i) * pitch) =
+                    *reinterpret_cast<uint4 *>(cur.out + static_cast<long long>(32 * i) * pitch) =
                         *reinterpret_cast<const uint4 *>(tl + tile_off<V>(orow + 32 * i, och));
             // Second copy for the weight-gradient kernel of tiny planes: the images one below the other as tall images, a row of
             // zeros after every image (what a tap that leaves an image must read). Any number of images per tall image.
             if (STACK) {
-                const int tall = HW + p.plane_w;
-                unsigned short *to = out_stack + static_cast<long long>(now.b) * p.G * tall * C + now.c * kTC + och;
 #pragma unroll
                 for (int i = 0; i < kTP / 32; ++i) {
                     const int r = orow + 32 * i, g = r / HW;
                     if (r < rows)
-                        *reinterpret_cast<uint4 *>(to + static_cast<long long>(r + g * p.plane_w) * C) =
+                        *reinterpret_cast<uint4 *>(cur.tall + static_cast<long long>(r + g * p.plane_w) * C) =
                             *reinterpret_cast<const uint4 *>(tl + tile_off<V>(r, och));
                 }
                 const int images = rows / HW;
                 for (int r = orow; r < images * p.plane_w; r += 32) {
                     const int g = r / p.plane_w;
-                    *reinterpret_cast<uint4 *>(to + static_cast<long long>((g + 1) * HW + r) * C) = make_uint4(0u, 0u, 0u, 0u);
+                    *reinterpret_cast<uint4 *>(cur.tall + static_cast<long long>((g + 1) * HW + r) * C) = make_uint4(0u, 0u, 0u, 0u);
                 }
             }
         }
+        go_out(cur, p.far);
+        if (past_p) go_out(cur, p.wrap_p);
+        if (past_c) go_out(cur, p.wrap_c);
         // the other buffer is written next; this one again only after the next barrier
         if (nz2 & 0x80008000u) { nnz += pairs_total(nz2); nz2 = 0; }
     }
@@ -486,6 +500,15 @@ cudaError_t run_nhwc(dbp_ctx *ctx, const void *delta, int B, int C, int HW, unsi
     p.step_p = static_cast<int>(blocks % p.pt);
     p.step_c = static_cast<int>(blocks / p.pt % p.ct);
     p.step_b = static_cast<int>(blocks / p.pt / p.ct);
+    // (positions, channels, groups of images) -> distances
+    auto far = [&](long long np, long long nc, long long nb) {
+        const long long pitch = (C + 7) & ~7, e = np * p.P + nc * kTC * HW + nb * p.G * C * HW;
+        return NhwcP::Far{e, np * p.P * pitch + nc * kTC + nb * p.G * HW * pitch, nc * kTC + nb * p.G * (HW + plane_w) * static_cast<long long>(C),
+                          static_cast<unsigned long long>(e / 2) * kGamma};
+    };
+    p.far = far(p.step_p, p.step_c, p.step_b);
+    p.wrap_p = far(-p.pt, 1, 0);
+    p.wrap_c = far(0, -p.ct, 1);
     auto go = [&](auto kern) {
         return launch_chained(kern, dim3(static_cast<unsigned>(blocks)), dim3(kThreads), 0, ctx->stream,
                               static_cast<const T *>(delta), p, seed, step, static_cast<unsigned short *>(out),
