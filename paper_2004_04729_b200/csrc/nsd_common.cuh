@@ -58,23 +58,38 @@ __device__ __forceinline__ float max3_abs(float a, float b, float c) {
 // every second clock on another (wide ones every fourth), additions every clock. The draw takes 16.8 clocks an element (14 of
 // the first pipe), the whole decision 22, whether two or eight warps per scheduler run. Multiplications in place of shifts, or
 // mixed-precision additions in place of the conversion from bf16, are no faster.
+// SHORT: for a kernel that is a chain of latencies and not of instructions, a product is the sum of two independent ones: one
+// instruction more, one less behind another (a small linear layer's call 9.43 against 9.51 us; the thin 1x1 call 73.9 against 71.9).
+template <bool SHORT>
 __device__ __forceinline__ void mul_low64(unsigned &lo, unsigned &hi, unsigned clo, unsigned chi) {
-    asm("{\n\t.reg .u64 p;\n\t.reg .u32 a, b, h;\n\t"
-        "mul.wide.u32 p, %0, %2;\n\t"
-        "mov.b64 {a, b}, p;\n\t"
-        "mad.lo.u32 h, %0, %3, b;\n\t"
-        "mad.lo.u32 %1, %1, %2, h;\n\t"
-        "mov.b32 %0, a;\n\t}"
-        : "+r"(lo), "+r"(hi) : "r"(clo), "r"(chi));
+    if (SHORT) {
+        asm("{\n\t.reg .u64 p;\n\t.reg .u32 a, b, h;\n\t"
+            "mul.lo.u32 h, %0, %3;\n\t"
+            "mad.lo.u32 h, %1, %2, h;\n\t"
+            "mul.wide.u32 p, %0, %2;\n\t"
+            "mov.b64 {a, b}, p;\n\t"
+            "add.u32 %1, b, h;\n\t"
+            "mov.b32 %0, a;\n\t}"
+            : "+r"(lo), "+r"(hi) : "r"(clo), "r"(chi));
+    } else {
+        asm("{\n\t.reg .u64 p;\n\t.reg .u32 a, b, h;\n\t"
+            "mul.wide.u32 p, %0, %2;\n\t"
+            "mov.b64 {a, b}, p;\n\t"
+            "mad.lo.u32 h, %0, %3, b;\n\t"
+            "mad.lo.u32 %1, %1, %2, h;\n\t"
+            "mov.b32 %0, a;\n\t}"
+            : "+r"(lo), "+r"(hi) : "r"(clo), "r"(chi));
+    }
 }
+template <bool SHORT = false>
 __device__ __forceinline__ unsigned long long dither2(unsigned long long z) {
     unsigned lo = static_cast<unsigned>(z), hi = static_cast<unsigned>(z >> 32);
     lo ^= __funnelshift_r(lo, hi, 30);
     hi ^= hi >> 30;
-    mul_low64(lo, hi, 0x1CE4E5B9u, 0xBF58476Du);
+    mul_low64<SHORT>(lo, hi, 0x1CE4E5B9u, 0xBF58476Du);
     lo ^= __funnelshift_r(lo, hi, 27);
     hi ^= hi >> 27;
-    mul_low64(lo, hi, 0x133111EBu, 0x94D049BBu);
+    mul_low64<SHORT>(lo, hi, 0x133111EBu, 0x94D049BBu);
     lo ^= hi + hi;
     return add2(pack2(__uint_as_float(__funnelshift_r(lo, 0x7fu, 9)), __uint_as_float(__funnelshift_r(hi, 0x7fu, 9))),
                 pack2(kDitherShift, kDitherShift));
@@ -83,18 +98,18 @@ __device__ __forceinline__ unsigned long long counter_of(long long e, unsigned l
     return seed + (static_cast<unsigned long long>(e >> 1) + 1ull) * kGamma;
 }
 // dithers of V elements whose first pair has the counter z, pairs packed
-template <int V>
+template <int V, bool SHORT = false>
 __device__ __forceinline__ void dithers_at(unsigned long long z, unsigned long long (&u)[V / 2]) {
 #pragma unroll
     for (int j = 0; j < V / 2; ++j) {
-        u[j] = dither2(z);
+        u[j] = dither2<SHORT>(z);
         z += kGamma;
     }
 }
 // and of V elements whose first has the even index e0
-template <int V>
+template <int V, bool SHORT = false>
 __device__ __forceinline__ void dithers_of(long long e0, unsigned long long seed, unsigned long long (&u)[V / 2]) {
-    dithers_at<V>(counter_of(e0, seed), u);
+    dithers_at<V, SHORT>(counter_of(e0, seed), u);
 }
 // Dithers drawn ahead of a wait stay there: without this the compiler moves the arithmetic behind the wait (about 1 us of each
 // of the quantizers).

@@ -98,7 +98,7 @@ small_linear_quantize_kernel(const SmallLinP p) {
     const int v0 = blockIdx.x * kThreads + tid;
     unsigned long long u[NV][2];
 #pragma unroll
-    for (int i = 0; i < NV; ++i) dithers_of<4>(4ll * (v0 + i * step), p.seed, u[i]);
+    for (int i = 0; i < NV; ++i) dithers_of<4, true>(4ll * (v0 + i * step), p.seed, u[i]);
     if (tid == 0) {
         tc::mbar_init(&bar_s, 1);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");

@@ -70,3 +70,20 @@ def test_forms(ctx, B, Ci, Co, H, W, k, dtype, mask):
     g = out["dX"].double().cpu().numpy().reshape(ref["dX"].shape)
     rounded = 2.0 ** -8 * np.abs(ref["dX"]) if dtype == "bf16" else 0.0
     assert np.all(np.abs(g - ref["dX"]) <= rounded + TOL * ref["S_dX"] + 1e-30)
+
+
+@pytest.mark.parametrize("dtype", ["f32", "bf16"])
+@pytest.mark.parametrize("n", [1, 31, 1023, 1024, 1025, 1024 * 37 + 511, 1024 * 8 * 1200])
+def test_sparse_form(ctx, n, dtype):
+    """Whole segments without a code out of range, with some, and the last, partial one."""
+    import paper_2004_04729_b200 as dbp
+    tdt = torch.bfloat16 if dtype == "bf16" else torch.float32
+    x = np.random.default_rng(n).laplace(0.0, 1e-3, n).astype(np.float32)
+    for i, a in enumerate({0, n // 2, n - 1, max(0, n - 1025)}):
+        x[a] = (-1.0) ** i * (1.0 if i % 2 else 0.0635)
+    d = torch.from_numpy(x).to(tdt).cuda()
+    D = np.float32(5e-4)
+    codes, nnz, sat = oracle.nsd_codes(d.float().cpu().numpy(), 5, D)
+    q = dbp.nsd_quantize(ctx, d, 5, 0.0, delta_in=torch.tensor([float(D)], device="cuda"))
+    assert q.nnz.item() == nnz and ctx.last_device_status()[1] == sat
+    assert np.array_equal(dbp.nsd_decode_dense(ctx, q).cpu().numpy().reshape(-1), codes)
