@@ -123,8 +123,18 @@ statistics_kernel(const T *__restrict__ x, long long n, double *__restrict__ par
                   const unsigned char *__restrict__ mask, const SideJobs jobs) {
     constexpr int EPT = Vec<T>::V;
     const long long nvec = n / EPT;
+    // whole tiles of kUnroll x kThreads 128-bit vectors, a block at a time: kUnroll loads in flight
+    // per thread, consecutive threads on consecutive vectors
+    constexpr int kUnroll = 8;
+    const long long tile = static_cast<long long>(kUnroll) * kThreads, ntile = nvec / tile;
+    uint4 raw[kUnroll];
+    auto load = [&](long long t) {
+#pragma unroll
+        for (int u = 0; u < kUnroll; ++u) raw[u] = load_stream(x + (t * tile + threadIdx.x + static_cast<long long>(u) * kThreads) * EPT);
+    };
     chain_wait();
     chain_release();
+    if (blockIdx.x < ntile) load(blockIdx.x);       // on its way during the side jobs
     // side job for the layer's weight-gradient kernel, which adds its partial sums into dW: clear it
     {
         const long long first = static_cast<long long>(blockIdx.x) * kThreads + threadIdx.x, step = static_cast<long long>(gridDim.x) * kThreads;
@@ -149,45 +159,73 @@ statistics_kernel(const T *__restrict__ x, long long n, double *__restrict__ par
         const long long per_tap = w_cout * w_pitch;     // taps outermost: the copy engine takes several taps in one box
         for (long long co = blockIdx.x; co < w_cout; co += gridDim.x) {
             unsigned short *dst = w_dst + co * w_pitch;
-            // a thread takes one channel and all nine taps: nine independent loads, then stores that run along ci
-            for (int ci = threadIdx.x; ci < w_cin; ci += kThreads) {
-                int ph = 0;
-                long long base = (co * w_cin + ci) * 9;
-                if (w_phase_cin > 0) {
-                    ph = ci / w_phase_cin;
-                    base = (co * w_phase_cin + (ci - ph * w_phase_cin)) * 9;
-                }
-                int k[9];                                                  // source tap, or -1 for a zero weight
+            // A thread takes two neighbouring channels and all nine taps of them, all loads first (pairs of weights where the rows
+            // allow it), then one word per tap and piece, along ci. (Of an odd number of channels the last one's word reaches into
+            // the row's padding.)
+            const bool paired = w_phase_cin == 0 && (w_cin & 1) == 0;
+            for (int c0 = 2 * threadIdx.x; c0 < w_cin; c0 += 2 * kThreads) {
+                unsigned w[18];                                        // the bits of the weights: channel c0's, then channel c0 + 1's
+                unsigned dead = 0u;                                    // bit h * 9 + t: zero by construction
+                if (paired) {
+                    const long long base = (co * w_cin + c0) * 9;      // even
+                    if (w_f32) {
+                        const uint2 *src = reinterpret_cast<const uint2 *>(static_cast<const float *>(w_src) + base);
 #pragma unroll
-                for (int t = 0; t < 9; ++t) {
-                    const int ty = t / 3, tx = t % 3;
-                    k[t] = t;
-                    if (w_phase_cin > 0) {
-                        const int ky = (ph & 2) ? (ty == 0 ? 0 : (ty == 1 ? 2 : -1)) : (ty == 1 ? 1 : -1);
-                        const int kx = (ph & 1) ? (tx == 0 ? 0 : (tx == 1 ? 2 : -1)) : (tx == 1 ? 1 : -1);
-                        k[t] = (ky >= 0 && kx >= 0) ? ky * 3 + kx : -1;
-                    }
-                }
-                if (w_f32) {
-                    float w[9];
+                        for (int i = 0; i < 9; ++i) {
+                            const uint2 v = __ldg(src + i);
+                            w[2 * i] = v.x;
+                            w[2 * i + 1] = v.y;
+                        }
+                    } else {
+                        const unsigned *src = reinterpret_cast<const unsigned *>(static_cast<const unsigned short *>(w_src) + base);
 #pragma unroll
-                    for (int t = 0; t < 9; ++t) w[t] = k[t] >= 0 ? __ldg(static_cast<const float *>(w_src) + base + k[t]) : 0.f;
-#pragma unroll
-                    for (int t = 0; t < 9; ++t) {
-                        if (k[t] < 0 && jobs.skip_dead) continue;
-                        const __nv_bfloat16 hi = __float2bfloat16_rn(w[t]);
-                        const __nv_bfloat16 lo = __float2bfloat16_rn(w[t] - __bfloat162float(hi));
-                        dst[t * per_tap + ci] = *reinterpret_cast<const unsigned short *>(&hi);
-                        dst[(9 + t) * per_tap + ci] = *reinterpret_cast<const unsigned short *>(&lo);
+                        for (int i = 0; i < 9; ++i) {
+                            const unsigned v = __ldg(src + i);
+                            w[2 * i] = v & 0xffffu;
+                            w[2 * i + 1] = v >> 16;
+                        }
                     }
                 } else {
-                    unsigned short w[9];
 #pragma unroll
-                    for (int t = 0; t < 9; ++t)
-                        w[t] = k[t] >= 0 ? __ldg(static_cast<const unsigned short *>(w_src) + base + k[t]) : static_cast<unsigned short>(0);
+                    for (int h = 0; h < 2; ++h) {
+                        const int ci = c0 + h;
+                        int ph = 0;
+                        long long base = (co * w_cin + ci) * 9;
+                        if (w_phase_cin > 0) {
+                            ph = ci / w_phase_cin;
+                            base = (co * w_phase_cin + (ci - ph * w_phase_cin)) * 9;
+                        }
 #pragma unroll
-                    for (int t = 0; t < 9; ++t)
-                        if (k[t] >= 0 || !jobs.skip_dead) dst[t * per_tap + ci] = w[t];
+                        for (int t = 0; t < 9; ++t) {
+                            const int ty = t / 3, tx = t % 3;
+                            int k = t;                                 // source tap
+                            bool live = true;
+                            if (w_phase_cin > 0) {
+                                const int ky = (ph & 2) ? (ty == 0 ? 0 : (ty == 1 ? 2 : -1)) : (ty == 1 ? 1 : -1);
+                                const int kx = (ph & 1) ? (tx == 0 ? 0 : (tx == 1 ? 2 : -1)) : (tx == 1 ? 1 : -1);
+                                live = ky >= 0 && kx >= 0;
+                                k = ky * 3 + kx;
+                            }
+                            if (!live) dead |= 1u << (9 * h + t);
+                            w[9 * h + t] = 0u;
+                            if (live && ci < w_cin)
+                                w[9 * h + t] = w_f32 ? __float_as_uint(__ldg(static_cast<const float *>(w_src) + base + k))
+                                                     : static_cast<unsigned>(__ldg(static_cast<const unsigned short *>(w_src) + base + k));
+                        }
+                    }
+                }
+#pragma unroll
+                for (int t = 0; t < 9; ++t) {
+                    if (jobs.skip_dead && (dead >> t & 1u)) continue;   // (both channels are of one phase then)
+                    if (w_f32) {
+                        const __nv_bfloat162 hi = __floats2bfloat162_rn(__uint_as_float(w[t]), __uint_as_float(w[9 + t]));
+                        const float2 hf = __bfloat1622float2(hi);
+                        const __nv_bfloat162 lo = __floats2bfloat162_rn(__uint_as_float(w[t]) - hf.x, __uint_as_float(w[9 + t]) - hf.y);
+                        *reinterpret_cast<unsigned *>(dst + t * per_tap + c0) = *reinterpret_cast<const unsigned *>(&hi);
+                        *reinterpret_cast<unsigned *>(dst + (9 + t) * per_tap + c0) = *reinterpret_cast<const unsigned *>(&lo);
+                    } else {
+                        *reinterpret_cast<unsigned *>(dst + t * per_tap + c0) = w[t] | w[9 + t] << 16;
+                    }
                 }
             }
         }
@@ -199,15 +237,11 @@ statistics_kernel(const T *__restrict__ x, long long n, double *__restrict__ par
     }
     const float pivot = (!MASKED || __ldg(mask)) ? Vec<T>::one(x) : 0.f;
     const long long stride = static_cast<long long>(gridDim.x) * kThreads;
-    // whole tiles of kUnroll x kThreads 128-bit vectors, a block at a time: kUnroll loads in flight
-    // per thread, consecutive threads on consecutive vectors
-    constexpr int kUnroll = 8;
-    const long long tile = static_cast<long long>(kUnroll) * kThreads, ntile = nvec / tile;
     for (long long t = blockIdx.x; t < ntile; t += gridDim.x) {
-        const T *p = x + (t * tile + threadIdx.x) * EPT;
+        if (t != blockIdx.x) load(t);
         float v[kUnroll][EPT];
 #pragma unroll
-        for (int u = 0; u < kUnroll; ++u) Vec<T>::values(load_stream(p + static_cast<long long>(u) * kThreads * EPT), v[u]);
+        for (int u = 0; u < kUnroll; ++u) Vec<T>::values(raw[u], v[u]);
 #pragma unroll
         for (int u = 0; u < kUnroll; ++u) mask4<MASKED>(mask, (t * tile + threadIdx.x + static_cast<long long>(u) * kThreads) * EPT, v[u]);
 #pragma unroll
