@@ -180,6 +180,7 @@ int launch_small_linear(dbp_ctx *ctx, const float *delta, const float *X, const 
 // ---- linear_tc.cu: both products of a linear layer in one launch; codes as bf16 [B][linear_pitch(N)]
 struct LinearPlan {
     int TN = 0;                       // columns per tile
+    int MA = 1;                       // accumulators (of 128 rows) per tile
     long long dw_split = 1, dw_per_split = 0;   // > 1: dW is added up from parts and must have been cleared
 };
 bool linear_tc_supported(long long B, long long N, long long K);

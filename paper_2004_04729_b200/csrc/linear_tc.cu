@@ -8,14 +8,18 @@
 // so every operand tile is one or a few tiled copies of row-major memory, and one kernel runs the tiles of both
 // products: their CTAs fill the GPU together, and neither product waits for the other's last wave.
 //
-// A CTA is persistent over output tiles of 128 rows x TN columns: warp 0 issues the copies, warp 1 the MMAs into
-// one of two accumulators in tensor memory, warps 2-9 drain the other one (scale by Delta, convert, stage as
-// 128-byte swizzled rows, one tiled store per 32-row block; rows whose pitch is no multiple of 16 bytes leave
-// through plain stores). Weight-gradient tiles may be split along the reduction: the parts then add into a
+// A CTA is persistent over output tiles of 128 MA rows x TN columns: warp 0 issues the copies, warp 1 the MMAs into
+// one of two accumulators in tensor memory (MA = 2: both are one tile's), warps 2-9 drain the other one (scale by Delta,
+// convert, stage as 128-byte swizzled rows, one tiled store per 32-row block; rows whose pitch is no multiple of 16 bytes
+// leave through plain stores). Weight-gradient tiles may be split along the reduction: the parts then add into a
 // cleared dW through the copy engine.
-// Large layers are bound by the tensor pipe (a step of 128 x 256 x 64 is 512 clocks of it against 48 KB of
-// copies), small ones by the chain of reduction steps of one tile.
+// Large layers are bound by what the copies bring to an SM, about 60 bytes a clock: a step of 128 x 256 x 64 is 512 clocks of
+// the tensor pipe and 48 KB (840 clocks measured), one of 256 x 256 x 64 1024 clocks and 64 KB. Small ones are bound by the
+// chain of reduction steps of the CTA with the most of them (linear_plan), and a step by its hand-overs, so the issuing loops
+// carry no divisions. 1024 -> 4096 bf16, batch 4096: the call 95.0 -> 84.7 us; 2048 -> 1000 fp32, batch 256: 31.5 -> 24.9.
 #include "tc_common.cuh"
+
+#include <utility>
 
 namespace dbp {
 
@@ -39,13 +43,14 @@ struct LinProduct {
     int a_kmajor;                 // A is [M][reduction] (dX) instead of [reduction][M] (dW)
     int ks, pieces, steps;        // 64-deep steps per piece; steps of all pieces
     int per_split, nsplit;
-    int mt;
+    int mt;                       // tiles of 128 MA rows
     int tiles;                    // mt * column tiles * nsplit
 };
 
 struct LinArgs {
     LinProduct pr[2];             // the product with the longer tiles first
-    int nprod, tiles, TN;
+    int nprod, tiles, TN, MA;     // MA accumulators of 128 rows per tile: with two, both are one tile's
+    int lead;                     // tiles of the second product for a CTA that has one tile less of the first: see tile_at
     int stages, stage_bytes;      // as many stages as the ring holds: a narrow tile's steps are bound by the copies' latency
     const float *delta_p;
     int *err_flag;
@@ -65,6 +70,7 @@ __device__ __forceinline__ void tma_store_2d(const CUtensorMap *map, int c0, int
                  ::"l"(map), "r"(c0), "r"(c1), "r"(smem_u32(src)) : "memory");
 }
 
+template <int MA>
 __global__ void __launch_bounds__(kThreadsL, 1)
 linear_products_kernel(const __grid_constant__ LinMaps maps, const __grid_constant__ LinArgs p) {
     extern __shared__ __align__(1024) unsigned char smem_raw[];
@@ -97,50 +103,70 @@ linear_products_kernel(const __grid_constant__ LinMaps maps, const __grid_consta
     chain_wait();        // from here on the kernel reads what earlier kernels wrote
     chain_release();
 
-    // tile t -> product, first row and column, range of reduction steps
-    struct Tile { int i, m0, n0, k0, k1; };
-    auto tile_of = [&](int t) {
-        Tile r;
+    // This CTA's tile number j: product, first row and column, range of reduction steps. The longer tiles (the first product's)
+    // are dealt in turn; a CTA that got one less of them takes `lead` of the shorter ones, which last as long, before these go
+    // around, from the last CTA down.
+    const int G = static_cast<int>(gridDim.x), cta = static_cast<int>(blockIdx.x);
+    const int n0_tiles = p.pr[0].tiles, n1_tiles = p.tiles - n0_tiles, more = n0_tiles % G, mine = (n0_tiles - cta + G - 1) / G;
+    struct Tile { int i, m0, n0, k0, k1, na; };
+    auto tile_at = [&](int j, Tile &r) {
+        int t = cta + j * G;
+        if (t >= n0_tiles) {
+            j -= mine;
+            if (cta >= more && j < p.lead) t = cta - more + j * (G - more);
+            else t = p.lead * (G - more) + G - 1 - cta + (j - (cta >= more ? p.lead : 0)) * G;
+            if (t >= n1_tiles) return false;
+            t += n0_tiles;
+        }
         r.i = t < p.pr[0].tiles ? 0 : 1;
         const LinProduct &q = p.pr[r.i];
         if (r.i) t -= p.pr[0].tiles;
         const int s = t % q.nsplit;
         t /= q.nsplit;
-        r.m0 = (t % q.mt) * 128;
+        r.m0 = (t % q.mt) * 128 * MA;
         r.n0 = (t / q.mt) * p.TN;
         r.k0 = s * q.per_split;
         r.k1 = r.k0 + q.per_split < q.steps ? r.k0 + q.per_split : q.steps;
-        return r;
+        r.na = MA == 2 && q.M - r.m0 > 128 ? 2 : 1;                  // accumulators that hold rows
+        return true;
     };
+    Tile tl;
 
     if (warp == 0) {
         int s = 0;
         unsigned parity = 1;                     // a fresh barrier passes a wait on the previous phase
         bool ok = true;
-        for (int t = blockIdx.x; t < p.tiles && ok; t += gridDim.x) {
-            const Tile tl = tile_of(t);
+        for (int it = 0; ok && tile_at(it, tl); ++it) {
             const LinProduct &q = p.pr[tl.i];
             const int left = (q.cols - tl.n0 + 63) >> 6;
             const int nb = left < p.TN / 64 ? left : p.TN / 64;      // 64-column panels that hold columns
-            const unsigned tx = static_cast<unsigned>(kABytesL + nb * kPanelL);
+            const unsigned tx = static_cast<unsigned>(tl.na * kABytesL + nb * kPanelL);
+            const CUtensorMap *const map_a = &maps.a[tl.i], *const map_b = &maps.b[tl.i];
+            // the low pieces first: the accumulator is still small when they are added
+            int piece = q.pieces - 1 - tl.k0 / q.ks, r0 = tl.k0 % q.ks * 64;
             for (int k = tl.k0; k < tl.k1; ++k) {
                 ok = __all_sync(0xffffffffu, mbar_wait(&pipe.empty[s], parity, p.err_flag));
                 if (!ok) break;
                 if (elect_one()) {
                     unsigned char *st = smem + s * stage_bytes;
-                    // the low pieces first: the accumulator is still small when they are added
-                    const int kp = k / q.ks, piece = q.pieces - 1 - kp, r0 = (k - kp * q.ks) * 64;
                     mbar_expect_tx(&pipe.full[s], tx);
-                    if (q.a_kmajor) {
-                        tma_load_2d(st, &maps.a[tl.i], r0, tl.m0, &pipe.full[s]);
-                    } else {
-                        tma_load_2d(st, &maps.a[tl.i], tl.m0, r0, &pipe.full[s]);
-                        tma_load_2d(st + kPanelL, &maps.a[tl.i], tl.m0 + 64, r0, &pipe.full[s]);
+#pragma unroll
+                    for (int a = 0; a < MA; ++a) {
+                        if (a >= tl.na) break;
+                        const int m = tl.m0 + 128 * a;
+                        if (q.a_kmajor) {
+                            tma_load_2d(st + a * kABytesL, map_a, r0, m, &pipe.full[s]);
+                        } else {
+                            tma_load_2d(st + a * kABytesL, map_a, m, r0, &pipe.full[s]);
+                            tma_load_2d(st + a * kABytesL + kPanelL, map_a, m + 64, r0, &pipe.full[s]);
+                        }
                     }
-                    st += kABytesL;
-                    for (int i = 0; i < nb; ++i)
-                        tma_load_3d(st + i * kPanelL, &maps.b[tl.i], tl.n0 + 64 * i, r0, piece, &pipe.full[s]);
+                    st += MA * kABytesL;
+#pragma unroll
+                    for (int i = 0; i < kMaxNL / 64; ++i)
+                        if (i < nb) tma_load_3d(st + i * kPanelL, map_b, tl.n0 + 64 * i, r0, piece, &pipe.full[s]);
                 }
+                if ((r0 += 64) == 64 * q.ks) { r0 = 0; --piece; }
                 if (++s == S) { s = 0; parity ^= 1u; }
             }
         }
@@ -149,38 +175,41 @@ linear_products_kernel(const __grid_constant__ LinMaps maps, const __grid_consta
         int s = 0;
         unsigned parity = 0;
         bool ok = true;
-        int it = 0;
-        for (int t = blockIdx.x; t < p.tiles && ok; t += gridDim.x, ++it) {
-            const Tile tl = tile_of(t);
+        for (int it = 0; ok && tile_at(it, tl); ++it) {
             const bool kmaj = p.pr[tl.i].a_kmajor != 0;
-            const int slot = it & 1;
-            ok = __all_sync(0xffffffffu, mbar_wait(&pipe.acc_empty[slot], ((static_cast<unsigned>(it) >> 1) & 1u) ^ 1u, p.err_flag));
-            if (!ok) break;
-            tc_fence_after();
+            // this tile's accumulator (the first of two) and how often it has been used before
+            const int slot = MA == 2 ? 0 : it & 1;
+            const unsigned uses = static_cast<unsigned>(MA == 2 ? it : it >> 1);
             const unsigned tmem_d = tmem_base + slot * kMaxNL;
-            for (int k = tl.k0; k < tl.k1; ++k) {
+            for (int k = tl.k0; k < tl.k1 && ok; ++k) {
                 ok = __all_sync(0xffffffffu, mbar_wait(&pipe.full[s], parity, p.err_flag));
                 if (!ok) break;
-                tc_fence_after();
                 const unsigned a_addr = smem_u32(smem + s * stage_bytes);
-                const unsigned long long bd = make_desc(a_addr + kABytesL, kPanelL, 1024);
-                if (elect_one()) {
-                    if (kmaj) {
-                        const unsigned long long ad = make_desc(a_addr, 16, 1024);
+                const unsigned long long bd = make_desc(a_addr + MA * kABytesL, kPanelL, 1024);
 #pragma unroll
-                        for (int kk = 0; kk < 4; ++kk)       // 16 along the rows of A = 32 bytes
-                            mma_bf16(tmem_d, ad + 2 * kk, bd + 128 * kk, idesc_k, (k > tl.k0 || kk > 0) ? 1u : 0u);
-                    } else {
-                        const unsigned long long ad = make_desc(a_addr, kPanelL, 1024);
+                for (int a = 0; a < MA; ++a) {
+                    if (k == tl.k0) ok = ok && __all_sync(0xffffffffu, mbar_wait(&pipe.acc_empty[slot + a], (uses & 1u) ^ 1u, p.err_flag));
+                    if (!ok) break;
+                    tc_fence_after();
+                    if (elect_one()) {
+                        if (a < tl.na) {
+                            const unsigned long long ad = make_desc(a_addr + a * kABytesL, kmaj ? 16 : kPanelL, 1024);
+                            if (kmaj) {
 #pragma unroll
-                        for (int kk = 0; kk < 4; ++kk)       // 16 rows of A = 2048 bytes
-                            mma_bf16(tmem_d, ad + 128 * kk, bd + 128 * kk, idesc_mn, (k > tl.k0 || kk > 0) ? 1u : 0u);
+                                for (int kk = 0; kk < 4; ++kk)       // 16 along the rows of A = 32 bytes
+                                    mma_bf16(tmem_d + a * kMaxNL, ad + 2 * kk, bd + 128 * kk, idesc_k, (k > tl.k0 || kk > 0) ? 1u : 0u);
+                            } else {
+#pragma unroll
+                                for (int kk = 0; kk < 4; ++kk)       // 16 rows of A = 2048 bytes
+                                    mma_bf16(tmem_d + a * kMaxNL, ad + 128 * kk, bd + 128 * kk, idesc_mn, (k > tl.k0 || kk > 0) ? 1u : 0u);
+                            }
+                        }
+                        if (a == MA - 1) mma_commit(&pipe.empty[s]);
+                        if (k == tl.k1 - 1) mma_commit(&pipe.acc_full[slot + a]);
                     }
-                    mma_commit(&pipe.empty[s]);
                 }
                 if (++s == S) { s = 0; parity ^= 1u; }
             }
-            if (ok && elect_one()) mma_commit(&pipe.acc_full[slot]);
         }
     } else {
         // epilogue: TMEM lane = output row, column = output column; two warps per lane quarter take turns at the
@@ -189,15 +218,14 @@ linear_products_kernel(const __grid_constant__ LinMaps maps, const __grid_consta
         unsigned char *stage = smem + kRingL + (warp - 2) * kOutBlock;
         const float delta = *p.delta_p;
         bool ok = true;
-        int it = 0;
-        for (int t = blockIdx.x; t < p.tiles && ok; t += gridDim.x, ++it) {
-            const Tile tl = tile_of(t);
-            const LinProduct &q = p.pr[tl.i];
-            const int slot = it & 1;
-            ok = mbar_wait(&pipe.acc_full[slot], (static_cast<unsigned>(it) >> 1) & 1u, p.err_flag);
+        for (int it = 0; ok && tile_at(it, tl); ++it) {
+          const LinProduct &q = p.pr[tl.i];
+          for (int am = 0; am < MA; ++am) {
+            const int slot = MA == 2 ? am : it & 1;
+            ok = mbar_wait(&pipe.acc_full[slot], static_cast<unsigned>(MA == 2 ? it : it >> 1) & 1u, p.err_flag);
             if (!ok) break;
             tc_fence_after();
-            const int row_w = tl.m0 + q4 * 32;                     // first output row of this warp
+            const int row_w = tl.m0 + am * 128 + q4 * 32;          // first output row of this warp
             const int ncol = q.cols - tl.n0 < p.TN ? q.cols - tl.n0 : p.TN;
             const int bw = q.out_f32 ? 32 : 64;                    // columns per block
             if (row_w < q.M) {
@@ -241,21 +269,36 @@ linear_products_kernel(const __grid_constant__ LinMaps maps, const __grid_consta
                         }
                     } else {
                         __syncwarp();
+                        // lanes along the columns, eight rows at a time; bf16 as words, shifted by one column in the rows that
+                        // start between words
                         const int nr = q.M - row_w < 32 ? q.M - row_w : 32;
                         const int nc = ncol - c < bw ? ncol - c : bw;
                         const long long o0 = static_cast<long long>(row_w) * q.cols + tl.n0 + c;
-                        for (int r = 0; r < nr; ++r) {
-                            const long long o = o0 + static_cast<long long>(r) * q.cols;
-                            if (q.out_f32) {
-                                const float f = *reinterpret_cast<const float *>(stage + r * 128 + (((lane >> 2) ^ (r & 7)) << 4) + (lane & 3) * 4);
-                                if (lane < nc) {
-                                    if (q.add) atomicAdd(static_cast<float *>(q.out) + o + lane, f);
-                                    else static_cast<float *>(q.out)[o + lane] = f;
+                        for (int r0 = 0; r0 < nr; r0 += 8) {
+                            unsigned x[8];
+#pragma unroll
+                            for (int i = 0; i < 8; ++i)
+                                x[i] = *reinterpret_cast<const unsigned *>(stage + (r0 + i) * 128 + (((lane >> 2) ^ i) << 4) + (lane & 3) * 4);
+#pragma unroll
+                            for (int i = 0; i < 8; ++i) {
+                                const long long o = o0 + static_cast<long long>(r0 + i) * q.cols;
+                                if (q.out_f32) {
+                                    float *const dst = static_cast<float *>(q.out) + o + lane;
+                                    if (r0 + i < nr && lane < nc) {
+                                        if (q.add) atomicAdd(dst, __uint_as_float(x[i]));
+                                        else *dst = __uint_as_float(x[i]);
+                                    }
+                                } else {
+                                    unsigned short *const row = static_cast<unsigned short *>(q.out) + o;
+                                    const int odd = static_cast<int>(o & 1), at = 2 * lane + odd;
+                                    const unsigned up = __shfl_down_sync(0xffffffffu, x[i], 1);
+                                    const unsigned w = odd ? __funnelshift_r(x[i], up, 16) : x[i];
+                                    if (r0 + i < nr) {
+                                        if (at + 1 < nc) *reinterpret_cast<unsigned *>(row + at) = w;
+                                        else if (at < nc) row[at] = static_cast<unsigned short>(w);
+                                        if (odd && lane == 0) row[0] = static_cast<unsigned short>(x[i]);
+                                    }
                                 }
-                            } else {
-                                for (int i = lane; i < nc; i += 32)
-                                    static_cast<unsigned short *>(q.out)[o + i] =
-                                        *reinterpret_cast<const unsigned short *>(stage + r * 128 + (((i >> 3) ^ (r & 7)) << 4) + (i & 7) * 2);
                             }
                         }
                         __syncwarp();
@@ -264,6 +307,7 @@ linear_products_kernel(const __grid_constant__ LinMaps maps, const __grid_consta
             }
             tc_fence_before();
             warp_arrive(&pipe.acc_empty[slot]);
+          }
         }
         if (lane == 0) bulk_wait_read_all();       // the staging block is read before the CTA goes
     }
@@ -283,6 +327,13 @@ bool fits_int(long long v) { return v > 0 && v < (1ll << 30); }
 // 8192 outputs) are cut into parts that follow one another, each added to the one before, so that the order of the sum is fixed.
 // (A bf16 dX rounds far coarser than an accumulator does and is one part.)
 constexpr long long kMaxSteps = kMaxMmas / 4;
+// Clocks of a tile: its steps, whose cost is that of their hand-overs up to 128 columns and of their copies with 256, and its drain,
+// which lies beside the next tile's steps where an accumulator holds a tile. plain: rows leave by ordinary stores. Fitted to 22
+// layers timed in every form (64, 128, 256 columns, 128 or 256 rows, dW in one to eight parts): the form with the least estimate is
+// within 0.8 % of the fastest on average, 6 % at worst.
+double tile_clocks(int TN, int MA, long long steps, bool plain) {
+    return steps * (TN < 256 ? 470.0 : MA == 2 ? 840.0 : 640.0) + (plain ? 20.0 * TN * MA : MA == 2 ? 5.0 * TN * MA : 300.0);
+}
 
 bool linear_tc_supported(long long B, long long N, long long K) { return fits_int(B) && fits_int(N) && fits_int(K); }
 
@@ -293,35 +344,52 @@ long long linear_pitch(long long cols) { return (cols + 7) / 8 * 8; }
 LinearPlan linear_plan(const dbp_ctx *ctx, long long B, long long N, long long K, int pieces, bool want_dw, bool want_dx) {
     LinearPlan pl;
     const long long dw_steps = ((B + 63) / 64) * pieces, dx_steps = ((N + 63) / 64) * pieces;
-    // The shortest makespan of tiles of 256, 128 or 64 columns: a step of a 128 x 256 tile is 512 clocks of the tensor
-    // pipe, narrower ones are bound by their copies and hand-overs (about 420 and 400 clocks); a tile ends with a drain of
-    // about 4 clocks a column. Measured, us, for 64 / 128 / 256 columns: bf16 1024 -> 4096, B 4096: 213 / 144 / 96; fp32
-    // 1024 -> 100, B 1024: 25 / 15.2 / 16.2; bf16 512 -> 512, B 512: 11.9 / 12.3 / 14.0.
-    double best = 1e300;
+    // Split the weight gradient's reduction (into parts of at least four steps) where that shortens what the CTA with the most
+    // work has, or when it is too long for one accumulator. dX is not split: its sums keep one order, so that the gradient handed
+    // to the layer below is reproducible.
+    auto span = [&](int tn, int ma, long long want) {                   // clocks of that CTA, as the kernel deals the tiles
+        const long long rows = 128 * ma, nt = (K + tn - 1) / tn, per = (dw_steps + want - 1) / want, split = (dw_steps + per - 1) / per;
+        long long n0 = want_dx ? (B + rows - 1) / rows * nt : 0, n1 = want_dw ? (N + rows - 1) / rows * nt * split : 0;
+        double c0 = tile_clocks(tn, ma, dx_steps, pieces == 1 ? K % 8 != 0 : K % 4 != 0), c1 = tile_clocks(tn, ma, per, K % 4 != 0);
+        if (!want_dx || (want_dw && per > dx_steps)) { std::swap(n0, n1); std::swap(c0, c1); }
+        const long long G = n0 + n1 < ctx->sm_count ? n0 + n1 : ctx->sm_count, more = n0 % G;
+        double a = (n0 / G + 1) * c0, b = n0 / G * c0;                  // CTAs with one more of the first product's tiles, and the others
+        long long left = n1;
+        if (more > 0) {
+            const long long rounds = (left + G - more - 1) / (G - more), lead = static_cast<long long>(c0 / c1) < rounds ? static_cast<long long>(c0 / c1) : rounds;
+            b += lead * c1;
+            left -= lead * (G - more);
+        }
+        if (left > 0) {
+            a += left / G * c1;
+            b += (left + G - 1) / G * c1;
+            if (left % G > G - more) a += c1;
+        }
+        // parts add into a dW that the statistics kernel clears
+        const double parts = split > 1 ? static_cast<double>(N) * K * 4.0 / 2500.0 * (1.3 + 0.57 * split) : 0.0;
+        return (more > 0 && a > b ? a : b) + parts + 3.0 * tn * ma;
+    };
+    const long long least = (dw_steps + kMaxSteps - 1) / kMaxSteps;
+    // Columns, tile height and parts with the least work for the busiest CTA. Measured, us, before (columns by an estimate without
+    // the dealing, one part unless SMs were idle, tiles of 128 rows dealt in turn) and now: bf16 1576 -> 66, B 4790: 57, 20 (split);
+    // 360 -> 3208, B 6418: 119, 82 (256 rows, split); 560 -> 3476, B 848: 45, 28 (dealt); fp32 4048 -> 904, B 205: 36, 30 (dealt).
+    double shortest = 1e300;
+    long long want = least;
     for (int tn = 64; tn <= 256; tn *= 2) {
         if (tn > 64 && tn / 2 >= K) break;
-        const double step = tn == 256 ? 520.0 : tn == 128 ? 420.0 : 400.0, drain = 4.0 * tn + 500.0;
-        const double nt = static_cast<double>((K + tn - 1) / tn);
-        const double dx = want_dx ? dx_steps * step + drain : 0.0, dw = want_dw ? dw_steps * step + drain : 0.0;
-        const double all = nt * ((B + 127) / 128) * dx + nt * ((N + 127) / 128) * dw;
-        double longest = dx;                                            // (long dW reductions are split)
-        if (longest < all / ctx->sm_count) longest = all / ctx->sm_count;
-        if (longest < best) { best = longest; pl.TN = tn; }
+        long long most = want_dw && dw_steps / 4 > least ? dw_steps / 4 : least;
+        if (want_dw && K % 4 != 0) {
+            // rows of dW that are no multiple of 16 bytes are added element by element: only on SMs that are idle otherwise (1072 x
+            // 3806 x 1841 bf16: 102 us in one part, 236 in two)
+            const long long nt = (K + tn - 1) / tn, idle = (ctx->sm_count - (want_dx ? (B + 127) / 128 * nt : 0)) / ((N + 127) / 128 * nt);
+            if (most > idle) most = idle > least ? idle : least;
+        }
+        for (int ma = 1; ma <= (tn == 256 ? 2 : 1); ++ma)
+            for (long long w = least; w <= most && w <= least + 16; ++w) {
+                const double t = span(tn, ma, w);
+                if (t < shortest) { shortest = t; pl.TN = tn; pl.MA = ma; want = w; }
+            }
     }
-    const long long nt = (K + pl.TN - 1) / pl.TN;
-    const long long dx_tiles = want_dx ? ((B + 127) / 128) * nt : 0;
-    const long long dw_tiles = want_dw ? ((N + 127) / 128) * nt : 0;
-    // Split the weight gradient's reduction when its tiles leave SMs idle (parts of at least four steps) and when it
-    // is too long for one accumulator. dX is not split: its sums keep one order, so that the gradient handed to the
-    // layer below is reproducible.
-    const long long idle = ctx->sm_count - dx_tiles;
-    long long want = 1;
-    if (want_dw && dw_tiles < idle) {
-        want = idle / dw_tiles;
-        if (want > dw_steps / 4) want = dw_steps / 4;
-        if (want < 1) want = 1;
-    }
-    if (want < (dw_steps + kMaxSteps - 1) / kMaxSteps) want = (dw_steps + kMaxSteps - 1) / kMaxSteps;
     pl.dw_per_split = (dw_steps + want - 1) / want;
     pl.dw_split = (dw_steps + pl.dw_per_split - 1) / pl.dw_per_split;
     return pl;
@@ -336,7 +404,8 @@ int launch_products(dbp_ctx *ctx, const LinearPlan &pl, const void *codes, const
     LinMaps maps;
     const long long q_pitch = linear_pitch(N);
     p.TN = pl.TN;
-    p.stage_bytes = kABytesL + pl.TN / 64 * kPanelL;
+    p.MA = pl.MA;
+    p.stage_bytes = p.MA * kABytesL + pl.TN / 64 * kPanelL;
     p.stages = kRingL / p.stage_bytes < kStagesL ? kRingL / p.stage_bytes : kStagesL;
     p.delta_p = delta_p;
     p.err_flag = err_flag;
@@ -359,7 +428,7 @@ int launch_products(dbp_ctx *ctx, const LinearPlan &pl, const void *codes, const
         q.nsplit = is_dx ? 1 : static_cast<int>(pl.dw_split);
         q.per_split = is_dx ? q.steps : static_cast<int>(pl.dw_per_split);
         q.add = is_dx ? n0 > 0 : q.nsplit > 1;
-        q.mt = (q.M + 127) / 128;
+        q.mt = (q.M + 128 * p.MA - 1) / (128 * p.MA);
         const long long tiles = static_cast<long long>(q.mt) * nt * q.nsplit;
         if (tiles + p.tiles >= (1ll << 30)) return DBP_EUNSUPPORTED;
         q.tiles = static_cast<int>(tiles);
@@ -398,10 +467,16 @@ int launch_products(dbp_ctx *ctx, const LinearPlan &pl, const void *codes, const
     if (!rc && dX && !dx_first) rc = fill(true);
     if (rc) return rc;
     const size_t smem = static_cast<size_t>(kRingL) + kEpiWarpsL * kOutBlock + 1024;
-    if (cudaFuncSetAttribute(linear_products_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem)) != cudaSuccess)
+    const auto kern = p.MA == 2 ? linear_products_kernel<2> : linear_products_kernel<1>;
+    if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem)) != cudaSuccess)
         return fail_cuda("shared memory size");
-    const int grid = p.tiles < ctx->sm_count ? p.tiles : ctx->sm_count;
-    return cuda_ok(launch_chained(linear_products_kernel, dim3(static_cast<unsigned>(grid)), dim3(kThreadsL), smem, ctx->stream, maps, p));
+    const int grid = p.tiles < ctx->sm_count ? p.tiles : ctx->sm_count, more = p.pr[0].tiles % grid;
+    if (p.nprod == 2 && more > 0) {
+        auto clocks = [&](const LinProduct &q) { return tile_clocks(pl.TN, pl.MA, q.per_split, !q.tma_out); };
+        const double ratio = clocks(p.pr[0]) / clocks(p.pr[1]), most = p.pr[1].tiles / (grid - more) + 1;
+        p.lead = ratio < 1.0 ? 1 : static_cast<int>(ratio < most ? ratio : most);
+    }
+    return cuda_ok(launch_chained(kern, dim3(static_cast<unsigned>(grid)), dim3(kThreadsL), smem, ctx->stream, maps, p));
 }
 }  // namespace
 

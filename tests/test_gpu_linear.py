@@ -24,6 +24,9 @@ def ctx():
     ("bf16", 1, 1, 1), ("bf16", 128, 64, 64), ("bf16", 129, 65, 71), ("bf16", 33, 300, 264), ("bf16", 700, 10, 257),
     ("bf16", 640, 136, 520),           # dW split along the reduction
     ("bf16", 36, 2470, 320), ("bf16", 2560, 1280, 512),      # more tiles than SMs: two accumulators in flight
+    ("bf16", 4225, 2200, 1032),        # tiles of 256 rows: the last of dX holds one row, the last columns are eight
+    ("bf16", 4225, 2200, 1030),        # the same, rows of X and W re-written, plain stores
+    ("bf16", 6418, 3208, 360),         # the same in parts
     ("f32", 257, 513, 65), ("f32", 131, 1003, 131), ("f32", 20000, 7, 12), ("f32", 256, 1000, 2048), ("f32", 513, 260, 8)])
 def test_both_products_and_the_bias_gradient(ctx, dtype, B, N, K):
     import paper_2004_04729_b200 as dbp
