@@ -33,17 +33,20 @@ struct DwT {
     long long nchunks;            // images of the activation tensor * cpi
     int ci_tiles, nsplit;
     long long per_split;          // chunks per CTA
-    int NT, NTp, MA, stages;      // ci tile, its accumulator stride (multiple of 32), accumulators
+    int NT, NTp;                  // ci tile, its accumulator stride (multiple of 32)
     int tmem_cols;
     int *err_flag;
     unsigned long long *stats;    // wait counters (may be null)
 };
+
+template <int MA> constexpr int kStagesW = MA == 2 ? 3 : 4;      // MA: accumulators of 128 output channels
 
 struct PipeW {
     unsigned long long full[4], empty[4], acc_full;
     unsigned tmem_base;
 };
 
+template <int MA>
 __global__ void __launch_bounds__(kThreadsW, 1)
 tma_dw_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUtensorMap map_x,
               const __grid_constant__ CUtensorMap map_dw, const DwT p) {
@@ -51,14 +54,13 @@ tma_dw_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant__
     unsigned char *smem = reinterpret_cast<unsigned char *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
     __shared__ PipeW pipe;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int S = p.stages;
-    const int stage_bytes = p.MA * kATile + kBMax;
+    constexpr int S = kStagesW<MA>, stage_bytes = MA * kATile + kBMax;
 
     // my work item: output tile (co group, ci tile) and a range of chunks
     const int split = blockIdx.x % p.nsplit;
     const int tile = blockIdx.x / p.nsplit;
     const int ci0 = (tile % p.ci_tiles) * p.NT;
-    const int co0 = (tile / p.ci_tiles) * 128 * p.MA;
+    const int co0 = (tile / p.ci_tiles) * 128 * MA;
     const long long k0 = split * p.per_split;
     const long long k1 = k0 + p.per_split < p.nchunks ? k0 + p.per_split : p.nchunks;
 
@@ -85,19 +87,22 @@ tma_dw_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant__
         if (lane == 0) {
             int s = 0;
             unsigned parity = 1;
-            long long b = k0 / p.cpi;
-            int c = static_cast<int>(k0 - b * p.cpi);
-            const unsigned bytes = static_cast<unsigned>(p.MA * kATile + p.NT * 128);
+            int b = static_cast<int>(k0 / p.cpi), c = static_cast<int>(k0 - static_cast<long long>(b) * p.cpi), bq = b % p.code_batch;
+            const unsigned bytes = static_cast<unsigned>(MA * kATile + p.NT * 128);
             long long waited = 0;
-            for (long long k = k0; k < k1; ++k) {
+            for (int k = static_cast<int>(k1 - k0); k > 0; --k) {
                 if (!mbar_wait_timed(&pipe.empty[s], parity, p.err_flag, waited)) break;
                 unsigned char *st = smem + s * stage_bytes;
                 mbar_expect_tx(&pipe.full[s], bytes);
-                const int bq = static_cast<int>(b % p.code_batch);
-                for (int a = 0; a < p.MA; ++a)
+#pragma unroll
+                for (int a = 0; a < MA; ++a)
                     tma_load_3d(st + a * kATile, &map_q, c * 64, co0 + a * 128, bq, &pipe.full[s]);
-                tma_load_3d(st + p.MA * kATile, &map_x, c * 64, ci0, static_cast<int>(b), &pipe.full[s]);
-                if (++c == p.cpi) { c = 0; ++b; }
+                tma_load_3d(st + MA * kATile, &map_x, c * 64, ci0, b, &pipe.full[s]);
+                if (++c == p.cpi) {
+                    c = 0;
+                    ++b;
+                    if (++bq == p.code_batch) bq = 0;
+                }
                 if (++s == S) { s = 0; parity ^= 1u; }
             }
             report_wait(p.stats, 3, waited);
@@ -111,7 +116,8 @@ tma_dw_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant__
             int c = static_cast<int>(k0 % p.cpi);
             long long wf = 0;
             const long long born = clock64();
-            for (long long k = k0; k < k1; ++k) {
+            unsigned on = 0u;
+            for (int k = static_cast<int>(k1 - k0); k > 0; --k) {
                 ok = __all_sync(0xffffffffu, mbar_wait_timed(&pipe.full[s], parity, p.err_flag, wf));
                 if (!ok) break;
                 tc_fence_after();
@@ -120,15 +126,22 @@ tma_dw_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant__
                 const int valid = p.HW - c * 64 < 64 ? p.HW - c * 64 : 64;
                 const int nk = (valid + 15) >> 4;
                 const unsigned a_addr = smem_u32(smem + s * stage_bytes);
-                const unsigned long long bd = make_desc(a_addr + p.MA * kATile, 16, 1024);
+                const unsigned long long bd = make_desc(a_addr + MA * kATile, 16, 1024);
                 if (elect_one()) {
-                    for (int a = 0; a < p.MA; ++a) {
+#pragma unroll
+                    for (int a = 0; a < MA; ++a) {
                         const unsigned long long ad = make_desc(a_addr + a * kATile, 16, 1024);
-                        for (int kk = 0; kk < nk; ++kk)       // 16 positions = 32 bytes further per MMA
-                            mma_bf16(tmem_base + a * p.NTp, ad + 2 * kk, bd + 2 * kk, idesc, (k > k0 || kk > 0) ? 1u : 0u);
+                        if (nk == 4) {
+#pragma unroll
+                            for (int kk = 0; kk < 4; ++kk)    // 16 positions = 32 bytes further per MMA
+                                mma_bf16(tmem_base + a * p.NTp, ad + 2 * kk, bd + 2 * kk, idesc, kk ? 1u : on);
+                        } else {
+                            for (int kk = 0; kk < nk; ++kk) mma_bf16(tmem_base + a * p.NTp, ad + 2 * kk, bd + 2 * kk, idesc, kk ? 1u : on);
+                        }
                     }
                     mma_commit(&pipe.empty[s]);
                 }
+                on = 1u;
                 if (++c == p.cpi) c = 0;
                 if (++s == S) { s = 0; parity ^= 1u; }
             }
@@ -151,7 +164,8 @@ tma_dw_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant__
             const long long t_epi = clock64();
             const float delta = *p.delta_p;
             int n = 0;
-            for (int a = 0; a < p.MA; ++a) {
+#pragma unroll 1
+            for (int a = 0; a < MA; ++a) {
                 const int co_w = co0 + a * 128 + q * 32;                 // first output channel of this warp
 #pragma unroll 1
                 for (int c0 = 0; c0 < p.NT; c0 += 32, ++n) {
@@ -213,12 +227,11 @@ int launch_tma_dw(dbp_ctx *ctx, const void *codes_bf16, const void *X, int piece
     p.nchunks = s.B * pieces * p.cpi;
     p.NT = s.Cin >= 256 ? 256 : static_cast<int>((s.Cin + 15) / 16 * 16);
     p.NTp = (p.NT + 31) / 32 * 32;
-    p.MA = s.Cout > 128 ? 2 : 1;
-    p.stages = p.MA == 2 ? 3 : 4;
+    const int MA = s.Cout > 128 ? 2 : 1;
     p.tmem_cols = 32;
-    while (p.tmem_cols < p.MA * p.NTp) p.tmem_cols *= 2;
+    while (p.tmem_cols < MA * p.NTp) p.tmem_cols *= 2;
     p.ci_tiles = static_cast<int>((s.Cin + p.NT - 1) / p.NT);
-    const long long co_tiles = (s.Cout + 128 * p.MA - 1) / (128 * p.MA);
+    const long long co_tiles = (s.Cout + 128 * MA - 1) / (128 * MA);
     const long long tiles = co_tiles * p.ci_tiles;
     // (a chunk of 64 positions is four MMAs)
     const long long nsplit = choose_split(tiles, p.nchunks, ctx->sm_count, kMaxMmas / 4, &p.per_split);
@@ -251,11 +264,12 @@ int launch_tma_dw(dbp_ctx *ctx, const void *codes_bf16, const void *X, int piece
         const unsigned box[3] = {64, static_cast<unsigned>(p.NT), 1};
         if (!encode_map_bf16(&map_x, X, 3, dims, str, box)) return fail_cuda("tensor map of the activations");
     }
-    const size_t smem = static_cast<size_t>(p.stages) * (p.MA * kATile + kBMax) + 1024;       // >= 4 warps x 4 staging blocks
-    if (cudaFuncSetAttribute(tma_dw_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem)) != cudaSuccess)
+    const size_t smem = static_cast<size_t>(MA == 2 ? kStagesW<2> : kStagesW<1>) * (MA * kATile + kBMax) + 1024;       // >= 4 warps x 4 staging blocks
+    const auto kern = MA == 2 ? tma_dw_kernel<2> : tma_dw_kernel<1>;
+    if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem)) != cudaSuccess)
         return DBP_ECUDA;
     // dW has been cleared by this layer's statistics kernel
-    return cuda_ok(launch_chained(tma_dw_kernel, dim3(static_cast<unsigned>(tiles * nsplit)), dim3(kThreadsW), smem,
+    return cuda_ok(launch_chained(kern, dim3(static_cast<unsigned>(tiles * nsplit)), dim3(kThreadsW), smem,
                                   ctx->stream, map_q, map_x, map_dw, p));
 }
 

@@ -106,6 +106,7 @@ struct PipeT {
     unsigned tmem_base;
 };
 
+template <int MA>
 __global__ void __launch_bounds__(kThreadsT, 1)
 tma_dx_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constant__ CUtensorMap map_q,
               const __grid_constant__ CUtensorMap map_dx, const DxT p) {
@@ -116,8 +117,7 @@ tma_dx_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constant__
     // With two accumulators a tile is 256 channels: both share the stage's code tile, each has its
     // own weight tile, and the two TMEM accumulators belong to one tile (no second tile in
     // flight). With one accumulator tiles alternate between the two TMEM accumulators.
-    const int MA = p.MA, S = MA == 2 ? 3 : 4;
-    const int a_bytes = MA * kABytes, stage_bytes = a_bytes + kBBytes;
+    constexpr int S = MA == 2 ? 3 : 4, a_bytes = MA * kABytes, stage_bytes = a_bytes + kBBytes;
 
     if (threadIdx.x == 0) {
         for (int s = 0; s < kStages; ++s) {
@@ -157,23 +157,28 @@ tma_dx_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constant__
                 const int b0 = static_cast<int>(g0 / p.chunks_per_img);
                 const int c0 = static_cast<int>(g0 - static_cast<long long>(b0) * p.chunks_per_img);
                 const unsigned tx = static_cast<unsigned>((2 * MA + nch) * kPanel);
-                for (int ks = 0; ks < p.ksteps && ok; ++ks) {
+                int cb[kNChunks], cp[kNChunks];
+#pragma unroll
+                for (int i = 0; i < kNChunks; ++i) {
+                    const bool wrap = i > 0 && cp[i ? i - 1 : 0] + 64 == p.chunks_per_img * 64;
+                    cp[i] = i == 0 ? c0 * 64 : wrap ? 0 : cp[i ? i - 1 : 0] + 64;
+                    cb[i] = i == 0 ? b0 : cb[i ? i - 1 : 0] + (wrap ? 1 : 0);
+                }
+                // the low pieces first: the accumulator is still small when they are added
+                int piece = p.pieces - 1, co0 = 0;
+                for (int ks = 0; ks < p.ksteps; ++ks) {
                     ok = __all_sync(0xffffffffu, mbar_wait_timed(&pipe.empty[s], parity, p.err_flag, waited));
                     if (!ok) break;
                     if (elect_one()) {
                         unsigned char *st = smem + s * stage_bytes;
-                        // the low pieces first: the accumulator is still small when they are added
-                        const int kp = ks / p.ks_piece, co0 = (ks - kp * p.ks_piece) * 64;
                         mbar_expect_tx(&pipe.full[s], tx);
-                        for (int h = 0; h < 2 * MA; ++h)
-                            tma_load_3d(st + h * kPanel, &map_w, ci0 + 64 * h, co0, p.pieces - 1 - kp, &pipe.full[s]);
-                        st += a_bytes;
-                        int b = b0, c = c0;
-                        for (int i = 0; i < nch; ++i, st += kPanel) {
-                            tma_load_3d(st, &map_q, c * 64, co0, b, &pipe.full[s]);
-                            if (++c == p.chunks_per_img) { c = 0; ++b; }
-                        }
+#pragma unroll
+                        for (int h = 0; h < 2 * MA; ++h) tma_load_3d(st + h * kPanel, &map_w, ci0 + 64 * h, co0, piece, &pipe.full[s]);
+#pragma unroll
+                        for (int i = 0; i < kNChunks; ++i)
+                            if (i < nch) tma_load_3d(st + a_bytes + i * kPanel, &map_q, cp[i], co0, cb[i], &pipe.full[s]);
                     }
+                    if ((co0 += 64) >= 64 * p.ks_piece) { co0 = 0; --piece; }
                     if (++s == S) { s = 0; parity ^= 1u; }
                 }
             }
@@ -205,6 +210,7 @@ tma_dx_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constant__
                     const unsigned a_addr = smem_u32(smem + s * stage_bytes);
                     const unsigned long long bd = make_desc(a_addr + a_bytes, kPanel, 1024);
                     if (elect_one()) {
+#pragma unroll
                         for (int a = 0; a < MA; ++a) {
                             const unsigned long long ad = make_desc(a_addr + a * kABytes, kPanel, 1024);
                             const unsigned tmem_d = tmem_base + (slot0 + a) * kAccCols;
@@ -217,6 +223,7 @@ tma_dx_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constant__
                     if (++s == S) { s = 0; parity ^= 1u; }
                 }
                 if (ok && elect_one())
+#pragma unroll
                     for (int a = 0; a < MA; ++a) mma_commit(&pipe.acc_full[slot0 + a]);
             }
             if (lane == 0) {
@@ -481,10 +488,11 @@ int launch_tma_dx_part(dbp_ctx *ctx, const void *codes_bf16, const void *W, int 
     p.err_flag = err_flag;
     p.stats = ctx->wait_stats;
     const size_t smem = static_cast<size_t>(kRing) + kEpiWarps * kStageOut + 1024;
-    if (cudaFuncSetAttribute(tma_dx_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem)) != cudaSuccess)
+    const auto kern = p.MA == 2 ? tma_dx_kernel<2> : tma_dx_kernel<1>;
+    if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem)) != cudaSuccess)
         return DBP_ECUDA;
     const long long grid = p.ntiles < ctx->sm_count ? p.ntiles : ctx->sm_count;
-    return cuda_ok(launch_chained(tma_dx_kernel, dim3(static_cast<unsigned>(grid)), dim3(kThreadsT), smem, ctx->stream,
+    return cuda_ok(launch_chained(kern, dim3(static_cast<unsigned>(grid)), dim3(kThreadsT), smem, ctx->stream,
                                   map_w, map_q, map_dx, p));
 }
 }  // namespace
