@@ -84,20 +84,31 @@ __device__ __forceinline__ void rows_job(const RowsJob &j, long long first, long
                 *reinterpret_cast<uint4 *>(dst) = make_uint4(a.x, a.y, b.x, b.y);
                 continue;
             }
-            // 32-bit loads whatever the row's start: a row that starts on an odd element is shifted by half a word
-            const long long off = row * j.cols + c0, total = j.rows * j.cols;
+            // the two 16-byte words that hold the eight values, whatever the row's start, and a shift (32-bit loads before: 59 x 344
+            // rows of 59 x 59 values 65 us)
+            const long long off = row * j.cols + c0, total = j.rows * j.cols, at = off & ~7ll;
             const unsigned short *src = static_cast<const unsigned short *>(j.src);
-            const int odd = static_cast<int>(off & 1), nv = left < 8 ? static_cast<int>(left) : 8;
-            unsigned v[5], w[4];
+            const int sh = static_cast<int>(off & 7), nv = left < 8 ? static_cast<int>(left) : 8;
+            unsigned w[4];
+            if (at + 16 <= total) {
+                const uint4 lo = __ldg(reinterpret_cast<const uint4 *>(src + at)), hi = __ldg(reinterpret_cast<const uint4 *>(src + at + 8));
+                const unsigned x[8] = {lo.x, lo.y, lo.z, lo.w, hi.x, hi.y, hi.z, hi.w};
+                unsigned y[6], z[5];
 #pragma unroll
-            for (int e = 0; e < 5; ++e) {
-                const long long i0 = (off & ~1ll) + 2 * e;
-                v[e] = 0u;
-                if (2 * e < odd + nv) v[e] = i0 + 1 < total ? __ldg(reinterpret_cast<const unsigned *>(src + i0)) : __ldg(src + i0);
+                for (int e = 0; e < 6; ++e) y[e] = sh & 4 ? x[e + 2] : x[e];
+#pragma unroll
+                for (int e = 0; e < 5; ++e) z[e] = sh & 2 ? y[e + 1] : y[e];
+#pragma unroll
+                for (int e = 0; e < 4; ++e) w[e] = __funnelshift_r(z[e], z[e + 1], (sh & 1) * 16);
+            } else {                               // the tensor's last values, one by one
+#pragma unroll
+                for (int e = 0; e < 4; ++e) {
+                    w[e] = 2 * e < nv ? __ldg(src + off + 2 * e) : 0u;
+                    if (2 * e + 1 < nv) w[e] |= static_cast<unsigned>(__ldg(src + off + 2 * e + 1)) << 16;
+                }
             }
 #pragma unroll
             for (int e = 0; e < 4; ++e) {
-                w[e] = odd ? __byte_perm(v[e], v[e + 1], 0x5432) : v[e];
                 if (2 * e >= nv) w[e] = 0u;
                 else if (2 * e + 1 >= nv) w[e] &= 0xffffu;
             }

@@ -172,19 +172,6 @@ __device__ __forceinline__ bool epilogue_all(bool mine) {
     return r != 0;
 }
 
-// The same between the two warps that share a block: named barriers 2 ..
-__device__ __forceinline__ bool pair_all(int id, bool mine) {
-    unsigned r;
-    asm volatile(
-        "{\n\t.reg .pred p, q;\n\t"
-        "setp.ne.b32 p, %1, 0;\n\t"
-        "bar.red.and.pred q, %2, 64, p;\n\t"
-        "selp.b32 %0, 1, 0, q;\n\t}"
-        : "=r"(r) : "r"(mine ? 1u : 0u), "r"(id) : "memory");
-    return r != 0;
-}
-__device__ __forceinline__ void pair_sync(int id) { asm volatile("bar.sync %0, 64;" ::"r"(id) : "memory"); }
-
 // BLOCKS: dX leaves in blocks by the copy engine (p.unit > 0, p.KS == 1); an instance of its own because the other paths' code
 // in the same kernel costs each of them 3 %
 // LEAN: half an SM (shared memory, tensor memory, registers): one tile per CTA, a dW CTA beside it

@@ -72,6 +72,19 @@ __device__ __forceinline__ bool mbar_wait_timed(unsigned long long *bar, unsigne
     waited += clock64() - t0;
     return ok;
 }
+// Named barriers of two warps that share a block of shared memory; pair_all also tells both whether both are still fine (one whose
+// bounded wait ran out arrives like the other, so neither is left waiting).
+__device__ __forceinline__ bool pair_all(int id, bool mine) {
+    unsigned r;
+    asm volatile(
+        "{\n\t.reg .pred p, q;\n\t"
+        "setp.ne.b32 p, %1, 0;\n\t"
+        "bar.red.and.pred q, %2, 64, p;\n\t"
+        "selp.b32 %0, 1, 0, q;\n\t}"
+        : "=r"(r) : "r"(mine ? 1u : 0u), "r"(id) : "memory");
+    return r != 0;
+}
+__device__ __forceinline__ void pair_sync(int id) { asm volatile("bar.sync %0, 64;" ::"r"(id) : "memory"); }
 __device__ __forceinline__ void report_wait(unsigned long long *stats, int slot, long long cycles) {
     if (stats != nullptr && cycles > 0) atomicAdd(stats + slot, static_cast<unsigned long long>(cycles));
 }

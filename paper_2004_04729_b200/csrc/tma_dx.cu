@@ -106,7 +106,9 @@ struct PipeT {
     unsigned tmem_base;
 };
 
-template <int MA>
+// SHIFTED: bf16 rows of dX that start on any element, which leave as 16-byte words put together from pairs of chunks; an instance
+// of its own because its code in the same kernel costs the others (ResNet-50 set 865 us with it, 860 without).
+template <int MA, bool SHIFTED>
 __global__ void __launch_bounds__(kThreadsT, 1)
 tma_dx_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constant__ CUtensorMap map_q,
               const __grid_constant__ CUtensorMap map_dx, const DxT p) {
@@ -252,8 +254,78 @@ tma_dx_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constant__
             const long long g0 = (tr / p.ci_tiles) * p.nct;
             const int nch = static_cast<int>(p.nchunks - g0 < p.nct ? p.nchunks - g0 : p.nct);
             ok = mbar_wait_timed(&pipe.acc_full[a], uses & 1u, p.err_flag, we);
+            if (SHIFTED) ok = pair_all(1 + q, ok);
             if (!ok) break;
             tc_fence_after();
+            if constexpr (SHIFTED) {
+                // Rows that start anywhere. The two warps of a lane quarter share a block of 32 channels x 128 positions (two
+                // chunks); each then takes sixteen of its rows, sixteen lanes to a row, as the 16-byte words of dX that lie
+                // within it, put together from two of the block's, and the codes before and behind these one by one. Chunk by
+                // chunk in 4-byte words, four requests for 128 bytes, 40 outputs of 344 channels at 59x59, batch 59, took this kernel
+                // 195 us instead of 90 (the whole call 318 instead of 211).
+                unsigned char *const block = smem + kRing + q * 2 * kStageOut;
+                for (int c = 0; c < nch; c += 2) {
+                    if (c + part < nch && ci_w < p.Cin) {
+#pragma unroll
+                        for (int half = 0; half < 2; ++half) {
+                            unsigned v[32];
+                            tmem_ld32(tmem_base + (static_cast<unsigned>(q * 32) << 16) + a * kAccCols + (c + part) * 64 + half * 32, v);
+#pragma unroll
+                            for (int j = 0; j < 4; ++j) {
+                                unsigned w[4];
+#pragma unroll
+                                for (int i = 0; i < 4; ++i) {
+                                    const __nv_bfloat162 h = __floats2bfloat162_rn(__uint_as_float(v[8 * j + 2 * i]) * delta,
+                                                                                   __uint_as_float(v[8 * j + 2 * i + 1]) * delta);
+                                    w[i] = *reinterpret_cast<const unsigned *>(&h);
+                                }
+                                *reinterpret_cast<uint4 *>(block + lane * 256 + ((8 * part + ((4 * half + j) ^ (lane & 7))) << 4)) =
+                                    make_uint4(w[0], w[1], w[2], w[3]);
+                            }
+                        }
+                    }
+                    pair_sync(1 + q);
+                    // `len` positions from p0 on of image b, which lie in the block from 16-byte piece `at` on
+                    auto leave = [&](long long b, int p0, int len, int at) {
+                        const int l = lane & 15;
+#pragma unroll 2
+                        for (int i = 0; i < 8; ++i) {
+                            const int r = 16 * part + 2 * i + (lane >> 4);
+                            if (ci_w + r >= p.Cin) break;
+                            const long long o = (b * p.Cin + ci_w + r) * p.HW + p0;
+                            unsigned short *const row = static_cast<unsigned short *>(p.dX) + o;
+                            int head = static_cast<int>(-o & 7);         // codes before the first whole word
+                            if (head > len) head = len;
+                            const int nw = (len - head) >> 3;
+                            auto piece = [&](int k) {
+                                return *reinterpret_cast<const uint4 *>(block + r * 256 + (((k & 8) | ((k ^ r) & 7)) << 4));
+                            };
+                            if (l < nw) {
+                                const uint4 lo = piece(at + l), hi = piece(at + l < 15 ? at + l + 1 : 15);
+                                const unsigned x[8] = {lo.x, lo.y, lo.z, lo.w, hi.x, hi.y, hi.z, hi.w};
+                                unsigned y[6], z[5];
+#pragma unroll
+                                for (int k = 0; k < 6; ++k) y[k] = head & 4 ? x[k + 2] : x[k];
+#pragma unroll
+                                for (int k = 0; k < 5; ++k) z[k] = head & 2 ? y[k + 1] : y[k];
+                                const int sh = (head & 1) * 16;
+                                *reinterpret_cast<uint4 *>(row + head + 8 * l) =
+                                    make_uint4(__funnelshift_r(z[0], z[1], sh), __funnelshift_r(z[1], z[2], sh),
+                                               __funnelshift_r(z[2], z[3], sh), __funnelshift_r(z[3], z[4], sh));
+                            }
+                            const int e = l < 8 ? l : head + 8 * nw + l - 8, k = at + (e >> 3);
+                            if (l < 8 ? e < head : e < len)
+                                row[e] = *reinterpret_cast<const unsigned short *>(block + r * 256 + (((k & 8) | ((k ^ r) & 7)) << 4) + (e & 7) * 2);
+                        }
+                    };
+                    const long long b = (g0 + c) / p.chunks_per_img;
+                    const int p0 = static_cast<int>((g0 + c) - b * p.chunks_per_img) * 64, here = p.HW - p0;
+                    const bool two = c + 1 < nch, same = two && here > 64;
+                    leave(b, p0, same ? (here < 128 ? here : 128) : here < 64 ? here : 64, 0);
+                    if (two && !same) leave(b + 1, 0, p.HW < 64 ? p.HW : 64, 8);
+                    pair_sync(1 + q);                                    // the block is written again
+                }
+            } else
             for (int c = part; c < nch; c += kEpiWarps / 4) {
                 const long long b = (g0 + c) / p.chunks_per_img;
                 const int p0 = static_cast<int>((g0 + c) % p.chunks_per_img) * 64;
@@ -359,9 +431,7 @@ tma_dx_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constant__
                     }
                 }
                 if (!p.dx_f32) {
-                    // staging block -> dX with lanes along the positions: 8-byte pieces where every row starts on 8 bytes,
-                    // else words, shifted by one position in the rows that start between words (55 x 24 -> 56 channels at
-                    // 39x41: this kernel 80 -> 32 us; element by element before, all lanes on the same banks). When the
+                    // staging block -> dX with lanes along the positions, in 8-byte pieces: every row starts on 8 bytes. When the
                     // chunk is the whole plane: one contiguous run of 32 channels x HW positions
                     __syncwarp();
                     const int nrows = p.Cin - ci_w < 32 ? p.Cin - ci_w : 32;
@@ -379,31 +449,12 @@ tma_dx_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constant__
                                     *reinterpret_cast<uint2 *>(base + static_cast<long long>(r) * p.HW + pc * 4) =
                                         *reinterpret_cast<const uint2 *>(stage + r * 128 + (((pc >> 1) ^ (r & 7)) << 4) + (pc & 1) * 8);
                             }
-                        } else if (p.HW % 4 == 0) {
+                        } else {
                             const int per_row = nv / 4, n8 = nrows * per_row;
                             for (int i = lane; i < n8; i += 32) {
                                 const int r = i / per_row, c4 = i - r * per_row;
                                 *reinterpret_cast<uint2 *>(base + static_cast<long long>(r) * p.HW + c4 * 4) =
                                     *reinterpret_cast<const uint2 *>(stage + r * 128 + (((c4 >> 1) ^ (r & 7)) << 4) + (c4 & 1) * 8);
-                            }
-                        } else {
-                            for (int r0 = 0; r0 < nrows; r0 += 8) {
-                                unsigned x[8];
-#pragma unroll
-                                for (int i = 0; i < 8; ++i)
-                                    x[i] = *reinterpret_cast<const unsigned *>(stage + (r0 + i) * 128 + (((lane >> 2) ^ i) << 4) + (lane & 3) * 4);
-#pragma unroll
-                                for (int i = 0; i < 8; ++i) {
-                                    __nv_bfloat16 *row = base + static_cast<long long>(r0 + i) * p.HW;
-                                    const int odd = static_cast<int>(reinterpret_cast<uintptr_t>(row) >> 1) & 1, at = 2 * lane + odd;
-                                    const unsigned up = __shfl_down_sync(0xffffffffu, x[i], 1);
-                                    const unsigned w = odd ? __funnelshift_r(x[i], up, 16) : x[i];
-                                    if (r0 + i < nrows) {
-                                        if (at + 1 < nv) *reinterpret_cast<unsigned *>(row + at) = w;
-                                        else if (at < nv) *reinterpret_cast<unsigned short *>(row + at) = static_cast<unsigned short>(w);
-                                        if (odd && lane == 0) *reinterpret_cast<unsigned short *>(row) = static_cast<unsigned short>(x[i]);
-                                    }
-                                }
                             }
                         }
                     }
@@ -462,6 +513,8 @@ int launch_tma_dx_part(dbp_ctx *ctx, const void *codes_bf16, const void *W, int 
     p.add = co0 > 0 ? 1 : 0;
     CUtensorMap map_dx = map_w;                  // a valid map when the store path is not used
     p.tma_out = HW % (dx_bf16 ? 8 : 4) == 0 ? 1 : 0;
+    // (planes of less than a chunk leave as one run of 32 channels, where the channels make that a multiple of 16 bytes)
+    const bool shifted = dx_bf16 && HW % 4 != 0 && !(HW < 64 && s.Cin % 8 == 0);
     if (p.tma_out) {
         const unsigned long long es = dx_bf16 ? 2 : 4;
         const unsigned long long dims[3] = {static_cast<unsigned long long>(HW), static_cast<unsigned long long>(s.Cin),
@@ -488,7 +541,8 @@ int launch_tma_dx_part(dbp_ctx *ctx, const void *codes_bf16, const void *W, int 
     p.err_flag = err_flag;
     p.stats = ctx->wait_stats;
     const size_t smem = static_cast<size_t>(kRing) + kEpiWarps * kStageOut + 1024;
-    const auto kern = p.MA == 2 ? tma_dx_kernel<2> : tma_dx_kernel<1>;
+    const auto kern = p.MA == 2 ? (shifted ? tma_dx_kernel<2, true> : tma_dx_kernel<2, false>)
+                                : (shifted ? tma_dx_kernel<1, true> : tma_dx_kernel<1, false>);
     if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem)) != cudaSuccess)
         return DBP_ECUDA;
     const long long grid = p.ntiles < ctx->sm_count ? p.ntiles : ctx->sm_count;

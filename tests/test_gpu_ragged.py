@@ -27,6 +27,8 @@ def ctx():
     (2, 300, 70, 5, 5, 1),        # three tiles of input channels, two accumulators' worth
     (9, 20, 24, 1, 2, 1),         # the smallest plane
     (4, 64, 40, 3, 3, 1), (1, 257, 129, 16, 12, 1),
+    (3, 41, 56, 13, 5, 1),        # one position behind a whole chunk, rows that start anywhere
+    (30, 257, 250, 31, 33, 1),    # the same in tiles of 256 input channels, pairs of chunks across images
     (2, 3, 8, 6, 6, 3), (2, 12, 20, 9, 9, 3), (3, 130, 65, 7, 5, 3), (2, 65, 67, 8, 8, 3), (4, 10, 6, 2, 3, 3),
     (1, 33, 129, 20, 17, 3), (3, 9, 1, 6, 7, 3)])
 @pytest.mark.parametrize("dtype", ["f32", "bf16"])
