@@ -605,12 +605,13 @@ quantize_nhwc_any_kernel(const T *__restrict__ x, int B, int C, int HW, unsigned
 // the piece starts on an odd element), and leave as one contiguous copy (the padding of a plane is never read by anybody).
 // Placing the codes one by one at their pitch instead took 52 instructions an element: 6.4 M elements of 7 x 7 planes 17.5 us,
 // 12 so.
-// NHWC: the run is a multiple of eight channels of one image, and leaves position-major: eight channels of a position are
+// NHWC: the run is a multiple of eight channels of one image (at 472 channels of 5x5 planes runs of eight, the only number that
+// divides them, took 34 us for 1.4 M elements), and leaves position-major: eight channels of a position are
 // eight 16-bit reads, a plane apart (in different banks for odd planes).
 constexpr int kOddElems = 6272;                   // most elements of a run
 
 struct NhwcOut {
-    int C;                        // channels: a multiple of 8, and of a run's
+    int C;                        // channels: a multiple of 8
     unsigned short *stack;        // the copy with rows of zeros after every image (may be null)
     int plane_w;                  // how many
 };
@@ -625,7 +626,9 @@ quantize_planes_odd_kernel(const T *__restrict__ x, long long nplanes, int hw, i
     constexpr int kBetween = kThreads * V;
     constexpr unsigned long long kBetweenZ = kBetween / 2 * kGamma;
     __shared__ __align__(16) unsigned run_s[kOddElems / 2 + 8];
-    const long long nruns = (nplanes + planes_per_run - 1) / planes_per_run;
+    // NHWC: a run's channels are of one image, whose last run has what is left of them
+    const int per_image = NHWC ? (nhwc.C + planes_per_run - 1) / planes_per_run : 1;
+    const long long nruns = NHWC ? nplanes / nhwc.C * per_image : (nplanes + planes_per_run - 1) / planes_per_run;
     uint4 raw[NV];
     unsigned msk[MASKED ? NV : 1];
     unsigned long long u[NV][V / 2];
@@ -642,9 +645,20 @@ quantize_planes_odd_kernel(const T *__restrict__ x, long long nplanes, int hw, i
         for (int k = 0; k < NV; ++k) dithers_at<V>(zz + k * kBetweenZ, u[k]);
     };
     const long long run_e = static_cast<long long>(planes_per_run) * hw, total = nplanes * hw;
-    long long r = blockIdx.x, base = r * run_e;
-    auto run_len = [&](long long b) { return static_cast<int>(total - b < run_e ? total - b : run_e); };       // a multiple of 8
-    int len = run_len(base), done = threadIdx.x * V;                // elements of the run; the thread's place in it
+    long long r = blockIdx.x, base = r * run_e, image = 0;
+    int c0 = 0, chans = 0, image_n = 0, c0_n = 0, chans_n = 0;       // NHWC: the run in hand, and the next one
+    // run r's first element and its length (a multiple of 8)
+    auto find = [&]() {
+        if (NHWC) {
+            image_n = static_cast<int>(r / per_image);
+            c0_n = static_cast<int>(r - static_cast<long long>(image_n) * per_image) * planes_per_run;
+            chans_n = nhwc.C - c0_n < planes_per_run ? nhwc.C - c0_n : planes_per_run;
+            base = (static_cast<long long>(image_n) * nhwc.C + c0_n) * hw;
+            return chans_n * hw;
+        }
+        return static_cast<int>(total - base < run_e ? total - base : run_e);
+    };
+    int len = find(), done = threadIdx.x * V;                // elements of the run; the thread's place in it
     const unsigned long long tid_z = counter_of(done, seed);
     unsigned long long z = tid_z + static_cast<unsigned long long>(base / 2) * kGamma;
     load(base + done, len - done);
@@ -657,11 +671,26 @@ quantize_planes_odd_kernel(const T *__restrict__ x, long long nplanes, int hw, i
     const float inv = delta > 0.f ? __fdiv_rn(1.0f, delta) : 0.f;      // Delta = 0: every code 0
     unsigned sat = 0, nz2 = 0, nnz = 0;
     // 16-byte words of the output: of a plane, or of a position
-    const int words = NHWC ? planes_per_run / 8 : pitch / 8, q_plane = kThreads / words, r_plane = kThreads - q_plane * words;
-    const int first_plane = threadIdx.x / words, first_word = threadIdx.x - first_plane * words;
+    int words = pitch / 8, q_plane = 0, r_plane = 0, first_plane = 0, first_word = 0;
+    auto spread = [&]() {
+        q_plane = kThreads / words;
+        r_plane = kThreads - q_plane * words;
+        first_plane = threadIdx.x / words;
+        first_word = threadIdx.x - first_plane * words;
+    };
+    if (!NHWC) spread();
     while (r < nruns) {
         const long long here = base;
         const int now = len;
+        if (NHWC) {
+            image = image_n;
+            c0 = c0_n;
+            if (chans != chans_n) {
+                chans = chans_n;
+                words = chans / 8;
+                spread();
+            }
+        }
         // the run in rounds of 16 elements per thread; after its last one the next run's first is on its way
         while (true) {
             unsigned h[NV][V / 2], m[NV][V], top = 0u;
@@ -684,7 +713,7 @@ quantize_planes_odd_kernel(const T *__restrict__ x, long long nplanes, int hw, i
             if (last) {
                 r += gridDim.x;
                 base += run_e * gridDim.x;
-                len = r < nruns ? run_len(base) : 0;
+                len = r < nruns ? find() : 0;
                 done = threadIdx.x * V;
                 z = tid_z + static_cast<unsigned long long>(base / 2) * kGamma;
             }
@@ -714,9 +743,8 @@ quantize_planes_odd_kernel(const T *__restrict__ x, long long nplanes, int hw, i
         }
         __syncthreads();
         if (NHWC) {
-            const long long plane = here / hw, b = plane / nhwc.C;
-            const int c0 = static_cast<int>(plane - b * nhwc.C), tall = hw + (nhwc.stack ? nhwc.plane_w : 0);
-            unsigned short *dst = out + b * hw * nhwc.C + c0, *to = nhwc.stack + b * tall * nhwc.C + c0;
+            const int tall = hw + (nhwc.stack ? nhwc.plane_w : 0);
+            unsigned short *dst = out + image * hw * nhwc.C + c0, *to = nhwc.stack + image * tall * nhwc.C + c0;
             const unsigned short *src = reinterpret_cast<const unsigned short *>(run_s);
             int pp = first_plane, w = first_word;
             for (int i = threadIdx.x; i < tall * words; i += kThreads) {
@@ -760,7 +788,7 @@ quantize_planes_odd_kernel(const T *__restrict__ x, long long nplanes, int hw, i
 template <typename T, bool NHWC>
 int run_planes_odd(dbp_ctx *ctx, const void *delta, long long nplanes, int hw, int pitch, int per_run, unsigned long long seed,
                    const StepSource &step, void *out, bool count, const uint8_t *mask, const NhwcOut &nhwc) {
-    const long long nruns = (nplanes + per_run - 1) / per_run, cap = static_cast<long long>(ctx->sm_count) * kBlocksPerSM;
+    const long long nruns = NHWC ? nplanes / nhwc.C * ((nhwc.C + per_run - 1) / per_run) : (nplanes + per_run - 1) / per_run, cap = static_cast<long long>(ctx->sm_count) * kBlocksPerSM;
     auto go = [&](auto kern) {
         return cuda_ok(launch_chained(kern, dim3(static_cast<unsigned>(nruns < cap ? nruns : cap)), dim3(kThreads), 0, ctx->stream,
                                       static_cast<const T *>(delta), nplanes, hw, pitch, per_run, seed, step,
@@ -773,16 +801,13 @@ int run_planes_odd(dbp_ctx *ctx, const void *delta, long long nplanes, int hw, i
     return go(quantize_planes_odd_kernel<T, false, NHWC>);
 }
 
-// Channels in a run of the position-major form: as many as fit of the numbers that divide C, at most 64 (a row of the output), but
-// fewer where the runs would not cover the SMs twice. 0: none does.
+// Channels in a run of the position-major form: as many as fit, at most 64 (a row of the output), but fewer (not below 16: 32 bytes
+// of a row) where the runs would not cover the SMs twice. 0: eight do not fit.
 int odd_channels_per_run(long long B, int C, int hw, int sms) {
-    int best = 0;
-    for (int n = 64; n >= 8; n -= 8) {
-        if (C % n != 0 || static_cast<long long>(n) * hw > kOddElems) continue;
-        best = n;
-        if (B * (C / n) >= 2ll * sms) break;
-    }
-    return best;
+    int n = kOddElems / hw / 8 * 8;
+    if (n > 64) n = 64;
+    while (n > 16 && B * ((C + n - 1) / n) < 2ll * sms) n -= 8;
+    return n;
 }
 
 // Planes in a run: as many as fit, in units of a vector's elements, of those numbers the one that leaves the fewest of a round's places empty (a

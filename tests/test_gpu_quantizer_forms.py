@@ -29,6 +29,7 @@ def ctx():
     # ... odd planes: runs of channels of one image, in one round and two; with the copy; channels that are no multiple of 8
     (3, 16, 64, 7, 7, 3, "bf16", False), (2, 24, 96, 13, 13, 3, "bf16", False), (2, 16, 40, 21, 37, 3, "f32", True),
     (9, 16, 72, 3, 5, 3, "f32", True), (2, 16, 30, 7, 7, 3, "f32", True), (1, 16, 24, 33, 41, 3, "bf16", False),
+    (150, 16, 184, 5, 5, 3, "bf16", False), (150, 16, 184, 5, 5, 3, "f32", True),      # ... runs of 64 and 56 channels, two to a block
     # planes at a padded pitch: a multiple of four, odd ones in one round and two, planes too large for a run
     (3, 24, 40, 14, 14, 1, "bf16", False), (7, 16, 72, 2, 6, 1, "bf16", False), (2, 24, 40, 10, 18, 1, "f32", True),
     (5, 16, 72, 7, 7, 1, "bf16", False), (4, 16, 24, 27, 19, 1, "f32", True), (1, 16, 16, 23, 45, 1, "bf16", False),
