@@ -87,9 +87,9 @@ __global__ void __launch_bounds__(256) phases_of_kernel(const T *__restrict__ X,
 // X [planes][H][W] -> bf16 rows for the copy engine, [piece][b][phase * Cin + ci][pitch] (pitch >= H/2 * W/2, a multiple of
 // 8; what lies behind a plane is never read). A thread takes eight consecutive positions of one plane's rows of parity py
 // and writes both column parities' rows (phases = 4; phases = 1: the even rows and columns only). fp32 values leave as two
-// pieces (rounded, and the remainder rounded). VEC: W/2 is a multiple of four, so four positions are one or two vectors.
+// pieces (rounded, and the remainder rounded). VEC: W/2 is a multiple of four, so four positions are one or two vectors. EVEN: of two, so two positions are one.
 // beside: see rows_job_kernel (nsd_kernels.cu).
-template <typename T, bool VEC>
+template <typename T, bool VEC, bool EVEN>
 __global__ void __launch_bounds__(256) phase_rows_kernel(const T *__restrict__ X, unsigned short *__restrict__ out, unsigned planes,
                                                          unsigned Cin, unsigned H, unsigned W, unsigned pitch, int phases, int beside) {
     if (!beside) chain_wait();
@@ -123,12 +123,34 @@ __global__ void __launch_bounds__(256) phase_rows_kernel(const T *__restrict__ X
                 }
 #pragma unroll
                 for (int k = 0; k < 4; ++k) { e[4 * h + k] = v[2 * k]; o[4 * h + k] = v[2 * k + 1]; }
+            } else if (EVEN) {
+                // two positions of a row are one vector; the next two may lie in the next row
+                unsigned y = p4 / Wo, x = p4 - y * Wo;
+#pragma unroll
+                for (int k = 0; k < 4; k += 2) {
+                    float v[4] = {};
+                    if (p4 + k < HW) {
+                        const T *q = src + static_cast<size_t>(2 * y) * W + 2 * x;
+                        if (sizeof(T) == 4) {
+                            const float4 a = __ldg(reinterpret_cast<const float4 *>(q));
+                            v[0] = a.x; v[1] = a.y; v[2] = a.z; v[3] = a.w;
+                        } else {
+                            const uint2 a = __ldg(reinterpret_cast<const uint2 *>(q));
+                            v[0] = __uint_as_float(a.x << 16); v[1] = __uint_as_float(a.x & 0xffff0000u);
+                            v[2] = __uint_as_float(a.y << 16); v[3] = __uint_as_float(a.y & 0xffff0000u);
+                        }
+                    }
+                    e[4 * h + k] = v[0]; o[4 * h + k] = v[1];
+                    e[4 * h + k + 1] = v[2]; o[4 * h + k + 1] = v[3];
+                    x += 2;
+                    if (x == Wo) { x = 0; ++y; }
+                }
             } else {
+                unsigned y = p4 / Wo, x = p4 - y * Wo;
 #pragma unroll
                 for (int k = 0; k < 4; ++k) {
-                    const unsigned pos = p4 + k, y = pos / Wo, x = pos - y * Wo;
                     e[4 * h + k] = o[4 * h + k] = 0.f;
-                    if (pos < HW) {
+                    if (p4 + k < HW) {
                         const T *q = src + static_cast<size_t>(2 * y) * W + 2 * x;
                         if (sizeof(T) == 4) {
                             const float2 a = __ldg(reinterpret_cast<const float2 *>(q));
@@ -138,6 +160,7 @@ __global__ void __launch_bounds__(256) phase_rows_kernel(const T *__restrict__ X
                             e[4 * h + k] = __uint_as_float(a << 16); o[4 * h + k] = __uint_as_float(a & 0xffff0000u);
                         }
                     }
+                    if (++x == Wo) { x = 0; ++y; }
                 }
             }
         }
@@ -263,7 +286,7 @@ int launch_phase_rows(dbp_ctx *ctx, const void *X, void *Xp, int io, long long B
     const long long n = B * Cin * (phases == 1 ? 1 : 2) * (pitch / 8);
     if (!fits32(n) || !fits32(B * Cin)) return DBP_EUNSUPPORTED;
     const int g = blocks_of(n, 256, ctx->sm_count * 8);
-    const bool vec = (W / 2) % 4 == 0;
+    const bool vec = (W / 2) % 4 == 0, even = (W / 2) % 2 == 0;
     auto go = [&](auto kern, auto x) {
         return cuda_ok(launch_chained(kern, dim3(g), dim3(256), 0, ctx->stream, x, static_cast<unsigned short *>(Xp), static_cast<unsigned>(B * Cin),
                                       static_cast<unsigned>(Cin), static_cast<unsigned>(H), static_cast<unsigned>(W),
@@ -271,8 +294,11 @@ int launch_phase_rows(dbp_ctx *ctx, const void *X, void *Xp, int io, long long B
     };
     const float *xf = static_cast<const float *>(X);
     const __nv_bfloat16 *xb = static_cast<const __nv_bfloat16 *>(X);
-    if (io == DBP_F32) return vec ? go(phase_rows_kernel<float, true>, xf) : go(phase_rows_kernel<float, false>, xf);
-    return vec ? go(phase_rows_kernel<__nv_bfloat16, true>, xb) : go(phase_rows_kernel<__nv_bfloat16, false>, xb);
+    if (io == DBP_F32)
+        return vec ? go(phase_rows_kernel<float, true, true>, xf) : even ? go(phase_rows_kernel<float, false, true>, xf) : go(phase_rows_kernel<float, false, false>, xf);
+    return vec    ? go(phase_rows_kernel<__nv_bfloat16, true, true>, xb)
+           : even ? go(phase_rows_kernel<__nv_bfloat16, false, true>, xb)
+                  : go(phase_rows_kernel<__nv_bfloat16, false, false>, xb);
 }
 
 int launch_from_phases(dbp_ctx *ctx, const void *dXp, void *dX, int f32, long long B, long long Cin, int H, int W, int phases) {
