@@ -39,6 +39,21 @@ __device__ __forceinline__ float value_of(__nv_bfloat16 v) { return __bfloat162f
 __device__ __forceinline__ void store_value(float *p, float v) { *p = v; }
 __device__ __forceinline__ void store_value(__nv_bfloat16 *p, float v) { *p = __float2bfloat16_rn(v); }
 
+// What the whole CTA brings into shared memory: a thread's next U values are loaded before the first of them is placed. One by one
+// each waited for its own trip to the L2: the codes of the second layer below were 3 us of this kernel, of the first 4.
+template <int U, typename V, typename F>
+__device__ __forceinline__ void each_of(int n, const V *src, F &&place) {
+    for (int i0 = threadIdx.x; i0 < n; i0 += U * kThreads5) {
+        V v[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u)
+            if (i0 + u * kThreads5 < n) v[u] = src[i0 + u * kThreads5];
+#pragma unroll
+        for (int u = 0; u < U; ++u)
+            if (i0 + u * kThreads5 < n) place(i0 + u * kThreads5, v[u]);
+    }
+}
+
 template <typename T, typename O>
 __global__ void __launch_bounds__(kThreads5)
 direct5_kernel(const Direct5P p) {
@@ -58,17 +73,17 @@ direct5_kernel(const Direct5P p) {
     __syncthreads();
     auto load_x = [&](int b) {
         const T *src = static_cast<const T *>(p.X) + static_cast<long long>(b) * p.Cin * HW;
-        for (int i = tid; i < p.Cin * HW; i += kThreads5) {
+        each_of<4>(p.Cin * HW, src, [&](int i, T v) {
             const int ci = i / HW, r = i - ci * HW, y = r / Wd, x = r - y * Wd;
-            x_s[(ci * Hp + y + 2) * p.pitch + x + 2] = value_of(src[i]);
-        }
+            x_s[(ci * Hp + y + 2) * p.pitch + x + 2] = value_of(v);
+        });
     };
     // the layer's inputs do not depend on the kernel before this one (the quantizer): they come in while it runs
     if (want_dx)
-        for (int i = tid; i < p.Cout * p.Cin * 25; i += kThreads5) {
+        each_of<4>(p.Cout * p.Cin * 25, static_cast<const T *>(p.W), [&](int i, T v) {
             const int t = i % 25, c = i / 25, co = c / p.Cin, ci = c - co * p.Cin;
-            w_s[((co * cip + ci) * 5 + t / 5) * 8 + t % 5] = value_of(static_cast<const T *>(p.W)[i]);
-        }
+            w_s[((co * cip + ci) * 5 + t / 5) * 8 + t % 5] = value_of(v);
+        });
     if (want_dw) load_x(blockIdx.x);
     chain_wait();
     chain_release();
@@ -90,11 +105,25 @@ direct5_kernel(const Direct5P p) {
             if (want_dw) load_x(b);
         }
         const int8_t *src = p.codes + static_cast<long long>(b) * p.Cout * HW;
-        for (int i = tid; i < p.Cout * HW; i += kThreads5) {
-            const int co = i / HW, r = i - co * HW, y = r / Wd, x = r - y * Wd;
-            const float f = static_cast<float>(src[i]);
-            if (want_dx) qa[(co * Hp + y + 2) * p.pitch + x + 2] = f;
-            if (want_dw) qb[(y * Wr + x) * p.cop + co] = f;
+        if ((Wd & 3) == 0) {                                         // four codes of a row at a time
+            const int quads = HW / 4, wq = Wd / 4;
+            each_of<4>(p.Cout * quads, reinterpret_cast<const char4 *>(src), [&](int i, char4 v) {
+                const int co = i / quads, r = i - co * quads, y = r / wq, x = (r - y * wq) * 4;
+                const float f[4] = {static_cast<float>(v.x), static_cast<float>(v.y), static_cast<float>(v.z), static_cast<float>(v.w)};
+                float *const a = qa + (co * Hp + y + 2) * p.pitch + x + 2, *const c = qb + (y * Wr + x) * p.cop + co;
+#pragma unroll
+                for (int k = 0; k < 4; ++k) {
+                    if (want_dx) a[k] = f[k];
+                    if (want_dw) c[k * p.cop] = f[k];
+                }
+            });
+        } else {
+            each_of<8>(p.Cout * HW, src, [&](int i, int8_t v) {
+                const int co = i / HW, r = i - co * HW, y = r / Wd, x = r - y * Wd;
+                const float f = static_cast<float>(v);
+                if (want_dx) qa[(co * Hp + y + 2) * p.pitch + x + 2] = f;
+                if (want_dw) qb[(y * Wr + x) * p.cop + co] = f;
+            });
         }
         __syncthreads();
         if (want_dx) {
