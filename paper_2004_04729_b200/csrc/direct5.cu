@@ -11,8 +11,10 @@
 //       columns two loads of activations, four of codes, 80 FMAs. Its sums stay in registers over the CTA's images; the
 //       row shares are added in shared memory and the copy engine adds the CTA's block into dW (cleared before by the
 //       statistics kernel; the order of the CTAs, hence the last bits of dW, can differ from run to run).
-// LeNet-5-like, batch 128, fp32: second layer (6 -> 16 channels at 16x16, both products) 165 us on the gather kernels, 19 here;
-// first layer (1 -> 6 at 32x32, dW) 111 us there, 11 here.
+// LeNet-5-like, batch 128, fp32: second layer (6 -> 16 channels at 16x16, both products) 165 us on the gather kernels, 19 here
+// with every value loaded and placed before the next; first layer (1 -> 6 at 32x32, dW) 111 us there, 11 here. Loaded ahead and
+// placed in different banks the two are 12 us shorter in the chain of the network's kernels (61.9 -> 49.3 us in all; by themselves
+// they are bound by the FMAs, 5 us of the second layer, and their start and end).
 #include "tc_common.cuh"
 
 namespace dbp {
@@ -30,6 +32,7 @@ struct Direct5P {
     void *dX;
     int B, Cin, Cout, H, Wd;
     int pitch;                    // floats per shared-memory row of an image with its border: W rounded up to 4, plus 4
+    int plane;                    // floats per output channel of the codes with their border: an odd multiple of 4 where that fits
     int cop, co4;                 // output channels rounded up to 4, and a quarter of that
     int rg;                       // row shares of dW
 };
@@ -41,13 +44,13 @@ __device__ __forceinline__ void store_value(__nv_bfloat16 *p, float v) { *p = __
 
 // What the whole CTA brings into shared memory: a thread's next U values are loaded before the first of them is placed. One by one
 // each waited for its own trip to the L2: the codes of the second layer below were 3 us of this kernel, of the first 4.
-template <int U, typename V, typename F>
-__device__ __forceinline__ void each_of(int n, const V *src, F &&place) {
+template <int U, typename V, typename A, typename F>
+__device__ __forceinline__ void each_of(int n, const V *src, A &&at, F &&place) {
     for (int i0 = threadIdx.x; i0 < n; i0 += U * kThreads5) {
         V v[U];
 #pragma unroll
         for (int u = 0; u < U; ++u)
-            if (i0 + u * kThreads5 < n) v[u] = src[i0 + u * kThreads5];
+            if (i0 + u * kThreads5 < n) v[u] = src[at(i0 + u * kThreads5)];
 #pragma unroll
         for (int u = 0; u < U; ++u)
             if (i0 + u * kThreads5 < n) place(i0 + u * kThreads5, v[u]);
@@ -61,26 +64,27 @@ direct5_kernel(const Direct5P p) {
     const int tid = threadIdx.x;
     const int H = p.H, Wd = p.Wd, Wr = p.pitch - 4, Hp = H + 4, HW = H * Wd;
     const bool want_dx = p.dX != nullptr, want_dw = p.dW != nullptr;
-    float *qa = smem5;                                               // [Cout][H + 4][pitch]: codes with a border of zeros (dX)
-    float *w_s = qa + (want_dx ? p.Cout * Hp * p.pitch : 0);         // [Cout][Cin rounded up to 2][5][8] (dX)
+    float *qa = smem5;                                               // [Cout][plane], rows of pitch: codes with a border of zeros (dX)
+    float *w_s = qa + (want_dx ? p.Cout * p.plane : 0);         // [Cout][Cin rounded up to 2][5][8] (dX)
     const int cip = (p.Cin + 1) & ~1;
     float *qb = w_s + (want_dx ? p.Cout * cip * 40 : 0);             // [H][Wr][cop]: codes, channels innermost (dW)
     float *x_s = qb + (want_dw ? H * Wr * p.cop : 0);                // [Cin][H + 4][pitch]: activations with their border (dW)
-    const int total = (want_dx ? p.Cout * (Hp * p.pitch + cip * 40) : 0) + (want_dw ? H * Wr * p.cop + p.Cin * Hp * p.pitch : 0);
+    const int total = (want_dx ? p.Cout * (p.plane + cip * 40) : 0) + (want_dw ? H * Wr * p.cop + p.Cin * Hp * p.pitch : 0);
 
     // borders and padding stay zero; the inside is written for every image
     for (int i = tid; i < total / 4; i += kThreads5) reinterpret_cast<float4 *>(smem5)[i] = make_float4(0.f, 0.f, 0.f, 0.f);
     __syncthreads();
+    auto same = [](int i) { return i; };
     auto load_x = [&](int b) {
         const T *src = static_cast<const T *>(p.X) + static_cast<long long>(b) * p.Cin * HW;
-        each_of<4>(p.Cin * HW, src, [&](int i, T v) {
+        each_of<4>(p.Cin * HW, src, same, [&](int i, T v) {
             const int ci = i / HW, r = i - ci * HW, y = r / Wd, x = r - y * Wd;
             x_s[(ci * Hp + y + 2) * p.pitch + x + 2] = value_of(v);
         });
     };
     // the layer's inputs do not depend on the kernel before this one (the quantizer): they come in while it runs
     if (want_dx)
-        each_of<4>(p.Cout * p.Cin * 25, static_cast<const T *>(p.W), [&](int i, T v) {
+        each_of<4>(p.Cout * p.Cin * 25, static_cast<const T *>(p.W), same, [&](int i, T v) {
             const int t = i % 25, c = i / 25, co = c / p.Cin, ci = c - co * p.Cin;
             w_s[((co * cip + ci) * 5 + t / 5) * 8 + t % 5] = value_of(v);
         });
@@ -105,12 +109,14 @@ direct5_kernel(const Direct5P p) {
             if (want_dw) load_x(b);
         }
         const int8_t *src = p.codes + static_cast<long long>(b) * p.Cout * HW;
-        if ((Wd & 3) == 0) {                                         // four codes of a row at a time
+        if ((Wd & 3) == 0) {
+            // four codes of a row at a time, neighbouring threads on neighbouring channels: their words lie in different banks in
+            // both copies (along a row they lay in two)
             const int quads = HW / 4, wq = Wd / 4;
-            each_of<4>(p.Cout * quads, reinterpret_cast<const char4 *>(src), [&](int i, char4 v) {
-                const int co = i / quads, r = i - co * quads, y = r / wq, x = (r - y * wq) * 4;
+            each_of<4>(p.Cout * quads, reinterpret_cast<const char4 *>(src), [&](int i) { return i % p.Cout * quads + i / p.Cout; }, [&](int i, char4 v) {
+                const int r = i / p.Cout, co = i - r * p.Cout, y = r / wq, x = (r - y * wq) * 4;
                 const float f[4] = {static_cast<float>(v.x), static_cast<float>(v.y), static_cast<float>(v.z), static_cast<float>(v.w)};
-                float *const a = qa + (co * Hp + y + 2) * p.pitch + x + 2, *const c = qb + (y * Wr + x) * p.cop + co;
+                float *const a = qa + co * p.plane + (y + 2) * p.pitch + x + 2, *const c = qb + (y * Wr + x) * p.cop + co;
 #pragma unroll
                 for (int k = 0; k < 4; ++k) {
                     if (want_dx) a[k] = f[k];
@@ -118,10 +124,10 @@ direct5_kernel(const Direct5P p) {
                 }
             });
         } else {
-            each_of<8>(p.Cout * HW, src, [&](int i, int8_t v) {
+            each_of<8>(p.Cout * HW, src, same, [&](int i, int8_t v) {
                 const int co = i / HW, r = i - co * HW, y = r / Wd, x = r - y * Wd;
                 const float f = static_cast<float>(v);
-                if (want_dx) qa[(co * Hp + y + 2) * p.pitch + x + 2] = f;
+                if (want_dx) qa[co * p.plane + (y + 2) * p.pitch + x + 2] = f;
                 if (want_dw) qb[(y * Wr + x) * p.cop + co] = f;
             });
         }
@@ -133,7 +139,7 @@ direct5_kernel(const Direct5P p) {
                 float acc[2][4] = {};
                 for (int co = 0; co < p.Cout; ++co) {
                     // code row y - ky + 2 lies at row y + 4 - ky of the bordered image, column x - kx + 2 at x - kx + 4
-                    const float *q = qa + (co * Hp + y) * p.pitch + x0;
+                    const float *q = qa + co * p.plane + y * p.pitch + x0;
                     const float *w = w_s + (co * cip + c2) * 40;
 #pragma unroll
                     for (int ky = 0; ky < 5; ++ky) {
@@ -215,7 +221,7 @@ direct5_kernel(const Direct5P p) {
 
 int floats5(const Direct5P &p) {
     const int Wr = p.pitch - 4, Hp = p.H + 4, cip = (p.Cin + 1) & ~1;
-    const int tiles = (p.dX ? p.Cout * (Hp * p.pitch + cip * 40) : 0) + (p.dW ? p.H * Wr * p.cop + p.Cin * Hp * p.pitch : 0);
+    const int tiles = (p.dX ? p.Cout * (p.plane + cip * 40) : 0) + (p.dW ? p.H * Wr * p.cop + p.Cin * Hp * p.pitch : 0);
     const int sums = p.dW ? ((p.Cout * p.Cin * 25 + 3) & ~3) + p.rg * p.cop * p.Cin * 25 : 0;
     return tiles > sums ? tiles : sums;
 }
@@ -230,6 +236,11 @@ Direct5P plan5(const ConvShape &s, float *dW, void *dX) {
     p.co4 = p.cop / 4;
     p.rg = kThreads5 / (p.co4 * p.Cin * 5);
     if (p.rg > p.H) p.rg = p.H;
+    p.plane = (p.H + 4) * p.pitch;
+    if (p.plane % 8 == 0) {
+        p.plane += 4;
+        if (floats5(p) > kMaxFloats5) p.plane -= 4;                  // (fits as it is)
+    }
     return p;
 }
 
