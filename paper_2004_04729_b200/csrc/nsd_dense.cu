@@ -25,9 +25,9 @@ constexpr int kBlocksPerSM = 3;                   // resident blocks the dense q
 // Where the codes of the flat quantizer go:
 //   kBytes: one byte per element, same order as delta_z;
 //   kSame:  bf16, same order;
-//   kPad4:  bf16 as [plane][hw + 4], planes of an odd multiple of four elements (so every plane starts on a 16-byte boundary);
-//   kAny:   bf16 as [plane][pitch], planes of any size.
-enum { kBytes, kSame, kPad4, kAny };
+//   kPad4:  bf16 as [plane][hw + 4], planes of an odd multiple of four elements (so every plane starts on a 16-byte boundary).
+// (Planes of other sizes: quantize_rows_kernel.)
+enum { kBytes, kSame, kPad4 };
 struct CodeSinks {
     int8_t *dense8;
     unsigned short *planes16;
@@ -52,29 +52,6 @@ __device__ __forceinline__ void split_index(long long e, long long hw, long long
     }
 }
 
-// kAny: code by code, or two at a time where the pair starts on an even offset of its plane and does not run over the plane's end
-template <int V>
-__device__ __forceinline__ void store_any(const CodeSinks &o, long long e0, const unsigned (&h)[V / 2]) {
-    long long plane, pp;
-    split_index(e0, o.hw, plane, pp);
-    unsigned short *dst = o.planes16 + plane * o.pitch + pp;
-    long long left = o.hw - pp;                           // codes until the plane ends
-    const long long gap = o.pitch - o.hw;
-#pragma unroll
-    for (int j = 0; j < V; j += 2) {
-        if (left >= 2 && (reinterpret_cast<uintptr_t>(dst) & 3) == 0) {
-            *reinterpret_cast<unsigned *>(dst) = h[j >> 1];
-            dst += 2;
-            left -= 2;
-            if (left == 0) { left = o.hw; dst += gap; }
-        } else {
-            *dst++ = static_cast<unsigned short>(h[j >> 1]);
-            if (--left == 0) { left = o.hw; dst += gap; }
-            *dst++ = static_cast<unsigned short>(h[j >> 1] >> 16);
-            if (--left == 0) { left = o.hw; dst += gap; }
-        }
-    }
-}
 __device__ __forceinline__ void store_code(const CodeSinks &o, long long e, unsigned byte) {
     if (o.dense8 != nullptr) o.dense8[e] = static_cast<int8_t>(byte);
     if (o.planes16 != nullptr) {
@@ -167,15 +144,13 @@ quantize_dense_kernel(const T *__restrict__ x, long long n, unsigned long long s
             else *reinterpret_cast<uint2 *>(dst) = make_uint2(pk[0], pk[V / 4 - 1]);
         } else if (SINK == kSame) {
             store_vec<V>(out.planes16 + e + k * kBetween, h);
-        } else if (SINK == kPad4) {
+        } else {
             // each group of four codes lies in one plane and starts on an 8-byte boundary there
             *reinterpret_cast<uint2 *>(po) = make_uint2(h[0], h[1]);
             if (V == 8) {
                 if (pp + 4 < static_cast<int>(out.hw)) *reinterpret_cast<uint2 *>(po + 4) = make_uint2(h[V / 2 - 2], h[V / 2 - 1]);
                 else *reinterpret_cast<uint2 *>(po + 8) = make_uint2(h[V / 2 - 2], h[V / 2 - 1]);
             }
-        } else {
-            store_any<V>(out, e + k * kBetween, h);
         }
     };
     auto walk = [&](int k) {
@@ -597,17 +572,143 @@ quantize_nhwc_any_kernel(const T *__restrict__ x, int B, int C, int HW, unsigned
 }
 
 // ---------------------------------------------------------------- bf16 planes of odd sizes
-// Planes whose size is no multiple of 4 (7 x 7, 9 x 9, ...) written at a pitch that is a multiple of 8: the codes
-// of eight consecutive elements then belong to unaligned places of one or two planes. A block takes a run of
-// whole planes (as many as a vector has elements, or a multiple, so that the run starts on a 16-byte boundary and on an even
-// element), quantizes it with whole-vector loads as everywhere and keeps the codes as they come, in whole words of shared
-// memory; the output's 16-byte words are put together from them on the way out (five words each, shifted by half a word where
-// the piece starts on an odd element), and leave as one contiguous copy (the padding of a plane is never read by anybody).
-// Placing the codes one by one at their pitch instead took 52 instructions an element: 6.4 M elements of 7 x 7 planes 17.5 us,
-// 12 so.
-// NHWC: the run is a multiple of eight channels of one image (at 472 channels of 5x5 planes runs of eight, the only number that
-// divides them, took 34 us for 1.4 M elements), and leaves position-major: eight channels of a position are
-// eight 16-bit reads, a plane apart (in different banks for odd planes).
+// Planes whose size is no multiple of 4 (7 x 7, 9 x 9, rows of 875 outputs, ...) written at a pitch that is a multiple of 8: the
+// codes of eight consecutive elements then belong to unaligned places of one or two planes. A block takes 4096 consecutive
+// elements, quantizes them with whole-vector loads as everywhere and keeps the codes as they come in shared memory; the output's
+// 16-byte words that start among the first 4088 are put together from them (five 32-bit words each, shifted by half of one where
+// a word starts on an odd element) and leave as one contiguous run. The last eight elements are the next run's first: it counts
+// them. (The padding of a plane is never read by anybody.) Whole planes to a run, and planes of more than 784 elements and odd
+// numbers of them code by code, before: 34 M elements of 53 x 53 planes 80 us.
+constexpr int kRowRun = kThreads * kPerThread, kRowStep = kRowRun - 8;
+
+template <typename T, bool MASKED>
+__global__ void __launch_bounds__(kThreads, kBlocksPerSM)
+quantize_rows_kernel(const T *__restrict__ x, long long n, int hw, int words, unsigned long long seed, const StepSource step,
+                     unsigned short *__restrict__ out, DeviceState *__restrict__ st, int count, const unsigned char *__restrict__ mask) {
+    constexpr int V = Vec<T>::V, NV = kPerThread / V, kBetween = kThreads * V;
+    constexpr unsigned long long kBetweenZ = kBetween / 2 * kGamma;
+    __shared__ __align__(16) unsigned run_s[2][kRowRun / 2 + 8];
+    const long long nruns = (n + kRowStep - 1) / kRowStep;
+    const bool counts_last = static_cast<int>(threadIdx.x) * V + (NV - 1) * kBetween < kRowStep;      // its last vector is not the next run's
+    uint4 raw[NV];
+    unsigned msk[MASKED ? NV : 1];
+    unsigned long long u[NV][V / 2];
+    // a vector that the tensor's end cuts: element by element
+    auto edge = [&](long long e, unsigned &mw) {
+        unsigned w[4] = {0u, 0u, 0u, 0u};
+#pragma unroll
+        for (int j = 0; j < V; ++j)
+            if (e + j < n) {
+                const unsigned b = __float_as_uint(Vec<T>::one(x + e + j));
+                if (V == 4) w[j] = b;
+                else w[j / 2] |= j & 1 ? b : b >> 16;
+            }
+        mw = 0u;
+        if (MASKED)
+            for (int j = 0; j < V && e + j < n; ++j) mw |= static_cast<unsigned>(__ldg(mask + e + j)) << (8 * j);
+        return make_uint4(w[0], w[1], w[2], w[3]);
+    };
+    auto load = [&](long long r) {
+        const long long e = r * kRowStep + threadIdx.x * V;
+        if (r * kRowStep + kRowRun <= n) {
+#pragma unroll
+            for (int k = 0; k < NV; ++k) {
+                raw[k] = Vec<T>::raw(x + e + k * kBetween);
+                if (MASKED) msk[k] = mask_word(mask, e + k * kBetween);
+            }
+        } else {
+#pragma unroll
+            for (int k = 0; k < NV; ++k) {
+                unsigned mw = 0u;
+                raw[k] = edge(e + k * kBetween, mw);
+                if (MASKED) msk[k] = mw;
+            }
+        }
+    };
+    long long r = blockIdx.x;
+    unsigned long long z = counter_of(r * kRowStep + threadIdx.x * V, seed);
+    const unsigned long long stride_z = static_cast<unsigned long long>(gridDim.x) * (kRowStep / 2) * kGamma;
+    auto draw = [&]() {
+#pragma unroll
+        for (int k = 0; k < NV; ++k) dithers_at<V>(z + k * kBetweenZ, u[k]);
+    };
+    load(r);
+    draw();
+    keep_here(u);
+    const StepSource from = step_ahead(step);
+    chain_wait();
+    chain_release();
+    const float delta = step_of<kThreads>(from, st);
+    const float inv = delta > 0.f ? __fdiv_rn(1.0f, delta) : 0.f;      // Delta = 0: every code 0
+    unsigned sat = 0, nz2 = 0, nnz = 0;
+    const int q_plane = kThreads / words, r_word = kThreads - q_plane * words;      // 16-byte words of the output: from a thread's one to its next
+    const int next_rel = q_plane * hw + 8 * r_word, wrap_rel = hw - 8 * words;
+    for (int buf = 0; r < nruns; buf ^= 1) {
+        const long long here = r * kRowStep;
+        unsigned short *const run = reinterpret_cast<unsigned short *>(run_s[buf]);
+        unsigned h[NV][V / 2], top = 0u;
+        const unsigned before = nz2;
+#pragma unroll
+        for (int k = 0; k < NV; ++k) {
+            float v[V];
+            Vec<T>::values(raw[k], v);
+            if (MASKED) apply_mask(msk[k], v);
+            quick_codes<V>(v, u[k], inv, h[k], top);
+            if (k < NV - 1 || counts_last) count_pairs<V>(h[k], nz2);
+        }
+        if (needs_care(top)) {                                         // rare: clip, count, NaN
+            nz2 = before;
+#pragma unroll
+            for (int k = 0; k < NV; ++k) {
+                float v[V];
+                unsigned long long d[V / 2];
+                unsigned mc[V], clipped = 0u;
+                Vec<T>::values(raw[k], v);
+                if (MASKED) apply_mask(msk[k], v);
+                dithers_at<V>(z + k * kBetweenZ, d);
+                careful_codes<V>(v, d, inv, h[k], mc, clipped);
+                if (k < NV - 1 || counts_last) {
+                    sat += clipped;
+                    count_pairs<V>(h[k], nz2);
+                }
+            }
+        }
+        r += gridDim.x;
+        if (r < nruns) load(r);
+#pragma unroll
+        for (int k = 0; k < NV; ++k) store_vec<V>(run + threadIdx.x * V + k * kBetween, h[k]);
+        z += stride_z;
+        if (r < nruns) draw();
+        __syncthreads();
+        // the first output word that starts in the run, and this thread's
+        long long plane, in_plane;
+        split_index(here, hw, plane, in_plane);
+        int w = (static_cast<int>(in_plane) + 7) >> 3, rel = 8 * w - static_cast<int>(in_plane);
+        if (w == words) { w = 0; ++plane; rel = hw - static_cast<int>(in_plane); }
+        uint4 *dst = reinterpret_cast<uint4 *>(out) + plane * words + w + threadIdx.x;
+        const int skip = (w + static_cast<int>(threadIdx.x)) / words, w1 = w + static_cast<int>(threadIdx.x) - skip * words;
+        const int end = static_cast<int>(n - here < kRowStep ? n - here : kRowStep);
+        long long at = rel + static_cast<long long>(skip) * hw + 8 * (w1 - w);
+        for (w = w1; at < end; dst += kThreads) {
+            const int sh = (static_cast<int>(at) & 1) * 16;
+            const unsigned *src = run_s[buf] + (at >> 1);
+            const unsigned v0 = src[0], v1 = src[1], v2 = src[2], v3 = src[3], v4 = src[4];
+            *dst = make_uint4(__funnelshift_r(v0, v1, sh), __funnelshift_r(v1, v2, sh), __funnelshift_r(v2, v3, sh), __funnelshift_r(v3, v4, sh));
+            at += next_rel;
+            w += r_word;
+            if (w >= words) { w -= words; at += wrap_rel; }
+        }
+        // the other buffer is written next; this one again only after the next barrier
+        if (nz2 & 0x80008000u) { nnz += pairs_total(nz2); nz2 = 0; }
+    }
+    nnz += pairs_total(nz2);
+    if (count) publish_counts<kThreads>(nnz, delta > 0.f ? sat : 0u, st, nullptr);
+}
+
+// Position-major planes of odd sizes: a run is a multiple of eight channels of one image (at 472 channels of 5x5 planes runs of eight, the only number that
+// divides them, took 34 us for 1.4 M elements), so that it starts on a 16-byte boundary and on an even element; its codes are kept
+// as they come in whole words of shared memory, and eight channels of a position are eight 16-bit reads, a plane apart (in
+// different banks for odd planes). Placing the codes one by one took 52 instructions an element.
 constexpr int kOddElems = 6272;                   // most elements of a run
 
 struct NhwcOut {
@@ -616,9 +717,9 @@ struct NhwcOut {
     int plane_w;                  // how many
 };
 
-template <typename T, bool MASKED, bool NHWC>
+template <typename T, bool MASKED>
 __global__ void __launch_bounds__(kThreads, kBlocksPerSM)
-quantize_planes_odd_kernel(const T *__restrict__ x, long long nplanes, int hw, int pitch, int planes_per_run,
+quantize_planes_odd_kernel(const T *__restrict__ x, long long nplanes, int hw, int per_run,
                            unsigned long long seed, const StepSource step, unsigned short *__restrict__ out,
                            DeviceState *__restrict__ st, int count, const unsigned char *__restrict__ mask, const NhwcOut nhwc) {
     constexpr int V = Vec<T>::V;
@@ -626,9 +727,9 @@ quantize_planes_odd_kernel(const T *__restrict__ x, long long nplanes, int hw, i
     constexpr int kBetween = kThreads * V;
     constexpr unsigned long long kBetweenZ = kBetween / 2 * kGamma;
     __shared__ __align__(16) unsigned run_s[kOddElems / 2 + 8];
-    // NHWC: a run's channels are of one image, whose last run has what is left of them
-    const int per_image = NHWC ? (nhwc.C + planes_per_run - 1) / planes_per_run : 1;
-    const long long nruns = NHWC ? nplanes / nhwc.C * per_image : (nplanes + planes_per_run - 1) / planes_per_run;
+    // a run's channels are of one image, whose last run has what is left of them
+    const int per_image = (nhwc.C + per_run - 1) / per_run;
+    const long long nruns = nplanes / nhwc.C * per_image;
     uint4 raw[NV];
     unsigned msk[MASKED ? NV : 1];
     unsigned long long u[NV][V / 2];
@@ -644,19 +745,15 @@ quantize_planes_odd_kernel(const T *__restrict__ x, long long nplanes, int hw, i
 #pragma unroll
         for (int k = 0; k < NV; ++k) dithers_at<V>(zz + k * kBetweenZ, u[k]);
     };
-    const long long run_e = static_cast<long long>(planes_per_run) * hw, total = nplanes * hw;
-    long long r = blockIdx.x, base = r * run_e, image = 0;
-    int c0 = 0, chans = 0, image_n = 0, c0_n = 0, chans_n = 0;       // NHWC: the run in hand, and the next one
+    long long r = blockIdx.x, base = 0, image = 0;
+    int c0 = 0, chans = 0, image_n = 0, c0_n = 0, chans_n = 0;       // the run in hand, and the next one
     // run r's first element and its length (a multiple of 8)
     auto find = [&]() {
-        if (NHWC) {
-            image_n = static_cast<int>(r / per_image);
-            c0_n = static_cast<int>(r - static_cast<long long>(image_n) * per_image) * planes_per_run;
-            chans_n = nhwc.C - c0_n < planes_per_run ? nhwc.C - c0_n : planes_per_run;
-            base = (static_cast<long long>(image_n) * nhwc.C + c0_n) * hw;
-            return chans_n * hw;
-        }
-        return static_cast<int>(total - base < run_e ? total - base : run_e);
+        image_n = static_cast<int>(r / per_image);
+        c0_n = static_cast<int>(r - static_cast<long long>(image_n) * per_image) * per_run;
+        chans_n = nhwc.C - c0_n < per_run ? nhwc.C - c0_n : per_run;
+        base = (static_cast<long long>(image_n) * nhwc.C + c0_n) * hw;
+        return chans_n * hw;
     };
     int len = find(), done = threadIdx.x * V;                // elements of the run; the thread's place in it
     const unsigned long long tid_z = counter_of(done, seed);
@@ -670,26 +767,19 @@ quantize_planes_odd_kernel(const T *__restrict__ x, long long nplanes, int hw, i
     const float delta = step_of<kThreads>(from, st);
     const float inv = delta > 0.f ? __fdiv_rn(1.0f, delta) : 0.f;      // Delta = 0: every code 0
     unsigned sat = 0, nz2 = 0, nnz = 0;
-    // 16-byte words of the output: of a plane, or of a position
-    int words = pitch / 8, q_plane = 0, r_plane = 0, first_plane = 0, first_word = 0;
-    auto spread = [&]() {
-        q_plane = kThreads / words;
-        r_plane = kThreads - q_plane * words;
-        first_plane = threadIdx.x / words;
-        first_word = threadIdx.x - first_plane * words;
-    };
-    if (!NHWC) spread();
+    int words = 1, q_pos = 0, r_word = 0, first_pos = 0, first_word = 0;      // 16-byte words of a position
     while (r < nruns) {
         const long long here = base;
         const int now = len;
-        if (NHWC) {
-            image = image_n;
-            c0 = c0_n;
-            if (chans != chans_n) {
-                chans = chans_n;
-                words = chans / 8;
-                spread();
-            }
+        image = image_n;
+        c0 = c0_n;
+        if (chans != chans_n) {
+            chans = chans_n;
+            words = chans / 8;
+            q_pos = kThreads / words;
+            r_word = kThreads - q_pos * words;
+            first_pos = threadIdx.x / words;
+            first_word = threadIdx.x - first_pos * words;
         }
         // the run in rounds of 16 elements per thread; after its last one the next run's first is on its way
         while (true) {
@@ -712,7 +802,6 @@ quantize_planes_odd_kernel(const T *__restrict__ x, long long nplanes, int hw, i
             const bool last = done - static_cast<int>(threadIdx.x) * V >= now;       // uniform
             if (last) {
                 r += gridDim.x;
-                base += run_e * gridDim.x;
                 len = r < nruns ? find() : 0;
                 done = threadIdx.x * V;
                 z = tid_z + static_cast<unsigned long long>(base / 2) * kGamma;
@@ -742,40 +831,24 @@ quantize_planes_odd_kernel(const T *__restrict__ x, long long nplanes, int hw, i
             if (done < now) draw(z);
         }
         __syncthreads();
-        if (NHWC) {
-            const int tall = hw + (nhwc.stack ? nhwc.plane_w : 0);
-            unsigned short *dst = out + image * hw * nhwc.C + c0, *to = nhwc.stack + image * tall * nhwc.C + c0;
-            const unsigned short *src = reinterpret_cast<const unsigned short *>(run_s);
-            int pp = first_plane, w = first_word;
-            for (int i = threadIdx.x; i < tall * words; i += kThreads) {
-                uint4 v = make_uint4(0u, 0u, 0u, 0u);
-                if (pp < hw) {
-                    unsigned k[8];
+        const int tall = hw + (nhwc.stack ? nhwc.plane_w : 0);
+        unsigned short *dst = out + image * hw * nhwc.C + c0, *to = nhwc.stack + image * tall * nhwc.C + c0;
+        const unsigned short *src = reinterpret_cast<const unsigned short *>(run_s);
+        int pp = first_pos, w = first_word;
+        for (int i = threadIdx.x; i < tall * words; i += kThreads) {
+            uint4 v = make_uint4(0u, 0u, 0u, 0u);
+            if (pp < hw) {
+                unsigned k[8];
 #pragma unroll
-                    for (int j = 0; j < 8; ++j) k[j] = src[(8 * w + j) * hw + pp];
-                    v = make_uint4(__byte_perm(k[0], k[1], 0x5410), __byte_perm(k[2], k[3], 0x5410), __byte_perm(k[4], k[5], 0x5410),
-                                   __byte_perm(k[6], k[7], 0x5410));
-                    *reinterpret_cast<uint4 *>(dst + static_cast<long long>(pp) * nhwc.C + 8 * w) = v;
-                }
-                if (nhwc.stack != nullptr) *reinterpret_cast<uint4 *>(to + static_cast<long long>(pp) * nhwc.C + 8 * w) = v;
-                pp += q_plane;
-                w += r_plane;
-                if (w >= words) { w -= words; ++pp; }
+                for (int j = 0; j < 8; ++j) k[j] = src[(8 * w + j) * hw + pp];
+                v = make_uint4(__byte_perm(k[0], k[1], 0x5410), __byte_perm(k[2], k[3], 0x5410), __byte_perm(k[4], k[5], 0x5410),
+                               __byte_perm(k[6], k[7], 0x5410));
+                *reinterpret_cast<uint4 *>(dst + static_cast<long long>(pp) * nhwc.C + 8 * w) = v;
             }
-        } else {
-            const int np = now / hw, n16 = np * words;
-            uint4 *dst = reinterpret_cast<uint4 *>(out + here / hw * pitch);
-            int pl = first_plane, w = first_word;
-            for (int i = threadIdx.x; i < n16; i += kThreads) {
-                const int s = pl * hw + 8 * w, sh = (s & 1) * 16;
-                const unsigned *src = run_s + (s >> 1);
-                const unsigned v0 = src[0], v1 = src[1], v2 = src[2], v3 = src[3], v4 = src[4];
-                dst[i] = make_uint4(__funnelshift_r(v0, v1, sh), __funnelshift_r(v1, v2, sh), __funnelshift_r(v2, v3, sh),
-                                    __funnelshift_r(v3, v4, sh));
-                pl += q_plane;
-                w += r_plane;
-                if (w >= words) { w -= words; ++pl; }
-            }
+            if (nhwc.stack != nullptr) *reinterpret_cast<uint4 *>(to + static_cast<long long>(pp) * nhwc.C + 8 * w) = v;
+            pp += q_pos;
+            w += r_word;
+            if (w >= words) { w -= words; ++pp; }
         }
         if (nz2 & 0x80008000u) { nnz += pairs_total(nz2); nz2 = 0; }
         if (r >= nruns) break;
@@ -785,20 +858,19 @@ quantize_planes_odd_kernel(const T *__restrict__ x, long long nplanes, int hw, i
     nnz += pairs_total(nz2);
     if (count) publish_counts<kThreads>(nnz, delta > 0.f ? sat : 0u, st, nullptr);
 }
-template <typename T, bool NHWC>
-int run_planes_odd(dbp_ctx *ctx, const void *delta, long long nplanes, int hw, int pitch, int per_run, unsigned long long seed,
-                   const StepSource &step, void *out, bool count, const uint8_t *mask, const NhwcOut &nhwc) {
-    const long long nruns = NHWC ? nplanes / nhwc.C * ((nhwc.C + per_run - 1) / per_run) : (nplanes + per_run - 1) / per_run, cap = static_cast<long long>(ctx->sm_count) * kBlocksPerSM;
+template <typename T>
+int run_planes_odd(dbp_ctx *ctx, const void *delta, long long B, int hw, int per_run, unsigned long long seed, const StepSource &step,
+                   void *out, bool count, const uint8_t *mask, const NhwcOut &nhwc) {
+    const long long nruns = B * ((nhwc.C + per_run - 1) / per_run), cap = static_cast<long long>(ctx->sm_count) * kBlocksPerSM;
     auto go = [&](auto kern) {
         return cuda_ok(launch_chained(kern, dim3(static_cast<unsigned>(nruns < cap ? nruns : cap)), dim3(kThreads), 0, ctx->stream,
-                                      static_cast<const T *>(delta), nplanes, hw, pitch, per_run, seed, step,
-                                      static_cast<unsigned short *>(out), ctx->state, count ? 1 : 0,
-                                      static_cast<const unsigned char *>(mask), nhwc));
+                                      static_cast<const T *>(delta), B * nhwc.C, hw, per_run, seed, step, static_cast<unsigned short *>(out),
+                                      ctx->state, count ? 1 : 0, static_cast<const unsigned char *>(mask), nhwc));
     };
     if constexpr (sizeof(T) == 4) {
-        if (mask != nullptr) return go(quantize_planes_odd_kernel<T, true, NHWC>);
+        if (mask != nullptr) return go(quantize_planes_odd_kernel<T, true>);
     }
-    return go(quantize_planes_odd_kernel<T, false, NHWC>);
+    return go(quantize_planes_odd_kernel<T, false>);
 }
 
 // Channels in a run of the position-major form: as many as fit, at most 64 (a row of the output), but fewer (not below 16: 32 bytes
@@ -808,20 +880,6 @@ int odd_channels_per_run(long long B, int C, int hw, int sms) {
     if (n > 64) n = 64;
     while (n > 16 && B * ((C + n - 1) / n) < 2ll * sms) n -= 8;
     return n;
-}
-
-// Planes in a run: as many as fit, in units of a vector's elements, of those numbers the one that leaves the fewest of a round's places empty (a
-// round is 4096 elements), but not so many that the blocks would not cover the SMs twice.
-int odd_planes_per_run(long long nplanes, int hw, int unit, int sms) {
-    int best = 0;
-    double best_eff = 0.0;
-    for (int np = unit; static_cast<long long>(np) * hw <= kOddElems; np += unit) {
-        if (best && (nplanes + np - 1) / np < 2 * sms) break;
-        const int e = np * hw, rounds = (e + kThreads * kPerThread - 1) / (kThreads * kPerThread);
-        const double eff = static_cast<double>(e) / rounds;
-        if (eff >= best_eff) { best = np; best_eff = eff; }
-    }
-    return best;
 }
 
 }  // namespace
@@ -836,14 +894,17 @@ int launch_quantize_dense(dbp_ctx *ctx, const void *delta, int dtype, long long 
     const float *xf = static_cast<const float *>(delta);
     const __nv_bfloat16 *xb = static_cast<const __nv_bfloat16 *>(delta);
     if ((dense != nullptr) == (planes != nullptr)) return DBP_EINVAL;          // one form a call
-    // odd plane sizes at a padded pitch: whole runs of planes through shared memory
-    if (planes != nullptr && hw > 0 && pitch != hw && (hw & 3) != 0 && numel % hw == 0 && (numel / hw) % v == 0 && v * hw <= kOddElems &&
-        pitch % 8 == 0 && pitch - hw < 8) {
-        const long long nplanes = numel / hw;
-        const int per_run = odd_planes_per_run(nplanes, static_cast<int>(hw), v, ctx->sm_count);
-        const int h = static_cast<int>(hw), pt = static_cast<int>(pitch);
-        return dtype != DBP_F32 ? run_planes_odd<__nv_bfloat16, false>(ctx, delta, nplanes, h, pt, per_run, seed, step, planes, count, mask, {})
-                                : run_planes_odd<float, false>(ctx, delta, nplanes, h, pt, per_run, seed, step, planes, count, mask, {});
+    // rows of the output start on 16-byte boundaries
+    if (planes != nullptr && pitch != hw && (hw <= 0 || hw >= (1 << 30) || numel % hw != 0 || pitch != (hw + 7) / 8 * 8)) return DBP_EINVAL;
+    if (planes != nullptr && pitch != hw && (hw & 3) != 0) {
+        const long long nruns = (numel + kRowStep - 1) / kRowStep, most = static_cast<long long>(ctx->sm_count) * kBlocksPerSM;
+        auto rows = [&](auto kern, auto x) {
+            return cuda_ok(launch_chained(kern, dim3(static_cast<unsigned>(nruns < most ? nruns : most)), dim3(kThreads), 0, ctx->stream, x, numel,
+                                          static_cast<int>(hw), static_cast<int>(pitch / 8), seed, step, planes, ctx->state, count ? 1 : 0, m));
+        };
+        return dtype != DBP_F32 ? rows(quantize_rows_kernel<__nv_bfloat16, false>, xb)
+               : m              ? rows(quantize_rows_kernel<float, true>, xf)
+                                : rows(quantize_rows_kernel<float, false>, xf);
     }
     constexpr int kTile = kThreads * kPerThread;
     long long blocks = (numel / v * v + kTile - 1) / kTile;
@@ -861,7 +922,7 @@ int launch_quantize_dense(dbp_ctx *ctx, const void *delta, int dtype, long long 
     out.rest2 = static_cast<int>(next % out.hw);
     out.dist1 = between / out.hw * out.pitch + out.rest1;
     out.dist2 = next / out.hw * out.pitch + out.rest2;
-    const int sink = dense ? kBytes : out.pitch == out.hw ? kSame : (out.hw & 7) == 4 && out.pitch == out.hw + 4 && out.hw < (1 << 30) ? kPad4 : kAny;
+    const int sink = dense ? kBytes : out.pitch == out.hw ? kSame : kPad4;
     auto go = [&](auto kern, auto x) {
         return cuda_ok(launch_chained(kern, dim3(static_cast<unsigned>(blocks)), dim3(kThreads), 0, ctx->stream, x, numel, seed, step, out,
                                       ctx->state, m));
@@ -875,8 +936,7 @@ int launch_quantize_dense(dbp_ctx *ctx, const void *delta, int dtype, long long 
     switch (sink) {
         case kBytes: return pick(std::integral_constant<int, kBytes>());
         case kSame: return pick(std::integral_constant<int, kSame>());
-        case kPad4: return pick(std::integral_constant<int, kPad4>());
-        default: return pick(std::integral_constant<int, kAny>());
+        default: return pick(std::integral_constant<int, kPad4>());
     }
 }
 
@@ -898,8 +958,8 @@ int launch_quantize_nhwc(dbp_ctx *ctx, const void *delta, int dtype, long long B
     if (c % 8 == 0) {
         if (const int n = odd_channels_per_run(B, c, hw, ctx->sm_count)) {
             const NhwcOut nh{c, static_cast<unsigned short *>(codes_stack), plane_w};
-            return dtype != DBP_F32 ? run_planes_odd<__nv_bfloat16, true>(ctx, delta, B * C, hw, 8, n, seed, step, codes_nhwc, count, mask, nh)
-                                    : run_planes_odd<float, true>(ctx, delta, B * C, hw, 8, n, seed, step, codes_nhwc, count, mask, nh);
+            return dtype != DBP_F32 ? run_planes_odd<__nv_bfloat16>(ctx, delta, B, hw, n, seed, step, codes_nhwc, count, mask, nh)
+                                    : run_planes_odd<float>(ctx, delta, B, hw, n, seed, step, codes_nhwc, count, mask, nh);
         }
     }
     const long long ntiles = B * ((C + kTC - 1) / kTC) * ((HW + kTP - 1) / kTP), cap = static_cast<long long>(ctx->sm_count) * kBlocksPerSM;

@@ -30,10 +30,13 @@ def ctx():
     (3, 16, 64, 7, 7, 3, "bf16", False), (2, 24, 96, 13, 13, 3, "bf16", False), (2, 16, 40, 21, 37, 3, "f32", True),
     (9, 16, 72, 3, 5, 3, "f32", True), (2, 16, 30, 7, 7, 3, "f32", True), (1, 16, 24, 33, 41, 3, "bf16", False),
     (150, 16, 184, 5, 5, 3, "bf16", False), (150, 16, 184, 5, 5, 3, "f32", True),      # ... runs of 64 and 56 channels, two to a block
-    # planes at a padded pitch: a multiple of four, odd ones in one round and two, planes too large for a run
+    # planes at a padded pitch: a multiple of four, odd ones of less and of more than a run, tensors that end within a vector, second
+    # runs of a block, the smallest
     (3, 24, 40, 14, 14, 1, "bf16", False), (7, 16, 72, 2, 6, 1, "bf16", False), (2, 24, 40, 10, 18, 1, "f32", True),
     (5, 16, 72, 7, 7, 1, "bf16", False), (4, 16, 24, 27, 19, 1, "f32", True), (1, 16, 16, 23, 45, 1, "bf16", False),
     (3, 24, 41, 5, 5, 1, "f32", False), (2, 16, 9, 7, 9, 1, "bf16", False),
+    (9, 16, 7, 59, 59, 1, "bf16", False), (33, 16, 20, 53, 53, 1, "bf16", False), (33, 16, 20, 53, 53, 1, "f32", True),
+    (1, 8, 3, 1, 2, 1, "bf16", False), (1001, 48, 9, 1, 1, 1, "bf16", False), (4003, 72, 463, 1, 1, 1, "f32", True),
     # planes back to back, with a last tile that is not whole and a tail shorter than a vector
     (3, 24, 40, 16, 16, 1, "bf16", False), (2, 16, 24, 24, 20, 1, "f32", True), (300, 200, 90, 1, 1, 1, "f32", True),
     (523, 72, 41, 1, 1, 1, "bf16", False), (600, 260, 257, 1, 1, 1, "f32", False),
