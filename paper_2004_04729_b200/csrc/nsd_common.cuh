@@ -271,6 +271,20 @@ struct Vec<__nv_bfloat16> {
     }
 };
 
+// A vector that the tensor's end cuts: its first `left` elements, the others zero
+template <typename T>
+__device__ __forceinline__ uint4 load_edge(const T *p, long long left) {
+    unsigned w[4] = {0u, 0u, 0u, 0u};
+#pragma unroll
+    for (int j = 0; j < Vec<T>::V; ++j)
+        if (j < left) {
+            const unsigned b = __float_as_uint(Vec<T>::one(p + j));
+            if (Vec<T>::V == 4) w[j] = b;
+            else w[j / 2] |= j & 1 ? b : b >> 16;
+        }
+    return make_uint4(w[0], w[1], w[2], w[3]);
+}
+
 // ---- the step size
 // Every CTA of a quantizer adds up the statistics kernel's partial sums by itself, in the same order, so all hold the
 // same Delta: one L2 round trip at the head of the quantizer instead of an election of a last block, a fence, a ticket

@@ -593,21 +593,6 @@ quantize_rows_kernel(const T *__restrict__ x, long long n, int hw, int words, un
     uint4 raw[NV];
     unsigned msk[MASKED ? NV : 1];
     unsigned long long u[NV][V / 2];
-    // a vector that the tensor's end cuts: element by element
-    auto edge = [&](long long e, unsigned &mw) {
-        unsigned w[4] = {0u, 0u, 0u, 0u};
-#pragma unroll
-        for (int j = 0; j < V; ++j)
-            if (e + j < n) {
-                const unsigned b = __float_as_uint(Vec<T>::one(x + e + j));
-                if (V == 4) w[j] = b;
-                else w[j / 2] |= j & 1 ? b : b >> 16;
-            }
-        mw = 0u;
-        if (MASKED)
-            for (int j = 0; j < V && e + j < n; ++j) mw |= static_cast<unsigned>(__ldg(mask + e + j)) << (8 * j);
-        return make_uint4(w[0], w[1], w[2], w[3]);
-    };
     auto load = [&](long long r) {
         const long long e = r * kRowStep + threadIdx.x * V;
         if (r * kRowStep + kRowRun <= n) {
@@ -619,9 +604,11 @@ quantize_rows_kernel(const T *__restrict__ x, long long n, int hw, int words, un
         } else {
 #pragma unroll
             for (int k = 0; k < NV; ++k) {
-                unsigned mw = 0u;
-                raw[k] = edge(e + k * kBetween, mw);
-                if (MASKED) msk[k] = mw;
+                raw[k] = load_edge(x + e + k * kBetween, n - e - k * kBetween);
+                if (MASKED) {
+                    msk[k] = 0u;
+                    for (int j = 0; j < V && e + k * kBetween + j < n; ++j) msk[k] |= static_cast<unsigned>(__ldg(mask + e + k * kBetween + j)) << (8 * j);
+                }
             }
         }
     };

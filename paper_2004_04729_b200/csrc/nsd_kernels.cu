@@ -340,7 +340,7 @@ __global__ void clear_counts_kernel(DeviceState *st, unsigned long long *nnz_out
 // lane are dumped to shared memory as bytes and the non-zero ones are picked out by walking the word's bits (a few per
 // lane at the sparsities this is used at); the segment leaves as coalesced stores of the 32 words, the 32 offsets and
 // the packed codes. A segment that ends the tensor or holds a code out of range is decided again element by element, so that
-// the others have no branch per vector: 26 instructions an element (16 of them the decision) against 31, the call of 12.8 M bf16
+// the others have no branch per vector (but not in a small tensor, where that is all there is: 9.8 against 8.5 us): 26 instructions an element (16 of them the decision) against 31, the call of 12.8 M bf16
 // elements with its decoding 29.5 us against 31.1.
 constexpr int kLanePitch = 36;                    // bytes between two lanes' codes: an odd number of words
 
@@ -360,13 +360,21 @@ quantize_kernel(const T *__restrict__ x, long long n, unsigned long long seed, c
     unsigned long long z = counter_of(seg * kSegment + lane * 32, seed);
     const unsigned long long stride_z = static_cast<unsigned long long>(nwarps) * (kSegment / 2) * kGamma;
     uint4 raw[NV];
-    auto load = [&](long long sg) {                                  // (a segment that is not whole is read element by element)
+    auto load = [&](long long sg) {
         if (sg >= whole) return;
         const T *src = x + sg * kSegment + lane * 32;
 #pragma unroll
         for (int i = 0; i < NV; ++i) raw[i] = Vec<T>::raw(src + i * V);
     };
     load(seg);
+    // A warp's first segment may be the one that ends the tensor (of a small one; later in the loop it is read element by element)
+    bool ready = seg < nseg;
+    if (ready && seg >= whole) {
+        const long long e = seg * kSegment + lane * 32;
+#pragma unroll
+        for (int i = 0; i < NV; ++i)
+            raw[i] = e + i * V + V <= n ? Vec<T>::raw(x + e + i * V) : load_edge(x + e + i * V, n - e - i * V);      // beyond the end: code 0
+    }
     const StepSource from = step_ahead(step);
     chain_wait();
     chain_release();
@@ -379,7 +387,7 @@ quantize_kernel(const T *__restrict__ x, long long n, unsigned long long seed, c
     for (; seg < nseg; seg += nwarps) {
         const long long e0 = seg * kSegment + lane * 32;
         unsigned word = 0, top = 0u;
-        if (seg < whole) {
+        if (ready) {
 #pragma unroll
             for (int i = 0; i < NV; ++i) {
                 float v[V];
@@ -398,7 +406,7 @@ quantize_kernel(const T *__restrict__ x, long long n, unsigned long long seed, c
         }
         z += stride_z;
         load(seg + nwarps);
-        if (seg >= whole || needs_care(top)) {                       // the last segment; rare: clip, count, NaN
+        if (!ready || needs_care(top)) {                             // the tensor's end; rare: clip, count, NaN
             word = 0;
 #pragma unroll 1
             for (int w = 0; w < 8; ++w) {
@@ -443,6 +451,7 @@ quantize_kernel(const T *__restrict__ x, long long n, unsigned long long seed, c
             *reinterpret_cast<uint4 *>(values + seg * kSegment + i) = *reinterpret_cast<const uint4 *>(&stage[warp][i]);
         __syncwarp();
         nnz += lane == 0 ? total : 0u;
+        ready = seg + nwarps < whole;
     }
     publish_counts<kThreads>(nnz, delta > 0.f ? sat : 0u, st, nnz_out);
 }
