@@ -823,7 +823,7 @@ def main():
         traffic = None if per_step is None else per_step / n_launch
         roof = {"kernel": {"dx_dense": "tensor-core dX (tma_dx_kernel for 1x1, tc3_tma_dx_kernel for 3x3)",
                            "dw_dense": "tensor-core dW (tma_dw_kernel for 1x1, tc3_tma_dw_kernel + tc3_dw_finish_kernel for 3x3)",
-                           "quantize": "NSD quantizer (quantize_dense_kernel / quantize_planes_odd_kernel for 1x1, quantize_nhwc_kernel for 3x3)"}.get(top, top + "_kernel"),
+                           "quantize": "NSD quantizer (quantize_dense_kernel / quantize_rows_kernel for 1x1, quantize_nhwc_kernel / quantize_planes_odd_kernel for 3x3)"}.get(top, top + "_kernel"),
                 "bound": "hbm", "achieved": ach, "peak": hbm_peak, "unit": "GB/s", "frac": ach / hbm_peak,
                 "traffic": traffic, "algorithmic_bytes_per_launch": work[top] / n_launch, "launches_per_step": n_launch,
                 "peak_source": peak_src + " (MEASURED_PEAKS.json hbm_gbs)",

@@ -2,10 +2,10 @@
 // the dense arrays the dX / dW kernels read, without the bitmap / offsets / packed-values structure. Used when the caller
 // did not ask for the sparse structure, so the pass costs one read of delta_z and one write of the codes.
 //
-// What bounds the kernels are instructions: 32 per element of a bf16 tensor (52 for planes of odd sizes), 13 of them the
-// SplitMix64 draw, at 66 % of the issue slots (56 %; 24 warps per SM, which wait for the ALU pipe, for fixed latencies and for
-// their turn) and 0.2 of the memory bandwidth. 12.8 M elements: 22 us, and 16 with the draw left out. So the arithmetic works
-// on pairs (nsd_common.cuh). A thread's first vectors of delta_z and their dithers need
+// What bounds the kernels are instructions: 16 per element are the decision, 11.5 of them the SplitMix64 draw (nsd_common.cuh), so
+// that the rest is kept small: pairs per instruction, addresses and counters by constants, one test for care per tile. 12.8 M
+// bf16 elements: 13.8 us, by vectors with their own bounds and branches 19.1 (32 instructions an element). A thread's first vectors of
+// delta_z and their dithers need
 // nothing of the statistics kernel that runs before: they are loaded and drawn before the wait for it. That is safe
 // because the statistics kernel lets this one start only once all of its own blocks have seen the kernels before it
 // complete. In the loop the next vectors are loaded before the current ones are stored.
@@ -692,10 +692,10 @@ quantize_rows_kernel(const T *__restrict__ x, long long n, int hw, int words, un
     if (count) publish_counts<kThreads>(nnz, delta > 0.f ? sat : 0u, st, nullptr);
 }
 
-// Position-major planes of odd sizes: a run is a multiple of eight channels of one image (at 472 channels of 5x5 planes runs of eight, the only number that
-// divides them, took 34 us for 1.4 M elements), so that it starts on a 16-byte boundary and on an even element; its codes are kept
-// as they come in whole words of shared memory, and eight channels of a position are eight 16-bit reads, a plane apart (in
-// different banks for odd planes). Placing the codes one by one took 52 instructions an element.
+// Position-major planes of odd sizes: a run is a multiple of eight channels of one image, so that it starts on a 16-byte boundary
+// and on an even element (the last run of an image has what is left; at 472 channels of 5x5 planes runs of eight, the only number
+// that divides them, took 34 us for 1.4 M elements); its codes are kept as they come in whole words of shared memory, and eight
+// channels of a position are eight 16-bit reads, a plane apart (in different banks for odd planes). Placing the codes one by one took 52 instructions an element.
 constexpr int kOddElems = 6272;                   // most elements of a run
 
 struct NhwcOut {
