@@ -455,12 +455,11 @@ int conv_backward_impl(dbp_ctx *ctx, const void *delta, const void *X, const voi
     // tiny planes: the weight-gradient kernel reads the images stacked into tall ones
     const int stack_g = (t3 && dW && !ctx->strided) ? tc3_stack_images(s, io) : 0;
     const void *codes_st = nullptr, *codes16 = nullptr, *codes_n = nullptr;
-    int rc = quantize_for_products(ctx, delta, io, numel, seed, scale, delta_in, q_out, &delta_p, &codes, false,
-                                   s.H * s.W, t1 ? tma_code_pitch(s) : 0, t1 ? &codes16 : nullptr,
-                                   t3 ? &s : nullptr, t3 ? &codes_n : nullptr, jobs, stack_g, &codes_st, mask_q);
-    if (rc) return rc;
     // Activations the copy engine cannot address as they are (fp32: two bf16 pieces; planes that are no multiple of 16
-    // bytes; stacked tiny planes) are re-written into the set's own buffer, beside the quantizer. A *_host call's
+    // bytes; stacked tiny planes) are re-written into the set's own buffer: by an overlapped call beside the quantizer, by a
+    // call that ends with its dW on the second stream from the start, where nothing else of the call runs yet (us beside the
+    // quantizer and so: 120 -> 56 fp32, stride 2 at 48x60, batch 8: 51.5, 48.7; bf16 512 -> 512 at 7x7, batch 64: 77.3, 76.0; the
+    // stride-2 layers of ResNet-50 617, 609). A *_host call's
     // activations are still on their way up: there it is done on the stream that waits for them.
     const void *Xp = X;
     long long x_pitch = s.H * s.W;
@@ -474,22 +473,43 @@ int conv_backward_impl(dbp_ctx *ctx, const void *delta, const void *X, const voi
         return stack_g > 0 ? launch_x_stacked(ctx, static_cast<const float *>(X), ctx->x_padded[k].ptr, s, stack_g, beside)
                            : launch_rows_job(ctx, RowsJob{X, ctx->x_padded[k].ptr, io == DBP_F32, s.B * s.Cin, s.H * s.W, x_pitch}, beside);
     };
+    const bool early_x = rewrite_x && forked && !late_x && !(flags & DBP_DW_ASYNC);
+    auto fork = [&]() -> int {
+        return cudaEventRecord(ctx->ev_fork, ctx->stream) == cudaSuccess && cudaStreamWaitEvent(ctx->aux, ctx->ev_fork, 0) == cudaSuccess
+                   ? DBP_OK : fail_cuda("forking the dW stream");
+    };
+    // a call that gives up after the fork: the caller's stream still comes after everything that reads its tensors
+    auto give_up = [&](int r) -> int {
+        if (early_x && cudaEventRecord(ctx->ev_set_free[k], ctx->aux) == cudaSuccess) cudaStreamWaitEvent(ctx->stream, ctx->ev_set_free[k], 0);
+        return r;
+    };
+    int rc = DBP_OK;
     if (rewrite_x) {
         const long long rows = stack_g > 0 ? s.B / stack_g * s.Cin : s.B * s.Cin;
         x_pitch = linear_pitch(stack_g > 0 ? stack_g * (s.H + 1) * s.W : s.H * s.W);
         if ((rc = ws_reserve(ctx, ctx->x_padded[k], static_cast<size_t>(rows) * x_pitch * 2 * pieces))) return rc;
         Xp = ctx->x_padded[k].ptr;
-        // (with a caller's structure the last kernel is not the position-major or plane quantizer's chained launch alone)
-        if (!late_x && (rc = write_x(!q_out))) return rc;
     }
+    if (early_x) {
+        if ((rc = fork())) return rc;
+        cudaStream_t main = ctx->stream;
+        ctx->stream = ctx->aux;
+        rc = write_x(false);
+        ctx->stream = main;
+        if (rc) return give_up(rc);
+    }
+    rc = quantize_for_products(ctx, delta, io, numel, seed, scale, delta_in, q_out, &delta_p, &codes, false,
+                               s.H * s.W, t1 ? tma_code_pitch(s) : 0, t1 ? &codes16 : nullptr,
+                               t3 ? &s : nullptr, t3 ? &codes_n : nullptr, jobs, stack_g, &codes_st, mask_q);
+    if (rc) return give_up(rc);
+    // (with a caller's structure the last kernel is not the position-major or plane quantizer's chained launch alone)
+    if (rewrite_x && !late_x && !early_x && (rc = write_x(!q_out))) return rc;
     read_density();
     // dX and dW read the same codes and nothing of each other: with both asked for, dW goes to the
     // context's second stream, so that its CTAs start as SMs come free instead of after the last dX CTA
     // (forking after the dX kernel instead, which would keep the quantizer -> dX boundary free of stream
     // operations, measured slower: dW then starts a kernel later and meets the next layer's dX)
-    if (forked && (cudaEventRecord(ctx->ev_fork, ctx->stream) != cudaSuccess ||
-                   cudaStreamWaitEvent(ctx->aux, ctx->ev_fork, 0) != cudaSuccess))
-        return fail_cuda("forking the dW stream");
+    if (forked && (rc = fork())) return give_up(rc);
     // A 3x3 call that ends with its dW: where dX is one round of CTAs, its kernel and the dW kernel take half of every SM each
     // and run beside one another, so that one's start and end (loads, partial sums, stores) lie beside the other's MMAs. Of 154
     // layers on both sides of one round (planes 7 to 56 wide, 32 to 256 channels in, 32 to 512 out, both types) 84 share;
@@ -503,19 +523,19 @@ int conv_backward_impl(dbp_ctx *ctx, const void *delta, const void *X, const voi
         KernelTimer t(ctx, DBP_K_DX_DENSE);
         rc = t1 ? launch_tma_dx(ctx, codes16, W, pieces, w_pitch, delta_p, s, dX, dx_bf16, &ctx->state->tc_timeout)
                 : launch_tc3_tma_dx(ctx, codes_n, W, io, delta_p, s, dX, dx_bf16, &ctx->state->tc_timeout, w_side, share ? &half : nullptr);
-        if (rc) return rc;
+        if (rc) return give_up(rc);
     }
     if (dX && st2) {                             // from the phase images to the layer's own dX, beside the dW kernels
         KernelTimer t(ctx, DBP_K_GLUE);
         rc = launch_from_phases(ctx, dX, st2->dX, st2->dx_f32, s.B, st2->Cin, st2->H, st2->W, st2->phases);
-        if (rc) return rc;
+        if (rc) return give_up(rc);
     }
-    if (ctx->hook_after_dx && cudaEventRecord(ctx->hook_after_dx, ctx->stream) != cudaSuccess) return DBP_ECUDA;
+    if (ctx->hook_after_dx && cudaEventRecord(ctx->hook_after_dx, ctx->stream) != cudaSuccess) return give_up(DBP_ECUDA);
     if (db && dX) {
         KernelTimer t(ctx, DBP_K_DB);
         rc = t1 ? launch_plane_sums(ctx, codes16, s.B, s.Cout, s.H * s.W, tma_code_pitch(s), delta_p, db, !ctx->hook_after_dx)
                 : launch_column_sums(ctx, codes_n, s.B * s.H * s.W, s.Cout, delta_p, db, !ctx->hook_after_dx);
-        if (rc) return rc;
+        if (rc) return give_up(rc);
     }
     cudaStream_t caller = ctx->stream;
     if (forked) ctx->stream = ctx->aux;          // the dW launchers enqueue on the context's stream
