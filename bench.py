@@ -493,7 +493,7 @@ def crossover_sweep(torch, dbp, ctx):
 
 # DRAM bytes (read + written) of one config-5 bench step's launches of each kernel kind, from the ncu capture summarised
 # in profiles/bench_step_config5_launch_list.md; None = the kernels of that kind changed after the capture
-NCU_DRAM_BYTES_PER_STEP = {"statistics": 1152359936, "quantize": 740692480, "dx_dense": 745508864, "dw_dense": 1503840768}
+NCU_DRAM_BYTES_PER_STEP = {"statistics": 1153780736, "quantize": 720554752, "dx_dense": 745198336, "dw_dense": 1504653056}
 
 
 def main():
