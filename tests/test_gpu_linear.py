@@ -55,3 +55,14 @@ def test_both_products_and_the_bias_gradient(ctx, dtype, B, N, K):
     if dtype == "bf16":
         low = dbp.dithered_linear_backward(ctx, d, X, W, L.seed, L.scale)
         assert torch.equal(low["dX"], out["dX"].to(torch.bfloat16))
+
+
+@pytest.mark.parametrize("B,N,K", [(1198, 241, 1992), (1089, 456, 1344), (2602, 548, 816), (64, 100, 72)])
+def test_weight_gradients_of_one_or_two_parts_are_the_same_bits_every_time(ctx, B, N, K):
+    """Layers whose estimate hardly differs between more and fewer parts, and one of one part."""
+    import paper_2004_04729_b200 as dbp
+    rng = np.random.default_rng(B)
+    d, X, W = (torch.from_numpy(rng.standard_normal(s).astype(np.float32)).bfloat16().cuda() for s in ((B, N), (B, K), (N, K)))
+    outs = [dbp.dithered_linear_backward(ctx, d, X, W, 3, 2.0)["dW"] for _ in range(12)]
+    for dW in outs[1:]:
+        assert torch.equal(dW, outs[0])
