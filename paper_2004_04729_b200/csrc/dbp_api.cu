@@ -459,7 +459,7 @@ int conv_backward_impl(dbp_ctx *ctx, const void *delta, const void *X, const voi
     // bytes; stacked tiny planes) are re-written into the set's own buffer: by an overlapped call beside the quantizer, by a
     // call that ends with its dW on the second stream from the start, where nothing else of the call runs yet (us beside the
     // quantizer and so: 120 -> 56 fp32, stride 2 at 48x60, batch 8: 51.5, 48.7; bf16 512 -> 512 at 7x7, batch 64: 77.3, 76.0; the
-    // stride-2 layers of ResNet-50 617, 609). A *_host call's
+    // stride-2 layers of ResNet-50 617, 609), unless an earlier call's dW may still lie in front of it there. A *_host call's
     // activations are still on their way up: there it is done on the stream that waits for them.
     const void *Xp = X;
     long long x_pitch = s.H * s.W;
@@ -473,7 +473,7 @@ int conv_backward_impl(dbp_ctx *ctx, const void *delta, const void *X, const voi
         return stack_g > 0 ? launch_x_stacked(ctx, static_cast<const float *>(X), ctx->x_padded[k].ptr, s, stack_g, beside)
                            : launch_rows_job(ctx, RowsJob{X, ctx->x_padded[k].ptr, io == DBP_F32, s.B * s.Cin, s.H * s.W, x_pitch}, beside);
     };
-    const bool early_x = rewrite_x && forked && !late_x && !(flags & DBP_DW_ASYNC);
+    const bool early_x = rewrite_x && forked && !late_x && !(flags & DBP_DW_ASYNC) && !ctx->aux_pending;
     auto fork = [&]() -> int {
         return cudaEventRecord(ctx->ev_fork, ctx->stream) == cudaSuccess && cudaStreamWaitEvent(ctx->aux, ctx->ev_fork, 0) == cudaSuccess
                    ? DBP_OK : fail_cuda("forking the dW stream");
