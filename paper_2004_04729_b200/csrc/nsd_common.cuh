@@ -223,16 +223,6 @@ __device__ __forceinline__ void low_bytes(const unsigned (&m)[V], unsigned (&pk)
     for (int w = 0; w < V / 4; ++w)
         pk[w] = __byte_perm(__byte_perm(m[4 * w], m[4 * w + 1], 0x0040), __byte_perm(m[4 * w + 2], m[4 * w + 3], 0x0040), 0x5410);
 }
-// the codes' bytes, four to a word in element order
-template <int V>
-__device__ __forceinline__ void pack_bytes(const float (&f)[V], unsigned (&pk)[V / 4]) {
-    unsigned b[V];
-#pragma unroll
-    for (int j = 0; j < V; ++j) b[j] = __float_as_uint(f[j] + kMagic);     // low byte: the code
-#pragma unroll
-    for (int w = 0; w < V / 4; ++w)
-        pk[w] = __byte_perm(__byte_perm(b[4 * w], b[4 * w + 1], 0x0040), __byte_perm(b[4 * w + 2], b[4 * w + 3], 0x0040), 0x5410);
-}
 // non-zero codes of the even and of the odd elements, counted in the halves of a word (a code's bf16 bits are zero only
 // for code 0); add up to 65535 of each before reading it with `pairs_total`
 template <int V>

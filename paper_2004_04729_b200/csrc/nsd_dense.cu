@@ -501,7 +501,7 @@ template <typename T, bool MASKED>
 __global__ void __launch_bounds__(kThreads, kBlocksPerSM)
 quantize_nhwc_any_kernel(const T *__restrict__ x, int B, int C, int HW, unsigned long long seed, const StepSource step,
                          unsigned short *__restrict__ out, DeviceState *__restrict__ st, int count,
-                         unsigned short *__restrict__ out_stack, int plane_w, const unsigned char *__restrict__ mask) {
+                         const unsigned char *__restrict__ mask) {
     __shared__ __align__(16) unsigned char tile[2][kTileBytes];
     constexpr int V = Vec<T>::V;
     const unsigned ct = (C + kTC - 1) / kTC, pt = (HW + kTP - 1) / kTP, per_img = ct * pt, ntiles = B * per_img;
@@ -558,11 +558,6 @@ quantize_nhwc_any_kernel(const T *__restrict__ x, int B, int C, int HW, unsigned
             if (p0 + pp < HW && c0 + ch * 8 < C)
                 *reinterpret_cast<uint4 *>(out + (static_cast<long long>(b) * HW + p0 + pp) * pitch + c0 + ch * 8) =
                     *reinterpret_cast<const uint4 *>(tl + tile_off<8>(pp, ch * 8));
-            if (out_stack != nullptr && pp < HW + plane_w && c0 + ch * 8 < C) {     // (planes of less than a tile: see above)
-                const uint4 val = pp < HW ? *reinterpret_cast<const uint4 *>(tl + tile_off<8>(pp, ch * 8)) : make_uint4(0u, 0u, 0u, 0u);
-                const long long row = static_cast<long long>(b) * (HW + plane_w) + pp;
-                *reinterpret_cast<uint4 *>(out_stack + row * C + c0 + ch * 8) = val;
-            }
         }
         // the other buffer is written next; this one again only after the next barrier
         if (nz2 & 0x80008000u) { nnz += pairs_total(nz2); nz2 = 0; }
@@ -953,7 +948,7 @@ int launch_quantize_nhwc(dbp_ctx *ctx, const void *delta, int dtype, long long B
     auto go = [&](auto kern, auto x) {
         return cuda_ok(launch_chained(kern, dim3(static_cast<unsigned>(ntiles < cap ? ntiles : cap)), dim3(kThreads), 0, ctx->stream, x, b, c,
                                       hw, seed, step, static_cast<unsigned short *>(codes_nhwc), ctx->state, count ? 1 : 0,
-                                      static_cast<unsigned short *>(codes_stack), plane_w, static_cast<const unsigned char *>(mask)));
+                                      static_cast<const unsigned char *>(mask)));
     };
     const float *xf = static_cast<const float *>(delta);
     return dtype != DBP_F32 ? go(quantize_nhwc_any_kernel<__nv_bfloat16, false>, static_cast<const __nv_bfloat16 *>(delta))
