@@ -705,7 +705,9 @@ quantize_planes_odd_kernel(const T *__restrict__ x, long long nplanes, int hw, i
                            unsigned long long seed, const StepSource step, unsigned short *__restrict__ out,
                            DeviceState *__restrict__ st, int count, const unsigned char *__restrict__ mask, const NhwcOut nhwc) {
     constexpr int V = Vec<T>::V;
-    constexpr int NV = kPerThread / V;                              // vectors in hand per thread
+    // Vectors in hand per thread. 16 elements of fp32 spill 68 bytes (132 with a mask): calls of 64 -> 64 at 27x27, batch 128, take 83.6
+    // us with them and 80.1 with eight (masked 89.7, 83.1); 64 -> 512 at 5x5, batch 300, 66.0 and 61.7 (71.7, 63.9)
+    constexpr int NV = (V == 4 ? kPerThread / 2 : kPerThread) / V;
     constexpr int kBetween = kThreads * V;
     constexpr unsigned long long kBetweenZ = kBetween / 2 * kGamma;
     __shared__ __align__(16) unsigned run_s[kOddElems / 2 + 8];
@@ -763,9 +765,9 @@ quantize_planes_odd_kernel(const T *__restrict__ x, long long nplanes, int hw, i
             first_pos = threadIdx.x / words;
             first_word = threadIdx.x - first_pos * words;
         }
-        // the run in rounds of 16 elements per thread; after its last one the next run's first is on its way
+        // the run in rounds of NV vectors per thread; after its last one the next run's first is on its way
         while (true) {
-            unsigned h[NV][V / 2], m[NV][V], top = 0u;
+            unsigned h[NV][V / 2], top = 0u;
             const unsigned before = nz2;
             const int at = done, left = now - at;
             const unsigned long long zz = z;
@@ -775,7 +777,7 @@ quantize_planes_odd_kernel(const T *__restrict__ x, long long nplanes, int hw, i
                     float v[V];
                     Vec<T>::values(raw[k], v);
                     if (MASKED) apply_mask(msk[k], v);
-                    quick_codes<V>(v, u[k], inv, h[k], m[k], top);
+                    quick_codes<V>(v, u[k], inv, h[k], top);
                     count_pairs<V>(h[k], nz2);
                 }
             }
