@@ -23,6 +23,7 @@ namespace {
 
 constexpr int kThreads5 = 512;
 constexpr int kMaxFloats5 = 56 * 1024;             // shared memory of a CTA
+constexpr int kHalfFloats5 = (228 / 2 - 1) * 256;  // and of one of two on an SM
 
 struct Direct5P {
     const int8_t *codes;          // [B][Cout][H][W]
@@ -46,6 +47,7 @@ __device__ __forceinline__ void store_value(__nv_bfloat16 *p, float v) { *p = __
 // each waited for its own trip to the L2: the codes of the second layer below were 3 us of this kernel, of the first 4.
 template <int U, typename V, typename A, typename F>
 __device__ __forceinline__ void each_of(int n, const V *src, A &&at, F &&place) {
+#pragma unroll 1
     for (int i0 = threadIdx.x; i0 < n; i0 += U * kThreads5) {
         V v[U];
 #pragma unroll
@@ -57,9 +59,11 @@ __device__ __forceinline__ void each_of(int n, const V *src, A &&at, F &&place) 
     }
 }
 
-template <typename T, typename O>
-__global__ void __launch_bounds__(kThreads5)
+// CTAS: how many share an SM: two in half the registers, with two values in flight per thread in place of four or eight.
+template <typename T, typename O, int CTAS>
+__global__ void __launch_bounds__(kThreads5, CTAS)
 direct5_kernel(const Direct5P p) {
+    constexpr int U = CTAS == 2 ? 2 : 4, UB = CTAS == 2 ? 2 : 8;
     extern __shared__ __align__(16) float smem5[];
     const int tid = threadIdx.x;
     const int H = p.H, Wd = p.Wd, Wr = p.pitch - 4, Hp = H + 4, HW = H * Wd;
@@ -77,14 +81,14 @@ direct5_kernel(const Direct5P p) {
     auto same = [](int i) { return i; };
     auto load_x = [&](int b) {
         const T *src = static_cast<const T *>(p.X) + static_cast<long long>(b) * p.Cin * HW;
-        each_of<4>(p.Cin * HW, src, same, [&](int i, T v) {
+        each_of<U>(p.Cin * HW, src, same, [&](int i, T v) {
             const int ci = i / HW, r = i - ci * HW, y = r / Wd, x = r - y * Wd;
             x_s[(ci * Hp + y + 2) * p.pitch + x + 2] = value_of(v);
         });
     };
     // the layer's inputs do not depend on the kernel before this one (the quantizer): they come in while it runs
     if (want_dx)
-        each_of<4>(p.Cout * p.Cin * 25, static_cast<const T *>(p.W), same, [&](int i, T v) {
+        each_of<U>(p.Cout * p.Cin * 25, static_cast<const T *>(p.W), same, [&](int i, T v) {
             const int t = i % 25, c = i / 25, co = c / p.Cin, ci = c - co * p.Cin;
             w_s[((co * cip + ci) * 5 + t / 5) * 8 + t % 5] = value_of(v);
         });
@@ -113,7 +117,7 @@ direct5_kernel(const Direct5P p) {
             // four codes of a row at a time, neighbouring threads on neighbouring channels: their words lie in different banks in
             // both copies (along a row they lay in two)
             const int quads = HW / 4, wq = Wd / 4;
-            each_of<4>(p.Cout * quads, reinterpret_cast<const char4 *>(src), [&](int i) { return i % p.Cout * quads + i / p.Cout; }, [&](int i, char4 v) {
+            each_of<U>(p.Cout * quads, reinterpret_cast<const char4 *>(src), [&](int i) { return i % p.Cout * quads + i / p.Cout; }, [&](int i, char4 v) {
                 const int r = i / p.Cout, co = i - r * p.Cout, y = r / wq, x = (r - y * wq) * 4;
                 const float f[4] = {static_cast<float>(v.x), static_cast<float>(v.y), static_cast<float>(v.z), static_cast<float>(v.w)};
                 float *const a = qa + co * p.plane + (y + 2) * p.pitch + x + 2, *const c = qb + (y * Wr + x) * p.cop + co;
@@ -124,7 +128,7 @@ direct5_kernel(const Direct5P p) {
                 }
             });
         } else {
-            each_of<8>(p.Cout * HW, src, same, [&](int i, int8_t v) {
+            each_of<UB>(p.Cout * HW, src, same, [&](int i, int8_t v) {
                 const int co = i / HW, r = i - co * HW, y = r / Wd, x = r - y * Wd;
                 const float f = static_cast<float>(v);
                 if (want_dx) qa[co * p.plane + (y + 2) * p.pitch + x + 2] = f;
@@ -260,16 +264,20 @@ int launch_direct5(dbp_ctx *ctx, const int8_t *codes, const void *X, const void 
     Direct5P p = plan5(s, dW, dX);
     p.codes = codes; p.X = X; p.W = W; p.delta_p = delta_p;
     const int smem = floats5(p) * 4;
-    // two CTAs per SM where there are images for them
-    const long long cap = 2ll * ctx->sm_count;
+    // dW by itself with more images than SMs: two CTAs on an SM. A CTA that also makes dX is bound by its FMAs, which want the
+    // registers of a whole SM; it keeps one to itself, for all of its images in turn. us by one, two: 1 -> 6 at 32x32, dW, batch 150:
+    // 16.6, 15.2; 300: 21.5, 19.0; 600: 32.8, 27.3. 6 -> 16 at 16x16, both products, batch 150: 32.6, 34.9; 300: 45.3, 57.9; 600: 71.8, 72.2.
+    const bool two = dX == nullptr && s.B > ctx->sm_count && floats5(p) <= kHalfFloats5;
+    const long long cap = (two ? 2ll : 1ll) * ctx->sm_count;
     const unsigned grid = static_cast<unsigned>(s.B < cap ? s.B : cap);
     auto go = [&](auto kern) -> int {
         if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxFloats5 * 4) != cudaSuccess)
             return fail_cuda("shared memory size");
         return cuda_ok(launch_chained(kern, dim3(grid), dim3(kThreads5), static_cast<size_t>(smem), ctx->stream, p));
     };
-    if (io == DBP_F32) return go(direct5_kernel<float, float>);
-    return dx_bf16 ? go(direct5_kernel<__nv_bfloat16, __nv_bfloat16>) : go(direct5_kernel<__nv_bfloat16, float>);
+    if (two) return io == DBP_F32 ? go(direct5_kernel<float, float, 2>) : go(direct5_kernel<__nv_bfloat16, float, 2>);
+    if (io == DBP_F32) return go(direct5_kernel<float, float, 1>);
+    return dx_bf16 ? go(direct5_kernel<__nv_bfloat16, __nv_bfloat16, 1>) : go(direct5_kernel<__nv_bfloat16, float, 1>);
 }
 
 }  // namespace dbp

@@ -48,3 +48,10 @@ def test_layers_of_few_channels(ctx, B, Ci, Co, H, W, dtype):
         assert np.all(np.abs(g - ref[key]) <= TOL * ref["S_" + key] + 1e-30), key
     assert torch.equal(call(need_dW=False)["dX"], out["dX"])
     assert (call(need_dX=False)["dW"] - out["dW"]).abs().max().item() <= 1e-5 * out["dW"].abs().max().item() + 1e-30
+
+
+@pytest.mark.parametrize("B,Ci,Co,H,W,dtype", [
+    (149, 6, 16, 16, 16, "f32"), (310, 6, 16, 16, 16, "bf16"), (160, 1, 6, 32, 32, "f32"), (301, 3, 5, 7, 9, "f32"),
+    (150, 12, 32, 18, 18, "f32"), (299, 2, 16, 9, 12, "bf16")])
+def test_more_images_than_sms(ctx, B, Ci, Co, H, W, dtype):
+    test_layers_of_few_channels(ctx, B, Ci, Co, H, W, dtype)
