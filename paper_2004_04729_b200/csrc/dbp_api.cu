@@ -456,11 +456,15 @@ int conv_backward_impl(dbp_ctx *ctx, const void *delta, const void *X, const voi
     const int stack_g = (t3 && dW && !ctx->strided) ? tc3_stack_images(s, io) : 0;
     const void *codes_st = nullptr, *codes16 = nullptr, *codes_n = nullptr;
     // Activations the copy engine cannot address as they are (fp32: two bf16 pieces; planes that are no multiple of 16
-    // bytes; stacked tiny planes) are re-written into the set's own buffer: by an overlapped call beside the quantizer, by a
-    // call that ends with its dW on the second stream from the start, where nothing else of the call runs yet (us beside the
-    // quantizer and so: 120 -> 56 fp32, stride 2 at 48x60, batch 8: 51.5, 48.7; bf16 512 -> 512 at 7x7, batch 64: 77.3, 76.0; the
-    // stride-2 layers of ResNet-50 617, 609), unless an earlier call's dW may still lie in front of it there. A *_host call's
-    // activations are still on their way up: there it is done on the stream that waits for them.
+    // bytes; stacked tiny planes) are re-written into the set's own buffer: beside the quantizer, or by a call that ends with its dW
+    // on the second stream from the start, where nothing else of the call runs yet. Not that where an earlier call's dW may still
+    // lie in front of it (an overlapped 256 -> 256 at 14x14 and then 72 -> 136 at 27x19: 86.3 us early, 82.3 beside); not in calls of
+    // less than 2^25 multiply-adds a product, which wait for the host's launches (64 -> 64 at 14x14, batch 16: 17.4, 16.7 before
+    // there was an early form; batch 64, 51 M: the same); and of stride-2 3x3 layers only in phase mode: otherwise dX and dW,
+    // ready at once, take longer together. us early, beside: 1x1 fp32 128 -> 128 at 28x28, batch 32: 26.8,
+    // 28.8; 3x3 fp32 184 -> 432 at 8x8, batch 22: 39.4, 41.3; bf16 256 -> 256 at 14x14, batch 16: 33.2, 35.0; stride 2 at 28x28, batch 32,
+    // 128 -> 128: 36.3, 39.5, but fp32 32 -> 32: 36.4, 31.4 and 64 -> 64 at 48x60, batch 8: 46.6, 37.4. A *_host call's activations are
+    // still on their way up: there it is done on the stream that waits for them.
     const void *Xp = X;
     long long x_pitch = s.H * s.W;
     const StridedLayer *st2 = ctx->strided;
@@ -473,7 +477,8 @@ int conv_backward_impl(dbp_ctx *ctx, const void *delta, const void *X, const voi
         return stack_g > 0 ? launch_x_stacked(ctx, static_cast<const float *>(X), ctx->x_padded[k].ptr, s, stack_g, beside)
                            : launch_rows_job(ctx, RowsJob{X, ctx->x_padded[k].ptr, io == DBP_F32, s.B * s.Cin, s.H * s.W, x_pitch}, beside);
     };
-    const bool early_x = rewrite_x && forked && !late_x && !(flags & DBP_DW_ASYNC) && !ctx->aux_pending;
+    const bool large = numel * s.Cin * s.k * s.k >= (1ll << 25), unphased = st2 && s.k == 3 && ctx->phase_cin % 128 != 0;
+    const bool early_x = rewrite_x && forked && !late_x && !(flags & DBP_DW_ASYNC) && !ctx->aux_pending && large && !unphased;
     auto fork = [&]() -> int {
         return cudaEventRecord(ctx->ev_fork, ctx->stream) == cudaSuccess && cudaStreamWaitEvent(ctx->aux, ctx->ev_fork, 0) == cudaSuccess
                    ? DBP_OK : fail_cuda("forking the dW stream");

@@ -11,9 +11,11 @@ import workloads as wl
 pytestmark = pytest.mark.gpu
 TOL = 1e-5
 
-# B, Ci, Co, H, W (of X), k, stride, dtype
+# B, Ci, Co, H, W (of X), k, stride, dtype: small ones, re-written beside the quantizer, and ones of 2^25 multiply-adds and more
 LAYERS = [(4, 72, 40, 9, 11, 1, 1, "f32"), (3, 64, 48, 7, 7, 3, 1, "bf16"), (2, 40, 64, 20, 20, 3, 1, "f32"), (8, 32, 64, 4, 4, 3, 1, "f32"),
-          (4, 128, 64, 14, 14, 3, 2, "bf16"), (4, 64, 40, 14, 14, 1, 2, "bf16")]
+          (4, 128, 64, 14, 14, 3, 2, "bf16"), (4, 64, 40, 14, 14, 1, 2, "bf16"),
+          (16, 72, 136, 27, 19, 1, 1, "f32"), (16, 128, 128, 7, 7, 3, 1, "bf16"), (8, 128, 64, 14, 14, 3, 1, "f32"), (64, 64, 64, 4, 4, 3, 1, "f32"),
+          (8, 128, 64, 14, 14, 3, 2, "bf16"), (32, 128, 192, 14, 14, 1, 2, "bf16"), (8, 64, 64, 28, 28, 3, 2, "f32")]
 
 
 @pytest.fixture(scope="module")
