@@ -16,8 +16,8 @@
 //
 // Per CTA: a range of segments (runs of up to 512 positions of one image, with a halo of W+1 rows
 // on either side), an output tile of 128 input channels x 64 or 128 output channels, the three
-// taps ky of its kx as three accumulators in tensor memory. With 64 output channels the taps ky = 1
-// and ky = 0 share one MMA of N = 128: its second 64-column group starts W rows further on.
+// taps ky of its kx as three accumulators in tensor memory. The three taps of 64 output channels
+// share one MMA of N = 192, whose 64-column groups start W rows apart.
 // fp32 activations are two bf16 pieces, one after the other along the batch. Layers of at most 64 input channels put both
 // pieces of a position on the two halves of one tile (half as many MMAs, the codes are read once; 64 -> 64 at 32x32, batch
 // 128: 100 -> 91 us for the whole call).
@@ -36,9 +36,9 @@ using namespace tc;
 
 constexpr int kThreadsW3 = 8 * 32;
 constexpr int kXTile = 16384;             // [128 ci][64 positions] bf16
-constexpr int kXS = 2;                    // 64-position stages per activation slot (one hand-over)
-constexpr int kXSlot = kXS * kXTile;
-constexpr int kMaxNX = 6;
+constexpr int kXS = 2;                    // most 64-position stages per activation slot (one hand-over)
+constexpr int kMaxNX = 4;
+constexpr int kMaxNQ = 3;                 // most code buffers
 
 struct Dw3T {
     int Cout, W, HW;
@@ -51,7 +51,8 @@ struct Dw3T {
     int ci_tiles, co_tiles;
     int rows_box, nload;          // a panel is copied as nload boxes of rows_box rows
     int panel_bytes;              // multiple of 1024
-    int nx;                       // activation slots in flight
+    int nx, xs;                   // activation slots in flight, 64-position stages of one
+    int nq;                       // code buffers in flight
     int stage_chunks;             // 32-column chunks of the accumulators that fit the shared memory at once
     int phase_tiles;              // > 0: a stride-2 layer on phase images, this many 128-channel tiles per phase (phase
                                   // ph = 2 py + px holds channels ph * 128 * phase_tiles ...). Only the taps with
@@ -62,7 +63,7 @@ struct Dw3T {
 };
 
 struct PipeW3 {
-    unsigned long long x_full[kMaxNX], x_empty[kMaxNX], q_full[2], q_ready[2], q_empty[2], acc;
+    unsigned long long x_full[kMaxNX], x_empty[kMaxNX], q_full[kMaxNQ], q_ready[kMaxNQ], q_empty[kMaxNQ], acc;
     unsigned tmem_base;
 };
 
@@ -75,7 +76,8 @@ tc3_tma_dw_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
     extern __shared__ __align__(1024) unsigned char smem_raw[];
     unsigned char *smem = reinterpret_cast<unsigned char *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
     unsigned char *x_s = smem;                                   // nx activation slots
-    unsigned char *q_s = x_s + p.nx * kXSlot;                    // 2 buffers x NP panels
+    const int x_slot = p.xs * kXTile;
+    unsigned char *q_s = x_s + p.nx * x_slot;                    // nq buffers x NP panels
     const int qbuf_bytes = NP * p.panel_bytes;
     __shared__ PipeW3 pipe;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -83,7 +85,7 @@ tc3_tma_dw_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
     // work item: (output tile, kernel column, range of segments)
     const int split = blockIdx.x % p.nsplit;
     int rest = blockIdx.x / p.nsplit;
-    int kx, ci_t, co_t, live_lo = 0, live_hi = 3;       // rows ky in [live_lo, live_hi) are accumulated (NP == 2)
+    int kx, ci_t, co_t, live_lo = 0;                    // phase images: taps ky = live_lo .. 1 are accumulated (NP == 2)
     int c_lo = 0, c_hi = (NP == 2 ? 384 : 192) / 32;    // 32-column chunks of the accumulators that are handed over
     if (p.phase_tiles > 0) {
         // per output-channel tile: the phases in order, one kernel column (kx = 1) per channel tile of a phase with
@@ -95,8 +97,8 @@ tc3_tma_dw_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
         r -= py * 3 * tp;
         if (r < tp) { ci_t = 2 * py * tp + r; kx = 1; }
         else { r -= tp; ci_t = (2 * py + 1) * tp + (r >> 1); kx = r & 1; }
-        // NP == 2: columns 0-127 are ky = 0, 128-255 ky = 1, 256-383 ky = 2; NP == 1: 0-63 ky = 2, 64-127 ky = 1, 128-191 ky = 0
-        if (NP == 2) { live_lo = py ? 0 : 1; live_hi = 2; c_lo = 4 * live_lo; c_hi = 8; }
+        // NP == 2: columns 0-127 are ky = 0, 128-255 ky = 1; NP == 1: 0-63 ky = 2, 64-127 ky = 1, 128-191 ky = 0
+        if (NP == 2) { live_lo = py ? 0 : 1; c_lo = 4 * live_lo; c_hi = 8; }
         else { c_lo = 2; c_hi = py ? 6 : 4; }
     } else {
         kx = rest % 3;
@@ -112,7 +114,7 @@ tc3_tma_dw_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
 
     if (threadIdx.x == 0) {
         for (int s = 0; s < kMaxNX; ++s) { mbar_init(&pipe.x_full[s], 1); mbar_init(&pipe.x_empty[s], 1); }
-        for (int s = 0; s < 2; ++s) { mbar_init(&pipe.q_full[s], 1); mbar_init(&pipe.q_ready[s], 1); mbar_init(&pipe.q_empty[s], 1); }
+        for (int s = 0; s < kMaxNQ; ++s) { mbar_init(&pipe.q_full[s], 1); mbar_init(&pipe.q_ready[s], 1); mbar_init(&pipe.q_empty[s], 1); }
         mbar_init(&pipe.acc, 1);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         tma_prefetch_desc(&map_q);
@@ -126,28 +128,35 @@ tc3_tma_dw_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
     const unsigned tmem_base = pipe.tmem_base;
     chain_wait();        // from here on the kernel reads what earlier kernels wrote
 
-    // segment g: image, first position, number of 64-position stages
-    auto seg_of = [&](long long g, int &b, int &u0, int &ns) {
-        b = static_cast<int>(g / p.segs_per_img);
-        u0 = static_cast<int>(g - static_cast<long long>(b) * p.segs_per_img) * p.SEG;
-        const int left = p.HW - u0;
-        ns = ((left < p.SEG ? left : p.SEG) + 63) >> 6;
+    // a segment: image and first position; they are walked one after the other
+    struct Seg { int b, u0; };
+    auto first_seg = [&] {
+        const int b = static_cast<int>(g0 / p.segs_per_img);
+        return Seg{b, static_cast<int>(g0 - static_cast<long long>(b) * p.segs_per_img) * p.SEG};
     };
+    auto next_seg = [&](Seg &s) {
+        s.u0 += p.SEG;
+        if (s.u0 >= p.HW) { s.u0 = 0; ++s.b; }
+    };
+    auto stages_of = [&](const Seg &s) {         // of 64 positions
+        const int left = p.HW - s.u0;
+        return ((left < p.SEG ? left : p.SEG) + 63) >> 6;
+    };
+    const int nseg = g1 > g0 ? static_cast<int>(g1 - g0) : 0;
     // The activation stages of this CTA are consecutive 64-position blocks of consecutive images; a
-    // slot holds kXS consecutive blocks of one image. A new slot starts at the CTA's first stage, at
-    // the first block of an image, and after kXS stages (copy and MMA threads follow the same rule).
+    // slot holds xs consecutive blocks of one image. A new slot starts at the CTA's first stage, at
+    // the first block of an image, and after xs stages (copy and MMA threads follow the same rule).
 
     if (warp == 0) {
         if (lane == 0) {
             bool ok = true;
             const unsigned tx = static_cast<unsigned>(NP * p.nload * p.rows_box * 128);
-            int sg = 0;
+            int buf = 0;
+            unsigned parity = 1;                   // a fresh barrier passes a wait on the previous phase
+            Seg sg = first_seg();
             long long waited = 0;
-            for (long long g = g0; g < g1 && ok; ++g, ++sg) {
-                int b, u0, ns;
-                seg_of(g, b, u0, ns);
-                const int buf = sg & 1;
-                ok = mbar_wait_timed(&pipe.q_empty[buf], ((sg >> 1) & 1) ^ 1, p.err_flag, waited);
+            for (int i = 0; i < nseg; ++i, next_seg(sg)) {
+                ok = mbar_wait_timed(&pipe.q_empty[buf], parity, p.err_flag, waited);
                 if (!ok) break;
                 unsigned char *dst = q_s + buf * qbuf_bytes;
                 mbar_expect_tx(&pipe.q_full[buf], tx);
@@ -155,29 +164,32 @@ tc3_tma_dw_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
                 for (int pn = 0; pn < NP; ++pn)
                     for (int l = 0; l < p.nload; ++l)
                         tma_load_3d(dst + pn * p.panel_bytes + l * p.rows_box * 128, &map_q, co0 + 64 * pn,
-                                    u0 - halo + l * p.rows_box, b % p.code_batch, &pipe.q_full[buf]);
+                                    sg.u0 - halo + l * p.rows_box, sg.b % p.code_batch, &pipe.q_full[buf]);
+                if (++buf == p.nq) { buf = 0; parity ^= 1u; }
             }
             report_wait(p.stats, 3, waited);
         }
     } else if (warp == 1) {
         if (lane == 0) {
             bool ok = true;
-            int s = 0, j = kXS;                    // j: stages already in the current slot
+            int s = 0, j = p.xs;                   // j: stages already in the current slot
             unsigned parity = 1;
             long long waited = 0;
-            for (long long g = g0; g < g1 && ok; ++g) {
-                int b, u0, ns;
-                seg_of(g, b, u0, ns);
+            Seg sg = first_seg();
+            for (int i = 0; i < nseg && ok; ++i, next_seg(sg)) {
+                const int ns = stages_of(sg), b = sg.b;
                 for (int k = 0; k < ns; ++k) {
-                    const int blk = (u0 >> 6) + k;
-                    if (j == kXS || blk == 0) {
+                    const int blk = (sg.u0 >> 6) + k;
+                    if (j == p.xs || blk == 0) {
                         ok = mbar_wait_timed(&pipe.x_empty[s], parity, p.err_flag, waited);
                         if (!ok) break;
-                        unsigned char *dst = x_s + s * kXSlot;
-                        mbar_expect_tx(&pipe.x_full[s], kXSlot);
-                        // positions past the image's end read as zero (a block past its end is all zero)
+                        unsigned char *dst = x_s + s * x_slot;
+                        // blocks of the image that the slot takes; positions past the image's end read as zero
+                        const int nx = p.HW - blk * 64 > 64 ? p.xs : 1;
+                        mbar_expect_tx(&pipe.x_full[s], nx * kXTile);
 #pragma unroll
                         for (int i = 0; i < kXS; ++i) {
+                            if (i >= nx) break;
                             tma_load_3d(dst + i * kXTile, &map_x, (blk + i) * 64, ci0, b, &pipe.x_full[s]);
                             if (p.split)
                                 tma_load_3d(dst + i * kXTile + kXTile / 2, &map_x, (blk + i) * 64, 0, b + p.code_batch, &pipe.x_full[s]);
@@ -192,34 +204,35 @@ tc3_tma_dw_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
         }
     } else if (warp == 2) {
         {   // the whole warp runs the loop (uniform control flow and operands); one elected lane issues
-            // tap ky reads the panel from row (2 - ky) W + (2 - kx) on. NP == 2: one MMA of N = 128 per tap
-            // (accumulator columns 128 ky ...). NP == 1: the three taps share ONE MMA of N = 192 whose
-            // 64-column groups start W rows apart (columns 0-63: ky = 2, 64-127: ky = 1, 128-191: ky = 0):
-            // an MMA of N columns takes max(N/2, 32 + N/4) clocks, 96 for one of 192 against 144 for three of 64.
+            // tap ky reads a panel from row (2 - ky) W + (2 - kx) on. The three taps of a panel share ONE MMA of N = 192 whose
+            // 64-column groups start W rows apart (columns 0-63: ky = 2, 64-127: ky = 1, 128-191: ky = 0; the second panel's
+            // behind them). An MMA of N columns takes max(N/2, 32 + N/4) clocks, 96 for one of 192 against 144 for three of 64;
+            // and where three of N = 128 over both panels read 24 KB of shared memory per 16 positions, two of 192 read 20, beside
+            // the 8 that the copies write: 128 bytes a clock is what there is (260 clocks per 16 positions where it was 290).
+            // Phase images have one or two live taps: an MMA of N = 128 over both panels per tap (columns 128 ky ...).
             constexpr unsigned idesc128 = make_idesc(128, 128, false, true), idesc192 = make_idesc(128, 192, false, true);
+            const bool phases = NP == 2 && p.phase_tiles > 0;
             const unsigned r0 = static_cast<unsigned>((2 * p.W + 2 - kx) * 8), r1 = static_cast<unsigned>((p.W + 2 - kx) * 8),
                            r2 = static_cast<unsigned>((2 - kx) * 8);     // start rows in 16-byte units
             bool ok = true;
-            int slot = -1, j = kXS, sg = 0;
-            unsigned xpar = 0;
+            int slot = -1, j = p.xs, buf = 0;
+            unsigned xpar = 0, qpar = 0;
             unsigned acc_on = 0u;
+            Seg sg = first_seg();
             long long wq = 0, wx = 0;
             const long long born = clock64();
-            for (long long g = g0; g < g1 && ok; ++g, ++sg) {
-                int b, u0, ns;
-                seg_of(g, b, u0, ns);
-                const int buf = sg & 1;
-                ok = __all_sync(0xffffffffu, mbar_wait_timed(&pipe.q_ready[buf], (sg >> 1) & 1, p.err_flag, wq));
+            for (int i = 0; i < nseg && ok; ++i, next_seg(sg)) {
+                ok = __all_sync(0xffffffffu, mbar_wait_timed(&pipe.q_ready[buf], qpar, p.err_flag, wq));
                 if (!ok) break;
                 tc_fence_after();
+                const int u0 = sg.u0, ns = stages_of(sg);
                 const unsigned q_addr = smem_u32(q_s + buf * qbuf_bytes);
-                const unsigned long long bA = NP == 2 ? make_desc(q_addr, p.panel_bytes, 1024) + r0
-                                                      : make_desc(q_addr, p.W * 128, 1024) + r2;
-                const unsigned long long bB = make_desc(q_addr, p.panel_bytes, 1024) + r1;     // NP == 2 only
-                const unsigned long long bC = make_desc(q_addr, p.panel_bytes, 1024) + r2;     // NP == 2 only
+                // the panels' three taps; in phase mode tap ky = 0 and tap ky = 1 of both panels
+                const unsigned long long bA = phases ? make_desc(q_addr, p.panel_bytes, 1024) + r0 : make_desc(q_addr, p.W * 128, 1024) + r2;
+                const unsigned long long bB = phases ? make_desc(q_addr, p.panel_bytes, 1024) + r1 : bA + (static_cast<unsigned>(p.panel_bytes) >> 4);
                 for (int k = 0; k < ns && ok; ++k) {
                     const int blk = (u0 >> 6) + k;
-                    if (j == kXS || blk == 0) {
+                    if (j == p.xs || blk == 0) {
                         if (slot >= 0 && elect_one()) mma_commit(&pipe.x_empty[slot]);
                         if (++slot == p.nx) { slot = 0; xpar ^= 1u; }
                         ok = __all_sync(0xffffffffu, mbar_wait_timed(&pipe.x_full[slot], xpar, p.err_flag, wx));
@@ -231,16 +244,16 @@ tc3_tma_dw_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
                     // slices that are entirely zero fill
                     const int left = p.HW - (u0 + 64 * k);
                     const int nk = left >= 64 ? 4 : (left + 15) >> 4;
-                    const unsigned long long ad = make_desc(smem_u32(x_s + slot * kXSlot + j * kXTile), 16, 1024);
+                    const unsigned long long ad = make_desc(smem_u32(x_s + slot * x_slot + j * kXTile), 16, 1024);
                     const unsigned radv = static_cast<unsigned>(64 * k * 8);
                     auto slice = [&](int kk, unsigned on) {
                         const unsigned adv = radv + kk * 128;                 // 16 rows = 2048 bytes
-                        if (NP == 2) {
+                        if (phases) {
                             if (live_lo == 0) mma_bf16(tmem_base, ad + 2 * kk, bA + adv, idesc128, on);
                             mma_bf16(tmem_base + 128, ad + 2 * kk, bB + adv, idesc128, on);
-                            if (live_hi == 3) mma_bf16(tmem_base + 256, ad + 2 * kk, bC + adv, idesc128, on);
                         } else {
                             mma_bf16(tmem_base, ad + 2 * kk, bA + adv, idesc192, on);
+                            if (NP == 2) mma_bf16(tmem_base + 192, ad + 2 * kk, bB + adv, idesc192, on);
                         }
                     };
                     if (elect_one()) {
@@ -256,6 +269,7 @@ tc3_tma_dw_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
                     ++j;
                 }
                 if (ok && elect_one()) mma_commit(&pipe.q_empty[buf]);
+                if (++buf == p.nq) { buf = 0; qpar ^= 1u; }
             }
             if (ok && slot >= 0 && elect_one()) mma_commit(&pipe.x_empty[slot]);
             if (ok && g1 > g0 && elect_one()) mma_commit(&pipe.acc);
@@ -269,26 +283,23 @@ tc3_tma_dw_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
     } else if (warp == 3) {
         // masked rows: image column 0 for kx = 0, W-1 for kx = 2 (generic-proxy writes, then a proxy
         // fence so that the tensor core sees them)
-        bool ok = true;
-        int sg = 0;
+        int buf = 0;
+        unsigned parity = 0;
         const int zc = kx == 0 ? 0 : p.W - 1;
         const int rows_total = p.nload * p.rows_box;
-        for (long long g = g0; g < g1 && ok; ++g, ++sg) {
-            int b, u0, ns;
-            seg_of(g, b, u0, ns);
-            const int buf = sg & 1;
-            ok = mbar_wait(&pipe.q_full[buf], (sg >> 1) & 1, p.err_flag);
-            if (!ok) break;
+        Seg sg = first_seg();
+        for (int i = 0; i < nseg; ++i, next_seg(sg)) {
+            if (!mbar_wait(&pipe.q_full[buf], parity, p.err_flag)) break;
             if (kx != 1) {
                 unsigned char *qb = q_s + buf * qbuf_bytes;
-                const int i_lo = u0 - halo;                       // image position of panel row 0
+                const int i_lo = sg.u0 - halo;                       // image position of panel row 0
                 // first image position >= max(i_lo, 0) in column zc
                 const int start = i_lo > 0 ? i_lo : 0;
-                int i = start + ((zc - start % p.W) + p.W) % p.W;
+                int at = start + ((zc - start % p.W) + p.W) % p.W;
                 const int sub = lane >> 3, chunk = lane & 7;      // four rows x eight 16-byte pieces per pass
-                i += sub * p.W;
-                for (; i < p.HW && i - i_lo < rows_total; i += 4 * p.W) {
-                    const int r = i - i_lo;
+                at += sub * p.W;
+                for (; at < p.HW && at - i_lo < rows_total; at += 4 * p.W) {
+                    const int r = at - i_lo;
 #pragma unroll
                     for (int pn = 0; pn < NP; ++pn)
                         *reinterpret_cast<uint4 *>(qb + pn * p.panel_bytes + r * 128 + chunk * 16) = make_uint4(0u, 0u, 0u, 0u);
@@ -297,6 +308,7 @@ tc3_tma_dw_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
             }
             __syncwarp();
             if (lane == 0) mbar_arrive(&pipe.q_ready[buf]);
+            if (++buf == p.nq) { buf = 0; parity ^= 1u; }
         }
     } else {
         // epilogue: TMEM lane = input channel, column = (tap, output channel). Every buffer of the
@@ -321,38 +333,44 @@ tc3_tma_dw_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
             chain_release();
             tc_fence_after();
             const long long t_epi = clock64();
-            const int nchunks = c_hi;                  // only the rows the layer wants are handed over
+            // Only the rows the layer wants are handed over, 32 columns at a time: while the copy engine adds one block the next is
+            // staged. What bounds this is an SM's way out, 24 bytes a clock for additions (30 for stores) whatever their form
+            // or number (196 KB: 8.8 thousand clocks alone; 12 where all blocks were staged first, 9.5 so).
             float *stg = reinterpret_cast<float *>(smem);
-            for (int c0 = c_lo; c0 < nchunks; c0 += p.stage_chunks) {
-                const int nb = nchunks - c0 < p.stage_chunks ? nchunks - c0 : p.stage_chunks;
-                for (int i = 0; i < nb; ++i) {
-                    unsigned v[32];
-                    tmem_ld32(tmem_base + (static_cast<unsigned>(q * 32) << 16) + (c0 + i) * 32, v);
-                    float *dst = stg + i * 4096 + (p.split ? (q >> 1) * 2048 + (q & 1) * 32 : q * 32) + lane;
-                    const int pitch = p.split ? 64 : 128;
-#pragma unroll
-                    for (int j = 0; j < 32; ++j) dst[j * pitch] = __uint_as_float(v[j]);
+            for (int c = c_lo, n = 0; c < c_hi; ++c, ++n) {
+                float *const blk = stg + n % p.stage_chunks * 4096;
+                if (n >= p.stage_chunks) {                     // the engine must have read the block's last use
+                    if (et == 0) bulk_wait_read_all();
+                    asm volatile("bar.sync 1, 128;" ::: "memory");
                 }
+                unsigned v[32];
+                tmem_ld32(tmem_base + (static_cast<unsigned>(q * 32) << 16) + c * 32, v);
+                float *dst = blk + (p.split ? (q >> 1) * 2048 + (q & 1) * 32 : q * 32) + lane;
+                const int pitch = p.split ? 64 : 128;
+#pragma unroll
+                for (int j = 0; j < 32; ++j) dst[j * pitch] = __uint_as_float(v[j]);
                 fence_async_proxy();
                 asm volatile("bar.sync 1, 128;" ::: "memory");
-                if (et == 0) {
-                    for (int i = 0; i < nb; ++i) {
-                        const int c = c0 + i;
-                        int ky, col0;                           // tap and first output channel of these 32 columns
-                        if (NP == 2) { ky = c >> 2; col0 = (c & 3) * 32; }     // columns 0-127: ky = 0, 128-255: ky = 1, ...
-                        else { ky = 2 - (c >> 1); col0 = (c & 1) * 32; }       // columns 0-63: ky = 2, 64-127: ky = 1, 128-191: ky = 0
-                        // The rows of output channels past Cout are outside the tap's matrix: the engine skips them. (They are
-                        // zeros only while the activations are finite: NaN added to the next tap's first rows would stay in
-                        // the scratch where nobody reads that tap.)
-                        if (co0 + col0 >= p.Cout) continue;
-                        tma_reduce_add_3d(&map_acc, ci0, co0 + col0, ky * 3 + kx, stg + i * 4096);
-                        if (p.split) tma_reduce_add_3d(&map_acc, 0, co0 + col0, ky * 3 + kx, stg + i * 4096 + 2048);
-                    }
-                    bulk_commit();
-                    bulk_wait_read_all();
+                if (et != 0) continue;
+                int ky, col0;                                  // tap and first output channel of these 32 columns
+                if (NP == 2 && p.phase_tiles > 0) {            // columns 0-127: ky = 0, 128-255: ky = 1
+                    ky = c >> 2;
+                    col0 = (c & 3) * 32;
+                } else {                                       // columns 0-63: ky = 2, 64-127: ky = 1, 128-191: ky = 0, then the next 64 channels
+                    const int pn = c >= 6 ? 1 : 0, r = c - 6 * pn;
+                    ky = 2 - (r >> 1);
+                    col0 = 64 * pn + (r & 1) * 32;
                 }
-                asm volatile("bar.sync 1, 128;" ::: "memory");
+                // The rows of output channels past Cout are outside the tap's matrix: the engine skips them. (They are
+                // zeros only while the activations are finite: NaN added to the next tap's first rows would stay in
+                // the scratch where nobody reads that tap.)
+                if (co0 + col0 < p.Cout) {
+                    tma_reduce_add_3d(&map_acc, ci0, co0 + col0, ky * 3 + kx, blk);
+                    if (p.split) tma_reduce_add_3d(&map_acc, 0, co0 + col0, ky * 3 + kx, blk + 2048);
+                }
+                bulk_commit();
             }
+            if (et == 0) bulk_wait_read_all();                 // the blocks are read before the CTA goes
             if (et == 0) report_wait(p.stats, 5, clock64() - t_epi);     // how long handing over the sums took
         }
     }
@@ -365,82 +383,53 @@ tc3_tma_dw_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
 }
 
 // dW[co][ci][tap] = Delta * acc[tap][co][cip]; the scratch goes back to zero for the next call. The scratch
-// rows hold cin_pad >= Cin channels (activations whose channel count is no multiple of 8 were padded).
-// A block takes 256 consecutive (co, cip) pairs, one per thread: nine coalesced reads (and the zeros written
-// back), a transposition through shared memory (row pitch 9 words: no bank conflicts either way), and the
-// results leave as one contiguous run.
-__global__ void __launch_bounds__(256)
-tc3_dw_finish_kernel(float *__restrict__ acc, const float *__restrict__ delta_p, float *__restrict__ dW, long long pairs,
-                     int cin, int cin_pad) {
-    __shared__ float t_s[256 * 9];
-    chain_wait();
-    chain_release();
-    const float delta = *delta_p;
-    for (long long i0 = blockIdx.x * 256ll; i0 < pairs; i0 += gridDim.x * 256ll) {
-        const long long i = i0 + threadIdx.x;
-        if (i < pairs) {
-            float v[9];
-#pragma unroll
-            for (int t = 0; t < 9; ++t) v[t] = __ldcg(acc + t * pairs + i);
-#pragma unroll
-            for (int t = 0; t < 9; ++t) {
-                __stcg(acc + t * pairs + i, 0.f);
-                t_s[threadIdx.x * 9 + t] = v[t] * delta;
-            }
-        }
-        __syncthreads();
-        const long long left = pairs - i0;
-        const int np = static_cast<int>(left < 256 ? left : 256);
-        if (cin == cin_pad) {
-            for (int k = threadIdx.x; k < np * 9; k += 256) dW[i0 * 9 + k] = t_s[k];
-        } else {
-            for (int k = threadIdx.x; k < np * 9; k += 256) {
-                const long long pr = i0 + k / 9;
-                const long long co = pr / cin_pad;
-                const int ci = static_cast<int>(pr - co * cin_pad);
-                if (ci < cin) dW[(co * cin + ci) * 9 + k % 9] = t_s[k];
-            }
-        }
-        __syncthreads();
-    }
-}
-
-// The same for a stride-2 layer run on phase images (scratch rows of 4 cin channels, phase ph = 2 py + px at channels
+// rows hold cin_pad >= cin channels (activations whose channel count is no multiple of 8 were padded).
+// PHASES: a stride-2 layer run on phase images (scratch rows of 4 cin channels, phase ph = 2 py + px at channels
 // ph * cin ...): the strided layer's tap (ky, kx) of (co, ci) is tap (ty, tx) of channel ph * cin + ci with
 // ky = 0 -> (py, ty) = (1, 0), 1 -> (0, 1), 2 -> (1, 1), kx likewise; the other scratch entries were never touched.
-// dW[co][ci][ky][kx] is written directly, one (co, ci) pair per thread.
-__global__ void __launch_bounds__(256)
-tc3_dw_finish_phases_kernel(float *__restrict__ acc, const float *__restrict__ delta_p, float *__restrict__ dW, int cout, int cin) {
-    __shared__ float t_s[256 * 9];
+// A thread takes four neighbouring channels of an output channel: nine 16-byte loads (and the zeros written back), and their
+// 144 bytes of dW. No shared memory and few threads: the blocks become resident while the dW kernel still hands over its sums,
+// and what they hold then is missing to the next layer's quantization and dX, which want to start at the same time. (Seven blocks
+// of 256 threads per SM and a transposition through shared memory: VGG-16 layer set 747 us against 735; two blocks of these
+// per SM: 749, eight: 736. 512 -> 512 channels by itself: 8.6 us, 7.5.)
+constexpr int kThreadsF3 = 128;
+template <bool PHASES>
+__global__ void __launch_bounds__(kThreadsF3)
+tc3_dw_finish_kernel(float *__restrict__ acc, const float *__restrict__ delta_p, float *__restrict__ dW, int cout, int cin, int cin_pad) {
+    const unsigned per_row = (PHASES ? cin : cin_pad) / 4, quads = static_cast<unsigned>(cout) * per_row;      // multiples of four
+    const size_t tap = static_cast<size_t>(cout) * cin_pad;         // (PHASES: cin_pad = 4 cin)
     chain_wait();
     chain_release();
     const float delta = *delta_p;
-    const long long pairs = static_cast<long long>(cout) * cin, pairs4 = 4 * pairs;
-    for (long long i0 = blockIdx.x * 256ll; i0 < pairs; i0 += gridDim.x * 256ll) {
-        const long long i = i0 + threadIdx.x;
-        if (i < pairs) {
-            const long long co = i / cin, ci = i - co * cin;
-            float *base = acc + co * 4 * cin + ci;
-            float v[9];
+    for (unsigned i = blockIdx.x * kThreadsF3 + threadIdx.x; i < quads; i += gridDim.x * kThreadsF3) {
+        const unsigned co = i / per_row, ci = (i - co * per_row) * 4;
+        float *const base = acc + static_cast<size_t>(co) * cin_pad + ci;
+        float4 *at[9], v[9];
 #pragma unroll
-            for (int t = 0; t < 9; ++t) {
-                const int ky = t / 3, kx = t % 3;
-                const int ph = (ky != 1) * 2 + (kx != 1), tp = (ky == 0 ? 0 : 1) * 3 + (kx == 0 ? 0 : 1);
-                v[t] = __ldcg(base + tp * pairs4 + static_cast<long long>(ph) * cin);
-            }
-#pragma unroll
-            for (int t = 0; t < 9; ++t) {
-                const int ky = t / 3, kx = t % 3;
-                const int ph = (ky != 1) * 2 + (kx != 1), tp = (ky == 0 ? 0 : 1) * 3 + (kx == 0 ? 0 : 1);
-                __stcg(base + tp * pairs4 + static_cast<long long>(ph) * cin, 0.f);
-                t_s[threadIdx.x * 9 + t] = v[t] * delta;
-            }
+        for (int t = 0; t < 9; ++t) {
+            const int ky = t / 3, kx = t % 3;
+            const int ph = PHASES ? (ky != 1) * 2 + (kx != 1) : 0, tp = PHASES ? (ky == 0 ? 0 : 1) * 3 + (kx == 0 ? 0 : 1) : t;
+            at[t] = reinterpret_cast<float4 *>(base + tp * tap + static_cast<size_t>(ph) * cin);
+            v[t] = __ldcg(at[t]);
         }
-        __syncthreads();
-        const long long left = pairs - i0;
-        const int np = static_cast<int>(left < 256 ? left : 256);
-        for (int k = threadIdx.x; k < np * 9; k += 256) dW[i0 * 9 + k] = t_s[k];
-        __syncthreads();
+        float o[36];
+#pragma unroll
+        for (int t = 0; t < 9; ++t) {
+            __stcg(at[t], make_float4(0.f, 0.f, 0.f, 0.f));
+            o[t] = v[t].x * delta;
+            o[9 + t] = v[t].y * delta;
+            o[18 + t] = v[t].z * delta;
+            o[27 + t] = v[t].w * delta;
+        }
+        float *const out = dW + (static_cast<size_t>(co) * cin + ci) * 9;
+        if (PHASES || cin == cin_pad) {                              // 16-byte aligned
+#pragma unroll
+            for (int k = 0; k < 9; ++k) reinterpret_cast<float4 *>(out)[k] = make_float4(o[4 * k], o[4 * k + 1], o[4 * k + 2], o[4 * k + 3]);
+        } else {
+#pragma unroll
+            for (int k = 0; k < 36; ++k)
+                if (ci + k / 9 < static_cast<unsigned>(cin)) out[k] = o[k];
+        }
     }
 }
 
@@ -498,7 +487,7 @@ Panel panel_of(int seg, int W) {
 
 // Whether the kernel fits half an SM: two code buffers of the shortest segment beside two activation slots (W up to 59)
 bool tc3_dw_fits_half(const ConvShape &s) {
-    return 2 * static_cast<size_t>(panel_of(64, static_cast<int>(s.W)).bytes) + 1024 + 2 * kXSlot <= kHalfSm;
+    return 2 * static_cast<size_t>(panel_of(64, static_cast<int>(s.W)).bytes) + 1024 + 2 * kXS * kXTile <= kHalfSm;
 }
 
 // DBP_EUNSUPPORTED: the shape does not fit (the caller uses another kernel)
@@ -540,17 +529,25 @@ int launch_tc3_tma_dw(dbp_ctx *ctx, const void *codes_nhwc, const void *X, int p
     p.ci_tiles = static_cast<int>((cin_pad + 127) / 128);
     p.co_tiles = static_cast<int>((s.Cout + 64 * NP - 1) / (64 * NP));
     // the longest segment whose two code buffers fit beside at least three activation slots
-    const size_t budget = half ? kHalfSm : 227 * 1024 - 2048;
+    // with 128 output channels 17 KB are left to a block of the next layer's position-major quantizer (VGG-16 layer set 747 us
+    // with, 751 without; 34 KB: 752, 51 KB: 762); the long segments of 64 channels are worth more (64 -> 64 at 32x32: 22.0 us, 24.0)
+    const size_t budget = half ? kHalfSm : (NP == 2 ? 210 : 227) * 1024 - 2048;
     const int seg_cap = static_cast<int>(HW < 512 ? (HW + 63) / 64 * 64 : 512);
     size_t smem = 0;
+    p.xs = HW > 64 ? kXS : 1;
+    const size_t x_slot = static_cast<size_t>(p.xs) * kXTile;
     for (int seg = seg_cap; seg >= 64; seg -= 64) {
         const Panel pn = panel_of(seg, p.W);
-        const size_t fixed = 2 * static_cast<size_t>(NP) * pn.bytes + 1024;
-        if (fixed + (half ? 2 : 3) * kXSlot > budget) continue;
+        const size_t qbuf = static_cast<size_t>(NP) * pn.bytes;
+        size_t fixed = 2 * qbuf + 1024;
+        if (fixed + (half ? 2 : 3) * kXS * kXTile > budget) continue;
         p.SEG = seg; p.nload = pn.nload; p.rows_box = pn.rows_box; p.panel_bytes = pn.bytes;
-        p.nx = static_cast<int>((budget - fixed) / kXSlot);
+        // short segments: their MMAs (about 950 clocks of 64 positions) do not cover a copy's way and the zeroing of its columns
+        p.nq = 2;
+        while (seg <= 128 && p.nq < kMaxNQ && fixed + qbuf + 4 * x_slot <= budget) { ++p.nq; fixed += qbuf; }
+        p.nx = static_cast<int>((budget - fixed) / x_slot);
         if (p.nx > kMaxNX) p.nx = kMaxNX;
-        smem = fixed + static_cast<size_t>(p.nx) * kXSlot;
+        smem = fixed + static_cast<size_t>(p.nx) * x_slot;
         break;
     }
     if (smem == 0) return DBP_EUNSUPPORTED;
@@ -609,18 +606,14 @@ int launch_tc3_tma_dw(dbp_ctx *ctx, const void *codes_nhwc, const void *X, int p
     if ((rc = cuda_ok(launch_chained(kern, dim3(static_cast<unsigned>(tiles * nsplit)), dim3(kThreadsW3), smem,
                                      ctx->stream, map_q, map_x, map_acc, p))))
         return rc;
-    if (p.phase_tiles > 0 && ctx->phase_dw_out != nullptr) {
-        // the strided layer's own weight gradient, straight from the scratch
-        long long blocks = (static_cast<long long>(pairs / 4) + 255) / 256;
-        if (blocks > ctx->sm_count * 16) blocks = ctx->sm_count * 16;
-        ctx->phase_dw_done = true;
-        return cuda_ok(launch_chained(tc3_dw_finish_phases_kernel, dim3(static_cast<unsigned>(blocks)), dim3(256), 0, ctx->stream,
-                                      acc, delta_p, ctx->phase_dw_out, static_cast<int>(s.Cout), ctx->phase_cin));
-    }
-    long long blocks = (static_cast<long long>(pairs) + 255) / 256;
-    if (blocks > ctx->sm_count * 16) blocks = ctx->sm_count * 16;
-    return cuda_ok(launch_chained(tc3_dw_finish_kernel, dim3(static_cast<unsigned>(blocks)), dim3(256), 0, ctx->stream, acc,
-                                  delta_p, dW, static_cast<long long>(pairs), static_cast<int>(s.Cin), static_cast<int>(cin_pad)));
+    // a stride-2 layer's own weight gradient comes straight from the scratch
+    const bool phases = p.phase_tiles > 0 && ctx->phase_dw_out != nullptr;
+    if (phases) ctx->phase_dw_done = true;
+    const long long quads = s.Cout * ((phases ? ctx->phase_cin : cin_pad) / 4), need = (quads + kThreadsF3 - 1) / kThreadsF3;
+    const long long most = 4ll * ctx->sm_count, blocks = need < most ? need : most;
+    return cuda_ok(launch_chained(phases ? tc3_dw_finish_kernel<true> : tc3_dw_finish_kernel<false>, dim3(static_cast<unsigned>(blocks)),
+                                  dim3(kThreadsF3), 0, ctx->stream, acc, delta_p, phases ? ctx->phase_dw_out : dW, static_cast<int>(s.Cout),
+                                  static_cast<int>(phases ? ctx->phase_cin : s.Cin), static_cast<int>(cin_pad)));
 }
 
 }  // namespace dbp

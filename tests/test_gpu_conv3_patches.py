@@ -48,3 +48,28 @@ def test_input_gradient(ctx, B, Ci, Co, H, W, dtype):
         again = dbp.dithered_conv_backward(ctx, d, X, Wt, L.seed, L.scale, **kw)["dX"]
         ctx.join()
         assert torch.equal(again, out["dX"].to(again.dtype)), kw
+
+
+@pytest.mark.parametrize("B,Ci,Co,H,W,dtype", [
+    (50, 72, 136, 8, 8, "bf16"), (41, 130, 72, 7, 9, "f32"),           # images of one block: several code buffers, ragged channels
+    (70, 40, 200, 3, 5, "bf16"), (33, 16, 65, 8, 16, "f32"),           # ... and of two blocks, one output channel past a panel
+    (3, 7, 130, 12, 11, "bf16"), (2, 129, 129, 20, 9, "f32")])         # channels that are no multiple of four in dW's rows
+def test_weight_gradient_of_a_whole_sm(ctx, B, Ci, Co, H, W, dtype):
+    """An overlapped call's dW kernel has the SMs to itself. Twice: the second call adds into a scratch that the first put back to zero.
+    (Tolerance: fp32 sums of exact products, as above.)"""
+    import paper_2004_04729_b200 as dbp
+    L = wl.conv_layer(B, Ci, Co, H, W, 3, data_seed=B + Ci + 3 * Co + H, scale=2.0, seed=11, dtype=dtype)
+    tdt = torch.bfloat16 if dtype == "bf16" else torch.float32
+    d, X, Wt = (torch.from_numpy(np.ascontiguousarray(a)).to(tdt).cuda() for a in (L.delta, L.X, L.W))
+    ref = None
+    for _ in range(2):
+        out = dbp.dithered_conv_backward(ctx, d, X, Wt, L.seed, L.scale, flags=dbp.DBP_DW_ASYNC)
+        ctx.join()
+        D, _ = ctx.last_step()
+        if ref is None:
+            codes, _, _ = oracle.nsd_codes(L.delta, L.seed, np.float32(D))
+            ref = oracle.conv_backward(codes, np.float32(D), L.X, L.W, with_abs=True)
+        g = out["dW"].double().cpu().numpy()
+        assert np.linalg.norm(g - ref["dW"]) <= TOL * np.linalg.norm(ref["dW"]) + 1e-30
+        assert np.all(np.abs(g - ref["dW"]) <= TOL * ref["S_dW"] + 1e-30)
+    assert ctx.last_device_status() == (0, 0)
