@@ -4,22 +4,24 @@
 // For gradients of a few tens of thousands of elements every separate kernel (statistics, quantizer,
 // weight re-layout, dX, dW) is a handful of microseconds of work behind a launch and a dependent wait,
 // and the layer is bound by those round trips.
-//   1. small_linear_quantize_kernel: ONE cluster of up to eight CTAs holds the whole gradient in registers. The dithers
-//      are drawn before the kernel waits for what came before it; every CTA adds up its share, the eight pairs of sums
-//      are exchanged through distributed shared memory and added in rank order, so all CTAs hold the same Delta, and
-//      each quantizes its share into bf16 codes [B][N rounded up to 8] and counts the non-zero and clipped ones. The
-//      first CTA publishes Delta; the second kernel adds up the counts. (Before: every CTA of 4096 elements read the
-//      whole gradient for its sums.)
-//   2. small_linear_products_kernel: every CTA owns one 64 x 64 tile of dW or of dX and accumulates it
-//      on the tensor cores: the codes are exact in bf16, the fp32 operand (X or W) is split into two
-//      bf16 pieces (the value rounded to bf16 and what that left over, rounded again: the pair is within
-//      2^-17 of the value), so a k-step is two warp-level MMAs with fp32 accumulation; Delta is applied
-//      once at the end. Warp-level MMAs (not the CTA-wide ones with accumulators in tensor memory)
-//      because a whole tile is a few hundred of them and nothing here can hide a tensor-memory
-//      allocation, a commit and a read-back. The dW tiles of column 0 add up the bias gradient.
+//   1. small_linear_quantize_kernel: one to five clusters of up to eight CTAs. Every cluster holds the whole gradient in
+//      registers. The dithers are drawn before the kernel waits for what came before it; every CTA adds up its share, the
+//      cluster's pairs of sums are exchanged through distributed shared memory and added in rank order, so all CTAs hold the
+//      same Delta, and each cluster quantizes its part of the vectors into bf16 codes [B][N rounded up to 8] and counts the non-zero and
+//      clipped ones. The first CTA publishes Delta; the second kernel adds up the counts.
+//   2. small_linear_products_kernel: every CTA owns one 64 x 64 tile of dW or of dX and accumulates it on the tensor cores:
+//      the codes are exact in bf16, the fp32 operand (X or W) is split into two bf16 pieces (the value rounded to bf16 and
+//      what that left over, rounded again: the pair is within 2^-17 of the value), whose panels lie beside one another as one
+//      operand of 128 columns; Delta is applied once at the end. The dW tiles of column 0 add up the bias gradient.
 //      X and W are inputs of the call: a tile's operand of up to 512 reduction indices is loaded, split and laid in shared
-//      memory while the first kernel runs; what is left after it is one round trip for the codes and the MMAs.
+//      memory while the first kernel runs; what is left after it is one tiled copy per chunk of codes and the MMAs.
 // The second kernel is launched with programmatic stream serialization: it becomes resident while the first runs.
+//
+// Bound by the chain: two kernel boundaries and, for 784 -> 300 at batch 128 in thousands of clocks, loads and sums 2.4, Delta 1.2,
+// decisions 0.9 (one cluster: 2.0), codes by the copy engine and their MMAs, then the tile through shared memory to whole
+// lines. With codes loaded and laid out by the threads (3.7), warp-level MMAs (4.5 of a five-chunk tile) and stores of 32 rows an
+// instruction (1.5) the call took 9.45 us; it takes 7.95. 784-300-100-10, batch 256: 26.6, 22.6. Registers held to 80 or 64, so that the
+// first kernel of the next call fits beside the second: 8.03, 8.73.
 #include "nsd_common.cuh"
 #include "tc_common.cuh"
 
@@ -31,30 +33,18 @@ using namespace nsd;
 
 constexpr int kThreads = 512;
 constexpr int kRows = 64, kCols = 64, kRed = 64;      // output tile and reduction chunk
-constexpr int kPitch = 72;                            // halfwords per shared-memory row: a 16-byte multiple whose eight
-                                                      // consecutive rows fall into different 16-byte bank groups
-constexpr int kChunkTile = 64 * kPitch;               // halfwords of one operand's chunk
+constexpr int kChunkTile = 64 * 128;                  // bytes of one operand's chunk: 64 rows of 64 bf16, 16-byte pieces swizzled by the row
 constexpr int kMaxChunks = 8;                         // chunks whose operands lie in shared memory at once (three tiles each)
+constexpr int kTmemCols = 128;                        // accumulators: 64 columns of the high pieces' products, 64 of the low ones'
 constexpr int kMaxCluster = 8;
 constexpr int kMaxVec = 8;                            // 16-byte vectors per thread of the first kernel
 
 __device__ __forceinline__ unsigned smem_addr(const void *p) { return static_cast<unsigned>(__cvta_generic_to_shared(p)); }
-// four 8x8 matrices of 16-bit elements from shared memory: lane l gives the address of row l % 8 of matrix l / 8;
-// register m of lane (g, tig) receives elements (g, 2 tig) and (g, 2 tig + 1) of matrix m, or, transposed,
-// elements (2 tig, g) and (2 tig + 1, g)
-__device__ __forceinline__ void ldmatrix_x4(unsigned (&r)[4], unsigned addr) {
-    asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0, %1, %2, %3}, [%4];"
-                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(addr));
-}
-__device__ __forceinline__ void ldmatrix_x4_trans(unsigned (&r)[4], unsigned addr) {
-    asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0, %1, %2, %3}, [%4];"
-                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(addr));
-}
-// D += A (16 x 16, row-major fragments) * B (16 x 8, column-major fragments), bf16 in, fp32 accumulate
-__device__ __forceinline__ void mma_bf16_16816(float (&d)[4], const unsigned (&a)[4], unsigned b0, unsigned b1) {
-    asm volatile("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, {%0, %1, %2, %3};"
-                 : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
-                 : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
+// sixteen accumulator columns (the caller waits)
+__device__ __forceinline__ void tmem_ld16(unsigned taddr, unsigned (&r)[16]) {
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, [%16];"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]),
+                   "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15]) : "r"(taddr));
 }
 
 struct SmallLinP {
@@ -85,20 +75,24 @@ __device__ __forceinline__ void store_remote(double *p, unsigned long long *bar,
                  ::"r"(addr), "l"(__double_as_longlong(v)), "r"(baddr) : "memory");
 }
 
-// NV: vectors of four elements per thread (vector i of a thread: blockIdx.x * kThreads + tid + i * all threads)
-template <int NV>
+// NV: vectors of four elements per thread of a cluster (vector i of a thread: rank * kThreads + tid + i * all threads). There are
+// NCL clusters; every one of them has the whole gradient for the sums, and decides the vectors i = its number, + NCL, ...
+// (see the head of this file)
+template <int NV, int NCL>
 __global__ void __launch_bounds__(kThreads)
 small_linear_quantize_kernel(const SmallLinP p) {
+    constexpr int ND = (NV + NCL - 1) / NCL;       // vectors a thread decides, at most
     __shared__ double red_s[2][kThreads / 32];
     __shared__ double all_s[kMaxCluster][2];
     __shared__ unsigned long long bar_s;           // counts the bytes of the sums that arrive from the cluster's CTAs
     __shared__ float delta_s;
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nctas = gridDim.x;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nctas = gridDim.x / NCL;
+    const int cluster = NCL == 1 ? 0 : static_cast<int>(blockIdx.x) / nctas, rank = static_cast<int>(blockIdx.x) - cluster * nctas;
     const int n = static_cast<int>(p.B * p.N), nvec = (n + 3) / 4, step = nctas * kThreads;
-    const int v0 = blockIdx.x * kThreads + tid;
-    unsigned long long u[NV][2];
+    const int v0 = rank * kThreads + tid;
+    unsigned long long u[ND][2];
 #pragma unroll
-    for (int i = 0; i < NV; ++i) dithers_of<4, true>(4ll * (v0 + i * step), p.seed, u[i]);
+    for (int d = 0; d < ND; ++d) dithers_of<4, true>(4ll * (v0 + (cluster + d * NCL) * step), p.seed, u[d]);
     if (tid == 0) {
         tc::mbar_init(&bar_s, 1);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -164,9 +158,9 @@ small_linear_quantize_kernel(const SmallLinP p) {
 #pragma unroll
             for (int o = 8; o > 0; o >>= 1) v += __shfl_xor_sync(kFull, v, o);
             const double a = __shfl_sync(kFull, v, 0), b = __shfl_sync(kFull, v, 16);
-            if (lane < nctas) {                                        // the grid is one cluster: rank = blockIdx.x
-                store_remote(&all_s[blockIdx.x][0], &bar_s, lane, a);
-                store_remote(&all_s[blockIdx.x][1], &bar_s, lane, b);
+            if (lane < nctas) {
+                store_remote(&all_s[rank][0], &bar_s, lane, a);
+                store_remote(&all_s[rank][1], &bar_s, lane, b);
             }
         }
         // (a CTA ends only after all sums have arrived here, so nothing is still on its way to it then)
@@ -199,12 +193,17 @@ small_linear_quantize_kernel(const SmallLinP p) {
     unsigned nz2 = 0, sat = 0;
     const unsigned N = static_cast<unsigned>(p.N);
 #pragma unroll
-    for (int i = 0; i < NV; ++i) {
-        const int e = 4 * (v0 + i * step);
-        if (v0 + i * step < nvec) {
-            float f[4];
+    for (int d = 0; d < ND; ++d) {
+        const int i = cluster + d * NCL, e = 4 * (v0 + i * step);
+        if (i < NV && v0 + i * step < nvec) {
+            float f[4], xi[4];
             unsigned h[2];
-            decide<4>(x[i], u[i], inv, f, sat);                        // elements past the end were read as 0: code 0
+#pragma unroll
+            for (int k = 0; k < NCL; ++k)                              // (an index that is no constant would put x into memory)
+                if (d * NCL + k < NV && k == cluster)
+#pragma unroll
+                    for (int j = 0; j < 4; ++j) xi[j] = x[d * NCL + k < NV ? d * NCL + k : 0][j];
+            decide<4>(xi, u[d], inv, f, sat);                          // elements past the end were read as 0: code 0
             pack_bf16<4>(f, h);
             count_pairs<4>(h, nz2);
             const unsigned b = static_cast<unsigned>(e) / N, j = static_cast<unsigned>(e) - b * N;
@@ -238,12 +237,15 @@ small_linear_quantize_kernel(const SmallLinP p) {
 }
 
 // ---------------------------------------------------------------- both products
-__global__ void __launch_bounds__(kThreads)
-small_linear_products_kernel(const SmallLinP p) {
+__global__ void __launch_bounds__(kThreads, 1)
+small_linear_products_kernel(const __grid_constant__ CUtensorMap map_q, const SmallLinP p) {
     // per chunk of 64 reduction indices: codes (dX tiles [row][reduction index], dW tiles [reduction index][row], the order
     // they are stored in either way), then rows of X (dW) or W (dX), [reduction index][column], as two bf16 pieces
-    extern __shared__ __align__(16) unsigned short tiles_s[];
+    extern __shared__ __align__(1024) unsigned char smem_raw[];
+    unsigned char *const tiles_s = reinterpret_cast<unsigned char *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
     __shared__ float db_s[kRows];
+    __shared__ unsigned long long codes_in[kMaxChunks], mma_done;
+    __shared__ unsigned tmem_s;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
 
     const int t = blockIdx.x;
@@ -257,15 +259,21 @@ small_linear_products_kernel(const SmallLinP p) {
     const float *Bsrc = is_dw ? p.X : p.W;                           // [nred][K]
     const bool do_db = is_dw && kt == 0 && p.db != nullptr;
     if (tid < kRows) db_s[tid] = 0.f;
+    if (tid == 0) {
+        for (int c = 0; c < kMaxChunks; ++c) tc::mbar_init(&codes_in[c], 1);
+        tc::mbar_init(&mma_done, 1);
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+        tc::tma_prefetch_desc(&map_q);
+    }
+    if (warp == 1) tc::tmem_alloc(&tmem_s, kTmemCols);
 
-    // Loads of a chunk: eight consecutive codes per thread, one 16-byte load (dX: row hi, reduction indices
-    // lo..lo+7; dW: reduction index hi, rows lo..lo+7), and eight consecutive columns of row hi of X or W.
+    // Of a chunk a thread loads eight consecutive columns of row hi of X or W.
     const int hi = tid >> 3, lo = (tid & 7) * 8;
-    // warp tiling of the 64 x 64 tile: 16 rows x 16 columns per warp (two 16 x 8 accumulators)
-    const int wr = (warp >> 2) * 16, wc = (warp & 3) * 16;
-    const int g = lane >> 2, tig = lane & 3;
-    float acc[2][4] = {}, sum[2][4] = {};
-    float dbacc[8] = {};
+    const int place = hi * 128 + (((tid & 7) ^ (hi & 7)) << 4);      // where they lie in a tile
+    // Of the accumulators' lanes the first 64 are rows of the tile: the warps of the first two lane quarters read them, sixteen
+    // columns each.
+    const int q = warp & 3, c16 = (warp >> 2) * 16;
+    float sum[16] = {};
 
     auto load_b = [&](long long r0, float4 (&b_reg)[2]) {
         const long long r = r0 + hi;
@@ -287,44 +295,15 @@ small_linear_products_kernel(const SmallLinP p) {
             b_reg[h] = v;
         }
     };
-    // Codes outside the tensor read as zero; the padding of a row is cleared when a vector is used (clear_pad), so that the
-    // loads of all chunks are in flight together.
-    auto load_a = [&](long long r0) {
-        const long long bb = is_dw ? r0 + hi : row0 + hi;            // image (row of delta_z)
-        const long long jj = is_dw ? row0 + lo : r0 + lo;            // first of eight output channels
-        return bb < p.B && jj < p.N ? __ldcg(reinterpret_cast<const uint4 *>(p.codes + bb * p.Np + jj)) : make_uint4(0u, 0u, 0u, 0u);
-    };
-    auto clear_pad = [&](long long r0, uint4 &v) {
-        const long long left = p.N - (is_dw ? row0 + lo : r0 + lo);  // valid codes from the vector's first on
-        if (left < 8) {
-            unsigned w[4] = {v.x, v.y, v.z, v.w};
-#pragma unroll
-            for (int i = 0; i < 4; ++i) {
-                if (2 * i >= left) w[i] = 0u;
-                else if (2 * i + 1 >= left) w[i] &= 0xffffu;
-            }
-            v = make_uint4(w[0], w[1], w[2], w[3]);
-        }
-    };
-    // the addresses this lane hands to the 8x8-matrix loads (lane l: row l % 8 of matrix l / 8)
-    const int lm = lane >> 3, lr = lane & 7;
-    // A, four matrices: (rows 0-7, k 0-7), (rows 8-15, k 0-7), (rows 0-7, k 8-15), (rows 8-15, k 8-15);
-    // dW tiles hold them [k][row] and load them transposed
-    const unsigned a_base = smem_addr(tiles_s) + 2u * (is_dw ? static_cast<unsigned>(((lm >> 1) * 8 + lr) * kPitch + wr + (lm & 1) * 8)
-                                                             : static_cast<unsigned>((wr + (lm & 1) * 8 + lr) * kPitch + (lm >> 1) * 8));
-    const unsigned a_kstep = 2u * (is_dw ? 16u * kPitch : 16u);
-    // B, four matrices: (k 0-7, n 0-7), (k 8-15, n 0-7), (k 0-7, n 8-15), (k 8-15, n 8-15), stored [k][n]: transposed loads
-    const unsigned b_base = smem_addr(tiles_s) + 2u * static_cast<unsigned>(kChunkTile + ((lm & 1) * 8 + lr) * kPitch + wc + (lm >> 1) * 8);
-
-    // fp32 operand of `count` chunks from r0 on -> its two pieces in shared memory, four chunks' loads in flight
+    // fp32 operand of `count` chunks from r0 on -> its two pieces in shared memory, two chunks' loads in flight
     auto fill_b = [&](long long r0, int count) {
-        for (int c0 = 0; c0 < count; c0 += 4) {
-            float4 b_reg[4][2];
+        for (int c0 = 0; c0 < count; c0 += 2) {
+            float4 b_reg[2][2];
 #pragma unroll
-            for (int c = 0; c < 4; ++c)
+            for (int c = 0; c < 2; ++c)
                 if (c0 + c < count) load_b(r0 + (c0 + c) * kRed, b_reg[c]);
 #pragma unroll
-            for (int c = 0; c < 4; ++c)
+            for (int c = 0; c < 2; ++c)
                 if (c0 + c < count) {
                     const float v[8] = {b_reg[c][0].x, b_reg[c][0].y, b_reg[c][0].z, b_reg[c][0].w,
                                         b_reg[c][1].x, b_reg[c][1].y, b_reg[c][1].z, b_reg[c][1].w};
@@ -337,32 +316,9 @@ small_linear_products_kernel(const SmallLinP p) {
                         h2[i] = *reinterpret_cast<const unsigned *>(&hh);
                         l2[i] = *reinterpret_cast<const unsigned *>(&ll);
                     }
-                    unsigned short *dst = tiles_s + (c0 + c) * 3 * kChunkTile + kChunkTile + hi * kPitch + lo;
+                    unsigned char *dst = tiles_s + (c0 + c) * 3 * kChunkTile + kChunkTile + place;
                     *reinterpret_cast<uint4 *>(dst) = make_uint4(h2[0], h2[1], h2[2], h2[3]);
                     *reinterpret_cast<uint4 *>(dst + kChunkTile) = make_uint4(l2[0], l2[1], l2[2], l2[3]);
-                }
-        }
-    };
-    // codes of `count` chunks: one round trip for all of them
-    auto fill_a = [&](long long r0, int count) {
-        {
-            uint4 a_reg[kMaxChunks];
-#pragma unroll
-            for (int c = 0; c < kMaxChunks; ++c)
-                a_reg[c] = c < count ? load_a(r0 + c * kRed) : make_uint4(0u, 0u, 0u, 0u);
-#pragma unroll
-            for (int c = 0; c < kMaxChunks; ++c)
-                if (c < count) {
-                    clear_pad(r0 + c * kRed, a_reg[c]);
-                    *reinterpret_cast<uint4 *>(tiles_s + c * 3 * kChunkTile + hi * kPitch + lo) = a_reg[c];
-                    if (do_db) {
-                        const unsigned w[4] = {a_reg[c].x, a_reg[c].y, a_reg[c].z, a_reg[c].w};
-#pragma unroll
-                        for (int i = 0; i < 4; ++i) {
-                            dbacc[2 * i] += __uint_as_float(w[i] << 16);
-                            dbacc[2 * i + 1] += __uint_as_float(w[i] & 0xffff0000u);
-                        }
-                    }
                 }
         }
     };
@@ -370,6 +326,11 @@ small_linear_products_kernel(const SmallLinP p) {
     // X and W are inputs of the call: the first chunks' operand is laid out before the first kernel is done
     int count = nchunks < p.chunks ? nchunks : p.chunks;
     fill_b(0, count);
+    tc::fence_async_proxy();
+    tc::tc_fence_before();
+    __syncthreads();
+    tc::tc_fence_after();
+    const unsigned tmem = tmem_s;
     chain_wait();
     chain_release();
     const float delta = __ldcg(&p.st->delta);
@@ -381,54 +342,107 @@ small_linear_products_kernel(const SmallLinP p) {
         for (int o = 16; o > 0; o >>= 1) total += __shfl_xor_sync(kFull, total, o);
         if (lane == 0) p.st->nnz = total;
     }
-    for (int c0 = 0; c0 < nchunks; c0 += p.chunks) {
+    // A chunk's codes come as one tiled copy, rows of 64 swizzled as an MMA reads them; outside the tensor they are zero. They are
+    // used as they lie (dX: K-major, 16 reduction indices 32 bytes further; dW: MN-major, 16 rows = 2048 bytes further); X or
+    // W MN-major, the low pieces' panel as columns 64-127. An MMA has 128 rows and the tile 64: the upper ones are whatever
+    // follows the codes (dX) or the same codes (dW), and nobody reads them.
+    const unsigned idesc = tc::make_idesc(128, 128, is_dw, true);
+    const unsigned long long a_desc = tc::make_desc(smem_addr(tiles_s), is_dw ? 0 : 16, 1024);
+    const unsigned long long b_desc = tc::make_desc(smem_addr(tiles_s) + kChunkTile, kChunkTile, 1024);
+    const unsigned a_step = is_dw ? 128 : 2;
+    const int j0 = static_cast<int>(row0), jr = static_cast<int>(kRed);
+    float dbacc[8] = {};
+    unsigned parity = 0;
+    bool ok = true;
+    for (int c0 = 0; c0 < nchunks && ok; c0 += p.chunks) {
         count = nchunks - c0 < p.chunks ? nchunks - c0 : p.chunks;
         if (c0 > 0) {
-            // an accumulator is truncated when an MMA adds to it: after the 64 MMAs of eight chunks it is added to a sum that rounds
-#pragma unroll
-            for (int i = 0; i < 8; ++i) { sum[i >> 2][i & 3] += acc[i >> 2][i & 3]; acc[i >> 2][i & 3] = 0.f; }
-            __syncthreads();                             // the previous chunks have been used
             fill_b(static_cast<long long>(c0) * kRed, count);
+            tc::fence_async_proxy();
+            tc::tc_fence_before();
+            __syncthreads();
+            tc::tc_fence_after();
         }
-        fill_a(static_cast<long long>(c0) * kRed, count);
-        __syncthreads();
-        for (int c = 0; c < count; ++c) {
-            const unsigned off = 2u * static_cast<unsigned>(c * 3 * kChunkTile);
+        if (warp == 0) {
+            if (tc::elect_one())
+                for (int c = 0; c < count; ++c) {
+                    tc::mbar_expect_tx(&codes_in[c], kChunkTile);
+                    tc::tma_load_2d(tiles_s + c * 3 * kChunkTile, &map_q, is_dw ? j0 : (c0 + c) * jr, is_dw ? (c0 + c) * jr : j0, &codes_in[c]);
+                }
+            __syncwarp();
+        } else if (warp == 1) {
+            for (int c = 0; c < count && ok; ++c) {
+                ok = __all_sync(kFull, tc::mbar_wait(&codes_in[c], parity, &p.st->tc_timeout));
+                tc::tc_fence_after();
+                const unsigned long long ad = a_desc + static_cast<unsigned>(c * 3 * (kChunkTile >> 4)), bd = b_desc + static_cast<unsigned>(c * 3 * (kChunkTile >> 4));
+                if (ok && tc::elect_one())
 #pragma unroll
-            for (int ks = 0; ks < kRed / 16; ++ks) {
-                unsigned a[4], bh[4], bl[4];
-                if (is_dw) ldmatrix_x4_trans(a, a_base + off + ks * a_kstep);
-                else ldmatrix_x4(a, a_base + off + ks * a_kstep);
-                ldmatrix_x4_trans(bh, b_base + off + ks * 2u * 16u * kPitch);
-                ldmatrix_x4_trans(bl, b_base + off + 2u * kChunkTile + ks * 2u * 16u * kPitch);
-                mma_bf16_16816(acc[0], a, bh[0], bh[1]);
-                mma_bf16_16816(acc[1], a, bh[2], bh[3]);
-                mma_bf16_16816(acc[0], a, bl[0], bl[1]);
-                mma_bf16_16816(acc[1], a, bl[2], bl[3]);
+                    for (int k = 0; k < kRed / 16; ++k) tc::mma_bf16(tmem, ad + k * a_step, bd + 128 * k, idesc, c + k ? 1u : 0u);
             }
+            if (ok && tc::elect_one()) tc::mma_commit(&mma_done);
+            __syncwarp();
         }
+        // an accumulator is truncated when an MMA adds to it: after the MMAs of eight chunks it is added to a sum that rounds
+        // (and the chunks' places are written again only when they have been read)
+        ok = tc::mbar_wait(&mma_done, parity, &p.st->tc_timeout) && ok;
+        tc::tc_fence_after();
+        if (do_db)
+            for (int c = 0; c < count && ok; ++c) {
+                ok = tc::mbar_wait(&codes_in[c], parity, &p.st->tc_timeout);       // (the copy's bytes are seen by who waits for it)
+                const uint4 v = *reinterpret_cast<const uint4 *>(tiles_s + c * 3 * kChunkTile + place);
+                const unsigned w[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                    dbacc[2 * i] += __uint_as_float(w[i] << 16);
+                    dbacc[2 * i + 1] += __uint_as_float(w[i] & 0xffff0000u);
+                }
+            }
+        parity ^= 1u;
+        __syncwarp();
+        if (q < 2) {
+            unsigned h[16], l[16];
+            const unsigned at = tmem + (static_cast<unsigned>(q * 32) << 16) + c16;
+            tmem_ld16(at, h);
+            tmem_ld16(at + 64, l);
+            asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+#pragma unroll
+            for (int i = 0; i < 16; ++i) sum[i] += __uint_as_float(h[i]) + __uint_as_float(l[i]);
+            tc::tc_fence_before();
+        }
+        ok = __syncthreads_and(ok) != 0;
     }
+    if (warp == 1) tc::tmem_dealloc(tmem, kTmemCols);
 
-    // the tile, scaled by Delta once: accumulator t holds rows g and g + 8, columns 2 tig, 2 tig + 1 of n-tile t
-    float *out = is_dw ? p.dW : p.dX;
+    // The tile, scaled by Delta once: a thread has sixteen columns of a row. Through shared memory (16-byte pieces swizzled by the
+    // row), so that lanes store along the rows: 32 rows an instruction took 1500 clocks.
+    if (ok) {
+        float4 *const stg = reinterpret_cast<float4 *>(tiles_s);
+        if (q < 2) {
+            const int r = q * 32 + lane;
 #pragma unroll
-    for (int tn = 0; tn < 2; ++tn) {
+            for (int i = 0; i < 4; ++i)
+                stg[r * 16 + (((c16 >> 2) + i) ^ (r & 7))] = make_float4(sum[4 * i] * dscale, sum[4 * i + 1] * dscale, sum[4 * i + 2] * dscale, sum[4 * i + 3] * dscale);
+        }
+        __syncthreads();
+        float *const out = is_dw ? p.dW : p.dX;
+        const long long col = k0 + (lane & 15) * 4;
 #pragma unroll
-        for (int h = 0; h < 2; ++h) {
-            const long long row = row0 + wr + g + 8 * h;
-            const long long col = k0 + wc + 8 * tn + 2 * tig;
-            if (row >= nrows || col >= p.K) continue;
-            float *dst = out + row * p.K + col;
-            const float v0 = (sum[tn][2 * h] + acc[tn][2 * h]) * dscale, v1 = (sum[tn][2 * h + 1] + acc[tn][2 * h + 1]) * dscale;
-            if ((p.K & 1) == 0) {
-                *reinterpret_cast<float2 *>(dst) = make_float2(v0, v1);
+        for (int i = 0; i < 2; ++i) {
+            const int r = warp * 4 + 2 * i + (lane >> 4);
+            if (row0 + r >= nrows || col >= p.K) continue;
+            const float4 v = stg[r * 16 + ((lane & 15) ^ (r & 7))];
+            float *const dst = out + (row0 + r) * p.K + col;
+            if (p.vec4) {
+                *reinterpret_cast<float4 *>(dst) = v;
             } else {
-                dst[0] = v0;
-                if (col + 1 < p.K) dst[1] = v1;
+                dst[0] = v.x;
+                if (col + 1 < p.K) dst[1] = v.y;
+                if (col + 2 < p.K) dst[2] = v.z;
+                if (col + 3 < p.K) dst[3] = v.w;
             }
         }
     }
-    if (do_db) {                                         // threads that share lo hold the same eight rows
+    if (do_db && ok) {                                         // threads that share lo hold the same eight rows
 #pragma unroll
         for (int i = 0; i < 8; ++i) atomicAdd(&db_s[lo + i], dbacc[i]);     // small integers: exact in any order
         __syncthreads();
@@ -438,11 +452,12 @@ small_linear_products_kernel(const SmallLinP p) {
 
 }  // namespace
 
-// Shapes the two-launch path takes: a gradient that one cluster holds in registers, and one tile per SM at most. The legacy
-// warp-level MMA runs at about 550 multiply-adds per clock and SM here (a 64 x 64 x 16 step with two pieces takes 240
-// clocks), so a second tile per SM costs more than the third launch of the CTA-wide kernels (linear_tc.cu). Measured, us,
-// this path against that one: 784 -> 300, B 128 (91 tiles): 9.5 against 14.9; 512 -> 1000, B 128 (144): 22.4 against
-// 22.8; 1024 -> 100, B 1024 (288): 24.2 against 15.0.
+// Shapes the two-launch path takes: a gradient that one cluster holds in registers, and one tile per SM at most, or two of
+// reductions that lie in shared memory at once. More cost more than the third launch of the CTA-wide kernels (linear_tc.cu).
+// us, this path against that one, fp32 as (batch, outputs, inputs): (128, 300, 784), 91 tiles: 7.95, 14.9; (128, 1000, 512), 144:
+// 17.1, 22.4; (128, 512, 1024), 160: 14.0, 16.4; (300, 300, 1500), 240: 14.8, 16.1; (64, 512, 2048), 288: 14.0, 15.2;
+// two rounds of chunks: (1024, 100, 1024), 288: 16.0, 14.3; (1000, 64, 1000), 272: 14.7, 13.1; three tiles: (500, 128, 2048),
+// 320: 15.5, 14.0.
 bool small_linear_fits(const dbp_ctx *ctx, long long B, long long N, long long K, bool want_dw, bool want_dx) {
     const long long n = B * N;
     if (n <= 0 || n > 4ll * kMaxCluster * kThreads * kMaxVec || K <= 0 || K > (1ll << 24)) return false;
@@ -450,7 +465,8 @@ bool small_linear_fits(const dbp_ctx *ctx, long long B, long long N, long long K
     const long long n_dw = want_dw ? ((N + kRows - 1) / kRows) * tiles_k : 0;
     const long long n_dx = want_dx ? ((B + kRows - 1) / kRows) * tiles_k : 0;
     const long long ctas = n_dw + n_dx;
-    return ctas > 0 && ctas <= ctx->sm_count;
+    const long long red = want_dw && (!want_dx || B > N) ? B : N;
+    return ctas > 0 && ctas <= (red <= kMaxChunks * kRed ? 2 : 1) * ctx->sm_count;
 }
 
 int launch_small_linear(dbp_ctx *ctx, const float *delta, const float *X, const float *W, long long B, long long N,
@@ -474,20 +490,28 @@ int launch_small_linear(dbp_ctx *ctx, const float *delta, const float *X, const 
     int ctas = 1;
     while (ctas < kMaxCluster && ctas * kThreads < nvec) ctas *= 2;
     const int per = static_cast<int>((nvec + ctas * kThreads - 1) / (ctas * kThreads));
-    p.n_qctas = ctas;
+    const int ncl = per <= 1 ? 1 : per <= 2 ? 2 : per <= 5 ? 5 : 4;
+    p.n_qctas = ctas * ncl;
     p.inv_numel = 1.0 / static_cast<double>(n);
-    auto kern = per <= 1 ? small_linear_quantize_kernel<1> : per <= 2 ? small_linear_quantize_kernel<2>
-              : per <= 5 ? small_linear_quantize_kernel<5> : small_linear_quantize_kernel<kMaxVec>;
-    if (int rc = cuda_ok(launch_chained_cluster(kern, static_cast<unsigned>(ctas), static_cast<unsigned>(ctas), dim3(kThreads), 0, ctx->stream, p))) return rc;
+    auto kern = per <= 1 ? small_linear_quantize_kernel<1, 1> : per <= 2 ? small_linear_quantize_kernel<2, 2>
+              : per <= 5 ? small_linear_quantize_kernel<5, 5> : small_linear_quantize_kernel<kMaxVec, 4>;
+    if (int rc = cuda_ok(launch_chained_cluster(kern, static_cast<unsigned>(ctas * ncl), static_cast<unsigned>(ctas), dim3(kThreads), 0, ctx->stream, p))) return rc;
+    CUtensorMap map_q;
+    {
+        const unsigned long long dims[2] = {static_cast<unsigned long long>(N), static_cast<unsigned long long>(B)};
+        const unsigned long long str[1] = {static_cast<unsigned long long>(p.Np) * 2};
+        const unsigned box[2] = {kRed, kRows};
+        if (!tc::encode_map_bf16(&map_q, p.codes, 2, dims, str, box)) return fail_cuda("tensor map of the codes");
+    }
     const long long red = (dW && (!dX || B > N)) ? B : N;               // the longest reduction of the tiles
     const long long chunks = (red + kRed - 1) / kRed;
     p.chunks = chunks < kMaxChunks ? static_cast<int>(chunks) : kMaxChunks;
-    const size_t smem = static_cast<size_t>(p.chunks) * 3 * kChunkTile * 2;
+    const size_t smem = static_cast<size_t>(p.chunks) * 3 * kChunkTile + 1024;
     if (cudaFuncSetAttribute(small_linear_products_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             kMaxChunks * 3 * kChunkTile * 2) != cudaSuccess)
+                             kMaxChunks * 3 * kChunkTile + 1024) != cudaSuccess)
         return fail_cuda("shared memory size");
     return cuda_ok(launch_chained(small_linear_products_kernel, dim3(static_cast<unsigned>(p.n_dw + p.n_dx)), dim3(kThreads), smem,
-                                  ctx->stream, p));
+                                  ctx->stream, map_q, p));
 }
 
 }  // namespace dbp

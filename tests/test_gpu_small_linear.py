@@ -54,6 +54,9 @@ def _fused_was_used(ctx, fn):
     (33, 7, 50),         # ragged everywhere, K % 4 != 0: element-wise accesses along K
     (1, 1, 1),
     (70, 129, 65),       # one past a tile in every direction
+    (300, 400, 64),      # eight vectors per thread, shared by four clusters
+    (1000, 100, 72),     # a reduction of sixteen chunks: two rounds of eight
+    (577, 17, 33),       # ... and of ten, the last one of a single row; odd rows and columns
 ])
 def test_small_linear_matches_the_oracle(ctx, B, N, K):
     import paper_2004_04729_b200 as dbp
