@@ -12,6 +12,7 @@ namespace {
 using namespace nsd;
 
 constexpr int kThreads = 256;
+constexpr int kStatBlocksPerSM = 4, kStatUnroll = 4;       // of the statistics kernel: blocks per SM, vectors of a thread per tile
 
 // read-once data: do not keep the line in L1
 __device__ __forceinline__ uint4 load_stream(const void *p) {
@@ -134,18 +135,23 @@ statistics_kernel(const T *__restrict__ x, long long n, double *__restrict__ par
                   const unsigned char *__restrict__ mask, const SideJobs jobs) {
     constexpr int EPT = Vec<T>::V;
     const long long nvec = n / EPT;
-    // whole tiles of kUnroll x kThreads 128-bit vectors, a block at a time: kUnroll loads in flight
-    // per thread, consecutive threads on consecutive vectors
-    constexpr int kUnroll = 8;
-    const long long tile = static_cast<long long>(kUnroll) * kThreads, ntile = nvec / tile;
-    uint4 raw[kUnroll];
-    auto load = [&](long long t) {
+    // whole tiles of kStatUnroll x kThreads 128-bit vectors, a block at a time, consecutive threads on consecutive vectors; the
+    // next tile's loads are under way while a tile's values are added up
+    constexpr int U = kStatUnroll;
+    constexpr long long tile = static_cast<long long>(U) * kThreads;
+    const long long ntile = nvec / tile;
+    struct Batch { uint4 raw[U]; unsigned msk[MASKED ? U : 1]; } even, odd;
+    auto load = [&](long long t, Batch &b) {
+        const long long v0 = t * tile + threadIdx.x;
 #pragma unroll
-        for (int u = 0; u < kUnroll; ++u) raw[u] = load_stream(x + (t * tile + threadIdx.x + static_cast<long long>(u) * kThreads) * EPT);
+        for (int u = 0; u < U; ++u) {
+            b.raw[u] = load_stream(x + (v0 + u * kThreads) * EPT);
+            if (MASKED) b.msk[u] = __ldg(reinterpret_cast<const unsigned *>(mask) + v0 + u * kThreads);
+        }
     };
     chain_wait();
     chain_release();
-    if (blockIdx.x < ntile) load(blockIdx.x);       // on its way during the side jobs
+    if (blockIdx.x < ntile) load(blockIdx.x, even);       // on its way during the side jobs
     // side job for the layer's weight-gradient kernel, which adds its partial sums into dW: clear it
     {
         const long long first = static_cast<long long>(blockIdx.x) * kThreads + threadIdx.x, step = static_cast<long long>(gridDim.x) * kThreads;
@@ -269,25 +275,32 @@ statistics_kernel(const T *__restrict__ x, long long n, double *__restrict__ par
     }
     const float pivot = (!MASKED || __ldg(mask)) ? Vec<T>::one(x) : 0.f;
     const long long stride = static_cast<long long>(gridDim.x) * kThreads;
-    for (long long t = blockIdx.x; t < ntile; t += gridDim.x) {
-        if (t != blockIdx.x) load(t);
-        float v[kUnroll][EPT];
+    auto add = [&](const Batch &b) {
 #pragma unroll
-        for (int u = 0; u < kUnroll; ++u) Vec<T>::values(raw[u], v[u]);
+        for (int u = 0; u < U; ++u) {
+            float v[EPT];
+            Vec<T>::values(b.raw[u], v);
+            if (MASKED) {
 #pragma unroll
-        for (int u = 0; u < kUnroll; ++u) mask4<MASKED>(mask, (t * tile + threadIdx.x + static_cast<long long>(u) * kThreads) * EPT, v[u]);
-#pragma unroll
-        for (int u = 0; u < kUnroll; ++u) {
+                for (int j = 0; j < EPT; ++j) v[j] = b.msk[u] >> (8 * j & 31) & 0xffu ? v[j] : 0.f;
+            }
             float s1 = 0.f, s2 = 0.f;
 #pragma unroll
             for (int j = 0; j < EPT; ++j) {
-                const float c = v[u][j] - pivot;
+                const float c = v[j] - pivot;
                 s1 += c;
                 s2 = fmaf(c, c, s2);
             }
             d1 += static_cast<double>(s1);
             d2 += static_cast<double>(s2);
         }
+    };
+    for (long long t = blockIdx.x; t < ntile; t += 2 * gridDim.x) {
+        const long long t1 = t + gridDim.x, t2 = t1 + gridDim.x;
+        if (t1 < ntile) load(t1, odd);
+        add(even);
+        if (t2 < ntile) load(t2, even);
+        if (t1 < ntile) add(odd);
     }
     // the vectors after the last whole tile
     long long i = ntile * tile + static_cast<long long>(blockIdx.x) * kThreads + threadIdx.x;
@@ -509,7 +522,6 @@ decode_kernel(const uint32_t *__restrict__ bitmap, const uint16_t *__restrict__ 
 
 }  // namespace
 
-constexpr int kStatBlocksPerSM = 2;
 
 int launch_rows_job(dbp_ctx *ctx, const RowsJob &job, bool beside) {
     long long b = (job.rows * (job.pitch / 8) + kThreads - 1) / kThreads;
@@ -532,7 +544,7 @@ int launch_statistics(dbp_ctx *ctx, const void *delta, int dtype, long long nume
         return cuda_ok(launch_chained(clear_counts_kernel, dim3(1), dim3(1), 0, ctx->stream, ctx->state, nnz_out));
     }
     const int ept = dtype == DBP_F32 ? 4 : 8;
-    long long blocks = numel / ept / (kThreads * 8);          // one block per tile of eight vectors per thread
+    long long blocks = numel / ept / (kThreads * kStatUnroll);          // one block per tile
     if (blocks < 1) blocks = 1;
     // the side jobs want blocks of their own when the tensor is small (a block beyond the tensor's tiles adds zeros)
     if (jobs.w_src != nullptr && blocks < jobs.Cout) blocks = jobs.Cout;
@@ -542,9 +554,10 @@ int launch_statistics(dbp_ctx *ctx, const void *delta, int dtype, long long nume
         if (blocks < b) blocks = b;
     }
     if (blocks > ctx->partial_blocks) blocks = ctx->partial_blocks;
-    // two resident blocks per SM, each walking several tiles, finish sooner than one block per tile: fewer partial sums
-    // for every CTA of the quantizer to add (one or four blocks per SM: 119 -> 124 us for a thin 1x1 layer, 1044 -> 1055 for
-    // the ResNet-50 layer set, the whole calls). The weight re-laying side job wants one block per output channel.
+    // Four resident blocks per SM, each walking its tiles of four vectors a thread with the next tile's loads under way (two blocks,
+    // eight vectors, one tile's loads at a time before: ResNet-50 layer set 845 us against 839, VGG-16 762 against 756, 2048 -> 1000 at
+    // batch 256 23.6 against 23.1, the largest tensors the same: 103 MB in 16 us). Two, three or six blocks with this kernel: 853, 847,
+    // 847. The weight re-laying side job wants one block per output channel.
     if (jobs.w_src == nullptr && blocks > static_cast<long long>(ctx->sm_count) * kStatBlocksPerSM)
         blocks = static_cast<long long>(ctx->sm_count) * kStatBlocksPerSM;
     auto go = [&](auto kern, auto x, const unsigned char *m) {
