@@ -232,6 +232,15 @@ bool tc3_tma_supported(const ConvShape &s, int io, bool dx_f32);
 // whether it did. dX is the same either way.
 int launch_tc3_tma_dx(dbp_ctx *ctx, const void *codes_nhwc, const void *W, int io, const float *delta_p,
                       const ConvShape &s, void *dX, bool dx_bf16, int *err_flag, bool weights_ready = false, bool *lean = nullptr);
+// ---- tc3_rows_dx.cu: the same for small planes, a row of several images at a time
+struct RowsPlan {
+    int nimg = 0, KS = 1;               // images per tile, CTAs that share its reduction
+};
+// max_cols: accumulator columns of a tile, at most; lean: as for launch_tc3_tma_dx
+double tc3_rows_plan(const dbp_ctx *ctx, const ConvShape &s, int pieces, int max_cols, RowsPlan *plan);
+int launch_tc3_rows_dx(dbp_ctx *ctx, const RowsPlan &plan, const void *codes_nhwc, int pieces, const float *delta_p, const ConvShape &s,
+                       void *dX, bool dx_bf16, int *err_flag, bool *lean);
+constexpr int kRowsLeanCols = 128, kRowsMaxCols = 256;       // accumulator columns of a tile: that fits half an SM, at most
 // Dynamic shared memory of a kernel two of whose CTAs share an SM (228 KB, of which a CTA takes 1 KB and the 1 KB of its own variables)
 constexpr size_t kHalfSm = 112 * 1024;
 // X: bf16 planes of x_pitch values, pieces of every image one after the other

@@ -788,10 +788,40 @@ int launch_tc3_tma_dx(dbp_ctx *ctx, const void *codes_nhwc, const void *W, int i
     };
     search();
     if (smem == 0) return DBP_EUNSUPPORTED;
+    // Rows of several images instead of patches (tc3_rows_dx.cu), by the same count of clocks and whatever else is asked for, because
+    // the order of a sum depends on the way it is made: tiles that fit half an SM where they take less than 0.85, wider ones,
+    // beside which no dW CTA fits, where they take less than 0.65. dX alone and the joined call, us, patches against rows, by the ratio of the counts:
+    // 0.60 512 -> 512 fp32 at 2x2, batch 128: 29.2, 21.0; 52.1, 48.7; 0.59 at 4x4: 45.3, 30.6; 75.1, 68.1; 0.70 256 -> 512 at 4x4: 31.6, 23.6;
+    // 49.0, 44.2; 0.73 128 -> 256 at 8x8: 33.2, 26.6; 47.7, 40.3 (wide: 25.5, 51.2); 0.85 bf16 768 -> 384 at 3x4, batch 70: 29.5, 25.7;
+    // 65.8, 57.8; 0.86 512 -> 512 at 7x7, batch 64: 36.6, 41.4; 67.9, 69.3; 0.91 256 -> 256 fp32 at 8x8, batch 128: 34.4, 34.8; 54.3, 53.9.
+    RowsPlan rows_plan, rows_wide;
+    const int weight_pieces = io == DBP_F32 ? 2 : 1;
+    const double rows_cost = tc3_rows_plan(ctx, s, weight_pieces, kRowsLeanCols, &rows_plan);
+    bool by_rows = false;
+    if (rows_cost > 0) {
+        double patches = best;
+        if (p.es == 2) {                         // decided for an fp32 dX, so that the bf16 one is that one rounded
+            const Dx3T found = chosen;
+            const size_t found_smem = smem;
+            p.es = 4;
+            best = 1e300;
+            search();
+            p.es = 2;
+            patches = best;
+            chosen = found;
+            smem = found_smem;
+        }
+        by_rows = rows_cost < 0.85 * patches;
+        const double wide_cost = tc3_rows_plan(ctx, s, weight_pieces, kRowsMaxCols, &rows_wide);
+        if (wide_cost < 0.65 * patches && wide_cost < rows_cost) {
+            by_rows = true;
+            rows_plan = rows_wide;
+        }
+    }
     // Half an SM's worth of it, when the caller can use the other half: only with one round of CTAs (then the staging block can
     // lie over the operands), and not for phase images, whose slots of two taps do not fit
     const bool one_wave = chosen.ntiles * chosen.KS <= sms;
-    if (lean != nullptr) {
+        if (lean != nullptr && !by_rows) {
         const Dx3T wide = chosen;
         const size_t wide_smem = smem;
         if (one_wave && p.phase_cin == 0) {
@@ -823,6 +853,7 @@ int launch_tc3_tma_dx(dbp_ctx *ctx, const void *codes_nhwc, const void *W, int i
                                         static_cast<const __nv_bfloat16 *>(W), taps, s.Cout, s.Cin, w_pitch));
         if (rc) return rc;
     }
+    if (by_rows) return launch_tc3_rows_dx(ctx, rows_plan, codes_nhwc, weight_pieces, delta_p, s, dX, dx_bf16, err_flag, lean);
     CUtensorMap map_q, map_w;
     {
         const unsigned long long dims[4] = {static_cast<unsigned long long>(s.Cout), static_cast<unsigned long long>(s.W),

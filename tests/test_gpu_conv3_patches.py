@@ -29,7 +29,10 @@ def ctx():
     (9, 40, 72, 6, 24, "bf16"), (5, 200, 72, 6, 25, "f32"), (40, 130, 136, 5, 5, "f32"),       # dX and dW share every SM, or not
     (3, 64, 72, 26, 26, "f32"), (2, 72, 136, 7, 56, "bf16"), (1, 256, 128, 12, 59, "f32"), (1, 136, 72, 9, 60, "bf16"),   # half an SM: widest rows
     (3, 40, 24, 9, 56, "bf16"), (2, 72, 16, 10, 28, "bf16"), (2, 24, 24, 22, 60, "bf16"),      # dX by whole blocks: partial last
-    (2, 136, 40, 11, 16, "f32"), (9, 136, 64, 4, 8, "f32"), (1, 64, 8, 31, 48, "f32")])       # patches, several images, ragged rows
+    (2, 136, 40, 11, 16, "f32"), (9, 136, 64, 4, 8, "f32"), (1, 64, 8, 31, 48, "f32"),        # patches, several images, ragged rows
+    (69, 98, 274, 2, 2, "f32"), (33, 136, 520, 2, 3, "bf16"), (60, 200, 392, 1, 4, "f32"),    # rows of several images: no kernel row above or
+    (50, 130, 456, 5, 1, "f32"), (33, 128, 312, 7, 7, "f32"), (17, 72, 500, 4, 5, "bf16"),    # ... below, one column, ragged images and channels,
+    (14, 896, 352, 9, 9, "f32"), (24, 136, 1000, 2, 2, "f32")])                                # ... clusters of two to eight, wide tiles
 def test_input_gradient(ctx, B, Ci, Co, H, W, dtype):
     import paper_2004_04729_b200 as dbp
     L = wl.conv_layer(B, Ci, Co, H, W, 3, data_seed=B + Ci + 5 * Co + H, scale=2.0, seed=9, dtype=dtype)
