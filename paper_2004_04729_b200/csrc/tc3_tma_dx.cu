@@ -668,18 +668,23 @@ bool tc3_tma_supported(const ConvShape &s, int io, bool dx_f32) {
            (!dx_f32 || s.Cout <= 64ll * kMaxBlocks * kMaxKS);
 }
 
-// DBP_EUNSUPPORTED: the shape does not fit (the caller uses another kernel)
-int launch_tc3_tma_dx(dbp_ctx *ctx, const void *codes_nhwc, const void *W, int io, const float *delta_p,
-                      const ConvShape &s, void *dX, bool dx_bf16, int *err_flag, bool weights_ready, bool *lean) {
-    if (!tc3_tma_supported(s, io, false)) return DBP_EUNSUPPORTED;
+namespace {
+// How a layer's dX is made: patches (t, with no pointers in it) or rows of several images
+struct Dx3Plan {
+    Dx3T t{};
+    size_t smem = 0;
+    bool small = false, by_rows = false;
+    RowsPlan rows;
+    int map_taps = 9;
+};
+
+// share: the caller can use the other half of every SM. false: the shape does not fit
+bool plan_tc3_dx(const dbp_ctx *ctx, const ConvShape &s, int io, int es, bool share, Dx3Plan &plan) {
     Dx3T p{};
-    p.delta_p = delta_p; p.dX = dX;
-    p.es = dx_bf16 ? 2 : 4;
+    p.es = es;
     p.ntaps = io == DBP_F32 ? 18 : 9;
     p.B = static_cast<int>(s.B); p.Cin = static_cast<int>(s.Cin); p.Cout = static_cast<int>(s.Cout);
     p.H = static_cast<int>(s.H); p.W = static_cast<int>(s.W);
-    p.err_flag = err_flag;
-    p.stats = ctx->wait_stats;
     p.phase_cin = (ctx->phase_cin > 0 && ctx->phase_cin % 128 == 0 && s.Cin == 4ll * ctx->phase_cin) ? ctx->phase_cin : 0;
     p.ncb = (p.Cout + 63) / 64;
     p.ci_tiles = (p.Cin + 127) / 128;
@@ -690,7 +695,7 @@ int launch_tc3_tma_dx(dbp_ctx *ctx, const void *codes_nhwc, const void *W, int i
     while (p.es == 4 && min_ks < kMaxKS && min_ks * kMaxBlocks < p.ncb) min_ks *= 2;
     p.split = io == DBP_F32 && p.Cin <= 64 && min_ks == 1 ? 1 : 0;
     p.a_panels = p.Cin <= 64 && !p.split ? 1 : 2;
-    const int map_taps = p.ntaps;
+    plan.map_taps = p.ntaps;
     if (p.split) p.ntaps = 9;
     p.nq = kMaxQ;
     const int sms = ctx->sm_count;
@@ -787,17 +792,17 @@ int launch_tc3_tma_dx(dbp_ctx *ctx, const void *codes_nhwc, const void *W, int i
         }
     };
     search();
-    if (smem == 0) return DBP_EUNSUPPORTED;
+    if (smem == 0) return false;
     // Rows of several images instead of patches (tc3_rows_dx.cu), by the same count of clocks and whatever else is asked for, because
     // the order of a sum depends on the way it is made: tiles that fit half an SM where they take less than 0.85, wider ones,
     // beside which no dW CTA fits, where they take less than 0.65. dX alone and the joined call, us, patches against rows, by the ratio of the counts:
     // 0.60 512 -> 512 fp32 at 2x2, batch 128: 29.2, 21.0; 52.1, 48.7; 0.59 at 4x4: 45.3, 30.6; 75.1, 68.1; 0.70 256 -> 512 at 4x4: 31.6, 23.6;
     // 49.0, 44.2; 0.73 128 -> 256 at 8x8: 33.2, 26.6; 47.7, 40.3 (wide: 25.5, 51.2); 0.85 bf16 768 -> 384 at 3x4, batch 70: 29.5, 25.7;
     // 65.8, 57.8; 0.86 512 -> 512 at 7x7, batch 64: 36.6, 41.4; 67.9, 69.3; 0.91 256 -> 256 fp32 at 8x8, batch 128: 34.4, 34.8; 54.3, 53.9.
-    RowsPlan rows_plan, rows_wide;
+    RowsPlan rows_wide, &rows_plan = plan.rows;
     const int weight_pieces = io == DBP_F32 ? 2 : 1;
     const double rows_cost = tc3_rows_plan(ctx, s, weight_pieces, kRowsLeanCols, &rows_plan);
-    bool by_rows = false;
+    bool &by_rows = plan.by_rows;
     if (rows_cost > 0) {
         double patches = best;
         if (p.es == 2) {                         // decided for an fp32 dX, so that the bf16 one is that one rounded
@@ -821,20 +826,63 @@ int launch_tc3_tma_dx(dbp_ctx *ctx, const void *codes_nhwc, const void *W, int i
     // Half an SM's worth of it, when the caller can use the other half: only with one round of CTAs (then the staging block can
     // lie over the operands), and not for phase images, whose slots of two taps do not fit
     const bool one_wave = chosen.ntiles * chosen.KS <= sms;
-        if (lean != nullptr && !by_rows) {
+    if (share && one_wave && p.phase_cin == 0 && !by_rows) {
         const Dx3T wide = chosen;
         const size_t wide_smem = smem;
-        if (one_wave && p.phase_cin == 0) {
-            small = true;
-            wide_ks = wide.KS;
-            best = 1e300;
-            smem = 0;
-            search();
-        }
-        *lean = small = small && smem != 0;
+        small = true;
+        wide_ks = wide.KS;
+        best = 1e300;
+        smem = 0;
+        search();
+        small = smem != 0;
         if (!small) { chosen = wide; smem = wide_smem; }
     }
-    p = chosen;
+    plan.small = small;
+    plan.t = chosen;
+    plan.smem = smem;
+    return true;
+}
+
+// The search is a microsecond of divisions on the host, of the twenty that a small layer's call is bound by (bf16 128 -> 128 at 7x7,
+// batch 8, joined: 20.2 us of host time without the kept plans, 19.1 with). A thread keeps the plans of the shapes it saw last.
+const Dx3Plan *plan_of(const dbp_ctx *ctx, const ConvShape &s, int io, int es, bool share) {
+    struct Entry {
+        ConvShape s{};
+        int io = 0, es = 0, phase_cin = 0, sms = 0;
+        bool share = false, fits = false;
+        Dx3Plan plan;
+    };
+    constexpr int kKept = 32;
+    static thread_local Entry kept[kKept];
+    static thread_local int count = 0, next = 0;
+    for (int i = 0; i < count; ++i) {
+        const Entry &e = kept[i];
+        if (e.s.B == s.B && e.s.Cin == s.Cin && e.s.Cout == s.Cout && e.s.H == s.H && e.s.W == s.W && e.io == io && e.es == es &&
+            e.share == share && e.phase_cin == ctx->phase_cin && e.sms == ctx->sm_count)
+            return e.fits ? &e.plan : nullptr;
+    }
+    Entry &e = kept[next];
+    next = (next + 1) % kKept;
+    if (count < kKept) ++count;
+    e = Entry{};
+    e.s = s; e.io = io; e.es = es; e.share = share; e.phase_cin = ctx->phase_cin; e.sms = ctx->sm_count;
+    e.fits = plan_tc3_dx(ctx, s, io, es, share, e.plan);
+    return e.fits ? &e.plan : nullptr;
+}
+}  // namespace
+
+// DBP_EUNSUPPORTED: the shape does not fit (the caller uses another kernel)
+int launch_tc3_tma_dx(dbp_ctx *ctx, const void *codes_nhwc, const void *W, int io, const float *delta_p,
+                      const ConvShape &s, void *dX, bool dx_bf16, int *err_flag, bool weights_ready, bool *lean) {
+    if (!tc3_tma_supported(s, io, false)) return DBP_EUNSUPPORTED;
+    const Dx3Plan *const plan = plan_of(ctx, s, io, dx_bf16 ? 2 : 4, lean != nullptr);
+    if (plan == nullptr) return DBP_EUNSUPPORTED;
+    Dx3T p = plan->t;
+    p.delta_p = delta_p; p.dX = dX; p.err_flag = err_flag; p.stats = ctx->wait_stats;
+    const bool small = plan->small;
+    const size_t smem = plan->smem;
+    const int map_taps = plan->map_taps, sms = ctx->sm_count;
+    if (lean != nullptr) *lean = small;
 
     // re-laid weights
     const long long w_pitch = (s.Cin + 7) / 8 * 8, q_pitch = (s.Cout + 7) / 8 * 8;
@@ -853,7 +901,7 @@ int launch_tc3_tma_dx(dbp_ctx *ctx, const void *codes_nhwc, const void *W, int i
                                         static_cast<const __nv_bfloat16 *>(W), taps, s.Cout, s.Cin, w_pitch));
         if (rc) return rc;
     }
-    if (by_rows) return launch_tc3_rows_dx(ctx, rows_plan, codes_nhwc, weight_pieces, delta_p, s, dX, dx_bf16, err_flag, lean);
+    if (plan->by_rows) return launch_tc3_rows_dx(ctx, plan->rows, codes_nhwc, io == DBP_F32 ? 2 : 1, delta_p, s, dX, dx_bf16, err_flag, lean);
     CUtensorMap map_q, map_w;
     {
         const unsigned long long dims[4] = {static_cast<unsigned long long>(s.Cout), static_cast<unsigned long long>(s.W),
