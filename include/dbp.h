@@ -273,6 +273,17 @@ int dithered_conv_backward(dbp_ctx *ctx, const void *delta, const void *X, const
                            dbp_sparse *q_out, float *dW, void *dX, float *db, unsigned flags);
 
 /*
+ * The same where a 2x2 max-pool follows the layer and the gradient at hand is that of the pooled output: `g`
+ * [B,Cout,H/2,W/2] goes through its routing (`argmax`, as for dbp_maxpool2x2_backward) into `delta` [B,Cout,H,W], a buffer
+ * that the call overwrites, which then is the layer's gradient. fp32, stride 1, H and Wd even. Layers of few channels with
+ * 5x5 kernels are routed by the kernel that takes the statistics.
+ */
+int dithered_conv_backward_pooled(dbp_ctx *ctx, const float *g, const int8_t *argmax, float *delta, const void *X,
+                                  const void *W, long long B, long long Cin, long long Cout, long long H, long long Wd,
+                                  int k, int pad, unsigned long long seed, float scale, const float *delta_in,
+                                  dbp_sparse *q_out, float *dW, void *dX, float *db, unsigned flags);
+
+/*
  * Host-buffer variants: every pointer (delta, X, W, dW, dX, db, and the two scalars) is a
  * HOST pointer. The call copies the inputs to the device workspace, runs the same kernels,
  * copies the results back and synchronises. delta_out / nnz_out (may be NULL) receive the

@@ -221,6 +221,7 @@ int gather_backward(dbp_ctx *ctx, const void *delta, const void *X, const void *
     }
     const bool direct = !(flags & DBP_FORCE_SPARSE) && direct5_supported(s, dW != nullptr, dX != nullptr);
     SideJobs jobs;
+    jobs.pool = ctx->pooled;
     if (direct && dW) { jobs.zero = dW; jobs.zero_bytes = sizeof(float) * static_cast<size_t>(s.Cout) * s.Cin * 25; }
     // a *_host call: X is still on its way up on another stream
     if (direct && dW && ctx->hook_before_dw && cudaStreamWaitEvent(ctx->stream, ctx->hook_before_dw, 0) != cudaSuccess) return DBP_ECUDA;
@@ -953,6 +954,34 @@ int dithered_conv_backward(dbp_ctx *ctx, const void *delta, const void *X, const
     if (!conv_form_supported(k, stride, pad)) return DBP_EUNSUPPORTED;
     ConvShape s{B, Cin, Cout, H, Wd, k};
     return conv_backward_any(ctx, delta, X, W, io, s, stride, seed, scale, delta_in, q_out, dW, dX, db, flags);
+}
+
+int dithered_conv_backward_pooled(dbp_ctx *ctx, const float *g, const int8_t *argmax, float *delta, const void *X, const void *W,
+                                  long long B, long long Cin, long long Cout, long long H, long long Wd, int k, int pad,
+                                  unsigned long long seed, float scale, const float *delta_in, dbp_sparse *q_out, float *dW, void *dX,
+                                  float *db, unsigned flags) {
+    const MaskUse mask_use{ctx};
+    if (!ctx || !g || !argmax || !delta) return DBP_EINVAL;
+    if (!conv_form_supported(k, 1, pad)) return DBP_EUNSUPPORTED;
+    if (B <= 0 || Cout <= 0 || H <= 0 || Wd <= 0) return DBP_EINVAL;
+    if ((H & 1) || (Wd & 1)) return DBP_EUNSUPPORTED;
+    const ConvShape s{B, Cin, Cout, H, Wd, k};
+    // By the statistics kernel where what follows it is the flat quantizer (the 5x5 kernels): rows of whole vectors, masks that
+    // are folded into the loads, a step size to be found. Else by the routing kernel in front of everything.
+    const bool fold = k == 5 && Wd % 4 == 0 && scale > 0.f && !q_out && (dW || dX) && !(flags & DBP_FORCE_SPARSE) && Cin > 0 &&
+                      direct5_supported(s, dW != nullptr, dX != nullptr) &&
+                      ((reinterpret_cast<uintptr_t>(ctx->next_mask) & 3) | (reinterpret_cast<uintptr_t>(g) & 7) | (reinterpret_cast<uintptr_t>(argmax) & 1)) == 0;
+    if (!fold) {
+        DeviceGuard guard(ctx->device);
+        if (!guard.ok) return DBP_ECUDA;
+        KernelTimer t(ctx, DBP_K_GLUE);
+        if (int rc = launch_maxpool_backward(ctx, g, argmax, delta, B * Cout, H / 2, Wd / 2)) return rc;
+    } else {
+        ctx->pooled = PoolRouting{g, argmax, delta, static_cast<int>(Wd / 2)};
+    }
+    const int rc = conv_backward_impl(ctx, delta, X, W, DBP_F32, s, seed, scale, delta_in, q_out, dW, dX, db, flags);
+    ctx->pooled = PoolRouting{};
+    return rc;
 }
 
 static int host_backward(dbp_ctx *ctx, const void *delta, const void *X, const void *W, int io,

@@ -43,6 +43,15 @@ struct StridedLayer {
     int H, W, phases;
 };
 
+// The gradient is routed from a pooled one by the statistics kernel, which writes it and adds it up in one pass: planes of
+// 2h x 2w elements, w even.
+struct PoolRouting {
+    const float *g = nullptr;          // [planes][h][w]; null: the gradient is there
+    const int8_t *argmax = nullptr;
+    float *out = nullptr;
+    int w = 0;
+};
+
 }  // namespace dbp
 
 struct dbp_ctx {
@@ -62,6 +71,7 @@ struct dbp_ctx {
     dbp::Workspace codes16[2];          // bf16 code planes for the TMA-fed kernels
     dbp::Workspace w_taps;              // fp32 weights as [Cout][k*k][Cin]
     dbp::Workspace codes_nhwc[2];       // bf16 codes [B][position][Cout] for the TMA-fed 3x3 kernels
+    dbp::PoolRouting pooled;            // set while dithered_conv_backward_pooled runs a call whose statistics kernel routes the gradient
     const uint8_t *next_mask = nullptr; // ReLU mask for the next backward call (dbp_set_relu_mask)
     dbp::Workspace dz_tmp;              // delta_z = delta_a (.) mask when that call cannot fold the mask into its loads
     dbp::Workspace codes_stack[2];      // the same codes with G images stacked into one tall image (tiny planes, dW)
@@ -120,6 +130,7 @@ struct StepSource {
     int nparts = 0;
     double inv_numel = 0;
     float scale = 0.f;
+    int late = 0;                       // the statistics kernel writes the gradient: it is read behind the wait for that kernel
     float *publish[3] = {nullptr, nullptr, nullptr};   // where the quantizer writes it for the kernels behind it
 };
 
@@ -137,6 +148,7 @@ struct RowsJob {
     long long rows = 0, cols = 0, pitch = 0;
 };
 struct SideJobs {
+    PoolRouting pool;                  // (the only jobs beside it: clearing a buffer)
     RowsJob rows[2];
     int nrows = 0;
     void *zero = nullptr;

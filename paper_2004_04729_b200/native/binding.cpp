@@ -88,13 +88,18 @@ int linear(const Call &c, const at::Tensor &delta, const at::Tensor &X, const at
                                     c.q, static_cast<float *>(ptr(dW)), ptr(dX), static_cast<float *>(ptr(db)), c.flags);
 }
 
+// g, argmax: not null where delta is to be routed from a pooled gradient (fp32)
 int conv(const Call &c, const at::Tensor &delta, const at::Tensor &X, const at::Tensor &W, int io, int stride, int pad, at::Tensor &dW,
-         at::Tensor &dX, at::Tensor &db) {
+         at::Tensor &dX, at::Tensor &db, const at::Tensor *g = nullptr, const at::Tensor *argmax = nullptr) {
     NoGil nogil;
     const int64_t B = delta.size(0), Co = delta.size(1), Ci = X.size(1), H = X.size(2), Wd = X.size(3), k = W.size(2);
     if (c.need_dW) dW = empty_on(delta, {Co, Ci, k, k}, at::kFloat);
     if (c.need_dX) dX = empty_on(delta, {B, Ci, H, Wd}, (c.flags & DBP_DX_F32) ? at::kFloat : delta.scalar_type());
     if (c.need_db) db = empty_on(delta, {Co}, at::kFloat);
+    if (g)
+        return dithered_conv_backward_pooled(c.ctx, static_cast<const float *>(g->data_ptr()), static_cast<const int8_t *>(argmax->data_ptr()),
+                                             static_cast<float *>(delta.data_ptr()), X.data_ptr(), W.data_ptr(), B, Ci, Co, H, Wd, static_cast<int>(k),
+                                             pad, c.seed, c.scale, c.delta_in, c.q, static_cast<float *>(ptr(dW)), ptr(dX), static_cast<float *>(ptr(db)), c.flags);
     return dithered_conv_backward(c.ctx, delta.data_ptr(), X.data_ptr(), W.data_ptr(), io, B, Ci, Co, H, Wd, static_cast<int>(k),
                                   stride, pad, c.seed, c.scale, c.delta_in, c.q, static_cast<float *>(ptr(dW)), ptr(dX),
                                   static_cast<float *>(ptr(db)), c.flags);
@@ -259,7 +264,7 @@ PyObject *network(PyObject *const *a, Py_ssize_t n) {
     if (!on_device(*d0) || d0->scalar_type() != at::kFloat) return none();
     Owned res(PyList_New(L));
     if (!res.o) return nullptr;
-    at::Tensor delta = *d0;
+    at::Tensor delta = *d0, pooled;                  // pooled: what delta is to be routed from
     for (Py_ssize_t l = L - 1; l >= 0; --l) {
         const Layer &y = layers[l];
         int rc = 0;
@@ -274,7 +279,8 @@ PyObject *network(PyObject *const *a, Py_ssize_t n) {
         c.need_dX = l > 0 || first_dX;
         at::Tensor dW, dX, db;
         if (!rc)
-            rc = y.conv ? conv(c, delta, *y.X, *y.W, DBP_F32, 1, static_cast<int>((y.W->size(2) - 1) / 2), dW, dX, db)
+            rc = y.conv ? conv(c, delta, *y.X, *y.W, DBP_F32, 1, static_cast<int>((y.W->size(2) - 1) / 2), dW, dX, db,
+                             pooled.defined() ? &pooled : nullptr, y.pool)
                         : linear(c, delta, *y.X, *y.W, DBP_F32, dW, dX, db);
         if (rc) return PyLong_FromLong(rc);
         Owned d(result(dW, dX, db));
@@ -283,19 +289,18 @@ PyObject *network(PyObject *const *a, Py_ssize_t n) {
         if (l == 0) break;
         const Layer &below = layers[l - 1];
         delta = dX;
+        pooled.reset();
         if (!y.conv && below.conv) {
             const at::Tensor &s = below.pool ? *below.pool : *below.mask;
             delta = dX.view({below.mask->size(0), below.mask->size(1), s.size(2), s.size(3)});
         }
         if (below.pool) {
-            at::Tensor routed;
             if (delta.dim() != 4 || below.pool->numel() != delta.numel()) {
                 PyErr_SetString(PyExc_ValueError, "shapes of a pool and its gradient differ");
                 return nullptr;
             }
-            rc = maxpool(c.ctx, delta, *below.pool, routed);
-            if (rc) return PyLong_FromLong(rc);
-            delta = routed;
+            pooled = delta;
+            delta = empty_on(pooled, {pooled.size(0), pooled.size(1), 2 * pooled.size(2), 2 * pooled.size(3)}, pooled.scalar_type());
         }
     }
     return res.release();

@@ -55,3 +55,33 @@ def test_layers_of_few_channels(ctx, B, Ci, Co, H, W, dtype):
     (150, 12, 32, 18, 18, "f32"), (299, 2, 16, 9, 12, "bf16")])
 def test_more_images_than_sms(ctx, B, Ci, Co, H, W, dtype):
     test_layers_of_few_channels(ctx, B, Ci, Co, H, W, dtype)
+
+
+@pytest.mark.parametrize("B,Ci,Co,H,W", [(3, 6, 16, 16, 16), (5, 1, 6, 32, 28), (2, 3, 5, 6, 8), (1, 2, 1, 2, 4), (150, 4, 12, 12, 12),
+                                         (2, 3, 5, 8, 10)])          # (rows that are no whole vectors: routed first)
+def test_gradient_routed_by_the_statistics(ctx, B, Ci, Co, H, W):
+    """A network's 5x5 layer below a pool: the same step size, count and products as from the routed gradient. (The step size is
+    rounded from sums in another order: 1e-6; where its bits are the same, so are the codes, and the products are sums of the same
+    terms: fp32 sums agree to 1e-5.)"""
+    import paper_2004_04729_b200 as dbp
+    g = torch.Generator(device="cuda").manual_seed(B + 7 * Co + H)
+    rnd = lambda *s: torch.randn(*s, generator=g, device="cuda")
+    mask = (torch.rand(B, Co, H, W, generator=g, device="cuda") < 0.6).to(torch.uint8)
+    argmax = torch.randint(0, 4, (B, Co, H // 2, W // 2), generator=g, device="cuda", dtype=torch.int8)
+    X, Wt, n = rnd(B, Ci, H, W), rnd(Co, Ci, 5, 5), Co * (H // 2) * (W // 2)
+    X2, W2, top = rnd(B, n), rnd(10, n) / n ** 0.5, rnd(B, 10)
+    net = dbp.network_backward(ctx, ["conv", "linear"], [X, X2], [Wt, W2], [mask, None], [argmax, None], top, 2.0, 5,
+                               first_layer_dX=True, with_sparse=False)
+    step = ctx.last_step()
+    above = dbp.dithered_linear_backward(ctx, top, X2, W2, dbp.layer_seed(5, 1), 2.0)
+    assert torch.equal(above["dX"], net[1]["dX"])
+    routed = dbp.maxpool2x2_backward(ctx, above["dX"].view(argmax.shape), argmax)
+    ctx.set_relu_mask(mask)
+    ref = dbp.dithered_conv_backward(ctx, routed, X, Wt, dbp.layer_seed(5, 0), 2.0)
+    want = ctx.last_step()
+    assert abs(step[0] - want[0]) <= 1e-6 * want[0]
+    if step[0] == want[0]:
+        assert step[1] == want[1]
+        for key in ("dW", "dX"):
+            assert (net[0][key] - ref[key]).norm().item() <= TOL * ref[key].norm().item(), key
+    assert ctx.last_device_status() == (0, 0)
