@@ -5,7 +5,9 @@
 //
 // `beside`: the kernel before this one on the stream writes nothing this one reads and has let it start when all of its
 // CTAs had seen everything before them complete. Such a call works first, beside that kernel (a product, bound by the
-// tensor pipe or by its stores), and waits for it only before it ends, so that whatever comes behind waits for both.
+// tensor pipe or by its stores), and waits for it only before it ends, so that whatever comes behind waits for both. One block does:
+// where all did, the blocks that the product's CTAs leave room for held it until the product was done and the others ran behind it
+// (1024 -> 4096 bf16, batch 4096, with its bias gradient: 85.2 us, 79.4 so).
 #include "dbp_internal.cuh"
 
 namespace dbp {
@@ -85,7 +87,7 @@ column_sums_kernel(const unsigned short *__restrict__ codes, long long rows, int
     } else if (threadIdx.x < 64 && c < cols) {
         db[c] = static_cast<float>(total) * (*delta_p);
     }
-    if (beside) chain_wait();
+    if (beside && blockIdx.x == 0 && blockIdx.y == 0) chain_wait();
 }
 
 // Planes [image][channel][pitch]: a block owns one channel and a range of images, a warp one plane at a time.
@@ -133,7 +135,7 @@ plane_sums_kernel(const unsigned short *__restrict__ codes, int B, long long hw,
         }
         if (last) db[blockIdx.x] = static_cast<float>(total) * (*delta_p);
     }
-    if (beside) chain_wait();
+    if (beside && blockIdx.x == 0 && blockIdx.y == 0) chain_wait();
 }
 
 // counters (zero between calls) at the start of the workspace, partial sums after them

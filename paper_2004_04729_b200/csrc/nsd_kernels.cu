@@ -120,12 +120,15 @@ __device__ __forceinline__ void rows_job(const RowsJob &j, long long first, long
 
 // beside: the kernel before this one on the stream writes nothing this one reads (the quantizer, whose CTAs let this
 // kernel start once they have seen everything before them complete): it works beside that kernel, whose issue slots are
-// what is busy, and waits for it only before it ends, so that the kernels behind this one still come after both.
+// what is busy, and waits for it only before it ends, so that the kernels behind this one still come after both. For that one waiting
+// block is enough, and the others leave their places to blocks that found none (fp32 rows: VGG-16 layer set 683 us with all of them
+// waiting, 677 so); of bf16 rows all wait, which keeps dX's CTAs from taking the SMs in front of an earlier call's dW
+// (ResNet-50 layer set 841 us, 845 with one).
 __global__ void __launch_bounds__(kThreads) rows_job_kernel(const RowsJob j, int beside) {
     if (!beside) chain_wait();
     chain_release();
     rows_job(j, static_cast<long long>(blockIdx.x) * kThreads + threadIdx.x, static_cast<long long>(gridDim.x) * kThreads);
-    if (beside) chain_wait();
+    if (beside && (blockIdx.x == 0 || !j.f32)) chain_wait();
 }
 
 // a block's sums

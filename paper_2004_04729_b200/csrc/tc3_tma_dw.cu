@@ -437,7 +437,7 @@ tc3_dw_finish_kernel(float *__restrict__ acc, const float *__restrict__ delta_p,
 // after the other: the values rounded to bf16 and what that rounding left over, rounded again. out is
 // [2][B / G][Cin][pitch] with G (H + 1) W positions per tall image; position q of tall image t is position
 // q % ((H + 1) W) of image t G + q / ((H + 1) W), or zero in the extra row and in the padding.
-// beside: see rows_job_kernel (nsd_kernels.cu).
+// beside: see rows_job_kernel (nsd_kernels.cu); one block waits.
 // A thread takes eight consecutive positions of one tall image's row: index arithmetic in 32 bits, one division per row and
 // then step and wrap, one 16-byte store per piece (the previous form, a position per thread with 64-bit divisions, took 25 to
 // 50 us beside a dX kernel at 512 channels of 4x4; the data are 4 MB).
@@ -471,7 +471,7 @@ x_split_stacked_kernel(const float *__restrict__ X, __nv_bfloat16 *__restrict__ 
         *reinterpret_cast<uint4 *>(out + o) = make_uint4(h[0], h[1], h[2], h[3]);
         *reinterpret_cast<uint4 *>(out + piece + o) = make_uint4(l[0], l[1], l[2], l[3]);
     }
-    if (beside) chain_wait();
+    if (beside && blockIdx.x == 0) chain_wait();
 }
 
 int round_up(int v, int m) { return (v + m - 1) / m * m; }
