@@ -117,13 +117,14 @@ quantize_dense_kernel(const T *__restrict__ x, long long n, unsigned long long s
 #pragma unroll
         for (int k = 0; k < NV; ++k) dithers_at<V>(zz + k * kBetweenZ, u[k]);
     };
-    if (!step.late) load(t, e0);
+    const bool late = SINK == kBytes && step.late;                     // (only the 5x5 layers' gradients are written by the statistics kernel)
+    if (!late) load(t, e0);
     draw(z);
     keep_here(u);
     const StepSource from = step_ahead(step);
     chain_wait();
     chain_release();
-    if (step.late) load(t, e0);
+    if (late) load(t, e0);
     const float delta = step_of<kThreads>(from, st);
     const float inv = delta > 0.f ? __fdiv_rn(1.0f, delta) : 0.f;      // Delta = 0: x * 0 + u < 1, every code 0 (NaN too)
     unsigned sat = 0, nz2 = 0, nnz = 0;
