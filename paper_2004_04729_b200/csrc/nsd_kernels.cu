@@ -42,6 +42,9 @@ __device__ __forceinline__ void mask4(const unsigned char *, long long, float (&
 // Rows of a matrix re-written as bf16 rows of `pitch` values (a multiple of 8, the extra columns zero): bf16 rows
 // copied, fp32 rows as two pieces, [rows][pitch] the rounded values and, rows * pitch further on, what the rounding
 // left over, rounded again. A thread takes eight columns of one row.
+// ODD: fp32 rows may start on any element; an instance of its own, because its registers keep blocks of the others out of places beside
+// other kernels (38 and 32; ResNet-50 layer set 844 us in one kernel, 839 in two, 64 -> 64 fp32 at 32x32 80.7 and 79.5).
+template <bool ODD>
 __device__ __forceinline__ void rows_job(const RowsJob &j, long long first, long long stride) {
     const unsigned gpr = static_cast<unsigned>(j.pitch / 8);
     const long long n = j.rows * gpr, piece = j.rows * j.pitch;
@@ -68,7 +71,7 @@ __device__ __forceinline__ void rows_job(const RowsJob &j, long long first, long
                 // of 275 outputs of 3761 inputs, batch 31, takes 20.7 us, 19.2 so)
                 const long long off = row * j.cols + c0, at = off & ~3ll;
                 const int sh = static_cast<int>(off & 3);
-                if (at + 12 <= j.rows * j.cols) {
+                if (ODD && at + 12 <= j.rows * j.cols) {
                     const float4 *const p4 = reinterpret_cast<const float4 *>(static_cast<const float *>(j.src) + at);
                     const float4 a = __ldg(p4), b = __ldg(p4 + 1), c = __ldg(p4 + 2);
                     const float w[12] = {a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w, c.x, c.y, c.z, c.w};
@@ -139,10 +142,11 @@ __device__ __forceinline__ void rows_job(const RowsJob &j, long long first, long
 // block is enough, and the others leave their places to blocks that found none (fp32 rows: VGG-16 layer set 683 us with all of them
 // waiting, 677 so); of bf16 rows all wait, which keeps dX's CTAs from taking the SMs in front of an earlier call's dW
 // (ResNet-50 layer set 841 us, 845 with one).
+template <bool ODD>
 __global__ void __launch_bounds__(kThreads) rows_job_kernel(const RowsJob j, int beside) {
     if (!beside) chain_wait();
     chain_release();
-    rows_job(j, static_cast<long long>(blockIdx.x) * kThreads + threadIdx.x, static_cast<long long>(gridDim.x) * kThreads);
+    rows_job<ODD>(j, static_cast<long long>(blockIdx.x) * kThreads + threadIdx.x, static_cast<long long>(gridDim.x) * kThreads);
     if (beside && (blockIdx.x == 0 || !j.f32)) chain_wait();
 }
 
@@ -192,7 +196,7 @@ statistics_kernel(const T *__restrict__ x, long long n, double *__restrict__ par
         for (long long i = first; i < zero_n16; i += step) static_cast<uint4 *>(jobs.zero)[i] = make_uint4(0u, 0u, 0u, 0u);
         if (first < static_cast<long long>(jobs.zero_bytes / 4) - 4 * zero_n16) static_cast<unsigned *>(jobs.zero)[4 * zero_n16 + first] = 0u;
         // side jobs for the layer's product kernels: operands re-written as bf16 rows the copy engine can address
-        for (int j = 0; j < jobs.nrows; ++j) rows_job(jobs.rows[j], first, step);
+        for (int j = 0; j < jobs.nrows; ++j) rows_job<true>(jobs.rows[j], first, step);
     }
     // side job for the layer's 3x3 input-gradient kernel: weights [co][ci][9] -> [tap][co][ci] bf16 (for fp32
     // weights two pieces: taps 0-8 the values rounded to bf16, taps 9-17 the remainders rounded to bf16).
@@ -595,7 +599,8 @@ decode_kernel(const uint32_t *__restrict__ bitmap, const uint16_t *__restrict__ 
 int launch_rows_job(dbp_ctx *ctx, const RowsJob &job, bool beside) {
     long long b = (job.rows * (job.pitch / 8) + kThreads - 1) / kThreads;
     if (b > static_cast<long long>(ctx->sm_count) * 8) b = static_cast<long long>(ctx->sm_count) * 8;
-    return cuda_ok(launch_chained(rows_job_kernel, dim3(static_cast<unsigned>(b)), dim3(kThreads), 0, ctx->stream, job, beside ? 1 : 0));
+    const bool odd = job.f32 && (job.cols & 3) != 0;
+    return cuda_ok(launch_chained(odd ? rows_job_kernel<true> : rows_job_kernel<false>, dim3(static_cast<unsigned>(b)), dim3(kThreads), 0, ctx->stream, job, beside ? 1 : 0));
 }
 
 int launch_statistics(dbp_ctx *ctx, const void *delta, int dtype, long long numel, float scale,
