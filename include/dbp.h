@@ -276,8 +276,9 @@ int dithered_conv_backward(dbp_ctx *ctx, const void *delta, const void *X, const
 /*
  * The same where a 2x2 max-pool follows the layer and the gradient at hand is that of the pooled output: `g`
  * [B,Cout,H/2,W/2] goes through its routing (`argmax`, as for dbp_maxpool2x2_backward) into `delta` [B,Cout,H,W], a buffer
- * that the call overwrites, which then is the layer's gradient. fp32, stride 1, H and Wd even. Layers of few channels with
- * 5x5 kernels are routed by the kernel that takes the statistics.
+ * that the call overwrites, which then is the layer's gradient (a call that is refused leaves it alone). fp32, stride 1, H and Wd
+ * even. delta starts on a 16-byte boundary, g on a 4-byte one, argmax anywhere. Layers of few channels with 5x5 kernels are
+ * routed by the kernel that takes the statistics.
  */
 int dithered_conv_backward_pooled(dbp_ctx *ctx, const float *g, const int8_t *argmax, float *delta, const void *X,
                                   const void *W, long long B, long long Cin, long long Cout, long long H, long long Wd,

@@ -74,6 +74,8 @@ def load_library():
                                              ctypes.POINTER(_Sparse), vp, vp, vp, u32]
     lib.dithered_conv_backward.argtypes = [vp, vp, vp, vp, i32, ll, ll, ll, ll, ll, i32, i32, i32,
                                            ull, f32, vp, ctypes.POINTER(_Sparse), vp, vp, vp, u32]
+    lib.dithered_conv_backward_pooled.argtypes = [vp, vp, vp, vp, vp, vp, ll, ll, ll, ll, ll, i32, i32,
+                                                  ull, f32, vp, ctypes.POINTER(_Sparse), vp, vp, vp, u32]
     lib.dithered_linear_backward_host.argtypes = [vp, vp, vp, vp, i32, ll, ll, ll, ull, f32,
                                                   vp, vp, vp, u32, ctypes.POINTER(f32),
                                                   ctypes.POINTER(ll)]

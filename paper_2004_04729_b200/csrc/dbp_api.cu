@@ -76,6 +76,11 @@ int wait_code_set(dbp_ctx *ctx) {
     return DBP_OK;
 }
 
+int check_sparse(const dbp_sparse &q) {
+    if (!q.bitmap || !q.offsets || !q.values || !q.delta || !q.nnz) return DBP_EINVAL;
+    return aligned16(q.bitmap) && aligned16(q.offsets) && aligned16(q.values) ? DBP_OK : DBP_EINVAL;
+}
+
 // Quantize delta into `sp` (caller's arrays, or the context's internal ones) and into the
 // context's dense code buffer, which the product kernels read.
 int quantize_for_products(dbp_ctx *ctx, const void *delta, int dtype, long long numel,
@@ -90,8 +95,7 @@ int quantize_for_products(dbp_ctx *ctx, const void *delta, int dtype, long long 
     sp.bitmap = nullptr; sp.offsets = nullptr; sp.values = nullptr; sp.delta = nullptr; sp.nnz = nullptr;
     sp.numel = numel;
     if (q_out) {
-        if (!q_out->bitmap || !q_out->offsets || !q_out->values || !q_out->delta || !q_out->nnz) return DBP_EINVAL;
-        if (!aligned16(q_out->bitmap) || !aligned16(q_out->offsets) || !aligned16(q_out->values)) return DBP_EINVAL;
+        if ((rc = check_sparse(*q_out))) return rc;
         q_out->numel = numel;
         sp = *q_out;
     }
@@ -276,6 +280,30 @@ int gather_backward(dbp_ctx *ctx, const void *delta, const void *X, const void *
     return DBP_OK;
 }
 
+// What the tensor-core kernels take: linear layers, 1x1 and 3x3 layers of either type and any channel counts
+struct DenseForms { bool linear, conv1, conv3; };
+
+// What of a layer's call can be refused before anything is launched
+int check_conv(const void *delta, const void *X, const void *W, int io, const ConvShape &s, float scale, const float *delta_in,
+               const float *dW, const void *dX, unsigned flags, bool masked, DenseForms *forms) {
+    if (!delta || (io != DBP_F32 && io != DBP_BF16)) return DBP_EINVAL;
+    if (s.B <= 0 || s.Cin <= 0 || s.Cout <= 0 || s.H <= 0 || s.W <= 0) return DBP_EINVAL;
+    if (s.B > 65535 * 32 || s.Cin > (1 << 20) || s.Cout > (1 << 20) || s.H > 4096 || s.W > 4096) return DBP_EINVAL;
+    if (!(scale > 0.f) && !delta_in) return DBP_EINVAL;
+    if ((dW && !X) || (dX && !W)) return DBP_EINVAL;
+    if (!aligned16(delta) || !aligned16(X) || !aligned16(W) || !aligned16(dW) || !aligned16(dX)) return DBP_EINVAL;
+    if ((flags & DBP_FORCE_SPARSE) && (flags & DBP_FORCE_DENSE)) return DBP_EINVAL;
+    forms->linear = s.k == 1 && s.H == 1 && s.W == 1 && linear_tc_supported(s.B, s.Cout, s.Cin);
+    forms->conv1 = tma_dx_supported(s, io);
+    forms->conv3 = tc3_tma_supported(s, io, dX && !(flags & DBP_FORCE_DENSE) && (io == DBP_F32 || (flags & DBP_DX_F32)));
+    // DBP_FORCE_DENSE keeps its documented range: channel counts that are multiples of 8 (of an fp32 3x3 layer's weight
+    // gradient alone, only the output channels), and no fp32 linear or 1x1 layers
+    const bool force_ok = s.k == 1 ? io == DBP_BF16 && s.Cin % 8 == 0
+                                   : s.Cout % 8 == 0 && (s.Cin % 8 == 0 || (io == DBP_F32 && dW && !dX));
+    if ((flags & DBP_FORCE_DENSE) && !((forms->linear || forms->conv1 || forms->conv3) && force_ok)) return DBP_EUNSUPPORTED;
+    return masked && io != DBP_F32 ? DBP_EUNSUPPORTED : DBP_OK;
+}
+
 int conv_backward_impl(dbp_ctx *ctx, const void *delta, const void *X, const void *W, int io,
                        const ConvShape &s, unsigned long long seed, float scale,
                        const float *delta_in, dbp_sparse *q_out, float *dW, void *dX, float *db,
@@ -284,28 +312,14 @@ int conv_backward_impl(dbp_ctx *ctx, const void *delta, const void *X, const voi
     // a ReLU mask set for this call: consumed here whatever happens next
     const uint8_t *mask = ctx->next_mask;
     ctx->next_mask = nullptr;
-    if (io != DBP_F32 && io != DBP_BF16) return DBP_EINVAL;
-    if (s.B <= 0 || s.Cin <= 0 || s.Cout <= 0 || s.H <= 0 || s.W <= 0) return DBP_EINVAL;
-    if (s.B > 65535 * 32 || s.Cin > (1 << 20) || s.Cout > (1 << 20) || s.H > 4096 || s.W > 4096) return DBP_EINVAL;
-    if (!(scale > 0.f) && !delta_in) return DBP_EINVAL;
-    if ((dW && !X) || (dX && !W)) return DBP_EINVAL;
-    if (!aligned16(delta) || !aligned16(X) || !aligned16(W) || !aligned16(dW) || !aligned16(dX)) return DBP_EINVAL;
-    if ((flags & DBP_FORCE_SPARSE) && (flags & DBP_FORCE_DENSE)) return DBP_EINVAL;
-    // What the tensor-core kernels take: linear layers, 1x1 and 3x3 layers of either type and any channel counts
-    const bool linear = s.k == 1 && s.H == 1 && s.W == 1 && linear_tc_supported(s.B, s.Cout, s.Cin);
-    const bool conv1 = tma_dx_supported(s, io), conv3 = tc3_tma_supported(s, io, dX && !(flags & DBP_FORCE_DENSE) && (io == DBP_F32 || (flags & DBP_DX_F32)));
-    const bool can_dense = linear || conv1 || conv3;
-    // DBP_FORCE_DENSE keeps its documented range: channel counts that are multiples of 8 (of an fp32 3x3 layer's weight
-    // gradient alone, only the output channels), and no fp32 linear or 1x1 layers
-    const bool force_ok = s.k == 1 ? io == DBP_BF16 && s.Cin % 8 == 0
-                                   : s.Cout % 8 == 0 && (s.Cin % 8 == 0 || (io == DBP_F32 && dW && !dX));
-    if ((flags & DBP_FORCE_DENSE) && !(can_dense && force_ok)) return DBP_EUNSUPPORTED;
+    DenseForms forms;
+    if (int cr = check_conv(delta, X, W, io, s, scale, delta_in, dW, dX, flags, mask != nullptr, &forms)) return cr;
+    const bool linear = forms.linear, conv1 = forms.conv1, conv3 = forms.conv3, can_dense = linear || conv1 || conv3;
     DeviceGuard guard(ctx->device);
     if (!guard.ok) return DBP_ECUDA;
     const long long numel = s.B * s.Cout * s.H * s.W;
     const float *delta_p = nullptr;
     const int8_t *codes = nullptr;
-    if (mask && io != DBP_F32) return DBP_EUNSUPPORTED;
     // Masks are read four bytes at a time where they are folded into a kernel's loads. One that does not start on
     // a 4-byte boundary is applied by the ReLU-derivative kernel here and now, and the call goes on without it.
     if (mask != nullptr && (reinterpret_cast<uintptr_t>(mask) & 3) != 0) {
@@ -963,12 +977,17 @@ int dithered_conv_backward_pooled(dbp_ctx *ctx, const float *g, const int8_t *ar
     const MaskUse mask_use{ctx};
     if (!ctx || !g || !argmax || !delta) return DBP_EINVAL;
     if (!conv_form_supported(k, 1, pad)) return DBP_EUNSUPPORTED;
-    if (B <= 0 || Cout <= 0 || H <= 0 || Wd <= 0) return DBP_EINVAL;
-    if ((H & 1) || (Wd & 1)) return DBP_EUNSUPPORTED;
     const ConvShape s{B, Cin, Cout, H, Wd, k};
+    // everything that the layer's call would refuse, before the routing writes delta
+    DenseForms forms;
+    if (int cr = check_conv(delta, X, W, DBP_F32, s, scale, delta_in, dW, dX, flags, ctx->next_mask != nullptr, &forms)) return cr;
+    if (q_out)
+        if (int cr = check_sparse(*q_out)) return cr;
+    if ((reinterpret_cast<uintptr_t>(g) & 3) != 0) return DBP_EINVAL;
+    if ((H & 1) || (Wd & 1)) return DBP_EUNSUPPORTED;
     // By the statistics kernel where what follows it is the flat quantizer (the 5x5 kernels): rows of whole vectors, masks that
     // are folded into the loads, a step size to be found. Else by the routing kernel in front of everything.
-    const bool fold = k == 5 && Wd % 4 == 0 && scale > 0.f && !q_out && (dW || dX) && !(flags & DBP_FORCE_SPARSE) && Cin > 0 &&
+    const bool fold = k == 5 && Wd % 4 == 0 && scale > 0.f && !q_out && (dW || dX) && !(flags & DBP_FORCE_SPARSE) &&
                       direct5_supported(s, dW != nullptr, dX != nullptr) &&
                       ((reinterpret_cast<uintptr_t>(ctx->next_mask) & 3) | (reinterpret_cast<uintptr_t>(g) & 7) | (reinterpret_cast<uintptr_t>(argmax) & 1)) == 0;
     if (!fold) {

@@ -85,3 +85,48 @@ def test_gradient_routed_by_the_statistics(ctx, B, Ci, Co, H, W):
         for key in ("dW", "dX"):
             assert (net[0][key] - ref[key]).norm().item() <= TOL * ref[key].norm().item(), key
     assert ctx.last_device_status() == (0, 0)
+
+
+def _pooled(ctx, g, argmax, delta, X, Wt, dW=None, dX=None, db=None, *, scale=2.0, delta_in=None, q=None, flags=0, seed=5, sizes=None, address=None,
+            null=()):
+    """The C entry point: nothing of it is checked in Python. `address`: delta's, where it is not the tensor's own."""
+    import paper_2004_04729_b200.binding as b
+    B, Co, H, W = delta.shape
+    at = lambda t: None if t is None else t.data_ptr()
+    s = sizes or (B, X.shape[1], Co, H, W)
+    k = Wt.shape[2]
+    return b.load_library().dithered_conv_backward_pooled(ctx._h, at(g), at(argmax), address or at(delta),
+                                                          None if "X" in null else at(X), None if "W" in null else at(Wt), *s, k, (k - 1) // 2, seed,
+                                                          scale, at(delta_in), q.c() if q else None, at(dW), at(dX), at(db), flags)
+
+
+def _pooled_layer(B, Ci, Co, H, W, k):
+    g = torch.Generator(device="cuda").manual_seed(B + 7 * Co + H + k)
+    rnd = lambda *s: torch.randn(*s, generator=g, device="cuda")
+    argmax = torch.randint(0, 4, (B, Co, H // 2, W // 2), generator=g, device="cuda", dtype=torch.int8)
+    return g, rnd(B, Co, H // 2, W // 2), argmax, rnd(B, Ci, H, W), rnd(Co, Ci, k, k)
+
+
+@pytest.mark.parametrize("k", [1, 3, 5])
+def test_refused_pooled_calls_write_nothing(ctx, k):
+    """What the layer's call refuses is refused before the routing kernel: delta keeps its values and nothing is launched."""
+    import paper_2004_04729_b200 as dbp
+    import paper_2004_04729_b200.binding as b
+    _, g, argmax, X, Wt = _pooled_layer(3, 4, 6, 8, 12, k)
+    room = torch.full((3 * 6 * 8 * 12 + 4,), 7.0, device="cuda")
+    delta = room[:-4].view(3, 6, 8, 12)
+    whole = dict(dW=torch.empty_like(Wt), dX=torch.empty_like(X), q=dbp.SparseGradient(delta.numel()))
+    bad = dbp.SparseGradient(delta.numel())
+    bad._c.values = bad.values.data_ptr() + 1
+    at = delta.data_ptr()
+    torch.cuda.synchronize()
+    before = b.load_library().dbp_kernel_launches()
+    for wrong in (dict(null=("X",)), dict(null=("W",)), dict(flags=dbp.DBP_FORCE_SPARSE | dbp.DBP_FORCE_DENSE), dict(scale=0.0),
+                  dict(scale=float("nan")), dict(address=at + 4), dict(address=at + 8), dict(dW=room[1:]), dict(dX=room[2:]), dict(q=bad),
+                  dict(sizes=(0, 4, 6, 8, 12)), dict(sizes=(3, 0, 6, 8, 12)), dict(sizes=(3, 4, -6, 8, 12)), dict(sizes=(3, 4, 6, 8, 5000))):
+        assert _pooled(ctx, g, argmax, delta, X, Wt, **{**whole, **wrong}) == -1, wrong
+    assert _pooled(ctx, g, argmax, delta, X, Wt, **whole, flags=dbp.DBP_FORCE_DENSE) == -2       # (six output channels)
+    assert _pooled(ctx, g, argmax, delta, X, Wt, **whole, sizes=(3, 4, 6, 7, 12)) == -2
+    assert b.load_library().dbp_kernel_launches() == before
+    torch.cuda.synchronize()
+    assert bool((room == 7.0).all())
