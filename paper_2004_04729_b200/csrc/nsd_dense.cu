@@ -79,7 +79,15 @@ __device__ __forceinline__ void apply_mask(unsigned, float (&)[8]) {}           
 // and every counter of the dither is the first one's plus a constant, and from tile to tile all of them advance by constants.
 constexpr int kPerThread = 16;
 
-template <typename T, bool MASKED, int SINK>
+// A gradient that the statistics kernel writes (LATE) is read behind the wait for it, by loads that are no read-only ones and
+// that the compiler leaves in their places.
+__device__ __forceinline__ uint4 load_written(const void *p) {
+    uint4 v;
+    asm volatile("ld.global.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "l"(p) : "memory");
+    return v;
+}
+
+template <typename T, bool MASKED, int SINK, bool LATE = false>
 __global__ void __launch_bounds__(kThreads, kBlocksPerSM)
 quantize_dense_kernel(const T *__restrict__ x, long long n, unsigned long long seed, const StepSource step,
                       const __grid_constant__ CodeSinks out, DeviceState *__restrict__ st, const unsigned char *__restrict__ mask) {
@@ -97,18 +105,19 @@ quantize_dense_kernel(const T *__restrict__ x, long long n, unsigned long long s
     uint4 raw[NV];
     unsigned msk[MASKED ? NV : 1];
     unsigned long long u[NV][V / 2];
+    auto vec = [&](const T *p) { return LATE ? load_written(p) : Vec<T>::raw(p); };
     auto there = [&](int k) { return static_cast<int>(threadIdx.x) + k * kThreads < ragged; };      // in the tile after the whole ones
     auto load = [&](long long tile, long long e) {
         if (tile < whole) {
 #pragma unroll
             for (int k = 0; k < NV; ++k) {
-                raw[k] = Vec<T>::raw(x + e + k * kBetween);
+                raw[k] = vec(x + e + k * kBetween);
                 if (MASKED) msk[k] = mask_word(mask, e + k * kBetween);
             }
         } else if (tile == whole) {
 #pragma unroll
             for (int k = 0; k < NV; ++k) {
-                raw[k] = there(k) ? Vec<T>::raw(x + e + k * kBetween) : make_uint4(0u, 0u, 0u, 0u);
+                raw[k] = there(k) ? vec(x + e + k * kBetween) : make_uint4(0u, 0u, 0u, 0u);
                 if (MASKED) msk[k] = there(k) ? mask_word(mask, e + k * kBetween) : 0u;
             }
         }
@@ -117,14 +126,13 @@ quantize_dense_kernel(const T *__restrict__ x, long long n, unsigned long long s
 #pragma unroll
         for (int k = 0; k < NV; ++k) dithers_at<V>(zz + k * kBetweenZ, u[k]);
     };
-    const bool late = SINK == kBytes && step.late;                     // (only the 5x5 layers' gradients are written by the statistics kernel)
-    if (!late) load(t, e0);
+    if (!LATE) load(t, e0);
     draw(z);
     keep_here(u);
     const StepSource from = step_ahead(step);
     chain_wait();
     chain_release();
-    if (late) load(t, e0);
+    if (LATE) load(t, e0);
     const float delta = step_of<kThreads>(from, st);
     const float inv = delta > 0.f ? __fdiv_rn(1.0f, delta) : 0.f;      // Delta = 0: x * 0 + u < 1, every code 0 (NaN too)
     unsigned sat = 0, nz2 = 0, nnz = 0;
@@ -183,7 +191,7 @@ quantize_dense_kernel(const T *__restrict__ x, long long n, unsigned long long s
                     float v[V];
                     unsigned long long d[V / 2];
                     unsigned hc[V / 2], mc[V];
-                    Vec<T>::values(Vec<T>::raw(x + e + k * kBetween), v);
+                    Vec<T>::values(vec(x + e + k * kBetween), v);
                     if (MASKED) apply_mask(mask_word(mask, e + k * kBetween), v);
                     dithers_at<V>(z + k * kBetweenZ, d);
                     careful_codes<V>(v, d, inv, hc, mc, sat);
@@ -919,6 +927,10 @@ int launch_quantize_dense(dbp_ctx *ctx, const void *delta, int dtype, long long 
                : m              ? go(quantize_dense_kernel<float, true, S>, xf)
                                 : go(quantize_dense_kernel<float, false, S>, xf);
     };
+    if (step.late) {                             // fp32 gradients of 5x5 layers, whole vectors, one byte per element
+        if (sink != kBytes || dtype != DBP_F32 || numel % 4 != 0) return DBP_EINVAL;
+        return m ? go(quantize_dense_kernel<float, true, kBytes, true>, xf) : go(quantize_dense_kernel<float, false, kBytes, true>, xf);
+    }
     switch (sink) {
         case kBytes: return pick(std::integral_constant<int, kBytes>());
         case kSame: return pick(std::integral_constant<int, kSame>());

@@ -60,9 +60,9 @@ def test_more_images_than_sms(ctx, B, Ci, Co, H, W, dtype):
 @pytest.mark.parametrize("B,Ci,Co,H,W", [(3, 6, 16, 16, 16), (5, 1, 6, 32, 28), (2, 3, 5, 6, 8), (1, 2, 1, 2, 4), (150, 4, 12, 12, 12),
                                          (2, 3, 5, 8, 10)])          # (rows that are no whole vectors: routed first)
 def test_gradient_routed_by_the_statistics(ctx, B, Ci, Co, H, W):
-    """A network's 5x5 layer below a pool: the same step size, count and products as from the routed gradient. (The step size is
-    rounded from sums in another order: 1e-6; where its bits are the same, so are the codes, and the products are sums of the same
-    terms: fp32 sums agree to 1e-5.)"""
+    """A network's 5x5 layer below a pool: the step size of the routed gradient (1e-6 of the one in 64 bits), and, with that step
+    size given, the count and the products of the routed gradient (the codes are the same, so the products are sums of the same terms:
+    fp32 sums agree to 1e-5)."""
     import paper_2004_04729_b200 as dbp
     g = torch.Generator(device="cuda").manual_seed(B + 7 * Co + H)
     rnd = lambda *s: torch.randn(*s, generator=g, device="cuda")
@@ -70,20 +70,21 @@ def test_gradient_routed_by_the_statistics(ctx, B, Ci, Co, H, W):
     argmax = torch.randint(0, 4, (B, Co, H // 2, W // 2), generator=g, device="cuda", dtype=torch.int8)
     X, Wt, n = rnd(B, Ci, H, W), rnd(Co, Ci, 5, 5), Co * (H // 2) * (W // 2)
     X2, W2, top = rnd(B, n), rnd(10, n) / n ** 0.5, rnd(B, 10)
-    net = dbp.network_backward(ctx, ["conv", "linear"], [X, X2], [Wt, W2], [mask, None], [argmax, None], top, 2.0, 5,
-                               first_layer_dX=True, with_sparse=False)
-    step = ctx.last_step()
-    above = dbp.dithered_linear_backward(ctx, top, X2, W2, dbp.layer_seed(5, 1), 2.0)
-    assert torch.equal(above["dX"], net[1]["dX"])
-    routed = dbp.maxpool2x2_backward(ctx, above["dX"].view(argmax.shape), argmax)
-    ctx.set_relu_mask(mask)
-    ref = dbp.dithered_conv_backward(ctx, routed, X, Wt, dbp.layer_seed(5, 0), 2.0)
-    want = ctx.last_step()
-    assert abs(step[0] - want[0]) <= 1e-6 * want[0]
-    if step[0] == want[0]:
-        assert step[1] == want[1]
-        for key in ("dW", "dX"):
+    for first_dX in (True, False):
+        net = dbp.network_backward(ctx, ["conv", "linear"], [X, X2], [Wt, W2], [mask, None], [argmax, None], top, 2.0, 5,
+                                   first_layer_dX=first_dX, with_sparse=False)
+        step = ctx.last_step()
+        above = dbp.dithered_linear_backward(ctx, top, X2, W2, dbp.layer_seed(5, 1), 2.0)
+        assert torch.equal(above["dX"], net[1]["dX"])
+        routed = dbp.maxpool2x2_backward(ctx, above["dX"].view(argmax.shape), argmax)
+        want = 2.0 * (routed * mask).double().std(unbiased=False).item()
+        assert abs(step[0] - want) <= 1e-6 * want
+        ctx.set_relu_mask(mask)
+        ref = dbp.dithered_conv_backward(ctx, routed, X, Wt, dbp.layer_seed(5, 0), 0.0, delta_in=torch.tensor([step[0]], device="cuda"))
+        assert step[1] == ctx.last_step()[1]
+        for key in ("dW", "dX") if first_dX else ("dW",):
             assert (net[0][key] - ref[key]).norm().item() <= TOL * ref[key].norm().item(), key
+        assert first_dX or net[0]["dX"] is None
     assert ctx.last_device_status() == (0, 0)
 
 
@@ -130,3 +131,40 @@ def test_refused_pooled_calls_write_nothing(ctx, k):
     assert b.load_library().dbp_kernel_launches() == before
     torch.cuda.synchronize()
     assert bool((room == 7.0).all())
+
+
+@pytest.mark.parametrize("k,B,Ci,Co,H,W,how", [
+    (5, 3, 6, 16, 16, 16, ""), (5, 150, 4, 12, 12, 12, ""), (5, 200, 3, 24, 20, 36, ""),       # routed by the statistics; several tiles a block
+    (5, 4, 2, 5, 8, 8, "mask"), (5, 4, 2, 5, 8, 8, "argmax"), (5, 4, 2, 5, 8, 8, "g"), (5, 4, 2, 5, 8, 10, ""),      # ... not these: routed first
+    (5, 4, 2, 5, 8, 8, "given"), (5, 4, 2, 5, 8, 8, "sparse"), (3, 5, 20, 24, 12, 8, ""), (3, 5, 20, 24, 12, 8, "sparse"), (1, 4, 9, 17, 6, 14, "")])
+def test_pooled_calls(ctx, k, B, Ci, Co, H, W, how):
+    """dithered_conv_backward_pooled against the routed gradient's own call with the same step size: the written delta and the bias
+    gradient are the same bits, the products sums of the same terms (1e-5). The buffer is used again with other gradients, which have to be
+    the ones that are quantized. `how`: the operand that starts off its boundary, or the option that is set."""
+    import paper_2004_04729_b200 as dbp
+    gen, g, argmax, X, Wt = _pooled_layer(B, Ci, Co, H, W, k)
+    delta = torch.full((B, Co, H, W), 9.0, device="cuda")
+    dW, dX, db = torch.empty_like(Wt), torch.empty_like(X), torch.empty(Co, device="cuda")
+    off = lambda t, by: torch.cat([t.new_zeros(int(by)), t.reshape(-1)])[int(by):].view(t.shape)          # starts `by` elements into its storage
+    for turn in range(3):
+        g = torch.randn(g.shape, generator=gen, device="cuda")
+        mask = (torch.rand(B, Co, H, W, generator=gen, device="cuda") < 0.6).to(torch.uint8)
+        am, mk, gg = off(argmax, how == "argmax"), off(mask, how == "mask"), off(g, how == "g")
+        given = torch.tensor([0.5], device="cuda") if how == "given" else None
+        q = dbp.SparseGradient(delta.numel()) if how == "sparse" else None
+        ctx.set_relu_mask(mk)
+        assert _pooled(ctx, gg, am, delta, X, Wt, dW, dX, db, scale=0.0 if how == "given" else 2.0, delta_in=given, q=q, seed=turn) == 0
+        step = ctx.last_step()
+        routed = dbp.maxpool2x2_backward(ctx, g, argmax)
+        assert torch.equal(delta, routed)
+        want = 0.5 if how == "given" else 2.0 * (routed * mask).double().std(unbiased=False).item()
+        assert abs(step[0] - want) <= 1e-6 * want
+        ctx.set_relu_mask(mask)
+        ref = dbp.dithered_conv_backward(ctx, routed, X, Wt, turn, 0.0, delta_in=torch.tensor([step[0]], device="cuda"), need_db=True)
+        assert step[1] == ctx.last_step()[1]
+        assert torch.equal(db, ref["db"])
+        for got, key in ((dW, "dW"), (dX, "dX")):
+            assert (got - ref[key]).norm().item() <= TOL * ref[key].norm().item(), key
+        if q is not None:
+            assert q.nnz.item() == step[1] and q.delta.item() == step[0]
+    assert ctx.last_device_status() == (0, 0)
