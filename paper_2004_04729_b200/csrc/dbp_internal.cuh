@@ -402,6 +402,13 @@ inline cudaError_t launch_chained_cluster(void (*kern)(KArgs...), unsigned ctas,
     note_launch();
     return cudaLaunchKernelEx(&cfg, kern, static_cast<KArgs>(args)...);
 }
+// Dynamic shared memory that a kernel may be launched with. The limit belongs to the function on the device and not to a launch, and
+// threads with a context each set it at the same time: every call sets one value, the most that any launch of the kernel asks for.
+constexpr int kMostShared = 226 * 1024;          // a CTA has 227 KB, 1 KB of them for its own variables
+template <typename Kern>
+inline cudaError_t allow_shared(Kern kern, int most = kMostShared) {
+    return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
+}
 #endif
 
 }  // namespace dbp

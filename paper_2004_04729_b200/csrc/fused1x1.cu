@@ -453,7 +453,7 @@ int launch_fused1x1(dbp_ctx *ctx, const void *delta, const void *X, const void *
         if (!encode_map_f32_sw128(&map_dw, dW, 2, dims, str, box)) return fail_cuda("tensor map of dW");
     }
     auto go = [&](auto kern) -> int {
-        if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem)) != cudaSuccess)
+        if (allow_shared(kern) != cudaSuccess)
             return fail_cuda("shared memory size");
         // One CTA per SM, or as many whole rounds of them as keep a CTA's dW accumulators to kMaxMmas (a chunk is four MMAs)
         const long long most = kMaxMmas / (4 * nch), rounds = (p.ntiles + most * ctx->sm_count - 1) / (most * ctx->sm_count);

@@ -414,7 +414,7 @@ template <int KS, int VEC, typename OutT>
 static int launch_dx_t(dbp_ctx *ctx, const DxParams &p, size_t smem) {
     auto kern = conv_dx_kernel<KS, VEC, OutT>;
     if (smem > 48 * 1024) {
-        cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
+        cudaError_t e = allow_shared(kern, 227 * 1024);
         if (e != cudaSuccess) return DBP_ECUDA;
     }
     const int CI_T = 32 * VEC;
@@ -461,7 +461,7 @@ template <int KS, int CI_T, typename T>
 static int launch_dw_t(dbp_ctx *ctx, const DwParams &p, size_t smem, dim3 grid) {
     auto kern = conv_dw_kernel<KS, CI_T, T>;
     if (smem > 48 * 1024) {
-        cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
+        cudaError_t e = allow_shared(kern, 227 * 1024);
         if (e != cudaSuccess) return DBP_ECUDA;
     }
     note_launch();

@@ -16,6 +16,7 @@ namespace dbp {
 
 namespace {
 
+constexpr int kSharedGather = 220 * 1024;          // dynamic shared memory, at most
 constexpr unsigned kFull = 0xffffffffu;
 constexpr int kWarps = 16;
 constexpr int kThreads = kWarps * 32;
@@ -278,7 +279,7 @@ int launch_one(dbp_ctx *ctx, Dw2Params &p, const ConvShape &s) {
     const int nhp = (p.TH + 2 * PAD) * (p.TW + 2 * PAD);
     const size_t smem = static_cast<size_t>(nhp) * 32 * LB + static_cast<size_t>(CO_T) * p.pt_pad +
                         static_cast<size_t>(p.pt_pad) * (2 + 16) + 16;
-    if (smem > 220 * 1024 || nhp >= 0xffff) return DBP_EUNSUPPORTED;
+    if (smem > kSharedGather || nhp >= 0xffff) return DBP_EUNSUPPORTED;
     const long long out_blocks = ((s.Cout + CO_T - 1) / CO_T) * ((s.Cin + CI_T - 1) / CI_T);
     long long splits = (2LL * ctx->sm_count) / out_blocks;
     if (splits < 1) splits = 1;
@@ -286,7 +287,7 @@ int launch_one(dbp_ctx *ctx, Dw2Params &p, const ConvShape &s) {
     if (splits > 65535) splits = 65535;
     p.splits = static_cast<int>(splits);
     auto kern = conv_dw2_kernel<KS, LB, CPG, XT>;
-    if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem)) != cudaSuccess)
+    if (allow_shared(kern, kSharedGather) != cudaSuccess)
         return DBP_ECUDA;
     dim3 grid(static_cast<unsigned>((s.Cout + CO_T - 1) / CO_T), static_cast<unsigned>((s.Cin + CI_T - 1) / CI_T),
               static_cast<unsigned>(splits));

@@ -16,6 +16,7 @@ namespace dbp {
 
 namespace {
 
+constexpr int kSharedGather = 220 * 1024;          // dynamic shared memory, at most
 constexpr unsigned kFull = 0xffffffffu;
 constexpr int kWarps = 8;
 constexpr int kCC = 32;   // output channels per chunk (one ballot)
@@ -274,9 +275,9 @@ int launch_one(dbp_ctx *ctx, Dx2Params &p, const ConvShape &s) {
                   static_cast<size_t>(kCC) * ps + nhp + 16;
     const size_t stage = static_cast<size_t>(CI_T) * (PT + 1) * 4;
     const size_t smem = work > stage ? work : stage;
-    if (smem > 220 * 1024) return DBP_EUNSUPPORTED;
+    if (smem > kSharedGather) return DBP_EUNSUPPORTED;
     auto kern = conv_dx2_kernel<KS, LB, NPW, WT, OutT>;
-    if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem)) != cudaSuccess)
+    if (allow_shared(kern, kSharedGather) != cudaSuccess)
         return DBP_ECUDA;
     const long long tiles = KS == 1 ? (p.total_rows + PT - 1) / PT
                                     : s.B * p.tiles_y * p.tiles_x;

@@ -345,7 +345,7 @@ int launch_tc3_rows_dx(dbp_ctx *ctx, const RowsPlan &plan, const void *codes_nhw
     }
     const auto kern = small ? tc3_rows_dx_kernel<true> : tc3_rows_dx_kernel<false>;
     if (small) cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
-    if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem)) != cudaSuccess)
+    if (allow_shared(kern) != cudaSuccess)
         return fail_cuda("shared memory size");
     if (p.KS > 1)
         return cuda_ok(launch_chained_cluster(kern, ctas, static_cast<unsigned>(p.KS), dim3(kThreadsR), smem, ctx->stream, map_q, map_w, p));

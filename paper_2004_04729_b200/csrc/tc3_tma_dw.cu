@@ -601,7 +601,7 @@ int launch_tc3_tma_dw(dbp_ctx *ctx, const void *codes_nhwc, const void *X, int p
     }
     if (half) cudaFuncSetAttribute(tc3_tma_dw_kernel<1>, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
     auto kern = NP == 2 ? tc3_tma_dw_kernel<2> : tc3_tma_dw_kernel<1>;
-    if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem)) != cudaSuccess)
+    if (allow_shared(kern) != cudaSuccess)
         return fail_cuda("shared memory size");
     if ((rc = cuda_ok(launch_chained(kern, dim3(static_cast<unsigned>(tiles * nsplit)), dim3(kThreadsW3), smem,
                                      ctx->stream, map_q, map_x, map_acc, p))))

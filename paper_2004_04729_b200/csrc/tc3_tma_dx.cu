@@ -935,7 +935,7 @@ int launch_tc3_tma_dx(dbp_ctx *ctx, const void *codes_nhwc, const void *W, int i
                       : (p.unit > 0 ? tc3_tma_dx_kernel<true, false> : tc3_tma_dx_kernel<false, false>);
     const int threads = small ? kThreads3<true> : kThreads3<false>;
     if (small) cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
-    if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem)) != cudaSuccess)
+    if (allow_shared(kern) != cudaSuccess)
         return fail_cuda("shared memory size");
     if (p.KS > 1)
         return cuda_ok(launch_chained_cluster(kern, static_cast<unsigned>(p.ntiles) * p.KS, static_cast<unsigned>(p.KS),

@@ -76,3 +76,39 @@ def test_weight_gradient_of_a_whole_sm(ctx, B, Ci, Co, H, W, dtype):
         assert np.linalg.norm(g - ref["dW"]) <= TOL * np.linalg.norm(ref["dW"]) + 1e-30
         assert np.all(np.abs(g - ref["dW"]) <= TOL * ref["S_dW"] + 1e-30)
     assert ctx.last_device_status() == (0, 0)
+
+
+def test_threads_launch_the_same_kernels_with_other_sizes():
+    """Two threads, a context and a stream each, with layers whose kernels are the same functions with different amounts of shared
+    memory: every call goes through, and dX has the bits that it has alone (dW's partial sums meet in any order: fp32 sums)."""
+    import threading
+    import paper_2004_04729_b200 as dbp
+    shapes = [[(70, 128, 256, 8, 8), (40, 72, 136, 14, 14), (8, 16, 128, 24, 24)], [(33, 128, 64, 2, 3), (5, 96, 72, 5, 5), (4, 64, 72, 7, 20)]]
+    errors = []
+
+    def work(which):
+        try:
+            stream = torch.cuda.Stream()
+            with torch.cuda.stream(stream):
+                ctx = dbp.Context(0, stream)
+                gen = torch.Generator(device="cuda").manual_seed(which)
+                rnd = lambda *s: torch.randn(*s, generator=gen, device="cuda")
+                layers = [(rnd(B, Co, H, W), rnd(B, Ci, H, W), rnd(Co, Ci, 3, 3)) for B, Ci, Co, H, W in shapes[which]]
+                first = [None] * len(layers)
+                for turn in range(200):
+                    for i, (d, X, Wt) in enumerate(layers):
+                        out = dbp.dithered_conv_backward(ctx, d, X, Wt, 7, 2.0)
+                        if turn % 20 == 0:
+                            if first[i] is None:
+                                first[i] = {k: out[k].clone() for k in ("dX", "dW")}
+                            assert torch.equal(out["dX"], first[i]["dX"])
+                            assert (out["dW"] - first[i]["dW"]).norm().item() <= TOL * first[i]["dW"].norm().item()
+                assert ctx.last_device_status() == (0, 0)
+                ctx.close()
+        except BaseException as e:                       # (an assertion in a thread would be lost)
+            errors.append(e)
+
+    threads = [threading.Thread(target=work, args=(t,)) for t in (0, 1)]
+    for t in threads: t.start()
+    for t in threads: t.join()
+    assert not errors, errors
