@@ -56,7 +56,9 @@ def test_input_gradient(ctx, B, Ci, Co, H, W, dtype):
 @pytest.mark.parametrize("B,Ci,Co,H,W,dtype", [
     (50, 72, 136, 8, 8, "bf16"), (41, 130, 72, 7, 9, "f32"),           # images of one block: several code buffers, ragged channels
     (70, 40, 200, 3, 5, "bf16"), (33, 16, 65, 8, 16, "f32"),           # ... and of two blocks, one output channel past a panel
-    (3, 7, 130, 12, 11, "bf16"), (2, 129, 129, 20, 9, "f32")])         # channels that are no multiple of four in dW's rows
+    (3, 7, 130, 12, 11, "bf16"), (2, 129, 129, 20, 9, "f32"),          # channels that are no multiple of four in dW's rows
+    (2, 1, 65, 5, 4, "f32"), (2, 4, 72, 3, 6, "bf16"), (3, 13, 40, 6, 6, "f32"),      # ... rows of one to four groups of channels, the last one empty
+    (2, 332, 1000, 4, 5, "bf16")])                                     # ... more groups than the finishing kernel has threads
 def test_weight_gradient_of_a_whole_sm(ctx, B, Ci, Co, H, W, dtype):
     """An overlapped call's dW kernel has the SMs to itself. Twice: the second call adds into a scratch that the first put back to zero.
     (Tolerance: fp32 sums of exact products, as above.)"""
