@@ -387,44 +387,43 @@ tc3_tma_dw_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
 // PHASES: a stride-2 layer run on phase images (scratch rows of 4 cin channels, phase ph = 2 py + px at channels
 // ph * cin ...): the strided layer's tap (ky, kx) of (co, ci) is tap (ty, tx) of channel ph * cin + ci with
 // ky = 0 -> (py, ty) = (1, 0), 1 -> (0, 1), 2 -> (1, 1), kx likewise; the other scratch entries were never touched.
-// A thread takes four neighbouring channels of an output channel: nine 16-byte loads (and the zeros written back). Their 36 values
-// follow its neighbour's in dW, whatever rows they belong to and whatever the channel count (channels of the padding are left out):
-// a warp packs them in shared memory and they leave as whole lines. Straight from the threads, 144 bytes apart, they were 9 stores of 32
-// pieces, or 36 where channels are no multiple of eight, 13 us of this kernel at 326 -> 432: bf16, 6x6, batch 22, joined 52.4 us, 41.8 so;
-// fp32 961 -> 224 at 14x15, batch 8, overlapped 79.8, 50.0; of channels that are multiples of eight bf16 784 -> 760 at 10x10, batch 13,
-// joined 85.8, 73.8; VGG-16 layer set 680, 674.5; ResNet-50 842, 835.
-// Few threads: the blocks become resident while the dW kernel still hands over its sums, and what they hold then is missing to the
-// next layer's quantization and dX, which want to start at the same time (seven blocks of 256 threads per SM: VGG-16 layer set 747 us
-// against 735; two blocks of these per SM: 749, eight: 736).
+// A thread takes four neighbouring channels of an output channel: nine 16-byte loads (and the zeros written back), 36 values that
+// follow its neighbour's in dW, whatever rows they belong to and whatever the channel count (channels of the padding are left out).
+// They are handed round within the warp and leave as whole lines. Straight from the threads, 144 bytes apart, they were 9 stores of 32
+// pieces, or 36 where channels are no multiple of eight: bf16 326 -> 432 at 6x6, batch 22, joined 52.4 us, 41.9 so; fp32 961 -> 224 at
+// 14x15, batch 8, overlapped 79.5, 51.6; of channels that are multiples of eight bf16 784 -> 760 at 10x10, batch 13, joined 85.8, 73.0;
+// VGG-16 layer set 680, 664; ResNet-50 841, 835.
+// No shared memory (a dW CTA leaves none: packed there, bf16 128 -> 256 at 20x20, batch 30, dW alone, takes 30.0 us, 26.6 so) and few threads:
+// the blocks become resident while the dW kernel still hands over its sums, and
+// what they hold then is missing to the next layer's quantization and dX, which want to start at the same time (seven blocks of
+// 256 threads per SM: VGG-16 layer set 747 us against 735; two blocks of these per SM: 749, eight: 736).
 constexpr int kThreadsF3 = 128;
 template <bool PHASES, bool VECTORS>                                // VECTORS: channels are a multiple of four, dW leaves 16 bytes a thread
 __global__ void __launch_bounds__(kThreadsF3)
 tc3_dw_finish_kernel(float *__restrict__ acc, const float *__restrict__ delta_p, float *__restrict__ dW, int cout, int cin, int cin_pad) {
-    constexpr int kWords = 32 * 36;
-    __shared__ float4 pack_s[kThreadsF3 / 32][(kWords + kWords / 32) / 4];         // (single words leave every 33rd out: banks)
+    constexpr unsigned kAll = 0xffffffffu;
     const unsigned per_row = (PHASES ? cin : cin_pad) / 4, quads = static_cast<unsigned>(cout) * per_row;      // multiples of four
     const size_t tap = static_cast<size_t>(cout) * cin_pad;         // (PHASES: cin_pad = 4 cin)
     chain_wait();
     chain_release();
     const float delta = *delta_p;
-    const unsigned lane = threadIdx.x & 31;
-    float4 *const pack4 = pack_s[threadIdx.x >> 5];
-    float *const pack = reinterpret_cast<float *>(pack4);
+    const int lane = threadIdx.x & 31, turn = lane % 9;
     for (unsigned i = blockIdx.x * kThreadsF3 + threadIdx.x; i - lane < quads; i += gridDim.x * kThreadsF3) {
         const bool mine = i < quads;
         const unsigned co = i / per_row, ci = (i - co * per_row) * 4;
-        float4 v[9];
         float *const base = acc + static_cast<size_t>(co) * cin_pad + ci;
         auto place = [&](int t) {
             const int ky = t / 3, kx = t % 3;
             const int ph = PHASES ? (ky != 1) * 2 + (kx != 1) : 0, tp = PHASES ? (ky == 0 ? 0 : 1) * 3 + (kx == 0 ? 0 : 1) : t;
             return reinterpret_cast<float4 *>(base + tp * tap + static_cast<size_t>(ph) * cin);
         };
+        float4 v[9];
 #pragma unroll
         for (int t = 0; t < 9; ++t) v[t] = mine ? __ldcg(place(t)) : make_float4(0.f, 0.f, 0.f, 0.f);
+        // where my values go, behind the warp's first one, and how many there are
         const int left = cin - static_cast<int>(ci), words = !mine || left <= 0 ? 0 : left < 4 ? 9 * left : 36;
-        const size_t to = (static_cast<size_t>(co) * cin + (left > 0 ? ci : cin)) * 9, first = __shfl_sync(0xffffffffu, to, 0);
-        const int from = mine ? static_cast<int>(to - first) : 0, total = __reduce_max_sync(0xffffffffu, from + words);
+        const size_t to = (static_cast<size_t>(co) * cin + (left > 0 ? ci : cin)) * 9, first = __shfl_sync(kAll, to, 0);
+        const int from = mine ? static_cast<int>(to - first) : 0;
         float o[36];
 #pragma unroll
         for (int t = 0; t < 9; ++t) {
@@ -434,28 +433,37 @@ tc3_dw_finish_kernel(float *__restrict__ acc, const float *__restrict__ delta_p,
             o[18 + t] = v[t].z * delta;
             o[27 + t] = v[t].w * delta;
         }
-        if (VECTORS) {
+        // Group k (four values) of lane s is the warp's group 9 s + k; lane l stores the groups 32 j + l. Nine is odd, so for one k all lanes
+        // send to different ones: to lane (9 s + k) % 32, from which lane l receives with s = 25 (l - k) % 32 ...
 #pragma unroll
-            for (int k = 0; k < 9; ++k)
-                if (words > 0) pack4[from / 4 + k] = make_float4(o[4 * k], o[4 * k + 1], o[4 * k + 2], o[4 * k + 3]);
-            __syncwarp();
+        for (int k = 0; k < 9; ++k) {
+            const int s = 25 * (lane - k) & 31;
 #pragma unroll
-            for (int j = 0; j < 9; ++j) {
-                const int k = 32 * j + static_cast<int>(lane);
-                if (4 * k < total) reinterpret_cast<float4 *>(dW + first)[k] = pack4[k];
-            }
-        } else {
+            for (int e = 0; e < 4; ++e) o[4 * k + e] = __shfl_sync(kAll, o[4 * k + e], s);
+        }
+        // ... and has the group of its j-th store as k = (5 j + l) % 9: turned by l % 9, that is 5 j % 9 in every lane
 #pragma unroll
-            for (int k = 0; k < 36; ++k)
-                if (k < words) pack[from + k + ((from + k) >> 5)] = o[k];
-            __syncwarp();
-#pragma unroll 12
-            for (int j = 0; j < 36; ++j) {
-                const int k = 32 * j + static_cast<int>(lane);
-                if (k < total) dW[first + k] = pack[33 * j + static_cast<int>(lane)];
+        for (int b = 1; b <= 8; b *= 2) {
+            float r[36];
+#pragma unroll
+            for (int e = 0; e < 36; ++e) r[e] = turn & b ? o[(e + 4 * b) % 36] : o[e];
+#pragma unroll
+            for (int e = 0; e < 36; ++e) o[e] = r[e];
+        }
+#pragma unroll
+        for (int j = 0; j < 9; ++j) {
+            const int g = 32 * j + lane, s = g * 57 >> 9, k = g - 9 * s;                           // s = g / 9
+            const int n = __shfl_sync(kAll, words, s) - 4 * k;
+            float *const out = dW + first + __shfl_sync(kAll, from, s) + 4 * k;
+            const float *const q = o + 4 * (5 * j % 9);
+            if (VECTORS) {
+                if (n > 0) *reinterpret_cast<float4 *>(out) = make_float4(q[0], q[1], q[2], q[3]);
+            } else {
+#pragma unroll
+                for (int e = 0; e < 4; ++e)
+                    if (e < n) out[e] = q[e];
             }
         }
-        __syncwarp();
     }
 }
 
