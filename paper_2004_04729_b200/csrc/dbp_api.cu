@@ -566,7 +566,8 @@ int conv_backward_impl(dbp_ctx *ctx, const void *delta, const void *X, const voi
         ConvShape sw = s;
         if (stack_g > 0) sw = ConvShape{s.B / stack_g, s.Cin, s.Cout, static_cast<long long>(stack_g) * (s.H + 1), s.W, 3};
         rc = t1 ? launch_tma_dw(ctx, codes16, Xp, pieces, x_pitch, delta_p, s, dW, &ctx->state->tc_timeout)
-                : launch_tc3_tma_dw(ctx, stack_g > 0 ? codes_st : codes_n, Xp, pieces, x_pitch, delta_p, sw, dW, &ctx->state->tc_timeout, half);
+                : launch_tc3_tma_dw(ctx, stack_g > 0 ? codes_st : codes_n, Xp, pieces, x_pitch, delta_p, sw, dW, &ctx->state->tc_timeout, half,
+                                    forked && (flags & DBP_DW_ASYNC));
         if (!rc && st2 && s.k == 3 && !ctx->phase_dw_done)
             rc = launch_strided_dw(ctx, dW, st2->dW, s.Cout, st2->Cin);
     }

@@ -257,7 +257,7 @@ constexpr int kRowsLeanCols = 128, kRowsMaxCols = 256;       // accumulator colu
 constexpr size_t kHalfSm = 112 * 1024;
 // X: bf16 planes of x_pitch values, pieces of every image one after the other
 int launch_tc3_tma_dw(dbp_ctx *ctx, const void *codes_nhwc, const void *X, int pieces, long long x_pitch, const float *delta_p,
-                      const ConvShape &s, float *dW, int *err_flag, bool half = false);
+                      const ConvShape &s, float *dW, int *err_flag, bool half, bool overlapped);
 bool tc3_dw_fits_half(const ConvShape &s);
 // fp32 activations split and stacked for it (out: [2][B / G][Cin][pitch]); beside: as for launch_rows_job
 int launch_x_stacked(dbp_ctx *ctx, const float *X, void *out, const ConvShape &s, int stack_g, bool beside);

@@ -547,8 +547,9 @@ int launch_x_stacked(dbp_ctx *ctx, const float *X, void *out, const ConvShape &s
 
 // X: bf16 planes of x_pitch values (a multiple of 8); fp32 activations as two pieces (as if the batch were twice as long).
 // Tiny planes stacked into tall images: `s` describes the tall images and codes and X are their stacked copies.
+// overlapped: the next layer's kernels come beside this one.
 int launch_tc3_tma_dw(dbp_ctx *ctx, const void *codes_nhwc, const void *X, int pieces, long long x_pitch, const float *delta_p,
-                      const ConvShape &s, float *dW, int *err_flag, bool half) {
+                      const ConvShape &s, float *dW, int *err_flag, bool half, bool overlapped) {
     // the scratch's rows are padded to a multiple of 16 bytes
     const long long cin_pad = (s.Cin + 7) / 8 * 8, q_pitch = (s.Cout + 7) / 8 * 8;
     const long long HW = s.H * s.W;
@@ -562,29 +563,53 @@ int launch_tc3_tma_dw(dbp_ctx *ctx, const void *codes_nhwc, const void *X, int p
     const int NP = s.Cout > 64 && !half ? 2 : 1;
     p.ci_tiles = static_cast<int>((cin_pad + 127) / 128);
     p.co_tiles = static_cast<int>((s.Cout + 64 * NP - 1) / (64 * NP));
-    // the longest segment whose two code buffers fit beside at least three activation slots
-    // with 128 output channels 17 KB are left to a block of the next layer's position-major quantizer (VGG-16 layer set 747 us
-    // with, 751 without; 34 KB: 752, 51 KB: 762); the long segments of 64 channels are worth more (64 -> 64 at 32x32: 22.0 us, 24.0)
-    const size_t budget = half ? kHalfSm : (NP == 2 ? 210 : 227) * 1024 - 2048;
-    const int seg_cap = static_cast<int>(HW < 512 ? (HW + 63) / 64 * 64 : 512);
-    size_t smem = 0;
+    // The segment whose copies are the least, of those whose two code buffers fit beside at least three activation slots: every segment
+    // copies its halo too, boxes come whole, and a segment costs about ten rows' time besides. 72 -> 72 fp32 at 14x14, batch 128, with 192
+    // positions (444 rows an image) and 128 (316): 63.6, 60.7 us; 360 -> 112 at 12x12, batch 113, with 128 (308) and 192 (218): 102, 88;
+    // 200 -> 48 at 24x24, batch 43, with 192 instead of 320: 53.4, 51.4. In half an SM, beside two slots, the longest:
+    // 64 -> 64 at 13x13, batch 128, with 64 positions 32.4, with 128 30.8.
     p.xs = HW > 64 ? kXS : 1;
     const size_t x_slot = static_cast<size_t>(p.xs) * kXTile;
-    for (int seg = seg_cap; seg >= 64; seg -= 64) {
+    auto copied = [&](int seg) {                          // rows of codes per image, with what a segment costs
         const Panel pn = panel_of(seg, p.W);
-        const size_t qbuf = static_cast<size_t>(NP) * pn.bytes;
-        size_t fixed = 2 * qbuf + 1024;
-        if (fixed + (half ? 2 : 3) * kXS * kXTile > budget) continue;
-        p.SEG = seg; p.nload = pn.nload; p.rows_box = pn.rows_box; p.panel_bytes = pn.bytes;
-        // short segments: their MMAs (about 950 clocks of 64 positions) do not cover a copy's way and the zeroing of its columns
-        p.nq = 2;
-        while (seg <= 128 && p.nq < kMaxNQ && fixed + qbuf + 4 * x_slot <= budget) { ++p.nq; fixed += qbuf; }
-        p.nx = static_cast<int>((budget - fixed) / x_slot);
-        if (p.nx > kMaxNX) p.nx = kMaxNX;
-        smem = fixed + static_cast<size_t>(p.nx) * x_slot;
-        break;
+        return (HW + seg - 1) / seg * (pn.nload * pn.rows_box + 10);
+    };
+    auto best_segment = [&](size_t budget) {
+        int best = 0;
+        for (int seg = static_cast<int>(HW < 512 ? (HW + 63) / 64 * 64 : 512); seg >= 64; seg -= 64)
+            if (2ll * NP * panel_of(seg, p.W).bytes + 1024 + (half ? 2 : 3) * kXS * kXTile <= static_cast<long long>(budget) &&
+                (best == 0 || (!half && copied(seg) < copied(best))))
+                best = seg;
+        return best;
+    };
+    size_t budget = half ? kHalfSm : 227 * 1024 - 2048;
+    int seg = best_segment(budget);
+    if (seg == 0) return DBP_EUNSUPPORTED;
+    // An overlapped call's kernel of 128 output channels leaves 17 KB to a block of the next layer's position-major quantizer (256 -> 256
+    // fp32 at 16x16, batch 128: 145 us, 168 without; VGG-16 layer set 747, 751; 34 KB: 752, 51 KB: 762). What shorter segments cost for it, the
+    // share of bytes that is copied more, counts once per tile of channels, what it brings goes with the output channels. The line lies between, us with
+    // the room and without: 0.46 (72 -> 72 fp32 at 44x44, batch 16) 49.7, 50.5; 0.28 (128 -> 128 bf16 at 48x48) 40.6, 42.0; 0.22 (128 -> 128 fp32
+    // at 12x12, batch 128) 39.7, 41.8; and 0.49 (72 -> 72 fp32 at 48x48) 66.9, 62.5; 0.75 (360 -> 112 fp32 at 12x12, batch 113) 86.6, 75.3.
+    // Kernels of 64 channels: long segments are worth more (64 -> 64 at 32x32: 22.0 us, 24.0).
+    if (overlapped && !half && NP == 2) {
+        const size_t less = 210 * 1024 - 2048;
+        const int with_room = best_segment(less);
+        const double row = 128.0 * NP, bytes = copied(seg) * row + (HW + 63) / 64 * kXTile;
+        if (with_room != 0 && (copied(with_room) - copied(seg)) * row / bytes * p.ci_tiles * p.co_tiles * 128 <= 0.47 * s.Cout) {
+            budget = less;
+            seg = with_room;
+        }
     }
-    if (smem == 0) return DBP_EUNSUPPORTED;
+    const Panel pn = panel_of(seg, p.W);
+    const size_t qbuf = static_cast<size_t>(NP) * pn.bytes;
+    size_t fixed = 2 * qbuf + 1024;
+    p.SEG = seg; p.nload = pn.nload; p.rows_box = pn.rows_box; p.panel_bytes = pn.bytes;
+    // short segments: their MMAs (about 950 clocks of 64 positions) do not cover a copy's way and the zeroing of its columns
+    p.nq = 2;
+    while (seg <= 128 && p.nq < kMaxNQ && fixed + qbuf + 4 * x_slot <= budget) { ++p.nq; fixed += qbuf; }
+    p.nx = static_cast<int>((budget - fixed) / x_slot);
+    if (p.nx > kMaxNX) p.nx = kMaxNX;
+    const size_t smem = fixed + static_cast<size_t>(p.nx) * x_slot;
     p.segs_per_img = (p.HW + p.SEG - 1) / p.SEG;
     p.code_batch = static_cast<int>(s.B);
     p.split = pieces == 2 && s.Cin <= 64 ? 1 : 0;

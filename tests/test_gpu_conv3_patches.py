@@ -58,17 +58,19 @@ def test_input_gradient(ctx, B, Ci, Co, H, W, dtype):
     (70, 40, 200, 3, 5, "bf16"), (33, 16, 65, 8, 16, "f32"),           # ... and of two blocks, one output channel past a panel
     (3, 7, 130, 12, 11, "bf16"), (2, 129, 129, 20, 9, "f32"),          # channels that are no multiple of four in dW's rows
     (2, 1, 65, 5, 4, "f32"), (2, 4, 72, 3, 6, "bf16"), (3, 13, 40, 6, 6, "f32"),      # ... rows of one to four groups of channels, the last one empty
-    (2, 332, 1000, 4, 5, "bf16")])                                     # ... more groups than the finishing kernel has threads
+    (2, 332, 1000, 4, 5, "bf16"),                                      # ... more groups than the finishing kernel has threads
+    (2, 24, 72, 9, 60, "f32"), (2, 40, 130, 7, 44, "bf16"),            # segments of 128 positions, or of 64 for the next quantizer's sake
+    (3, 200, 72, 13, 13, "f32"), (2, 16, 48, 24, 24, "f32"), (2, 16, 72, 5, 62, "bf16")])       # ... of a whole image, of 192, the widest rows
 def test_weight_gradient_of_a_whole_sm(ctx, B, Ci, Co, H, W, dtype):
-    """An overlapped call's dW kernel has the SMs to itself. Twice: the second call adds into a scratch that the first put back to zero.
-    (Tolerance: fp32 sums of exact products, as above.)"""
+    """An overlapped call's dW kernel has the SMs to itself, and so has that of a call without dX, with other segments. Twice each: the
+    next call adds into a scratch that the one before put back to zero. (Tolerance: fp32 sums of exact products, as above.)"""
     import paper_2004_04729_b200 as dbp
     L = wl.conv_layer(B, Ci, Co, H, W, 3, data_seed=B + Ci + 3 * Co + H, scale=2.0, seed=11, dtype=dtype)
     tdt = torch.bfloat16 if dtype == "bf16" else torch.float32
     d, X, Wt = (torch.from_numpy(np.ascontiguousarray(a)).to(tdt).cuda() for a in (L.delta, L.X, L.W))
     ref = None
-    for _ in range(2):
-        out = dbp.dithered_conv_backward(ctx, d, X, Wt, L.seed, L.scale, flags=dbp.DBP_DW_ASYNC)
+    for kw in 2 * (dict(flags=dbp.DBP_DW_ASYNC), dict(need_dX=False)):
+        out = dbp.dithered_conv_backward(ctx, d, X, Wt, L.seed, L.scale, **kw)
         ctx.join()
         D, _ = ctx.last_step()
         if ref is None:
