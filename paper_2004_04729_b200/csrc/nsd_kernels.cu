@@ -151,7 +151,7 @@ __global__ void __launch_bounds__(kThreads) rows_job_kernel(const RowsJob j, int
 }
 
 // a block's sums
-__device__ __forceinline__ void leave_sums(double d1, double d2, double *__restrict__ partials) {
+__device__ __forceinline__ void leave_sums(double d1, double d2, double *__restrict__ to) {
     __shared__ double sh1[kThreads / 32], sh2[kThreads / 32];
     d1 = warp_sum(d1);
     d2 = warp_sum(d2);
@@ -161,13 +161,14 @@ __device__ __forceinline__ void leave_sums(double d1, double d2, double *__restr
     if (threadIdx.x == 0) {
         double a = 0.0, b = 0.0;
         for (int w = 0; w < kThreads / 32; ++w) { a += sh1[w]; b += sh2[w]; }
-        reinterpret_cast<double2 *>(partials)[blockIdx.x] = make_double2(a, b);
+        *reinterpret_cast<double2 *>(to) = make_double2(a, b);
     }
 }
 
-template <typename T, bool MASKED = false>
+// PARTS: there are more parts (pairs of sums) than blocks, and a block makes several of them one after the other
+template <typename T, bool MASKED, bool PARTS = false>
 __global__ void __launch_bounds__(kThreads)
-statistics_kernel(const T *__restrict__ x, long long n, double *__restrict__ partials,
+statistics_kernel(const T *__restrict__ x, long long n, int nparts, double *__restrict__ partials,
                   DeviceState *__restrict__ st, unsigned long long *__restrict__ nnz_out,
                   const unsigned char *__restrict__ mask, const SideJobs jobs) {
     constexpr int EPT = Vec<T>::V;
@@ -311,7 +312,8 @@ statistics_kernel(const T *__restrict__ x, long long n, double *__restrict__ par
         if (nnz_out) *nnz_out = 0ull;
     }
     const float pivot = (!MASKED || __ldg(mask)) ? Vec<T>::one(x) : 0.f;
-    const long long stride = static_cast<long long>(gridDim.x) * kThreads;
+    const int parts = PARTS ? nparts : static_cast<int>(gridDim.x);
+    const long long stride = static_cast<long long>(parts) * kThreads;
     auto add = [&](const Batch &b) {
 #pragma unroll
         for (int u = 0; u < U; ++u) {
@@ -332,38 +334,45 @@ statistics_kernel(const T *__restrict__ x, long long n, double *__restrict__ par
             d2 += static_cast<double>(s2);
         }
     };
-    for (long long t = blockIdx.x; t < ntile; t += 2 * gridDim.x) {
-        const long long t1 = t + gridDim.x, t2 = t1 + gridDim.x;
-        if (t1 < ntile) load(t1, odd);
-        add(even);
-        if (t2 < ntile) load(t2, even);
-        if (t1 < ntile) add(odd);
-    }
-    // the vectors after the last whole tile
-    long long i = ntile * tile + static_cast<long long>(blockIdx.x) * kThreads + threadIdx.x;
-    for (; i < nvec; i += stride) {
-        float v[EPT];
-        Vec<T>::values(Vec<T>::raw(x + i * EPT), v);
-        mask4<MASKED>(mask, i * EPT, v);
-        float s1 = 0.f, s2 = 0.f;
+    for (int part = blockIdx.x;;) {
+        for (long long t = part; t < ntile; t += 2 * parts) {
+            const long long t1 = t + parts, t2 = t1 + parts;
+            if (t1 < ntile) load(t1, odd);
+            add(even);
+            if (t2 < ntile) load(t2, even);
+            if (t1 < ntile) add(odd);
+        }
+        // the vectors after the last whole tile
+        long long i = ntile * tile + static_cast<long long>(part) * kThreads + threadIdx.x;
+        for (; i < nvec; i += stride) {
+            float v[EPT];
+            Vec<T>::values(Vec<T>::raw(x + i * EPT), v);
+            mask4<MASKED>(mask, i * EPT, v);
+            float s1 = 0.f, s2 = 0.f;
 #pragma unroll
-        for (int j = 0; j < EPT; ++j) {
-            const float c = v[j] - pivot;
-            s1 += c;
-            s2 = fmaf(c, c, s2);
+            for (int j = 0; j < EPT; ++j) {
+                const float c = v[j] - pivot;
+                s1 += c;
+                s2 = fmaf(c, c, s2);
+            }
+            d1 += static_cast<double>(s1);
+            d2 += static_cast<double>(s2);
         }
-        d1 += static_cast<double>(s1);
-        d2 += static_cast<double>(s2);
-    }
-    if (blockIdx.x == 0 && threadIdx.x == 0) {
-        for (long long i = nvec * EPT; i < n; ++i) {
-            const float xi = (!MASKED || __ldg(mask + i)) ? Vec<T>::one(x + i) : 0.f;
-            const double c = static_cast<double>(xi) - static_cast<double>(pivot);
-            d1 += c;
-            d2 += c * c;
+        if (part == 0 && threadIdx.x == 0) {
+            for (long long i = nvec * EPT; i < n; ++i) {
+                const float xi = (!MASKED || __ldg(mask + i)) ? Vec<T>::one(x + i) : 0.f;
+                const double c = static_cast<double>(xi) - static_cast<double>(pivot);
+                d1 += c;
+                d2 += c * c;
+            }
         }
+        leave_sums(d1, d2, partials + 2 * part);
+        part += gridDim.x;
+        if (!PARTS || part >= parts) break;
+        __syncthreads();                             // (the sums have been read)
+        if (part < ntile) load(part, even);
+        d1 = d2 = 0.0;
     }
-    leave_sums(d1, d2, partials);
 }
 
 // The statistics of a gradient that comes out of a 2x2 max-pool's routing, written on the way (one launch and one pass less than
@@ -409,7 +418,7 @@ statistics_pool_kernel(const PoolRouting pool, long long n2, double *__restrict_
             d2 += static_cast<double>(s2);
         }
     }
-    leave_sums(d1, d2, partials);
+    leave_sums(d1, d2, partials + 2 * blockIdx.x);
 }
 
 // A given step size: no statistics; the counters the quantizer adds to are cleared.
@@ -636,9 +645,16 @@ int launch_statistics(dbp_ctx *ctx, const void *delta, int dtype, long long nume
     // 847. The weight re-laying side job wants one block per output channel.
     if (jobs.w_src == nullptr && blocks > static_cast<long long>(ctx->sm_count) * kStatBlocksPerSM)
         blocks = static_cast<long long>(ctx->sm_count) * kStatBlocksPerSM;
+    // Beside an earlier call's dW, whose CTAs leave the registers for two of them, four blocks ran two after two, and the quantizer came to
+    // its loads and dithers only when the last ones had started. fp32 tensors of 100 MB and more are taken by two blocks per SM there, two
+    // parts each (the sums are the same: the step size does not depend on what is beside): 1x1 64 -> 256 at 56x56, batch 64, overlapped
+    // 176 us, 166 so; 128 -> 512 at 28x28 (103 MB) 93.1, 88.0. Smaller ones wait for memory's latency then: 300 -> 200 at 30x31, batch 100
+    // (74 MB), 206, 211; bf16 tensors too (ResNet-50 set 840, 855).
+    const bool halved = dtype == DBP_F32 && numel >= 25000000 && ctx->aux_pending && blocks > 2ll * ctx->sm_count;
+    const long long grid = halved ? 2ll * ctx->sm_count : blocks;
     auto go = [&](auto kern, auto x, const unsigned char *m) {
-        return launch_chained(kern, dim3(static_cast<unsigned>(blocks)), dim3(kThreads), 0, ctx->stream, x, numel, ctx->partials,
-                              ctx->state, nnz_out, m, jobs);
+        return launch_chained(kern, dim3(static_cast<unsigned>(grid)), dim3(kThreads), 0, ctx->stream, x, numel, static_cast<int>(blocks),
+                              ctx->partials, ctx->state, nnz_out, m, jobs);
     };
     step->partials = ctx->partials;
     step->nparts = static_cast<int>(blocks);
@@ -652,8 +668,8 @@ int launch_statistics(dbp_ctx *ctx, const void *delta, int dtype, long long nume
     }
     const float *xf = static_cast<const float *>(delta);
     const cudaError_t e = dtype != DBP_F32 ? go(statistics_kernel<__nv_bfloat16, false>, static_cast<const __nv_bfloat16 *>(delta), m)
-                          : mask != nullptr ? go(statistics_kernel<float, true>, xf, m)
-                                            : go(statistics_kernel<float, false>, xf, m);
+                          : mask != nullptr ? (halved ? go(statistics_kernel<float, true, true>, xf, m) : go(statistics_kernel<float, true>, xf, m))
+                                            : (halved ? go(statistics_kernel<float, false, true>, xf, m) : go(statistics_kernel<float, false>, xf, m));
     return cuda_ok(e);
 }
 

@@ -91,3 +91,27 @@ def test_sparse_form(ctx, n, dtype):
     q = dbp.nsd_quantize(ctx, d, 5, 0.0, delta_in=torch.tensor([float(D)], device="cuda"))
     assert q.nnz.item() == nnz and ctx.last_device_status()[1] == sat
     assert np.array_equal(dbp.nsd_decode_dense(ctx, q).cpu().numpy().reshape(-1), codes)
+
+
+@pytest.mark.parametrize("masked", [False, True])
+def test_step_size_of_a_large_tensor_beside_an_earlier_dw(ctx, masked):
+    """Large fp32 gradients are added up by fewer blocks while an earlier call's dW is outstanding: the step size and the count keep their
+    bits, and the step size is the one in 64 bits to 1e-6. (Ragged planes: the last tile of the sums is not whole.)"""
+    import paper_2004_04729_b200 as dbp
+    g = torch.Generator(device="cuda").manual_seed(3)
+    delta = torch.randn(16, 128, 111, 111, generator=g, device="cuda") + 0.25
+    X, W = torch.randn(16, 8, 111, 111, generator=g, device="cuda"), torch.randn(128, 8, 1, 1, generator=g, device="cuda")
+    mask = (torch.rand(delta.shape, generator=g, device="cuda") < 0.6).to(torch.uint8) if masked else None
+    steps = []
+    for flags in (0, dbp.DBP_DW_ASYNC, dbp.DBP_DW_ASYNC):          # the last call comes behind an outstanding dW
+        ctx.set_relu_mask(mask)
+        out = dbp.dithered_conv_backward(ctx, delta, X, W, 11, 2.0, flags=flags)
+        if len(steps) == 1:
+            steps.append(None)
+            continue
+        ctx.join()
+        steps.append(ctx.last_step())
+    assert steps[0] == steps[2]
+    want = 2.0 * (delta * mask if masked else delta).double().std(unbiased=False).item()
+    assert abs(steps[0][0] - want) <= 1e-6 * want
+    assert ctx.last_device_status() == (0, 0)
