@@ -588,14 +588,15 @@ int launch_tc3_tma_dw(dbp_ctx *ctx, const void *codes_nhwc, const void *X, int p
     // An overlapped call's kernel of 128 output channels leaves 17 KB to a block of the next layer's position-major quantizer (256 -> 256
     // fp32 at 16x16, batch 128: 145 us, 168 without; VGG-16 layer set 747, 751; 34 KB: 752, 51 KB: 762). What shorter segments cost for it, the
     // share of bytes that is copied more, counts once per tile of channels, what it brings goes with the output channels. The line lies between, us with
-    // the room and without: 0.46 (72 -> 72 fp32 at 44x44, batch 16) 49.7, 50.5; 0.28 (128 -> 128 bf16 at 48x48) 40.6, 42.0; 0.22 (128 -> 128 fp32
-    // at 12x12, batch 128) 39.7, 41.8; and 0.49 (72 -> 72 fp32 at 48x48) 66.9, 62.5; 0.75 (360 -> 112 fp32 at 12x12, batch 113) 86.6, 75.3.
+    // the room and without: 0.22 (72 -> 72 fp32 at 24x24, batch 43) 40.4, 43.5; 0.22 (128 -> 128 fp32 at 12x12, batch 128) 39.7, 41.8; and 0.30
+    // (128 -> 128 bf16 at 56x56, batch 16) 51.4, 47.4; 0.33 (100 -> 100 bf16 at 44x44, batch 100) 168.9, 148.6; 0.75 (360 -> 112 fp32 at
+    // 12x12, batch 113) 86.6, 75.3. Wide planes of few images gain from the room for longer: 0.26 (128 -> 128 fp32 at 44x44, batch 16) 51.9, 57.4.
     // Kernels of 64 channels: long segments are worth more (64 -> 64 at 32x32: 22.0 us, 24.0).
     if (overlapped && !half && NP == 2) {
         const size_t less = 210 * 1024 - 2048;
         const int with_room = best_segment(less);
         const double row = 128.0 * NP, bytes = copied(seg) * row + (HW + 63) / 64 * kXTile;
-        if (with_room != 0 && (copied(with_room) - copied(seg)) * row / bytes * p.ci_tiles * p.co_tiles * 128 <= 0.47 * s.Cout) {
+        if (with_room != 0 && (copied(with_room) - copied(seg)) * row / bytes * p.ci_tiles * p.co_tiles * 128 <= 0.25 * s.Cout) {
             budget = less;
             seg = with_room;
         }

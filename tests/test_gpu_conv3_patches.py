@@ -59,8 +59,8 @@ def test_input_gradient(ctx, B, Ci, Co, H, W, dtype):
     (3, 7, 130, 12, 11, "bf16"), (2, 129, 129, 20, 9, "f32"),          # channels that are no multiple of four in dW's rows
     (2, 1, 65, 5, 4, "f32"), (2, 4, 72, 3, 6, "bf16"), (3, 13, 40, 6, 6, "f32"),      # ... rows of one to four groups of channels, the last one empty
     (2, 332, 1000, 4, 5, "bf16"),                                      # ... more groups than the finishing kernel has threads
-    (2, 24, 72, 9, 60, "f32"), (2, 40, 130, 7, 44, "bf16"),            # segments of 128 positions, or of 64 for the next quantizer's sake
-    (3, 200, 72, 13, 13, "f32"), (2, 16, 48, 24, 24, "f32"), (2, 16, 72, 5, 62, "bf16")])       # ... of a whole image, of 192, the widest rows
+    (2, 24, 72, 24, 24, "f32"), (2, 40, 130, 9, 44, "bf16"),           # segments of 192 positions, of 128 for the next quantizer's sake, of 128
+    (3, 200, 72, 13, 13, "f32"), (2, 16, 48, 24, 24, "f32"), (2, 16, 72, 5, 62, "bf16")])       # ... of a whole image, one panel, the widest rows
 def test_weight_gradient_of_a_whole_sm(ctx, B, Ci, Co, H, W, dtype):
     """An overlapped call's dW kernel has the SMs to itself, and so has that of a call without dX, with other segments. Twice each: the
     next call adds into a scratch that the one before put back to zero. (Tolerance: fp32 sums of exact products, as above.)"""
