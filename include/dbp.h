@@ -239,8 +239,8 @@ int nsd_decode_dense(dbp_ctx *ctx, const dbp_sparse *q, int8_t *codes);
  * Outputs are overwritten, not accumulated.
  * dX (in fp32) and dW are within 1e-5 of the sum of their terms' sizes; fp32 operands that all have one and the same mantissa
  * may cost up to 2^-17 on top (they enter the tensor cores as two bf16 pieces).
- * Small fp32 layers (at most 2^17 gradient elements, products of no more tiles than the GPU has SMs, or twice as many where
- * the reductions are at most 512 long), no q_out and no
+ * Small fp32 layers (at most 2^17 gradient elements, products of no more 64 x 64 tiles than the GPU has SMs, or twice as many
+ * where the reductions are at most 512 long and all tiles together no more than ten chunks of 64 per SM), no q_out and no
  * FORCE flag, run as two chained kernels (statistics, dither and quantization; then the products; profiling kind
  * DBP_K_FUSED): same results to the same tolerances, Delta and nnz through dbp_last_step.
  */

@@ -57,6 +57,10 @@ def _fused_was_used(ctx, fn):
     (300, 400, 64),      # eight vectors per thread, shared by four clusters
     (1000, 100, 72),     # a reduction of sixteen chunks: two rounds of eight
     (577, 17, 33),       # ... and of ten, the last one of a single row; odd rows and columns
+    (300, 300, 1500),    # 240 tiles: a second wave of CTAs
+    (64, 512, 2048),     # 288, reductions of one and of eight chunks
+    (90, 200, 2002),     # 192, K % 4 != 0
+    (512, 66, 960),      # 150, of eight chunks (dW) and of two: the second wave is a few dX tiles
 ])
 def test_small_linear_matches_the_oracle(ctx, B, N, K):
     import paper_2004_04729_b200 as dbp
@@ -71,6 +75,31 @@ def test_small_linear_matches_the_oracle(ctx, B, N, K):
     codes, onnz, _ = oracle.nsd_codes(L.delta, L.seed, D)
     assert nnz == onnz
     _check_products(out, oracle.linear_backward(codes, D, L.X, L.W, with_abs=True), ("dW", "dX", "db"))
+
+
+@pytest.mark.parametrize("B,N,K", [
+    (64, 512, 2112),     # 297 tiles: a third wave
+    (513, 100, 960),     # 165 with a reduction of nine chunks: two rounds
+    (327, 384, 1496),    # 288 of six chunks: more than ten an SM
+])
+def test_linear_layers_just_past_the_small_path(ctx, B, N, K):
+    """(The lines lie at multiples of the SMs: 148.) The kernels for larger layers take these, to the same tolerances."""
+    import paper_2004_04729_b200 as dbp
+    L = wl.linear_layer(B, N, K, data_seed=500 + B + N + K, scale=2.0, seed=7)
+    d, X, W = _cu(L.delta), _cu(L.X), _cu(L.W)
+    ctx.profile_enable(True)
+    ctx.profile_select(None)
+    ctx.profile_read()
+    out = dbp.dithered_linear_backward(ctx, d, X, W, L.seed, L.scale, need_db=True)
+    pr = ctx.profile_read()
+    ctx.profile_enable(False)
+    if torch.cuda.get_device_properties(0).multi_processor_count == 148:
+        assert pr["fused"][1] == 0 and pr["statistics"][1] == 1, pr
+    D, nnz = ctx.last_step()
+    codes, onnz, _ = oracle.nsd_codes(L.delta, L.seed, np.float32(D))
+    assert nnz == onnz
+    _check_products(out, oracle.linear_backward(codes, np.float32(D), L.X, L.W, with_abs=True), ("dW", "dX", "db"))
+    assert ctx.last_device_status() == (0, 0)
 
 
 def test_small_linear_one_product_and_given_step(ctx):
