@@ -166,8 +166,9 @@ __device__ __forceinline__ void leave_sums(double d1, double d2, double *__restr
 }
 
 // PARTS: there are more parts (pairs of sums) than blocks, and a block makes several of them one after the other
-template <typename T, bool MASKED, bool PARTS = false>
-__global__ void __launch_bounds__(kThreads)
+// MOST: blocks of an SM that the registers have to allow
+template <typename T, bool MASKED, bool PARTS = false, int MOST = kStatBlocksPerSM>
+__global__ void __launch_bounds__(kThreads, MOST < kStatBlocksPerSM ? MOST : 0)
 statistics_kernel(const T *__restrict__ x, long long n, int nparts, double *__restrict__ partials,
                   DeviceState *__restrict__ st, unsigned long long *__restrict__ nnz_out,
                   const unsigned char *__restrict__ mask, const SideJobs jobs) {
@@ -667,7 +668,16 @@ int launch_statistics(dbp_ctx *ctx, const void *delta, int dtype, long long nume
                                       dim3(kThreads), 0, ctx->stream, jobs.pool, numel / 8, ctx->partials, ctx->state, nnz_out, m, jobs));
     }
     const float *xf = static_cast<const float *>(delta);
-    const cudaError_t e = dtype != DBP_F32 ? go(statistics_kernel<__nv_bfloat16, false>, static_cast<const __nv_bfloat16 *>(delta), m)
+    // A grid of two blocks per SM at most, with nothing beside it, takes the instance with up to 128 registers: its side jobs keep more loads
+    // under way than in the 64 that four blocks leave. us with 64, with more: fp32 1000 -> 999 of 777, batch 1000, 32.6, 30.6; 384 of
+    // 1496, batch 327, 16.3, 15.2; 3x3 961 -> 224 at 14x15, batch 8, dX alone 42.2, 37.7; bf16 999 of 777 25.6, 24.8. (Everywhere: ResNet-50 set
+    // 836, 850.)
+    const __nv_bfloat16 *xb = static_cast<const __nv_bfloat16 *>(delta);
+    const bool few = grid <= 2ll * ctx->sm_count && !ctx->aux_pending;
+    const cudaError_t e = few ? (dtype != DBP_F32 ? go(statistics_kernel<__nv_bfloat16, false, false, 2>, xb, m)
+                                 : mask != nullptr ? go(statistics_kernel<float, true, false, 2>, xf, m)
+                                                   : go(statistics_kernel<float, false, false, 2>, xf, m))
+                          : dtype != DBP_F32 ? go(statistics_kernel<__nv_bfloat16, false>, xb, m)
                           : mask != nullptr ? (halved ? go(statistics_kernel<float, true, true>, xf, m) : go(statistics_kernel<float, true>, xf, m))
                                             : (halved ? go(statistics_kernel<float, false, true>, xf, m) : go(statistics_kernel<float, false>, xf, m));
     return cuda_ok(e);
