@@ -467,9 +467,9 @@ small_linear_products_kernel(const __grid_constant__ CUtensorMap map_q, const Sm
 // reductions that lie in shared memory at once and are at most ten chunks of 64 an SM, all tiles together. More cost more
 // than the third launch of the CTA-wide kernels (linear_tc.cu).
 // us, this path against that one, fp32 as (batch, outputs, inputs): (128, 300, 784), 91 tiles: 7.95, 14.9; (128, 1000, 512), 144:
-// 17.1, 22.4; (128, 512, 1024), 160: 14.0, 16.4; (300, 300, 1500), 240 of five chunks: 14.7, 16.2; (228, 437, 1368), 242, 8.3 chunks an SM: 15.9,
-// 17.2; (288, 262, 1812), 290, 9.8: 15.6, 16.9; (64, 512, 2048), 288: 13.9, 15.7; more chunks: (256, 512, 1500), 288, 10.4: 17.1, 16.7;
-// (512, 256, 1500), 288, 10.4: 15.6, 16.0; (327, 384, 1496), 288, 11.7: 16.8, 16.2; (350, 370, 1500), 288, 11.7: 17.5, 17.0;
+// 17.1, 22.4; (128, 512, 1024), 160: 14.0, 16.4; (300, 300, 1500), 240 of five chunks, 8.1 an SM: 14.7, 15.4; (288, 262, 1812), 290, 9.8:
+// 15.6, 16.5; (64, 512, 2048), 288: 13.9, 15.7; more chunks: (256, 512, 1500), 288, 10.4: 17.1, 15.5; (512, 256, 1500), 288, 10.4: 15.6, 14.8;
+// (327, 384, 1496), 288, 11.7: 16.8, 15.2;
 // two rounds of chunks: (1024, 100, 1024), 288: 16.0, 14.3; (1000, 64, 1000), 272: 14.7, 13.1; three tiles: (500, 128, 2048),
 // 320: 15.5, 14.0.
 bool small_linear_fits(const dbp_ctx *ctx, long long B, long long N, long long K, bool want_dw, bool want_dx) {
