@@ -88,7 +88,9 @@ __global__ void __launch_bounds__(256) phases_of_kernel(const T *__restrict__ X,
 // 8; what lies behind a plane is never read). A thread takes eight consecutive positions of one plane's rows of parity py
 // and writes both column parities' rows (phases = 4; phases = 1: the even rows and columns only). fp32 values leave as two
 // pieces (rounded, and the remainder rounded). VEC: W/2 is a multiple of four, so four positions are one or two vectors. EVEN: of two, so two positions are one.
-// beside: see rows_job_kernel (nsd_kernels.cu).
+// beside: see rows_job_kernel (nsd_kernels.cu). All blocks wait: where one does, dX's CTAs take the SMs in front of dW's more often (3x3 stride
+// 2, bf16 228 -> 82 at 10x10, batch 45: 45.4 us, 56.7 with one; fp32 248 -> 96 at 12x12, batch 23: 44.7, 49.7; 32 -> 32 at 28x28, batch 32:
+// 31.8, 35.5; but bf16 120 -> 56 at 60x60, batch 8, 42.6, 38.4, and 64 -> 64 at 14x14, batch 64, 37.0, 34.6).
 template <typename T, bool VEC, bool EVEN>
 __global__ void __launch_bounds__(256) phase_rows_kernel(const T *__restrict__ X, unsigned short *__restrict__ out, unsigned planes,
                                                          unsigned Cin, unsigned H, unsigned W, unsigned pitch, int phases, int beside) {
