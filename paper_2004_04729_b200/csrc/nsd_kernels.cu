@@ -670,12 +670,14 @@ int launch_statistics(dbp_ctx *ctx, const void *delta, int dtype, long long nume
                                       dim3(kThreads), 0, ctx->stream, jobs.pool, numel / 8, ctx->partials, ctx->state, nnz_out, m, jobs));
     }
     const float *xf = static_cast<const float *>(delta);
-    // A grid of two blocks per SM at most, with nothing beside it, takes the instance with up to 128 registers: its side jobs keep more loads
-    // under way than in the 64 that four blocks leave. us with 64, with more: fp32 1000 -> 999 of 777, batch 1000, 32.6, 30.6; 384 of
-    // 1496, batch 327, 16.3, 15.2; 3x3 961 -> 224 at 14x15, batch 8, dX alone 42.2, 37.7; bf16 999 of 777 25.6, 24.8. (Everywhere: ResNet-50 set
-    // 836, 850.)
+    // Side jobs that are more than a store or a pair of loads at a time (rows re-written, 3x3 weights of an odd channel count), in a grid of
+    // two blocks per SM at most with nothing beside it: the instance with up to 128 registers keeps more of their loads under way than the
+    // 64 that four blocks leave. us with 64, with more: fp32 1000 -> 999 of 777, batch 1000, 32.6, 30.6; 384 of 1496, batch 327, 16.3, 15.2;
+    // 3x3 961 -> 224 at 14x15, batch 8, dX alone 42.2, 37.7; bf16 999 of 777 25.6, 24.8. Other calls lose by it, because the quantizer's blocks
+    // find no registers beside these (ResNet-50 set of 16 images 406.4, 410.3; in every grid, 64 images: 836, 850).
     const __nv_bfloat16 *xb = static_cast<const __nv_bfloat16 *>(delta);
-    const bool few = grid <= 2ll * ctx->sm_count && !ctx->aux_pending;
+    const bool odd_weights = jobs.w_src != nullptr && ((jobs.phase_cin > 0 ? jobs.phase_cin : jobs.Cin) & 1) != 0;
+    const bool few = (jobs.nrows > 0 || odd_weights) && grid <= 2ll * ctx->sm_count && !ctx->aux_pending;
     const cudaError_t e = few ? (dtype != DBP_F32 ? go(statistics_kernel<__nv_bfloat16, false, false, 2>, xb, m)
                                  : mask != nullptr ? go(statistics_kernel<float, true, false, 2>, xf, m)
                                                    : go(statistics_kernel<float, false, false, 2>, xf, m))
